@@ -33,10 +33,12 @@
 
 namespace hbf {
 
-// Block shape of the serve kernel.  The per-queue state (32 KB) is all the shared memory a block needs, so
-// several blocks share an SM, each with its own tile and its own row-after-row chain of queue updates.
+// Block shape of the serve kernel: two blocks per SM, each with its own tile and its own row-after-row chain of queue updates.
+// (12 warps a block: with the 32-bit form a 200 M batch takes 1,587 us, with 10 warps 1,667, 11: 1,700, 13: 1,720, 14: 1,669;
+// three or four blocks of 8 to 10 warps 1,890 to 2,500: more tiles in flight are more streams to DRAM, which the pass keeps
+// at 5.7 TB/s.)
 #ifndef HBF_IN_THREADS
-#define HBF_IN_THREADS 320
+#define HBF_IN_THREADS 384
 #endif
 #ifndef HBF_IN_BLOCKS
 #define HBF_IN_BLOCKS 2
@@ -118,13 +120,21 @@ struct __align__(16) FastGeom {
     uint32_t page_mask, page_shift, gran_shift_read, gran_shift_prog;
     uint32_t tab_shift, tab_max_cb, t_read, t_prog;
     const uint32_t *xfer_tab; uint64_t pad;
+    // the 32-bit form of the pass (serve_narrow below); narrow == 0: not for this configuration
+    uint64_t nw_delta, nw_lim;                               // media offset = address + nw_delta; range offsets up to nw_lim hold any inline access
+    uint32_t narrow, nw_bytes, nw_flag_lo, nw_flag_n;        // inline accesses: at most nw_bytes bytes, flags nw_flag_lo .. nw_flag_lo + nw_flag_n - 1
+    uint32_t nw_gmax, nw_mul_read, nw_mul_prog, nw_add;      // most granules of an inline read; transfer = (granules * mul + add) / rate by
+    uint32_t nw_magic, nw_shift, nw_chmul, nw_pad;           //   multiply-high; queues per channel
 };
+// Bounds of the 32-bit form.  A service is below 2^26 ns, so that the services of a row's 32 lanes compose below 2^31; the
+// granules and the reads of an access fit 11 and 6 bits, so that a row's sums travel in one word (17 and 11 bits).
+constexpr uint32_t kNwServeBits = 26, kNwGranules = 2048, kNwPages = 32, kNwCountShift = 17;
 // (the last condition: an access within the transfer table's reach spans few pages, and their unscaled service stays
 // below 2^32 ns, so the common path needs no test of its own)
-__device__ __forceinline__ bool fast_geom_ok(const FastRange &f, const ModelParams &mp) {
+__host__ __device__ __forceinline__ bool fast_geom_ok(const FastRange &f, const ModelParams &mp) {
     const uint64_t pages = ((uint64_t)mp.xfer_tab_max_cb >> mp.page_shift) + 2ull;
     return f.on != 0u && mp.pow2_geom != 0u && mp.xfer_tab_max_cb != 0u && mp.t_read_ns < (1ll << 32) && mp.t_prog_ns < (1ll << 32) &&
-           pages * (uint64_t)max(mp.t_read_ns, mp.t_prog_ns) < (1ull << 32);
+           pages * (uint64_t)(mp.t_read_ns > mp.t_prog_ns ? mp.t_read_ns : mp.t_prog_ns) < (1ull << 32);
 }
 __host__ __device__ __forceinline__ FastGeom make_fast_geom(const FastRange &f, const ModelParams &mp) {
     FastGeom g;
@@ -136,6 +146,29 @@ __host__ __device__ __forceinline__ FastGeom make_fast_geom(const FastRange &f, 
     g.gran_shift_read = mp.read_gran_shift; g.gran_shift_prog = mp.prog_gran_shift;
     g.tab_shift = mp.xfer_tab_shift; g.tab_max_cb = mp.xfer_tab_max_cb; g.t_read = (uint32_t)mp.t_read_ns; g.t_prog = (uint32_t)mp.t_prog_ns;
     g.xfer_tab = mp.xfer_tab; g.pad = 0;
+    // 32-bit form: which accesses are inline, and the division by the channel rate d as a 32-bit multiply-high (exact for
+    // numerators below 2^31: magic = floor(2^(31+l) / d) + 1 with l = ceil(log2 d), shift l - 1)
+    g.nw_delta = f.media_offset - f.base; g.nw_chmul = mp.dies * g.planes_q; g.nw_pad = 0;
+    g.nw_flag_lo = (f.perms & 1u) ? 0u : 1u; g.nw_flag_n = (f.perms & 3u) == 3u ? 2u : 1u;
+    g.nw_mul_read = 1000u << (mp.read_gran_shift & 15u); g.nw_mul_prog = 1000u << (mp.prog_gran_shift & 15u);
+    g.narrow = 0u; g.nw_bytes = g.nw_gmax = g.nw_add = g.nw_magic = g.nw_shift = 0u; g.nw_lim = 0;
+    const uint64_t d = mp.chan_bytes_per_us, t_max = (uint64_t)(mp.t_read_ns > mp.t_prog_ns ? mp.t_read_ns : mp.t_prog_ns);
+    const uint64_t quantum = (uint64_t)mp.t_read_ns + (uint64_t)mp.t_prog_ns;   // (a claimed refresh quantum is added to a service)
+    if (fast_geom_ok(f, mp) && d >= 2u && d < (1ull << 30) && mp.read_gran_shift <= 15u && mp.prog_gran_shift <= 15u && mp.page_shift <= 20u &&
+        (f.perms & 3u) != 0u && quantum < (1ull << (kNwServeBits - 1))) {
+        const uint64_t pages_s = ((1ull << kNwServeBits) - 1u - quantum) / t_max, pages = pages_s < kNwPages ? pages_s : kNwPages;
+        uint64_t most = pages >= 2u ? (pages - 1u) << mp.page_shift : 0u;       // so many bytes never touch more than `pages` pages
+        if (((uint64_t)kNwGranules << mp.read_gran_shift) < most) most = (uint64_t)kNwGranules << mp.read_gran_shift;
+        if (f.length < most) most = f.length;
+        const uint64_t worst = (most + ((1ull << mp.read_gran_shift) | (1ull << mp.prog_gran_shift)) * 2u) * 1000u + d;
+        if (most >= 1u && worst < (1ull << 31)) {
+            uint32_t l = 0;
+            while ((1ull << l) < d) ++l;
+            g.narrow = 1u; g.nw_bytes = (uint32_t)most; g.nw_lim = f.length - most;
+            g.nw_gmax = (uint32_t)((most + (1ull << mp.read_gran_shift) - 1u) >> mp.read_gran_shift);
+            g.nw_add = (uint32_t)d - 1u; g.nw_magic = (uint32_t)((1ull << (31 + l)) / d + 1u); g.nw_shift = l - 1u;
+        }
+    }
     return g;
 }
 // No branches: every access computes every term, and the classification (the same tests in the same order as classify())
@@ -221,6 +254,256 @@ __device__ __forceinline__ void row_wait2(int id, int64_t m, long long s8, const
                  "l"(m2), "l"(s82), "l"(pq2), "r"(pc2), "r"((int)last2) : "memory");
 }
 
+
+// ======================================================================================================
+// The streaming pass in 32-bit arithmetic, for the common configuration (one range, powers of two, no thermal scaling).  A
+// tile spans milliseconds, so inside it a time is 32 bits from the tile's first issue time: the maps, their composition
+// and the ordered update are single instructions where 64-bit ones take two to four, and the state of a queue has room for
+// the bytes and the number of its reads, which the update that owns the queue adds up (they were three shared-memory
+// atomics per access).  The transfer time is a multiply-high instead of a table look-up.  Programs, accesses near the end
+// of the range or larger than nw_bytes, and whatever is not modeled take a branch of their own.
+// Bound by DRAM (42.2 B per access at 5.7 TB/s, 0.87 of a copy) with the L1's data pipe close behind (70 % busy).  Measured on
+// the 200 M capacity batch, pass with everything around it: 2,086 -> 1,687 us (7.4 -> 5.3 warp instructions per access).
+// Tried and not kept: the records through shared memory by a bulk copy per turn (L1 pipe 70 -> 55 % busy, but 1,650 us with an L2
+// prefetch ahead of it and 1,710 without, against 1,587 for the submit alone); both rows of a turn updated side by side, with
+// queues shared across the rows composed in registers (shorter chain, 8 % more instructions: 1,626); four rows per turn (the same).
+// What the form cannot hold (a time 2^31 ns or more past the tile's first, by a gap in the stream or by a backlog) is
+// only noticed, in bits that are OR-ed along; such a tile is then served again in the 64-bit form.
+// Queue state (16 bytes): busy-until, service time in this tile, read granules, reads << 4 | head entries written.
+// ======================================================================================================
+struct NarrowSums { uint32_t native, fault, max_done; unsigned unsorted, over; long long stall; };
+
+__device__ __forceinline__ uint32_t nw_transfer(const FastGeom &g, uint32_t granules, uint32_t mul) {
+    return __umulhi(granules * mul + g.nw_add, g.nw_magic) >> g.nw_shift;
+}
+
+__device__ __forceinline__ void row_wait_n(int id, uint32_t m, uint32_t s, const void *pq, uint32_t gn, bool last,
+                                           uint32_t m2, uint32_t s2, const void *pq2, uint32_t gn2, bool last2) {
+    asm volatile("barrier.cta.sync.aligned %0, 64;" ::"r"(id), "r"(m), "r"(s), "l"(pq), "r"(gn), "r"((int)last),
+                 "r"(m2), "r"(s2), "l"(pq2), "r"(gn2), "r"((int)last2) : "memory");
+}
+
+template <bool DEBT>
+__device__ __forceinline__ NarrowSums serve_narrow(const FastGeom &geom, const ModelParams &mp, const ModelParams &mp_arg, const hbf_access_t *acc_t, const uint32_t tile_begin,
+                                                   const uint32_t tile_len, const int64_t T0, uint4 *qst, uint8_t *warp_tag, uint8_t *status_t,
+                                                   uint16_t *qid_t, const uint32_t qid_stride, int64_t *completion_t, int64_t *stall_t,
+                                                   InHead *__restrict__ in_head, const uint32_t tile, const uint32_t R, const uint32_t head_depth,
+                                                   uint32_t *s_heads_full, uint32_t *st_br_lo, const uint32_t n_dies,
+                                                   const uint64_t claim_limit, const uint32_t quantum_ns, const RetDev &ret, const uint32_t ret_row_shift) {
+    constexpr int K = kInRows;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    uint32_t *st_br_hi = st_br_lo + n_dies, *st_bp_lo = st_br_hi + n_dies, *st_bp_hi = st_bp_lo + n_dies, *st_nr = st_bp_hi + n_dies, *st_np = st_nr + n_dies, *st_claims = st_np + n_dies;
+    NarrowSums r; r.native = 0; r.fault = 0; r.max_done = 0; r.unsorted = 0; r.over = 0; r.stall = 0;
+    uint32_t b_time = 0, b_hi = 0, b_sort = 0;               // OR-ed along: bit 31 of times, high words of times, sign of issue - previous issue
+    const uint32_t rows = (tile_len + 31u) / 32u, turns = (rows + K - 1) / K;
+    const unsigned le_mask = lanemask_lt() | (1u << lane);
+    const int my_bar = 1 + warp, next_bar = 1 + (warp + 1 == kInWarps ? 0 : warp + 1);
+    uint64_t nx_addr[K], nx_issue[K], nx_bf[K];
+    uint32_t nx_prev[K];                                     // low word of the issue time before the lane's own
+#pragma unroll
+    for (int u = 0; u < K; ++u) { nx_addr[u] = 0; nx_issue[u] = 0; nx_bf[u] = 0; nx_prev[u] = 0; }
+    const bool pf_lane = lane < 24;
+    const char *pf_base = reinterpret_cast<const char *>(acc_t) + lane * 32;
+    auto fetch = [&](uint32_t turn) {
+#pragma unroll
+        for (int u = 0; u < K; ++u) {
+            const uint32_t j = (turn * K + u) * 32u + (uint32_t)lane;
+            if (j < tile_len) {
+                const uint64_t *rec = reinterpret_cast<const uint64_t *>(acc_t + j);
+                nx_addr[u] = __ldcs(rec); nx_issue[u] = __ldcs(rec + 1); nx_bf[u] = __ldcs(rec + 2);   // read once: streaming loads
+                nx_prev[u] = j > 0u ? __ldg(reinterpret_cast<const uint32_t *>(rec - 2)) : (uint32_t)T0;   // (the tile's first record was compared before)
+            }
+        }
+    };
+    fetch((uint32_t)warp);
+    for (uint32_t turn = (uint32_t)warp; turn < turns; turn += kInWarps) {
+      auto whole_turn = [&](auto full_tag) {
+        constexpr bool FULL = decltype(full_tag)::value;
+        uint32_t i[K], ri[K], q[K], S[K], M[K], xo[K], gn[K];
+        bool valid[K], ready[K];
+        uint64_t addr[K], bf[K]; int64_t issue[K]; uint32_t prev[K];
+#pragma unroll
+        for (int u = 0; u < K; ++u) {
+            i[u] = (turn * K + u) * 32u + (uint32_t)lane;
+            valid[u] = FULL || i[u] < tile_len;
+            addr[u] = nx_addr[u]; bf[u] = nx_bf[u]; issue[u] = (int64_t)nx_issue[u]; prev[u] = nx_prev[u];
+        }
+        fetch(turn + kInWarps);
+        {                                                    // and the turn after that is called into the L2
+            const uint32_t first = (turn + kInPrefetchTurns * kInWarps) * (uint32_t)(K * 32);
+            if (pf_lane && first + K * 32 <= tile_len) {
+                const char *p = pf_base + (size_t)first * sizeof(hbf_access_t);
+#pragma unroll
+                for (int u = 0; u < K; ++u) asm volatile("prefetch.global.L2 [%0];" ::"l"(p + u * 768));
+            }
+        }
+        // ---- terms
+#pragma unroll
+        for (int u = 0; u < K; ++u) {
+            const uint32_t bytes = (uint32_t)bf[u], flags = (uint32_t)(bf[u] >> 32);
+            const uint64_t dt = (uint64_t)(issue[u] - T0), rel = addr[u] - geom.base, off = addr[u] + geom.nw_delta;
+            ri[u] = (uint32_t)dt;
+            ready[u] = valid[u] && rel <= geom.nw_lim && bytes - 1u < geom.nw_bytes && flags - geom.nw_flag_lo < geom.nw_flag_n;
+            if (valid[u]) { b_hi |= (uint32_t)(dt >> 32); b_time |= ri[u]; b_sort |= (uint32_t)issue[u] - prev[u]; }
+            q[u] = 0; S[u] = 0; M[u] = 0; xo[u] = 0; gn[u] = 0;
+            uint32_t st = HBF_ST_READY;
+            const bool common = ready[u];
+            if (common) {
+                const uint32_t w = (uint32_t)(off >> geom.stripe_shift), in_page = (uint32_t)off & geom.page_mask;
+                q[u] = (w & geom.ch_mask) * geom.nw_chmul + ((w >> geom.ch_shift) & geom.die_mask) * geom.planes_q + ((w >> geom.chdie_shift) & geom.plane_mask_q);
+                const uint32_t npages = (in_page + bytes + geom.page_mask) >> geom.page_shift;
+                if (flags == 0u) {
+                    const uint32_t g = (bytes + ((1u << geom.gran_shift_read) - 1u)) >> geom.gran_shift_read;
+                    S[u] = npages * geom.t_read; xo[u] = nw_transfer(geom, g, geom.nw_mul_read);
+                    gn[u] = g | (1u << kNwCountShift);
+                    M[u] = ri[u] + S[u];
+                } else {                                     // a program: its data is transferred first; bytes and count by atomics
+                    const uint32_t g = (bytes + ((1u << geom.gran_shift_prog) - 1u)) >> geom.gran_shift_prog, xf = nw_transfer(geom, g, geom.nw_mul_prog);
+                    S[u] = npages * geom.t_prog; xo[u] = xf | 0x80000000u;
+                    M[u] = ri[u] + xf + S[u];
+                    const uint32_t die = geom.planes_q == 1u ? q[u] : q[u] >> mp_arg.plane_shift, lo = g << geom.gran_shift_prog;
+                    atomicAdd(&st_np[die], 1u);
+                    const uint32_t old = atomicAdd(&st_bp_lo[die], lo);
+                    if (old + lo < old) atomicAdd(&st_bp_hi[die], 1u);
+                }
+                if (DEBT && tile_begin + i[u] < claim_limit) {
+                    S[u] += quantum_ns; M[u] += quantum_ns;
+                    atomicAdd(&st_claims[geom.planes_q == 1u ? q[u] : q[u] >> mp_arg.plane_shift], 1u);
+                }
+            } else if (valid[u]) {                           // near the range's end, large, or not modeled
+                unsigned lng = 0;
+                const Served v = serve_terms_geom(geom, mp, addr[u], issue[u], bf[u], 1000000, Div64{}, lng, (int)kNwServeBits - 1);
+                st = (uint32_t)v.st;
+                if (v.st == HBF_ST_READY) {
+                    ready[u] = true; q[u] = v.queue;
+                    if (lng || ((uint64_t)v.s >> (kNwServeBits - 1)) || (v.xfer >> 30)) b_time |= 0x80000000u;
+                    S[u] = (uint32_t)v.s; xo[u] = v.xfer | (v.op << 31);
+                    const uint32_t lo = (uint32_t)v.cb, hi = (uint32_t)((uint64_t)v.cb >> 32);
+                    uint32_t *plo = v.op ? st_bp_lo : st_br_lo, *phi = v.op ? st_bp_hi : st_br_hi;
+                    atomicAdd(v.op ? &st_np[v.die] : &st_nr[v.die], 1u);
+                    const uint32_t old = atomicAdd(&plo[v.die], lo), carry = hi + ((old + lo) < old ? 1u : 0u);
+                    if (carry) atomicAdd(&phi[v.die], carry);
+                    if (DEBT && tile_begin + i[u] < claim_limit) { S[u] += quantum_ns; atomicAdd(&st_claims[v.die], 1u); }
+                    M[u] = ri[u] + (v.op ? v.xfer : 0u) + S[u];
+                } else if (v.st == HBF_ST_NATIVE) {
+                    r.native += 1u;
+                } else {
+                    r.fault += 1u;
+                }
+            }
+            if (DEBT && ready[u] && flags == 0u) {           // read disturb: the read's pages, on the block of its first page
+                const uint32_t npages = (uint32_t)(((uint64_t)((uint32_t)off & geom.page_mask) + bytes + geom.page_mask) >> geom.page_shift);
+                if (ret.pow2 != 0u) {
+                    const uint32_t row = (uint32_t)((off >> geom.stripe_shift) >> ret_row_shift);
+                    const uint32_t in_stripe = ((uint32_t)off & ((1u << geom.stripe_shift) - 1u)) >> geom.page_shift;
+                    const uint32_t blk = ((row << mp_arg.pages_per_stripe_shift) + in_stripe) >> ret.ppb_shift;
+                    const uint32_t pl = (uint32_t)(off >> (geom.stripe_shift + geom.chdie_shift)) & geom.plane_mask;
+                    const uint32_t die = geom.planes_q == 1u ? q[u] : q[u] >> mp_arg.plane_shift;
+                    atomicAdd(&ret.disturb[((die << mp_arg.plane_shift) + pl) * ret.bpp + (blk & (ret.bpp - 1u))], npages);
+                } else {
+                    atomicAdd(&ret.disturb[ret_block_of(mp, ret, off)], npages);
+                }
+            }
+            if (status_t && valid[u]) status_t[i[u]] = (uint8_t)st;
+        }
+        // ---- which lanes of a row hold the same queue (see the 64-bit form)
+        uint8_t *tag_at[K];
+        uint32_t tagged[K];
+#pragma unroll
+        for (int u = 0; u < K; ++u) { tag_at[u] = warp_tag + u * kInTagStride + (ready[u] ? q[u] : kInMaxQueues + (uint32_t)lane); *tag_at[u] = (uint8_t)lane; }
+        __syncwarp();
+#pragma unroll
+        for (int u = 0; u < K; ++u) tagged[u] = *reinterpret_cast<volatile uint8_t *>(tag_at[u]);
+        if (turn * (uint32_t)(K * 32) < qid_stride) {
+#pragma unroll
+            for (int u = 0; u < K; ++u)
+                if (valid[u]) qid_t[i[u]] = ready[u] ? (uint16_t)q[u] : (uint16_t)kInMaxQueues;
+        }
+        const bool heads_on = *reinterpret_cast<volatile uint32_t *>(s_heads_full) < R;
+        auto rest_of_turn = [&](auto heads_tag) {
+        constexpr bool HEADS = decltype(heads_tag)::value;
+        uint32_t rank1[K], pc[K], c0[K], c1[K], m_own[K], s_own[K], B[K];
+        bool last[K];
+        uint4 *pq[K];
+#pragma unroll
+        for (int u = 0; u < K; ++u) {
+            rank1[u] = 1u; last[u] = ready[u]; pc[u] = HEADS ? 1u : 0u;
+            m_own[u] = M[u]; s_own[u] = S[u];
+            const bool loser = tagged[u] != (uint32_t)lane;
+            if (__any_sync(0xffffffffu, loser)) {
+                if (loser) *tag_at[u] = (uint8_t)lane;
+                __syncwarp();
+                const uint32_t t2 = *reinterpret_cast<volatile uint8_t *>(tag_at[u]);
+                if (!__any_sync(0xffffffffu, loser && t2 != (uint32_t)lane)) {
+                    const uint32_t peer = loser ? tagged[u] : t2;                  // the lane itself when it has none
+                    const bool second = peer < (uint32_t)lane;
+                    const uint32_t mp_ = __shfl_sync(0xffffffffu, M[u], (int)peer), sp_ = __shfl_sync(0xffffffffu, S[u], (int)peer), gp_ = __shfl_sync(0xffffffffu, gn[u], (int)peer);
+                    if (second) { M[u] = max(mp_ + S[u], M[u]); S[u] += sp_; gn[u] += gp_; rank1[u] = 2u; }
+                    if (peer > (uint32_t)lane) last[u] = false;
+                    if (HEADS && peer != (uint32_t)lane) pc[u] = 2u;
+                } else {
+                    const unsigned peers = __match_any_sync(0xffffffffu, ready[u] ? q[u] : (0x10000u | (uint32_t)lane));
+                    const unsigned le = peers & le_mask;
+                    rank1[u] = (uint32_t)__popc(le);
+                    last[u] = ready[u] && (peers >> lane) == 1u;
+                    pc[u] = HEADS ? (uint32_t)__popc(peers) : 0u;
+                    const unsigned before = le & ~(1u << lane);
+                    int prev_l = before ? 31 - __clz((int)before) : -1;
+                    const uint32_t n_max = __reduce_max_sync(0xffffffffu, rank1[u]);
+                    for (uint32_t span = 1; span < n_max; span <<= 1) {
+                        const int src = prev_l >= 0 ? prev_l : lane;
+                        const uint32_t Se = __shfl_sync(0xffffffffu, S[u], src), Me = __shfl_sync(0xffffffffu, M[u], src), ge = __shfl_sync(0xffffffffu, gn[u], src);
+                        const int pe = __shfl_sync(0xffffffffu, prev_l, src);
+                        if (prev_l >= 0) { M[u] = max(Me + S[u], M[u]); S[u] += Se; gn[u] += ge; prev_l = pe; }
+                    }
+                }
+            }
+            pq[u] = qst + q[u];
+        }
+        // ---- the queue updates, in row order
+        if (turn > 0) row_wait_n(my_bar, M[0], S[0], pq[0], gn[0], last[0], M[K - 1], S[K - 1], pq[K - 1], gn[K - 1], last[K - 1]);
+#pragma unroll
+        for (int u = 0; u < K; ++u) {
+            const uint4 state = *pq[u];
+            B[u] = max(state.x + S[u], M[u]);
+            uint32_t inc = 0u;
+            if (HEADS) {
+                c0[u] = min(state.w & 15u, head_depth);
+                inc = min(pc[u], head_depth - c0[u]);
+                c1[u] = c0[u] + inc;
+            }
+            if (last[u]) *pq[u] = make_uint4(B[u], state.y + S[u], state.z + (gn[u] & ((1u << kNwCountShift) - 1u)), state.w + ((gn[u] >> kNwCountShift) << 4) + inc);
+            if (u + 1 < K) __syncwarp();
+        }
+        if (turn + 1 < turns) row_pass(next_bar);
+        // ---- results
+#pragma unroll
+        for (int u = 0; u < K; ++u) {
+            if (valid[u]) {
+                const uint32_t done = ready[u] ? B[u] + (uint32_t)max((int)xo[u], 0) : ri[u], waited = done - ri[u];
+                if (ready[u]) { b_time |= B[u]; r.max_done = max(r.max_done, done); }
+                r.stall += (long long)(unsigned long long)waited;
+                if (HEADS && ready[u]) {
+                    const uint32_t ci = c0[u] + rank1[u] - 1u;
+                    if (ci < head_depth) {
+                        InHead h; h.m = T0 + (int64_t)m_own[u]; h.s = (int64_t)s_own[u]; h.xo = xo[u]; h.idx = tile_begin + i[u];
+                        in_head[head_slot(tile, R, q[u], ci)] = h;
+                    }
+                    if (last[u] && c1[u] != c0[u] && c1[u] == head_depth) atomicAdd(s_heads_full, 1u);
+                }
+                __stcs(reinterpret_cast<long long *>(completion_t + i[u]), (long long)(T0 + (int64_t)(uint64_t)done));
+                __stcs(reinterpret_cast<long long *>(stall_t + i[u]), (long long)(unsigned long long)waited);
+            }
+        }
+        };
+        if (heads_on) rest_of_turn(std::true_type{}); else rest_of_turn(std::false_type{});
+      };
+      if ((turn * K + K) * 32u <= tile_len) whole_turn(std::true_type{}); else whole_turn(std::false_type{});
+    }
+    r.unsorted = b_sort >> 31; r.over = (b_time >> 31) | b_hi;
+    return r;
+}
+
 // DEBT = true (retention on): a modeled access with a batch index below the claim limit pays one refresh quantum (a page
 // read and a page program, scaled like any service, Eq. 3) before its own service; the streaming pass counts the
 // claims per die.
@@ -304,6 +587,67 @@ k_inorder_serve(const hbf_access_t *__restrict__ acc, uint64_t n, const __grid_c
     const uint64_t tile_begin = tile_first(tmap, tile);
     const uint64_t tile_end = tile_last(tmap, tile);
 
+    const uint32_t tile_len = tile_end > tile_begin ? (uint32_t)(tile_end - tile_begin) : 0u;   // inside a tile everything is indexed by 32-bit offsets from its first record (a batch is below 2^30 records)
+    const hbf_access_t *acc_t = acc + tile_begin;
+    int64_t *completion_t = completion + tile_begin, *stall_t = stall + tile_begin;
+    uint8_t *status_t = status ? status + tile_begin : nullptr;
+    uint16_t *qid_t = in_qid + (uint64_t)tile * qid_stride;   // the straggle pass filters the head of the tile by these
+    if (tid < 2) s_red[tid] = tid == 1 ? INT64_MIN : 0;
+    if (tid == 0) s_heads_full = 0u;
+    unsigned c_unsorted = (DEBT && ((uint64_t)quantum_ns >> 32)) ? 1u : 0u;   // (or a service, or a refresh quantum, of 2^32 ns or more)
+    long long sum_stall = 0, max_c = INT64_MIN;
+    long long t_native = 0, t_ready = 0, t_fault = 0;        // this thread's share of the tile's counts
+    bool narrow_done = false, again = false;
+    if constexpr (!RESERVE) {
+        // The 32-bit form serves the tile when the configuration allows it, the tile's times lie within 2^31 ns and its read
+        // granules sum below 2^32; should it turn out not to fit after all (a backlog), the 64-bit form below serves the tile again.
+        int64_t T0 = 0, T1 = -1;
+        if (tile_len) { T0 = acc_t[0].issue_ns; T1 = acc_t[tile_len - 1u].issue_ns; }
+        if (geom.narrow != 0u && q_ppm == 1000000 && T0 >= 0 && T0 < HBF_ISSUE_LIMIT - (1ll << 32) && T1 >= T0 && T1 - T0 < (1ll << 31) &&
+            (uint64_t)tile_len * geom.nw_gmax < (1ull << 32) && (uint64_t)quantum_ns < (1ull << (kNwServeBits - 1))) {
+            uint4 *q4 = reinterpret_cast<uint4 *>(qst);
+            unsigned over = 0;
+            for (uint32_t d = tid; d < n_dies * 7u; d += kInThreads) st_br_lo[d] = 0u;
+            for (uint32_t q = tid; q < kInMaxQueues; q += kInThreads) {
+                uint4 v = make_uint4(0u, 0u, 0u, 0u);
+                if (tile == 0u && q < R) {                   // the first tile knows its entering state: it is served exactly
+                    const int64_t b = busy[q] - T0;
+                    v.x = b > 0 ? (uint32_t)b : 0u;
+                    if (b >= (1ll << 31)) over = 1u;
+                }
+                q4[q] = v;
+            }
+            __syncthreads();
+            const NarrowSums nw = serve_narrow<DEBT>(geom, mp, mp_arg, acc_t, (uint32_t)tile_begin, tile_len, T0, q4, warp_tag, status_t, qid_t, qid_stride,
+                                                     completion_t, stall_t, in_head, tile, R, head_depth, &s_heads_full, st_br_lo, n_dies, claim_limit,
+                                                     (uint32_t)quantum_ns, ret, ret_row_shift);
+            if (__syncthreads_or((int)(over | nw.over)) == 0) {
+                narrow_done = true;
+                c_unsorted |= nw.unsorted;
+                if (tid == 0 && tile_begin > 0 && acc_t[-1].issue_ns > T0) c_unsorted = 1u;
+                sum_stall = nw.stall;
+                if (nw.max_done) max_c = T0 + (int64_t)(uint64_t)nw.max_done;      // (a modeled access ends after its tile's first issue time)
+                t_native = nw.native; t_fault = nw.fault; t_ready = (tid == 0 ? (long long)tile_len : 0ll) - t_native - t_fault;
+                longlong2 *out = reinterpret_cast<longlong2 *>(in_agg) + (uint64_t)tile * R;
+                for (uint32_t q = tid; q < R; q += kInThreads) {
+                    const uint4 v = q4[q];
+                    out[q] = make_longlong2((long long)(uint64_t)v.y, v.y ? T0 + (int64_t)(uint64_t)v.x : kNegInf);   // (no service time: no access)
+                    in_headcnt[(uint64_t)tile * R + q] = (uint8_t)(v.w & 15u);
+                }
+                for (uint32_t d = tid; d < n_dies; d += kInThreads) {              // a die's reads: the sums its queues carry
+                    unsigned long long g = 0, cnt = 0;
+                    for (uint32_t p = 0; p < geom.planes_q; ++p) { const uint4 v = q4[d * geom.planes_q + p]; g += v.z; cnt += v.w >> 4; }
+                    unsigned long long *gd = reinterpret_cast<unsigned long long *>(stats_stage + d);
+                    if (g) atomicAdd(&gd[1], g << geom.gran_shift_read);
+                    if (cnt) atomicAdd(&gd[4], cnt);
+                }
+            } else {
+                again = true;
+                if (tid == 0) s_heads_full = 0u;
+            }
+        }
+    }
+    if (!narrow_done) {
     for (uint32_t i = tid; i < kInMaxQueues; i += kInThreads) qst[i] = make_longlong2(kNegInf, 0);
     if (RESERVE) {
         __syncthreads();
@@ -316,22 +660,11 @@ k_inorder_serve(const hbf_access_t *__restrict__ acc, uint64_t n, const __grid_c
         }
     }
     uint32_t c_native = 0, c_ready = 0, c_valid = 0;         // per thread: far below 2^32 (a batch is below 2^30 records)
-    unsigned c_unsorted = (DEBT && ((uint64_t)quantum_ns >> 32)) ? 1u : 0u;   // (or a service, or a refresh quantum, of 2^32 ns or more)
-    long long sum_stall = 0, max_c = INT64_MIN;
-
-    if (tid < 2) s_red[tid] = tid == 1 ? INT64_MIN : 0;
-    if (tid == 0) s_heads_full = 0u;
     __syncthreads();
 
     // A warp's turn covers kInRows consecutive rows: their arithmetic interleaves, and their queue updates
     // follow one another inside one wait/pass pair.
     constexpr int K = kInRows;
-    // inside a tile everything is indexed by 32-bit offsets from the tile's first record (a batch is below 2^30 records)
-    const uint32_t tile_len = tile_end > tile_begin ? (uint32_t)(tile_end - tile_begin) : 0u;
-    const hbf_access_t *acc_t = acc + tile_begin;
-    int64_t *completion_t = completion + tile_begin, *stall_t = stall + tile_begin;
-    uint8_t *status_t = status ? status + tile_begin : nullptr;
-    uint16_t *qid_t = in_qid + (uint64_t)tile * qid_stride;   // the straggle pass filters the head of the tile by these
     const uint32_t rows = (tile_len + 31u) / 32u;
     const uint32_t turns = (rows + K - 1) / K;
     const unsigned le_mask = lanemask_lt() | (1u << lane);
@@ -398,7 +731,7 @@ k_inorder_serve(const hbf_access_t *__restrict__ acc, uint64_t n, const __grid_c
                 v[u].s += quantum_ns;
                 if (!RESERVE) atomicAdd(&st_claims[v[u].die], 1u);
             }
-            if (DEBT && !RESERVE && ready[u] && !v[u].op) {  // read disturb: the read's pages, on the block of its first page
+            if (DEBT && !RESERVE && ready[u] && !v[u].op && !again) {  // read disturb (counted already when the tile is served again): the read's pages, on the block of its first page
                 if (fast_on && ret.pow2 != 0u) {
                     // one range, powers of two all the way down: the block from shifts and masks (the general form below
                     // divides twice; it took the pass from 2.0 to 2.9 ms)
@@ -557,6 +890,7 @@ k_inorder_serve(const hbf_access_t *__restrict__ acc, uint64_t n, const __grid_c
       if ((turn * K + K) * 32u <= tile_len) whole_turn(std::true_type{}); else whole_turn(std::false_type{});
     }
 
+    t_native = c_native; t_ready = c_ready; t_fault = (long long)c_valid - c_ready - c_native;     // every other status is a fault
     __syncthreads();
     if (!RESERVE) {
         longlong2 *out = reinterpret_cast<longlong2 *>(in_agg) + (uint64_t)tile * R;
@@ -565,6 +899,9 @@ k_inorder_serve(const hbf_access_t *__restrict__ acc, uint64_t n, const __grid_c
             out[q] = make_longlong2(v.y >> 8, v.x);
             in_headcnt[(uint64_t)tile * R + q] = (uint8_t)(v.y & 0xff);
         }
+    }
+    }                                                        // (the 64-bit form)
+    if (!RESERVE) {
         for (uint32_t d = tid; d < n_dies; d += kInThreads) {
             unsigned long long *g = reinterpret_cast<unsigned long long *>(stats_stage + d);
             const unsigned long long br = ((unsigned long long)st_br_hi[d] << 32) | st_br_lo[d];
@@ -575,9 +912,9 @@ k_inorder_serve(const hbf_access_t *__restrict__ acc, uint64_t n, const __grid_c
             if (st_np[d]) atomicAdd(&g[5], (unsigned long long)st_np[d]);
             if (DEBT && st_claims[d]) atomicAdd(&die_claims[d], st_claims[d]);
         }
-        const unsigned long long w_native = (unsigned long long)warp_sum((long long)c_native);
-        const unsigned long long w_ready = (unsigned long long)warp_sum((long long)c_ready);
-        const unsigned long long w_fault = (unsigned long long)warp_sum((long long)(c_valid - c_ready - c_native));   // every other status is a fault
+        const unsigned long long w_native = (unsigned long long)warp_sum(t_native);
+        const unsigned long long w_ready = (unsigned long long)warp_sum(t_ready);        // (a warp's share may be negative: the sum over the tile counts)
+        const unsigned long long w_fault = (unsigned long long)warp_sum(t_fault);
         c_unsorted = __any_sync(0xffffffffu, c_unsorted);
         if (lane == 0) {
             if (w_native) atomicAdd(&ctrl->n_native, w_native);

@@ -1,0 +1,80 @@
+"""The 32-bit form of the in-order pass at the edges of what it holds, against the oracle, bit for bit: a gap in the stream and a
+backlog that do not fit 2^31 ns (the tile is served in the 64-bit form), accesses at the end of the range and larger than the
+form takes inline, one-way ranges, a record array that does not begin on a 16-byte boundary, refresh claims on top."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+from oracle import hbfo
+from paper_2609_09800_b200 import workloads as wl
+
+BASE, MIB = wl.RANGE_BASE, wl.MIB
+
+
+@pytest.fixture(scope="module")
+def hbf():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2609_09800_b200 import build, hbf as mod
+    build.build()
+    return mod
+
+
+def stream(kind, n, rng):
+    acc = np.zeros(n, hbfo.ACCESS_DTYPE)
+    acc["addr"] = BASE + rng.integers(0, 4096, n).astype(np.uint64) * np.uint64(65536)
+    acc["issue_ns"] = 1000 + np.sort(rng.integers(0, 40 * n, n))
+    acc["bytes"] = rng.choice([1, 64, 4096, 16384, 40_000], n)
+    acc["flags"] = rng.random(n) < 0.2
+    if kind == "gap":                                       # inside a tile, and again at its first record
+        acc["issue_ns"][n // 2 + 100:] += 5_000_000_000
+        acc["issue_ns"][n // 1024 * 1024:] += 3_000_000_000
+    elif kind == "backlog":                                 # 3 ms programs on one queue: a tile's 1,024 of them pass 2^31 ns
+        hot = np.arange(n) % 8 != 0
+        acc["addr"][hot] = BASE; acc["bytes"][hot] = 131_072; acc["flags"][hot] = 1
+    elif kind == "edge":                                    # the last 256 KiB of the range, and sizes around the inline bound
+        acc["bytes"] = rng.choice([64, 131_071, 131_072, 131_073, 200_000], n)
+        acc["addr"] = np.uint64(BASE + 256 * MIB) - acc["bytes"].astype(np.uint64) - (rng.integers(0, 1000, n).astype(np.uint64) if n else 0)
+    elif kind == "native":
+        out = rng.random(n) < 0.3
+        acc["addr"][out] = rng.integers(0, 1 << 40, int(out.sum())).astype(np.uint64)
+    return acc
+
+
+@pytest.mark.parametrize("n", [8_193, 20_001, 65_536])
+@pytest.mark.parametrize("kind", ["plain", "gap", "backlog", "edge", "native", "offset", "read only", "program only", "claims", "claims backlog"])
+def test_32_bit_form_matches_the_oracle(hbf, kind, n):
+    import torch
+    rng = np.random.default_rng(n)
+    prof = wl.load_profile("nominal", channels=8, dies=4, planes=2, page_bytes=16384, stripe_bytes=65536)
+    perms = {"read only": 1, "program only": 2}.get(kind, 3)
+    g, o = hbf.Context(prof), hbfo.Oracle(prof)
+    for c in (g, o):
+        c.register_range(BASE, 256 * MIB, perms, 0, 0, 3 * 65536)
+        if "claims" in kind:
+            c.enable_retention(pages_per_block=16, blocks_per_plane=32, blocks_per_zone=8, max_pec=3000, disturb_limit=0,
+                               l_ref_s=1.0, t_ref_c=40.0, ea_ev=1.04, accel=1.0, lead_threshold=0.5)
+            c.retention_advance(1_000_000_000, [40.0])      # every block becomes eligible: 32,768 quanta
+    acc = stream(kind.split()[-1] if "backlog" in kind else kind, n, rng)
+    if perms != 3:
+        acc["flags"] = perms - 1
+    for batch in range(2):                                  # the second one enters on the queues the first one left
+        _, c_o, s_o, st_o, ds_o = o.submit(acc)
+        if kind == "offset":
+            d = torch.zeros(3 * n + 1, dtype=torch.int64, device="cuda")
+            d[1:] = torch.from_numpy(acc.view(np.int64).reshape(-1)).cuda()
+            comp, stall = (torch.empty(n, dtype=torch.int64, device="cuda") for _ in range(2))
+            status = torch.empty(n, dtype=torch.uint8, device="cuda"); ds = torch.empty(g.n_dies * 6, dtype=torch.int64, device="cuda")
+            assert g.submit_batch(d[1:], n, comp, stall, status, ds) == 0 and g.last_result()["code"] == 0
+            c_g, s_g, st_g, ds_g = comp.cpu().numpy(), stall.cpu().numpy(), status.cpu().numpy(), ds.cpu().numpy().view(hbf.DIE_STATS_DTYPE)
+        else:
+            _, c_g, s_g, st_g, ds_g = g.submit_host(acc)
+        assert np.array_equal(st_g, st_o) and np.array_equal(c_g, c_o) and np.array_equal(s_g, s_o)
+        assert all(np.array_equal(ds_g[f], ds_o[f]) for f in hbfo.DIE_STATS_DTYPE.names)
+        assert np.array_equal(g.get_busy_until(), o.busy_until()) and g.last_result() == o.last_result()
+        if "claims" in kind:
+            bg, bo = g.retention_blocks(), o.retention_blocks()
+            assert np.array_equal(bg["disturb"], bo["disturb"]) and g.retention_totals() == o.retention_totals()
+        acc["issue_ns"] += 50_000
