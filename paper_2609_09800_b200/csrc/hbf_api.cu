@@ -473,7 +473,7 @@ int hbf_set_head_entries(hbf_ctx *c, uint32_t entries) {
 static int serve_records(hbf_ctx *c, SubmitArgs &a) {
     a.ranges = c->d_ranges; a.mp_dev = c->d_mp; a.mp = c->mp; a.state = c->d_state; a.ctrl = c->d_ctrl; a.result = c->d_result;
     a.busy = c->d_busy; a.busy_stage = c->d_busy_stage; a.pending = c->d_pending; a.stats_stage = c->d_stats_stage;
-    a.path = c->path; a.sm_count = c->sm_count; a.inorder_ok = c->inorder_ok ? 1 : 0;
+    a.path = a.paged ? (int32_t)HBF_PATH_INORDER : c->path; a.sm_count = c->sm_count; a.inorder_ok = c->inorder_ok ? 1 : 0;
     if (c->ranges.size() == 1) {
         const HostRange &r = c->ranges[0];
         a.fast.base = r.base; a.fast.length = r.length; a.fast.media_offset = r.media_offset; a.fast.perms = r.perms; a.fast.on = 1u;
@@ -622,28 +622,53 @@ int hbf_submit_batch_paged(hbf_ctx *c, const hbf_access_t *d_acc, uint64_t n, ui
     const int with_bus = c->d_bus_busy ? 1 : 0;
     const size_t need = paged_layout(n, capacity, c->mp.n_queues, &pw, d_workspace, with_bus);
     if (!d_workspace || workspace_bytes < need || (reinterpret_cast<uintptr_t>(d_workspace) & 255u)) return HBF_E_WORKSPACE;
-    // how many parts: the one point where the host waits for the device inside a submit
-    CK(launch_paged_count(d_acc, n, c->d_ranges, c->d_mp, pw, c->stream));
-    unsigned long long *h_total = reinterpret_cast<unsigned long long *>(c->h_result);     // pinned, free between calls
-    CK(cudaMemcpyAsync(h_total, pw.total, sizeof(unsigned long long), cudaMemcpyDeviceToHost, c->stream));
-    CK(cudaStreamSynchronize(c->stream));
-    const uint64_t total = *h_total;
-    if (total > capacity) return HBF_E_WORKSPACE;            // nothing has changed: the caller may come back with more room
     FastRange fast{};
     if (c->ranges.size() == 1) {
         const HostRange &r = c->ranges[0];
         fast.base = r.base; fast.length = r.length; fast.media_offset = r.media_offset; fast.perms = r.perms; fast.on = 1u;
     }
-    CK(launch_paged_expand(d_acc, n, c->d_ranges, c->d_mp, fast, c->mp.page_shift, capacity, pw, c->sm_count, c->stream));
+    // A batch the in-order kernels can take, with nothing on that looks at parts, is cut at stripe units only (the pages of
+    // one are served as one entry); should it turn out not to be in issue order after all, it is counted again by pages.
+    // (Small batches go by pages: their route has no form for such entries.)
+    bool by_unit = c->inorder_ok && (c->path == HBF_PATH_AUTO || c->path == HBF_PATH_INORDER) && !c->bin_ns && !c->d_bus_busy && !c->ret_on &&
+                   n > kInSmallMax && c->mp.stripe_shift < 31u;
+    // how many parts: the one point where the host waits for the device inside a submit
+    unsigned long long *h_total = reinterpret_cast<unsigned long long *>(c->h_result);     // pinned, free between calls
+    static_assert(sizeof(hbf_batch_result_t) >= kPagedTotals * sizeof(unsigned long long), "the totals fit where the result goes");
+    auto count = [&](bool unit) -> int {
+        CK(launch_paged_count(d_acc, n, c->d_ranges, c->d_mp, fast, c->mp, c->d_state, unit, pw, c->stream));
+        CK(cudaMemcpyAsync(h_total, pw.total, kPagedTotals * sizeof(unsigned long long), cudaMemcpyDeviceToHost, c->stream));
+        CK(cudaStreamSynchronize(c->stream));
+        return HBF_OK;
+    };
+    int rc = count(by_unit);
+    if (rc != HBF_OK) return rc;
+    if (by_unit && (h_total[kPagedUnsorted] || h_total[kPagedLong])) {
+        by_unit = false;
+        if ((rc = count(false)) != HBF_OK) return rc;
+    }
+    const uint64_t total = h_total[kPagedParts];
+    if ((by_unit ? (uint64_t)h_total[kPagedPages] : total) > capacity) return HBF_E_WORKSPACE;   // nothing has changed: the caller may come back with more room
+    c->prof_inorder = false; c->prof_submit = false;
+    if (by_unit && total == n) {                             // no access crosses a stripe unit: the caller's records are the list
+        SubmitArgs a{};
+        workspace_layout(n, c->mp.n_queues, &a.ws, pw.inner, 0);
+        a.acc = d_acc; a.n = n; a.completion = d_completion_ns; a.stall = d_stall_ns; a.status = d_status; a.die_stats = d_die_stats;
+        a.paged = 1;
+        if ((rc = serve_records(c, a)) != HBF_OK) return rc;
+        c->submitted = true;
+        return HBF_OK;
+    }
+    CK(launch_paged_offsets(n, pw, c->stream));
+    CK(launch_paged_expand(d_acc, n, c->d_ranges, c->d_mp, fast, by_unit ? c->mp.stripe_shift : c->mp.page_shift, capacity, pw, c->sm_count, c->stream));
     // the list of parts is a batch of records like any other: the ledger, the bus stage and retention, when on, see parts
     SubmitArgs a{};
     workspace_layout(total, c->mp.n_queues, &a.ws, pw.inner, with_bus);
     a.acc = pw.parts; a.n = total; a.completion = pw.part_completion; a.stall = pw.part_stall; a.status = pw.part_status;
     a.die_stats = d_die_stats;
-    c->prof_inorder = false; c->prof_submit = false;
+    a.paged = by_unit ? 1 : 0;
     a.ev = nullptr;
-    const int rc = serve_records(c, a);
-    if (rc != HBF_OK) return rc;
+    if ((rc = serve_records(c, a)) != HBF_OK) return rc;
     CK(launch_paged_join(d_acc, n, pw, c->d_result, d_completion_ns, d_stall_ns, d_status, c->sm_count, c->stream));
     c->submitted = true;
     return HBF_OK;

@@ -115,6 +115,7 @@ struct SubmitArgs {
     Workspace ws; int32_t path; int sm_count; int inorder_ok;
     FastRange fast;
     int binned;                          // the batch's energy goes to the time-bin ledger, not to the pending totals
+    int paged;                           // every record is an access inside one stripe unit whose pages are queued on their own (declared in issue order)
     int bus_on;                          // the channel-bus stage follows: array-done times must fit its 47-bit key field
     const unsigned long long *claim_limit;  // retention on: batch index below which a modeled access claims a refresh quantum
     uint32_t *die_claims;                   // retention on: [dies] claims of the batch
@@ -192,7 +193,7 @@ cudaError_t launch_queue_order(const BatchCtrl *ctrl, const Workspace &ws, uint3
 struct PagedWorkspace {
     unsigned long long *tile_sum;        // [tiles of 2,048 accesses] parts per tile, then exclusive offsets
     uint32_t *row_off;                   // [rows of 32 accesses] parts before the row within its tile
-    unsigned long long *total;           // parts of the batch
+    unsigned long long *total;           // [kPagedTotals] what the count found (PagedTotal)
     void *sums;                          // accesses served and their stall total
     uint32_t *part_first;                // [n + 1] first part of every access
     hbf_access_t *parts;                 // [capacity] the parts as access records
@@ -200,11 +201,14 @@ struct PagedWorkspace {
     void *inner; size_t inner_bytes;     // workspace of the ordinary path for `capacity` records
     size_t bytes;
 };
+// parts of the list; pages of all accesses; accesses issued before their predecessor; set when a service of a stripe unit's pages is too long for the in-order kernels
+enum PagedTotal { kPagedParts = 0, kPagedPages = 1, kPagedUnsorted = 2, kPagedLong = 3, kPagedTotals = 4 };
 size_t paged_layout(uint64_t n, uint64_t capacity, uint32_t n_queues, PagedWorkspace *pw, void *base, int with_bus = 0);
-cudaError_t launch_paged_count(const hbf_access_t *acc, uint64_t n, const RangeSnap *ranges, const ModelParams *mp_dev,
-                               const PagedWorkspace &pw, cudaStream_t st);
+cudaError_t launch_paged_count(const hbf_access_t *acc, uint64_t n, const RangeSnap *ranges, const ModelParams *mp_dev, const FastRange &fast,
+                               const ModelParams &mp, const DevState *state, bool by_unit, const PagedWorkspace &pw, cudaStream_t st);
+cudaError_t launch_paged_offsets(uint64_t n, const PagedWorkspace &pw, cudaStream_t st);
 cudaError_t launch_paged_expand(const hbf_access_t *acc, uint64_t n, const RangeSnap *ranges, const ModelParams *mp_dev,
-                                const FastRange &fast, uint32_t page_shift, uint64_t capacity, const PagedWorkspace &pw, int sm_count,
+                                const FastRange &fast, uint32_t cut_shift, uint64_t capacity, const PagedWorkspace &pw, int sm_count,
                                 cudaStream_t st);
 cudaError_t launch_paged_join(const hbf_access_t *acc, uint64_t n, const PagedWorkspace &pw, hbf_batch_result_t *result,
                               int64_t *completion, int64_t *stall, uint8_t *status, int sm_count, cudaStream_t st);

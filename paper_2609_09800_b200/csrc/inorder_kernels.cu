@@ -59,14 +59,14 @@ static_assert(kInWarps >= 2 && kInWarps <= 15, "every warp owns one of the hardw
 
 // One access, from its record: status, and for a modeled access its queue, die and service terms.
 // (the in-order path is only chosen when every transfer time fits 31 bits)
-struct Served { int st; uint32_t queue, die, op, xfer; int64_t s, cb; };
+struct Served { int st; uint32_t queue, die, op, xfer; int64_t s, cb; uint32_t parts; };
 // long_service (here and below): set when one access's service time reaches 2^long_bits ns.  The serve pass keeps a tile's
 // service-time sum per queue in 56 bits (55 and a sign); a tile has fewer than 2^22 records, so with every service below
 // 2^33 ns (8.6 s) the sum cannot overflow; with retention on a claimed refresh quantum is added to a service, and both
 // stay below 2^32.  A batch with a longer service is handed to the sort path like an unsorted one.
 __device__ __forceinline__ Served serve_terms(const RangeSnap &rs, const ModelParams &mp, uint64_t addr, int64_t issue,
                                               uint64_t bf, int64_t q_ppm, const Div64 &div_q, unsigned &long_service, int long_bits) {
-    Served r; r.queue = 0; r.die = 0; r.op = 0; r.s = 0; r.xfer = 0; r.cb = 0;
+    Served r; r.queue = 0; r.die = 0; r.op = 0; r.s = 0; r.xfer = 0; r.cb = 0; r.parts = 1;
     const uint32_t bytes = (uint32_t)bf, flags = (uint32_t)(bf >> 32);
     int g = 0;
     r.st = classify(rs, addr, issue, bytes, flags, &g);
@@ -84,7 +84,7 @@ __device__ __forceinline__ Served serve_terms(const RangeSnap &rs, const ModelPa
 // The same terms for the common configuration (one registered range, power-of-two geometry, no thermal
 // scaling in force, transfer table present): 32-bit arithmetic wherever the values allow it.
 __device__ __forceinline__ Served serve_terms_fast(const FastRange &f, const ModelParams &mp, uint64_t addr, int64_t issue, uint64_t bf) {
-    Served r; r.queue = 0; r.die = 0; r.op = 0; r.s = 0; r.xfer = 0; r.cb = 0;
+    Served r; r.queue = 0; r.die = 0; r.op = 0; r.s = 0; r.xfer = 0; r.cb = 0; r.parts = 1;
     const uint32_t bytes = (uint32_t)bf, flags = (uint32_t)(bf >> 32);
     const uint64_t rel = addr - f.base;                       // wraps to a huge value below the base
     if (bytes == 0u || (flags & ~1u) != 0u || (uint32_t)((uint64_t)issue >> 32) >= (1u << (kIssueBits - 32))) { r.st = HBF_ST_UNSUPPORTED; return r; }
@@ -125,6 +125,7 @@ struct __align__(16) FastGeom {
     uint32_t narrow, nw_bytes, nw_flag_lo, nw_flag_n;        // inline accesses: at most nw_bytes bytes, flags nw_flag_lo .. nw_flag_lo + nw_flag_n - 1
     uint32_t nw_gmax, nw_mul_read, nw_mul_prog, nw_add;      // most granules of an inline read; transfer = (granules * mul + add) / rate by
     uint32_t nw_magic, nw_shift, nw_chmul, nw_pad;           //   multiply-high; queues per channel
+    uint32_t nw_page_read, nw_page_prog, nw_page_gran, nw_pad2;   // page-granular submit: transfer of a whole page, read granules of one
 };
 // Bounds of the 32-bit form.  A service is below 2^26 ns, so that the services of a row's 32 lanes compose below 2^31; the
 // granules and the reads of an access fit 11 and 6 bits, so that a row's sums travel in one word (17 and 11 bits).
@@ -151,7 +152,7 @@ __host__ __device__ __forceinline__ FastGeom make_fast_geom(const FastRange &f, 
     g.nw_delta = f.media_offset - f.base; g.nw_chmul = mp.dies * g.planes_q; g.nw_pad = 0;
     g.nw_flag_lo = (f.perms & 1u) ? 0u : 1u; g.nw_flag_n = (f.perms & 3u) == 3u ? 2u : 1u;
     g.nw_mul_read = 1000u << (mp.read_gran_shift & 15u); g.nw_mul_prog = 1000u << (mp.prog_gran_shift & 15u);
-    g.narrow = 0u; g.nw_bytes = g.nw_gmax = g.nw_add = g.nw_magic = g.nw_shift = 0u; g.nw_lim = 0;
+    g.narrow = 0u; g.nw_bytes = g.nw_gmax = g.nw_add = g.nw_magic = g.nw_shift = 0u; g.nw_lim = 0; g.nw_page_read = g.nw_page_prog = g.nw_page_gran = g.nw_pad2 = 0u;
     const uint64_t d = mp.chan_bytes_per_us, t_max = (uint64_t)(mp.t_read_ns > mp.t_prog_ns ? mp.t_read_ns : mp.t_prog_ns);
     const uint64_t quantum = (uint64_t)mp.t_read_ns + (uint64_t)mp.t_prog_ns;   // (a claimed refresh quantum is added to a service)
     if (fast_geom_ok(f, mp) && d >= 2u && d < (1ull << 30) && mp.read_gran_shift <= 15u && mp.prog_gran_shift <= 15u && mp.page_shift <= 20u &&
@@ -165,8 +166,11 @@ __host__ __device__ __forceinline__ FastGeom make_fast_geom(const FastRange &f, 
             uint32_t l = 0;
             while ((1ull << l) < d) ++l;
             g.narrow = 1u; g.nw_bytes = (uint32_t)most; g.nw_lim = f.length - most;
-            g.nw_gmax = (uint32_t)((most + (1ull << mp.read_gran_shift) - 1u) >> mp.read_gran_shift);
+            g.nw_gmax = (uint32_t)((most + (1ull << mp.read_gran_shift) - 1u) >> mp.read_gran_shift) + kNwPages;   // (every part of a paged access may round up)
             g.nw_add = (uint32_t)d - 1u; g.nw_magic = (uint32_t)((1ull << (31 + l)) / d + 1u); g.nw_shift = l - 1u;
+            const uint64_t page = 1ull << mp.page_shift, gr = (1ull << mp.read_gran_shift) - 1u, gp = (1ull << mp.prog_gran_shift) - 1u;
+            g.nw_page_read = (uint32_t)((((page + gr) & ~gr) * 1000u + d - 1u) / d); g.nw_page_prog = (uint32_t)((((page + gp) & ~gp) * 1000u + d - 1u) / d);
+            g.nw_page_gran = (uint32_t)((page + gr) >> mp.read_gran_shift);
         }
     }
     return g;
@@ -176,7 +180,7 @@ __host__ __device__ __forceinline__ FastGeom make_fast_geom(const FastRange &f, 
 // about 47 instructions per row of 32 accesses, measured.)
 __device__ __forceinline__ Served serve_terms_geom(const FastGeom &g, const ModelParams &mp, uint64_t addr, int64_t issue, uint64_t bf,
                                                   int64_t q_ppm, const Div64 &div_q, unsigned &long_service, int long_bits) {
-    Served r;
+    Served r; r.parts = 1;
     const uint32_t bytes = (uint32_t)bf, flags = (uint32_t)(bf >> 32);
     const uint64_t rel = addr - g.base;                       // wraps to a huge value below the base
     const uint32_t op = flags & 1u;
@@ -213,6 +217,46 @@ __device__ __forceinline__ Served serve_terms_geom(const FastGeom &g, const Mode
         if ((uint64_t)r.s >> long_bits) long_service = 1u;
     }
     return r;
+}
+// ---- page-granular submit, without the list of parts ----------------------------------------------------------------
+// The pages of an access that stays inside one stripe unit lie on one plane, so its parts are consecutive requests of one
+// queue: together they are one map B -> max(B + S, M) again, and the access ends with the latest of them.  With k parts of
+// service s each and transfers x_1, x, ..., x, x_k (the first and the last part may be shorter than a page):
+//   reads     all parts arrive when the access is issued: M = issue + k s; part j is done k - j services before the last, so the
+//             access ends max(x_k, x - s, x_1 - (k - 1) s) after the last service
+//   programs  part j arrives x_j after the issue: M = issue + max(x_1 + k s, x + (k - 1) s, x_k + s), S = k s; it ends with the
+//             last service
+// so an access is served as one entry with these terms in the place of its own (xfer: what follows the service of a read, or
+// M - S - issue of a program).  Bytes are charged and operations counted per part.
+__device__ __forceinline__ void paged_terms(const ModelParams &mp, uint64_t off, uint32_t bytes, int64_t q_ppm, const Div64 &div_q,
+                                            unsigned &long_service, int long_bits, Served &r) {
+    const uint64_t page = 1ull << mp.page_shift, in_page = off & (page - 1ull);
+    const uint64_t k = (in_page + bytes + page - 1ull) >> mp.page_shift;
+    const uint64_t head = min((uint64_t)bytes, page - in_page), tail = in_page + bytes - (k - 1ull) * page;      // (k == 1: the head is the access)
+    const uint64_t gm = (1ull << (r.op ? mp.prog_gran_shift : mp.read_gran_shift)) - 1ull;
+    auto charged = [&](uint64_t b) { return (b + gm) & ~gm; };
+    auto transfer = [&](uint64_t cb) { return (int64_t)div64(cb * 1000ull + mp.chan_bytes_per_us - 1ull, mp.div_chan); };
+    const int64_t t = r.op ? mp.t_prog_ns : mp.t_read_ns;
+    const int64_t s1 = q_ppm == 1000000 ? t : (int64_t)div64((uint64_t)t * 1000000ull + (uint64_t)q_ppm - 1ull, div_q);
+    r.parts = (uint32_t)k;
+    r.s = (int64_t)k * s1;
+    if ((uint64_t)r.s >> long_bits) long_service = 1u;
+    const int64_t xh = transfer(charged(head));
+    r.cb = (int64_t)charged(head);
+    if (k == 1ull) { r.xfer = (uint32_t)xh; return; }
+    const int64_t xp = transfer(charged(page)), xt = transfer(charged(tail));
+    r.cb += (int64_t)(charged(tail) + (k - 2ull) * charged(page));
+    const int64_t n1 = (int64_t)k - 1;
+    int64_t x = r.op ? max(xh, xt - n1 * s1) : max(xt, xh - n1 * s1);
+    if (k > 2ull) x = max(x, xp - s1);
+    r.xfer = (uint32_t)x;
+}
+// media offset of a modeled access
+__device__ __forceinline__ uint64_t media_offset_of(const RangeSnap &rs, const FastRange &f, bool one, uint64_t addr, int64_t issue, uint64_t bf) {
+    if (one) return f.media_offset + (addr - f.base);
+    int g = 0;
+    classify(rs, addr, issue, (uint32_t)bf, (uint32_t)(bf >> 32), &g);
+    return rs.media_offset[g] + (addr - rs.base[g]);
 }
 // The first kInHead accesses of every (tile, queue), as the serve pass saw them: all the fix-up needs in the common case.
 // (Six, measured on the capacity stream at loads 0.3 to 0.9: eight cost 2.5 % more at every load for the table's traffic
@@ -283,7 +327,7 @@ __device__ __forceinline__ void row_wait_n(int id, uint32_t m, uint32_t s, const
                  "r"(m2), "r"(s2), "l"(pq2), "r"(gn2), "r"((int)last2) : "memory");
 }
 
-template <bool DEBT>
+template <bool DEBT, bool PAGED>
 __device__ __forceinline__ NarrowSums serve_narrow(const FastGeom &geom, const ModelParams &mp, const ModelParams &mp_arg, const hbf_access_t *acc_t, const uint32_t tile_begin,
                                                    const uint32_t tile_len, const int64_t T0, uint4 *qst, uint8_t *warp_tag, uint8_t *status_t,
                                                    uint16_t *qid_t, const uint32_t qid_stride, int64_t *completion_t, int64_t *stall_t,
@@ -356,13 +400,31 @@ __device__ __forceinline__ NarrowSums serve_narrow(const FastGeom &geom, const M
                     const uint32_t g = (bytes + ((1u << geom.gran_shift_read) - 1u)) >> geom.gran_shift_read;
                     S[u] = npages * geom.t_read; xo[u] = nw_transfer(geom, g, geom.nw_mul_read);
                     gn[u] = g | (1u << kNwCountShift);
+                    if (PAGED && npages > 1u) {              // (see paged_terms)
+                        const uint32_t head = geom.page_mask + 1u - in_page, tail = in_page + bytes - (npages - 1u) * (geom.page_mask + 1u), gm = (1u << geom.gran_shift_read) - 1u;
+                        const uint32_t gh = (head + gm) >> geom.gran_shift_read, gt = (tail + gm) >> geom.gran_shift_read;
+                        const int32_t s1 = (int32_t)geom.t_read;
+                        int32_t x = max((int32_t)nw_transfer(geom, gt, geom.nw_mul_read), (int32_t)nw_transfer(geom, gh, geom.nw_mul_read) - (int32_t)(npages - 1u) * s1);
+                        if (npages > 2u) x = max(x, (int32_t)geom.nw_page_read - s1);
+                        xo[u] = (uint32_t)x;
+                        gn[u] = (gh + gt + (npages - 2u) * geom.nw_page_gran) | (npages << kNwCountShift);
+                    }
                     M[u] = ri[u] + S[u];
                 } else {                                     // a program: its data is transferred first; bytes and count by atomics
-                    const uint32_t g = (bytes + ((1u << geom.gran_shift_prog) - 1u)) >> geom.gran_shift_prog, xf = nw_transfer(geom, g, geom.nw_mul_prog);
-                    S[u] = npages * geom.t_prog; xo[u] = xf | 0x80000000u;
+                    uint32_t g = (bytes + ((1u << geom.gran_shift_prog) - 1u)) >> geom.gran_shift_prog, xf = nw_transfer(geom, g, geom.nw_mul_prog);
+                    S[u] = npages * geom.t_prog;
+                    if (PAGED && npages > 1u) {
+                        const uint32_t head = geom.page_mask + 1u - in_page, tail = in_page + bytes - (npages - 1u) * (geom.page_mask + 1u), gm = (1u << geom.gran_shift_prog) - 1u;
+                        const uint32_t gh = (head + gm) >> geom.gran_shift_prog, gt = (tail + gm) >> geom.gran_shift_prog;
+                        const int32_t s1 = (int32_t)geom.t_prog;
+                        int32_t x = max((int32_t)nw_transfer(geom, gh, geom.nw_mul_prog), (int32_t)nw_transfer(geom, gt, geom.nw_mul_prog) - (int32_t)(npages - 1u) * s1);
+                        if (npages > 2u) x = max(x, (int32_t)geom.nw_page_prog - s1);
+                        xf = (uint32_t)x; g = gh + gt + (npages - 2u) * ((geom.page_mask + 1u + gm) >> geom.gran_shift_prog);
+                    }
+                    xo[u] = xf | 0x80000000u;
                     M[u] = ri[u] + xf + S[u];
                     const uint32_t die = geom.planes_q == 1u ? q[u] : q[u] >> mp_arg.plane_shift, lo = g << geom.gran_shift_prog;
-                    atomicAdd(&st_np[die], 1u);
+                    atomicAdd(&st_np[die], PAGED ? npages : 1u);
                     const uint32_t old = atomicAdd(&st_bp_lo[die], lo);
                     if (old + lo < old) atomicAdd(&st_bp_hi[die], 1u);
                 }
@@ -372,7 +434,8 @@ __device__ __forceinline__ NarrowSums serve_narrow(const FastGeom &geom, const M
                 }
             } else if (valid[u]) {                           // near the range's end, large, or not modeled
                 unsigned lng = 0;
-                const Served v = serve_terms_geom(geom, mp, addr[u], issue[u], bf[u], 1000000, Div64{}, lng, (int)kNwServeBits - 1);
+                Served v = serve_terms_geom(geom, mp, addr[u], issue[u], bf[u], 1000000, Div64{}, lng, (int)kNwServeBits - 1);
+                if (PAGED && v.st == HBF_ST_READY) paged_terms(mp, off, bytes, 1000000, Div64{}, lng, (int)kNwServeBits - 1, v);
                 st = (uint32_t)v.st;
                 if (v.st == HBF_ST_READY) {
                     ready[u] = true; q[u] = v.queue;
@@ -380,7 +443,7 @@ __device__ __forceinline__ NarrowSums serve_narrow(const FastGeom &geom, const M
                     S[u] = (uint32_t)v.s; xo[u] = v.xfer | (v.op << 31);
                     const uint32_t lo = (uint32_t)v.cb, hi = (uint32_t)((uint64_t)v.cb >> 32);
                     uint32_t *plo = v.op ? st_bp_lo : st_br_lo, *phi = v.op ? st_bp_hi : st_br_hi;
-                    atomicAdd(v.op ? &st_np[v.die] : &st_nr[v.die], 1u);
+                    atomicAdd(v.op ? &st_np[v.die] : &st_nr[v.die], v.parts);
                     const uint32_t old = atomicAdd(&plo[v.die], lo), carry = hi + ((old + lo) < old ? 1u : 0u);
                     if (carry) atomicAdd(&phi[v.die], carry);
                     if (DEBT && tile_begin + i[u] < claim_limit) { S[u] += quantum_ns; atomicAdd(&st_claims[v.die], 1u); }
@@ -507,7 +570,8 @@ __device__ __forceinline__ NarrowSums serve_narrow(const FastGeom &geom, const M
 // DEBT = true (retention on): a modeled access with a batch index below the claim limit pays one refresh quantum (a page
 // read and a page program, scaled like any service, Eq. 3) before its own service; the streaming pass counts the
 // claims per die.
-template <bool RESERVE, bool DEBT>
+// PAGED = true: the page-granular submit of accesses that stay inside one stripe unit each (paged_terms).
+template <bool RESERVE, bool DEBT, bool PAGED>
 __global__ void __launch_bounds__(kInThreads, kInBlocksPerSM)
 k_inorder_serve(const hbf_access_t *__restrict__ acc, uint64_t n, const __grid_constant__ InTileMap tmap, const RangeSnap *__restrict__ ranges_g,
                 const __grid_constant__ ModelParams mp_arg, const __grid_constant__ FastRange fast_arg, BatchCtrl *ctrl, uint8_t *__restrict__ status, int64_t *__restrict__ in_agg,
@@ -618,7 +682,7 @@ k_inorder_serve(const hbf_access_t *__restrict__ acc, uint64_t n, const __grid_c
                 q4[q] = v;
             }
             __syncthreads();
-            const NarrowSums nw = serve_narrow<DEBT>(geom, mp, mp_arg, acc_t, (uint32_t)tile_begin, tile_len, T0, q4, warp_tag, status_t, qid_t, qid_stride,
+            const NarrowSums nw = serve_narrow<DEBT, PAGED>(geom, mp, mp_arg, acc_t, (uint32_t)tile_begin, tile_len, T0, q4, warp_tag, status_t, qid_t, qid_stride,
                                                      completion_t, stall_t, in_head, tile, R, head_depth, &s_heads_full, st_br_lo, n_dies, claim_limit,
                                                      (uint32_t)quantum_ns, ret, ret_row_shift);
             if (__syncthreads_or((int)(over | nw.over)) == 0) {
@@ -727,6 +791,7 @@ k_inorder_serve(const hbf_access_t *__restrict__ acc, uint64_t n, const __grid_c
                 v[u] = fast_on ? serve_terms_geom(geom, mp, addr[u], issue[u], bf[u], q_ppm, div_q, c_unsorted, DEBT ? 32 : 33)
                                  : serve_terms(rs, mp, addr[u], issue[u], bf[u], q_ppm, div_q, c_unsorted, DEBT ? 32 : 33);
             ready[u] = valid[u] && v[u].st == HBF_ST_READY;
+            if (PAGED && ready[u]) paged_terms(mp, media_offset_of(rs, fast_range, fast_on, addr[u], issue[u], bf[u]), (uint32_t)bf[u], q_ppm, div_q, c_unsorted, 33, v[u]);
             if (DEBT && ready[u] && tile_begin + i[u] < claim_limit) {
                 v[u].s += quantum_ns;
                 if (!RESERVE) atomicAdd(&st_claims[v[u].die], 1u);
@@ -743,9 +808,7 @@ k_inorder_serve(const hbf_access_t *__restrict__ acc, uint64_t n, const __grid_c
                     const uint32_t pl = (uint32_t)(off >> (geom.stripe_shift + geom.chdie_shift)) & geom.plane_mask;
                     atomicAdd(&ret.disturb[((v[u].die << mp_arg.plane_shift) + pl) * ret.bpp + (blk & (ret.bpp - 1u))], npages);
                 } else {
-                    uint64_t off;
-                    if (fast_on) off = fast_range.media_offset + (addr[u] - fast_range.base);
-                    else { int g = 0; classify(rs, addr[u], issue[u], (uint32_t)bf[u], (uint32_t)(bf[u] >> 32), &g); off = rs.media_offset[g] + (addr[u] - rs.base[g]); }
+                    const uint64_t off = media_offset_of(rs, fast_range, fast_on, addr[u], issue[u], bf[u]);
                     const uint32_t page_mask = (1u << mp.page_shift) - 1u;
                     const uint32_t npages = (uint32_t)(((uint64_t)((uint32_t)off & page_mask) + (uint32_t)bf[u] + page_mask) >> mp.page_shift);
                     atomicAdd(&ret.disturb[ret_block_of(mp, ret, off)], npages);
@@ -782,7 +845,7 @@ k_inorder_serve(const hbf_access_t *__restrict__ acc, uint64_t n, const __grid_c
                         // granules in one word and sends oversized accesses to the 64-bit totals measured slower)
                         const uint32_t lo = (uint32_t)v[u].cb, hi = (uint32_t)((uint64_t)v[u].cb >> 32);
                         uint32_t *plo = v[u].op ? st_bp_lo : st_br_lo, *phi = v[u].op ? st_bp_hi : st_br_hi;
-                        atomicAdd(v[u].op ? &st_np[v[u].die] : &st_nr[v[u].die], 1u);
+                        atomicAdd(v[u].op ? &st_np[v[u].die] : &st_nr[v[u].die], PAGED ? v[u].parts : 1u);
                         const uint32_t old = atomicAdd(&plo[v[u].die], lo);
                         const uint32_t carry = hi + ((old + lo) < old ? 1u : 0u);
                         if (carry) atomicAdd(&phi[v[u].die], carry);
@@ -1032,10 +1095,13 @@ __device__ __forceinline__ uint32_t fast_queue(const FastRange &f, const ModelPa
 // The general form of the terms (several ranges, any geometry, thermal scaling), kept out of line here: this kernel runs
 // nearly straight through once per block, so what it costs is fetching its instructions, and the common configuration
 // never takes this path.
+template <bool PAGED>
 __device__ __noinline__ Served serve_terms_general(const RangeSnap &rs, const ModelParams &mp, uint64_t addr, int64_t issue, uint64_t bf,
                                                    int64_t q_ppm, Div64 div_q) {
     unsigned ignored = 0;                                    // (the serve pass has already vetted every service time)
-    return serve_terms(rs, mp, addr, issue, bf, q_ppm, div_q, ignored, 33);
+    Served r = serve_terms(rs, mp, addr, issue, bf, q_ppm, div_q, ignored, 33);
+    if (PAGED && r.st == HBF_ST_READY) paged_terms(mp, media_offset_of(rs, FastRange{}, false, addr, issue, bf), (uint32_t)bf, q_ppm, div_q, ignored, 33, r);
+    return r;
 }
 
 struct FixRun { int64_t B, Bs; long long dstall, max_c; bool settled; };
@@ -1063,7 +1129,7 @@ constexpr int kInStrQueuesPerThread = (kInMaxQueues + kInStrThreads - 1) / kInSt
 static_assert(kInStrQChunk <= 65536, "a kept record's position in its chunk is stored in 16 bits");
 static_assert(kInQidPrefix % kInStrQChunk == 0 && kInStrQItems == 32, "a thread's 32 queue numbers are four 16-byte loads");
 
-template <bool DEBT>
+template <bool DEBT, bool PAGED>
 __global__ void __launch_bounds__(kInStrThreads, 2)
 k_inorder_fixstraggle(const hbf_access_t *__restrict__ acc, uint64_t n, const __grid_constant__ InTileMap tmap,
                       const RangeSnap *__restrict__ ranges_g, const __grid_constant__ ModelParams mp_arg,
@@ -1176,7 +1242,7 @@ k_inorder_fixstraggle(const hbf_access_t *__restrict__ acc, uint64_t n, const __
     const int64_t q_ppm = ctrl->q_ppm;
     const Div64 div_q = ctrl->div_q;
     const bool one_range = fast_arg.on != 0u && mp_arg.pow2_geom != 0u;
-    const bool fast_terms = one_range && mp_arg.xfer_tab_max_cb != 0u && q_ppm == 1000000;
+    const bool fast_terms = !PAGED && one_range && mp_arg.xfer_tab_max_cb != 0u && q_ppm == 1000000;
     const uint64_t claim_limit = DEBT ? *claim_limit_p : 0ull;     // as in the serve pass
     const int64_t quantum_ns = !DEBT ? 0 : q_ppm == 1000000 ? mp_arg.t_read_ns + mp_arg.t_prog_ns
         : (int64_t)div64((uint64_t)(mp_arg.t_read_ns + mp_arg.t_prog_ns) * 1000000ull + (uint64_t)q_ppm - 1ull, div_q);
@@ -1214,7 +1280,7 @@ k_inorder_fixstraggle(const hbf_access_t *__restrict__ acc, uint64_t n, const __
             const uint32_t slot = (uint32_t)(k * kInStrThreads + tid);
             if (slot < wn) {
                 Served v = fast_terms ? serve_terms_fast(fast_range, mp, r_addr[k], r_issue[k], r_bf[k])
-                                      : serve_terms_general(rs, mp, r_addr[k], r_issue[k], r_bf[k], q_ppm, div_q);
+                                      : serve_terms_general<PAGED>(rs, mp, r_addr[k], r_issue[k], r_bf[k], q_ppm, div_q);
                 if (DEBT && tile_begin + cb + r_e[k] < claim_limit) v.s += quantum_ns;
                 ent_as[slot] = make_longlong2(r_issue[k], v.s);
                 ent_pq[slot] = make_uint2(v.xfer | (v.op << 31), v.queue | (r_e[k] << 16));
@@ -1260,7 +1326,7 @@ k_inorder_fixstraggle(const hbf_access_t *__restrict__ acc, uint64_t n, const __
                         const uint32_t q = fast_queue(fast_range, mp, addr);
                         k = q != 0xffffffffu && open[q] != 0;
                     } else {
-                        const Served v = serve_terms_general(rs, mp, addr, (int64_t)__ldg(rec + 1), __ldg(rec + 2), q_ppm, div_q);
+                        const Served v = serve_terms_general<PAGED>(rs, mp, addr, (int64_t)__ldg(rec + 1), __ldg(rec + 2), q_ppm, div_q);
                         k = v.st == HBF_ST_READY && open[v.queue] != 0;
                     }
                     keep |= k ? 1u << j : 0u;
@@ -1601,7 +1667,7 @@ k_small_serve(const hbf_access_t *__restrict__ acc, const uint32_t n, const Rang
                 const bool writer = (i / kInSmallThreads) % n_slices == slice;       // the block that writes what is not queue work
                 if (r_issue[k] < r_prev[k]) c_unsorted = 1u;
                 const Served v = fast_terms ? serve_terms_fast(fast_range, mp, r_addr[k], r_issue[k], r_bf[k])
-                                            : serve_terms_general(rs, mp, r_addr[k], r_issue[k], r_bf[k], q_ppm, div_q);
+                                            : serve_terms_general<false>(rs, mp, r_addr[k], r_issue[k], r_bf[k], q_ppm, div_q);
                 if (status && writer) status[i] = (uint8_t)v.st;
                 if (v.st == HBF_ST_READY) {
                     ++c_ready;
@@ -1763,7 +1829,7 @@ size_t inorder_head_bytes(uint64_t tiles, uint32_t n_queues) { return tiles * n_
 
 cudaError_t launch_inorder(const SubmitArgs &a, cudaStream_t st) {
     const uint64_t n = a.n;
-    if (inorder_small_batch(n)) {                            // one launch, a block per 64 queues
+    if (inorder_small_batch(n) && !a.paged) {                // one launch, a block per 64 queues
         const bool debt = a.claim_limit != nullptr;
         const size_t smem = inorder_small_smem();
         cudaError_t e = ensure_dyn_smem((const void *)k_small_serve<false>, smem);
@@ -1821,15 +1887,15 @@ cudaError_t launch_inorder(const SubmitArgs &a, cudaStream_t st) {
     const uint32_t R = a.mp.n_queues, nd = a.mp.n_dies;
     const size_t smem_serve = inorder_serve_smem(nd), smem_str = inorder_straggle_smem();
     {
-        const void *serve_fns[4] = {(const void *)k_inorder_serve<false, false>, (const void *)k_inorder_serve<true, false>,
-                                    (const void *)k_inorder_serve<false, true>, (const void *)k_inorder_serve<true, true>};
+        const void *serve_fns[6] = {(const void *)k_inorder_serve<false, false, false>, (const void *)k_inorder_serve<true, false, false>,
+                                    (const void *)k_inorder_serve<false, true, false>, (const void *)k_inorder_serve<true, true, false>,
+                                    (const void *)k_inorder_serve<false, false, true>, (const void *)k_inorder_serve<true, false, true>};
         for (const void *f : serve_fns) { cudaError_t e = ensure_dyn_smem(f, smem_serve); if (e != cudaSuccess) return e; }
         cudaError_t e = ensure_dyn_smem((const void *)k_inorder_scan, 0);
         if (e != cudaSuccess) return e;
-        e = ensure_dyn_smem((const void *)k_inorder_fixstraggle<false>, smem_str);
-        if (e != cudaSuccess) return e;
-        e = ensure_dyn_smem((const void *)k_inorder_fixstraggle<true>, smem_str);
-        if (e != cudaSuccess) return e;
+        const void *fix_fns[3] = {(const void *)k_inorder_fixstraggle<false, false>, (const void *)k_inorder_fixstraggle<true, false>,
+                                  (const void *)k_inorder_fixstraggle<false, true>};
+        for (const void *f : fix_fns) { e = ensure_dyn_smem(f, smem_str); if (e != cudaSuccess) return e; }
     }
     InTile *tiles = reinterpret_cast<InTile *>(a.ws.in_tile);
     InHead *heads = reinterpret_cast<InHead *>(a.ws.in_head);
@@ -1837,8 +1903,9 @@ cudaError_t launch_inorder(const SubmitArgs &a, cudaStream_t st) {
     const uint32_t qid_stride = (uint32_t)std::min<uint64_t>(tile_records, kInQidPrefix);
     if ((uint64_t)n_tiles * qid_stride > inorder_qid_entries(n)) return cudaErrorInvalidValue;
     auto serve = [&](bool reserve) {
-        auto k = reserve ? (debt ? k_inorder_serve<true, true> : k_inorder_serve<true, false>)
-                         : (debt ? k_inorder_serve<false, true> : k_inorder_serve<false, false>);
+        auto k = a.paged ? (reserve ? k_inorder_serve<true, false, true> : k_inorder_serve<false, false, true>)
+               : reserve ? (debt ? k_inorder_serve<true, true, false> : k_inorder_serve<true, false, false>)
+                         : (debt ? k_inorder_serve<false, true, false> : k_inorder_serve<false, false, false>);
         k<<<n_tiles, kInThreads, smem_serve, st>>>(a.acc, n, tmap, a.ranges, a.mp, a.fast, a.ctrl, a.status, a.ws.in_agg,
                                                    a.stats_stage, a.completion, a.stall, a.ws.in_bin, tiles, heads, a.ws.in_headcnt,
                                                    a.busy, a.claim_limit, a.die_claims, debt ? *a.ret : RetDev{}, a.ws.in_qid, qid_stride,
@@ -1847,7 +1914,7 @@ cudaError_t launch_inorder(const SubmitArgs &a, cudaStream_t st) {
     serve(false);
     k_inorder_scan<<<(R + kInScanQueues - 1) / kInScanQueues, dim3(kInScanQueues, kInScanChunks), 0, st>>>(
         a.ctrl, a.mp_dev, n_tiles, a.ws.in_agg, a.ws.in_bin, a.busy, a.busy_stage, a.stats_stage, a.path == HBF_PATH_INORDER ? 1 : 0);
-    (debt ? k_inorder_fixstraggle<true> : k_inorder_fixstraggle<false>)<<<n_tiles, kInStrThreads, smem_str, st>>>(
+    (a.paged ? k_inorder_fixstraggle<false, true> : debt ? k_inorder_fixstraggle<true, false> : k_inorder_fixstraggle<false, false>)<<<n_tiles, kInStrThreads, smem_str, st>>>(
         a.acc, n, tmap, a.ranges, a.mp, a.fast, a.ctrl, a.ws.in_bin, heads, a.ws.in_headcnt, a.completion, a.stall, tiles,
         a.claim_limit, a.ws.in_qid, qid_stride, depth, bal ? bal->dev : nullptr);
     serve(true);

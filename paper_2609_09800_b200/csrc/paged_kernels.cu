@@ -1,9 +1,12 @@
 // Page-granular submit: every page a modeled access touches becomes a request of its own (decoded by its own
 // first byte, one page of array time, the transfer of its own bytes), and the access completes with its last
 // part.  The paper's back end is a page-based flash simulator; the splitting rule itself is this library's.
+// A batch in issue order, with nothing switched on that looks at parts (ledger, bus, retention), is not cut into pages at all:
+// the pages of one stripe unit lie on one queue, and the in-order kernels serve them as one entry (paged_terms in
+// inorder_kernels.cu).  It is cut at stripe units only, and where no access crosses one, its own records are served.
 //   count   parts per access (1 for an access that is not modeled), summed per row of 32 accesses and per tile of 64 rows;
-//           a row's parts-before-it within its tile are kept
-//   scan    exclusive scan of the tile sums by one block; the total goes back to the host, which sizes the rest
+//           a row's parts-before-it within its tile are kept.  By stripe unit it also finds the batch's pages and whether it is in order
+//   scan    exclusive scan of the tile sums by one block; the totals go back to the host, which sizes the rest
 //   expand  a warp per row, no block-wide step: the warp reads its 32 records, knows where its parts begin (tile offset
 //           + row offset), and writes them, in (access, part) order, as ordinary access records
 //   serve   the ordinary submit path runs on the part records (they keep the batch's issue order)
@@ -19,65 +22,112 @@ constexpr int kPgItems = 8;
 constexpr int kPgTile = kPgThreads * kPgItems;
 constexpr int kPgRows = kPgTile / 32;                    // rows of 32 consecutive accesses per tile
 
-// parts of one access: its pages when it is modeled, one (the record itself) otherwise
-__device__ __forceinline__ uint32_t parts_of(const RangeSnap &rs, const ModelParams &mp, const uint64_t *rec, uint64_t *first_bytes) {
+// parts of one access: the pieces of 1 << shift bytes (pages, or stripe units) it touches when it is modeled, one (the record
+// itself) otherwise
+__device__ __forceinline__ uint32_t parts_of(const RangeSnap &rs, uint32_t shift, const uint64_t *rec, uint64_t *first_bytes, uint32_t page_shift = 0, uint32_t *pages = nullptr) {
     const uint64_t addr = __ldg(rec), bf = __ldg(rec + 2);
     const int64_t issue = (int64_t)__ldg(rec + 1);
     const uint32_t bytes = (uint32_t)bf, flags = (uint32_t)(bf >> 32);
     int g = 0;
     *first_bytes = bytes;
+    if (pages) *pages = 1u;
     if (classify(rs, addr, issue, bytes, flags, &g) != HBF_ST_READY) return 1u;
     const uint64_t off = rs.media_offset[g] + (addr - rs.base[g]);
-    const uint64_t page = 1ull << mp.page_shift, in_page = off & (page - 1ull);
+    if (pages) *pages = (uint32_t)(((off & ((1ull << page_shift) - 1ull)) + bytes + (1ull << page_shift) - 1ull) >> page_shift);
+    const uint64_t page = 1ull << shift, in_page = off & (page - 1ull);
     *first_bytes = min((uint64_t)bytes, page - in_page);     // bytes of the access that fall into its first page
-    return (uint32_t)((in_page + bytes + page - 1ull) >> mp.page_shift);
+    return (uint32_t)((in_page + bytes + page - 1ull) >> shift);
 }
 
 // the same with the one registered range in the kernel's arguments: nothing is read from memory to classify
-__device__ __forceinline__ uint32_t parts_of_fast(const FastRange &fr, uint32_t page_shift, uint64_t addr, int64_t issue, uint64_t bf,
-                                                  uint32_t *first_bytes) {
+__device__ __forceinline__ uint32_t parts_of_fast(const FastRange &fr, uint32_t shift, uint64_t addr, int64_t issue, uint64_t bf,
+                                                  uint32_t *first_bytes, uint32_t page_shift = 0, uint32_t *pages = nullptr) {
     const uint32_t bytes = (uint32_t)bf, flags = (uint32_t)(bf >> 32);
     const uint64_t rel = addr - fr.base;
     const uint32_t need = (flags & 1u) ? (uint32_t)HBF_PERM_PROGRAM : (uint32_t)HBF_PERM_READ;
     const bool ready = bytes != 0u && (flags & ~1u) == 0u && issue >= 0 && issue < HBF_ISSUE_LIMIT && addr >= fr.base &&
                        rel < fr.length && (uint64_t)bytes <= fr.length - rel && (fr.perms & need) != 0u;
     *first_bytes = bytes;
+    if (pages) *pages = 1u;
     if (!ready) return 1u;
-    const uint32_t page = 1u << page_shift, in_page = (uint32_t)(fr.media_offset + rel) & (page - 1u);
+    const uint32_t off = (uint32_t)(fr.media_offset + rel);
+    if (pages) *pages = (uint32_t)(((uint64_t)(off & ((1u << page_shift) - 1u)) + bytes + ((1u << page_shift) - 1u)) >> page_shift);
+    const uint32_t page = 1u << shift, in_page = off & (page - 1u);
     *first_bytes = min(bytes, page - in_page);
-    return (uint32_t)(((uint64_t)in_page + bytes + page - 1u) >> page_shift);
+    return (uint32_t)(((uint64_t)in_page + bytes + page - 1u) >> shift);
 }
 
+// BY_UNIT: parts are stripe units; the pages are summed beside them, and the batch's order is checked.  A grid of a few blocks per
+// SM walks the tiles, so that the totals take one atomic per block (64 M accesses: 0.25 ms, 6.1 TB/s).
+template <bool FAST, bool BY_UNIT>
 __global__ void __launch_bounds__(kPgThreads)
-k_paged_count(const hbf_access_t *__restrict__ acc, uint64_t n, const RangeSnap *__restrict__ ranges, const ModelParams *__restrict__ mp,
-              unsigned long long *__restrict__ tile_sum, uint32_t *__restrict__ row_off) {
+k_paged_count(const hbf_access_t *__restrict__ acc, uint64_t n, const RangeSnap *__restrict__ ranges, const __grid_constant__ FastRange fast,
+              const uint32_t page_shift, const uint32_t stripe_shift, const int64_t unit_ns, const DevState *__restrict__ state,
+              unsigned long long *__restrict__ tile_sum, uint32_t *__restrict__ row_off, unsigned long long *totals) {
     __shared__ uint32_t s_row[kPgRows];
-    const uint64_t base = (uint64_t)blockIdx.x * kPgTile;
+    __shared__ unsigned long long s_pages, s_parts;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    if (tid == 0) { s_pages = 0ull; s_parts = 0ull; }
+    unsigned long long pages_sum = 0;
+    unsigned unsorted = 0;
+    for (uint64_t tile = blockIdx.x; tile * kPgTile < n; tile += gridDim.x) {
+        const uint64_t base = tile * kPgTile;
+        uint64_t r_addr[kPgItems], r_issue[kPgItems], r_bf[kPgItems];
+        if (FAST || BY_UNIT) {
 #pragma unroll
-    for (int j = 0; j < kPgItems; ++j) {                     // row j * 8 + warp of the tile: accesses base + 32 row .. + 31
-        const uint64_t i = base + (uint64_t)(j * kPgThreads + tid);
-        uint64_t fb;
-        uint32_t c = i < n ? parts_of(*ranges, *mp, reinterpret_cast<const uint64_t *>(acc + i), &fb) : 0u;
-        c = (uint32_t)warp_sum((long long)c);
-        if (lane == 0) s_row[j * (kPgThreads / 32) + warp] = c;
-    }
-    __syncthreads();
-    if (warp == 0) {                                         // exclusive scan of the 64 row sums: two per lane
-        const uint32_t a = s_row[2 * lane], b = s_row[2 * lane + 1];
-        uint32_t incl = a + b;
+            for (int j = 0; j < kPgItems; ++j) {             // the tile's loads go out together
+                const uint64_t i = base + (uint64_t)(j * kPgThreads + tid);
+                r_addr[j] = r_issue[j] = r_bf[j] = 0ull;
+                if (i < n) { const uint64_t *rec = reinterpret_cast<const uint64_t *>(acc + i); r_addr[j] = __ldg(rec); r_issue[j] = __ldg(rec + 1); r_bf[j] = __ldg(rec + 2); }
+            }
+        }
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) { const uint32_t t = __shfl_up_sync(0xffffffffu, incl, o); if (lane >= o) incl += t; }
-        const uint32_t before = incl - (a + b);
-        uint32_t *ro = row_off + (uint64_t)blockIdx.x * kPgRows;
-        ro[2 * lane] = before; ro[2 * lane + 1] = before + a;
-        if (lane == 31) tile_sum[blockIdx.x] = incl;
+        for (int j = 0; j < kPgItems; ++j) {                 // row j * 8 + warp of the tile: accesses base + 32 row .. + 31
+            const uint64_t i = base + (uint64_t)(j * kPgThreads + tid);
+            uint32_t c = 0u, pages = 0u;
+            if (i < n) {
+                if (FAST) { uint32_t fb; c = parts_of_fast(fast, BY_UNIT ? stripe_shift : page_shift, r_addr[j], (int64_t)r_issue[j], r_bf[j], &fb, page_shift, BY_UNIT ? &pages : nullptr); }
+                else { uint64_t fb; c = parts_of(*ranges, BY_UNIT ? stripe_shift : page_shift, reinterpret_cast<const uint64_t *>(acc + i), &fb, page_shift, BY_UNIT ? &pages : nullptr); }
+            }
+            if (BY_UNIT) {
+                pages_sum += pages;
+                int64_t prev = (int64_t)__shfl_up_sync(0xffffffffu, r_issue[j], 1);
+                if (lane == 0) prev = i > 0 && i < n ? (int64_t)__ldg(reinterpret_cast<const uint64_t *>(acc + i - 1) + 1) : INT64_MIN;
+                if (i < n && (int64_t)r_issue[j] < prev) unsorted = 1u;
+            }
+            c = __reduce_add_sync(0xffffffffu, c);
+            if (lane == 0) s_row[j * (kPgThreads / 32) + warp] = c;
+        }
+        __syncthreads();
+        if (warp == 0) {                                     // exclusive scan of the 64 row sums: two per lane
+            const uint32_t a = s_row[2 * lane], b = s_row[2 * lane + 1];
+            uint32_t incl = a + b;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) { const uint32_t t = __shfl_up_sync(0xffffffffu, incl, o); if (lane >= o) incl += t; }
+            const uint32_t before = incl - (a + b);
+            uint32_t *ro = row_off + tile * kPgRows;
+            ro[2 * lane] = before; ro[2 * lane + 1] = before + a;
+            if (lane == 31) { tile_sum[tile] = incl; s_parts += incl; }
+        }
+        __syncthreads();
     }
+    if (BY_UNIT) {
+        pages_sum = (unsigned long long)warp_sum((long long)pages_sum);
+        unsorted = __any_sync(0xffffffffu, unsorted);
+        if (lane == 0) { if (pages_sum) atomicAdd(&s_pages, pages_sum); if (unsorted) atomicOr(&totals[kPagedUnsorted], 1ull); }
+        __syncthreads();
+        if (tid == 0 && s_pages) atomicAdd(&totals[kPagedPages], s_pages);
+        if (tid == 0 && blockIdx.x == 0) {                   // the longest service of one stripe unit, at the service fraction in force
+            const int64_t q = state->q_ppm;
+            if (unit_ns >= (1ll << 33) || q < 1 || (double)unit_ns * 1e6 / (double)q >= 8.0e9) totals[kPagedLong] = 1ull;
+        }
+    }
+    if (tid == 0 && s_parts) atomicAdd(&totals[kPagedParts], s_parts);
 }
 
-// one block: tile sums -> exclusive offsets, in place; total[0] = number of parts of the batch
+// one block: tile sums -> exclusive offsets, in place
 __global__ void __launch_bounds__(1024)
-k_paged_tile_scan(unsigned long long *tile_sum, uint64_t n_tiles, unsigned long long *total) {
+k_paged_tile_scan(unsigned long long *tile_sum, uint64_t n_tiles) {
     __shared__ unsigned long long s_warp[32];
     __shared__ unsigned long long s_carry;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -98,7 +148,6 @@ k_paged_tile_scan(unsigned long long *tile_sum, uint64_t n_tiles, unsigned long 
         if (tid == 1023) s_carry = before + incl;
         __syncthreads();
     }
-    if (tid == 0) *total = s_carry;
 }
 
 // A warp per row of 32 consecutive accesses, rows dealt round-robin to the grid's warps; no block-wide step.  The warp
@@ -114,11 +163,11 @@ constexpr int kPgWaves = 4;                              // blocks of the expand
 template <bool FAST>
 __global__ void __launch_bounds__(kPgThreads)
 k_paged_expand(const hbf_access_t *__restrict__ acc, uint64_t n, const RangeSnap *__restrict__ ranges, const ModelParams *__restrict__ mp,
-               const FastRange fast, const uint32_t page_shift, const unsigned long long *__restrict__ tile_off,
+               const FastRange fast, const uint32_t cut_shift, const unsigned long long *__restrict__ tile_off,
                const uint32_t *__restrict__ row_off, uint64_t capacity, hbf_access_t *__restrict__ parts, uint32_t *__restrict__ part_first) {
     const int lane = threadIdx.x & 31;
     const uint64_t warps = (uint64_t)gridDim.x * (kPgThreads / 32), rows = (n + 31) / 32;
-    const uint32_t page = 1u << page_shift;
+    const uint32_t page = 1u << cut_shift;
     uint64_t *out = reinterpret_cast<uint64_t *>(parts);
     for (uint64_t row0 = (uint64_t)blockIdx.x * (kPgThreads / 32) + (threadIdx.x >> 5); row0 < rows; row0 += warps * kPgUnroll) {
         // the loads of kPgUnroll rows go out together
@@ -143,8 +192,8 @@ k_paged_expand(const hbf_access_t *__restrict__ acc, uint64_t n, const RangeSnap
         uint32_t cnt = 0u, head = 0u;
         const uint64_t row_at = r_at[u];
         if (have) {
-            if (FAST) cnt = parts_of_fast(fast, page_shift, addr, (int64_t)issue, bf, &head);
-            else { uint64_t h; cnt = parts_of(*ranges, *mp, reinterpret_cast<const uint64_t *>(acc + i), &h); head = (uint32_t)h; }
+            if (FAST) cnt = parts_of_fast(fast, cut_shift, addr, (int64_t)issue, bf, &head);
+            else { uint64_t h; cnt = parts_of(*ranges, cut_shift, reinterpret_cast<const uint64_t *>(acc + i), &h); head = (uint32_t)h; }
         }
         uint32_t incl = cnt;
 #pragma unroll
@@ -226,39 +275,49 @@ size_t paged_layout(uint64_t n, uint64_t capacity, uint32_t n_queues, PagedWorks
     size_t off = 0;
     char *b = static_cast<char *>(base_ptr);
     auto take = [&](size_t bytes) { size_t o = off; off = (off + bytes + 255) / 256 * 256; return b ? b + o : nullptr; };
-    void *ts = take(tiles * 8), *ro = take(tiles * kPgRows * 4), *tot = take(sizeof(PagedSums) + 8), *pf = take((nn + 1) * 4);
+    void *ts = take(tiles * 8), *ro = take(tiles * kPgRows * 4), *tot = take(sizeof(PagedSums) + kPagedTotals * 8), *pf = take((nn + 1) * 4);
     void *pa = take(cap * sizeof(hbf_access_t)), *pc = take(cap * 8), *ps = take(cap * 8), *pst = take(cap);
     const size_t inner = workspace_layout(cap, n_queues, nullptr, nullptr, with_bus);
     void *in = take(inner);
     if (pw) {
         pw->tile_sum = (unsigned long long *)ts; pw->row_off = (uint32_t *)ro; pw->total = (unsigned long long *)tot;
-        pw->sums = (void *)((char *)tot + (tot ? 8 : 0)); pw->part_first = (uint32_t *)pf;
+        pw->sums = (void *)((char *)tot + (tot ? kPagedTotals * 8 : 0)); pw->part_first = (uint32_t *)pf;
         pw->parts = (hbf_access_t *)pa; pw->part_completion = (int64_t *)pc; pw->part_stall = (int64_t *)ps; pw->part_status = (uint8_t *)pst;
         pw->inner = in; pw->inner_bytes = inner; pw->bytes = off;
     }
     return off;
 }
 
-cudaError_t launch_paged_count(const hbf_access_t *acc, uint64_t n, const RangeSnap *ranges, const ModelParams *mp_dev,
-                               const PagedWorkspace &pw, cudaStream_t st) {
+cudaError_t launch_paged_count(const hbf_access_t *acc, uint64_t n, const RangeSnap *ranges, const ModelParams *mp_dev, const FastRange &fast,
+                               const ModelParams &mp, const DevState *state, bool by_unit, const PagedWorkspace &pw, cudaStream_t st) {
+    (void)mp_dev;
     const uint64_t tiles = (n + kPgTile - 1) / kPgTile;
-    cudaError_t e = cudaMemsetAsync(pw.total, 0, sizeof(PagedSums) + 8, st);
+    cudaError_t e = cudaMemsetAsync(pw.total, 0, sizeof(PagedSums) + kPagedTotals * 8, st);
     if (e != cudaSuccess) return e;
-    k_paged_count<<<(unsigned)tiles, kPgThreads, 0, st>>>(acc, n, ranges, mp_dev, pw.tile_sum, pw.row_off);
-    k_paged_tile_scan<<<1, 1024, 0, st>>>(pw.tile_sum, tiles, pw.total);
-    g_kernel_launches += 2;
+    const unsigned grid = (unsigned)std::min<uint64_t>(tiles, 148u * 16u);
+    const int64_t unit_ns = std::max(mp.t_read_ns, mp.t_prog_ns) > (1ll << 40) ? (1ll << 40) : std::max(mp.t_read_ns, mp.t_prog_ns) << mp.pages_per_stripe_shift;
+    auto k = fast.on ? (by_unit ? k_paged_count<true, true> : k_paged_count<true, false>) : (by_unit ? k_paged_count<false, true> : k_paged_count<false, false>);
+    k<<<grid, kPgThreads, 0, st>>>(acc, n, ranges, fast, mp.page_shift, mp.stripe_shift, unit_ns, state, pw.tile_sum, pw.row_off, pw.total);
+    g_kernel_launches += 1;
+    return cudaGetLastError();
+}
+
+// tile sums -> where every tile's parts begin (only a batch that is expanded needs it)
+cudaError_t launch_paged_offsets(uint64_t n, const PagedWorkspace &pw, cudaStream_t st) {
+    k_paged_tile_scan<<<1, 1024, 0, st>>>(pw.tile_sum, (n + kPgTile - 1) / kPgTile);
+    g_kernel_launches += 1;
     return cudaGetLastError();
 }
 
 cudaError_t launch_paged_expand(const hbf_access_t *acc, uint64_t n, const RangeSnap *ranges, const ModelParams *mp_dev,
-                                const FastRange &fast, uint32_t page_shift, uint64_t capacity, const PagedWorkspace &pw, int sm_count,
+                                const FastRange &fast, uint32_t cut_shift, uint64_t capacity, const PagedWorkspace &pw, int sm_count,
                                 cudaStream_t st) {
     const uint64_t blocks = ((n + 31) / 32 + kPgThreads / 32 - 1) / (kPgThreads / 32);
     const unsigned grid = (unsigned)std::min<uint64_t>(blocks, (uint64_t)std::max(1, sm_count) * 8 * kPgWaves);
     if (fast.on)
-        k_paged_expand<true><<<grid, kPgThreads, 0, st>>>(acc, n, ranges, mp_dev, fast, page_shift, pw.tile_sum, pw.row_off, capacity, pw.parts, pw.part_first);
+        k_paged_expand<true><<<grid, kPgThreads, 0, st>>>(acc, n, ranges, mp_dev, fast, cut_shift, pw.tile_sum, pw.row_off, capacity, pw.parts, pw.part_first);
     else
-        k_paged_expand<false><<<grid, kPgThreads, 0, st>>>(acc, n, ranges, mp_dev, fast, page_shift, pw.tile_sum, pw.row_off, capacity, pw.parts, pw.part_first);
+        k_paged_expand<false><<<grid, kPgThreads, 0, st>>>(acc, n, ranges, mp_dev, fast, cut_shift, pw.tile_sum, pw.row_off, capacity, pw.parts, pw.part_first);
     g_kernel_launches += 1;
     return cudaGetLastError();
 }

@@ -173,3 +173,38 @@ def test_a_refused_paged_batch_changes_nothing_with_everything_on(hbf):
     assert compare(g, o, wf.acc) == hbfo.E_ACCESS_FAULT
     same_extras(g, o, True, True, True)
     assert not g.energy_bins()[1].any() and not g.get_bus_busy_until().any() and not g.retention_blocks()["disturb"].any()
+
+
+# ---- batches in issue order are cut at stripe units, their pages served as one entry (above 8,192 accesses) ----------------
+
+@pytest.mark.parametrize("n", [8_193, 40_003])
+@pytest.mark.parametrize("kind", ["inside", "crossing", "programs", "native", "fault", "odd geometry", "queue per die", "one page units", "scaled", "load", "unordered"])
+def test_stripe_units_match_the_oracle(hbf, kind, n):
+    rng = np.random.default_rng(n)
+    geo = dict(channels=8, dies=4, planes=2, page_bytes=16384, stripe_bytes=131072)
+    if kind == "odd geometry": geo.update(channels=5, dies=3, planes=3)
+    if kind == "queue per die": geo.update(queue_level=1)
+    if kind == "one page units": geo.update(stripe_bytes=16384)
+    prof = wl.load_profile("nominal", **geo)
+    prof.update(read_granule=256)
+    ranges = [(wl.RANGE_BASE, 1 << 30, 3, 0, 0, 5 * 16384)]
+    g, o = contexts(hbf, prof, ranges)
+    acc = np.zeros(n, hbfo.ACCESS_DTYPE)
+    cross = kind in ("crossing", "one page units", "native", "fault", "unordered")
+    size = rng.choice([1, 300, 16384, 40_000, 65_536, 131_072], n)
+    unit = rng.integers(0, 8000, n)
+    # inside: a place in the unit that leaves room for the access (the media begins 5 pages into its first unit)
+    place = rng.integers(0, 131_072, n) if cross else (rng.random(n) * (131_072 - size + 1)).astype(np.int64)
+    acc["addr"] = (wl.RANGE_BASE + (3 + 8 * unit.astype(np.int64)) * 16384 + place).astype(np.uint64)
+    acc["bytes"] = size
+    acc["flags"] = rng.random(n) < (0.6 if kind == "programs" else 0.1)
+    gap = 2000 if kind == "load" else 40_000
+    acc["issue_ns"] = np.sort(rng.integers(0, gap * n, n))
+    if kind == "unordered": acc["issue_ns"][n // 2] = 0
+    if kind == "native": acc["addr"][rng.random(n) < 0.3] = 77
+    if kind == "fault": acc["bytes"][n - 3] = 0
+    if kind == "scaled":
+        g.force_mode(1, 333_333); hbfo.lib().hbfo_force_mode(o._h, 1, 333_333)
+    for _ in range(2):
+        compare(g, o, acc)
+        acc["issue_ns"] += 1000
