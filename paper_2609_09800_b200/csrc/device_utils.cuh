@@ -27,6 +27,12 @@ __device__ __forceinline__ uint64_t ld_nc_u64(const uint64_t *p) {
     uint64_t v; asm volatile("ld.global.nc.u64 %0, [%1];" : "=l"(v) : "l"(p)); return v;
 }
 
+// Programmatic dependent launch: a kernel launched with the attribute may begin while the one before it still runs; up to its
+// pdl_wait it touches only what no kernel writes, and behind it everything the kernels before left is visible.  Every path of
+// such a kernel passes its pdl_wait (the kernel behind it counts on that).  pdl_trigger lets the next one begin.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 // ---- division by a run-time constant ----------------------------------------------------------------
 // For d not a power of two, l = ceil(log2 d), magic = floor(2^(63+l) / d) + 1: floor(n / d) =
 // mulhi(n, magic) >> (l - 1) for every n < 2^63 (the error term n * (magic*d - 2^(63+l)) stays below 2^(63+l)).

@@ -865,17 +865,16 @@ int hbf_thermal_step(hbf_ctx *c, int64_t dt_ns, const float *ext_power_w, uint32
         CK(cudaMemcpyAsync(c->td.ext_power, ext_power_w, n_ext * sizeof(float), cudaMemcpyHostToDevice, c->stream));
         c->last_ext.assign(ext_power_w, ext_power_w + n_ext);
     }
-    if (c->bin_ns) {                                         // the step is the bin the thermal clock stands in
-        CK(launch_take_bin(c->d_ledger + (size_t)(c->cur_bin % c->n_bins) * c->mp.n_dies, c->d_pending, c->mp.n_dies, c->stream));
-        c->cur_bin += 1;
-    }
+    unsigned long long *bin_row = nullptr;                   // the step is the bin the thermal clock stands in
+    if (c->bin_ns) { bin_row = c->d_ledger + (size_t)(c->cur_bin % c->n_bins) * c->mp.n_dies; c->cur_bin += 1; }
     if (c->profiling) CK(cudaEventRecord(c->ev_th[0], c->stream));
     if (c->rom) {                                            // the attached model stands in for the grid
+        if (bin_row) CK(launch_take_bin(bin_row, c->d_pending, c->mp.n_dies, c->stream));
         CK(launch_rom_power(c->td, c->d_pending, dt_ns, n_ext != 0, c->d_rom_p, c->stream));
         { const int rc_ = hbf_rom_step(c->rom, c->d_rom_p, 1, c->d_rom_T); if (rc_ != HBF_OK) return rc_; }
         CK(launch_rom_controller(c->td, c->d_rom_T, c->d_rom_kind, hbf_rom_outputs(c->rom), c->d_state, c->stream));
     } else {
-        CK(launch_thermal_step(c->td, c->d_state, c->d_pending, dt_ns, n_ext != 0, d_temps_out, &c->cur, c->thermal_generic ? 1 : 0, c->stream));
+        CK(launch_thermal_step(c->td, c->d_state, c->d_pending, bin_row, dt_ns, n_ext != 0, d_temps_out, &c->cur, c->thermal_generic ? 1 : 0, c->stream));
     }
     if (c->profiling) { CK(cudaEventRecord(c->ev_th[1], c->stream)); c->prof_thermal = true; }
     if (hot_c_out) {

@@ -275,7 +275,8 @@ struct ThermalDev {
     float *theta[2]; float *comp; float *P; double *region_power; float *ext_power;
     float *hot;                          // [3] device
 };
-cudaError_t launch_thermal_step(const ThermalDev &t, DevState *state, int64_t *pending, int64_t dt_ns,
+// bin_row: the ledger's bin that the step takes besides the pending totals (null without the time bins)
+cudaError_t launch_thermal_step(const ThermalDev &t, DevState *state, int64_t *pending, unsigned long long *bin_row, int64_t dt_ns,
                                 int has_ext, float *d_temps_out, int *cur, int generic_only, cudaStream_t st);
 
 cudaError_t launch_rom_power(const ThermalDev &t, int64_t *pending, int64_t dt_ns, int has_ext, double *p_out, cudaStream_t st);
