@@ -143,6 +143,14 @@ __device__ __forceinline__ uint64_t ret_block_of(const ModelParams &mp, const Re
     return (((uint64_t)ch * mp.dies + di) * mp.planes + pl) * r.bpp + bip;
 }
 
+// a retention block whose last quantum has been claimed or drained commits one cycle and clears its counters
+__device__ __forceinline__ void ret_commit_block(const RetDev &r, uint64_t b) {
+    const uint32_t pec = r.pec[b] + 1u;
+    r.pec[b] = pec; r.damage[b] = 0.0; r.disturb[b] = 0u; r.epoch_of[b] = 0u;
+    atomicAdd(&r.st->commits, 1ull);
+    if (pec >= r.max_pec) { r.worn[b] = 1; atomicAdd(&r.st->worn_blocks, 1ull); }
+}
+
 // ---- service terms (Eq. 3 for the array time; transfer is pure latency) ---------------------------
 
 struct Terms { int64_t s, xfer, energy, cb; };

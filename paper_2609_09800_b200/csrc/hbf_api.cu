@@ -42,6 +42,7 @@ struct hbf_ctx {
     BatchCtrl *d_ctrl = nullptr; hbf_batch_result_t *d_result = nullptr;
     int64_t *d_busy = nullptr, *d_busy_stage = nullptr, *d_pending = nullptr; hbf_die_stats_t *d_stats_stage = nullptr;
     hbf_batch_result_t *h_result = nullptr;      // pinned
+    SmallTotals *d_small = nullptr;              // small batches: totals over the blocks of the launch
     TileBalanceHost bal;                         // tile sizes of the in-order path from the times earlier batches left
     // thermal steps on a reduced-order model instead of the grid (off while rom == nullptr)
     hbf_rom *rom = nullptr; int64_t rom_dt_ns = 0; int32_t *d_rom_kind = nullptr; double *d_rom_p = nullptr, *d_rom_T = nullptr;
@@ -328,6 +329,7 @@ int hbf_create(const hbf_config_t *cfg, void *cuda_stream, hbf_ctx **out) {
     if (cudaMallocHost(&c->h_result, sizeof(hbf_batch_result_t)) != cudaSuccess) return fail(HBF_E_NOMEM);
     memset(c->h_result, 0, sizeof(hbf_batch_result_t));
     if (cudaMallocHost(&c->h_hot, 3 * sizeof(float)) != cudaSuccess) return fail(HBF_E_NOMEM);
+    if ((rc = dev_copy(c, &c->d_small, nullptr, 1))) return fail(rc);
     if ((rc = dev_copy(c, &c->bal.dev, nullptr, 1))) return fail(rc);
     if (cudaMallocHost(&c->bal.pinned, sizeof(TileBalance)) != cudaSuccess) return fail(HBF_E_NOMEM);
     memset(c->bal.pinned, 0, sizeof(TileBalance));
@@ -480,11 +482,18 @@ static int serve_records(hbf_ctx *c, SubmitArgs &a) {
     }
     a.binned = c->bin_ns != 0; a.bus_on = c->d_bus_busy ? 1 : 0;
     a.bal = &c->bal;
-    if (c->ret_on) {                                         // how far the outstanding refresh quanta reach into this batch
-        CK(launch_ret_window(a.acc, a.n, c->d_ranges, c->ret, c->sm_count, c->stream));
-        a.claim_limit = &c->ret.st->claim_limit; a.die_claims = c->ret.die_claims; a.ret = &c->ret;
+    if (c->ret_on) { a.claim_limit = &c->ret.st->claim_limit; a.die_claims = c->ret.die_claims; a.ret = &c->ret; }
+    if (small_route(a)) {                                    // one launch, everything included (with the bus on it stops before the ledger)
+        auto mark = [&](int k) { if (a.ev) cudaEventRecord(a.ev[k], c->stream); };
+        mark(0); mark(7);
+        CK(launch_small(a, SmallExtras{c->d_small, a.binned ? c->d_ledger : nullptr, c->bin_ns, c->cur_bin, c->n_bins}, c->stream));
+        mark(8); for (int k = 1; k <= 6; ++k) mark(k);
+        if (!a.bus_on) return HBF_OK;
+    } else {
+        if (c->ret_on)                                       // how far the outstanding refresh quanta reach into this batch
+            CK(launch_ret_window(a.acc, a.n, c->d_ranges, c->ret, c->sm_count, c->stream));
+        CK(launch_submit(a, c->stream));
     }
-    CK(launch_submit(a, c->stream));
     if (a.binned) {
         const int64_t page = (int64_t)1 << c->mp.page_shift;
         const int64_t quantum_pj = c->mp.e_cmd_read_pj + c->mp.e_byte_read_pj * page + c->mp.e_cmd_prog_pj + c->mp.e_byte_prog_pj * page;
@@ -928,6 +937,7 @@ int hbf_reset(hbf_ctx *c) {
     CK(cudaMemsetAsync(c->d_busy, 0, c->mp.n_queues * sizeof(int64_t), c->stream));
     CK(cudaMemsetAsync(c->d_pending, 0, c->mp.n_dies * sizeof(int64_t), c->stream));
     CK(cudaMemsetAsync(c->d_result, 0, sizeof(hbf_batch_result_t), c->stream));
+    CK(cudaMemsetAsync(c->d_small, 0, sizeof(SmallTotals), c->stream));
     if (c->bin_ns) { CK(cudaMemsetAsync(c->d_ledger, 0, (size_t)c->n_bins * c->mp.n_dies * 8, c->stream)); c->cur_bin = 0; }
     if (c->d_bus_busy) CK(cudaMemsetAsync(c->d_bus_busy, 0, (size_t)c->mp.channels * 8, c->stream));
     if (c->ret_on) { int rc = retention_clear(c); if (rc != HBF_OK) return rc; }

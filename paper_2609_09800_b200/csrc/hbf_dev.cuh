@@ -128,6 +128,16 @@ extern std::atomic<unsigned long long> g_kernel_launches;
 // The dynamic shared memory a kernel may use is an attribute of the (device, kernel) pair: raises it on the current device
 // when `bytes` exceeds what this process has set there so far.  Thread-safe.
 cudaError_t ensure_dyn_smem(const void *kernel, size_t bytes);
+// a launch that may begin while the kernel before it still runs: for kernels that pass pdl_wait() (device_utils.cuh) on every path
+template <class Kernel, class... Args>
+inline cudaError_t launch_pdl(Kernel k, dim3 grid, dim3 block, size_t smem, cudaStream_t st, const Args &...args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization; at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at; cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k, args...);
+}
 
 constexpr uint32_t kInMaxQueues = 2048;  // the in-order path keeps per-queue state in shared memory
 constexpr uint32_t kInMaxTiles = 1024;
@@ -179,9 +189,12 @@ struct InTile { long long spec_sum, fix_delta, true_sum; uint32_t reserve; uint3
 size_t inorder_head_bytes(uint64_t tiles, uint32_t n_queues);
 size_t inorder_serve_smem(uint32_t n_dies);
 cudaError_t launch_inorder(const SubmitArgs &a, cudaStream_t st);
-constexpr uint32_t kInSmallMax = 8192;   // batches of at most this many records are served by one block in one launch
-bool inorder_small_batch(uint64_t n);   // whether launch_inorder takes that route
-uint32_t inorder_small_blocks(uint32_t n_queues);   // its blocks: each leaves one entry of the tile table (the slice's stall total)
+// small batches: one launch that serves and commits the batch, claims, ledger and read disturb included (small_kernels.cu)
+constexpr uint32_t kInSmallMax = 8192;   // records
+struct SmallTotals { unsigned long long modeled_ns, service_ns; long long max_completion_ns; uint32_t done, pad; };   // zero between batches
+struct SmallExtras { SmallTotals *tot; unsigned long long *ledger; int64_t bin_ns, cur_bin; uint32_t n_bins; };
+bool small_route(const SubmitArgs &a);
+cudaError_t launch_small(const SubmitArgs &a, const SmallExtras &x, cudaStream_t st);
 cudaError_t launch_submit(const SubmitArgs &a, cudaStream_t st);
 // total[i] += part[i] over the 6 * n_dies counters of a per-die statistics array (host-buffer pipeline: totals over its chunks)
 cudaError_t launch_add_stats(hbf_die_stats_t *total, const hbf_die_stats_t *part, uint32_t n_dies, cudaStream_t st);

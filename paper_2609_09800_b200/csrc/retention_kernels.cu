@@ -181,10 +181,7 @@ k_ret_commit(const hbf_batch_result_t *result, RetDev r) {
     const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
     for (uint64_t b = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; b < r.n_blocks; b += stride) {
         if (r.epoch_of[b] == 0u || r.last_pos[b] >= mark) continue;
-        const uint32_t pec = r.pec[b] + 1u;
-        r.pec[b] = pec; r.damage[b] = 0.0; r.disturb[b] = 0u; r.epoch_of[b] = 0u;
-        atomicAdd(&st->commits, 1ull);
-        if (pec >= r.max_pec) { r.worn[b] = 1; atomicAdd(&st->worn_blocks, 1ull); }
+        ret_commit_block(r, b);
     }
 }
 

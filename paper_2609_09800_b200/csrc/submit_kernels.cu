@@ -1038,8 +1038,7 @@ size_t workspace_layout(uint64_t n, uint32_t n_queues, Workspace *ws, void *base
     const uint64_t in_tiles = inorder_tiles_bound(nn);
     const bool inorder = n_queues <= kInMaxQueues;
     void *ia = take(inorder ? in_tiles * n_queues * 16 : 0), *ib = take(inorder ? in_tiles * n_queues * 8 : 0);
-    // (the tile table also takes one entry per block of the small-batch route, which a batch of few records has more of than tiles)
-    void *it = take(inorder ? std::max<uint64_t>(in_tiles, inorder_small_blocks(n_queues)) * sizeof(InTile) : 0);
+    void *it = take(inorder ? in_tiles * sizeof(InTile) : 0);
     void *ih = take(inorder ? inorder_head_bytes(in_tiles, n_queues) : 0);
     void *ic = take(inorder ? in_tiles * n_queues : 0);
     void *iq = take(inorder ? inorder_qid_entries(nn) * 2 : 0);
@@ -1187,7 +1186,7 @@ static cudaError_t launch_after_inorder(const SubmitArgs &a, bool may_sort, cuda
     c.stall_grid = (unsigned)std::max<uint64_t>(1, std::min<uint64_t>((n + 255) / 256, (uint64_t)a.sm_count * 16));
     const InTileMap tmap = inorder_tile_map(n, a.sm_count, a.bal && a.bal->on && a.bal->dev);
     c.in_tile = reinterpret_cast<const InTile *>(a.ws.in_tile);
-    c.n_tiles = inorder_small_batch(n) && !a.paged ? inorder_small_blocks(a.mp.n_queues) : tmap.n_tiles;
+    c.n_tiles = tmap.n_tiles;
     if (may_sort) k_after_inorder<true><<<1, 256, 0, st>>>(c); else k_after_inorder<false><<<1, 256, 0, st>>>(c);
     g_kernel_launches += 1;
     return cudaGetLastError();

@@ -213,6 +213,7 @@ k_thermal_cluster(const __grid_constant__ ThermalDev t, float *theta, DevState *
     const uint32_t up_bar = has_up ? th_remote(bar0, rank - 1u) : 0u, down_bar = has_down ? th_remote(bar0, rank + 1u) : 0u;
     const uint32_t expect = ((has_up ? 1u : 0u) + (has_down ? 1u : 0u)) * W * 4u;
     pdl_wait();                                               // from here on: what the kernels before left
+    pdl_trigger();
     // field: own rows and the neighbours' boundary rows, from global memory (the second buffer's rows outside the grid stay 0)
     for (uint32_t i = tid; i < pitch; i += kThThreads) {
         const uint32_t r = i / W, x = i - r * W;
