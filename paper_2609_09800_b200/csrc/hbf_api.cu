@@ -42,7 +42,6 @@ struct hbf_ctx {
     BatchCtrl *d_ctrl = nullptr; hbf_batch_result_t *d_result = nullptr;
     int64_t *d_busy = nullptr, *d_busy_stage = nullptr, *d_pending = nullptr; hbf_die_stats_t *d_stats_stage = nullptr;
     hbf_batch_result_t *h_result = nullptr;      // pinned
-    SmallTotals *d_small = nullptr;              // small batches: totals over the blocks of the launch
     TileBalanceHost bal;                         // tile sizes of the in-order path from the times earlier batches left
     // thermal steps on a reduced-order model instead of the grid (off while rom == nullptr)
     hbf_rom *rom = nullptr; int64_t rom_dt_ns = 0; int32_t *d_rom_kind = nullptr; double *d_rom_p = nullptr, *d_rom_T = nullptr;
@@ -329,7 +328,6 @@ int hbf_create(const hbf_config_t *cfg, void *cuda_stream, hbf_ctx **out) {
     if (cudaMallocHost(&c->h_result, sizeof(hbf_batch_result_t)) != cudaSuccess) return fail(HBF_E_NOMEM);
     memset(c->h_result, 0, sizeof(hbf_batch_result_t));
     if (cudaMallocHost(&c->h_hot, 3 * sizeof(float)) != cudaSuccess) return fail(HBF_E_NOMEM);
-    if ((rc = dev_copy(c, &c->d_small, nullptr, 1))) return fail(rc);
     if ((rc = dev_copy(c, &c->bal.dev, nullptr, 1))) return fail(rc);
     if (cudaMallocHost(&c->bal.pinned, sizeof(TileBalance)) != cudaSuccess) return fail(HBF_E_NOMEM);
     memset(c->bal.pinned, 0, sizeof(TileBalance));
@@ -486,7 +484,7 @@ static int serve_records(hbf_ctx *c, SubmitArgs &a) {
     if (small_route(a)) {                                    // one launch, everything included (with the bus on it stops before the ledger)
         auto mark = [&](int k) { if (a.ev) cudaEventRecord(a.ev[k], c->stream); };
         mark(0); mark(7);
-        CK(launch_small(a, SmallExtras{c->d_small, a.binned ? c->d_ledger : nullptr, c->bin_ns, c->cur_bin, c->n_bins}, c->stream));
+        CK(launch_small(a, SmallExtras{a.binned ? c->d_ledger : nullptr, c->bin_ns, c->cur_bin, c->n_bins}, c->stream));
         mark(8); for (int k = 1; k <= 6; ++k) mark(k);
         if (!a.bus_on) return HBF_OK;
     } else {
@@ -937,7 +935,6 @@ int hbf_reset(hbf_ctx *c) {
     CK(cudaMemsetAsync(c->d_busy, 0, c->mp.n_queues * sizeof(int64_t), c->stream));
     CK(cudaMemsetAsync(c->d_pending, 0, c->mp.n_dies * sizeof(int64_t), c->stream));
     CK(cudaMemsetAsync(c->d_result, 0, sizeof(hbf_batch_result_t), c->stream));
-    CK(cudaMemsetAsync(c->d_small, 0, sizeof(SmallTotals), c->stream));
     if (c->bin_ns) { CK(cudaMemsetAsync(c->d_ledger, 0, (size_t)c->n_bins * c->mp.n_dies * 8, c->stream)); c->cur_bin = 0; }
     if (c->d_bus_busy) CK(cudaMemsetAsync(c->d_bus_busy, 0, (size_t)c->mp.channels * 8, c->stream));
     if (c->ret_on) { int rc = retention_clear(c); if (rc != HBF_OK) return rc; }

@@ -191,8 +191,7 @@ size_t inorder_serve_smem(uint32_t n_dies);
 cudaError_t launch_inorder(const SubmitArgs &a, cudaStream_t st);
 // small batches: one launch that serves and commits the batch, claims, ledger and read disturb included (small_kernels.cu)
 constexpr uint32_t kInSmallMax = 8192;   // records
-struct SmallTotals { unsigned long long modeled_ns, service_ns; long long max_completion_ns; uint32_t done, pad; };   // zero between batches
-struct SmallExtras { SmallTotals *tot; unsigned long long *ledger; int64_t bin_ns, cur_bin; uint32_t n_bins; };
+struct SmallExtras { unsigned long long *ledger; int64_t bin_ns, cur_bin; uint32_t n_bins; };
 bool small_route(const SubmitArgs &a);
 cudaError_t launch_small(const SubmitArgs &a, const SmallExtras &x, cudaStream_t st);
 cudaError_t launch_submit(const SubmitArgs &a, cudaStream_t st);
