@@ -125,21 +125,24 @@ static cudaError_t launch_thermal_generic(const ThermalDev &t, DevState *state, 
 
 // ======================================================================================================
 // The whole step in one launch, for grids that fit the shared memory of one thread-block cluster: the blocks each keep a
-// band of rows of the field (both Jacobi buffers, with one halo row above and below) in shared memory and every cell's
+// band of rows of the field (both Jacobi buffers, with a halo row above and below) in shared memory and every cell's
 // constants, power and compensation term in registers.  After each substep a block sends its first and last row into its
 // neighbours' halo rows (st.async, counted in bytes by a barrier in the neighbour's shared memory): a block waits for its two
 // neighbours only, not for the whole cluster.  A neighbour cannot run ahead into a buffer that is still read: it needs this
 // block's rows of a substep before it starts the next.  The arithmetic of a cell is the same, in the same order, as in
 // k_euler_substep (a missing neighbour has conductance 0, which adds nothing); the power map is formed by every block for its
 // own cells and the hotspots are reduced through block 0.
-// 16,384 cells are far too few to fill the device: a step lasts as long as its chain of substeps (read the neighbours, twelve
-// dependent operations, send, wait).  With CPT cells per thread known at compile time, no tests and no division in the
-// substep, and waits for neighbours only: see launch_thermal_step for what it measured.
+// 16,384 cells are far too few to fill the device: a step lasts as long as its chain of substeps.  A thread holds pairs of cells,
+// one above the other, and a buffer holds the two rows of a pair side by side, so that a pair's substep is three 8-byte and two
+// 4-byte loads (its own, east, west; north, south) and one store: a substep's arithmetic takes 300 cycles of the cluster's SMs
+// where cell by cell, five loads each, it took 720; the wait for the neighbours' rows takes 150.  (Rows sent every fourth
+// substep only, each block advancing its neighbours' three nearest rows itself: slower, the wait is not what a substep costs.)
+// Whatever no kernel changes is read before the wait for the kernel before.
 // ======================================================================================================
 constexpr int kThClusterBlocks = 16;                       // blocks of the cluster when the device takes that many (not a portable size), else 8
 constexpr int kThClusterPortable = 8;
 constexpr int kThThreads = 512;
-constexpr int kThCellsPerThread = 8;
+constexpr int kThPairsPerThread = 4;
 constexpr int kThMaxRegions = 1024;
 constexpr uint32_t kThTermDies = 1024;                     // dies whose power terms are formed a thread each
 constexpr uint32_t kThWaitPolls = 1u << 22;
@@ -158,129 +161,169 @@ __device__ __forceinline__ bool th_poll(uint32_t bar, uint32_t parity) {
     return done != 0u;
 }
 
-template <int CPT>
+// floats as integers of the same order
+__device__ __forceinline__ int th_order(float f) { const int k = __float_as_int(f); return k >= 0 ? k : k ^ 0x7fffffff; }
+__device__ __forceinline__ float th_unorder(int k) { return __int_as_float(k >= 0 ? k : k ^ 0x7fffffff); }
+
+template <int PPT>
 __global__ void __launch_bounds__(kThThreads, 1)
 k_thermal_cluster(const __grid_constant__ ThermalDev t, float *theta, DevState *state, int64_t *pending, unsigned long long *bin_row, int64_t dt_ns,
                   int has_ext, float dt_sub, float *temps_out) {
     extern __shared__ __align__(16) unsigned char th_smem_buf[];
     __shared__ double s_region_power[kThMaxRegions];
     __shared__ double s_term[kThTermDies];
-    __shared__ float s_hot[kThClusterBlocks][3];
-    __shared__ float s_part[3][kThThreads / 32];
+    __shared__ uint16_t s_list[kThTermDies];
+    __shared__ int s_hot[3][kThClusterBlocks];
+    __shared__ int s_part[3][kThThreads / 32];
     __shared__ __align__(8) uint64_t s_bar[2];
+    __shared__ __align__(8) uint64_t s_bar_hot;               // (first block) every block's hotspots have come
     cg::cluster_group cluster = cg::this_cluster();
     const uint32_t rank = cluster.block_rank(), n_blocks = cluster.num_blocks();      // (the cluster's size is chosen at launch)
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const uint32_t H = t.H, W = t.W;
     const uint32_t rows = (H + n_blocks - 1) / n_blocks;
-    const uint32_t y0 = min(H, rank * rows), y1 = min(H, y0 + rows);
-    const uint32_t band_cells = (y1 - y0) * W;
-    const uint32_t pitch = (rows + 2) * W;                    // one buffer: halo row, band, halo row
-    float *buf0 = reinterpret_cast<float *>(th_smem_buf);
-    const bool has_up = rank > 0u && y1 > y0, has_down = y1 < H && y1 > y0;
-    if (tid < 2) {
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(th_smem(&s_bar[tid])) : "memory");
+    const uint32_t y0 = min(H, rank * rows), y1 = min(H, y0 + rows), mine = y1 - y0;
+    const uint32_t pairs = (mine + 1u) / 2u * W, pitch = ((rows + 1u) / 2u + 2u) * W;   // a buffer: pairs of rows (-2, -1), (0, 1), ... up to the one with the lower halo row
+    float2 *buf0 = reinterpret_cast<float2 *>(th_smem_buf);
+    const bool has_up = rank > 0u && mine > 0u, has_down = y1 < H && mine > 0u;
+    if (tid < 3) {
+        const uint32_t bar = th_smem(tid < 2 ? &s_bar[tid] : &s_bar_hot);
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar) : "memory");
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        if (tid == 2) asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(n_blocks * 12u) : "memory");
     }
-    // what no kernel changes: this thread's cells' constants
-    float kC[CPT], gE[CPT], gW_[CPT], gS[CPT], gN[CPT], gs[CPT], P[CPT], cmp[CPT];
-    uint32_t off[CPT], up[CPT], down[CPT];                    // place in a buffer; the same cell in the neighbours' halo rows (0: not a boundary row)
-    int32_t region[CPT];
-    bool live[CPT];
+    // where row r of a block with `rows` rows lies in its buffer, in bytes
+    auto row_at = [&](int32_t r, uint32_t x) { return ((((uint32_t)(r + 2) >> 1) * W + x) * 2u + ((uint32_t)r & 1u)) * 4u; };
+    // what no kernel changes: the constants of this thread's cells, the regions' dies
+    float kC[PPT][2], gE[PPT][2], gW_[PPT][2], gS[PPT][2], gN[PPT][2], gs[PPT][2], P[PPT][2], cmp[PPT][2], inv[PPT][2];
+    uint32_t off[PPT], up[PPT], down[PPT];                    // place in a buffer; the boundary cell's place in the neighbours' halo rows (0: none)
+    int32_t region[PPT][2], kind[PPT][2];
+    bool live[PPT][2];
 #pragma unroll
-    for (int c = 0; c < CPT; ++c) {
-        const uint32_t li = (uint32_t)c * kThThreads + tid;   // cell of the band, row-major
-        live[c] = li < band_cells;
-        off[c] = W; up[c] = down[c] = 0u; region[c] = -1;
-        kC[c] = gE[c] = gW_[c] = gS[c] = gN[c] = gs[c] = P[c] = cmp[c] = 0.0f;
-        if (live[c]) {
-            const uint32_t r = li / W, x = li - r * W, y = y0 + r;
-            const uint64_t i = (uint64_t)y * W + x;
-            off[c] = (r + 1) * W + x;
-            kC[c] = dt_sub / t.C[i];
-            if (x + 1 < W) gE[c] = t.Gx[i];
-            if (x > 0) gW_[c] = t.Gx[i - 1];
-            if (y + 1 < H) gS[c] = t.Gy[i];
-            if (y > 0) gN[c] = t.Gy[i - W];
-            gs[c] = t.Gs[i];
-            region[c] = t.cell_region[i];
+    for (int c = 0; c < PPT; ++c) {
+        const uint32_t li = (uint32_t)c * kThThreads + tid, pr = li / W, x = li - pr * W;
+        off[c] = W; up[c] = down[c] = 0u;
+        if (li < pairs) {
             const uint32_t b0 = th_smem(buf0);
-            if (r == 0u && has_up) up[c] = th_remote(b0 + ((rows + 1) * W + x) * 4u, rank - 1u);              // (a block above another is full: its lower halo row sits behind `rows` rows)
-            if (r + 1u == y1 - y0 && has_down) down[c] = th_remote(b0 + x * 4u, rank + 1u);
+            off[c] = (pr + 1u) * W + x;
+            if (pr == 0u && has_up) up[c] = th_remote(b0 + row_at((int32_t)rows, x), rank - 1u);          // (a block above another is full)
+            if (pr == (mine - 1u) / 2u && has_down) down[c] = th_remote(b0 + row_at(-1, x), rank + 1u);
+        }
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const uint32_t r = pr * 2u + h, y = y0 + r;
+            live[c][h] = li < pairs && r < mine;
+            region[c][h] = -1; kind[c][h] = HBF_KIND_NONE;
+            kC[c][h] = gE[c][h] = gW_[c][h] = gS[c][h] = gN[c][h] = gs[c][h] = P[c][h] = cmp[c][h] = inv[c][h] = 0.0f;
+            if (live[c][h]) {
+                const uint64_t i = (uint64_t)y * W + x;
+                kC[c][h] = dt_sub / t.C[i];
+                if (x + 1 < W) gE[c][h] = t.Gx[i];
+                if (x > 0) gW_[c][h] = t.Gx[i - 1];
+                if (y + 1 < H) gS[c][h] = t.Gy[i];
+                if (y > 0) gN[c][h] = t.Gy[i - W];
+                gs[c][h] = t.Gs[i];
+                region[c][h] = t.cell_region[i];
+                if (region[c][h] >= 0) { inv[c][h] = t.region_inv_cells[region[c][h]]; kind[c][h] = t.region_kind[region[c][h]]; }
+            }
         }
     }
+    const bool by_die = t.n_dies <= kThTermDies;
+    if (by_die) for (uint32_t d = tid; d < t.n_dies; d += kThThreads) s_list[d] = (uint16_t)t.region_die_list[d];
+    int32_t g0 = 0, g1 = 0;                                   // this thread's first region: its dies and its other power (the host writes ext_power between kernels only)
+    double p_idle = 0.0, p_ext = 0.0;
+    if ((uint32_t)tid < t.n_regions) { g0 = t.region_die_ptr[tid]; g1 = t.region_die_ptr[tid + 1]; p_idle = (double)t.region_idle_w[tid]; if (has_ext) p_ext = (double)t.ext_power[tid]; }
+    for (uint32_t i = tid; i < 2u * pitch; i += kThThreads) buf0[i] = make_float2(0.0f, 0.0f);      // (rows outside the grid stay 0)
     const uint32_t bar0 = th_smem(&s_bar[0]);
     const uint32_t up_bar = has_up ? th_remote(bar0, rank - 1u) : 0u, down_bar = has_down ? th_remote(bar0, rank + 1u) : 0u;
     const uint32_t expect = ((has_up ? 1u : 0u) + (has_down ? 1u : 0u)) * W * 4u;
+    __syncthreads();
     pdl_wait();                                               // from here on: what the kernels before left
     pdl_trigger();
-    // field: own rows and the neighbours' boundary rows, from global memory (the second buffer's rows outside the grid stay 0)
-    for (uint32_t i = tid; i < pitch; i += kThThreads) {
-        const uint32_t r = i / W, x = i - r * W;
-        const int64_t y = (int64_t)y0 + r - 1;
-        buf0[i] = (r < y1 - y0 + 2 && y >= 0 && y < (int64_t)H) ? theta[(uint64_t)y * W + x] : 0.0f;
-        buf0[pitch + i] = 0.0f;
-    }
+    // the energies, the cells' own state and the neighbours' boundary rows: all loads go out together
+    const int32_t mode0 = state->mode;
+    int64_t e0 = 0;
+    auto energy = [&](uint32_t d) { return pending[d] + (bin_row ? (int64_t)bin_row[d] : 0); };
+    if (by_die && (uint32_t)tid < t.n_dies) e0 = energy(tid);
+    float own[PPT][2];
 #pragma unroll
-    for (int c = 0; c < CPT; ++c) if (live[c]) cmp[c] = t.comp[(uint64_t)y0 * W + (uint32_t)c * kThThreads + tid];
+    for (int c = 0; c < PPT; ++c)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const uint32_t li = (uint32_t)c * kThThreads + tid, pr = li / W, x = li - pr * W;
+            own[c][h] = 0.0f;
+            if (live[c][h]) { const uint64_t i = (uint64_t)(y0 + pr * 2u + h) * W + x; own[c][h] = theta[i]; cmp[c][h] = t.comp[i]; }
+        }
+    for (uint32_t x = tid; x < W; x += kThThreads) {
+        if (has_up) reinterpret_cast<float *>(buf0)[row_at(-1, x) / 4u] = theta[(uint64_t)(y0 - 1u) * W + x];
+        if (has_down) reinterpret_cast<float *>(buf0)[row_at((int32_t)mine, x) / 4u] = theta[(uint64_t)y1 * W + x];
+    }
     // power of every region over the window (every block forms the same values, summed in the order of the region's dies), then
     // of this block's cells.  The ledger's bin, when there is one, is taken with the pending totals.
-    auto term = [&](uint32_t d) {
-        const int64_t e = pending[d] + (bin_row ? (int64_t)bin_row[d] : 0);
-        return ((double)e * 1e-12) / ((double)dt_ns * 1e-9);
-    };
-    const bool by_die = t.n_dies <= kThTermDies;
-    if (by_die) {
-        for (uint32_t d = tid; d < t.n_dies; d += kThThreads) s_term[d] = term(d);
-        __syncthreads();
-    }
-    for (uint32_t g = tid; g < t.n_regions; g += kThThreads) {
-        double p = 0.0;
-        const int32_t k0 = t.region_die_ptr[g], k1 = t.region_die_ptr[g + 1];
-        for (int32_t k = k0; k < k1; k += 8) {
-            uint32_t d[8];
+    auto term = [&](int64_t e) { return ((double)e * 1e-12) / ((double)dt_ns * 1e-9); };
+    if (by_die)
+        for (uint32_t d = tid; d < t.n_dies; d += kThThreads) s_term[d] = term(d < (uint32_t)kThThreads ? e0 : energy(d));
 #pragma unroll
-            for (int j = 0; j < 8; ++j) d[j] = k + j < k1 ? (uint32_t)t.region_die_list[k + j] : 0u;
-#pragma unroll
-            for (int j = 0; j < 8; ++j) if (k + j < k1) p += by_die ? s_term[d[j]] : term(d[j]);
-        }
-        p += (double)t.region_idle_w[g];
-        if (has_ext) p += (double)t.ext_power[g];
-        s_region_power[g] = p;
+    for (int c = 0; c < PPT; ++c) {
+        if (live[c][1]) buf0[off[c]] = make_float2(own[c][0], own[c][1]);
+        else if (live[c][0]) buf0[off[c]].x = own[c][0];      // (the other half of a last odd row's pair is the halo row)
     }
     __syncthreads();
+    for (uint32_t g = tid; g < t.n_regions; g += kThThreads) {
+        if (g >= (uint32_t)kThThreads) { g0 = t.region_die_ptr[g]; g1 = t.region_die_ptr[g + 1]; p_idle = (double)t.region_idle_w[g]; if (has_ext) p_ext = (double)t.ext_power[g]; }
+        double p = 0.0;
+        for (int32_t k = g0; k < g1; ++k) p += by_die ? s_term[s_list[k]] : term(energy((uint32_t)t.region_die_list[k]));
+        p += p_idle;
+        if (has_ext) p += p_ext;
+        s_region_power[g] = p;
+    }
+    cluster.barrier_arrive();                                 // this block's buffers and barriers stand, and it has read the energies
+    __syncthreads();
 #pragma unroll
-    for (int c = 0; c < CPT; ++c) if (region[c] >= 0) P[c] = (float)(s_region_power[region[c]] * (double)t.region_inv_cells[region[c]]);
-    cluster.sync();                                           // every block's buffers and barriers stand, and every block has read the energies
+    for (int c = 0; c < PPT; ++c)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) if (region[c][h] >= 0) P[c][h] = (float)(s_region_power[region[c][h]] * (double)inv[c][h]);
+    cluster.barrier_wait();
     if (rank == 0)
         for (uint32_t d = tid; d < t.n_dies; d += kThThreads) { pending[d] = 0; if (bin_row) bin_row[d] = 0ull; }
 
     bool lost = false;
     for (uint32_t k = 0; k < t.n_sub; ++k) {
         const uint32_t ob = (k + 1u) & 1u;                    // the buffer written
-        const float *in = buf0 + (k & 1u) * pitch;
-        float *out = buf0 + ob * pitch;
+        const float2 *in = buf0 + (k & 1u) * pitch;
+        float2 *out = buf0 + ob * pitch;
         const bool more = k + 1u < t.n_sub;
         if (more && expect && tid == 0)
             asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar0 + ob * 8u), "r"(expect) : "memory");
 #pragma unroll
-        for (int c = 0; c < CPT; ++c) {
-            if (live[c]) {
+        for (int c = 0; c < PPT; ++c) {
+            if (live[c][0]) {
                 const uint32_t o = off[c];
-                const float Ti = in[o];
-                float flow = 0.0f;
-                flow += gE[c] * (Ti - in[o + 1]);
-                flow += gW_[c] * (Ti - in[o - 1]);
-                flow += gS[c] * (Ti - in[o + W]);
-                flow += gN[c] * (Ti - in[o - W]);
-                const float inc = kC[c] * (P[c] - flow - gs[c] * Ti);
-                const float yv = inc - cmp[c];
-                const float tn = Ti + yv;
-                cmp[c] = (tn - Ti) - yv;
-                out[o] = tn;
+                const float2 T = in[o], E = in[o + 1], Wt = in[o - 1];
+                const float N = in[o - W].y, S = in[o + W].x;
+                auto cell = [&](int h, float Ti, float te, float tw, float ts, float tn_) {
+                    float flow = 0.0f;
+                    flow += gE[c][h] * (Ti - te);
+                    flow += gW_[c][h] * (Ti - tw);
+                    flow += gS[c][h] * (Ti - ts);
+                    flow += gN[c][h] * (Ti - tn_);
+                    const float inc = kC[c][h] * (P[c][h] - flow - gs[c][h] * Ti);
+                    const float yv = inc - cmp[c][h];
+                    const float tn = Ti + yv;
+                    cmp[c][h] = (tn - Ti) - yv;
+                    return tn;
+                };
+                const float a = cell(0, T.x, E.x, Wt.x, T.y, N);
+                float last = a;
+                if (live[c][1]) {
+                    last = cell(1, T.y, E.y, Wt.y, S, T.x);
+                    out[o] = make_float2(a, last);
+                } else {
+                    out[o].x = a;
+                }
                 if (more) {
-                    if (up[c]) th_send(up[c] + ob * pitch * 4u, tn, up_bar + ob * 8u);
-                    if (down[c]) th_send(down[c] + ob * pitch * 4u, tn, down_bar + ob * 8u);
+                    if (up[c]) th_send(up[c] + ob * pitch * 8u, a, up_bar + ob * 8u);
+                    if (down[c]) th_send(down[c] + ob * pitch * 8u, last, down_bar + ob * 8u);
                 }
             }
         }
@@ -292,45 +335,48 @@ k_thermal_cluster(const __grid_constant__ ThermalDev t, float *theta, DevState *
     }
     if (lost) state->poisoned = 1;                            // a neighbour's rows never came: the context is given up
     // results: field and compensation back to global memory, hotspots to block 0
-    const float *in = buf0 + (t.n_sub & 1u) * pitch;
+    const float2 *in = buf0 + (t.n_sub & 1u) * pitch;
     float hot[3] = {-INFINITY, -INFINITY, -INFINITY};
 #pragma unroll
-    for (int c = 0; c < CPT; ++c) {
-        if (live[c]) {
-            const uint64_t i = (uint64_t)y0 * W + (uint32_t)c * kThThreads + tid;
-            const float th = in[off[c]];
-            theta[i] = th; t.comp[i] = cmp[c];
-            const float T = t.ambient_c + th;
-            if (temps_out) temps_out[i] = T;
-            if (region[c] >= 0) {
-                const int32_t kind = t.region_kind[region[c]];
-                if (kind == HBF_KIND_HBF) hot[0] = fmaxf(hot[0], T); else if (kind == HBF_KIND_HBM) hot[1] = fmaxf(hot[1], T);
-                else if (kind == HBF_KIND_GPU) hot[2] = fmaxf(hot[2], T);
+    for (int c = 0; c < PPT; ++c)
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+            if (live[c][h]) {
+                const uint32_t li = (uint32_t)c * kThThreads + tid, pr = li / W, x = li - pr * W;
+                const uint64_t i = (uint64_t)(y0 + pr * 2u + h) * W + x;
+                const float th = h ? in[off[c]].y : in[off[c]].x;
+                theta[i] = th; t.comp[i] = cmp[c][h];
+                const float T = t.ambient_c + th;
+                if (temps_out) temps_out[i] = T;
+                if (kind[c][h] == HBF_KIND_HBF) hot[0] = fmaxf(hot[0], T); else if (kind[c][h] == HBF_KIND_HBM) hot[1] = fmaxf(hot[1], T);
+                else if (kind[c][h] == HBF_KIND_GPU) hot[2] = fmaxf(hot[2], T);
             }
-        }
-    }
+    // (as ordered integers: one reduction instruction per warp and medium; the other blocks send theirs to the first and are done)
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-        for (int o = 16; o > 0; o >>= 1) hot[k] = fmaxf(hot[k], __shfl_xor_sync(0xffffffffu, hot[k], o));
-        if (lane == 0) s_part[k][warp] = hot[k];
+        const int v = __reduce_max_sync(0xffffffffu, th_order(hot[k]));
+        if (lane == 0) s_part[k][warp] = v;
     }
     __syncthreads();
-    if (tid < 3) {
-        float v = -INFINITY;
-        for (int w = 0; w < kThThreads / 32; ++w) v = fmaxf(v, s_part[tid][w]);
-        float *dst = cluster.map_shared_rank(&s_hot[0][0], 0);
-        dst[rank * 3 + tid] = v;
+    if (warp < 3) {
+        const int v = __reduce_max_sync(0xffffffffu, lane < kThThreads / 32 ? s_part[warp][lane] : th_order(-INFINITY));
+        if (lane == 0) th_send(th_remote(th_smem(&s_hot[warp][rank]), 0u), __int_as_float(v), th_remote(th_smem(&s_bar_hot), 0u));
     }
-    cluster.sync();
-    if (rank == 0 && tid == 0) {
-        float h[3];
-        for (int k = 0; k < 3; ++k) {
-            float v = -INFINITY;
-            for (uint32_t b = 0; b < n_blocks; ++b) v = fmaxf(v, s_hot[b][k]);
-            h[k] = v == -INFINITY ? t.ambient_c : v;
-            t.hot[k] = h[k];
-        }
-        const int mode = next_mode(t, state->mode, quantise_mk(h[0]));
+    if (rank != 0u || warp != 0) return;
+    {
+        const uint32_t bar = th_smem(&s_bar_hot);
+        uint32_t polls = 0;
+        while (!th_poll(bar, 0u)) if (++polls > kThWaitPolls) { state->poisoned = 1; break; }
+    }
+    float h[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        const float v = th_unorder(__reduce_max_sync(0xffffffffu, (uint32_t)lane < n_blocks ? s_hot[k][lane] : th_order(-INFINITY)));
+        h[k] = v == -INFINITY ? t.ambient_c : v;
+    }
+    if (lane == 0) {
+        t.hot[0] = h[0]; t.hot[1] = h[1]; t.hot[2] = h[2];
+        const int mode = next_mode(t, mode0, quantise_mk(h[0]));
         state->mode = mode;
         if (mode == HBF_MODE_NORMAL) state->q_ppm = 1000000;
         else if (mode == HBF_MODE_LIGHT) state->q_ppm = t.q_light_ppm;
@@ -338,18 +384,17 @@ k_thermal_cluster(const __grid_constant__ ThermalDev t, float *theta, DevState *
 }
 
 using ThermalKernel = void (*)(const ThermalDev, float *, DevState *, int64_t *, unsigned long long *, int64_t, int, float, float *);
-// the kernel whose threads hold just as many cells as the grid needs on a cluster of n_blocks
+// the kernel whose threads hold just as many pairs of cells as the grid needs on a cluster of n_blocks
 static ThermalKernel thermal_cluster_kernel(const ThermalDev &t, int n_blocks) {
-    const uint64_t cells = (uint64_t)((t.H + n_blocks - 1) / n_blocks) * t.W;
-    return cells <= 1u * kThThreads ? k_thermal_cluster<1> : cells <= 2u * kThThreads ? k_thermal_cluster<2> : cells <= 4u * kThThreads ? k_thermal_cluster<4>
-                                                                                                               : k_thermal_cluster<kThCellsPerThread>;
+    const uint64_t pairs = (uint64_t)((t.H + n_blocks - 1) / n_blocks + 1) / 2 * t.W;
+    return pairs <= 1u * kThThreads ? k_thermal_cluster<1> : pairs <= 2u * kThThreads ? k_thermal_cluster<2> : k_thermal_cluster<kThPairsPerThread>;
 }
 
 static bool thermal_cluster_fits(const ThermalDev &t, int n_blocks, size_t *smem_bytes) {
     const uint32_t rows = (t.H + n_blocks - 1) / n_blocks;
-    const size_t smem = (size_t)2 * (rows + 2) * t.W * sizeof(float);
+    const size_t smem = (size_t)2 * ((rows + 1) / 2 + 2) * t.W * sizeof(float2);
     *smem_bytes = smem;
-    return (size_t)rows * t.W <= (size_t)kThThreads * kThCellsPerThread && smem <= 200u * 1024u && t.n_regions <= (uint32_t)kThMaxRegions;
+    return (size_t)((rows + 1) / 2) * t.W <= (size_t)kThThreads * kThPairsPerThread && smem <= 200u * 1024u && t.n_regions <= (uint32_t)kThMaxRegions;
 }
 
 // How many blocks the cluster of the one-launch step gets on the current device: 16 where the device can place such a
