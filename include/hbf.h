@@ -217,7 +217,7 @@ HBF_API int hbf_thermal_step(hbf_ctx *ctx, int64_t dt_ns, const float *ext_power
  * deterministic experiments (Design D3). */
 HBF_API int hbf_force_mode(hbf_ctx *ctx, int32_t mode, int64_t q_ppm);
 HBF_API int hbf_get_mode(hbf_ctx *ctx, int32_t *mode, int64_t *q_ppm);           /* waits for pending work */
-HBF_API int hbf_reset(hbf_ctx *ctx);                                             /* queues idle, field at ambient, mode Normal */
+HBF_API int hbf_reset(hbf_ctx *ctx);                                             /* queues idle, field at ambient, mode Normal; in stream order, waits for nothing */
 
 /* Chooses how batches are ordered: HBF_PATH_AUTO (default) serves a batch whose records arrive in
  * non-decreasing issue order without a global sort and falls back to the radix sort otherwise (also for a batch in

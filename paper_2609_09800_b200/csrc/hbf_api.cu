@@ -5,6 +5,7 @@
 #include <cstdlib>
 #include <cstring>
 #include <new>
+#include <type_traits>
 #include <vector>
 
 #include "hbf_dev.cuh"
@@ -41,7 +42,11 @@ struct hbf_ctx {
     RangeSnap *d_ranges = nullptr; ModelParams *d_mp = nullptr; DevState *d_state = nullptr;
     BatchCtrl *d_ctrl = nullptr; hbf_batch_result_t *d_result = nullptr;
     int64_t *d_busy = nullptr, *d_busy_stage = nullptr, *d_pending = nullptr; hbf_die_stats_t *d_stats_stage = nullptr;
-    hbf_batch_result_t *h_result = nullptr;      // pinned
+    // pinned: the last batch's summary (written by its last kernel), part counts on their way back, the hotspots (written by the
+    // thermal step), the tiles' times
+    struct Pinned { hbf_batch_result_t result; unsigned long long totals[kPagedTotals]; float hot[4]; TileBalance bal; } *pinned = nullptr;
+    bool result_on_host = false;                 // pinned->result is the last batch's summary (small batches leave theirs on the device only)
+    bool plain_next = false;                     // what was enqueued last may launch kernels of its own: see launch_first
     TileBalanceHost bal;                         // tile sizes of the in-order path from the times earlier batches left
     // thermal steps on a reduced-order model instead of the grid (off while rom == nullptr)
     hbf_rom *rom = nullptr; int64_t rom_dt_ns = 0; int32_t *d_rom_kind = nullptr; double *d_rom_p = nullptr, *d_rom_T = nullptr;
@@ -51,8 +56,6 @@ struct hbf_ctx {
     int64_t bin_ns = 0, cur_bin = 0; uint32_t n_bins = 0; unsigned long long *d_ledger = nullptr;
     // retention, refresh and wear (off while ret_on == false)
     bool ret_on = false; RetDev ret{}; hbf_retention_config_t ret_cfg{};
-    float *h_hot = nullptr;                      // pinned [3]
-    float *h_ext = nullptr;                      // pinned [n_regions]
     std::vector<float> last_ext;                 // the external powers the device holds (empty: none sent yet)
     bool submitted = false;
     uint32_t spin_limit = kSpinLimit, test_stage = 0, test_tile = 0;   // bounded device-side waits (test support: hbf_debug_wait_test)
@@ -99,6 +102,36 @@ static int dev_copy(hbf_ctx *c, T **dst, const void *src, size_t count) {
     return HBF_OK;
 }
 
+// A context's arrays in one allocation: what has contents first (one copy), what starts as zero behind it (one memset).
+// (An allocation and a copy for each of some forty arrays made hbf_create take 3 ms.)
+class Arena {
+    struct Item { void **dst; const void *src; size_t bytes; };
+    std::vector<Item> items_;
+public:
+    template <typename T> void add(T **dst, const void *src, size_t count) {
+        items_.push_back({reinterpret_cast<void **>(const_cast<typename std::remove_const<T>::type **>(dst)), src, std::max<size_t>(count, 1) * sizeof(T)});
+    }
+    int commit(hbf_ctx *c) {
+        auto round = [](size_t v) { return (v + 255) / 256 * 256; };
+        size_t full = 0, zero = 0;
+        for (const Item &i : items_) (i.src ? full : zero) += round(i.bytes);
+        char *base = nullptr;
+        if (cudaMalloc(&base, std::max<size_t>(full + zero, 256)) != cudaSuccess) return HBF_E_NOMEM;
+        c->owned.push_back(base);
+        std::vector<char> image(full, 0);
+        size_t at = 0, behind = full;
+        for (const Item &i : items_) {
+            size_t &o = i.src ? at : behind;
+            if (i.src) memcpy(image.data() + o, i.src, i.bytes);
+            *i.dst = base + o;
+            o += round(i.bytes);
+        }
+        if (full && cudaMemcpyAsync(base, image.data(), full, cudaMemcpyHostToDevice, c->stream) != cudaSuccess) return HBF_E_CUDA;
+        if (zero && cudaMemsetAsync(base + full, 0, zero, c->stream) != cudaSuccess) return HBF_E_CUDA;
+        return cudaStreamSynchronize(c->stream) == cudaSuccess ? HBF_OK : HBF_E_CUDA;
+    }
+};
+
 static int publish_ranges(hbf_ctx *c) {
     RangeSnap snap; memset(&snap, 0, sizeof(snap));
     std::vector<HostRange> sorted = c->ranges;
@@ -111,19 +144,6 @@ static int publish_ranges(hbf_ctx *c) {
     // ordered after every batch already enqueued, before every later one
     CK(cudaMemcpyAsync(c->d_ranges, &snap, sizeof(snap), cudaMemcpyHostToDevice, c->stream));
     CK(cudaStreamSynchronize(c->stream));
-    return HBF_OK;
-}
-
-// ---- retention, refresh and wear (Design D4) ----------------------------------------------------------------
-static int retention_clear(hbf_ctx *c) {
-    const RetDev &r = c->ret;
-    CK(cudaMemsetAsync(r.damage, 0, r.n_blocks * 8, c->stream));
-    CK(cudaMemsetAsync(r.disturb, 0, r.n_blocks * 4, c->stream));
-    CK(cudaMemsetAsync(r.pec, 0, r.n_blocks * 4, c->stream));
-    CK(cudaMemsetAsync(r.epoch_of, 0, r.n_blocks * 4, c->stream));
-    CK(cudaMemsetAsync(r.worn, 0, r.n_blocks, c->stream));
-    CK(cudaMemsetAsync(r.die_claims, 0, (size_t)c->mp.n_dies * 4, c->stream));
-    CK(cudaMemsetAsync(r.st, 0, sizeof(RetState), c->stream));
     return HBF_OK;
 }
 
@@ -235,15 +255,12 @@ int hbf_destroy(hbf_ctx *c) {
     cudaStreamSynchronize(c->stream);
     for (void *p : c->owned) cudaFree(p);
     if (c->ev_made) { for (auto &e : c->ev) cudaEventDestroy(e); for (auto &e : c->ev_th) cudaEventDestroy(e); }
-    if (c->h_result) cudaFreeHost(c->h_result);
-    if (c->bal.pinned) cudaFreeHost(c->bal.pinned);
+    if (c->pinned) cudaFreeHost(c->pinned);
     if (c->d_ledger) cudaFree(c->d_ledger);
     if (c->d_bus_busy) cudaFree(c->d_bus_busy);
     if (c->d_bus_ctrl) cudaFree(c->d_bus_ctrl);
     if (c->d_rom_kind) cudaFree(c->d_rom_kind);
     if (c->d_rom_p) cudaFree(c->d_rom_p);
-    if (c->h_hot) cudaFreeHost(c->h_hot);
-    if (c->h_ext) cudaFreeHost(c->h_ext);
     if (c->pipe.made) {
         hbf_ctx::HostPipe &p = c->pipe;
         cudaStreamSynchronize(p.s_in); cudaStreamSynchronize(p.s_out);
@@ -275,9 +292,8 @@ int hbf_create(const hbf_config_t *cfg, void *cuda_stream, hbf_ctx **out) {
     int rc = HBF_OK;
     auto fail = [&](int code) { hbf_destroy(c); return code; };
     if (cudaGetDevice(&c->device) != cudaSuccess) return fail(HBF_E_CUDA);
-    cudaDeviceProp prop;
-    if (cudaGetDeviceProperties(&prop, c->device) != cudaSuccess) return fail(HBF_E_CUDA);
-    c->sm_count = prop.multiProcessorCount;
+    if (cudaDeviceGetAttribute(&c->sm_count, cudaDevAttrMultiProcessorCount, c->device) != cudaSuccess) return fail(HBF_E_CUDA);
+    Arena arena;
 
     ModelParams &mp = c->mp;
     mp.channels = cfg->channels; mp.dies = cfg->dies; mp.planes = cfg->planes;
@@ -298,9 +314,10 @@ int hbf_create(const hbf_config_t *cfg, void *cuda_stream, hbf_ctx **out) {
         c->inorder_ok = nq <= kInMaxQueues && worst / cfg->chan_bytes_per_us < ((unsigned __int128)1 << 31) &&
                         inorder_serve_smem((uint32_t)nd) + 8u * 1024u <= 227u * 1024u;
     }
+    std::vector<uint32_t> tab(1025);
+    const uint32_t *tab_dev = nullptr;
     {   // transfer times of the small charged sizes, looked up instead of divided (every charged size is a multiple of its granule)
         const uint32_t g = std::min(mp.read_gran_shift, mp.prog_gran_shift);
-        std::vector<uint32_t> tab(1025);
         bool fits = true;
         for (uint32_t k = 0; k <= 1024; ++k) {
             const unsigned __int128 x = (((unsigned __int128)k << g) * 1000u + cfg->chan_bytes_per_us - 1) / cfg->chan_bytes_per_us;
@@ -308,30 +325,25 @@ int hbf_create(const hbf_config_t *cfg, void *cuda_stream, hbf_ctx **out) {
             tab[k] = (uint32_t)x;
         }
         mp.xfer_tab = nullptr; mp.xfer_tab_shift = g; mp.xfer_tab_max_cb = 0;
-        if (fits && g < 21) {
-            uint32_t *d = nullptr;
-            if ((rc = dev_copy(c, &d, tab.data(), tab.size()))) return fail(rc);
-            mp.xfer_tab = d; mp.xfer_tab_max_cb = 1024u << g;
-        }
+        if (fits && g < 21) { arena.add(&tab_dev, tab.data(), tab.size()); mp.xfer_tab_max_cb = 1024u << g; }
     }
     DevState st0; st0.mode = HBF_MODE_NORMAL; st0.poisoned = 0; st0.q_ppm = 1000000;
     st0.spin_limit = c->spin_limit; st0.test_stage = c->test_stage; st0.test_tile = c->test_tile; st0.pad = 0;
-    if ((rc = dev_copy(c, &c->d_ranges, nullptr, 1))) return fail(rc);
-    if ((rc = dev_copy(c, &c->d_mp, &mp, 1))) return fail(rc);
-    if ((rc = dev_copy(c, &c->d_state, &st0, 1))) return fail(rc);
-    if ((rc = dev_copy(c, &c->d_ctrl, nullptr, 1))) return fail(rc);
-    if ((rc = dev_copy(c, &c->d_result, nullptr, 1))) return fail(rc);
-    if ((rc = dev_copy(c, &c->d_busy, nullptr, nq))) return fail(rc);
-    if ((rc = dev_copy(c, &c->d_busy_stage, nullptr, nq))) return fail(rc);
-    if ((rc = dev_copy(c, &c->d_pending, nullptr, nd))) return fail(rc);
-    if ((rc = dev_copy(c, &c->d_stats_stage, nullptr, nd))) return fail(rc);
-    if (cudaMallocHost(&c->h_result, sizeof(hbf_batch_result_t)) != cudaSuccess) return fail(HBF_E_NOMEM);
-    memset(c->h_result, 0, sizeof(hbf_batch_result_t));
-    if (cudaMallocHost(&c->h_hot, 3 * sizeof(float)) != cudaSuccess) return fail(HBF_E_NOMEM);
-    if ((rc = dev_copy(c, &c->bal.dev, nullptr, 1))) return fail(rc);
-    if (cudaMallocHost(&c->bal.pinned, sizeof(TileBalance)) != cudaSuccess) return fail(HBF_E_NOMEM);
-    memset(c->bal.pinned, 0, sizeof(TileBalance));
+    arena.add(&c->d_ranges, nullptr, 1);
+    arena.add(&c->d_mp, nullptr, 1);
+    arena.add(&c->d_state, &st0, 1);
+    arena.add(&c->d_ctrl, nullptr, 1);
+    arena.add(&c->d_result, nullptr, 1);
+    arena.add(&c->d_busy, nullptr, nq);
+    arena.add(&c->d_busy_stage, nullptr, nq);
+    arena.add(&c->d_pending, nullptr, nd);
+    arena.add(&c->d_stats_stage, nullptr, nd);
+    arena.add(&c->bal.dev, nullptr, 1);
+    if (cudaMallocHost(&c->pinned, sizeof(hbf_ctx::Pinned)) != cudaSuccess) return fail(HBF_E_NOMEM);
+    memset(c->pinned, 0, sizeof(hbf_ctx::Pinned));
+    c->bal.pinned = &c->pinned->bal;
 
+    std::vector<float> inv_cells; std::vector<int32_t> ptr, list;      // (their contents are copied by the commit below)
     c->thermal = cfg->cell_C != nullptr;
     if (c->thermal) {
         if (!cfg->grid_h || !cfg->grid_w || !cfg->n_sub || !cfg->n_regions || !cfg->cell_Gx || !cfg->cell_Gy ||
@@ -341,7 +353,7 @@ int hbf_create(const hbf_config_t *cfg, void *cuda_stream, hbf_ctx **out) {
         const uint32_t H = cfg->grid_h, W = cfg->grid_w, NR = cfg->n_regions;
         const size_t nc = (size_t)H * W;
         if (nc > (1u << 30)) return fail(HBF_E_INVAL);
-        std::vector<float> inv_cells(NR, 0.0f); std::vector<double> cells(NR, 0.0);
+        inv_cells.assign(NR, 0.0f); std::vector<double> cells(NR, 0.0);
         double lim = INFINITY;
         for (uint32_t y = 0; y < H; ++y) for (uint32_t x = 0; x < W; ++x) {
             const size_t i = (size_t)y * W + x;
@@ -357,7 +369,7 @@ int hbf_create(const hbf_config_t *cfg, void *cuda_stream, hbf_ctx **out) {
             if (gs > 0.0) lim = std::min(lim, (double)cfg->cell_C[i] / gs);
         }
         c->euler_limit_s = lim;
-        std::vector<int32_t> ptr(NR + 1, 0), list(nd);
+        ptr.assign(NR + 1, 0); list.resize(nd);
         for (uint64_t d = 0; d < nd; ++d) {
             const int32_t g = cfg->die_region[d];
             if (g < 0 || g >= (int32_t)NR || cells[g] == 0.0) return fail(HBF_E_INVAL);
@@ -371,33 +383,20 @@ int hbf_create(const hbf_config_t *cfg, void *cuda_stream, hbf_ctx **out) {
         auto mk = [](float v) { return (int64_t)std::floor((double)v * 1000.0 + 0.5); };
         t.rtt_mk = mk(cfg->rtt_c); t.ltt_mk = mk(cfg->ltt_c); t.stt_mk = mk(cfg->stt_c); t.shut_mk = mk(cfg->shutdown_c);
         t.q_light_ppm = cfg->q_light_ppm;
-        float *p;
-        int32_t *q;
-        double *dp;
-        if ((rc = dev_copy(c, &p, cfg->cell_C, nc))) return fail(rc); t.C = p;
-        if ((rc = dev_copy(c, &p, cfg->cell_Gx, nc))) return fail(rc); t.Gx = p;
-        if ((rc = dev_copy(c, &p, cfg->cell_Gy, nc))) return fail(rc); t.Gy = p;
-        if ((rc = dev_copy(c, &p, cfg->cell_Gsink, nc))) return fail(rc); t.Gs = p;
-        if ((rc = dev_copy(c, &q, cfg->cell_region, nc))) return fail(rc); t.cell_region = q;
-        if ((rc = dev_copy(c, &q, cfg->die_region, nd))) return fail(rc); t.die_region = q;
-        if ((rc = dev_copy(c, &q, cfg->region_kind, NR))) return fail(rc); t.region_kind = q;
-        if ((rc = dev_copy(c, &p, cfg->region_idle_w, NR))) return fail(rc); t.region_idle_w = p;
-        if ((rc = dev_copy(c, &p, inv_cells.data(), NR))) return fail(rc); t.region_inv_cells = p;
-        if ((rc = dev_copy(c, &q, ptr.data(), NR + 1))) return fail(rc); t.region_die_ptr = q;
-        if ((rc = dev_copy(c, &q, list.data(), nd))) return fail(rc); t.region_die_list = q;
-        if ((rc = dev_copy(c, &t.theta[0], nullptr, nc))) return fail(rc);
-        if ((rc = dev_copy(c, &t.theta[1], nullptr, nc))) return fail(rc);
-        if ((rc = dev_copy(c, &t.comp, nullptr, nc))) return fail(rc);
-        if ((rc = dev_copy(c, &t.P, nullptr, nc))) return fail(rc);
-        if ((rc = dev_copy(c, &dp, nullptr, NR))) return fail(rc); t.region_power = dp;
-        if ((rc = dev_copy(c, &t.ext_power, nullptr, NR))) return fail(rc);
-        if ((rc = dev_copy(c, &t.hot, nullptr, 3))) return fail(rc);
-        if (cudaMallocHost(&c->h_ext, NR * sizeof(float)) != cudaSuccess) return fail(HBF_E_NOMEM);
+        arena.add(&t.C, cfg->cell_C, nc); arena.add(&t.Gx, cfg->cell_Gx, nc); arena.add(&t.Gy, cfg->cell_Gy, nc); arena.add(&t.Gs, cfg->cell_Gsink, nc);
+        arena.add(&t.cell_region, cfg->cell_region, nc); arena.add(&t.die_region, cfg->die_region, nd); arena.add(&t.region_kind, cfg->region_kind, NR);
+        arena.add(&t.region_idle_w, cfg->region_idle_w, NR); arena.add(&t.region_inv_cells, inv_cells.data(), NR);
+        arena.add(&t.region_die_ptr, ptr.data(), NR + 1); arena.add(&t.region_die_list, list.data(), nd);
+        arena.add(&t.theta[0], nullptr, nc); arena.add(&t.theta[1], nullptr, nc); arena.add(&t.comp, nullptr, nc); arena.add(&t.P, nullptr, nc);
+        arena.add(&t.region_power, nullptr, NR); arena.add(&t.ext_power, nullptr, NR);
+        arena.add(&t.hot, nullptr, 4);
         // the descriptor keeps no pointer into the caller's arrays
         c->cfg.cell_C = c->cfg.cell_Gx = c->cfg.cell_Gy = c->cfg.cell_Gsink = c->cfg.region_idle_w = nullptr;
         c->cfg.cell_region = c->cfg.die_region = c->cfg.region_kind = nullptr;
     }
-    if (cudaDeviceSynchronize() != cudaSuccess) return fail(HBF_E_CUDA);
+    if ((rc = arena.commit(c)) != HBF_OK) return fail(rc);
+    mp.xfer_tab = tab_dev;
+    if (cudaMemcpy(c->d_mp, &mp, sizeof(mp), cudaMemcpyHostToDevice) != cudaSuccess) return fail(HBF_E_CUDA);
     *out = c;
     return HBF_OK;
 }
@@ -472,6 +471,7 @@ int hbf_set_head_entries(hbf_ctx *c, uint32_t entries) {
 // accesses) and hbf_submit_batch_paged (the list of parts).
 static int serve_records(hbf_ctx *c, SubmitArgs &a) {
     a.ranges = c->d_ranges; a.mp_dev = c->d_mp; a.mp = c->mp; a.state = c->d_state; a.ctrl = c->d_ctrl; a.result = c->d_result;
+    a.result_host = &c->pinned->result; a.plain_next = &c->plain_next;
     a.busy = c->d_busy; a.busy_stage = c->d_busy_stage; a.pending = c->d_pending; a.stats_stage = c->d_stats_stage;
     a.path = a.paged ? (int32_t)HBF_PATH_INORDER : c->path; a.sm_count = c->sm_count; a.inorder_ok = c->inorder_ok ? 1 : 0;
     if (c->ranges.size() == 1) {
@@ -481,11 +481,13 @@ static int serve_records(hbf_ctx *c, SubmitArgs &a) {
     a.binned = c->bin_ns != 0; a.bus_on = c->d_bus_busy ? 1 : 0;
     a.bal = &c->bal;
     if (c->ret_on) { a.claim_limit = &c->ret.st->claim_limit; a.die_claims = c->ret.die_claims; a.ret = &c->ret; }
+    c->result_on_host = true;
     if (small_route(a)) {                                    // one launch, everything included (with the bus on it stops before the ledger)
         auto mark = [&](int k) { if (a.ev) cudaEventRecord(a.ev[k], c->stream); };
         mark(0); mark(7);
         CK(launch_small(a, SmallExtras{a.binned ? c->d_ledger : nullptr, c->bin_ns, c->cur_bin, c->n_bins}, c->stream));
         mark(8); for (int k = 1; k <= 6; ++k) mark(k);
+        c->result_on_host = false;
         if (!a.bus_on) return HBF_OK;
     } else {
         if (c->ret_on)                                       // how far the outstanding refresh quanta reach into this batch
@@ -640,8 +642,7 @@ int hbf_submit_batch_paged(hbf_ctx *c, const hbf_access_t *d_acc, uint64_t n, ui
     bool by_unit = c->inorder_ok && (c->path == HBF_PATH_AUTO || c->path == HBF_PATH_INORDER) && !c->bin_ns && !c->d_bus_busy && !c->ret_on &&
                    n > kInSmallMax && c->mp.stripe_shift < 31u;
     // how many parts: the one point where the host waits for the device inside a submit
-    unsigned long long *h_total = reinterpret_cast<unsigned long long *>(c->h_result);     // pinned, free between calls
-    static_assert(sizeof(hbf_batch_result_t) >= kPagedTotals * sizeof(unsigned long long), "the totals fit where the result goes");
+    unsigned long long *h_total = c->pinned->totals;
     auto count = [&](bool unit) -> int {
         CK(launch_paged_count(d_acc, n, c->d_ranges, c->d_mp, fast, c->mp, c->d_state, unit, pw, c->stream));
         CK(cudaMemcpyAsync(h_total, pw.total, kPagedTotals * sizeof(unsigned long long), cudaMemcpyDeviceToHost, c->stream));
@@ -676,7 +677,7 @@ int hbf_submit_batch_paged(hbf_ctx *c, const hbf_access_t *d_acc, uint64_t n, ui
     a.paged = by_unit ? 1 : 0;
     a.ev = nullptr;
     if ((rc = serve_records(c, a)) != HBF_OK) return rc;
-    CK(launch_paged_join(d_acc, n, pw, c->d_result, d_completion_ns, d_stall_ns, d_status, c->sm_count, c->stream));
+    CK(launch_paged_join(d_acc, n, pw, c->d_result, &c->pinned->result, d_completion_ns, d_stall_ns, d_status, c->sm_count, c->stream));
     c->submitted = true;
     return HBF_OK;
 }
@@ -838,9 +839,10 @@ int hbf_get_energy_bins(hbf_ctx *c, int64_t *host_out, uint64_t cap, int64_t *fi
 int hbf_last_result(hbf_ctx *c, hbf_batch_result_t *host_out) {
     if (!c || !host_out) return HBF_E_INVAL;
     if (!c->submitted) { memset(host_out, 0, sizeof(*host_out)); return HBF_OK; }
-    CK(cudaMemcpyAsync(c->h_result, c->d_result, sizeof(hbf_batch_result_t), cudaMemcpyDeviceToHost, c->stream));
-    CK(cudaStreamSynchronize(c->stream));
-    *host_out = *c->h_result;
+    if (!c->result_on_host) CK(cudaMemcpyAsync(&c->pinned->result, c->d_result, sizeof(hbf_batch_result_t), cudaMemcpyDeviceToHost, c->stream));
+    c->result_on_host = true;
+    CK(cudaStreamSynchronize(c->stream));                    // (a large batch's last kernel wrote its summary to the host)
+    *host_out = c->pinned->result;
     if (host_out->code == HBF_E_LINK_SHUTDOWN) c->terminal = true;
     return host_out->code;
 }
@@ -862,6 +864,8 @@ int hbf_thermal_step(hbf_ctx *c, int64_t dt_ns, const float *ext_power_w, uint32
     if (!c || !c->thermal || dt_ns <= 0 || !on_own_device(c)) return HBF_E_INVAL;
     if (n_ext != 0 && (n_ext != c->td.n_regions || !ext_power_w)) return HBF_E_INVAL;
     const double dt_sub = (double)dt_ns * 1e-9 / (double)c->td.n_sub;
+    ThermalDev td = c->td;
+    if (hot_c_out) td.hot = c->pinned->hot;                  // the step's last store goes straight to the host (a microsecond more: only when it is asked for)
     // every refusal comes before the first enqueue: a refused call leaves the ledger, the clock and the stream as they were
     if (!c->rom && dt_sub > c->euler_limit_s) return HBF_E_INVAL;
     if (c->bin_ns && dt_ns != c->bin_ns) return HBF_E_INVAL;
@@ -877,17 +881,16 @@ int hbf_thermal_step(hbf_ctx *c, int64_t dt_ns, const float *ext_power_w, uint32
     if (c->profiling) CK(cudaEventRecord(c->ev_th[0], c->stream));
     if (c->rom) {                                            // the attached model stands in for the grid
         if (bin_row) CK(launch_take_bin(bin_row, c->d_pending, c->mp.n_dies, c->stream));
-        CK(launch_rom_power(c->td, c->d_pending, dt_ns, n_ext != 0, c->d_rom_p, c->stream));
+        CK(launch_rom_power(td, c->d_pending, dt_ns, n_ext != 0, c->d_rom_p, c->stream));
         { const int rc_ = hbf_rom_step(c->rom, c->d_rom_p, 1, c->d_rom_T); if (rc_ != HBF_OK) return rc_; }
-        CK(launch_rom_controller(c->td, c->d_rom_T, c->d_rom_kind, hbf_rom_outputs(c->rom), c->d_state, c->stream));
+        CK(launch_rom_controller(td, c->d_rom_T, c->d_rom_kind, hbf_rom_outputs(c->rom), c->d_state, c->stream));
     } else {
-        CK(launch_thermal_step(c->td, c->d_state, c->d_pending, bin_row, dt_ns, n_ext != 0, d_temps_out, &c->cur, c->thermal_generic ? 1 : 0, c->stream));
+        CK(launch_thermal_step(td, c->d_state, c->d_pending, bin_row, dt_ns, n_ext != 0, d_temps_out, &c->cur, c->thermal_generic ? 1 : 0, &c->plain_next, c->stream));
     }
     if (c->profiling) { CK(cudaEventRecord(c->ev_th[1], c->stream)); c->prof_thermal = true; }
     if (hot_c_out) {
-        CK(cudaMemcpyAsync(c->h_hot, c->td.hot, 3 * sizeof(float), cudaMemcpyDeviceToHost, c->stream));
         CK(cudaStreamSynchronize(c->stream));
-        memcpy(hot_c_out, c->h_hot, 3 * sizeof(float));
+        memcpy(hot_c_out, c->pinned->hot, 3 * sizeof(float));
     }
     return HBF_OK;
 }
@@ -928,24 +931,27 @@ int hbf_get_mode(hbf_ctx *c, int32_t *mode, int64_t *q_ppm) {
 
 int hbf_reset(hbf_ctx *c) {
     if (!c) return HBF_E_INVAL;
-    DevState s; s.mode = HBF_MODE_NORMAL; s.poisoned = 0; s.q_ppm = 1000000;
-    s.spin_limit = c->spin_limit; s.test_stage = c->test_stage; s.test_tile = c->test_tile; s.pad = 0;
-    CK(cudaStreamSynchronize(c->stream));
-    CK(cudaMemcpyAsync(c->d_state, &s, sizeof(s), cudaMemcpyHostToDevice, c->stream));
-    CK(cudaMemsetAsync(c->d_busy, 0, c->mp.n_queues * sizeof(int64_t), c->stream));
-    CK(cudaMemsetAsync(c->d_pending, 0, c->mp.n_dies * sizeof(int64_t), c->stream));
-    CK(cudaMemsetAsync(c->d_result, 0, sizeof(hbf_batch_result_t), c->stream));
-    if (c->bin_ns) { CK(cudaMemsetAsync(c->d_ledger, 0, (size_t)c->n_bins * c->mp.n_dies * 8, c->stream)); c->cur_bin = 0; }
-    if (c->d_bus_busy) CK(cudaMemsetAsync(c->d_bus_busy, 0, (size_t)c->mp.channels * 8, c->stream));
-    if (c->ret_on) { int rc = retention_clear(c); if (rc != HBF_OK) return rc; }
+    ResetArgs r{};
+    r.initial.mode = HBF_MODE_NORMAL; r.initial.q_ppm = 1000000;
+    r.initial.spin_limit = c->spin_limit; r.initial.test_stage = c->test_stage; r.initial.test_tile = c->test_tile;
+    r.state = c->d_state; r.result = c->d_result; r.result_host = &c->pinned->result;
+    auto clear = [&](void *at, size_t bytes) { r.seg[r.count].at = at; r.seg[r.count].bytes = bytes; ++r.count; };
+    clear(c->d_busy, c->mp.n_queues * sizeof(int64_t));
+    clear(c->d_pending, c->mp.n_dies * sizeof(int64_t));
+    if (c->bin_ns) { clear(c->d_ledger, (size_t)c->n_bins * c->mp.n_dies * 8); c->cur_bin = 0; }
+    if (c->d_bus_busy) clear(c->d_bus_busy, (size_t)c->mp.channels * 8);
+    if (c->ret_on) {
+        const RetDev &t = c->ret;
+        clear(t.damage, t.n_blocks * 8); clear(t.disturb, t.n_blocks * 4); clear(t.pec, t.n_blocks * 4); clear(t.epoch_of, t.n_blocks * 4);
+        clear(t.worn, t.n_blocks); clear(t.die_claims, (size_t)c->mp.n_dies * 4); clear(t.st, sizeof(RetState));
+    }
     if (c->thermal) {
         const size_t nc = (size_t)c->td.H * c->td.W;
-        CK(cudaMemsetAsync(c->td.theta[0], 0, nc * sizeof(float), c->stream));
-        CK(cudaMemsetAsync(c->td.theta[1], 0, nc * sizeof(float), c->stream));
-        CK(cudaMemsetAsync(c->td.comp, 0, nc * sizeof(float), c->stream));
+        clear(c->td.theta[0], nc * sizeof(float)); clear(c->td.theta[1], nc * sizeof(float)); clear(c->td.comp, nc * sizeof(float));
         c->cur = 0;
     }
-    CK(cudaStreamSynchronize(c->stream));
+    c->result_on_host = true;
+    CK(launch_reset(r, &c->plain_next, c->stream));          // one launch, in stream order: nothing waits for it here
     c->terminal = false;
     return HBF_OK;
 }

@@ -110,7 +110,8 @@ struct SubmitArgs {
     const hbf_access_t *acc; uint64_t n;
     int64_t *completion, *stall; uint8_t *status; hbf_die_stats_t *die_stats;
     const RangeSnap *ranges; const ModelParams *mp_dev; ModelParams mp;
-    DevState *state; BatchCtrl *ctrl; hbf_batch_result_t *result;
+    DevState *state; BatchCtrl *ctrl; hbf_batch_result_t *result, *result_host;   // (result_host: pinned, the same summary for the caller)
+    bool *plain_next;                    // see launch_first
     int64_t *busy, *busy_stage, *pending; hbf_die_stats_t *stats_stage;
     Workspace ws; int32_t path; int sm_count; int inorder_ok;
     FastRange fast;
@@ -123,6 +124,18 @@ struct SubmitArgs {
     cudaEvent_t *ev;                     // [kProfEvents] or null: recorded between kernel groups
     TileBalanceHost *bal;                // tile sizes from measurements (null: off)
 };
+// what the last kernel of a batch needs
+struct FinishArgs {
+    uint64_t n; BatchCtrl *ctrl; DevState *state; int64_t *busy; const int64_t *busy_stage; int64_t *pending; const hbf_die_stats_t *stats_stage;
+    hbf_die_stats_t *die_stats; int64_t *completion, *stall; hbf_batch_result_t *result, *result_host; const ModelParams *mp;
+    uint32_t n_queues, n_dies; int binned, bus_on;
+};
+// hbf_reset: memory to clear, and the state that is not zero
+struct ResetArgs {
+    struct { void *at; size_t bytes; } seg[16]; uint32_t count;
+    DevState *state; DevState initial; hbf_batch_result_t *result, *result_host;
+};
+cudaError_t launch_reset(const ResetArgs &r, bool *plain_next, cudaStream_t st);
 constexpr int kProfEvents = 10;
 extern std::atomic<unsigned long long> g_kernel_launches;
 // The dynamic shared memory a kernel may use is an attribute of the (device, kernel) pair: raises it on the current device
@@ -137,6 +150,17 @@ inline cudaError_t launch_pdl(Kernel k, dim3 grid, dim3 block, size_t smem, cuda
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization; at[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at; cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, k, args...);
+}
+// the first kernel of a call: the same, unless what the context enqueued last may still launch kernels of its own (*plain_next)
+template <class Kernel, class... Args>
+inline cudaError_t launch_first(bool *plain_next, Kernel k, dim3 grid, dim3 block, size_t smem, cudaStream_t st, const Args &...args) {
+    if (plain_next && *plain_next) {
+        *plain_next = false;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = st;
+        return cudaLaunchKernelEx(&cfg, k, args...);
+    }
+    return launch_pdl(k, grid, block, smem, st, args...);
 }
 
 constexpr uint32_t kInMaxQueues = 2048;  // the in-order path keeps per-queue state in shared memory
@@ -222,7 +246,7 @@ cudaError_t launch_paged_offsets(uint64_t n, const PagedWorkspace &pw, cudaStrea
 cudaError_t launch_paged_expand(const hbf_access_t *acc, uint64_t n, const RangeSnap *ranges, const ModelParams *mp_dev,
                                 const FastRange &fast, uint32_t cut_shift, uint64_t capacity, const PagedWorkspace &pw, int sm_count,
                                 cudaStream_t st);
-cudaError_t launch_paged_join(const hbf_access_t *acc, uint64_t n, const PagedWorkspace &pw, hbf_batch_result_t *result,
+cudaError_t launch_paged_join(const hbf_access_t *acc, uint64_t n, const PagedWorkspace &pw, hbf_batch_result_t *result, hbf_batch_result_t *result_host,
                               int64_t *completion, int64_t *stall, uint8_t *status, int sm_count, cudaStream_t st);
 
 // ---- time-bin energy ledger ----------------------------------------------------------------------------
@@ -289,7 +313,7 @@ struct ThermalDev {
 };
 // bin_row: the ledger's bin that the step takes besides the pending totals (null without the time bins)
 cudaError_t launch_thermal_step(const ThermalDev &t, DevState *state, int64_t *pending, unsigned long long *bin_row, int64_t dt_ns,
-                                int has_ext, float *d_temps_out, int *cur, int generic_only, cudaStream_t st);
+                                int has_ext, float *d_temps_out, int *cur, int generic_only, bool *plain_next, cudaStream_t st);
 
 cudaError_t launch_rom_power(const ThermalDev &t, int64_t *pending, int64_t dt_ns, int has_ext, double *p_out, cudaStream_t st);
 cudaError_t launch_rom_controller(const ThermalDev &t, const double *temps, const int32_t *kind, uint32_t n_out, DevState *state,

@@ -469,6 +469,8 @@ k_inorder_serve(const hbf_access_t *__restrict__ acc, uint64_t n, const __grid_c
     __shared__ ModelParams mp;                            // measured: reads from shared memory beat reads of the argument
     __shared__ FastRange fast_range;
 
+    pdl_wait();
+    pdl_trigger();
     if (ctrl->skip || ctrl->run_sort) return;             // (run_sort set this early: the batch went to the sort path at its start)
     if (RESERVE && (!ctrl->inorder_used || !in_tile[blockIdx.x].reserve)) return;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -900,6 +902,8 @@ k_inorder_scan(BatchCtrl *ctrl, const ModelParams *__restrict__ mp, uint32_t n_t
                int64_t *__restrict__ in_bin, const int64_t *__restrict__ busy, int64_t *__restrict__ busy_stage,
                hbf_die_stats_t *stats_stage, int forced) {
     __shared__ longlong2 s_map[kInScanChunks][kInScanQueues];
+    pdl_wait();
+    pdl_trigger();
     if (ctrl->skip || ctrl->run_sort) return;
     const bool fault = ctrl->n_fault != 0, unsorted = ctrl->unsorted != 0u;   // settled by the serve pass: every thread sees the same
     if (blockIdx.x == 0 && threadIdx.x == 0 && threadIdx.y == 0) {
@@ -1029,6 +1033,8 @@ k_inorder_fixstraggle(const hbf_access_t *__restrict__ acc, uint64_t n, const __
     __shared__ int s_open;                                   // those whose two runs have not met yet
     __shared__ long long s_red[2];
 
+    pdl_wait();
+    pdl_trigger();
     if (ctrl->skip || ctrl->run_sort || !ctrl->inorder_used) return;
     const uint32_t tile = blockIdx.x;
     if (tile == 0u) return;                                  // the first tile was served from its true entering state
@@ -1476,18 +1482,21 @@ cudaError_t launch_inorder(const SubmitArgs &a, cudaStream_t st) {
         auto k = a.paged ? (reserve ? k_inorder_serve<true, false, true> : k_inorder_serve<false, false, true>)
                : reserve ? (debt ? k_inorder_serve<true, true, false> : k_inorder_serve<true, false, false>)
                          : (debt ? k_inorder_serve<false, true, false> : k_inorder_serve<false, false, false>);
-        k<<<n_tiles, kInThreads, smem_serve, st>>>(a.acc, n, tmap, a.ranges, a.mp, a.fast, a.ctrl, a.status, a.ws.in_agg,
-                                                   a.stats_stage, a.completion, a.stall, a.ws.in_bin, tiles, heads, a.ws.in_headcnt,
-                                                   a.busy, a.claim_limit, a.die_claims, debt ? *a.ret : RetDev{}, a.ws.in_qid, qid_stride,
-                                                   bal ? bal->dev : nullptr, bal_seq, make_fast_geom(a.fast, a.mp), depth);
+        return launch_pdl(k, n_tiles, kInThreads, smem_serve, st, a.acc, n, tmap, a.ranges, a.mp, a.fast, a.ctrl, a.status, a.ws.in_agg,
+                          a.stats_stage, a.completion, a.stall, (const int64_t *)a.ws.in_bin, tiles, heads, a.ws.in_headcnt,
+                          (const int64_t *)a.busy, a.claim_limit, a.die_claims, debt ? *a.ret : RetDev{}, a.ws.in_qid, qid_stride,
+                          bal ? bal->dev : nullptr, bal_seq, make_fast_geom(a.fast, a.mp), depth);
     };
-    serve(false);
-    k_inorder_scan<<<(R + kInScanQueues - 1) / kInScanQueues, dim3(kInScanQueues, kInScanChunks), 0, st>>>(
-        a.ctrl, a.mp_dev, n_tiles, a.ws.in_agg, a.ws.in_bin, a.busy, a.busy_stage, a.stats_stage, a.path == HBF_PATH_INORDER ? 1 : 0);
-    (a.paged ? k_inorder_fixstraggle<false, true> : debt ? k_inorder_fixstraggle<true, false> : k_inorder_fixstraggle<false, false>)<<<n_tiles, kInStrThreads, smem_str, st>>>(
-        a.acc, n, tmap, a.ranges, a.mp, a.fast, a.ctrl, a.ws.in_bin, heads, a.ws.in_headcnt, a.completion, a.stall, tiles,
-        a.claim_limit, a.ws.in_qid, qid_stride, depth, bal ? bal->dev : nullptr);
-    serve(true);
+    cudaError_t le = serve(false);
+    if (le == cudaSuccess)
+        le = launch_pdl(k_inorder_scan, (R + kInScanQueues - 1) / kInScanQueues, dim3(kInScanQueues, kInScanChunks), 0, st, a.ctrl, a.mp_dev, n_tiles,
+                        (const int64_t *)a.ws.in_agg, a.ws.in_bin, (const int64_t *)a.busy, a.busy_stage, a.stats_stage, a.path == HBF_PATH_INORDER ? 1 : 0);
+    if (le == cudaSuccess)
+        le = launch_pdl(a.paged ? k_inorder_fixstraggle<false, true> : debt ? k_inorder_fixstraggle<true, false> : k_inorder_fixstraggle<false, false>, n_tiles, kInStrThreads,
+                        smem_str, st, a.acc, n, tmap, a.ranges, a.mp, a.fast, a.ctrl, (const int64_t *)a.ws.in_bin, (const InHead *)heads, (const uint8_t *)a.ws.in_headcnt,
+                        a.completion, a.stall, tiles, a.claim_limit, (const uint16_t *)a.ws.in_qid, qid_stride, depth, bal ? bal->dev : nullptr);
+    if (le == cudaSuccess) le = serve(true);
+    if (le != cudaSuccess) return le;
     if (bal) {                                               // the tiles' times and straggler counts, for later batches; nothing waits for this copy
         cudaError_t e = cudaMemcpyAsync(bal->pinned, bal->dev, offsetof(TileBalance, first), cudaMemcpyDeviceToHost, st);
         if (e != cudaSuccess) return e;

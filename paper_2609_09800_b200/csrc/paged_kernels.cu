@@ -265,8 +265,8 @@ k_paged_join(uint64_t n, const uint32_t *__restrict__ part_first, const int64_t 
 }
 
 // the summary counts accesses, not parts
-__global__ void k_paged_finish(hbf_batch_result_t *result, const PagedSums *sums) {
-    if (result->code == HBF_OK) { result->n_modeled = sums->n_ready; result->modeled_ns = (int64_t)sums->stall_sum; }
+__global__ void k_paged_finish(hbf_batch_result_t *result, hbf_batch_result_t *result_host, const PagedSums *sums) {
+    if (result->code == HBF_OK) { result->n_modeled = sums->n_ready; result->modeled_ns = (int64_t)sums->stall_sum; *result_host = *result; }
 }
 
 size_t paged_layout(uint64_t n, uint64_t capacity, uint32_t n_queues, PagedWorkspace *pw, void *base_ptr, int with_bus) {
@@ -322,12 +322,12 @@ cudaError_t launch_paged_expand(const hbf_access_t *acc, uint64_t n, const Range
     return cudaGetLastError();
 }
 
-cudaError_t launch_paged_join(const hbf_access_t *acc, uint64_t n, const PagedWorkspace &pw, hbf_batch_result_t *result,
+cudaError_t launch_paged_join(const hbf_access_t *acc, uint64_t n, const PagedWorkspace &pw, hbf_batch_result_t *result, hbf_batch_result_t *result_host,
                               int64_t *completion, int64_t *stall, uint8_t *status, int sm_count, cudaStream_t st) {
     const unsigned grid = (unsigned)std::min<uint64_t>((n + 255) / 256, (uint64_t)std::max(1, sm_count) * 8);
     k_paged_join<<<grid, 256, 0, st>>>(n, pw.part_first, pw.part_completion, pw.part_stall, pw.part_status, result, completion, stall, status,
                                       reinterpret_cast<PagedSums *>(pw.sums));
-    k_paged_finish<<<1, 1, 0, st>>>(result, reinterpret_cast<const PagedSums *>(pw.sums));
+    k_paged_finish<<<1, 1, 0, st>>>(result, result_host, reinterpret_cast<const PagedSums *>(pw.sums));
     g_kernel_launches += 2;
     return cudaGetLastError();
 }

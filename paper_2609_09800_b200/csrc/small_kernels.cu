@@ -453,7 +453,7 @@ k_small_serve(const __grid_constant__ SmallArgs a) {
         r.code = code; r.mode = mode; r.q_ppm = q_ppm;
         r.n_native = seen ? n_native : 0u; r.n_modeled = ok ? n_ready : 0u; r.n_fault = n_fault;
         r.modeled_ns = ok ? modeled : 0; r.service_ns = ok ? service : 0; r.max_completion_ns = ok && n_ready ? latest : 0;
-        *a.result = r;
+        *a.result = r;                                       // (not to the host as well: the kernel would end a microsecond later)
         BatchCtrl *c = a.ctrl;                               // what later stages and hbf_queue_order read of a batch
         c->code = code; c->skip = ok ? 0 : 1; c->mode = mode; c->q_ppm = q_ppm; c->div_q = div_q;
         c->n_ready = n_ready; c->inorder_used = ok && !unsorted ? 1u : 0u; c->run_sort = 0u; c->plan.n_passes = 1u;
@@ -520,7 +520,8 @@ cudaError_t launch_small(const SubmitArgs &a, const SmallExtras &x, cudaStream_t
     cudaLaunchAttribute at[2];
     at[0].id = cudaLaunchAttributeClusterDimension; at[0].val.clusterDim.x = blocks; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
     at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization; at[1].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = at; cfg.numAttrs = 2;
+    cfg.attrs = at; cfg.numAttrs = a.plain_next && *a.plain_next ? 1 : 2;      // (see launch_first)
+    if (a.plain_next) *a.plain_next = false;
     g_kernel_launches += 1;
     return cudaLaunchKernelEx(&cfg, small_kernel(blocks, s.n, s.ledger || s.ret_on), s);
 }

@@ -22,6 +22,8 @@ __global__ void k_begin(BatchCtrl *ctrl, const DevState *state, const int64_t *b
                         hbf_die_stats_t *stats_stage, uint32_t *hist, uint32_t n_queues, uint32_t n_dies,
                         int role, int run_sort, uint32_t *die_claims) {
     const int tid = threadIdx.x;
+    pdl_wait();
+    pdl_trigger();
     if (role == 1) {
         if (ctrl->skip || !ctrl->run_sort) return;
         run_sort = 1;
@@ -33,7 +35,7 @@ __global__ void k_begin(BatchCtrl *ctrl, const DevState *state, const int64_t *b
     if (tid == 0) {
         int32_t mode = state->mode;
         ctrl->mode = mode; ctrl->q_ppm = state->q_ppm;
-        ctrl->div_q = make_div64((uint64_t)state->q_ppm);
+        if (state->q_ppm != 1000000) ctrl->div_q = make_div64((uint64_t)state->q_ppm);   // (a 128-bit division; nothing looks at it without scaling)
         ctrl->key_and = ~0ull;
         ctrl->run_sort = (uint32_t)run_sort;
         if (state->poisoned) { ctrl->code = HBF_E_TIMEOUT; ctrl->skip = 1; }
@@ -698,31 +700,30 @@ k_stalls(const hbf_access_t *__restrict__ acc, uint64_t n, const BatchCtrl *ctrl
 // =====================================================================================================
 // finish: commit the staged state, or zero the outputs of a refused batch; write the batch summary
 // =====================================================================================================
-__global__ void k_finish(uint64_t n, BatchCtrl *ctrl, DevState *state, int64_t *busy, const int64_t *busy_stage,
-                         int64_t *pending, const hbf_die_stats_t *stats_stage, hbf_die_stats_t *die_stats,
-                         int64_t *completion, int64_t *stall, hbf_batch_result_t *result,
-                         const ModelParams *__restrict__ mp, uint32_t n_queues, uint32_t n_dies, int binned, int bus_on) {
+__device__ __forceinline__ void finish_batch(const FinishArgs &f, long long modeled) {
+    BatchCtrl *ctrl = f.ctrl;
+    const uint64_t n = f.n;
     int code = ctrl->code;
     // With the channel-bus stage on, array-done times become sort keys of 47 bits: a batch that reaches 2^47 ns is refused
     // here, before anything is committed (every array-done time is at most the largest completion).  Every thread reads
     // the same settled values, so every thread takes the same decision.
-    if (bus_on && code == HBF_OK && ctrl->n_ready && ctrl->max_completion_ns >= HBF_ISSUE_LIMIT) code = HBF_E_INVAL;
+    if (f.bus_on && code == HBF_OK && ctrl->n_ready && ctrl->max_completion_ns >= HBF_ISSUE_LIMIT) code = HBF_E_INVAL;
     const uint64_t gtid = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (code == HBF_E_TIMEOUT && gtid == 0) state->poisoned = 1;         // a bounded device-side wait expired
+    if (code == HBF_E_TIMEOUT && gtid == 0) f.state->poisoned = 1;       // a bounded device-side wait expired
     const uint64_t gsz = (uint64_t)gridDim.x * blockDim.x;
     if (code == HBF_E_ACCESS_FAULT || code == HBF_E_TIMEOUT || code == HBF_E_INVAL) {
-        for (uint64_t i = gtid; i < n; i += gsz) { completion[i] = 0; stall[i] = 0; }
-        if (die_stats) for (uint64_t i = gtid; i < (uint64_t)n_dies * 6u; i += gsz) reinterpret_cast<int64_t *>(die_stats)[i] = 0;
+        for (uint64_t i = gtid; i < n; i += gsz) { f.completion[i] = 0; f.stall[i] = 0; }
+        if (f.die_stats) for (uint64_t i = gtid; i < (uint64_t)f.n_dies * 6u; i += gsz) reinterpret_cast<int64_t *>(f.die_stats)[i] = 0;
     } else if (code == HBF_OK) {
         const bool inorder = ctrl->inorder_used != 0u;
-        for (uint64_t r = gtid; r < n_queues; r += gsz) busy[r] = busy_stage[r];
-        for (uint64_t d = gtid; d < n_dies; d += gsz) {
-            hbf_die_stats_t ds = stats_stage[d];
+        for (uint64_t r = gtid; r < f.n_queues; r += gsz) f.busy[r] = f.busy_stage[r];
+        for (uint64_t d = gtid; d < f.n_dies; d += gsz) {
+            hbf_die_stats_t ds = f.stats_stage[d];
             // the in-order path keeps byte and access counts only: the energy is linear in them
-            if (inorder) ds.energy_pj = mp->e_cmd_read_pj * ds.n_read + mp->e_byte_read_pj * ds.bytes_read +
-                                        mp->e_cmd_prog_pj * ds.n_prog + mp->e_byte_prog_pj * ds.bytes_prog;
-            if (!binned) pending[d] += ds.energy_pj;          // with the time-bin ledger on, the energy is booked per event
-            if (die_stats) die_stats[d] = ds;
+            if (inorder) ds.energy_pj = f.mp->e_cmd_read_pj * ds.n_read + f.mp->e_byte_read_pj * ds.bytes_read +
+                                        f.mp->e_cmd_prog_pj * ds.n_prog + f.mp->e_byte_prog_pj * ds.bytes_prog;
+            if (!f.binned) f.pending[d] += ds.energy_pj;      // with the time-bin ledger on, the energy is booked per event
+            if (f.die_stats) f.die_stats[d] = ds;
         }
     }
     if (gtid == 0) {
@@ -731,12 +732,13 @@ __global__ void k_finish(uint64_t n, BatchCtrl *ctrl, DevState *state, int64_t *
         r.n_native = code == HBF_OK || code == HBF_E_ACCESS_FAULT ? ctrl->n_native : 0;
         r.n_modeled = code == HBF_OK ? ctrl->n_ready : 0;
         r.n_fault = ctrl->n_fault;
-        r.modeled_ns = code == HBF_OK ? ctrl->modeled_ns : 0;
+        r.modeled_ns = code == HBF_OK ? modeled : 0;
         r.service_ns = code == HBF_OK ? ctrl->service_ns : 0;
         r.max_completion_ns = code == HBF_OK && ctrl->n_ready ? ctrl->max_completion_ns : 0;
-        *result = r;
+        *f.result = r; *f.result_host = r;
     }
 }
+__global__ void k_finish(const __grid_constant__ FinishArgs f) { finish_batch(f, f.ctrl->modeled_ns); }
 
 // copy of the served order out of the workspace (sort path only)
 __global__ void k_queue_order(const BatchCtrl *ctrl, const uint32_t *idx0, const uint32_t *idx1, uint32_t *out, uint64_t n) {
@@ -980,11 +982,12 @@ k_bus_commit(const BatchCtrl *bc, const uint64_t *k0, const uint64_t *k1, const 
     }
 }
 
-__global__ void k_bus_finish(const BatchCtrl *bc, hbf_batch_result_t *result, DevState *state) {
-    if (bc->code != HBF_OK) { result->code = bc->code; state->poisoned = 1; return; }   // the array stage is committed: the context cannot go on
+__global__ void k_bus_finish(const BatchCtrl *bc, hbf_batch_result_t *result, hbf_batch_result_t *result_host, DevState *state) {
+    if (bc->code != HBF_OK) { result->code = bc->code; *result_host = *result; state->poisoned = 1; return; }   // the array stage is committed: the context cannot go on
     if (bc->skip) return;
     result->modeled_ns += bc->modeled_ns;
     if (bc->max_completion_ns > result->max_completion_ns) result->max_completion_ns = bc->max_completion_ns;
+    *result_host = *result;
 }
 
 cudaError_t launch_bus_stage(const SubmitArgs &a, BatchCtrl *bc, int64_t *bus_busy, cudaStream_t st) {
@@ -1014,7 +1017,7 @@ cudaError_t launch_bus_stage(const SubmitArgs &a, BatchCtrl *bc, int64_t *bus_bu
     k_bus_apply<<<tiles_grid, kBusThreads, 0, st>>>(a.acc, bc, a.ws.keys[0], a.ws.keys[1], a.ws.idx[0], a.ws.idx[1], a.ws.bus_xfer, bus_busy,
                                                     agg, a.completion, a.stall);
     k_bus_commit<<<wide, 256, 0, st>>>(bc, a.ws.keys[0], a.ws.keys[1], a.ws.idx[0], a.ws.idx[1], a.completion, bus_busy);
-    k_bus_finish<<<1, 1, 0, st>>>(bc, a.result, a.state);
+    k_bus_finish<<<1, 1, 0, st>>>(bc, a.result, a.result_host, a.state);
     g_kernel_launches += 10 + kMaxPasses;
     return cudaGetLastError();
 }
@@ -1131,25 +1134,33 @@ __global__ void k_zero_words(uint32_t *p, uint64_t words) {
     for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < words; i += (uint64_t)gridDim.x * blockDim.x) p[i] = 0u;
 }
 
+// The last kernel of a batch on the in-order path: the commit, and the hand-over of a batch that it did not serve.
 // (MAY_SORT = false, for a context whose caller declares issue order: the same kernel without the device-side launches,
 // which cost a kernel that contains them several microseconds even when none is made)
 template <bool MAY_SORT>
-__global__ void __launch_bounds__(256) k_after_inorder(const __grid_constant__ SortChain c) {
-    if (c.ctrl->skip) return;                                // refused: nothing to do
-    if (c.ctrl->inorder_used) {
-        // served in issue order.  Stall total of the batch: per tile the exact sum if it was re-served, else the as-if
-        // sum plus its corrections
+__global__ void __launch_bounds__(256) k_finish_inorder(const __grid_constant__ SortChain c, const __grid_constant__ FinishArgs f) {
+    pdl_wait();
+    if constexpr (!MAY_SORT) pdl_trigger();                  // (what follows a kernel that may launch others is launched plainly)
+    if (!MAY_SORT || c.ctrl->skip || c.ctrl->inorder_used) {
+        // Stall total of the batch: per tile the exact sum if it was re-served, else the as-if sum plus its corrections
+        __shared__ long long s_tot[8];
         long long tot = 0;
-        for (uint32_t t = threadIdx.x; t < c.n_tiles; t += blockDim.x) {
-            const InTile v = c.in_tile[t];
-            tot += v.reserve ? v.true_sum : v.spec_sum + v.fix_delta;
+        if (blockIdx.x == 0) {
+            if (!c.ctrl->skip) for (uint32_t t = threadIdx.x; t < c.n_tiles; t += blockDim.x) {
+                const InTile v = c.in_tile[t];
+                tot += v.reserve ? v.true_sum : v.spec_sum + v.fix_delta;
+            }
+            tot = warp_sum(tot);
+            if ((threadIdx.x & 31) == 0) s_tot[threadIdx.x >> 5] = tot;
+            __syncthreads();
+            tot = 0;
+            for (int w = 0; w < 8; ++w) tot += s_tot[w];
         }
-        tot = warp_sum(tot);
-        if ((threadIdx.x & 31) == 0 && tot) atomicAdd((unsigned long long *)&c.ctrl->modeled_ns, (unsigned long long)tot);
+        finish_batch(f, tot);
         return;
     }
     if constexpr (MAY_SORT) {
-    if (!c.ctrl->run_sort || threadIdx.x != 0) return;
+    if (threadIdx.x != 0 || blockIdx.x != 0) return;
     cudaStream_t st = cudaStreamTailLaunch;
     k_begin<<<1, 1024, 0, st>>>(c.ctrl, c.state, c.busy, c.busy_stage, c.stats_stage, c.hist, c.n_queues, c.n_dies, 1, 1, c.die_claims);
     k_zero_words<<<(unsigned)min((unsigned long long)((c.desc_words + 1023) / 1024), 592ull), 1024, 0, st>>>(c.desc0, c.desc_words);
@@ -1163,10 +1174,21 @@ __global__ void __launch_bounds__(256) k_after_inorder(const __grid_constant__ S
                                                  (ScanDesc *)c.scan_desc, c.busy, c.busy_stage, c.stats_stage, c.completion, c.stall,
                                                  c.claim_limit, c.die_claims);
     k_stalls<<<c.stall_grid, 256, 0, st>>>(c.acc, c.n, c.ctrl, c.completion, c.stall);
+    k_finish<<<gridDim.x, 256, 0, st>>>(f);
     }
 }
 
-static cudaError_t launch_after_inorder(const SubmitArgs &a, bool may_sort, cudaStream_t st) {
+static FinishArgs finish_args(const SubmitArgs &a) {
+    FinishArgs f{};
+    f.n = a.n; f.ctrl = a.ctrl; f.state = a.state; f.busy = a.busy; f.busy_stage = a.busy_stage; f.pending = a.pending;
+    f.stats_stage = a.stats_stage; f.die_stats = a.die_stats; f.completion = a.completion; f.stall = a.stall;
+    f.result = a.result; f.result_host = a.result_host; f.mp = a.mp_dev; f.n_queues = a.mp.n_queues; f.n_dies = a.mp.n_dies;
+    f.binned = a.binned; f.bus_on = a.bus_on;
+    return f;
+}
+static unsigned finish_grid(const SubmitArgs &a) { return (unsigned)std::max<uint64_t>(1, std::min<uint64_t>((a.n + 1023) / 1024, (uint64_t)a.sm_count * 4)); }
+
+static cudaError_t launch_finish_inorder(const SubmitArgs &a, bool may_sort, cudaStream_t st) {
     const uint64_t n = a.n;
     const uint64_t sort_tiles = (n + kSortTile - 1) / kSortTile, scan_tiles = (n + kScanTile - 1) / kScanTile;
     cudaError_t e = ensure_dyn_smem((const void *)k_sort_pass, kSortSmem);   // (an attribute of the kernel: device-side launches use it too)
@@ -1187,7 +1209,9 @@ static cudaError_t launch_after_inorder(const SubmitArgs &a, bool may_sort, cuda
     const InTileMap tmap = inorder_tile_map(n, a.sm_count, a.bal && a.bal->on && a.bal->dev);
     c.in_tile = reinterpret_cast<const InTile *>(a.ws.in_tile);
     c.n_tiles = tmap.n_tiles;
-    if (may_sort) k_after_inorder<true><<<1, 256, 0, st>>>(c); else k_after_inorder<false><<<1, 256, 0, st>>>(c);
+    e = launch_pdl(may_sort ? k_finish_inorder<true> : k_finish_inorder<false>, finish_grid(a), 256, 0, st, c, finish_args(a));
+    if (e != cudaSuccess) return e;
+    if (may_sort && a.plain_next) *a.plain_next = true;      // (kernels that may overlap their predecessor must not overlap one that may launch others)
     g_kernel_launches += 1;
     return cudaGetLastError();
 }
@@ -1200,13 +1224,12 @@ cudaError_t launch_submit(const SubmitArgs &a, cudaStream_t st) {
     auto mark = [&](int k) { if (a.ev) cudaEventRecord(a.ev[k], st); };
     const bool try_inorder = a.inorder_ok && (a.path == HBF_PATH_AUTO || a.path == HBF_PATH_INORDER);
     const bool sort_kernels = a.path != HBF_PATH_INORDER || !a.inorder_ok;
-    {
-        const void *small[] = {(const void *)k_begin, (const void *)k_finish};
-        for (const void *f : small) { cudaError_t e = ensure_dyn_smem(f, 0); if (e != cudaSuccess) return e; }
-    }
     mark(0);
-    k_begin<<<1, 1024, 0, st>>>(a.ctrl, a.state, a.busy, a.busy_stage, a.stats_stage, a.ws.hist, a.mp.n_queues, a.mp.n_dies,
-                               0, try_inorder ? 0 : 1, a.die_claims);
+    {
+        const cudaError_t e = launch_first(a.plain_next, k_begin, 1, 1024, 0, st, a.ctrl, (const DevState *)a.state, (const int64_t *)a.busy, a.busy_stage, a.stats_stage, a.ws.hist,
+                                           a.mp.n_queues, a.mp.n_dies, 0, try_inorder ? 0 : 1, a.die_claims);
+        if (e != cudaSuccess) return e;
+    }
     g_kernel_launches += 1;
     if (n > 0) {
         if (try_inorder) {
@@ -1214,23 +1237,41 @@ cudaError_t launch_submit(const SubmitArgs &a, cudaStream_t st) {
             cudaError_t e = launch_inorder(a, st);
             if (e != cudaSuccess) return e;
             mark(8);
-            e = launch_after_inorder(a, sort_kernels, st);
+            e = launch_finish_inorder(a, sort_kernels, st);
             if (e != cudaSuccess) return e;
-            mark(1); mark(2); mark(3); mark(4);
-        } else {
-            cudaError_t e = launch_sort_path(a, st);
-            if (e != cudaSuccess) return e;
+            mark(1); mark(2); mark(3); mark(4); mark(5); mark(6);
+            return cudaSuccess;
         }
+        cudaError_t e = launch_sort_path(a, st);
+        if (e != cudaSuccess) return e;
     } else {
         mark(1); mark(2); mark(3); mark(4);
     }
     mark(5);
-    const unsigned fin_grid = (unsigned)std::max<uint64_t>(1, std::min<uint64_t>((n + 1023) / 1024, (uint64_t)a.sm_count * 4));
-    k_finish<<<fin_grid, 256, 0, st>>>(n, a.ctrl, a.state, a.busy, a.busy_stage, a.pending, a.stats_stage, a.die_stats,
-                                       a.completion, a.stall, a.result, a.mp_dev, a.mp.n_queues, a.mp.n_dies, a.binned, a.bus_on);
+    k_finish<<<finish_grid(a), 256, 0, st>>>(finish_args(a));
     g_kernel_launches += 1;
     mark(6);
     return cudaGetLastError();
+}
+
+// everything a context holds back to its initial state, in one launch
+__global__ void __launch_bounds__(256) k_reset(const __grid_constant__ ResetArgs r) {
+    pdl_wait();
+    pdl_trigger();
+    const uint64_t gtid = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x, gsz = (uint64_t)gridDim.x * blockDim.x;
+    for (uint32_t k = 0; k < r.count; ++k) {
+        const uint64_t words = r.seg[k].bytes / 4;
+        uint32_t *p = static_cast<uint32_t *>(r.seg[k].at);
+        for (uint64_t i = gtid; i < words; i += gsz) p[i] = 0u;
+        if (gtid < (r.seg[k].bytes & 3u)) reinterpret_cast<unsigned char *>(p + words)[gtid] = 0;
+    }
+    if (gtid == 0) { *r.state = r.initial; hbf_batch_result_t none{}; *r.result = none; *r.result_host = none; }
+}
+cudaError_t launch_reset(const ResetArgs &r, bool *plain_next, cudaStream_t st) {
+    uint64_t most = 0;
+    for (uint32_t k = 0; k < r.count; ++k) most = std::max<uint64_t>(most, r.seg[k].bytes);
+    g_kernel_launches += 1;
+    return launch_first(plain_next, k_reset, (unsigned)std::max<uint64_t>(1, std::min<uint64_t>((most + 1023) / 1024, 592)), 256, 0, st, r);
 }
 
 __global__ void k_add_stats(long long *total, const long long *part, uint32_t words) {

@@ -438,7 +438,7 @@ static int thermal_cluster_blocks(const ThermalDev &t, size_t *smem_bytes) {
 // (1 ms step of the 128 x 128 package, 16 substeps, one after the other: 13.8 us; 25 us while every substep tested eight cells a
 // thread, divided by the row length and ended in a barrier of the whole cluster)
 cudaError_t launch_thermal_step(const ThermalDev &t, DevState *state, int64_t *pending, unsigned long long *bin_row, int64_t dt_ns, int has_ext,
-                                float *d_temps_out, int *cur, int generic_only, cudaStream_t st) {
+                                float *d_temps_out, int *cur, int generic_only, bool *plain_next, cudaStream_t st) {
     const float dt_sub_f = (float)((double)dt_ns * 1e-9 / (double)t.n_sub);
     size_t smem = 0;
     const int blocks = generic_only ? 0 : thermal_cluster_blocks(t, &smem);
@@ -450,7 +450,8 @@ cudaError_t launch_thermal_step(const ThermalDev &t, DevState *state, int64_t *p
         cudaLaunchAttribute at[2];
         at[0].id = cudaLaunchAttributeClusterDimension; at[0].val.clusterDim.x = blocks; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
         at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization; at[1].val.programmaticStreamSerializationAllowed = 1;
-        cfg.attrs = at; cfg.numAttrs = 2;
+        cfg.attrs = at; cfg.numAttrs = *plain_next ? 1 : 2;   // (see launch_first)
+        *plain_next = false;
         float *theta = t.theta[*cur];
         const cudaError_t e = cudaLaunchKernelEx(&cfg, k, t, theta, state, pending, bin_row, dt_ns, has_ext, dt_sub_f, d_temps_out);
         if (e != cudaSuccess) return e;
