@@ -851,11 +851,21 @@ int hbf_queue_order(hbf_ctx *c, const void *d_workspace, uint64_t n, uint32_t *d
     if (!c || !d_workspace || !d_order || !count) return HBF_E_INVAL;
     Workspace ws;
     workspace_layout(n, c->mp.n_queues, &ws, const_cast<void *>(d_workspace));
-    CK(launch_queue_order(c->d_ctrl, ws, d_order, n, c->stream));
     BatchCtrl hc;
     CK(cudaMemcpyAsync(&hc, c->d_ctrl, sizeof(hc), cudaMemcpyDeviceToHost, c->stream));
     CK(cudaStreamSynchronize(c->stream));
-    if (hc.code != HBF_OK || hc.inorder_used) return HBF_E_INVAL;
+    if (hc.code != HBF_OK || (hc.inorder_used && !hc.regrouped)) return HBF_E_INVAL;
+    if (hc.regrouped) {
+        BatchCtrl *bc = nullptr;
+        if (cudaMalloc(&bc, sizeof(BatchCtrl)) != cudaSuccess) return HBF_E_NOMEM;
+        const cudaError_t e = launch_regrouped_order(bc, c->d_state, c->d_ranges, c->d_mp, ws, d_order, n, c->sm_count, c->stream);
+        const cudaError_t f = cudaStreamSynchronize(c->stream);
+        cudaFree(bc);
+        if (e != cudaSuccess || f != cudaSuccess) return HBF_E_CUDA;
+    } else {
+        CK(launch_queue_order(c->d_ctrl, ws, d_order, n, c->stream));
+        CK(cudaStreamSynchronize(c->stream));
+    }
     *count = hc.n_ready;
     return HBF_OK;
 }

@@ -67,7 +67,8 @@ struct BatchCtrl {
     uint32_t unsorted;                   // some record has a smaller issue time than its predecessor
     uint32_t inorder_used;               // the in-order path served this batch
     uint32_t run_sort;                   // the sort path has to serve this batch
-    uint32_t pad1;
+    uint32_t regrouped;                  // the in-order path served it on an ordered copy of the records
+    int64_t issue_lo, issue_hi;          // smallest and largest issue time among the begin kernel's samples
     uint32_t role_count[2];              // in-order serve pass: tiles handed out so far, per size class
     uint32_t tile_counter[kMaxPasses + 2];
     long long modeled_ns, service_ns, max_completion_ns;
@@ -97,6 +98,7 @@ struct Workspace {
     void *in_head;                       // [tiles]: the first 8 accesses of every (tile, queue) for the fix-up: a tile's first entries, then each queue's other seven
     uint8_t *in_headcnt;                 // [tiles][queues]: how many of them exist; 0xff marks a queue for the straggle pass
     uint16_t *in_qid;                    // [tiles][stride]: queue of each of the first records of every tile (0xffff: not modeled), for the straggle pass
+    void *rg_ctrl, *rg_slots, *rg_recs, *rg_idx;   // a batch out of issue order: see regroup.cuh (the slots share memory with keys, idx and terms)
     uint32_t *bus_xfer;                  // [n] transfer time of every read (only with the channel-bus stage on)
     size_t bytes;
 };
@@ -212,6 +214,7 @@ InTileMap inorder_tile_map(uint64_t n, int sm_count, bool by_table);   // by_tab
 struct InTile { long long spec_sum, fix_delta, true_sum; uint32_t reserve; uint32_t stragglers; };
 size_t inorder_head_bytes(uint64_t tiles, uint32_t n_queues);
 size_t inorder_serve_smem(uint32_t n_dies);
+size_t inorder_straggle_smem();
 cudaError_t launch_inorder(const SubmitArgs &a, cudaStream_t st);
 // small batches: one launch that serves and commits the batch, claims, ledger and read disturb included (small_kernels.cu)
 constexpr uint32_t kInSmallMax = 8192;   // records
@@ -224,6 +227,9 @@ cudaError_t launch_add_stats(hbf_die_stats_t *total, const hbf_die_stats_t *part
 // the same for batch summaries: counts and times added, the largest completion, the first code that is not HBF_OK; first != 0 starts over
 cudaError_t launch_add_result(hbf_batch_result_t *sum, const hbf_batch_result_t *part, int first, cudaStream_t st);
 cudaError_t launch_queue_order(const BatchCtrl *ctrl, const Workspace &ws, uint32_t *out, uint64_t n, cudaStream_t st);
+// the same for a batch that was served on an ordered copy: its queue-major order is sorted out only now (bc: a control block of its own)
+cudaError_t launch_regrouped_order(BatchCtrl *bc, DevState *state, const RangeSnap *ranges, const ModelParams *mp, const Workspace &ws, uint32_t *out, uint64_t n,
+                                   int sm_count, cudaStream_t st);
 
 // ---- page-granular submit ---------------------------------------------------------------------------
 struct PagedWorkspace {

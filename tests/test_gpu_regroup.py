@@ -1,0 +1,54 @@
+"""Batches out of issue order on the automatic path: brought into order in buckets by issue time and served by the in-order
+kernels, or handed to the radix sort where the times do not spread; against the oracle, bit for bit."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+from oracle import hbfo
+from paper_2609_09800_b200 import workloads as wl
+
+
+@pytest.fixture(scope="module")
+def hbf():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2609_09800_b200 import build, hbf as mod
+    build.build()
+    return mod
+
+
+@pytest.mark.parametrize("n", [8_193, 24_575, 24_577, 200_003])
+@pytest.mark.parametrize("kind", ["shuffled", "rings", "ties", "bunched", "one time", "long span", "negative", "natives", "fault", "late", "long service", "three ranges"])
+def test_unordered_batches_match_the_oracle(hbf, kind, n):
+    rng = np.random.default_rng(n)
+    w = wl.capacity_mode(n=n, seed=n, rho=0.6)
+    ranges = w.ranges if kind != "three ranges" else [(wl.RANGE_BASE, 1 << 39, 3, 0, 0, 0), (wl.RANGE_BASE + (1 << 39), 1 << 38, 3, 0, 0, 1 << 40), (wl.RANGE_BASE + (3 << 38), 1 << 39, 1, 0, 0, 1 << 41)]
+    g, o = hbf.Context(w.profile), hbfo.Oracle(w.profile)
+    for r in ranges:
+        g.register_range(*r); o.register_range(*r)
+    acc = w.acc.copy()
+    acc["flags"][:n // 2] = (rng.random(n // 2) < 0.1) & (acc["addr"][:n // 2] < wl.RANGE_BASE + (1 << 39))
+    if kind == "ties": acc["issue_ns"] //= 40_000                    # about forty records at a time and 1/64 of the bins of a bucket
+    if kind == "bunched": acc["issue_ns"][n // 2:] = acc["issue_ns"][n // 2] + np.arange(n - n // 2) // 500
+    if kind == "one time": acc["issue_ns"][1:] = 77
+    if kind == "long span": acc["issue_ns"] *= 1 + (1 << 46) // int(acc["issue_ns"][-1]) // 2
+    order = rng.permutation(n) if kind != "rings" else np.argsort(rng.integers(0, 148, n), kind="stable")
+    if kind == "late":                                              # one record out of place: the samples do not see it
+        order = np.arange(n); order[[n // 3, n // 3 + 700]] = order[[n // 3 + 700, n // 3]]
+    acc = acc[order]
+    if kind == "negative": acc["issue_ns"][5] = -3
+    if kind == "natives": acc["addr"][rng.random(n) < 0.3] = 4096
+    if kind == "fault": acc["bytes"][n - 2] = 0
+    if kind == "long service": acc["bytes"][n // 2] = 1 << 31; acc["flags"][n // 2] = 1; acc["addr"][n // 2] = wl.RANGE_BASE
+    for batch in range(2):
+        rc_o, c_o, s_o, st_o, ds_o = o.submit(acc, check=False)
+        rc_g, c_g, s_g, st_g, ds_g = g.submit_host(acc, check=False)
+        assert rc_g == rc_o and np.array_equal(st_g, st_o) and np.array_equal(c_g, c_o) and np.array_equal(s_g, s_o)
+        assert all(np.array_equal(ds_g[f], ds_o[f]) for f in hbfo.DIE_STATS_DTYPE.names)
+        assert np.array_equal(g.get_busy_until(), o.busy_until()) and g.last_result() == o.last_result()
+        assert np.array_equal(g.get_pending_energy(), o.pending_energy())
+        if rc_o == 0:
+            assert np.array_equal(g.queue_order(n), o.last_order())
+        acc["issue_ns"] += 10_000
