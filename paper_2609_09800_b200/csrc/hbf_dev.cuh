@@ -142,7 +142,8 @@ constexpr int kProfEvents = 10;
 extern std::atomic<unsigned long long> g_kernel_launches;
 // The dynamic shared memory a kernel may use is an attribute of the (device, kernel) pair: raises it on the current device
 // when `bytes` exceeds what this process has set there so far.  Thread-safe.
-cudaError_t ensure_dyn_smem(const void *kernel, size_t bytes);
+// most_shared: as much of the on-chip memory as there is for shared memory.
+cudaError_t ensure_dyn_smem(const void *kernel, size_t bytes, bool most_shared = false);
 // a launch that may begin while the kernel before it still runs: for kernels that pass pdl_wait() (device_utils.cuh) on every path
 template <class Kernel, class... Args>
 inline cudaError_t launch_pdl(Kernel k, dim3 grid, dim3 block, size_t smem, cudaStream_t st, const Args &...args) {

@@ -39,6 +39,10 @@ struct RegroupArgs {
     int64_t *comp, *stall; ulonglong2 *entries;                  // inside the slots' memory, once they have been read
     uint32_t max_buckets, out_buckets; uint64_t zero_words;
 };
+// Where place p of bucket b lies: the buckets' stretches of 32 slots side by side, then their next 32.  All buckets fill at much
+// the same pace, so the places in use at a time lie in some 16 MB; with every bucket's slots in one piece each store fell into
+// another page (scatter 1,054 us for 40 M records, most of it address translation).
+__device__ __forceinline__ uint64_t rg_place(uint32_t buckets, uint32_t b, uint32_t p) { return ((uint64_t)(p >> 5) * buckets + b) * 32u + (p & 31u); }
 inline uint32_t regroup_buckets(uint64_t n) { return (uint32_t)(n / kRgAvg) + kRgSegs + 1u; }
 inline uint32_t regroup_out_buckets(uint64_t n) { return (uint32_t)((n + kRgOut - 1) / kRgOut); }
 inline size_t regroup_slot_bytes(uint64_t n) { return std::max<size_t>((size_t)regroup_buckets(n) * kRgCap * sizeof(RegroupSlot), (size_t)n * 16 + (size_t)regroup_out_buckets(n) * kRgOut * 16 + 512); }
@@ -63,7 +67,7 @@ k_regroup_sample(const hbf_access_t *__restrict__ acc, uint64_t n, const BatchCt
     const int tid = threadIdx.x;
     if (tid < (int)kRgSegs) sh[tid] = 0u;
     // the span that the begin kernel's samples showed, with a margin; stretches of a power of two of nanoseconds
-    const int64_t first = ctrl->issue_lo, last = ctrl->issue_hi, margin = (last - first) / 256 + 1, lo = first - margin;
+    const int64_t first = ctrl->issue_lo, last = ctrl->issue_hi, margin = (last - first) / 128 + 1, lo = first - margin;
     const uint64_t span = (uint64_t)(last - first + 2 * margin);
     uint32_t shift = 0;
     while (((uint64_t)(kRgSegs - 1) << shift) < span) ++shift;
@@ -97,7 +101,7 @@ k_regroup_scatter(const hbf_access_t *__restrict__ acc, uint64_t n, const RangeS
     for (uint32_t k = threadIdx.x; k <= kRgSegs; k += blockDim.x) s_base[k] = r.rg->base[k];
     __syncthreads();
     const int64_t lo = r.rg->lo;
-    const uint32_t shift = r.rg->shift;
+    const uint32_t shift = r.rg->shift, buckets = r.rg->base[kRgSegs];
     for (uint64_t i0 = (uint64_t)blockIdx.x * (256 * kRgScatterItems) + threadIdx.x; i0 < n; i0 += (uint64_t)gridDim.x * (256 * kRgScatterItems)) {
         uint64_t addr[kRgScatterItems], issue[kRgScatterItems], bf[kRgScatterItems];
         uint32_t at[kRgScatterItems], bucket[kRgScatterItems];
@@ -125,7 +129,7 @@ k_regroup_scatter(const hbf_access_t *__restrict__ acc, uint64_t n, const RangeS
             const uint64_t i = i0 + (uint64_t)k * 256;
             if (i < n) {
                 if (at[k] < kRgCap)
-                    asm volatile("st.global.v4.b64 [%0], {%1, %2, %3, %4};" ::"l"(r.slots + (uint64_t)bucket[k] * kRgCap + at[k]), "l"(addr[k]), "l"(issue[k]), "l"(bf[k]), "l"(i) : "memory");
+                    asm volatile("st.global.v4.b64 [%0], {%1, %2, %3, %4};" ::"l"(r.slots + rg_place(buckets, bucket[k], at[k])), "l"(addr[k]), "l"(issue[k]), "l"(bf[k]), "l"(i) : "memory");
                 else r.rg->overflow = 1u;
                 if (status) {
                     const uint32_t bytes = (uint32_t)bf[k], flags = (uint32_t)(bf[k] >> 32);
@@ -176,7 +180,7 @@ __global__ void __launch_bounds__(kRgThreads, 3) k_regroup_sort(RegroupArgs r) {
     if (r.rg->overflow) return;
     for (uint32_t b = blockIdx.x; b < buckets; b += gridDim.x) {
         const uint32_t m = min(r.cursor[b], kRgCap), off = r.offset[b];
-        const RegroupSlot *slot = r.slots + (uint64_t)b * kRgCap;
+        auto slot = [&](uint32_t e) { return r.slots + rg_place(buckets, b, e); };
         __syncthreads();                                     // shared memory of the bucket before is no longer read
         if (tid == 0) { s_min = INT64_MAX; s_max = INT64_MIN; }
         for (uint32_t e = tid; e < kRgBins; e += kRgThreads) s_cnt[e] = 0u;
@@ -185,7 +189,7 @@ __global__ void __launch_bounds__(kRgThreads, 3) k_regroup_sort(RegroupArgs r) {
 #pragma unroll
         for (int k = 0; k < kRgItems; ++k) {
             const uint32_t e = k * kRgThreads + tid;
-            if (e < m) { issue[k] = slot[e].issue; idx[k] = (uint32_t)slot[e].idx; lo = min(lo, (long long)issue[k]); hi = max(hi, (long long)issue[k]); }
+            if (e < m) { issue[k] = slot(e)->issue; idx[k] = (uint32_t)slot(e)->idx; lo = min(lo, (long long)issue[k]); hi = max(hi, (long long)issue[k]); }
         }
         for (int o = 16; o > 0; o >>= 1) { lo = min(lo, __shfl_xor_sync(0xffffffffu, lo, o)); hi = max(hi, __shfl_xor_sync(0xffffffffu, hi, o)); }
         __syncthreads();
@@ -219,23 +223,28 @@ __global__ void __launch_bounds__(kRgThreads, 3) k_regroup_sort(RegroupArgs r) {
 #pragma unroll
         for (int k = 0; k < kRgItems; ++k) {
             const uint32_t e = k * kRgThreads + tid;
-            if (e < m) { const uint32_t p = s_cnt[bin[k] & 0xffffu] + (bin[k] >> 16); s_key[p] = ((uint64_t)(issue[k] - first) << 32) | idx[k]; s_slot[p] = (uint16_t)e; }
+            if (e < m) s_key[s_cnt[bin[k] & 0xffffu] + (bin[k] >> 16)] = ((uint64_t)(issue[k] - first) << 32) | idx[k];
         }
         __syncthreads();
-        for (uint32_t d = tid; d < kRgBins; d += kRgThreads) {                // bins with several records: in order, one by one
-            const uint32_t from = s_cnt[d], to = d + 1u < kRgBins ? s_cnt[d + 1u] : m;
-            if (to - from < 2u) continue;
-            if (to - from > kRgBinMax) { r.rg->overflow = 1u; continue; }
-            for (uint32_t i = from + 1u; i < to; ++i) {
-                const uint64_t key = s_key[i]; const uint16_t sl = s_slot[i];
-                uint32_t j = i;
-                while (j > from && s_key[j - 1u] > key) { s_key[j] = s_key[j - 1u]; s_slot[j] = s_slot[j - 1u]; --j; }
-                s_key[j] = key; s_slot[j] = sl;
+        bool over = false;
+        // a record's place within its bin: how many of the bin's keys are smaller (a bin rarely has more than four)
+#pragma unroll
+        for (int k = 0; k < kRgItems; ++k) {
+            const uint32_t e = k * kRgThreads + tid;
+            if (e < m) {
+                const uint32_t d = bin[k] & 0xffffu, from = s_cnt[d], to = d + 1u < kRgBins ? s_cnt[d + 1u] : m;
+                uint32_t before = 0;
+                if (to - from > kRgBinMax) over = true;
+                else if (to - from > 1u) {
+                    const uint64_t key = ((uint64_t)(issue[k] - first) << 32) | idx[k];
+                    for (uint32_t q = from; q < to; ++q) before += s_key[q] < key ? 1u : 0u;
+                }
+                s_slot[from + before] = (uint16_t)e;
             }
         }
-        __syncthreads();
+        if (__syncthreads_or(over)) { if (tid == 0) r.rg->overflow = 1u; return; }
         for (uint32_t j = tid; j < m; j += kRgThreads) {
-            const RegroupSlot *p = slot + s_slot[j];
+            const RegroupSlot *p = slot(s_slot[j]);
             uint64_t w0, w1, w2, w3;
             asm volatile("ld.global.v4.b64 {%0, %1, %2, %3}, [%4];" : "=l"(w0), "=l"(w1), "=l"(w2), "=l"(w3) : "l"(p));
             uint64_t *o = r.recs + (uint64_t)(off + j) * 3;
@@ -258,7 +267,7 @@ __global__ void __launch_bounds__(256) k_regroup_give(uint64_t n, const BatchCtr
         for (int k = 0; k < 4; ++k) if (i0 + (uint64_t)k * 256 < n) at[k] = atomicAdd(&r.cursor_out[idx[k] / kRgOut], 1u);
 #pragma unroll
         for (int k = 0; k < 4; ++k)
-            if (i0 + (uint64_t)k * 256 < n) r.entries[(uint64_t)(idx[k] / kRgOut) * kRgOut + at[k]] = make_ulonglong2(comp[k], idx[k] % kRgOut);   // (a permutation: no more than kRgOut each)
+            if (i0 + (uint64_t)k * 256 < n) r.entries[rg_place(r.out_buckets, idx[k] / kRgOut, at[k])] = make_ulonglong2(comp[k], idx[k] % kRgOut);   // (a permutation: no more than kRgOut each)
     }
 }
 
@@ -272,7 +281,7 @@ __global__ void __launch_bounds__(1024) k_regroup_place(const hbf_access_t *__re
         const uint64_t base = (uint64_t)b * kRgOut;
         const uint32_t m = (uint32_t)min((uint64_t)kRgOut, n - base);
         __syncthreads();
-        for (uint32_t e = threadIdx.x; e < m; e += 1024u) { const ulonglong2 v = __ldcs(r.entries + base + e); s_comp[v.y] = (int64_t)v.x; }
+        for (uint32_t e = threadIdx.x; e < m; e += 1024u) { const ulonglong2 v = __ldcs(r.entries + rg_place(r.out_buckets, b, e)); s_comp[v.y] = (int64_t)v.x; }
         __syncthreads();
         for (uint32_t e = threadIdx.x; e < m; e += 1024u) {
             const int64_t c = s_comp[e], issue = (int64_t)__ldcs(reinterpret_cast<const uint64_t *>(acc + base + e) + 1);

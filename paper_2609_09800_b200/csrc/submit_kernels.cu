@@ -18,7 +18,7 @@ namespace hbf {
 // role 0: first kernel of a batch; run_sort tells whether the sort path serves it.
 // role 1: placed between the in-order attempt and the sort kernels; it starts the batch over for the
 //         sort path when the in-order attempt found the records out of issue order, else does nothing.
-// acc != null: 4,096 pairs of neighbouring records are compared first; a batch that they show to be out of order is not attempted
+// acc != null: 1,024 pairs of neighbouring records are compared first; a batch that they show to be out of order is not attempted
 // on the in-order path (an attempt that finds out by itself took 2.7 of the 8.2 ms of 40 M shuffled records).
 __global__ void k_begin(BatchCtrl *ctrl, const DevState *state, const int64_t *busy, int64_t *busy_stage,
                         hbf_die_stats_t *stats_stage, uint32_t *hist, uint32_t n_queues, uint32_t n_dies,
@@ -38,20 +38,12 @@ __global__ void k_begin(BatchCtrl *ctrl, const DevState *state, const int64_t *b
         __shared__ long long s_lo, s_hi;
         if (tid == 0) { s_lo = INT64_MAX; s_hi = INT64_MIN; }
         long long lo = INT64_MAX, hi = INT64_MIN;
-        int64_t v[4][2];
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {                        // (blocks of 1,024 threads; n >= 2)
-            const uint64_t p = ((uint64_t)tid * 4u + k) * (n - 1ull) / 4096ull;
-            const uint64_t *rec = reinterpret_cast<const uint64_t *>(acc + p);
-            v[k][0] = (int64_t)__ldg(rec + 1); v[k][1] = (int64_t)__ldg(rec + 4);
-        }
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            bad = bad || v[k][1] < v[k][0] || (k > 0 && v[k][0] < v[k - 1][0]);
-            lo = min(lo, (long long)min(v[k][0], v[k][1])); hi = max(hi, (long long)max(v[k][0], v[k][1]));
-        }
-        const int64_t up = __shfl_up_sync(0xffffffffu, v[3][0], 1);
-        if ((tid & 31) != 0 && v[0][0] < up) bad = true;
+        // (blocks of 1,024 threads, n >= 2; one pair each: one multiprocessor takes 4 us longer to fetch four)
+        const uint64_t *rec = reinterpret_cast<const uint64_t *>(acc + (uint64_t)tid * (n - 1ull) / 1024ull);
+        const int64_t v0 = (int64_t)__ldg(rec + 1), v1 = (int64_t)__ldg(rec + 4);
+        const int64_t up = __shfl_up_sync(0xffffffffu, v0, 1);
+        bad = v1 < v0 || ((tid & 31) != 0 && v0 < up);
+        lo = min(v0, v1); hi = max(v0, v1);
         bad = __syncthreads_or(bad) != 0;
         if (bad) {                                           // how the times spread matters only then
             for (int o = 16; o > 0; o >>= 1) { lo = min(lo, __shfl_xor_sync(0xffffffffu, lo, o)); hi = max(hi, __shfl_xor_sync(0xffffffffu, hi, o)); }
@@ -1092,7 +1084,7 @@ size_t workspace_layout(uint64_t n, uint32_t n_queues, Workspace *ws, void *base
 
 std::atomic<unsigned long long> g_kernel_launches{0};
 
-cudaError_t ensure_dyn_smem(const void *kernel, size_t bytes) {
+cudaError_t ensure_dyn_smem(const void *kernel, size_t bytes, bool most_shared) {
     struct Entry { int device; const void *kernel; size_t bytes; };
     static std::mutex mu;
     static std::vector<Entry> set;
@@ -1108,6 +1100,7 @@ cudaError_t ensure_dyn_smem(const void *kernel, size_t bytes) {
             return e;
         }
     if (bytes > 48u * 1024u) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    if (e == cudaSuccess && most_shared) e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared);
     if (e == cudaSuccess) set.push_back(Entry{dev, kernel, bytes});
     return e;
 }
@@ -1297,7 +1290,9 @@ static cudaError_t launch_finish_inorder(const SubmitArgs &a, bool may_sort, cud
         const struct { const void *k; size_t bytes; } smem[] = {
             {(const void *)k_inorder_serve<false, false, false>, c.serve_smem}, {(const void *)k_inorder_serve<true, false, false>, c.serve_smem},
             {(const void *)k_inorder_fixstraggle<false, false>, c.fix_smem}, {(const void *)k_regroup_sort, kRgSortSmem}, {(const void *)k_regroup_place, kRgPlaceSmem}};
-        for (const auto &x : smem) if ((e = ensure_dyn_smem(x.k, x.bytes)) != cudaSuccess) return e;
+        // (launched from the device, a kernel gets the split between L1 and shared memory that its attribute names: without it one
+        // block at a time was resident where three fit)
+        for (const auto &x : smem) if ((e = ensure_dyn_smem(x.k, x.bytes, true)) != cudaSuccess) return e;
     }
     e = launch_pdl(may_sort ? k_finish_inorder<true> : k_finish_inorder<false>, finish_grid(a), 256, 0, st, c, finish_args(a));
     if (e != cudaSuccess) return e;
