@@ -40,7 +40,7 @@ struct hbf_ctx {
     bool terminal = false;           // a shutdown result has been observed
     // device state
     RangeSnap *d_ranges = nullptr; ModelParams *d_mp = nullptr; DevState *d_state = nullptr;
-    BatchCtrl *d_ctrl = nullptr; hbf_batch_result_t *d_result = nullptr;
+    BatchCtrl *d_ctrl = nullptr; RegroupSync *d_rg_sync = nullptr; hbf_batch_result_t *d_result = nullptr;
     int64_t *d_busy = nullptr, *d_busy_stage = nullptr, *d_pending = nullptr; hbf_die_stats_t *d_stats_stage = nullptr;
     // pinned: the last batch's summary (written by its last kernel), part counts on their way back, the hotspots (written by the
     // thermal step), the tiles' times
@@ -333,6 +333,7 @@ int hbf_create(const hbf_config_t *cfg, void *cuda_stream, hbf_ctx **out) {
     arena.add(&c->d_mp, nullptr, 1);
     arena.add(&c->d_state, &st0, 1);
     arena.add(&c->d_ctrl, nullptr, 1);
+    arena.add(&c->d_rg_sync, nullptr, 1);
     arena.add(&c->d_result, nullptr, 1);
     arena.add(&c->d_busy, nullptr, nq);
     arena.add(&c->d_busy_stage, nullptr, nq);
@@ -479,7 +480,7 @@ static int serve_records(hbf_ctx *c, SubmitArgs &a) {
         a.fast.base = r.base; a.fast.length = r.length; a.fast.media_offset = r.media_offset; a.fast.perms = r.perms; a.fast.on = 1u;
     }
     a.binned = c->bin_ns != 0; a.bus_on = c->d_bus_busy ? 1 : 0;
-    a.bal = &c->bal;
+    a.bal = &c->bal; a.rg_sync = c->d_rg_sync;
     if (c->ret_on) { a.claim_limit = &c->ret.st->claim_limit; a.die_claims = c->ret.die_claims; a.ret = &c->ret; }
     c->result_on_host = true;
     if (small_route(a)) {                                    // one launch, everything included (with the bus on it stops before the ledger)

@@ -56,6 +56,9 @@ struct SortPlan {
 };
 
 // Per-batch control block in device memory, cleared by the begin kernel.
+// regroup.cuh: the shares of every phase that are taken and done, the spread of the issue times.  Zero between batches: the begin
+// kernel clears what the last kernel uses, and the other way round.
+struct RegroupSync { uint32_t claim[8], done[8], hist[64], top[64], below[64]; };   // (samples of a stretch, their largest offset, 2^32 - 1 less their smallest)
 struct BatchCtrl {
     int32_t code;                        // HBF_OK or the batch's refusal / failure code
     int32_t skip;                        // later kernels do nothing when set
@@ -67,7 +70,7 @@ struct BatchCtrl {
     uint32_t unsorted;                   // some record has a smaller issue time than its predecessor
     uint32_t inorder_used;               // the in-order path served this batch
     uint32_t run_sort;                   // the sort path has to serve this batch
-    uint32_t regrouped;                  // the in-order path served it on an ordered copy of the records
+    uint32_t regrouped;                  // the in-order kernels serve it on an ordered copy of the records
     int64_t issue_lo, issue_hi;          // smallest and largest issue time among the begin kernel's samples
     uint32_t role_count[2];              // in-order serve pass: tiles handed out so far, per size class
     uint32_t tile_counter[kMaxPasses + 2];
@@ -125,6 +128,7 @@ struct SubmitArgs {
     const struct RetDev *ret;               // retention on: the block state (host copy of the device pointers)
     cudaEvent_t *ev;                     // [kProfEvents] or null: recorded between kernel groups
     TileBalanceHost *bal;                // tile sizes from measurements (null: off)
+    struct RegroupSync *rg_sync;
 };
 // what the last kernel of a batch needs
 struct FinishArgs {
@@ -142,8 +146,7 @@ constexpr int kProfEvents = 10;
 extern std::atomic<unsigned long long> g_kernel_launches;
 // The dynamic shared memory a kernel may use is an attribute of the (device, kernel) pair: raises it on the current device
 // when `bytes` exceeds what this process has set there so far.  Thread-safe.
-// most_shared: as much of the on-chip memory as there is for shared memory.
-cudaError_t ensure_dyn_smem(const void *kernel, size_t bytes, bool most_shared = false);
+cudaError_t ensure_dyn_smem(const void *kernel, size_t bytes);
 // a launch that may begin while the kernel before it still runs: for kernels that pass pdl_wait() (device_utils.cuh) on every path
 template <class Kernel, class... Args>
 inline cudaError_t launch_pdl(Kernel k, dim3 grid, dim3 block, size_t smem, cudaStream_t st, const Args &...args) {
@@ -215,8 +218,14 @@ InTileMap inorder_tile_map(uint64_t n, int sm_count, bool by_table);   // by_tab
 struct InTile { long long spec_sum, fix_delta, true_sum; uint32_t reserve; uint32_t stragglers; };
 size_t inorder_head_bytes(uint64_t tiles, uint32_t n_queues);
 size_t inorder_serve_smem(uint32_t n_dies);
-size_t inorder_straggle_smem();
 cudaError_t launch_inorder(const SubmitArgs &a, cudaStream_t st);
+// batches out of issue order (regroup.cuh): the copy of the records that the in-order kernels serve, and its results
+struct OrderedCopy { const hbf_access_t *recs; int64_t *comp, *stall; };
+OrderedCopy ordered_copy(uint64_t n, const Workspace &ws);
+size_t regroup_slot_bytes(uint64_t n);
+size_t regroup_ctrl_bytes(uint64_t n);
+struct BeginArgs;
+cudaError_t launch_begin_regroup(const SubmitArgs &a, const BeginArgs &b, cudaStream_t st);
 // small batches: one launch that serves and commits the batch, claims, ledger and read disturb included (small_kernels.cu)
 constexpr uint32_t kInSmallMax = 8192;   // records
 struct SmallExtras { unsigned long long *ledger; int64_t bin_ns, cur_bin; uint32_t n_bins; };

@@ -8,6 +8,7 @@
 #include <mutex>
 #include <vector>
 
+#include "begin.cuh"
 #include "regroup.cuh"
 
 namespace hbf {
@@ -18,57 +19,16 @@ namespace hbf {
 // role 0: first kernel of a batch; run_sort tells whether the sort path serves it.
 // role 1: placed between the in-order attempt and the sort kernels; it starts the batch over for the
 //         sort path when the in-order attempt found the records out of issue order, else does nothing.
-// acc != null: 1,024 pairs of neighbouring records are compared first; a batch that they show to be out of order is not attempted
-// on the in-order path (an attempt that finds out by itself took 2.7 of the 8.2 ms of 40 M shuffled records).
-__global__ void k_begin(BatchCtrl *ctrl, const DevState *state, const int64_t *busy, int64_t *busy_stage,
-                        hbf_die_stats_t *stats_stage, uint32_t *hist, uint32_t n_queues, uint32_t n_dies,
-                        int role, int run_sort, uint32_t *die_claims, const hbf_access_t *acc, uint64_t n) {
-    const int tid = threadIdx.x;
+// (a batch that may turn out to be out of issue order begins with k_begin_regroup)
+__global__ void k_begin(const __grid_constant__ BeginArgs b, int role, int run_sort) {
     pdl_wait();
     pdl_trigger();
     if (role == 1) {
-        if (ctrl->skip || !ctrl->run_sort) return;
+        if (b.ctrl->skip || !b.ctrl->run_sort) return;
         run_sort = 1;
     }
     __syncthreads();
-    uint32_t *w = reinterpret_cast<uint32_t *>(ctrl);
-    for (int i = tid; i < (int)(sizeof(BatchCtrl) / 4); i += blockDim.x) w[i] = 0u;
-    bool bad = false;
-    if (acc) {
-        __shared__ long long s_lo, s_hi;
-        if (tid == 0) { s_lo = INT64_MAX; s_hi = INT64_MIN; }
-        long long lo = INT64_MAX, hi = INT64_MIN;
-        // (blocks of 1,024 threads, n >= 2; one pair each: one multiprocessor takes 4 us longer to fetch four)
-        const uint64_t *rec = reinterpret_cast<const uint64_t *>(acc + (uint64_t)tid * (n - 1ull) / 1024ull);
-        const int64_t v0 = (int64_t)__ldg(rec + 1), v1 = (int64_t)__ldg(rec + 4);
-        const int64_t up = __shfl_up_sync(0xffffffffu, v0, 1);
-        bad = v1 < v0 || ((tid & 31) != 0 && v0 < up);
-        lo = min(v0, v1); hi = max(v0, v1);
-        bad = __syncthreads_or(bad) != 0;
-        if (bad) {                                           // how the times spread matters only then
-            for (int o = 16; o > 0; o >>= 1) { lo = min(lo, __shfl_xor_sync(0xffffffffu, lo, o)); hi = max(hi, __shfl_xor_sync(0xffffffffu, hi, o)); }
-            if ((tid & 31) == 0) { atomicMin(&s_lo, lo); atomicMax(&s_hi, hi); }
-            __syncthreads();
-            if (tid == 0) { ctrl->issue_lo = s_lo; ctrl->issue_hi = s_hi; run_sort = 1; }
-        }
-    }
-    __syncthreads();
-    if (tid == 0) {
-        int32_t mode = state->mode;
-        ctrl->mode = mode; ctrl->q_ppm = state->q_ppm;
-        if (state->q_ppm != 1000000) ctrl->div_q = make_div64((uint64_t)state->q_ppm);   // (a 128-bit division; nothing looks at it without scaling)
-        ctrl->key_and = ~0ull;
-        ctrl->run_sort = (uint32_t)run_sort;
-        if (state->poisoned) { ctrl->code = HBF_E_TIMEOUT; ctrl->skip = 1; }
-        else if (mode == HBF_MODE_SHUTDOWN) { ctrl->code = HBF_E_LINK_SHUTDOWN; ctrl->skip = 1; }
-        else if (mode == HBF_MODE_SEVERE) { ctrl->code = HBF_E_THROTTLED; ctrl->skip = 1; }
-    }
-    for (uint32_t r = tid; r < n_queues; r += blockDim.x) busy_stage[r] = busy[r];
-    int64_t *s = reinterpret_cast<int64_t *>(stats_stage);
-    for (uint32_t i = tid; i < n_dies * 6u; i += blockDim.x) s[i] = 0;
-    for (int i = tid; i < kMaxPasses * kRadix; i += blockDim.x) hist[i] = 0u;
-    if (die_claims)                                          // retention on: an in-order attempt that was handed over counted some
-        for (uint32_t d = tid; d < n_dies; d += blockDim.x) die_claims[d] = 0u;
+    begin_batch(b, run_sort, 0u);
 }
 
 // =====================================================================================================
@@ -721,7 +681,7 @@ k_stalls(const hbf_access_t *__restrict__ acc, uint64_t n, const BatchCtrl *ctrl
 // =====================================================================================================
 // finish: commit the staged state, or zero the outputs of a refused batch; write the batch summary
 // =====================================================================================================
-__device__ __forceinline__ void finish_batch(const FinishArgs &f, long long modeled) {
+__device__ __forceinline__ int finish_batch(const FinishArgs &f, long long modeled) {
     BatchCtrl *ctrl = f.ctrl;
     const uint64_t n = f.n;
     int code = ctrl->code;
@@ -758,6 +718,7 @@ __device__ __forceinline__ void finish_batch(const FinishArgs &f, long long mode
         r.max_completion_ns = code == HBF_OK && ctrl->n_ready ? ctrl->max_completion_ns : 0;
         *f.result = r; *f.result_host = r;
     }
+    return code;
 }
 __global__ void k_finish(const __grid_constant__ FinishArgs f) { finish_batch(f, f.ctrl->modeled_ns); }
 
@@ -1084,7 +1045,7 @@ size_t workspace_layout(uint64_t n, uint32_t n_queues, Workspace *ws, void *base
 
 std::atomic<unsigned long long> g_kernel_launches{0};
 
-cudaError_t ensure_dyn_smem(const void *kernel, size_t bytes, bool most_shared) {
+cudaError_t ensure_dyn_smem(const void *kernel, size_t bytes) {
     struct Entry { int device; const void *kernel; size_t bytes; };
     static std::mutex mu;
     static std::vector<Entry> set;
@@ -1100,7 +1061,6 @@ cudaError_t ensure_dyn_smem(const void *kernel, size_t bytes, bool most_shared) 
             return e;
         }
     if (bytes > 48u * 1024u) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-    if (e == cudaSuccess && most_shared) e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared);
     if (e == cudaSuccess) set.push_back(Entry{dev, kernel, bytes});
     return e;
 }
@@ -1154,11 +1114,7 @@ struct SortChain {
     const unsigned long long *claim_limit; uint32_t *die_claims;
     uint32_t n_queues, n_dies; uint64_t desc_words, scan_words;
     unsigned cls_grid, hist_grid, sort_grid, scan_grid, stall_grid;
-    const InTile *in_tile; uint32_t n_tiles, first_tiles;   // (first_tiles: those whose stall totals are added up)
-    // a batch out of issue order, brought into order and served by the in-order kernels (regroup.cuh)
-    uint32_t regroup;                                       // 1: to be tried; 0: the radix sort at once (or the second time)
-    RegroupArgs rg; ModelParams mp; FastRange fast; FastGeom geom; InTileMap tmap;
-    int64_t *in_agg, *in_bin; InHead *in_head; uint8_t *in_headcnt; uint16_t *in_qid; uint32_t qid_stride, serve_smem, fix_smem;
+    const InTile *in_tile; uint32_t n_tiles;
 };
 
 __global__ void k_zero_words(uint32_t *p, uint64_t words) {
@@ -1168,7 +1124,8 @@ __global__ void k_zero_words(uint32_t *p, uint64_t words) {
 // the radix sort's kernels, launched from the device (run_sort is set: the begin kernel starts the batch over)
 __device__ void launch_sort_chain(const SortChain &c, const FinishArgs &f, unsigned fin_grid) {
     cudaStream_t st = cudaStreamTailLaunch;
-    k_begin<<<1, 1024, 0, st>>>(c.ctrl, c.state, c.busy, c.busy_stage, c.stats_stage, c.hist, c.n_queues, c.n_dies, 1, 1, c.die_claims, nullptr, 0ull);
+    const BeginArgs b{c.ctrl, c.state, c.busy, c.busy_stage, c.stats_stage, c.hist, c.n_queues, c.n_dies, c.die_claims, c.claim_limit};
+    k_begin<<<1, 1024, 0, st>>>(b, 1, 1);
     k_zero_words<<<(unsigned)min((unsigned long long)((c.desc_words + 1023) / 1024), 592ull), 1024, 0, st>>>(c.desc0, c.desc_words);
     k_zero_words<<<(unsigned)min((unsigned long long)((c.scan_words + 1023) / 1024), 592ull), 1024, 0, st>>>((uint32_t *)c.scan_desc, c.scan_words);
     k_classify<<<c.cls_grid, kClsThreads, 0, st>>>(c.acc, c.n, c.ranges, c.mp_dev, c.ctrl, c.keys0, c.terms, c.status, c.completion, c.stall);
@@ -1183,44 +1140,25 @@ __device__ void launch_sort_chain(const SortChain &c, const FinishArgs &f, unsig
     k_finish<<<fin_grid, 256, 0, st>>>(f);
 }
 
-template <bool MAY_SORT>
-__global__ void k_finish_inorder(const __grid_constant__ SortChain c, const __grid_constant__ FinishArgs f);
-
-// the records are in order: the in-order kernels, the results back to batch order, the commit; or the radix sort after all
-__global__ void k_regroup_decide(const __grid_constant__ SortChain c, const __grid_constant__ FinishArgs f, unsigned fin_grid) {
-    if (c.rg.rg->overflow) { launch_sort_chain(c, f, fin_grid); return; }
-    cudaStream_t st = cudaStreamTailLaunch;
-    const hbf_access_t *recs = reinterpret_cast<const hbf_access_t *>(c.rg.recs);
-    InTile *tiles = const_cast<InTile *>(c.in_tile);
-    SortChain again = c;
-    again.regroup = 0u; again.first_tiles = c.tmap.n_tiles;
-    k_begin<<<1, 1024, 0, st>>>(c.ctrl, c.state, c.busy, c.busy_stage, c.stats_stage, c.hist, c.n_queues, c.n_dies, 2, 0, c.die_claims, nullptr, 0ull);
-    k_inorder_serve<false, false, false><<<c.tmap.n_tiles, kInThreads, c.serve_smem, st>>>(recs, c.n, c.tmap, c.ranges, c.mp, c.fast, c.ctrl, nullptr, c.in_agg, c.stats_stage,
-        c.rg.comp, c.rg.stall, c.in_bin, tiles, c.in_head, c.in_headcnt, c.busy, nullptr, nullptr, RetDev{}, c.in_qid, c.qid_stride, nullptr, 0u, c.geom, (uint32_t)kInHead);
-    k_inorder_scan<<<(c.n_queues + kInScanQueues - 1) / kInScanQueues, dim3(kInScanQueues, kInScanChunks), 0, st>>>(c.ctrl, c.mp_dev, c.tmap.n_tiles, c.in_agg, c.in_bin, c.busy,
-        c.busy_stage, c.stats_stage, 0);
-    k_inorder_fixstraggle<false, false><<<c.tmap.n_tiles, kInStrThreads, c.fix_smem, st>>>(recs, c.n, c.tmap, c.ranges, c.mp, c.fast, c.ctrl, c.in_bin, c.in_head, c.in_headcnt,
-        c.rg.comp, c.rg.stall, tiles, nullptr, c.in_qid, c.qid_stride, (uint32_t)kInHead, nullptr);
-    k_inorder_serve<true, false, false><<<c.tmap.n_tiles, kInThreads, c.serve_smem, st>>>(recs, c.n, c.tmap, c.ranges, c.mp, c.fast, c.ctrl, nullptr, c.in_agg, c.stats_stage,
-        c.rg.comp, c.rg.stall, c.in_bin, tiles, c.in_head, c.in_headcnt, c.busy, nullptr, nullptr, RetDev{}, c.in_qid, c.qid_stride, nullptr, 0u, c.geom, (uint32_t)kInHead);
-    k_regroup_give<<<(unsigned)min((unsigned long long)((c.n + 1023) / 1024), 1184ull), 256, 0, st>>>(c.n, c.ctrl, c.rg);
-    k_regroup_place<<<min(c.rg.out_buckets, 296u), 1024, kRgPlaceSmem, st>>>(c.acc, c.n, c.ctrl, c.rg, c.completion, c.stall);
-    k_finish_inorder<true><<<fin_grid, 256, 0, st>>>(again, f);
-}
-
 // The last kernel of a batch on the in-order path: the commit, and the hand-over of a batch that it did not serve.
 // (MAY_SORT = false, for a context whose caller declares issue order: the same kernel without the device-side launches,
 // which cost a kernel that contains them several microseconds even when none is made)
 template <bool MAY_SORT>
-__global__ void __launch_bounds__(256) k_finish_inorder(const __grid_constant__ SortChain c, const __grid_constant__ FinishArgs f) {
+__global__ void __launch_bounds__(256, 4) k_finish_inorder(const __grid_constant__ SortChain c, const __grid_constant__ FinishArgs f, const __grid_constant__ RegroupArgs rg) {
     pdl_wait();
     if constexpr (!MAY_SORT) pdl_trigger();                  // (what follows a kernel that may launch others is launched plainly)
+    const bool regrouped = MAY_SORT && rg.sync && c.ctrl->regrouped;
+    if (regrouped && blockIdx.x == 0) {                      // (the begin kernel's part of it: zero again for the next batch)
+        for (uint32_t i = threadIdx.x; i < 3u * 64u; i += blockDim.x) rg.sync->hist[i] = 0u;
+        if (threadIdx.x < 3) { rg.sync->claim[threadIdx.x] = 0u; rg.sync->done[threadIdx.x] = 0u; }
+        if (threadIdx.x == 3) rg.sync->claim[5] = 0u;
+    }
     if (!MAY_SORT || c.ctrl->skip || c.ctrl->inorder_used) {
         // Stall total of the batch: per tile the exact sum if it was re-served, else the as-if sum plus its corrections
         __shared__ long long s_tot[8];
         long long tot = 0;
         if (blockIdx.x == 0) {
-            if (!c.ctrl->skip) for (uint32_t t = threadIdx.x; t < c.first_tiles; t += blockDim.x) {
+            if (!c.ctrl->skip) for (uint32_t t = threadIdx.x; t < c.n_tiles; t += blockDim.x) {
                 const InTile v = c.in_tile[t];
                 tot += v.reserve ? v.true_sum : v.spec_sum + v.fix_delta;
             }
@@ -1230,21 +1168,15 @@ __global__ void __launch_bounds__(256) k_finish_inorder(const __grid_constant__ 
             tot = 0;
             for (int w = 0; w < 8; ++w) tot += s_tot[w];
         }
-        finish_batch(f, tot);
+        const int code = finish_batch(f, tot);
+        if constexpr (MAY_SORT) {
+            if (regrouped && code == HBF_OK && c.ctrl->inorder_used && !rg_give_back(rg, f.n, f.ctrl, f.completion, f.stall) && threadIdx.x == 0) {
+                f.state->poisoned = 1; f.result->code = HBF_E_TIMEOUT; f.result_host->code = HBF_E_TIMEOUT;
+            }
+        }
         return;
     }
-    if constexpr (MAY_SORT) {
-        if (threadIdx.x != 0 || blockIdx.x != 0) return;
-        // (refresh claims go by batch index: a batch that has to pay some is sorted; so is one whose samples were in order)
-        if (!c.regroup || c.ctrl->issue_lo >= c.ctrl->issue_hi || (c.claim_limit && *c.claim_limit > 0ull)) { launch_sort_chain(c, f, gridDim.x); return; }
-        cudaStream_t st = cudaStreamTailLaunch;
-        k_zero_words<<<(unsigned)min((unsigned long long)((c.rg.zero_words + 1023) / 1024), 592ull), 1024, 0, st>>>((uint32_t *)c.rg.rg, c.rg.zero_words);
-        k_regroup_sample<<<(unsigned)((min(c.n, (uint64_t)kRgSamples) + 1023) / 1024), 1024, 0, st>>>(c.acc, c.n, c.ctrl, c.rg);
-        k_regroup_scatter<<<(unsigned)min((unsigned long long)((c.n + 1023) / 1024), 1184ull), 256, 0, st>>>(c.acc, c.n, c.ranges, c.fast, c.rg, c.status);
-        k_regroup_offsets<<<1, 1024, 0, st>>>(c.n, c.rg);
-        k_regroup_sort<<<min(c.rg.max_buckets, 444u), kRgThreads, kRgSortSmem, st>>>(c.rg);
-        k_regroup_decide<<<1, 1, 0, st>>>(c, f, gridDim.x);
-    }
+    if constexpr (MAY_SORT) { if (threadIdx.x == 0 && blockIdx.x == 0) launch_sort_chain(c, f, gridDim.x); }
 }
 
 static FinishArgs finish_args(const SubmitArgs &a) {
@@ -1278,23 +1210,7 @@ static cudaError_t launch_finish_inorder(const SubmitArgs &a, bool may_sort, cud
     const InTileMap tmap = inorder_tile_map(n, a.sm_count, a.bal && a.bal->on && a.bal->dev);
     c.in_tile = reinterpret_cast<const InTile *>(a.ws.in_tile);
     c.n_tiles = tmap.n_tiles;
-    c.first_tiles = c.n_tiles;
-    if (may_sort && !a.paged) {
-        c.regroup = 1u; c.rg = regroup_args(n, a.ws); c.mp = a.mp; c.fast = a.fast; c.geom = make_fast_geom(a.fast, a.mp);
-        c.tmap = inorder_tile_map(n, a.sm_count, false);     // (no table: nothing the host would have to write)
-        if (c.tmap.n_tiles > inorder_tiles_bound(n)) return cudaErrorInvalidValue;
-        c.in_agg = a.ws.in_agg; c.in_bin = a.ws.in_bin; c.in_head = reinterpret_cast<InHead *>(a.ws.in_head); c.in_headcnt = a.ws.in_headcnt; c.in_qid = a.ws.in_qid;
-        c.qid_stride = (uint32_t)std::min<uint64_t>(c.tmap.max_tile, kInQidPrefix);
-        if ((uint64_t)c.tmap.n_tiles * c.qid_stride > inorder_qid_entries(n)) return cudaErrorInvalidValue;
-        c.serve_smem = (uint32_t)inorder_serve_smem(a.mp.n_dies); c.fix_smem = (uint32_t)inorder_straggle_smem();
-        const struct { const void *k; size_t bytes; } smem[] = {
-            {(const void *)k_inorder_serve<false, false, false>, c.serve_smem}, {(const void *)k_inorder_serve<true, false, false>, c.serve_smem},
-            {(const void *)k_inorder_fixstraggle<false, false>, c.fix_smem}, {(const void *)k_regroup_sort, kRgSortSmem}, {(const void *)k_regroup_place, kRgPlaceSmem}};
-        // (launched from the device, a kernel gets the split between L1 and shared memory that its attribute names: without it one
-        // block at a time was resident where three fit)
-        for (const auto &x : smem) if ((e = ensure_dyn_smem(x.k, x.bytes, true)) != cudaSuccess) return e;
-    }
-    e = launch_pdl(may_sort ? k_finish_inorder<true> : k_finish_inorder<false>, finish_grid(a), 256, 0, st, c, finish_args(a));
+    e = launch_pdl(may_sort ? k_finish_inorder<true> : k_finish_inorder<false>, finish_grid(a), 256, 0, st, c, finish_args(a), regroup_args(n, a.ws, may_sort && n >= 2 ? a.rg_sync : nullptr));
     if (e != cudaSuccess) return e;
     if (may_sort && a.plain_next) *a.plain_next = true;      // (kernels that may overlap their predecessor must not overlap one that may launch others)
     g_kernel_launches += 1;
@@ -1311,9 +1227,10 @@ cudaError_t launch_submit(const SubmitArgs &a, cudaStream_t st) {
     const bool sort_kernels = a.path != HBF_PATH_INORDER || !a.inorder_ok;
     mark(0);
     {
-        const cudaError_t e = launch_first(a.plain_next, k_begin, 1, 1024, 0, st, a.ctrl, (const DevState *)a.state, (const int64_t *)a.busy, a.busy_stage, a.stats_stage, a.ws.hist,
-                                           a.mp.n_queues, a.mp.n_dies, 0, try_inorder ? 0 : 1, a.die_claims,
-                                           try_inorder && sort_kernels && n >= 2 ? a.acc : nullptr, n);
+        const BeginArgs b{a.ctrl, a.state, a.busy, a.busy_stage, a.stats_stage, a.ws.hist, a.mp.n_queues, a.mp.n_dies, a.die_claims, a.claim_limit};
+        const cudaError_t e = try_inorder && sort_kernels && n >= 2
+            ? launch_begin_regroup(a, b, st)
+            : launch_first(a.plain_next, k_begin, 1, 1024, 0, st, b, 0, try_inorder ? 0 : 1);
         if (e != cudaSuccess) return e;
     }
     g_kernel_launches += 1;

@@ -19,7 +19,7 @@ def hbf():
     return mod
 
 
-@pytest.mark.parametrize("n", [8_193, 24_575, 24_577, 200_003])
+@pytest.mark.parametrize("n", [8_193, 24_575, 24_577, 100_003, 200_003])
 @pytest.mark.parametrize("kind", ["shuffled", "rings", "ties", "bunched", "one time", "long span", "negative", "natives", "fault", "late", "long service", "three ranges"])
 def test_unordered_batches_match_the_oracle(hbf, kind, n):
     rng = np.random.default_rng(n)
