@@ -424,7 +424,7 @@ int hbf_clear_ranges(hbf_ctx *c) {
 
 size_t hbf_workspace_bytes(const hbf_ctx *c, uint64_t n) {
     if (!c) return 0;
-    return workspace_layout(n, c->mp.n_queues, nullptr, nullptr, c->d_bus_busy ? 1 : 0);
+    return workspace_layout(n, c->mp.n_queues, c->mp.channels, nullptr, nullptr, c->d_bus_busy ? 1 : 0);
 }
 
 int hbf_set_thermal_path(hbf_ctx *c, int32_t generic_only) {
@@ -518,7 +518,7 @@ int hbf_submit_batch(hbf_ctx *c, const hbf_access_t *d_acc, uint64_t n, int64_t 
     if ((reinterpret_cast<uintptr_t>(d_acc) & 7u) || (reinterpret_cast<uintptr_t>(d_completion_ns) & 7u) ||
         (reinterpret_cast<uintptr_t>(d_stall_ns) & 7u) || (reinterpret_cast<uintptr_t>(d_die_stats) & 7u)) return HBF_E_INVAL;
     SubmitArgs a{};
-    const size_t need = workspace_layout(n, c->mp.n_queues, &a.ws, d_workspace, c->d_bus_busy ? 1 : 0);
+    const size_t need = workspace_layout(n, c->mp.n_queues, c->mp.channels, &a.ws, d_workspace, c->d_bus_busy ? 1 : 0);
     if (!d_workspace || workspace_bytes < need || (reinterpret_cast<uintptr_t>(d_workspace) & 255u)) return HBF_E_WORKSPACE;
     a.acc = d_acc; a.n = n; a.completion = d_completion_ns; a.stall = d_stall_ns; a.status = d_status; a.die_stats = d_die_stats;
     c->prof_inorder = c->profiling && n > 0 && c->inorder_ok && (c->path == HBF_PATH_AUTO || c->path == HBF_PATH_INORDER);
@@ -612,7 +612,7 @@ int hbf_submit_host(hbf_ctx *c, const hbf_access_t *h_acc, uint64_t n, int64_t *
 
 size_t hbf_workspace_bytes_paged(const hbf_ctx *c, uint64_t n, uint64_t parts_capacity) {
     if (!c) return 0;
-    return paged_layout(n, std::max<uint64_t>(parts_capacity, n), c->mp.n_queues, nullptr, nullptr, c->d_bus_busy ? 1 : 0);
+    return paged_layout(n, std::max<uint64_t>(parts_capacity, n), c->mp.n_queues, c->mp.channels, nullptr, nullptr, c->d_bus_busy ? 1 : 0);
 }
 
 int hbf_submit_batch_paged(hbf_ctx *c, const hbf_access_t *d_acc, uint64_t n, uint64_t parts_capacity,
@@ -630,7 +630,7 @@ int hbf_submit_batch_paged(hbf_ctx *c, const hbf_access_t *d_acc, uint64_t n, ui
     const uint64_t capacity = std::min<uint64_t>(std::max<uint64_t>(parts_capacity, n), HBF_MAX_BATCH);
     PagedWorkspace pw{};
     const int with_bus = c->d_bus_busy ? 1 : 0;
-    const size_t need = paged_layout(n, capacity, c->mp.n_queues, &pw, d_workspace, with_bus);
+    const size_t need = paged_layout(n, capacity, c->mp.n_queues, c->mp.channels, &pw, d_workspace, with_bus);
     if (!d_workspace || workspace_bytes < need || (reinterpret_cast<uintptr_t>(d_workspace) & 255u)) return HBF_E_WORKSPACE;
     FastRange fast{};
     if (c->ranges.size() == 1) {
@@ -661,7 +661,7 @@ int hbf_submit_batch_paged(hbf_ctx *c, const hbf_access_t *d_acc, uint64_t n, ui
     c->prof_inorder = false; c->prof_submit = false;
     if (by_unit && total == n) {                             // no access crosses a stripe unit: the caller's records are the list
         SubmitArgs a{};
-        workspace_layout(n, c->mp.n_queues, &a.ws, pw.inner, 0);
+        workspace_layout(n, c->mp.n_queues, c->mp.channels, &a.ws, pw.inner, 0);
         a.acc = d_acc; a.n = n; a.completion = d_completion_ns; a.stall = d_stall_ns; a.status = d_status; a.die_stats = d_die_stats;
         a.paged = 1;
         if ((rc = serve_records(c, a)) != HBF_OK) return rc;
@@ -672,7 +672,7 @@ int hbf_submit_batch_paged(hbf_ctx *c, const hbf_access_t *d_acc, uint64_t n, ui
     CK(launch_paged_expand(d_acc, n, c->d_ranges, c->d_mp, fast, by_unit ? c->mp.stripe_shift : c->mp.page_shift, capacity, pw, c->sm_count, c->stream));
     // the list of parts is a batch of records like any other: the ledger, the bus stage and retention, when on, see parts
     SubmitArgs a{};
-    workspace_layout(total, c->mp.n_queues, &a.ws, pw.inner, with_bus);
+    workspace_layout(total, c->mp.n_queues, c->mp.channels, &a.ws, pw.inner, with_bus);
     a.acc = pw.parts; a.n = total; a.completion = pw.part_completion; a.stall = pw.part_stall; a.status = pw.part_status;
     a.die_stats = d_die_stats;
     a.paged = by_unit ? 1 : 0;
@@ -851,7 +851,7 @@ int hbf_last_result(hbf_ctx *c, hbf_batch_result_t *host_out) {
 int hbf_queue_order(hbf_ctx *c, const void *d_workspace, uint64_t n, uint32_t *d_order, uint64_t *count) {
     if (!c || !d_workspace || !d_order || !count) return HBF_E_INVAL;
     Workspace ws;
-    workspace_layout(n, c->mp.n_queues, &ws, const_cast<void *>(d_workspace));
+    workspace_layout(n, c->mp.n_queues, c->mp.channels, &ws, const_cast<void *>(d_workspace), c->d_bus_busy ? 1 : 0);
     BatchCtrl hc;
     CK(cudaMemcpyAsync(&hc, c->d_ctrl, sizeof(hc), cudaMemcpyDeviceToHost, c->stream));
     CK(cudaStreamSynchronize(c->stream));

@@ -103,6 +103,7 @@ struct Workspace {
     uint16_t *in_qid;                    // [tiles][stride]: queue of each of the first records of every tile (0xffff: not modeled), for the straggle pass
     void *rg_ctrl, *rg_slots, *rg_recs, *rg_idx;   // a batch out of issue order: see regroup.cuh (the slots share memory with keys, idx and terms)
     uint32_t *bus_xfer;                  // [n] transfer time of every read (only with the channel-bus stage on)
+    void *bus_plan;                      // (likewise) see bus.cuh
     size_t bytes;
 };
 
@@ -183,9 +184,10 @@ inline uint64_t inorder_tiles_bound(uint64_t n) {
     const uint64_t t = (n + kInTileQuantum - 1) / kInTileQuantum;
     return t < 1 ? 1 : (t < kInMaxTiles ? t : kInMaxTiles);
 }
-size_t workspace_layout(uint64_t n, uint32_t n_queues, Workspace *ws, void *base, int with_bus = 0);
+size_t workspace_layout(uint64_t n, uint32_t n_queues, uint32_t channels, Workspace *ws, void *base, int with_bus = 0);
 // channel bus as a second queued stage, after launch_submit on the same arguments (bc: a control block of its own)
 cudaError_t launch_bus_stage(const SubmitArgs &a, BatchCtrl *bc, int64_t *bus_busy, cudaStream_t st);
+cudaError_t launch_bus_buckets(const SubmitArgs &a, BatchCtrl *bc, int64_t *bus_busy, cudaStream_t st);
 // How the in-order path cuts a batch of n records into contiguous tiles: n_big tiles of `big` records, then tiles of
 // `small` records (the last one ragged).  All sizes are multiples of kInTileQuantum.  n_big == 0: one size only.
 // With `first` set (device memory, n_tiles + 1 entries) the tiles begin where that table says instead: sizes that follow
@@ -255,7 +257,7 @@ struct PagedWorkspace {
 };
 // parts of the list; pages of all accesses; accesses issued before their predecessor; set when a service of a stripe unit's pages is too long for the in-order kernels
 enum PagedTotal { kPagedParts = 0, kPagedPages = 1, kPagedUnsorted = 2, kPagedLong = 3, kPagedTotals = 4 };
-size_t paged_layout(uint64_t n, uint64_t capacity, uint32_t n_queues, PagedWorkspace *pw, void *base, int with_bus = 0);
+size_t paged_layout(uint64_t n, uint64_t capacity, uint32_t n_queues, uint32_t channels, PagedWorkspace *pw, void *base, int with_bus = 0);
 cudaError_t launch_paged_count(const hbf_access_t *acc, uint64_t n, const RangeSnap *ranges, const ModelParams *mp_dev, const FastRange &fast,
                                const ModelParams &mp, const DevState *state, bool by_unit, const PagedWorkspace &pw, cudaStream_t st);
 cudaError_t launch_paged_offsets(uint64_t n, const PagedWorkspace &pw, cudaStream_t st);

@@ -9,6 +9,7 @@
 #include <vector>
 
 #include "begin.cuh"
+#include "bus.cuh"
 #include "regroup.cuh"
 
 namespace hbf {
@@ -732,25 +733,13 @@ __global__ void k_queue_order(const BatchCtrl *ctrl, const uint32_t *idx0, const
 }
 
 // =====================================================================================================
-// channel bus as a second queued stage (an extension; the library's own definition).  After the array
-// stage, a read's data-out transfer queues on the bus of its channel in (array-done time, index) order and
-// holds it for the transfer time; the read completes when the transfer does.  Programs are unchanged.
+// The channel-bus stage (bus_kernels.cu) by radix sort, for a batch whose reads its buckets do not hold; launched from the device.
 //   keys   per access: channel << 47 | array-done time (reads), a sentinel behind every channel (the rest)
 //   sort   the onesweep passes of the sort path, over the key bits that differ
 //   scan   in sorted order a read is the map B -> max(B, D) + x on its channel's bus; channels are segments
 //          whose first map starts from the bus state earlier batches left.  Three kernels, no look-back: tile
 //          aggregates, an exclusive scan of them by one block, tiles again with their carry.
 // =====================================================================================================
-struct BusMap { int64_t S, M; int f; };                    // B -> max(B + S, M); f: contains a segment head (then B does not matter)
-__device__ __forceinline__ BusMap bus_then(const BusMap &a, const BusMap &b) {       // a first, then b
-    if (b.f) return b;
-    BusMap r; r.S = a.S + b.S; r.M = max((int64_t)(a.M + b.S), b.M); r.f = a.f; return r;
-}
-__device__ __forceinline__ BusMap bus_identity() { BusMap r; r.S = 0; r.M = kNegInf; r.f = 0; return r; }
-__device__ __forceinline__ BusMap bus_shfl_up(const BusMap &v, int o) {
-    BusMap r; r.S = __shfl_up_sync(0xffffffffu, v.S, o); r.M = __shfl_up_sync(0xffffffffu, v.M, o); r.f = __shfl_up_sync(0xffffffffu, v.f, o);
-    return r;
-}
 constexpr int kBusThreads = 256;
 constexpr int kBusItems = 8;
 constexpr int kBusTile = kBusThreads * kBusItems;          // as many entries as a scan tile of the sort path: its descriptors are reused
@@ -964,44 +953,63 @@ k_bus_commit(const BatchCtrl *bc, const uint64_t *k0, const uint64_t *k1, const 
     }
 }
 
-__global__ void k_bus_finish(const BatchCtrl *bc, hbf_batch_result_t *result, hbf_batch_result_t *result_host, DevState *state) {
+__device__ __forceinline__ void bus_finish(const BatchCtrl *bc, hbf_batch_result_t *result, hbf_batch_result_t *result_host, DevState *state) {
     if (bc->code != HBF_OK) { result->code = bc->code; *result_host = *result; state->poisoned = 1; return; }   // the array stage is committed: the context cannot go on
     if (bc->skip) return;
     result->modeled_ns += bc->modeled_ns;
     if (bc->max_completion_ns > result->max_completion_ns) result->max_completion_ns = bc->max_completion_ns;
     *result_host = *result;
 }
+struct BusChain {
+    const hbf_access_t *acc; uint64_t n; int64_t *completion, *stall; const RangeSnap *ranges; const ModelParams *mp_dev; BatchCtrl *bc; DevState *state;
+    hbf_batch_result_t *result, *result_host; const BusPlan *plan; int64_t *busy; Workspace ws;
+    unsigned wide, hist_grid, sort_grid, tiles_grid; uint64_t desc_words;
+};
+__global__ void k_bus_sorted_finish(const __grid_constant__ BusChain c) { bus_finish(c.bc, c.result, c.result_host, c.state); }
+__global__ void k_zero_words(uint32_t *p, uint64_t words) {
+    for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < words; i += (uint64_t)gridDim.x * blockDim.x) p[i] = 0u;
+}
+__global__ void k_bus_finish(const __grid_constant__ BusChain c) {
+    pdl_wait();
+    if (c.bc->skip || c.bc->code != HBF_OK || !c.plan->overflow) { bus_finish(c.bc, c.result, c.result_host, c.state); return; }
+    cudaStream_t st = cudaStreamTailLaunch;
+    const Workspace &w = c.ws;
+    ScanDesc *agg = (ScanDesc *)w.scan_desc;
+    k_bus_begin<<<1, 256, 0, st>>>(c.bc, c.result, w.hist);
+    k_zero_words<<<(unsigned)min((unsigned long long)((c.desc_words + 1023) / 1024), 592ull), 1024, 0, st>>>(w.sort_desc[0], c.desc_words);
+    k_bus_keys<<<c.wide, 256, 0, st>>>(c.acc, c.n, c.completion, c.ranges, c.mp_dev, c.bc, w.keys[0], w.bus_xfer);
+    k_bus_check<<<1, 1, 0, st>>>(c.bc);
+    k_plan<<<1, 32, 0, st>>>(c.bc, 1);
+    k_hist<<<c.hist_grid, kHistThreads, 0, st>>>(w.keys[0], c.n, c.bc, w.hist);
+    for (int p = 0; p < kMaxPasses; ++p)
+        k_sort_pass<<<c.sort_grid, kSortThreads, kSortSmem, st>>>(p, c.n, c.bc, c.state, w.hist, w.keys[0], w.keys[1], w.idx[0], w.idx[1], w.sort_desc[0], w.sort_desc[1]);
+    k_bus_check<<<1, 1, 0, st>>>(c.bc);                      // a look-back that gave up sets the code
+    k_bus_reduce<<<c.tiles_grid, kBusThreads, 0, st>>>(c.bc, w.keys[0], w.keys[1], w.idx[0], w.idx[1], w.bus_xfer, c.busy, agg);
+    k_bus_tile_scan<<<1, 1024, 0, st>>>(c.bc, agg);
+    k_bus_apply<<<c.tiles_grid, kBusThreads, 0, st>>>(c.acc, c.bc, w.keys[0], w.keys[1], w.idx[0], w.idx[1], w.bus_xfer, c.busy, agg, c.completion, c.stall);
+    k_bus_commit<<<c.wide, 256, 0, st>>>(c.bc, w.keys[0], w.keys[1], w.idx[0], w.idx[1], c.completion, c.busy);
+    k_bus_sorted_finish<<<1, 1, 0, st>>>(c);
+}
 
 cudaError_t launch_bus_stage(const SubmitArgs &a, BatchCtrl *bc, int64_t *bus_busy, cudaStream_t st) {
     const uint64_t n = a.n;
     if (n == 0) return cudaSuccess;
+    cudaError_t e = ensure_dyn_smem((const void *)k_sort_pass, kSortSmem);
+    if (e == cudaSuccess) e = launch_bus_buckets(a, bc, bus_busy, st);
+    if (e != cudaSuccess) return e;
     const uint64_t sort_tiles = (n + kSortTile - 1) / kSortTile, bus_tiles = (n + kBusTile - 1) / kBusTile;
-    cudaError_t e = cudaMemsetAsync(a.ws.sort_desc[0], 0, sort_tiles * kRadix * 4, st);
-    if (e != cudaSuccess) return e;
-    k_bus_begin<<<1, 256, 0, st>>>(bc, a.result, a.ws.hist);
-    const unsigned wide = (unsigned)std::min<uint64_t>((n + 255) / 256, (uint64_t)a.sm_count * 8);
-    k_bus_keys<<<wide, 256, 0, st>>>(a.acc, n, a.completion, a.ranges, a.mp_dev, bc, a.ws.keys[0], a.ws.bus_xfer);
-    k_bus_check<<<1, 1, 0, st>>>(bc);
-    k_plan<<<1, 32, 0, st>>>(bc, 1);
-    const unsigned hist_grid = (unsigned)std::min<uint64_t>((n + kHistThreads * 8 - 1) / (kHistThreads * 8), (uint64_t)a.sm_count * 4);
-    k_hist<<<hist_grid, kHistThreads, 0, st>>>(a.ws.keys[0], n, bc, a.ws.hist);
-    e = ensure_dyn_smem((const void *)k_sort_pass, kSortSmem);
-    if (e != cudaSuccess) return e;
-    const unsigned sort_grid = (unsigned)std::min<uint64_t>(sort_tiles, (uint64_t)a.sm_count * 3);
-    for (int p = 0; p < kMaxPasses; ++p)
-        k_sort_pass<<<sort_grid, kSortThreads, kSortSmem, st>>>(p, n, bc, a.state, a.ws.hist, a.ws.keys[0], a.ws.keys[1],
-                                                                a.ws.idx[0], a.ws.idx[1], a.ws.sort_desc[0], a.ws.sort_desc[1]);
-    k_bus_check<<<1, 1, 0, st>>>(bc);                        // a look-back that gave up sets the code
-    const unsigned tiles_grid = (unsigned)std::min<uint64_t>(bus_tiles, (uint64_t)a.sm_count * 8);
-    ScanDesc *agg = (ScanDesc *)a.ws.scan_desc;
-    k_bus_reduce<<<tiles_grid, kBusThreads, 0, st>>>(bc, a.ws.keys[0], a.ws.keys[1], a.ws.idx[0], a.ws.idx[1], a.ws.bus_xfer, bus_busy, agg);
-    k_bus_tile_scan<<<1, 1024, 0, st>>>(bc, agg);
-    k_bus_apply<<<tiles_grid, kBusThreads, 0, st>>>(a.acc, bc, a.ws.keys[0], a.ws.keys[1], a.ws.idx[0], a.ws.idx[1], a.ws.bus_xfer, bus_busy,
-                                                    agg, a.completion, a.stall);
-    k_bus_commit<<<wide, 256, 0, st>>>(bc, a.ws.keys[0], a.ws.keys[1], a.ws.idx[0], a.ws.idx[1], a.completion, bus_busy);
-    k_bus_finish<<<1, 1, 0, st>>>(bc, a.result, a.result_host, a.state);
-    g_kernel_launches += 10 + kMaxPasses;
-    return cudaGetLastError();
+    BusChain c{};
+    c.acc = a.acc; c.n = n; c.completion = a.completion; c.stall = a.stall; c.ranges = a.ranges; c.mp_dev = a.mp_dev; c.bc = bc; c.state = a.state;
+    c.result = a.result; c.result_host = a.result_host; c.plan = static_cast<const BusPlan *>(a.ws.bus_plan); c.busy = bus_busy; c.ws = a.ws;
+    c.wide = (unsigned)std::min<uint64_t>((n + 255) / 256, (uint64_t)a.sm_count * 8);
+    c.hist_grid = (unsigned)std::min<uint64_t>((n + kHistThreads * 8 - 1) / (kHistThreads * 8), (uint64_t)a.sm_count * 4);
+    c.sort_grid = (unsigned)std::min<uint64_t>(sort_tiles, (uint64_t)a.sm_count * 3);
+    c.tiles_grid = (unsigned)std::min<uint64_t>(bus_tiles, (uint64_t)a.sm_count * 8);
+    c.desc_words = sort_tiles * kRadix;
+    e = launch_pdl(k_bus_finish, 1, 1, 0, st, c);
+    if (a.plain_next) *a.plain_next = true;
+    g_kernel_launches += 1;
+    return e;
 }
 
 // =====================================================================================================
@@ -1009,7 +1017,7 @@ cudaError_t launch_bus_stage(const SubmitArgs &a, BatchCtrl *bc, int64_t *bus_bu
 // =====================================================================================================
 static size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
-size_t workspace_layout(uint64_t n, uint32_t n_queues, Workspace *ws, void *base_ptr, int with_bus) {
+size_t workspace_layout(uint64_t n, uint32_t n_queues, uint32_t channels, Workspace *ws, void *base_ptr, int with_bus) {
     const uint64_t nn = n ? n : 1;
     const uint64_t sort_tiles = (nn + kSortTile - 1) / kSortTile, scan_tiles = (nn + kScanTile - 1) / kScanTile;
     size_t off = 0;
@@ -1021,6 +1029,7 @@ size_t workspace_layout(uint64_t n, uint32_t n_queues, Workspace *ws, void *base
     void *k0 = take(nn * 8), *k1 = take(nn * 8), *i0 = take(nn * 4), *i1 = take(nn * 4);
     void *tw = take(nn * 8);
     if (inorder) off = std::max(off, align_up(slots_at + regroup_slot_bytes(nn), 256));
+    if (with_bus) off = std::max(off, align_up(slots_at + bus_entry_bytes(nn, channels), 256));   // (the bus stage's entries, once the batch is served)
     void *rr = take(inorder ? nn * 24 : 0), *ri = take(inorder ? nn * 4 : 0), *rc = take(inorder ? regroup_ctrl_bytes(nn) : 0);
     void *h = take((size_t)kMaxPasses * kRadix * 4);
     void *d0 = take(sort_tiles * kRadix * 4), *d1 = take(sort_tiles * kRadix * 4);
@@ -1031,14 +1040,14 @@ size_t workspace_layout(uint64_t n, uint32_t n_queues, Workspace *ws, void *base
     void *ih = take(inorder ? inorder_head_bytes(in_tiles, n_queues) : 0);
     void *ic = take(inorder ? in_tiles * n_queues : 0);
     void *iq = take(inorder ? inorder_qid_entries(nn) * 2 : 0);
-    void *bx = take(with_bus ? nn * 4 : 0);
+    void *bx = take(with_bus ? nn * 4 : 0), *bp = take(with_bus ? bus_plan_bytes(nn, channels) : 0);
     if (ws) {
         ws->keys[0] = (uint64_t *)k0; ws->keys[1] = (uint64_t *)k1; ws->idx[0] = (uint32_t *)i0; ws->idx[1] = (uint32_t *)i1;
         ws->terms = (uint64_t *)tw;
         ws->rg_ctrl = rc; ws->rg_slots = b ? b + slots_at : nullptr; ws->rg_recs = rr; ws->rg_idx = ri;
         ws->hist = (uint32_t *)h; ws->sort_desc[0] = (uint32_t *)d0; ws->sort_desc[1] = (uint32_t *)d1;
         ws->scan_desc = sd; ws->in_agg = (int64_t *)ia; ws->in_bin = (int64_t *)ib;
-        ws->in_tile = it; ws->in_head = ih; ws->in_headcnt = (uint8_t *)ic; ws->in_qid = (uint16_t *)iq; ws->bus_xfer = (uint32_t *)bx; ws->bytes = off;
+        ws->in_tile = it; ws->in_head = ih; ws->in_headcnt = (uint8_t *)ic; ws->in_qid = (uint16_t *)iq; ws->bus_xfer = (uint32_t *)bx; ws->bus_plan = bp; ws->bytes = off;
     }
     return off;
 }
@@ -1116,10 +1125,6 @@ struct SortChain {
     unsigned cls_grid, hist_grid, sort_grid, scan_grid, stall_grid;
     const InTile *in_tile; uint32_t n_tiles;
 };
-
-__global__ void k_zero_words(uint32_t *p, uint64_t words) {
-    for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < words; i += (uint64_t)gridDim.x * blockDim.x) p[i] = 0u;
-}
 
 // the radix sort's kernels, launched from the device (run_sort is set: the begin kernel starts the batch over)
 __device__ void launch_sort_chain(const SortChain &c, const FinishArgs &f, unsigned fin_grid) {

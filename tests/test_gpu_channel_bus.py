@@ -133,3 +133,27 @@ def test_completion_past_the_key_width_is_refused_before_anything_is_committed(h
     rc_o, c_o, *_ = o_late.submit(late, check=False)
     assert rc_o == 0 and int(c_o.max()) >= (1 << 47)
     compare(g, o, w.acc[2000:])                              # the refusal left the context usable and its state exact
+
+
+@pytest.mark.parametrize("n", [4095, 4097, 21_840, 21_845, 130_001])
+@pytest.mark.parametrize("kind", ["dense", "idle", "one channel", "bunched", "same time", "long span", "shuffled", "programs"])
+def test_buckets_of_reads_match_the_oracle(hbf, kind, n):
+    """Slices of time and channels that hold the average, far more than it (the radix sort takes over), or nothing; times
+    that coincide, that lie seconds apart, or that jump from record to record."""
+    rng = np.random.default_rng(n)
+    acc = np.zeros(n, hbfo.ACCESS_DTYPE)
+    acc["addr"] = wl.RANGE_BASE + rng.integers(0, 1 << 24, n).astype(np.uint64) * 64
+    acc["issue_ns"] = np.sort(rng.integers(0, 150 * n, n))
+    acc["bytes"] = rng.choice([64, 4096, 16000], n)
+    if kind == "idle": acc["issue_ns"] *= 400
+    if kind == "one channel": acc["addr"] = wl.RANGE_BASE + (rng.integers(0, 1 << 8, n).astype(np.uint64) << np.uint64(22))
+    if kind == "bunched": acc["issue_ns"][n // 4:] = acc["issue_ns"][n // 4] + np.arange(n - n // 4) // 100
+    if kind == "same time": acc["issue_ns"][:] = 5
+    if kind == "long span": acc["issue_ns"][n // 2:] += 1 << 40
+    if kind == "shuffled": acc = acc[rng.permutation(n)]
+    acc["flags"] = rng.random(n) < (1.0 if kind == "programs" else 0.02)
+    prof = wl.load_profile("nominal", **wl.GEOMETRY["capacity"])
+    g, o = contexts(hbf, prof, [(wl.RANGE_BASE, wl.GIB, 3, 0, 0, 0)])
+    compare(g, o, acc)
+    acc["issue_ns"] += 20_000
+    compare(g, o, acc)
