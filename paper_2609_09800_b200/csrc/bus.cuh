@@ -16,18 +16,19 @@ __device__ __forceinline__ BusMap bus_shfl_up(const BusMap &v, int o) {
 }
 
 constexpr uint32_t kBusSegs = 64, kBusSamples = 65536;
-constexpr uint32_t kBusAvg = 1365, kBusCap = 4096;         // reads per bucket: aimed at, and at most (three times the average: channels and times differ)
+constexpr uint32_t kBusAvg = 682, kBusCap = 2048;          // reads per bucket: aimed at, and at most (three times the average: channels and times differ)
 constexpr uint32_t kBusMaxChannels = 2048;
+constexpr uint32_t kBusHead = 16;                          // first entries of a bucket, kept in order
 struct BusPlan {
     uint32_t hist[kBusSegs], top[kBusSegs], below[kBusSegs];  // samples of a stretch of time, their largest offset, 2^32 - 1 less their smallest
-    uint32_t blocks, overflow, ticket, shift;
+    uint32_t blocks, overflow, redo, shift;                 // redo: buckets on the list of those to be gone over again
     int64_t lo;
     uint32_t first[kBusSegs], last[kBusSegs];               // the part of a stretch that its share of the slices is spread over
     uint64_t cum[kBusSegs], mul[kBusSegs];                  // in 1/256 slices
 };
-struct __align__(32) BusState { int64_t S, M; uint32_t flag, pad[3]; };   // flag 1: the bucket's own map, 2: the bus after it (M)
+struct BusState { int64_t S, M; };                          // a bucket as one map; then M: the bus before it
 struct BusArgs {
-    BusPlan *plan; uint32_t *cursor; BusState *state; ulonglong2 *entries;
+    BusPlan *plan; uint32_t *cursor, *redo; BusState *state; ulonglong2 *entries, *heads;
     uint32_t channels, slices, cap; int64_t *busy;
 };
 inline uint32_t bus_slices(uint64_t n, uint32_t channels) { return (uint32_t)((n + (uint64_t)kBusAvg * channels - 1) / ((uint64_t)kBusAvg * channels)); }
@@ -36,10 +37,12 @@ inline uint32_t bus_cap(uint64_t n, uint32_t channels) {
     return (uint32_t)(cap < kBusCap ? cap : kBusCap);
 }
 inline size_t bus_entry_bytes(uint64_t n, uint32_t channels) {
-    return channels > kBusMaxChannels ? 0 : ((size_t)3 * n + (size_t)96 * bus_slices(n, channels) * channels) * sizeof(ulonglong2);   // (at least buckets times places)
+    if (channels > kBusMaxChannels) return 0;
+    const size_t buckets = (size_t)bus_slices(n, channels) * channels, a = (size_t)3 * n + 96 * buckets, b = (size_t)kBusCap * buckets;
+    return (a < b ? a : b) * sizeof(ulonglong2);             // (at least buckets times places, and never less for more records)
 }
 inline size_t bus_plan_bytes(uint64_t n, uint32_t channels) {
-    return 8192 + (channels > kBusMaxChannels ? 0 : (size_t)bus_slices(n, channels) * channels * (sizeof(BusState) + 4));
+    return 8192 + (channels > kBusMaxChannels ? 0 : (size_t)bus_slices(n, channels) * channels * (kBusHead * sizeof(ulonglong2) + sizeof(BusState) + 8));
 }
 static_assert(sizeof(BusPlan) <= 8192 && sizeof(BusPlan) % 4 == 0, "the plan's place");
 inline BusArgs bus_args(uint64_t n, uint32_t channels, const Workspace &ws, int64_t *busy) {
@@ -47,8 +50,10 @@ inline BusArgs bus_args(uint64_t n, uint32_t channels, const Workspace &ws, int6
     b.plan = static_cast<BusPlan *>(ws.bus_plan); b.channels = channels; b.busy = busy;
     if (channels > kBusMaxChannels) return b;               // slices = 0: the radix sort serves the batch
     b.slices = bus_slices(n, channels); b.cap = bus_cap(n, channels);
-    b.state = reinterpret_cast<BusState *>(static_cast<char *>(ws.bus_plan) + 8192);
-    b.cursor = reinterpret_cast<uint32_t *>(b.state + (size_t)b.slices * channels);
+    const size_t buckets = (size_t)b.slices * channels;
+    b.heads = reinterpret_cast<ulonglong2 *>(static_cast<char *>(ws.bus_plan) + 8192);
+    b.state = reinterpret_cast<BusState *>(b.heads + kBusHead * buckets);
+    b.cursor = reinterpret_cast<uint32_t *>(b.state + buckets); b.redo = b.cursor + buckets;
     b.entries = static_cast<ulonglong2 *>(ws.rg_slots);
     return b;
 }

@@ -2,16 +2,22 @@
 // transfer queues on the bus of its channel in (array-done time, index) order and holds it for the transfer time; the read
 // completes when the transfer does.  Programs are unchanged.
 //   plan     how the array-done times spread (65,536 samples over 64 stretches): slices of time with about as many reads each,
-//            1,365 per slice and channel
+//            682 per slice and channel
 //   scatter  every read becomes a 16-byte entry (time, index, transfer) in the bucket of its slice and channel.  A block takes
 //            4,096 records, puts their entries in bucket order in shared memory and writes them in runs: their times lie close
 //            together, so that they fall into one or two slices
-//   apply    a block per bucket puts its entries in order (times spread over 4,096 bins of shared memory, the place within a bin
-//            by comparing), composes their maps B -> max(B, D) + x, takes the bus as the slice before left it (look-back over the
-//            buckets of the channel), and writes the completions and stalls of the reads that waited
+//   order    a block per bucket puts its entries in order (times spread over bins of shared memory, the place within a bin by
+//            comparing), writes the completions and stalls of the reads that wait if the bus was idle before the bucket, and
+//            leaves the bucket's map B -> max(B + S, M) and its first 16 entries
+//   join     a block per channel: the bus before every bucket, from the maps; where it is busy, the first entries once more, up to
+//            the one that ends as before: behind it nothing changes
+//   redo     buckets in which the 16 do not reach that far, in full
 // A bucket with more than three times the average sends the batch to the radix sort of (channel, time) in submit_kernels.cu.
 // Bytes per read: 24 + 8 + 16, then 16 and the results that change.  32 M reads with the array stage: 4,112 us with the radix
-// sort (five passes over 12 bytes, two gathers by sorted index), 2,217 in buckets.
+// sort (five passes over 12 bytes, two gathers by sorted index), 1,618 in buckets; 20,011 reads 171 and 79.  What bounds it: scatter
+// 418 us (memory and instructions in equal parts), order some 650 (instructions: 18 per read and lane; barriers).  A block that
+// waited for the bus from the bucket before by look-back instead of assuming it idle: 1,245 us for that kernel; smaller buckets
+// of a warp each, with look-back: 3,100.
 #include <algorithm>
 
 #include "bus.cuh"
@@ -60,7 +66,7 @@ k_bus_start(const hbf_access_t *__restrict__ acc, uint64_t n, const int64_t *__r
     pdl_trigger();
     const int tid = threadIdx.x;
     const uint64_t buckets = (uint64_t)b.slices * b.channels;
-    for (uint64_t i = (uint64_t)blockIdx.x * 1024 + tid; i < buckets; i += (uint64_t)gridDim.x * 1024) { b.cursor[i] = 0u; b.state[i].flag = 0u; }
+    for (uint64_t i = (uint64_t)blockIdx.x * 1024 + tid; i < buckets; i += (uint64_t)gridDim.x * 1024) b.cursor[i] = 0u;
     if (blockIdx.x != 0) return;
     __shared__ long long s_lo, s_hi;
     uint32_t *w = reinterpret_cast<uint32_t *>(bc), *p = reinterpret_cast<uint32_t *>(b.plan);
@@ -250,58 +256,66 @@ k_bus_scatter(const hbf_access_t *__restrict__ acc, uint64_t n, const int64_t *_
     if (late) atomicExch(&bc->code, (int)HBF_E_INVAL);      // an array-done time beyond its 47 bits
 }
 
-constexpr int kBaThreads = 512;
-constexpr uint32_t kBaBins = 4096;
+constexpr int kBaThreads = 256, kBaBlocks = 4;               // (512 x 2 and 341 to 1,365 reads per bucket: 3 to 8 % slower at 32 M or at 20,000)
+constexpr uint32_t kBaBins = kBusCap;
 constexpr int kBaItems = kBusCap / kBaThreads;
 constexpr size_t kBaSmem = (size_t)kBusCap * 16 + (size_t)kBaBins * 4;
+static_assert(kBaItems == 8, "two words of four bins per thread");
+__device__ __forceinline__ int64_t entry_done(const ulonglong2 &e) { return (int64_t)(e.x & kBusDoneMask); }
+__device__ __forceinline__ int64_t entry_xfer(const ulonglong2 &e) { return (int64_t)((e.x >> 47) | ((e.y >> 32) << 17)); }
 
-__global__ void __launch_bounds__(kBaThreads, 2)
-k_bus_buckets(BatchCtrl *bc, const __grid_constant__ BusArgs b, int64_t *__restrict__ completion, int64_t *__restrict__ stall) {
+// REDO = false: the shares of the grid, in order.  REDO = true: the buckets of the list, with the bus before them known.
+template <bool REDO>
+__global__ void __launch_bounds__(kBaThreads, kBaBlocks)
+k_bus_order(BatchCtrl *bc, const __grid_constant__ BusArgs b, int64_t *__restrict__ completion, int64_t *__restrict__ stall) {
     extern __shared__ __align__(16) unsigned char bus_smem[];
     ulonglong2 *s_entry = reinterpret_cast<ulonglong2 *>(bus_smem);           // [kBusCap]
     uint32_t *s_cnt = reinterpret_cast<uint32_t *>(s_entry + kBusCap);        // [kBaBins]
-    __shared__ unsigned long long s_min, s_max;
-    __shared__ uint32_t s_w[kBaThreads / 32], s_bucket;
-    __shared__ BusMap s_map[kBaThreads / 32];
-    __shared__ int64_t s_carry;
-    __shared__ int s_ok;
+    constexpr int kWarps = kBaThreads / 32;
+    __shared__ unsigned long long s_min[kWarps], s_max[kWarps];
+    __shared__ uint32_t s_w[kWarps];
+    __shared__ BusState s_map[kWarps];
     pdl_wait();
     pdl_trigger();
     if (bc->skip || bc->code != HBF_OK || b.plan->overflow) return;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const uint32_t buckets = b.slices * b.channels;
+    const uint32_t count = REDO ? b.plan->redo : b.slices * b.channels;
     long long moved = 0, max_c = INT64_MIN;
-    for (;;) {
-        __syncthreads();
-        if (tid == 0) { s_bucket = atomicAdd(&b.plan->ticket, 1u); s_min = ~0ull; s_max = 0ull; s_ok = 1; }
-        for (uint32_t e = tid; e < kBaBins; e += kBaThreads) s_cnt[e] = 0u;
-        __syncthreads();
-        const uint32_t bucket = s_bucket;                    // (in order: what a bucket waits for is in the hands of blocks that run)
-        if (bucket >= buckets) break;
+    for (uint32_t turn = blockIdx.x; turn < count; turn += gridDim.x) {
+        const uint32_t bucket = REDO ? b.redo[turn] : turn;
         const uint32_t m = min(__ldcg(&b.cursor[bucket]), b.cap);
         ulonglong2 v[kBaItems]; uint32_t bin[kBaItems];
         unsigned long long mn = ~0ull, mx = 0ull;
 #pragma unroll
         for (int k = 0; k < kBaItems; ++k) {
-            const uint32_t e = k * kBaThreads + tid;
-            if (e < m) v[k] = __ldcs(b.entries + (uint64_t)bucket * b.cap + e);
+            if (k * kBaThreads >= m) break;
+            if (k * kBaThreads + tid < m) v[k] = __ldcs(b.entries + (uint64_t)bucket * b.cap + k * kBaThreads + tid);
+        }
+        __syncthreads();                                     // the bucket before is done with
+#pragma unroll
+        for (uint32_t e = 0; e < kBaBins; e += 4 * kBaThreads) *reinterpret_cast<uint4 *>(s_cnt + e + tid * 4) = make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+        for (int k = 0; k < kBaItems; ++k) {
+            if (k * kBaThreads >= m) break;
+            if (k * kBaThreads + tid < m) { const unsigned long long d = v[k].x & kBusDoneMask; mn = min(mn, d); mx = max(mx, d); }
         }
 #pragma unroll
-        for (int k = 0; k < kBaItems; ++k)
-            if (k * kBaThreads + tid < m) { const unsigned long long d = v[k].x & kBusDoneMask; mn = min(mn, d); mx = max(mx, d); }
-#pragma unroll
         for (int o = 16; o > 0; o >>= 1) { mn = min(mn, __shfl_xor_sync(0xffffffffu, mn, o)); mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o)); }
-        if (lane == 0 && mn <= mx) { atomicMin(&s_min, mn); atomicMax(&s_max, mx); }
+        if (lane == 0) { s_min[warp] = mn; s_max[warp] = mx; }
         __syncthreads();
-        const uint64_t t0 = s_min, wide = m ? s_max - t0 : 0ull;
-        const uint32_t sh = wide >> 32 ? 32u - (uint32_t)__clz((int)(wide >> 32)) : 0u;
-        const uint64_t mul = ((uint64_t)kBaBins << 32) / ((wide >> sh) + 1ull);
 #pragma unroll
-        for (int k = 0; k < kBaItems; ++k)
+        for (int w = 0; w < kWarps; ++w) { mn = min(mn, s_min[w]); mx = max(mx, s_max[w]); }
+        const uint64_t t0 = mn, wide = m ? mx - mn : 0ull;
+        const uint32_t sh = wide >> 32 ? 32u - (uint32_t)__clz((int)(wide >> 32)) : 0u;
+        const float scale = (float)kBaBins * 0.999f / ((float)(uint32_t)(wide >> sh) + 1.f);   // (where a bin ends need not be exact, only the same for all)
+#pragma unroll
+        for (int k = 0; k < kBaItems; ++k) {
+            if (k * kBaThreads >= m) break;
             if (k * kBaThreads + tid < m) {
-                const uint32_t d = (uint32_t)(((((v[k].x & kBusDoneMask) - t0) >> sh) * mul) >> 32);
+                const uint32_t d = min(kBaBins - 1u, (uint32_t)((float)(uint32_t)(((v[k].x & kBusDoneMask) - t0) >> sh) * scale));
                 bin[k] = d | (atomicAdd(&s_cnt[d], 1u) << 16);
             }
+        }
         __syncthreads();
         {                                                    // exclusive scan of the bins, eight per thread
             constexpr uint32_t kPer = kBaBins / kBaThreads;
@@ -316,7 +330,9 @@ k_bus_buckets(BatchCtrl *bc, const __grid_constant__ BusArgs b, int64_t *__restr
             for (int o = 1; o < 32; o <<= 1) { const uint32_t t = __shfl_up_sync(0xffffffffu, inc, o); if (lane >= o) inc += t; }
             if (lane == 31) s_w[warp] = inc;
             __syncthreads();
-            uint32_t run = inc - sum + __reduce_add_sync(0xffffffffu, lane < warp ? s_w[lane] : 0u);
+            uint32_t run = inc - sum;
+#pragma unroll
+            for (int w = 0; w < kWarps; ++w) run += w < warp ? s_w[w] : 0u;
 #pragma unroll
             for (uint32_t k = 0; k < kPer; k += 4) {
                 uint4 q;
@@ -326,13 +342,16 @@ k_bus_buckets(BatchCtrl *bc, const __grid_constant__ BusArgs b, int64_t *__restr
         }
         __syncthreads();
 #pragma unroll
-        for (int k = 0; k < kBaItems; ++k)
+        for (int k = 0; k < kBaItems; ++k) {
+            if (k * kBaThreads >= m) break;
             if (k * kBaThreads + tid < m) s_entry[s_cnt[bin[k] & 0xffffu] + (bin[k] >> 16)] = v[k];
+        }
         __syncthreads();
         // an entry's place within its bin: how many of the bin's come before it (rarely more than three in all; reads whose array
         // is done at the very same time share a bin, however many they are)
 #pragma unroll
         for (int k = 0; k < kBaItems; ++k) {
+            if (k * kBaThreads >= m) break;
             if (k * kBaThreads + tid < m) {
                 const uint32_t d = bin[k] & 0xffffu, from = s_cnt[d], to = d + 1u < kBaBins ? s_cnt[d + 1u] : m;
                 uint32_t before = 0;
@@ -349,82 +368,108 @@ k_bus_buckets(BatchCtrl *bc, const __grid_constant__ BusArgs b, int64_t *__restr
         }
         __syncthreads();
 #pragma unroll
-        for (int k = 0; k < kBaItems; ++k)
+        for (int k = 0; k < kBaItems; ++k) {
+            if (k * kBaThreads >= m) break;
             if (k * kBaThreads + tid < m) s_entry[bin[k]] = v[k];
+        }
         __syncthreads();
-        // every thread's stretch of the ordered entries as one map, what lies before it in the bucket, the bucket as a whole
+        // every thread's stretch of the ordered entries as one map, and what lies before it in the bucket
         const uint32_t per = (m + kBaThreads - 1u) / kBaThreads, j0 = min(m, tid * per), j1 = min(m, j0 + per);
-        BusMap mine = bus_identity();
+        int64_t S = 0, M = kNegInf;
         for (uint32_t j = j0; j < j1; ++j) {
             const ulonglong2 e = s_entry[j];
-            const int64_t x = (int64_t)((e.x >> 47) | ((e.y >> 32) << 17)), done = (int64_t)(e.x & kBusDoneMask);
-            mine.S += x; mine.M = max(mine.M, done) + x;     // (kNegInf + x stays far below any time)
+            const int64_t x = entry_xfer(e);
+            S += x; M = max(M, entry_done(e)) + x;           // (kNegInf + x stays far below any time)
         }
-        BusMap incl = mine;
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) { const BusMap p = bus_shfl_up(incl, o); if (lane >= o) incl = bus_then(p, incl); }
-        if (lane == 31) s_map[warp] = incl;
-        __syncthreads();
-        BusMap run = bus_identity();
-        for (int w = 0; w < warp; ++w) run = bus_then(run, s_map[w]);
-        BusMap prev = bus_shfl_up(incl, 1);
-        if (lane == 0) prev = bus_identity();
-        run = bus_then(run, prev);
-        if (warp == 0) {
-            BusMap all = bus_identity();
-            for (int w = 0; w < kBaThreads / 32; ++w) all = bus_then(all, s_map[w]);
-            const uint32_t channel = bucket % b.channels;
-            if (lane == 0) { b.state[bucket].S = all.S; b.state[bucket].M = all.M; st_release_u32(&b.state[bucket].flag, 1u); }
-            // look-back: the buckets of the channel, 32 at a time, the nearest first, as far as one that knows the bus after it
-            BusMap near = bus_identity();
-            int64_t p = (int64_t)(bucket / b.channels) - 1;
-            bool ok = true;
-            for (;; p -= 32) {
-                BusMap at; at.S = 0; at.f = 1; at.M = 0;
-                const int64_t slice = p - lane;
-                if (slice < 0) at.M = b.busy[channel];
-                else {
-                    BusState *st = b.state + ((uint64_t)slice * b.channels + channel);
-                    uint32_t polls = 0, flag;
-                    while ((flag = ld_acquire_u32(&st->flag)) == 0u) { if (++polls > kSpinLimit) { ok = false; break; } }
-                    at.S = ld_relaxed_s64(&st->S); at.M = ld_relaxed_s64(&st->M); at.f = flag == 2u ? 1 : 0;
-                }
-#pragma unroll
-                for (int o = 1; o < 32; o <<= 1) {
-                    BusMap far;
-                    far.S = __shfl_down_sync(0xffffffffu, at.S, o); far.M = __shfl_down_sync(0xffffffffu, at.M, o); far.f = __shfl_down_sync(0xffffffffu, at.f, o);
-                    if (lane + o < 32) at = bus_then(far, at);
-                }
-                at.S = __shfl_sync(0xffffffffu, at.S, 0); at.M = __shfl_sync(0xffffffffu, at.M, 0); at.f = __shfl_sync(0xffffffffu, at.f, 0);
-                near = bus_then(at, near);
-                ok = __all_sync(0xffffffffu, ok);
-                if (near.f || !ok) break;
-            }
-            if (lane == 0) {
-                const int64_t carry = near.M, after = max(carry + all.S, all.M);
-                s_carry = carry; s_ok = ok ? 1 : 0;
-                if (ok) {
-                    // (whoever read "own map" and finds this M already: max(carry + S, after) is the same `after`)
-                    BusState *st = b.state + bucket;
-                    st_relaxed_s64(&st->M, after);
-                    st_release_u32(&st->flag, 2u);
-                    if (bucket / b.channels == b.slices - 1u) b.busy[channel] = after;   // (every slice of the channel has read the old one)
-                }
-            }
+        for (int o = 1; o < 32; o <<= 1) {
+            const int64_t ps = __shfl_up_sync(0xffffffffu, S, o), pm = __shfl_up_sync(0xffffffffu, M, o);
+            if (lane >= o) { M = max(pm + S, M); S += ps; }
         }
+        if (lane == 31) { s_map[warp].S = S; s_map[warp].M = M; }
+        int64_t rs = __shfl_up_sync(0xffffffffu, S, 1), rm = __shfl_up_sync(0xffffffffu, M, 1);
+        if (lane == 0) { rs = 0; rm = kNegInf; }
         __syncthreads();
-        if (!s_ok) { if (tid == 0) atomicExch(&bc->code, (int)HBF_E_TIMEOUT); return; }
-        int64_t bus = max(s_carry + run.S, run.M);
+        int64_t ws = 0, wm = kNegInf;                        // the warps before this one
+        for (int w = 0; w < warp; ++w) { wm = max(wm + s_map[w].S, s_map[w].M); ws += s_map[w].S; }
+        if (!REDO) {
+            if (tid == kBaThreads - 1) { BusState t; t.S = ws + S; t.M = max(wm + S, M); b.state[bucket] = t; }
+            if (tid < (int)min(m, kBusHead)) b.heads[(uint64_t)bucket * kBusHead + tid] = s_entry[tid];
+        }
+        int64_t bus = max(wm + rs, rm), real = REDO ? max(b.state[bucket].M + ws + rs, bus) : 0;
         for (uint32_t j = j0; j < j1; ++j) {
             const ulonglong2 e = s_entry[j];
-            const int64_t x = (int64_t)((e.x >> 47) | ((e.y >> 32) << 17)), done = (int64_t)(e.x & kBusDoneMask);
+            const int64_t x = entry_xfer(e), done = entry_done(e);
             bus = max(bus, done) + x;
-            if (bus != done + x) {                           // the transfer waited for the bus: completion and stall move by the wait
+            if (REDO) real = max(real, done) + x;
+            const int64_t end = REDO ? real : bus, had = REDO ? bus : done + x;
+            if (end != had) {                                // the transfer waits for the bus: completion and stall move by the wait
                 const uint32_t idx = (uint32_t)e.y;
-                completion[idx] = bus; stall[idx] += bus - done - x;
-                moved += bus - done - x; max_c = max(max_c, (long long)bus);
+                completion[idx] = end;
+                atomicAdd(reinterpret_cast<unsigned long long *>(stall + idx), (unsigned long long)(end - had));   // (nothing waits for it)
+                moved += end - had; max_c = max(max_c, (long long)end);
             }
         }
+    }
+    moved = warp_sum(moved); max_c = warp_max(max_c);
+    if (lane == 0) {
+        if (moved) atomicAdd((unsigned long long *)&bc->modeled_ns, (unsigned long long)moved);
+        if (max_c != INT64_MIN) atomicMax(&bc->max_completion_ns, max_c);
+    }
+}
+
+// a block per channel (see above); what it leaves to be gone over again goes to the list
+constexpr int kBjThreads = 512;
+__global__ void __launch_bounds__(kBjThreads)
+k_bus_join(BatchCtrl *bc, const __grid_constant__ BusArgs b, int64_t *__restrict__ completion, int64_t *__restrict__ stall) {
+    __shared__ BusState s_map[kBjThreads / 32];
+    pdl_wait();
+    pdl_trigger();
+    if (bc->skip || bc->code != HBF_OK || b.plan->overflow) return;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    long long moved = 0, max_c = INT64_MIN;
+    for (uint32_t channel = blockIdx.x; channel < b.channels; channel += gridDim.x) {
+        const uint32_t per = (b.slices + kBjThreads - 1u) / kBjThreads, lo = min(b.slices, tid * per), hi = min(b.slices, lo + per);
+        int64_t S = 0, M = kNegInf;
+        for (uint32_t s = lo; s < hi; ++s) { const BusState t = b.state[(uint64_t)s * b.channels + channel]; M = max(M + t.S, t.M); S += t.S; }
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int64_t ps = __shfl_up_sync(0xffffffffu, S, o), pm = __shfl_up_sync(0xffffffffu, M, o);
+            if (lane >= o) { M = max(pm + S, M); S += ps; }
+        }
+        __syncthreads();
+        if (lane == 31) { s_map[warp].S = S; s_map[warp].M = M; }
+        int64_t rs = __shfl_up_sync(0xffffffffu, S, 1), rm = __shfl_up_sync(0xffffffffu, M, 1);
+        if (lane == 0) { rs = 0; rm = kNegInf; }
+        __syncthreads();
+        int64_t bus = b.busy[channel];
+        for (int w = 0; w < warp; ++w) bus = max(bus + s_map[w].S, s_map[w].M);
+        bus = max(bus + rs, rm);
+        for (uint32_t s = lo; s < hi; ++s) {                 // the bus before every bucket of this thread
+            const uint32_t bucket = s * b.channels + channel, m = min(b.cursor[bucket], b.cap), h = min(m, kBusHead);
+            const BusState t = b.state[bucket];
+            const ulonglong2 *head = b.heads + (uint64_t)bucket * kBusHead;
+            int64_t real = bus, had = kNegInf;
+            uint32_t same = 0;                               // the first entry that ends as if the bus had been idle
+            for (; same < h; ++same) {
+                const ulonglong2 e = head[same];
+                had = max(had, entry_done(e)) + entry_xfer(e); real = max(real, entry_done(e)) + entry_xfer(e);
+                if (real == had) break;
+            }
+            if (same == h && m > h) { b.state[bucket].M = bus; b.redo[atomicAdd(&b.plan->redo, 1u)] = bucket; }
+            else {
+                real = bus; had = kNegInf;
+                for (uint32_t j = 0; j < same; ++j) {
+                    const ulonglong2 e = head[j];
+                    had = max(had, entry_done(e)) + entry_xfer(e); real = max(real, entry_done(e)) + entry_xfer(e);
+                    completion[(uint32_t)e.y] = real; stall[(uint32_t)e.y] += real - had;
+                    moved += real - had; max_c = max(max_c, (long long)real);
+                }
+            }
+            bus = max(bus + t.S, t.M);
+        }
+        __syncthreads();                                     // (every thread has read the bus as the batch found it)
+        if (lo < hi && hi == b.slices) b.busy[channel] = bus;
     }
     moved = warp_sum(moved); max_c = warp_max(max_c);
     if (lane == 0) {
@@ -438,8 +483,10 @@ cudaError_t launch_bus_buckets(const SubmitArgs &a, BatchCtrl *bc, int64_t *bus_
     const BusArgs b = bus_args(n, a.mp.channels, a.ws, bus_busy);
     const int fast_ok = fast_geom_ok(a.fast, a.mp) ? 1 : 0;
     cudaError_t e = ensure_dyn_smem((const void *)k_bus_scatter, kBsSmem);
-    if (e == cudaSuccess) e = ensure_dyn_smem((const void *)k_bus_buckets, kBaSmem);
+    if (e == cudaSuccess) e = ensure_dyn_smem((const void *)k_bus_order<false>, kBaSmem);
+    if (e == cudaSuccess) e = ensure_dyn_smem((const void *)k_bus_order<true>, kBaSmem);
     const uint64_t buckets = (uint64_t)b.slices * b.channels;
+    const unsigned order_grid = (unsigned)std::max<uint64_t>(1, std::min<uint64_t>(buckets, (uint64_t)a.sm_count * kBaBlocks));
     if (e == cudaSuccess)
         e = launch_first(a.plain_next, k_bus_start, (unsigned)std::min<uint64_t>((buckets + 1023) / 1024 + 1, (uint64_t)a.sm_count), 1024, 0, st, a.acc, n, (const int64_t *)a.completion,
                          a.ranges, a.mp, a.fast, fast_ok, bc, (const hbf_batch_result_t *)a.result, b);
@@ -450,8 +497,10 @@ cudaError_t launch_bus_buckets(const SubmitArgs &a, BatchCtrl *bc, int64_t *bus_
         e = launch_pdl(k_bus_scatter, (unsigned)std::min<uint64_t>((n + kBsChunk - 1) / kBsChunk, (uint64_t)a.sm_count * 2), kBsThreads, kBsSmem, st, a.acc, n,
                        (const int64_t *)a.completion, a.ranges, a.mp, a.fast, fast_ok, bc, b);
     if (e == cudaSuccess)
-        e = launch_pdl(k_bus_buckets, (unsigned)std::max<uint64_t>(1, std::min<uint64_t>(buckets, (uint64_t)a.sm_count * 2)), kBaThreads, kBaSmem, st, bc, b, a.completion, a.stall);
-    g_kernel_launches += 4;
+        e = launch_pdl(k_bus_order<false>, order_grid, kBaThreads, kBaSmem, st, bc, b, a.completion, a.stall);
+    if (e == cudaSuccess) e = launch_pdl(k_bus_join, std::min<unsigned>(std::max(1u, b.channels), (unsigned)a.sm_count), kBjThreads, 0, st, bc, b, a.completion, a.stall);
+    if (e == cudaSuccess) e = launch_pdl(k_bus_order<true>, order_grid, kBaThreads, kBaSmem, st, bc, b, a.completion, a.stall);
+    g_kernel_launches += 6;
     return e;
 }
 
