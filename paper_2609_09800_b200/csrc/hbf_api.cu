@@ -736,16 +736,11 @@ int hbf_enable_retention(hbf_ctx *c, const hbf_retention_config_t *cfg) {
     if ((rc = dev_copy<uint32_t>(c, &r.rank, nullptr, nb)) != HBF_OK) return rc;
     if ((rc = dev_copy<unsigned long long>(c, &r.die_len, nullptr, c->mp.n_dies)) != HBF_OK) return rc;
     if ((rc = dev_copy<unsigned long long>(c, &r.chan_len, nullptr, c->mp.channels)) != HBF_OK) return rc;
-    r.chan_tab = nullptr;
-    if (c->mp.channels <= kRetTabChannels) {
-        const size_t C = c->mp.channels;
-        if ((rc = dev_copy<uint32_t>(c, &r.chan_tab, nullptr, 2 * C + 1 + C * C)) != HBF_OK) return rc;
-    }
     if ((rc = dev_copy<uint32_t>(c, &r.die_claims, nullptr, c->mp.n_dies)) != HBF_OK) return rc;
     if ((rc = dev_copy<uint32_t>(c, &r.tile_count, nullptr, (HBF_MAX_BATCH + 1023) / 1024 + 1)) != HBF_OK) return rc;
-    if ((rc = dev_copy<double>(c, &r.rate, nullptr, r.n_regions)) != HBF_OK) return rc;
     if ((rc = dev_copy<double>(c, &r.region_temp, nullptr, r.n_regions)) != HBF_OK) return rc;
-    if ((rc = dev_copy<int>(c, &r.region_max, nullptr, r.n_regions)) != HBF_OK) return rc;
+    const std::vector<int> coldest(r.n_regions, (int)0x807fffffu);          // no cell seen: -inf as an ordered integer
+    if ((rc = dev_copy<int>(c, &r.region_max, coldest.data(), r.n_regions)) != HBF_OK) return rc;
     if ((rc = dev_copy<RetState>(c, &r.st, nullptr, 1)) != HBF_OK) return rc;
     c->ret = r; c->ret_cfg = *cfg; c->ret_on = true;
     return HBF_OK;
@@ -757,7 +752,7 @@ int hbf_retention_advance(hbf_ctx *c, int64_t dt_ns, const double *region_temp_c
     if (region_temp_c)                                                      // pageable source: staged before the call returns
         CK(cudaMemcpyAsync(c->ret.region_temp, region_temp_c, c->ret.n_regions * sizeof(double), cudaMemcpyHostToDevice, c->stream));
     CK(launch_ret_advance(c->ret, c->mp, c->thermal ? &c->td : nullptr, c->thermal ? c->td.theta[c->cur] : nullptr,
-                          c->thermal ? c->td.die_region : nullptr, region_temp_c ? 1 : 0, dt_ns, c->sm_count, c->stream));
+                          c->thermal ? c->td.die_region : nullptr, region_temp_c ? 1 : 0, dt_ns, c->sm_count, &c->plain_next, c->stream));
     return HBF_OK;
 }
 

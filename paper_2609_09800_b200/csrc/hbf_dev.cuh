@@ -286,11 +286,11 @@ struct RetState {
     unsigned long long claim_limit;      // this batch: modeled accesses with a smaller batch index claim one quantum each
     unsigned long long claims_now;       // quanta this batch claims if it is accepted
     unsigned long long tickets, counted; // the claim window's tile counter and the modeled accesses counted so far
-    unsigned long long epoch_total;      // quanta the epoch in progress adds
+    unsigned long long epoch_blocks;     // thread blocks of the plan kernel that are done (0 between epochs)
     uint32_t epoch;
     uint32_t observed_inline;            // the in-order serve pass has counted this batch's reads into the disturb counters
 };
-constexpr uint32_t kRetTabChannels = 128;
+constexpr uint32_t kRetTabChannels = 128, kRetTabDies = 128;   // the plan kernel's tables in shared memory
 struct RetDev {
     uint32_t ppb, bpp, bpz, max_pec, disturb_limit, n_regions;
     Div64 div_ppb, div_bpp;              // exact division by pages_per_block and by blocks_per_plane
@@ -302,10 +302,9 @@ struct RetDev {
     uint32_t *plan;                      // [plan_cap] ring of quanta (block * ppb + page), position modulo plan_cap
     uint32_t *rank;                      // [blocks] rank of a newly eligible block in its die's (zone, plane, block) order
     unsigned long long *die_len, *chan_len;   // quanta the epoch in progress adds per die, per channel
-    uint32_t *chan_tab;                  // the channels' lengths sorted, their running sums, and per channel the sorted lengths of the channels before it (null: more than kRetTabChannels channels)
     uint32_t *die_claims;                // [dies] quanta claimed on each die by the batch in progress
     uint32_t *tile_count;                // [tiles of 1,024 records] modeled accesses, claim window
-    double *rate, *region_temp;          // [regions] damage per block of this epoch; temperatures
+    double *region_temp;                 // [regions] temperatures
     int *region_max;                     // [regions] hottest cell, as an ordered integer
     RetState *st;
 };
@@ -314,7 +313,7 @@ cudaError_t launch_ret_close(const hbf_access_t *acc, uint64_t n, const RangeSna
                              const hbf_batch_result_t *result, int64_t *pending, int binned, const RetDev &r, int sm_count, cudaStream_t st);
 struct ThermalDev;
 cudaError_t launch_ret_advance(const RetDev &r, const ModelParams &mp, const ThermalDev *field, const float *theta, const int32_t *die_region,
-                               int have_temps, int64_t dt_ns, int sm_count, cudaStream_t st);
+                               int have_temps, int64_t dt_ns, int sm_count, bool *plain_next, cudaStream_t st);
 cudaError_t launch_ret_decay(const RetDev &r, const ModelParams &mp, const DevState *state, int64_t idle_ns, int sm_count, cudaStream_t st);
 
 // ---- thermal -------------------------------------------------------------------------------------

@@ -215,27 +215,47 @@ cudaError_t launch_ret_close(const hbf_access_t *acc, uint64_t n, const RangeSna
 }
 
 // =====================================================================================================
-// one epoch: temperatures -> damage -> eligibility -> plan
+// one epoch: temperatures -> damage -> eligibility -> plan.  Three launches that overlap their starts (two when the caller gives
+// the temperatures): the regions' hottest cells; a block per die for rate, damage, eligibility and ranks; the plan, whose last
+// block closes the epoch.  65,536 blocks on a 128 x 128 field: 36 us of kernels and 8 gaps as eight
+// launches, 17 us and 3 overlapped starts now (a coupled window of 1 ms: 106 -> 76 us).
+// Between epochs region_max holds nothing and chan_len zeros: the last block of the plan kernel leaves them so.
 // =====================================================================================================
 __device__ __forceinline__ int ordered_int(float f) { const int k = __float_as_int(f); return k >= 0 ? k : k ^ 0x7fffffff; }
 __device__ __forceinline__ float ordered_float(int k) { return __int_as_float(k >= 0 ? k : k ^ 0x7fffffff); }
 
-__global__ void k_ret_region_clear(RetDev r) {
-    for (uint32_t g = threadIdx.x; g < r.n_regions; g += blockDim.x) r.region_max[g] = ordered_int(-INFINITY);
-}
 __global__ void __launch_bounds__(256)
 k_ret_region_max(const float *__restrict__ theta, const int32_t *__restrict__ cell_region, uint64_t n_cells, RetDev r) {
-    const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-    for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_cells; i += stride) {
-        const int32_t g = cell_region[i];
-        if (g >= 0) atomicMax(&r.region_max[g], ordered_int(theta[i]));
+    const uint64_t stride = (uint64_t)gridDim.x * blockDim.x, first = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    int32_t g = first < n_cells ? cell_region[first] : -1;   // (the floorplan does not change: read before the field is there)
+    pdl_wait();
+    pdl_trigger();
+    for (uint64_t i = first; i - threadIdx.x % 32u < n_cells; i += stride) {     // (whole warps)
+        if (i != first) g = i < n_cells ? cell_region[i] : -1;
+        const int v = g >= 0 ? ordered_int(__ldg(theta + i)) : 0;
+        int32_t same;
+        __match_all_sync(0xffffffffu, g, &same);             // cells side by side mostly lie in one region
+        if (same) {
+            const int m = __reduce_max_sync(0xffffffffu, v);
+            if (g >= 0 && lane_id() == 0) atomicMax(&r.region_max[g], m);
+        } else if (g >= 0) {
+            atomicMax(&r.region_max[g], v);
+        }
     }
 }
 
-// Arrhenius lifetime at each region's temperature (first equation of D4) and the damage it adds per block in this
-// epoch (second equation of D4); opens the epoch
-__global__ void k_ret_rate(RetDev r, int from_field, float ambient_c, double dt_s) {
-    for (uint32_t g = threadIdx.x; g < r.n_regions; g += blockDim.x) {
+// a block per die: Arrhenius lifetime at its region's temperature (first equation of D4) and the damage it adds per block in
+// this epoch (second equation of D4); eligibility; the rank of every newly eligible block in the die's (zone, plane, block) order
+constexpr int kRetDieThreads = 256;
+__global__ void __launch_bounds__(kRetDieThreads)
+k_ret_die(RetDev r, const int32_t *__restrict__ die_region, uint32_t planes, uint32_t dies, int from_field, float ambient_c, double dt_s) {
+    __shared__ double s_rate;
+    pdl_wait();
+    pdl_trigger();
+    const uint32_t epoch = r.st->epoch + 1u, die = blockIdx.x;
+    const uint32_t per_die = planes * r.bpp, zone_span = planes * r.bpz;
+    if (threadIdx.x == 0) {
+        const uint32_t g = die_region ? (uint32_t)die_region[die] : 0u;
         double temp_c;
         if (from_field) {
             const float rise = ordered_float(r.region_max[g]);
@@ -244,161 +264,157 @@ __global__ void k_ret_rate(RetDev r, int from_field, float ambient_c, double dt_
             temp_c = r.region_temp[g];
         }
         const double life = r.l_ref_s * exp(r.ea_over_kb * (1.0 / (temp_c + 273.15) - 1.0 / r.t_ref_k));
-        r.rate[g] = r.accel * dt_s / life;
+        s_rate = r.accel * dt_s / life;
     }
-    if (threadIdx.x == 0) r.st->epoch += 1u;
-}
-
-__global__ void __launch_bounds__(256)
-k_ret_damage(RetDev r, const int32_t *__restrict__ die_region, uint32_t blocks_per_die) {
-    const uint32_t epoch = r.st->epoch;
-    const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-    for (uint64_t b = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; b < r.n_blocks; b += stride) {
-        if (r.worn[b]) continue;
-        const uint32_t g = die_region ? (uint32_t)die_region[b / blocks_per_die] : 0u;
-        const double d = r.damage[b] + r.rate[g];
-        r.damage[b] = d;
-        if (r.epoch_of[b] == 0u && (d >= r.lead || (r.disturb_limit && r.disturb[b] >= r.disturb_limit))) r.epoch_of[b] = epoch;
-    }
-}
-
-// one thread block per die: rank of every newly eligible block in the die's (zone, plane, block) order
-constexpr int kRetRankThreads = 256;
-__global__ void __launch_bounds__(kRetRankThreads)
-k_ret_rank(RetDev r, uint32_t planes) {
-    const uint32_t epoch = r.st->epoch, die = blockIdx.x;
-    const uint32_t per_die = planes * r.bpp, zone_span = planes * r.bpz;
     uint32_t running = 0;
-    for (uint32_t o0 = 0; o0 < per_die; o0 += kRetRankThreads) {
+    for (uint32_t o0 = 0; o0 < per_die; o0 += kRetDieThreads) {
         const uint32_t o = o0 + threadIdx.x;
-        uint64_t b = 0; uint32_t flag = 0;
+        uint64_t b = 0; uint32_t flag = 0, was = 0, hits = 0; double d = 0.0; bool worn = true;
         if (o < per_die) {
             const uint32_t zone = o / zone_span, rem = o % zone_span, pl = rem / r.bpz, kk = rem % r.bpz;
             b = ((uint64_t)die * planes + pl) * r.bpp + zone * r.bpz + kk;
-            flag = r.epoch_of[b] == epoch ? 1u : 0u;
+            worn = r.worn[b] != 0; d = r.damage[b]; was = r.epoch_of[b];
+            if (r.disturb_limit) hits = r.disturb[b];
+        }
+        if (o0 == 0u) __syncthreads();                       // (the rate)
+        if (!worn) {
+            d += s_rate;
+            r.damage[b] = d;
+            if (was == 0u && (d >= r.lead || (r.disturb_limit && hits >= r.disturb_limit))) { r.epoch_of[b] = epoch; flag = 1u; }
         }
         uint32_t sum = 0;
-        const uint32_t incl = block_scan_incl<kRetRankThreads>(flag, &sum);
+        const uint32_t incl = block_scan_incl<kRetDieThreads>(flag, &sum);
         if (flag) r.rank[b] = running + incl - 1u;
         running += sum;
     }
-    if (threadIdx.x == 0) r.die_len[die] = (unsigned long long)running * r.ppb;
-}
-
-__global__ void k_ret_chan(RetDev r, uint32_t channels, uint32_t dies) {
-    __shared__ unsigned long long s_total;
-    if (threadIdx.x == 0) s_total = 0ull;
-    __syncthreads();
-    for (uint32_t c = threadIdx.x; c < channels; c += blockDim.x) {
-        unsigned long long s = 0;
-        for (uint32_t d = 0; d < dies; ++d) s += r.die_len[c * dies + d];
-        r.chan_len[c] = s;
-        atomicAdd(&s_total, s);
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) r.st->epoch_total = s_total;
-    // For the plan kernel: the lengths in ascending order with their running sums, and for every channel the lengths of
-    // the channels before it in ascending order.  With them the place of a quantum among the channels, a sum of
-    // min(length, x) over all channels and a count of longer channels before its own, takes two binary searches
-    // instead of a pass over the channels.  (Every length, and their sum, is below 2^32.)
-    if (r.chan_tab) {
-        uint32_t *sorted = r.chan_tab, *run = r.chan_tab + channels, *before = r.chan_tab + 2 * channels + 1;
-        for (uint32_t c = threadIdx.x; c < channels; c += blockDim.x) {
-            const unsigned long long lc = r.chan_len[c];
-            uint32_t at = 0;
-            for (uint32_t j = 0; j < channels; ++j) { const unsigned long long lj = r.chan_len[j]; at += (lj < lc || (lj == lc && j < c)) ? 1u : 0u; }
-            sorted[at] = (uint32_t)lc;
-        }
-        for (uint32_t k = threadIdx.x; k < channels * channels; k += blockDim.x) {
-            const uint32_t ch = k / channels, c = k % channels;      // channel c among the channels before ch
-            if (c >= ch) continue;
-            const unsigned long long lc = r.chan_len[c];
-            uint32_t at = 0;
-            for (uint32_t j = 0; j < ch; ++j) { const unsigned long long lj = r.chan_len[j]; at += (lj < lc || (lj == lc && j < c)) ? 1u : 0u; }
-            before[(size_t)ch * channels + at] = (uint32_t)lc;
-        }
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            uint32_t sum = 0;
-            for (uint32_t k = 0; k < channels; ++k) { run[k] = sum; sum += sorted[k]; }
-            run[channels] = sum;
-        }
+    if (threadIdx.x == 0) {
+        const unsigned long long len = (unsigned long long)running * r.ppb;
+        r.die_len[die] = len;
+        if (len) atomicAdd(&r.chan_len[die / dies], len);
     }
 }
 
 // how many of the n ascending values at tab are at most x
-__device__ __forceinline__ uint32_t count_at_most(const uint32_t *__restrict__ tab, uint32_t n, uint32_t x) {
+__device__ __forceinline__ uint32_t count_at_most(const uint32_t *tab, uint32_t n, uint32_t x) {
     uint32_t lo = 0, len = n;
     while (len > 0u) {
         const uint32_t half = len >> 1;
-        if (__ldg(tab + lo + half) <= x) { lo += half + 1u; len -= half + 1u; } else len = half;
+        if (tab[lo + half] <= x) { lo += half + 1u; len -= half + 1u; } else len = half;
     }
     return lo;
 }
 
-// one warp per block, its lanes over the block's pages.  Every length and rank of an epoch is below 2^32 (a quantum id
-// is 32 bits and a block is planned at most once at a time), so the arithmetic is 32-bit.
+// `split` blocks per die, one warp per eligible block, its lanes over the block's pages.  Every length and rank of an epoch is
+// below 2^32 (a quantum id is 32 bits and a block is planned at most once at a time), so the arithmetic is 32-bit.
+// TAB: the channels' lengths in ascending order with their running sums, and the lengths of the channels before the die's in
+// ascending order, in shared memory: the place of a quantum among the channels, a sum of min(length, x) over all channels and
+// a count of longer channels before its own, then takes two binary searches instead of a pass over the channels.
+template <bool TAB>
 __global__ void __launch_bounds__(256)
-k_ret_emit(RetDev r, uint32_t channels, uint32_t dies, uint32_t planes) {
-    const RetState *st = r.st;
-    const uint32_t epoch = st->epoch;
-    const unsigned long long base = st->planned;
-    const uint64_t base_mod = base % r.plan_cap;
-    const uint32_t blocks_per_die = planes * r.bpp;
-    const int lane = threadIdx.x & 31;
-    const uint64_t warps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
-    for (uint64_t b = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; b < r.n_blocks; b += warps) {
-        if (r.epoch_of[b] != epoch) continue;
-        const uint32_t die = (uint32_t)(b / blocks_per_die), ch = die / dies, di = die % dies;
-        const uint32_t first = r.rank[b] * r.ppb;
+k_ret_emit(RetDev r, uint32_t channels, uint32_t dies, uint32_t planes, uint32_t split) {
+    __shared__ uint32_t s_len[TAB ? kRetTabChannels : 1], s_sorted[TAB ? kRetTabChannels : 1], s_sum[TAB ? kRetTabChannels + 1 : 1], s_before[TAB ? kRetTabChannels : 1];
+    __shared__ uint32_t s_dies[TAB ? kRetTabDies : 1];
+    __shared__ uint32_t s_last;
+    pdl_wait();
+    pdl_trigger();
+    RetState *st = r.st;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const uint32_t die = blockIdx.x / split, part = blockIdx.x % split, ch = die / dies, di = die % dies;
+    if (r.die_len[die]) {
+        const uint32_t epoch = st->epoch + 1u;
+        const unsigned long long base = st->planned;
+        const uint64_t base_mod = base % r.plan_cap;
+        const uint32_t blocks_per_die = planes * r.bpp;
         const unsigned long long *dlen = r.die_len + (size_t)ch * dies;
-        for (uint32_t pg = (uint32_t)lane; pg < r.ppb; pg += 32u) {
-            const uint32_t r_die = first + pg;
-            uint32_t r_ch = 0;
-            for (uint32_t d = 0; d < dies; ++d) {
-                const uint32_t len = (uint32_t)__ldg(dlen + d);
-                r_ch += min(len, r_die) + ((d < di && len > r_die) ? 1u : 0u);
-            }
-            uint32_t pos = 0;
-            if (r.chan_tab) {
-                const uint32_t k = count_at_most(r.chan_tab, channels, r_ch);                       // channels no longer than r_ch: all of theirs
-                pos = __ldg(r.chan_tab + channels + k) + r_ch * (channels - k);                       // the others: r_ch each
-                pos += ch - count_at_most(r.chan_tab + 2 * channels + 1 + (size_t)ch * channels, ch, r_ch);   // and one more of every longer channel before this one
-            } else {
-                for (uint32_t c = 0; c < channels; ++c) {
-                    const uint32_t len = (uint32_t)__ldg(r.chan_len + c);
-                    pos += min(len, r_ch) + ((c < ch && len > r_ch) ? 1u : 0u);
+        uint32_t n_before = 0;
+        if constexpr (TAB) {
+            for (uint32_t c = tid; c < channels; c += 256u) s_len[c] = (uint32_t)r.chan_len[c];
+            for (uint32_t d = tid; d < dies; d += 256u) s_dies[d] = (uint32_t)dlen[d];
+            __syncthreads();
+            for (uint32_t c = tid; c < channels; c += 256u) {
+                const uint32_t lc = s_len[c];
+                uint32_t all = 0, before = 0;
+                for (uint32_t j = 0; j < channels; ++j) {
+                    const uint32_t first = s_len[j] < lc || (s_len[j] == lc && j < c) ? 1u : 0u;
+                    all += first; before += j < ch ? first : 0u;
                 }
+                s_sorted[all] = lc;
+                if (c < ch) s_before[before] = lc;
             }
-            uint64_t slot = base_mod + pos;
-            if (slot >= r.plan_cap) slot -= r.plan_cap;
-            r.plan[slot] = (uint32_t)(b * r.ppb + pg);
-            if (pg + 1u == r.ppb) r.last_pos[b] = base + pos;       // the last page's place: a block's pages go out in order
+            __syncthreads();
+            if (warp == 0) {
+                uint32_t run = 0;
+                for (uint32_t c0 = 0; c0 < channels; c0 += 32u) {
+                    const uint32_t v = c0 + lane < channels ? s_sorted[c0 + lane] : 0u;
+                    uint32_t inc = v;
+#pragma unroll
+                    for (int o = 1; o < 32; o <<= 1) { const uint32_t t = __shfl_up_sync(0xffffffffu, inc, o); if (lane >= o) inc += t; }
+                    if (c0 + lane < channels) s_sum[c0 + lane] = run + inc - v;
+                    run += __shfl_sync(0xffffffffu, inc, 31);
+                }
+                if (lane == 0) s_sum[channels] = run;
+            }
+            n_before = ch;
+            __syncthreads();
+        }
+        for (uint32_t k = part * 8u + warp; k < blocks_per_die; k += split * 8u) {
+            const uint64_t b = (uint64_t)die * blocks_per_die + k;
+            if (r.epoch_of[b] != epoch) continue;
+            const uint32_t first = r.rank[b] * r.ppb;
+            for (uint32_t pg = (uint32_t)lane; pg < r.ppb; pg += 32u) {
+                const uint32_t r_die = first + pg;
+                uint32_t r_ch = 0, pos = 0;
+                for (uint32_t d = 0; d < dies; ++d) {
+                    const uint32_t len = TAB ? s_dies[d] : (uint32_t)dlen[d];
+                    r_ch += min(len, r_die) + ((d < di && len > r_die) ? 1u : 0u);
+                }
+                if constexpr (TAB) {
+                    const uint32_t q = count_at_most(s_sorted, channels, r_ch);        // channels no longer than r_ch: all of theirs
+                    pos = s_sum[q] + r_ch * (channels - q);                             // the others: r_ch each
+                    pos += n_before - count_at_most(s_before, n_before, r_ch);          // and one more of every longer channel before this one
+                } else {
+                    for (uint32_t c = 0; c < channels; ++c) {
+                        const uint32_t len = (uint32_t)r.chan_len[c];
+                        pos += min(len, r_ch) + ((c < ch && len > r_ch) ? 1u : 0u);
+                    }
+                }
+                uint64_t slot = base_mod + pos;
+                if (slot >= r.plan_cap) slot -= r.plan_cap;
+                r.plan[slot] = (uint32_t)(b * r.ppb + pg);
+                if (pg + 1u == r.ppb) r.last_pos[b] = base + pos;       // the last page's place: a block's pages go out in order
+            }
         }
     }
+    __syncthreads();
+    if (tid == 0) { __threadfence(); s_last = atomicAdd(&st->epoch_blocks, 1ull) == gridDim.x - 1u ? 1u : 0u; }
+    __syncthreads();
+    if (!s_last) return;
+    // the last block: every other one has read what changes here
+    __threadfence();
+    unsigned long long total = 0;
+    for (uint32_t c = tid; c < channels; c += 256u) { total += __ldcg(r.chan_len + c); r.chan_len[c] = 0ull; }
+    total = (unsigned long long)warp_sum((long long)total);
+    if (lane == 0 && total) atomicAdd(&st->planned, total);
+    for (uint32_t g = tid; g < r.n_regions; g += 256u) r.region_max[g] = ordered_int(-INFINITY);
+    if (tid == 0) { st->epoch += 1u; st->epoch_blocks = 0ull; }
 }
 
-__global__ void k_ret_epoch_close(RetDev r) { r.st->planned += r.st->epoch_total; r.st->epoch_total = 0ull; }
-
 cudaError_t launch_ret_advance(const RetDev &r, const ModelParams &mp, const ThermalDev *field, const float *theta, const int32_t *die_region,
-                               int have_temps, int64_t dt_ns, int sm_count, cudaStream_t st) {
+                               int have_temps, int64_t dt_ns, int sm_count, bool *plain_next, cudaStream_t st) {
     const int from_field = have_temps ? 0 : 1;
-    float ambient = 0.0f;
+    const float ambient = from_field ? field->ambient_c : 0.0f;
+    cudaError_t e = cudaSuccess;
     if (from_field) {
         const uint64_t cells = (uint64_t)field->H * field->W;
-        ambient = field->ambient_c;
-        k_ret_region_clear<<<1, 256, 0, st>>>(r);
-        k_ret_region_max<<<ret_grid(cells, sm_count), 256, 0, st>>>(theta, field->cell_region, cells, r);
-        g_kernel_launches += 2;
+        e = launch_first(plain_next, k_ret_region_max, ret_grid(cells, sm_count), 256, 0, st, theta, field->cell_region, cells, r);
+        g_kernel_launches += 1;
     }
-    k_ret_rate<<<1, 256, 0, st>>>(r, from_field, ambient, (double)dt_ns * 1e-9);
-    k_ret_damage<<<ret_grid(r.n_blocks, sm_count), 256, 0, st>>>(r, die_region, mp.planes * r.bpp);
-    k_ret_rank<<<mp.n_dies, kRetRankThreads, 0, st>>>(r, mp.planes);
-    k_ret_chan<<<1, 256, 0, st>>>(r, mp.channels, mp.dies);
-    k_ret_emit<<<ret_grid(r.n_blocks * 32, sm_count), 256, 0, st>>>(r, mp.channels, mp.dies, mp.planes);
-    k_ret_epoch_close<<<1, 1, 0, st>>>(r);
-    g_kernel_launches += 6;
-    return cudaGetLastError();
+    if (e == cudaSuccess) e = launch_first(plain_next, k_ret_die, mp.n_dies, kRetDieThreads, 0, st, r, die_region, mp.planes, mp.dies, from_field, ambient, (double)dt_ns * 1e-9);
+    const uint32_t split = std::max<uint32_t>(1u, std::min<uint32_t>((uint32_t)(sm_count * 8) / mp.n_dies, (mp.planes * r.bpp + 7u) / 8u));   // eight blocks per multiprocessor where the dies are fewer
+    if (e == cudaSuccess)
+        e = launch_pdl(mp.channels <= kRetTabChannels && mp.dies <= kRetTabDies ? k_ret_emit<true> : k_ret_emit<false>, mp.n_dies * split, 256, 0, st, r, mp.channels, mp.dies, mp.planes, split);
+    g_kernel_launches += 2;
+    return e;
 }
 
 // =====================================================================================================

@@ -411,8 +411,13 @@ k_small_serve(const __grid_constant__ SmallArgs a) {
         }
         if (EXTRA && a.ret_on && !a.bus_on && claims) {      // blocks whose last quantum is now claimed commit one cycle
             const unsigned long long mark = a.ret.st->planned - debt + claims;
-            for (uint64_t b = (uint64_t)rank * kSmThreads + tid; b < a.ret.n_blocks; b += (uint64_t)blocks * kSmThreads)
-                if (a.ret.epoch_of[b] != 0u && a.ret.last_pos[b] < mark) ret_commit_block(a.ret, b);
+            for (uint64_t b = ((uint64_t)rank * kSmThreads + tid) * 4u; b < a.ret.n_blocks; b += (uint64_t)blocks * kSmThreads * 4u) {
+                uint32_t e[4] = {0u, 0u, 0u, 0u};            // (four at a time: most blocks wait for nothing)
+                if (b + 4u <= a.ret.n_blocks) *reinterpret_cast<uint4 *>(e) = *reinterpret_cast<const uint4 *>(a.ret.epoch_of + b);
+                else for (uint32_t k = 0; b + k < a.ret.n_blocks; ++k) e[k] = a.ret.epoch_of[b + k];
+#pragma unroll
+                for (uint32_t k = 0; k < 4u; ++k) if (e[k] != 0u && a.ret.last_pos[b + k] < mark) ret_commit_block(a.ret, b + k);
+            }
         }
         if (warp == kSmWarps - 1) {
             const long long stall = warp_sum(lane < kSmWarps ? w_stall[lane] : 0), latest = warp_max(lane < kSmWarps ? w_max[lane] : INT64_MIN);
