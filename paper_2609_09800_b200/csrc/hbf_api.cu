@@ -49,7 +49,7 @@ struct hbf_ctx {
     bool plain_next = false;                     // what was enqueued last may launch kernels of its own: see launch_first
     TileBalanceHost bal;                         // tile sizes of the in-order path from the times earlier batches left
     // thermal steps on a reduced-order model instead of the grid (off while rom == nullptr)
-    hbf_rom *rom = nullptr; int64_t rom_dt_ns = 0; int32_t *d_rom_kind = nullptr; double *d_rom_p = nullptr, *d_rom_T = nullptr;
+    hbf_rom *rom = nullptr; int64_t rom_dt_ns = 0; int32_t *d_rom_kind = nullptr; double *d_rom_T = nullptr;
     // channel bus as a second queued stage (off while d_bus_busy == nullptr)
     int64_t *d_bus_busy = nullptr; BatchCtrl *d_bus_ctrl = nullptr;
     // time-bin energy ledger (off while bin_ns == 0)
@@ -215,10 +215,11 @@ int hbf_attach_rom(hbf_ctx *c, hbf_rom *r, const int32_t *output_kind, int64_t d
     if (!r) { c->rom = nullptr; return HBF_OK; }               // back to the grid
     if (!output_kind || dt_ns <= 0 || r->m != c->td.n_regions || r->stream != c->stream) return HBF_E_INVAL;
     if (c->d_rom_kind) { cudaFree(c->d_rom_kind); c->d_rom_kind = nullptr; }
-    if (c->d_rom_p) { cudaFree(c->d_rom_p); c->d_rom_p = nullptr; }
+    if (c->d_rom_T) { cudaFree(c->d_rom_T); c->d_rom_T = nullptr; }
     if (cudaMalloc(&c->d_rom_kind, r->o * sizeof(int32_t)) != cudaSuccess) return HBF_E_NOMEM;
-    if (cudaMalloc(&c->d_rom_p, ((size_t)r->m + r->o) * sizeof(double)) != cudaSuccess) return HBF_E_NOMEM;
-    c->d_rom_T = c->d_rom_p + r->m;
+    const size_t bytes = ((size_t)r->o + r->n + 1) * sizeof(double);       // outputs, next state, the step kernel's block counter
+    if (cudaMalloc(&c->d_rom_T, bytes) != cudaSuccess) return HBF_E_NOMEM;
+    CK(cudaMemsetAsync(c->d_rom_T, 0, bytes, c->stream));
     CK(cudaMemcpyAsync(c->d_rom_kind, output_kind, r->o * sizeof(int32_t), cudaMemcpyHostToDevice, c->stream));
     CK(cudaStreamSynchronize(c->stream));
     c->rom = r; c->rom_dt_ns = dt_ns;
@@ -260,7 +261,7 @@ int hbf_destroy(hbf_ctx *c) {
     if (c->d_bus_busy) cudaFree(c->d_bus_busy);
     if (c->d_bus_ctrl) cudaFree(c->d_bus_ctrl);
     if (c->d_rom_kind) cudaFree(c->d_rom_kind);
-    if (c->d_rom_p) cudaFree(c->d_rom_p);
+    if (c->d_rom_T) cudaFree(c->d_rom_T);
     if (c->pipe.made) {
         hbf_ctx::HostPipe &p = c->pipe;
         cudaStreamSynchronize(p.s_in); cudaStreamSynchronize(p.s_out);
@@ -530,6 +531,7 @@ int hbf_submit_batch(hbf_ctx *c, const hbf_access_t *d_acc, uint64_t n, int64_t 
     return HBF_OK;
 }
 
+constexpr uint64_t kHostResultsMax = 65536;                  // records
 // Host-buffer submit: the batch is cut into chunks; the copy-in of chunk k+1, the service of chunk k (hbf_submit_batch)
 // and the read-back of chunk k-1 run on three streams, so the link moves both ways while the kernels run.
 static int host_pipe_prepare(hbf_ctx *c, uint64_t chunk) {
@@ -575,6 +577,39 @@ int hbf_submit_host(hbf_ctx *c, const hbf_access_t *h_acc, uint64_t n, int64_t *
     if (rc != HBF_OK) return rc;
     hbf_ctx::HostPipe &p = c->pipe;
     cudaStream_t main = c->stream;
+    if (n && n <= chunk) {                                   // one chunk: nothing to overlap, so one stream and no events
+        CK(cudaMemcpyAsync(p.acc[0], h_acc, n * sizeof(hbf_access_t), cudaMemcpyHostToDevice, main));
+        rc = hbf_submit_batch(c, p.acc[0], n, p.comp[0], p.stall[0], nullptr, h_die_stats ? p.stats : nullptr, p.ws, p.ws_bytes);
+        if (rc != HBF_OK) { cudaStreamSynchronize(main); return rc; }
+        // A small batch's results leave in one kernel where the device can write the caller's buffers (pinned memory): four
+        // copies cost more than the bytes.  The call as a whole with copies and so: 2,000 records 44 and 33 us, 5,900 48 and
+        // 39, 16,384 107 and 95, 65,536 218 and 160; at 262,144 the two are alike.
+        int64_t *dev[3] = {nullptr, nullptr, nullptr};
+        void *const host[3] = {h_completion_ns, h_stall_ns, h_die_stats};
+        bool writable = n <= kHostResultsMax;
+        for (int k = 0; k < 3 && writable; ++k) {
+            cudaPointerAttributes at;
+            if (!host[k]) continue;
+            writable = cudaPointerGetAttributes(&at, host[k]) == cudaSuccess && at.type == cudaMemoryTypeHost && at.devicePointer;
+            dev[k] = static_cast<int64_t *>(at.devicePointer);
+        }
+        if (!writable) (void)cudaGetLastError();
+        if (writable) {
+            CK(launch_host_results(p.comp[0], p.stall[0], p.stats, c->d_result, n, c->mp.n_dies, dev[0], dev[1], reinterpret_cast<hbf_die_stats_t *>(dev[2]), p.h_sum,
+                                   &c->plain_next, main));
+        } else {
+            CK(cudaMemcpyAsync(h_completion_ns, p.comp[0], n * 8, cudaMemcpyDeviceToHost, main));
+            CK(cudaMemcpyAsync(h_stall_ns, p.stall[0], n * 8, cudaMemcpyDeviceToHost, main));
+            if (h_die_stats) CK(cudaMemcpyAsync(h_die_stats, p.stats, (size_t)c->mp.n_dies * sizeof(hbf_die_stats_t), cudaMemcpyDeviceToHost, main));
+            CK(cudaMemcpyAsync(p.h_sum, c->d_result, sizeof(hbf_batch_result_t), cudaMemcpyDeviceToHost, main));
+        }
+        CK(cudaStreamSynchronize(main));
+        if (p.h_sum->code == HBF_E_LINK_SHUTDOWN) c->terminal = true;
+        if (p.h_sum->code == HBF_E_LINK_SHUTDOWN || p.h_sum->code == HBF_E_THROTTLED)       // (refused before anything was written)
+            if (h_die_stats) memset(h_die_stats, 0, (size_t)c->mp.n_dies * sizeof(hbf_die_stats_t));
+        if (summary_out) *summary_out = *p.h_sum;
+        return p.h_sum->code;
+    }
     CK(cudaEventRecord(p.start, main));                      // the side streams begin behind what the context has enqueued so far
     CK(cudaStreamWaitEvent(p.s_in, p.start, 0)); CK(cudaStreamWaitEvent(p.s_out, p.start, 0));
     CK(cudaMemsetAsync(p.total, 0, (size_t)c->mp.n_dies * sizeof(hbf_die_stats_t), main));
@@ -887,9 +922,9 @@ int hbf_thermal_step(hbf_ctx *c, int64_t dt_ns, const float *ext_power_w, uint32
     if (c->profiling) CK(cudaEventRecord(c->ev_th[0], c->stream));
     if (c->rom) {                                            // the attached model stands in for the grid
         if (bin_row) CK(launch_take_bin(bin_row, c->d_pending, c->mp.n_dies, c->stream));
-        CK(launch_rom_power(td, c->d_pending, dt_ns, n_ext != 0, c->d_rom_p, c->stream));
-        { const int rc_ = hbf_rom_step(c->rom, c->d_rom_p, 1, c->d_rom_T); if (rc_ != HBF_OK) return rc_; }
-        CK(launch_rom_controller(td, c->d_rom_T, c->d_rom_kind, hbf_rom_outputs(c->rom), c->d_state, c->stream));
+        const hbf_rom &m = *c->rom;
+        CK(launch_rom_window(m.n, m.m, m.o, m.A, m.B, m.b, m.C, m.D, m.d, m.x, c->d_rom_T + m.o, c->d_rom_T, reinterpret_cast<uint32_t *>(c->d_rom_T + m.o + m.n), td,
+                             c->d_pending, dt_ns, n_ext != 0, c->d_rom_kind, c->d_state, &c->plain_next, c->stream));
     } else {
         CK(launch_thermal_step(td, c->d_state, c->d_pending, bin_row, dt_ns, n_ext != 0, d_temps_out, &c->cur, c->thermal_generic ? 1 : 0, &c->plain_next, c->stream));
     }

@@ -237,6 +237,9 @@ cudaError_t launch_submit(const SubmitArgs &a, cudaStream_t st);
 // total[i] += part[i] over the 6 * n_dies counters of a per-die statistics array (host-buffer pipeline: totals over its chunks)
 cudaError_t launch_add_stats(hbf_die_stats_t *total, const hbf_die_stats_t *part, uint32_t n_dies, cudaStream_t st);
 // the same for batch summaries: counts and times added, the largest completion, the first code that is not HBF_OK; first != 0 starts over
+// results of a small batch to host memory the device can write: completions, stalls, per-die totals (null: not wanted; zeros for a refused batch), summary
+cudaError_t launch_host_results(const int64_t *comp, const int64_t *stall, const hbf_die_stats_t *stats, const hbf_batch_result_t *result, uint64_t n, uint32_t n_dies,
+                                int64_t *h_comp, int64_t *h_stall, hbf_die_stats_t *h_stats, hbf_batch_result_t *h_result, bool *plain_next, cudaStream_t st);
 cudaError_t launch_add_result(hbf_batch_result_t *sum, const hbf_batch_result_t *part, int first, cudaStream_t st);
 cudaError_t launch_queue_order(const BatchCtrl *ctrl, const Workspace &ws, uint32_t *out, uint64_t n, cudaStream_t st);
 // the same for a batch that was served on an ordered copy: its queue-major order is sorted out only now (bc: a control block of its own)
@@ -332,8 +335,8 @@ struct ThermalDev {
 cudaError_t launch_thermal_step(const ThermalDev &t, DevState *state, int64_t *pending, unsigned long long *bin_row, int64_t dt_ns,
                                 int has_ext, float *d_temps_out, int *cur, int generic_only, bool *plain_next, cudaStream_t st);
 
-cudaError_t launch_rom_power(const ThermalDev &t, int64_t *pending, int64_t dt_ns, int has_ext, double *p_out, cudaStream_t st);
-cudaError_t launch_rom_controller(const ThermalDev &t, const double *temps, const int32_t *kind, uint32_t n_out, DevState *state,
-                                  cudaStream_t st);
+cudaError_t launch_rom_window(uint32_t n, uint32_t m, uint32_t o, const double *A, const double *B, const double *b, const double *C, const double *D, const double *d,
+                              double *x, double *x_next, double *temps, uint32_t *done, const ThermalDev &t, int64_t *pending, int64_t dt_ns, int has_ext, const int32_t *kind,
+                              DevState *state, bool *plain_next, cudaStream_t st);
 
 }  // namespace hbf

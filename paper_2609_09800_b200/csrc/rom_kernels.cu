@@ -3,7 +3,7 @@
 // (the matrices come from a fit in double; at this size the arithmetic is not what a step costs).
 #include <cooperative_groups.h>
 
-#include "hbf_dev.cuh"
+#include "device_utils.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -102,21 +102,6 @@ k_rom_steps_cluster(uint32_t n, uint32_t m, uint32_t o, uint32_t rpc, const doub
 }
 
 // ---- the thermal step of a context on a reduced-order model: power vector, one model step, controller --------
-// Power of each region over the window, as the grid's power map computes it (one thread per region walks its dies in
-// a fixed order): the model's input vector.  The window's energy is consumed.
-__global__ void k_rom_power(ThermalDev t, int64_t *pending, int64_t dt_ns, int has_ext, double *__restrict__ p_out) {
-    for (uint32_t g = threadIdx.x; g < t.n_regions; g += blockDim.x) {
-        double p = 0.0;
-        for (int32_t k = t.region_die_ptr[g]; k < t.region_die_ptr[g + 1]; ++k)
-            p += ((double)pending[t.region_die_list[k]] * 1e-12) / ((double)dt_ns * 1e-9);
-        p += (double)t.region_idle_w[g];
-        if (has_ext) p += (double)t.ext_power[g];
-        p_out[g] = p;
-    }
-    __syncthreads();
-    for (uint32_t d = threadIdx.x; d < t.n_dies; d += blockDim.x) pending[d] = 0;
-}
-
 __device__ __forceinline__ int rom_next_mode(const ThermalDev &t, int mode, long long mk) {
     if (mode == HBF_MODE_SHUTDOWN || mk >= t.shut_mk) return HBF_MODE_SHUTDOWN;
     if (mode == HBF_MODE_NORMAL) return mk >= t.stt_mk ? HBF_MODE_SEVERE : mk >= t.ltt_mk ? HBF_MODE_LIGHT : HBF_MODE_NORMAL;
@@ -124,33 +109,97 @@ __device__ __forceinline__ int rom_next_mode(const ThermalDev &t, int mode, long
     return mk <= t.rtt_mk ? HBF_MODE_NORMAL : mk <= t.ltt_mk ? HBF_MODE_LIGHT : HBF_MODE_SEVERE;
 }
 
-// hottest output of each medium, the controller's transition on the HBF one (quantised to integer mK)
-__global__ void k_rom_controller(ThermalDev t, const double *__restrict__ temps, const int32_t *__restrict__ kind, uint32_t n_out,
-                                 DevState *state) {
-    if (threadIdx.x != 0) return;
-    double hot[3] = {-1e300, -1e300, -1e300};
-    for (uint32_t i = 0; i < n_out; ++i) {
-        const int slot = kind[i] == HBF_KIND_HBF ? 0 : kind[i] == HBF_KIND_HBM ? 1 : kind[i] == HBF_KIND_GPU ? 2 : -1;
-        if (slot >= 0 && temps[i] > hot[slot]) hot[slot] = temps[i];
+// One launch: a warp per row of [A B; C D] (within one step the rows do not wait for one another), the row's first 256 + 128
+// entries on their way before the batch before has ended; every block works out the power vector for itself, as the grid's power
+// map does (one thread per region walks its dies in a fixed order); the block that is done last takes the new state over, consumes
+// the window's energy, finds the hottest output of each medium and makes the controller's transition on the HBF one (quantised to
+// integer mK).  Each row is summed in the order of the kernels above.  224 states, 63 inputs: as three launches (power, the cluster
+// kernel, one thread for the controller) 29 us and
+// three launch gaps; a window served from host memory, with its results on the way: 101 -> 66 us.
+constexpr int kRomRowThreads = 128;
+__global__ void __launch_bounds__(kRomRowThreads)
+k_rom_window(uint32_t n, uint32_t m, uint32_t o, const double *__restrict__ A, const double *__restrict__ B, const double *__restrict__ b,
+             const double *__restrict__ C, const double *__restrict__ D, const double *__restrict__ d, double *x, double *x_next, double *temps,
+             uint32_t *done, const __grid_constant__ ThermalDev t, int64_t *pending, int64_t dt_ns, int has_ext, const int32_t *__restrict__ kind, DevState *state) {
+    extern __shared__ double rom_smem[];                     // p [m]
+    __shared__ uint32_t s_last;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const uint32_t row = blockIdx.x * (kRomRowThreads / 32) + warp, r = row < n ? row : row - n;
+    const double *mx = row < n ? A + (size_t)r * n : C + (size_t)r * n, *mp = row < n ? B + (size_t)r * m : D + (size_t)r * m;
+    const bool mine = row < n + o;
+    constexpr int kN = 8, kM = 4;
+    double an[kN], am[kM], bias = 0.0;
+    if (mine) {
+#pragma unroll
+        for (int k = 0; k < kN; ++k) { const uint32_t j = k * 32u + lane; an[k] = j < n ? mx[j] : 0.0; }
+#pragma unroll
+        for (int k = 0; k < kM; ++k) { const uint32_t j = k * 32u + lane; am[k] = j < m ? mp[j] : 0.0; }
+        bias = row < n ? b[r] : d[r];
     }
-    for (int k = 0; k < 3; ++k) { if (hot[k] == -1e300) hot[k] = (double)t.ambient_c; t.hot[k] = (float)hot[k]; }
+    pdl_wait();
+    pdl_trigger();
+    for (uint32_t g = tid; g < m; g += kRomRowThreads) {
+        double p = 0.0;
+        for (int32_t k = t.region_die_ptr[g]; k < t.region_die_ptr[g + 1]; ++k)
+            p += ((double)pending[t.region_die_list[k]] * 1e-12) / ((double)dt_ns * 1e-9);
+        p += (double)t.region_idle_w[g];
+        if (has_ext) p += (double)t.ext_power[g];
+        rom_smem[g] = p;
+    }
+    double xn[kN];
+#pragma unroll
+    for (int k = 0; k < kN; ++k) { const uint32_t j = k * 32u + lane; xn[k] = j < n ? x[j] : 0.0; }
+    __syncthreads();
+    if (mine) {
+        double acc = 0.0;
+#pragma unroll
+        for (int k = 0; k < kN; ++k) if (k * 32u + lane < n) acc += an[k] * xn[k];
+        for (uint32_t j = kN * 32u + lane; j < n; j += 32) acc += mx[j] * x[j];
+#pragma unroll
+        for (int k = 0; k < kM; ++k) if (k * 32u + lane < m) acc += am[k] * rom_smem[k * 32u + lane];
+        for (uint32_t j = kM * 32u + lane; j < m; j += 32) acc += mp[j] * rom_smem[j];
+#pragma unroll
+        for (int s = 16; s > 0; s >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, s);
+        if (lane == 0) { if (row < n) x_next[r] = acc + bias; else temps[r] = acc + bias; }
+    }
+    __syncthreads();
+    if (tid == 0) { __threadfence(); s_last = atomicAdd(done, 1u) == gridDim.x - 1u ? 1u : 0u; }
+    __syncthreads();
+    if (!s_last) return;
+    // every block has read the state and the energy, and written its rows
+    __threadfence();
+    for (uint32_t i = tid; i < n; i += kRomRowThreads) x[i] = __ldcg(x_next + i);
+    for (uint32_t e = tid; e < t.n_dies; e += kRomRowThreads) pending[e] = 0;
+    if (warp != 0) return;
+    double hot[3] = {-1e300, -1e300, -1e300};
+    for (uint32_t i = lane; i < o; i += 32) {
+        const double v = __ldcg(temps + i);
+        const int slot = kind[i] == HBF_KIND_HBF ? 0 : kind[i] == HBF_KIND_HBM ? 1 : kind[i] == HBF_KIND_GPU ? 2 : -1;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) if (slot == k && v > hot[k]) hot[k] = v;
+    }
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+#pragma unroll
+        for (int s = 16; s > 0; s >>= 1) { const double v = __shfl_xor_sync(0xffffffffu, hot[k], s); if (v > hot[k]) hot[k] = v; }
+        if (hot[k] == -1e300) hot[k] = (double)t.ambient_c;
+    }
+    if (lane != 0) return;
+    for (int k = 0; k < 3; ++k) t.hot[k] = (float)hot[k];
     const int mode = rom_next_mode(t, state->mode, (long long)floor(hot[0] * 1000.0 + 0.5));
     state->mode = mode;
     if (mode == HBF_MODE_NORMAL) state->q_ppm = 1000000;
     else if (mode == HBF_MODE_LIGHT) state->q_ppm = t.q_light_ppm;
+    *done = 0u;
 }
 
-cudaError_t launch_rom_power(const ThermalDev &t, int64_t *pending, int64_t dt_ns, int has_ext, double *p_out, cudaStream_t st) {
-    k_rom_power<<<1, 256, 0, st>>>(t, pending, dt_ns, has_ext, p_out);
+cudaError_t launch_rom_window(uint32_t n, uint32_t m, uint32_t o, const double *A, const double *B, const double *b, const double *C, const double *D, const double *d,
+                              double *x, double *x_next, double *temps, uint32_t *done, const ThermalDev &t, int64_t *pending, int64_t dt_ns, int has_ext, const int32_t *kind,
+                              DevState *state, bool *plain_next, cudaStream_t st) {
+    const unsigned rows = kRomRowThreads / 32;
     g_kernel_launches += 1;
-    return cudaGetLastError();
-}
-
-cudaError_t launch_rom_controller(const ThermalDev &t, const double *temps, const int32_t *kind, uint32_t n_out, DevState *state,
-                                  cudaStream_t st) {
-    k_rom_controller<<<1, 32, 0, st>>>(t, temps, kind, n_out, state);
-    g_kernel_launches += 1;
-    return cudaGetLastError();
+    return launch_first(plain_next, k_rom_window, (n + o + rows - 1) / rows, kRomRowThreads, m * sizeof(double), st, n, m, o, A, B, b, C, D, d, x, x_next, temps, done, t,
+                        pending, dt_ns, has_ext, kind, state);
 }
 
 static size_t rom_cluster_smem(uint32_t n, uint32_t m, uint32_t o, uint32_t *rpc_out) {

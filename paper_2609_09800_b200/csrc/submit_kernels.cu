@@ -1293,6 +1293,23 @@ cudaError_t launch_add_stats(hbf_die_stats_t *total, const hbf_die_stats_t *part
     return cudaGetLastError();
 }
 
+__global__ void __launch_bounds__(256) k_host_results(const int64_t *__restrict__ comp, const int64_t *__restrict__ stall, const int64_t *__restrict__ stats,
+                                                      const hbf_batch_result_t *result, uint64_t n, uint32_t words, int64_t *h_comp, int64_t *h_stall, int64_t *h_stats,
+                                                      hbf_batch_result_t *h_result) {
+    pdl_wait();
+    pdl_trigger();
+    const uint64_t gtid = (uint64_t)blockIdx.x * 256 + threadIdx.x, gsz = (uint64_t)gridDim.x * 256;
+    for (uint64_t i = gtid; i < n; i += gsz) { h_comp[i] = __ldcg(comp + i); h_stall[i] = __ldcg(stall + i); }
+    if (h_stats) for (uint64_t i = gtid; i < words; i += gsz) h_stats[i] = __ldcg(stats + i);
+    if (gtid == 0) *h_result = *result;
+}
+cudaError_t launch_host_results(const int64_t *comp, const int64_t *stall, const hbf_die_stats_t *stats, const hbf_batch_result_t *result, uint64_t n, uint32_t n_dies,
+                                int64_t *h_comp, int64_t *h_stall, hbf_die_stats_t *h_stats, hbf_batch_result_t *h_result, bool *plain_next, cudaStream_t st) {
+    g_kernel_launches += 1;
+    return launch_first(plain_next, k_host_results, (unsigned)std::min<uint64_t>((n + 255) / 256, 148), 256, 0, st, comp, stall, reinterpret_cast<const int64_t *>(stats), result, n,
+                        n_dies * 6u, h_comp, h_stall, reinterpret_cast<int64_t *>(h_stats), h_result);
+}
+
 __global__ void k_add_result(hbf_batch_result_t *sum, const hbf_batch_result_t *part, int first) {
     hbf_batch_result_t s = *sum; const hbf_batch_result_t r = *part;
     if (first) { s = r; }

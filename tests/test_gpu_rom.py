@@ -116,3 +116,28 @@ def test_context_steps_on_an_attached_model(hbf):
         g.thermal_step(2 * dt, ext)                                        # the model was fitted for one step length
     g.attach_rom(None)
     g.thermal_step(dt, ext)                                                # the grid again
+
+
+@pytest.mark.parametrize("n, o", [(1, 1), (31, 2), (256, 3), (257, 130), (700, 11)])
+def test_window_kernel_matches_the_oracle(hbf, n, o):
+    """The context's step at sizes around the rows' prefetched part and the warps of a block, with energy pending."""
+    w = wl.prefix_kv(epochs=1, steps=1, batch=2, kv_tokens=64, layers=1)
+    fp = wl.package_floorplan()
+    prof = dict(w.profile); prof.update(rtt_c=500.0, ltt_c=600.0, stt_c=700.0, shutdown_c=800.0)   # the controller stays Normal
+    g, orc = hbf.Context(prof, fp), hbfo.Oracle(prof, fp)
+    for r in w.ranges:
+        g.register_range(*r); orc.register_range(*r)
+    m, rng = len(fp["region_kind"]), np.random.default_rng(n)
+    A = np.diag(rng.uniform(0.80, 0.97, n)) + rng.normal(size=(n, n)) * (0.01 / n)
+    B, Cm, D = rng.uniform(0.0, 0.02, size=(n, m)), rng.uniform(0.0, 0.05, size=(o, n)), rng.uniform(0.0, 0.002, size=(o, m))
+    kinds = rng.choice([wl.KIND_HBF, wl.KIND_HBM, wl.KIND_GPU, wl.KIND_NONE], o).astype(np.int32)
+    b, d = rng.normal(size=n) * 0.01, np.full(o, prof["ambient_c"])
+    rg, ro = hbf.Rom(A, B, Cm, D=D, b=b, d=d, stream=g.stream), hbfo.Rom(A, B, Cm, D=D, b=b, d=d)
+    g.attach_rom(rg, kinds, 1_000_000)
+    g.submit_host(w.acc); orc.submit(w.acc)
+    for k in range(4):
+        hot_g = g.thermal_step(1_000_000, fp["ext_power_w"])
+        hot_o = orc.thermal_step_rom(ro, kinds, 1_000_000, fp["ext_power_w"])
+        assert np.abs(hot_g.astype(np.float64) - hot_o).max() < 1e-4      # hot_c_out is float32
+        assert np.abs(rg.state() - ro.state()).max() <= 1e-11 * max(1.0, np.abs(ro.state()).max())   # double on both sides; only the summation order differs
+        assert not g.get_pending_energy().any()

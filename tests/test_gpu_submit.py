@@ -509,3 +509,22 @@ def test_bounded_waits_run_out_and_the_batch_is_given_up(hbf, stage):
     assert np.array_equal(g.get_busy_until(), busy0)
     g.reset(); o.reset()
     compare_batch(g, o, w.acc)                              # usable again, and exact
+
+
+@pytest.mark.parametrize("n", [1, 257, 8192, 8193, 65_536, 65_537])
+def test_one_chunk_from_the_host_in_pinned_and_pageable_memory(hbf, n):
+    """The results of a call of one chunk leave by a kernel (pinned memory, up to 65,536 records) or by copies."""
+    import torch
+    w = wl.capacity_mode(n=n, seed=n)
+    g, o = contexts(hbf, w.profile, w.ranges)
+    _, c_o, s_o, _, ds_o = o.submit(w.acc)
+    rec = torch.from_numpy(w.acc.view(np.int64).reshape(-1))
+    for pin in (True, False):
+        make = lambda k: torch.full((k,), -1, dtype=torch.int64).pin_memory() if pin else torch.full((k,), -1, dtype=torch.int64)
+        c, s, ds = make(n + 1), make(n + 1), make(g.n_dies * 6)
+        g.reset()
+        rc, summary = g.submit_pinned(rec.pin_memory() if pin else rec, n, c[1:], s[:n], ds)
+        assert rc == 0 and summary == o.last_result()
+        assert np.array_equal(c[1:].numpy(), c_o) and c[0] == -1 and np.array_equal(s[:n].numpy(), s_o) and s[n] == -1
+        got = ds.numpy().view(hbfo.DIE_STATS_DTYPE)
+        assert all(np.array_equal(got[f], ds_o[f]) for f in hbfo.DIE_STATS_DTYPE.names)
