@@ -193,6 +193,9 @@ __device__ __forceinline__ void row_wait2(int id, int64_t m, long long s8, const
 // Tried and not kept: the records through shared memory by a bulk copy per turn (L1 pipe 70 -> 55 % busy, but 1,650 us with an L2
 // prefetch ahead of it and 1,710 without, against 1,587 for the submit alone); both rows of a turn updated side by side, with
 // queues shared across the rows composed in registers (shorter chain, 8 % more instructions: 1,626); four rows per turn (the same).
+// Queue states lie by slot (queue_slot), and tiles that have to be served again take this form too: 24 M records of the prefix
+// stream, whose rows walk along the channels, 359 -> 234 us and 306 -> 175 (the L1's data pipe was 84 % busy, 66 bank conflicts per
+// row); with everything around it 790 -> 503.  (In the 64-bit form the slots cost mixed batches 4 %: it keeps the queue's number.)
 // What the form cannot hold (a time 2^31 ns or more past the tile's first, by a gap in the stream or by a backlog) is
 // only noticed, in bits that are OR-ed along; such a tile is then served again in the 64-bit form.
 // Queue state (16 bytes): busy-until, service time in this tile, read granules, reads << 4 | head entries written.
@@ -209,7 +212,8 @@ __device__ __forceinline__ void row_wait_n(int id, uint32_t m, uint32_t s, const
                  "r"(m2), "r"(s2), "l"(pq2), "r"(gn2), "r"((int)last2) : "memory");
 }
 
-template <bool DEBT, bool PAGED>
+// RESERVE = true: the results only.  Everything per queue goes by the queue's slot.
+template <bool RESERVE, bool DEBT, bool PAGED>
 __device__ __forceinline__ NarrowSums serve_narrow(const FastGeom &geom, const ModelParams &mp, const ModelParams &mp_arg, const hbf_access_t *acc_t, const uint32_t tile_begin,
                                                    const uint32_t tile_len, const int64_t T0, uint4 *qst, uint8_t *warp_tag, uint8_t *status_t,
                                                    uint16_t *qid_t, const uint32_t qid_stride, int64_t *completion_t, int64_t *stall_t,
@@ -237,7 +241,7 @@ __device__ __forceinline__ NarrowSums serve_narrow(const FastGeom &geom, const M
             if (j < tile_len) {
                 const uint64_t *rec = reinterpret_cast<const uint64_t *>(acc_t + j);
                 nx_addr[u] = __ldcs(rec); nx_issue[u] = __ldcs(rec + 1); nx_bf[u] = __ldcs(rec + 2);   // read once: streaming loads
-                nx_prev[u] = j > 0u ? __ldg(reinterpret_cast<const uint32_t *>(rec - 2)) : (uint32_t)T0;   // (the tile's first record was compared before)
+                if (!RESERVE) nx_prev[u] = j > 0u ? __ldg(reinterpret_cast<const uint32_t *>(rec - 2)) : (uint32_t)T0;   // (the tile's first record was compared before)
             }
         }
     };
@@ -270,13 +274,13 @@ __device__ __forceinline__ NarrowSums serve_narrow(const FastGeom &geom, const M
             const uint64_t dt = (uint64_t)(issue[u] - T0), rel = addr[u] - geom.base, off = addr[u] + geom.nw_delta;
             ri[u] = (uint32_t)dt;
             ready[u] = valid[u] && rel <= geom.nw_lim && bytes - 1u < geom.nw_bytes && flags - geom.nw_flag_lo < geom.nw_flag_n;
-            if (valid[u]) { b_hi |= (uint32_t)(dt >> 32); b_time |= ri[u]; b_sort |= (uint32_t)issue[u] - prev[u]; }
+            if (valid[u]) { b_hi |= (uint32_t)(dt >> 32); b_time |= ri[u]; if (!RESERVE) b_sort |= (uint32_t)issue[u] - prev[u]; }
             q[u] = 0; S[u] = 0; M[u] = 0; xo[u] = 0; gn[u] = 0;
             uint32_t st = HBF_ST_READY;
             const bool common = ready[u];
             if (common) {
                 const uint32_t w = (uint32_t)(off >> geom.stripe_shift), in_page = (uint32_t)off & geom.page_mask;
-                q[u] = (w & geom.ch_mask) * geom.nw_chmul + ((w >> geom.ch_shift) & geom.die_mask) * geom.planes_q + ((w >> geom.chdie_shift) & geom.plane_mask_q);
+                q[u] = w & geom.nw_slot_mask;
                 const uint32_t npages = (in_page + bytes + geom.page_mask) >> geom.page_shift;
                 if (flags == 0u) {
                     const uint32_t g = (bytes + ((1u << geom.gran_shift_read) - 1u)) >> geom.gran_shift_read;
@@ -305,14 +309,16 @@ __device__ __forceinline__ NarrowSums serve_narrow(const FastGeom &geom, const M
                     }
                     xo[u] = xf | 0x80000000u;
                     M[u] = ri[u] + xf + S[u];
-                    const uint32_t die = geom.planes_q == 1u ? q[u] : q[u] >> mp_arg.plane_shift, lo = g << geom.gran_shift_prog;
-                    atomicAdd(&st_np[die], PAGED ? npages : 1u);
-                    const uint32_t old = atomicAdd(&st_bp_lo[die], lo);
-                    if (old + lo < old) atomicAdd(&st_bp_hi[die], 1u);
+                    if (!RESERVE) {
+                        const uint32_t die = slot_die(geom, q[u]), lo = g << geom.gran_shift_prog;
+                        atomicAdd(&st_np[die], PAGED ? npages : 1u);
+                        const uint32_t old = atomicAdd(&st_bp_lo[die], lo);
+                        if (old + lo < old) atomicAdd(&st_bp_hi[die], 1u);
+                    }
                 }
                 if (DEBT && tile_begin + i[u] < claim_limit) {
                     S[u] += quantum_ns; M[u] += quantum_ns;
-                    atomicAdd(&st_claims[geom.planes_q == 1u ? q[u] : q[u] >> mp_arg.plane_shift], 1u);
+                    if (!RESERVE) atomicAdd(&st_claims[slot_die(geom, q[u])], 1u);
                 }
             } else if (valid[u]) {                           // near the range's end, large, or not modeled
                 unsigned lng = 0;
@@ -320,15 +326,17 @@ __device__ __forceinline__ NarrowSums serve_narrow(const FastGeom &geom, const M
                 if (PAGED && v.st == HBF_ST_READY) paged_terms(mp, off, bytes, 1000000, Div64{}, lng, (int)kNwServeBits - 1, v);
                 st = (uint32_t)v.st;
                 if (v.st == HBF_ST_READY) {
-                    ready[u] = true; q[u] = v.queue;
+                    ready[u] = true; q[u] = queue_slot(geom, v.queue);
                     if (lng || ((uint64_t)v.s >> (kNwServeBits - 1)) || (v.xfer >> 30)) b_time |= 0x80000000u;
                     S[u] = (uint32_t)v.s; xo[u] = v.xfer | (v.op << 31);
-                    const uint32_t lo = (uint32_t)v.cb, hi = (uint32_t)((uint64_t)v.cb >> 32);
-                    uint32_t *plo = v.op ? st_bp_lo : st_br_lo, *phi = v.op ? st_bp_hi : st_br_hi;
-                    atomicAdd(v.op ? &st_np[v.die] : &st_nr[v.die], v.parts);
-                    const uint32_t old = atomicAdd(&plo[v.die], lo), carry = hi + ((old + lo) < old ? 1u : 0u);
-                    if (carry) atomicAdd(&phi[v.die], carry);
-                    if (DEBT && tile_begin + i[u] < claim_limit) { S[u] += quantum_ns; atomicAdd(&st_claims[v.die], 1u); }
+                    if (!RESERVE) {
+                        const uint32_t lo = (uint32_t)v.cb, hi = (uint32_t)((uint64_t)v.cb >> 32);
+                        uint32_t *plo = v.op ? st_bp_lo : st_br_lo, *phi = v.op ? st_bp_hi : st_br_hi;
+                        atomicAdd(v.op ? &st_np[v.die] : &st_nr[v.die], v.parts);
+                        const uint32_t old = atomicAdd(&plo[v.die], lo), carry = hi + ((old + lo) < old ? 1u : 0u);
+                        if (carry) atomicAdd(&phi[v.die], carry);
+                    }
+                    if (DEBT && tile_begin + i[u] < claim_limit) { S[u] += quantum_ns; if (!RESERVE) atomicAdd(&st_claims[v.die], 1u); }
                     M[u] = ri[u] + (v.op ? v.xfer : 0u) + S[u];
                 } else if (v.st == HBF_ST_NATIVE) {
                     r.native += 1u;
@@ -336,20 +344,20 @@ __device__ __forceinline__ NarrowSums serve_narrow(const FastGeom &geom, const M
                     r.fault += 1u;
                 }
             }
-            if (DEBT && ready[u] && flags == 0u) {           // read disturb: the read's pages, on the block of its first page
+            if (DEBT && !RESERVE && ready[u] && flags == 0u) {           // read disturb: the read's pages, on the block of its first page
                 const uint32_t npages = (uint32_t)(((uint64_t)((uint32_t)off & geom.page_mask) + bytes + geom.page_mask) >> geom.page_shift);
                 if (ret.pow2 != 0u) {
                     const uint32_t row = (uint32_t)((off >> geom.stripe_shift) >> ret_row_shift);
                     const uint32_t in_stripe = ((uint32_t)off & ((1u << geom.stripe_shift) - 1u)) >> geom.page_shift;
                     const uint32_t blk = ((row << mp_arg.pages_per_stripe_shift) + in_stripe) >> ret.ppb_shift;
                     const uint32_t pl = (uint32_t)(off >> (geom.stripe_shift + geom.chdie_shift)) & geom.plane_mask;
-                    const uint32_t die = geom.planes_q == 1u ? q[u] : q[u] >> mp_arg.plane_shift;
+                    const uint32_t die = slot_die(geom, q[u]);
                     atomicAdd(&ret.disturb[((die << mp_arg.plane_shift) + pl) * ret.bpp + (blk & (ret.bpp - 1u))], npages);
                 } else {
                     atomicAdd(&ret.disturb[ret_block_of(mp, ret, off)], npages);
                 }
             }
-            if (status_t && valid[u]) status_t[i[u]] = (uint8_t)st;
+            if (!RESERVE && status_t && valid[u]) status_t[i[u]] = (uint8_t)st;
         }
         // ---- which lanes of a row hold the same queue (see the 64-bit form)
         uint8_t *tag_at[K];
@@ -359,12 +367,12 @@ __device__ __forceinline__ NarrowSums serve_narrow(const FastGeom &geom, const M
         __syncwarp();
 #pragma unroll
         for (int u = 0; u < K; ++u) tagged[u] = *reinterpret_cast<volatile uint8_t *>(tag_at[u]);
-        if (turn * (uint32_t)(K * 32) < qid_stride) {
+        if (!RESERVE && turn * (uint32_t)(K * 32) < qid_stride) {
 #pragma unroll
             for (int u = 0; u < K; ++u)
-                if (valid[u]) qid_t[i[u]] = ready[u] ? (uint16_t)q[u] : (uint16_t)kInMaxQueues;
+                if (valid[u]) qid_t[i[u]] = ready[u] ? (uint16_t)slot_queue(geom, q[u]) : (uint16_t)kInMaxQueues;
         }
-        const bool heads_on = *reinterpret_cast<volatile uint32_t *>(s_heads_full) < R;
+        const bool heads_on = RESERVE ? false : *reinterpret_cast<volatile uint32_t *>(s_heads_full) < R;
         auto rest_of_turn = [&](auto heads_tag) {
         constexpr bool HEADS = decltype(heads_tag)::value;
         uint32_t rank1[K], pc[K], c0[K], c1[K], m_own[K], s_own[K], B[K];
@@ -432,7 +440,7 @@ __device__ __forceinline__ NarrowSums serve_narrow(const FastGeom &geom, const M
                     const uint32_t ci = c0[u] + rank1[u] - 1u;
                     if (ci < head_depth) {
                         InHead h; h.m = T0 + (int64_t)m_own[u]; h.s = (int64_t)s_own[u]; h.xo = xo[u]; h.idx = tile_begin + i[u];
-                        in_head[head_slot(tile, R, q[u], ci)] = h;
+                        in_head[head_slot(tile, R, slot_queue(geom, q[u]), ci)] = h;
                     }
                     if (last[u] && c1[u] != c0[u] && c1[u] == head_depth) atomicAdd(s_heads_full, 1u);
                 }
@@ -441,7 +449,8 @@ __device__ __forceinline__ NarrowSums serve_narrow(const FastGeom &geom, const M
             }
         }
         };
-        if (heads_on) rest_of_turn(std::true_type{}); else rest_of_turn(std::false_type{});
+        if constexpr (!RESERVE) { if (heads_on) rest_of_turn(std::true_type{}); else rest_of_turn(std::false_type{}); }
+        else { (void)heads_on; rest_of_turn(std::false_type{}); }
       };
       if ((turn * K + K) * 32u <= tile_len) whole_turn(std::true_type{}); else whole_turn(std::false_type{});
     }
@@ -547,7 +556,7 @@ k_inorder_serve(const hbf_access_t *__restrict__ acc, uint64_t n, const __grid_c
     long long sum_stall = 0, max_c = INT64_MIN;
     long long t_native = 0, t_ready = 0, t_fault = 0;        // this thread's share of the tile's counts
     bool narrow_done = false, again = false;
-    if constexpr (!RESERVE) {
+    {
         // The 32-bit form serves the tile when the configuration allows it, the tile's times lie within 2^31 ns and its read
         // granules sum below 2^32; should it turn out not to fit after all (a backlog), the 64-bit form below serves the tile again.
         int64_t T0 = 0, T1 = -1;
@@ -556,39 +565,43 @@ k_inorder_serve(const hbf_access_t *__restrict__ acc, uint64_t n, const __grid_c
             (uint64_t)tile_len * geom.nw_gmax < (1ull << 32) && (uint64_t)quantum_ns < (1ull << (kNwServeBits - 1))) {
             uint4 *q4 = reinterpret_cast<uint4 *>(qst);
             unsigned over = 0;
-            for (uint32_t d = tid; d < n_dies * 7u; d += kInThreads) st_br_lo[d] = 0u;
+            if (!RESERVE) for (uint32_t d = tid; d < n_dies * 7u; d += kInThreads) st_br_lo[d] = 0u;
             for (uint32_t q = tid; q < kInMaxQueues; q += kInThreads) {
                 uint4 v = make_uint4(0u, 0u, 0u, 0u);
-                if (tile == 0u && q < R) {                   // the first tile knows its entering state: it is served exactly
-                    const int64_t b = busy[q] - T0;
+                if ((RESERVE || tile == 0u) && q < R) {      // the first tile knows its entering state: it is served exactly
+                    const int64_t b = (RESERVE ? in_bin[(uint64_t)tile * R + q] : busy[q]) - T0;
                     v.x = b > 0 ? (uint32_t)b : 0u;
-                    if (b >= (1ll << 31)) over = 1u;
+                    if (b >= (RESERVE ? 1ll << 30 : 1ll << 31)) over = 1u;
                 }
-                q4[q] = v;
+                q4[q < R ? queue_slot(geom, q) : q] = v;
             }
-            __syncthreads();
-            const NarrowSums nw = serve_narrow<DEBT, PAGED>(geom, mp, mp_arg, acc_t, (uint32_t)tile_begin, tile_len, T0, q4, warp_tag, status_t, qid_t, qid_stride,
+            // (a backlog that reaches into the tile, from claims mostly, grows while the tile is served: not even tried then)
+            const bool try_narrow = __syncthreads_or((int)(RESERVE && over)) == 0;
+            NarrowSums nw{};
+            if (try_narrow) nw = serve_narrow<RESERVE, DEBT, PAGED>(geom, mp, mp_arg, acc_t, (uint32_t)tile_begin, tile_len, T0, q4, warp_tag, status_t, qid_t, qid_stride,
                                                      completion_t, stall_t, in_head, tile, R, head_depth, &s_heads_full, st_br_lo, n_dies, claim_limit,
                                                      (uint32_t)quantum_ns, ret, ret_row_shift);
             if (__syncthreads_or((int)(over | nw.over)) == 0) {
                 narrow_done = true;
-                c_unsorted |= nw.unsorted;
-                if (tid == 0 && tile_begin > 0 && acc_t[-1].issue_ns > T0) c_unsorted = 1u;
                 sum_stall = nw.stall;
                 if (nw.max_done) max_c = T0 + (int64_t)(uint64_t)nw.max_done;      // (a modeled access ends after its tile's first issue time)
+                if constexpr (!RESERVE) {
+                c_unsorted |= nw.unsorted;
+                if (tid == 0 && tile_begin > 0 && acc_t[-1].issue_ns > T0) c_unsorted = 1u;
                 t_native = nw.native; t_fault = nw.fault; t_ready = (tid == 0 ? (long long)tile_len : 0ll) - t_native - t_fault;
                 longlong2 *out = reinterpret_cast<longlong2 *>(in_agg) + (uint64_t)tile * R;
                 for (uint32_t q = tid; q < R; q += kInThreads) {
-                    const uint4 v = q4[q];
+                    const uint4 v = q4[queue_slot(geom, q)];
                     out[q] = make_longlong2((long long)(uint64_t)v.y, v.y ? T0 + (int64_t)(uint64_t)v.x : kNegInf);   // (no service time: no access)
                     in_headcnt[(uint64_t)tile * R + q] = (uint8_t)(v.w & 15u);
                 }
                 for (uint32_t d = tid; d < n_dies; d += kInThreads) {              // a die's reads: the sums its queues carry
                     unsigned long long g = 0, cnt = 0;
-                    for (uint32_t p = 0; p < geom.planes_q; ++p) { const uint4 v = q4[d * geom.planes_q + p]; g += v.z; cnt += v.w >> 4; }
+                    for (uint32_t p = 0; p < geom.planes_q; ++p) { const uint4 v = q4[queue_slot(geom, d * geom.planes_q + p)]; g += v.z; cnt += v.w >> 4; }
                     unsigned long long *gd = reinterpret_cast<unsigned long long *>(stats_stage + d);
                     if (g) atomicAdd(&gd[1], g << geom.gran_shift_read);
                     if (cnt) atomicAdd(&gd[4], cnt);
+                }
                 }
             } else {
                 again = true;

@@ -73,8 +73,17 @@ struct __align__(16) FastGeom {
     uint32_t narrow, nw_bytes, nw_flag_lo, nw_flag_n;        // inline accesses: at most nw_bytes bytes, flags nw_flag_lo .. nw_flag_lo + nw_flag_n - 1
     uint32_t nw_gmax, nw_mul_read, nw_mul_prog, nw_add;      // most granules of an inline read; transfer = (granules * mul + add) / rate by
     uint32_t nw_magic, nw_shift, nw_chmul, nw_pad;           //   multiply-high; queues per channel
-    uint32_t nw_page_read, nw_page_prog, nw_page_gran, nw_pad2;   // page-granular submit: transfer of a whole page, read granules of one
+    uint32_t nw_page_read, nw_page_prog, nw_page_gran, nw_chmul_shift;   // page-granular submit: transfer of a whole page, read granules of one
+    uint32_t nw_slot_mask, nw_plane_shift, nw_pad2, nw_pad3;  // a queue's slot (see queue_slot): these low bits of the stripe unit's number; planes_q as a shift
 };
+// Where a queue's state lies in shared memory (power-of-two geometry): channel first, then die, then plane, as in the number of
+// the stripe unit.  Neighbouring stripe units, which the streams of weights and prefixes walk along, lie on neighbouring channels:
+// by queue number (channel last) their 16-byte states were dies * planes apart, all in the same four banks.
+__device__ __forceinline__ uint32_t queue_slot(const FastGeom &g, uint32_t q) {
+    return (q >> g.nw_chmul_shift) | (((q >> g.nw_plane_shift) & g.die_mask) << g.ch_shift) | ((q & g.plane_mask_q) << g.chdie_shift);
+}
+__device__ __forceinline__ uint32_t slot_die(const FastGeom &g, uint32_t s) { return (s & g.ch_mask) * g.dies + ((s >> g.ch_shift) & g.die_mask); }
+__device__ __forceinline__ uint32_t slot_queue(const FastGeom &g, uint32_t s) { return (slot_die(g, s) << g.nw_plane_shift) + ((s >> g.chdie_shift) & g.plane_mask_q); }
 // Bounds of the 32-bit form.  A service is below 2^26 ns, so that the services of a row's 32 lanes compose below 2^31; the
 // granules and the reads of an access fit 11 and 6 bits, so that a row's sums travel in one word (17 and 11 bits).
 constexpr uint32_t kNwServeBits = 26, kNwGranules = 2048, kNwPages = 32, kNwCountShift = 17;
@@ -100,7 +109,8 @@ __host__ __device__ __forceinline__ FastGeom make_fast_geom(const FastRange &f, 
     g.nw_delta = f.media_offset - f.base; g.nw_chmul = mp.dies * g.planes_q; g.nw_pad = 0;
     g.nw_flag_lo = (f.perms & 1u) ? 0u : 1u; g.nw_flag_n = (f.perms & 3u) == 3u ? 2u : 1u;
     g.nw_mul_read = 1000u << (mp.read_gran_shift & 15u); g.nw_mul_prog = 1000u << (mp.prog_gran_shift & 15u);
-    g.narrow = 0u; g.nw_bytes = g.nw_gmax = g.nw_add = g.nw_magic = g.nw_shift = 0u; g.nw_lim = 0; g.nw_page_read = g.nw_page_prog = g.nw_page_gran = g.nw_pad2 = 0u;
+    g.narrow = 0u; g.nw_bytes = g.nw_gmax = g.nw_add = g.nw_magic = g.nw_shift = 0u; g.nw_lim = 0; g.nw_page_read = g.nw_page_prog = g.nw_page_gran = g.nw_pad2 = g.nw_pad3 = 0u;
+    g.nw_plane_shift = mp.queue_level == 0u ? mp.plane_shift : 0u; g.nw_chmul_shift = mp.die_shift + g.nw_plane_shift; g.nw_slot_mask = mp.channels * mp.dies * g.planes_q - 1u;
     const uint64_t d = mp.chan_bytes_per_us, t_max = (uint64_t)(mp.t_read_ns > mp.t_prog_ns ? mp.t_read_ns : mp.t_prog_ns);
     const uint64_t quantum = (uint64_t)mp.t_read_ns + (uint64_t)mp.t_prog_ns;   // (a claimed refresh quantum is added to a service)
     if (fast_geom_ok(f, mp) && d >= 2u && d < (1ull << 30) && mp.read_gran_shift <= 15u && mp.prog_gran_shift <= 15u && mp.page_shift <= 20u &&

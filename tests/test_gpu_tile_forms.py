@@ -44,11 +44,11 @@ def stream(kind, n, rng):
 
 
 @pytest.mark.parametrize("n", [8_193, 20_001, 65_536])
-@pytest.mark.parametrize("kind", ["plain", "gap", "backlog", "edge", "native", "offset", "read only", "program only", "claims", "claims backlog"])
+@pytest.mark.parametrize("kind", ["plain", "gap", "backlog", "edge", "native", "offset", "read only", "program only", "claims", "claims backlog", "neighbours", "queue per die", "claims queue per die"])
 def test_32_bit_form_matches_the_oracle(hbf, kind, n):
     import torch
     rng = np.random.default_rng(n)
-    prof = wl.load_profile("nominal", channels=8, dies=4, planes=2, page_bytes=16384, stripe_bytes=65536)
+    prof = wl.load_profile("nominal", channels=8, dies=4, planes=2, page_bytes=16384, stripe_bytes=65536, queue_level=int("queue per die" in kind))
     perms = {"read only": 1, "program only": 2}.get(kind, 3)
     g, o = hbf.Context(prof), hbfo.Oracle(prof)
     for c in (g, o):
@@ -58,6 +58,8 @@ def test_32_bit_form_matches_the_oracle(hbf, kind, n):
                                l_ref_s=1.0, t_ref_c=40.0, ea_ev=1.04, accel=1.0, lead_threshold=0.5)
             c.retention_advance(1_000_000_000, [40.0])      # every block becomes eligible: 32,768 quanta
     acc = stream(kind.split()[-1] if "backlog" in kind else kind, n, rng)
+    if kind == "neighbours":                                # walks along the stripe units; nearly every tile is served again
+        acc["addr"] = BASE + (np.arange(n) % 4000).astype(np.uint64) * np.uint64(65536)
     if perms != 3:
         acc["flags"] = perms - 1
     for batch in range(2):                                  # the second one enters on the queues the first one left
