@@ -200,6 +200,8 @@ __device__ __forceinline__ void row_wait2(int id, int64_t m, long long s8, const
 // only noticed, in bits that are OR-ed along; such a tile is then served again in the 64-bit form.
 // Queue state (16 bytes): busy-until, service time in this tile, read granules, reads << 4 | head entries written.
 // ======================================================================================================
+// what a launch of the pass does: all of it; the results only, from known busy-until; all but the results and the head entries
+enum { kInFull = 0, kInAgain = 1, kInLight = 2 };
 struct NarrowSums { uint32_t native, fault, max_done; unsigned unsorted, over; long long stall; };
 
 __device__ __forceinline__ uint32_t nw_transfer(const FastGeom &g, uint32_t granules, uint32_t mul) {
@@ -212,14 +214,15 @@ __device__ __forceinline__ void row_wait_n(int id, uint32_t m, uint32_t s, const
                  "r"(m2), "r"(s2), "l"(pq2), "r"(gn2), "r"((int)last2) : "memory");
 }
 
-// RESERVE = true: the results only.  Everything per queue goes by the queue's slot.
-template <bool RESERVE, bool DEBT, bool PAGED>
+// MODE: see k_inorder_serve.  Everything per queue goes by the queue's slot.
+template <int MODE, bool DEBT, bool PAGED>
 __device__ __forceinline__ NarrowSums serve_narrow(const FastGeom &geom, const ModelParams &mp, const ModelParams &mp_arg, const hbf_access_t *acc_t, const uint32_t tile_begin,
                                                    const uint32_t tile_len, const int64_t T0, uint4 *qst, uint8_t *warp_tag, uint8_t *status_t,
                                                    uint16_t *qid_t, const uint32_t qid_stride, int64_t *completion_t, int64_t *stall_t,
                                                    InHead *__restrict__ in_head, const uint32_t tile, const uint32_t R, const uint32_t head_depth,
                                                    uint32_t *s_heads_full, uint32_t *st_br_lo, const uint32_t n_dies,
                                                    const uint64_t claim_limit, const uint32_t quantum_ns, const RetDev &ret, const uint32_t ret_row_shift) {
+    constexpr bool RESERVE = MODE == kInAgain, LIGHT = MODE == kInLight;
     constexpr int K = kInRows;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     uint32_t *st_br_hi = st_br_lo + n_dies, *st_bp_lo = st_br_hi + n_dies, *st_bp_hi = st_bp_lo + n_dies, *st_nr = st_bp_hi + n_dies, *st_np = st_nr + n_dies, *st_claims = st_np + n_dies;
@@ -367,12 +370,12 @@ __device__ __forceinline__ NarrowSums serve_narrow(const FastGeom &geom, const M
         __syncwarp();
 #pragma unroll
         for (int u = 0; u < K; ++u) tagged[u] = *reinterpret_cast<volatile uint8_t *>(tag_at[u]);
-        if (!RESERVE && turn * (uint32_t)(K * 32) < qid_stride) {
+        if (MODE == kInFull && turn * (uint32_t)(K * 32) < qid_stride) {
 #pragma unroll
             for (int u = 0; u < K; ++u)
                 if (valid[u]) qid_t[i[u]] = ready[u] ? (uint16_t)slot_queue(geom, q[u]) : (uint16_t)kInMaxQueues;
         }
-        const bool heads_on = RESERVE ? false : *reinterpret_cast<volatile uint32_t *>(s_heads_full) < R;
+        const bool heads_on = MODE != kInFull ? false : *reinterpret_cast<volatile uint32_t *>(s_heads_full) < R;
         auto rest_of_turn = [&](auto heads_tag) {
         constexpr bool HEADS = decltype(heads_tag)::value;
         uint32_t rank1[K], pc[K], c0[K], c1[K], m_own[K], s_own[K], B[K];
@@ -432,7 +435,8 @@ __device__ __forceinline__ NarrowSums serve_narrow(const FastGeom &geom, const M
         // ---- results
 #pragma unroll
         for (int u = 0; u < K; ++u) {
-            if (valid[u]) {
+            if (LIGHT) { if (ready[u]) b_time |= B[u]; }
+            else if (valid[u]) {
                 const uint32_t done = ready[u] ? B[u] + (uint32_t)max((int)xo[u], 0) : ri[u], waited = done - ri[u];
                 if (ready[u]) { b_time |= B[u]; r.max_done = max(r.max_done, done); }
                 r.stall += (long long)(unsigned long long)waited;
@@ -449,7 +453,7 @@ __device__ __forceinline__ NarrowSums serve_narrow(const FastGeom &geom, const M
             }
         }
         };
-        if constexpr (!RESERVE) { if (heads_on) rest_of_turn(std::true_type{}); else rest_of_turn(std::false_type{}); }
+        if constexpr (MODE == kInFull) { if (heads_on) rest_of_turn(std::true_type{}); else rest_of_turn(std::false_type{}); }
         else { (void)heads_on; rest_of_turn(std::false_type{}); }
       };
       if ((turn * K + K) * 32u <= tile_len) whole_turn(std::true_type{}); else whole_turn(std::false_type{});
@@ -462,7 +466,7 @@ __device__ __forceinline__ NarrowSums serve_narrow(const FastGeom &geom, const M
 // read and a page program, scaled like any service, Eq. 3) before its own service; the streaming pass counts the
 // claims per die.
 // PAGED = true: the page-granular submit of accesses that stay inside one stripe unit each (paged_terms).
-template <bool RESERVE, bool DEBT, bool PAGED>
+template <int MODE, bool DEBT, bool PAGED>
 __global__ void __launch_bounds__(kInThreads, kInBlocksPerSM)
 k_inorder_serve(const hbf_access_t *__restrict__ acc, uint64_t n, const __grid_constant__ InTileMap tmap, const RangeSnap *__restrict__ ranges_g,
                 const __grid_constant__ ModelParams mp_arg, const __grid_constant__ FastRange fast_arg, BatchCtrl *ctrl, uint8_t *__restrict__ status, int64_t *__restrict__ in_agg,
@@ -471,6 +475,7 @@ k_inorder_serve(const hbf_access_t *__restrict__ acc, uint64_t n, const __grid_c
                 const int64_t *__restrict__ busy, const unsigned long long *claim_limit_p, uint32_t *die_claims,
                 const __grid_constant__ RetDev ret, uint16_t *__restrict__ in_qid, uint32_t qid_stride,
                 TileBalance *bal, uint32_t bal_seq, const __grid_constant__ FastGeom geom, const uint32_t head_depth, const OrderedCopy copy) {
+    constexpr bool RESERVE = MODE == kInAgain, LIGHT = MODE == kInLight;
     extern __shared__ __align__(16) unsigned char in_smem[];
     __shared__ long long s_red[2];
     __shared__ unsigned long long s_t0;                   // when this block took its tile (0: its time is not recorded)
@@ -578,7 +583,7 @@ k_inorder_serve(const hbf_access_t *__restrict__ acc, uint64_t n, const __grid_c
             // (a backlog that reaches into the tile, from claims mostly, grows while the tile is served: not even tried then)
             const bool try_narrow = __syncthreads_or((int)(RESERVE && over)) == 0;
             NarrowSums nw{};
-            if (try_narrow) nw = serve_narrow<RESERVE, DEBT, PAGED>(geom, mp, mp_arg, acc_t, (uint32_t)tile_begin, tile_len, T0, q4, warp_tag, status_t, qid_t, qid_stride,
+            if (try_narrow) nw = serve_narrow<MODE, DEBT, PAGED>(geom, mp, mp_arg, acc_t, (uint32_t)tile_begin, tile_len, T0, q4, warp_tag, status_t, qid_t, qid_stride,
                                                      completion_t, stall_t, in_head, tile, R, head_depth, &s_heads_full, st_br_lo, n_dies, claim_limit,
                                                      (uint32_t)quantum_ns, ret, ret_row_shift);
             if (__syncthreads_or((int)(over | nw.over)) == 0) {
@@ -593,7 +598,7 @@ k_inorder_serve(const hbf_access_t *__restrict__ acc, uint64_t n, const __grid_c
                 for (uint32_t q = tid; q < R; q += kInThreads) {
                     const uint4 v = q4[queue_slot(geom, q)];
                     out[q] = make_longlong2((long long)(uint64_t)v.y, v.y ? T0 + (int64_t)(uint64_t)v.x : kNegInf);   // (no service time: no access)
-                    in_headcnt[(uint64_t)tile * R + q] = (uint8_t)(v.w & 15u);
+                    if (!LIGHT) in_headcnt[(uint64_t)tile * R + q] = (uint8_t)(v.w & 15u);
                 }
                 for (uint32_t d = tid; d < n_dies; d += kInThreads) {              // a die's reads: the sums its queues carry
                     unsigned long long g = 0, cnt = 0;
@@ -724,7 +729,7 @@ k_inorder_serve(const hbf_access_t *__restrict__ acc, uint64_t n, const __grid_c
         __syncwarp();
 #pragma unroll
         for (int u = 0; u < K; ++u) tagged[u] = *reinterpret_cast<volatile uint8_t *>(tag_at[u]);
-        if (!RESERVE && turn * (uint32_t)(K * 32) < qid_stride) {   // (the stride is a multiple of a turn's records)
+        if (MODE == kInFull && turn * (uint32_t)(K * 32) < qid_stride) {   // (the stride is a multiple of a turn's records)
 #pragma unroll
             for (int u = 0; u < K; ++u)
                 if (valid[u]) qid_t[i[u]] = ready[u] ? (uint16_t)v[u].queue : (uint16_t)kInMaxQueues;   // (one past the last queue: not modeled)
@@ -753,7 +758,7 @@ k_inorder_serve(const hbf_access_t *__restrict__ acc, uint64_t n, const __grid_c
         }
         // The rest of the turn exists twice: with the head-table bookkeeping, and without it once every queue of the
         // tile has its head entries (after a few percent of a large tile).  The flag is the same for the whole warp.
-        const bool heads_on = !RESERVE && *reinterpret_cast<volatile uint32_t *>(&s_heads_full) < R;
+        const bool heads_on = MODE == kInFull && *reinterpret_cast<volatile uint32_t *>(&s_heads_full) < R;
         auto rest_of_turn = [&](auto heads_tag) {
         constexpr bool HEADS = decltype(heads_tag)::value;
         // ---- per row: the accesses of a lane's queue, up to the lane's own, as one map B -> max(B + S, M), composed
@@ -828,7 +833,7 @@ k_inorder_serve(const hbf_access_t *__restrict__ acc, uint64_t n, const __grid_c
         // ---- results ---------------------------------------------------------------------------------------
 #pragma unroll
         for (int u = 0; u < K; ++u) {
-            if (valid[u]) {
+            if (!LIGHT && valid[u]) {
                 const int64_t done = ready[u] ? B[u] + (int64_t)(v[u].op ? 0u : v[u].xfer) : issue[u];   // a read's data is transferred after its service;
                 const int64_t st = done - issue[u];                                                    // not modeled: completion = issue, no stall
                 sum_stall += st; max_c = max(max_c, ready[u] ? (long long)done : (long long)INT64_MIN);
@@ -858,7 +863,7 @@ k_inorder_serve(const hbf_access_t *__restrict__ acc, uint64_t n, const __grid_c
         for (uint32_t q = tid; q < R; q += kInThreads) {
             const longlong2 v = qst[q];
             out[q] = make_longlong2(v.y >> 8, v.x);
-            in_headcnt[(uint64_t)tile * R + q] = (uint8_t)(v.y & 0xff);
+            if (!LIGHT) in_headcnt[(uint64_t)tile * R + q] = (uint8_t)(v.y & 0xff);
         }
     }
     }                                                        // (the 64-bit form)
@@ -889,7 +894,7 @@ k_inorder_serve(const hbf_access_t *__restrict__ acc, uint64_t n, const __grid_c
     __syncthreads();
     if (tid == 0) {
         if (RESERVE) in_tile[tile].true_sum = s_red[0];
-        else { InTile t; t.spec_sum = s_red[0]; t.fix_delta = 0; t.true_sum = 0; t.reserve = 0u; t.stragglers = 0u; in_tile[tile] = t; }
+        else { InTile t; t.spec_sum = s_red[0]; t.fix_delta = 0; t.true_sum = 0; t.reserve = LIGHT ? 1u : 0u; t.stragglers = 0u; in_tile[tile] = t; }
         if (s_red[1] != INT64_MIN) atomicMax(&ctrl->max_completion_ns, s_red[1]);
         if (!RESERVE && bal) {                               // how many records, how long: what the next batches' tile sizes follow from
             unsigned long long now;
@@ -1431,6 +1436,17 @@ static size_t inorder_straggle_smem() {
 
 size_t inorder_head_bytes(uint64_t tiles, uint32_t n_queues) { return tiles * n_queues * (size_t)kInHead * sizeof(InHead); }
 
+// Batches whose tiles are all served twice, the first time without results and head entries (kInLight), in place of the fix-up.
+// The second time reads 24 and writes 16 bytes per record; the fix-up and its head entries cost some 30 us and what the tiles
+// times the queues make of them.  By records that meets at about 5 M with 64 queues, 11 M with 1,024, 20 M with 2,048 at a load of
+// 0.3, later at higher loads, where more queues are behind.  us, with the fix-up and served twice: 65,536 reads on 64 queues 66
+// and 38, 8 M 162 and 168; decode, 1,024 queues, 4 M 150 and 91, 12 M 207 and 192, 16 M 210 and 225 (load 0.3); capacity, 2,048
+// queues, 4 M 255 and 106, 16 M 323 and 251 (0.3), 28 M 369 and 418 (0.3).
+static uint64_t twice_max(uint32_t n_queues) { return 5000000ull + 7500ull * n_queues; }
+// Larger ones too where the last batch had to serve half of its tiles twice after all (fix-up and second pass: 24 M prefix records
+// 469 us, 48 M at load 0.85 963; served twice at once 357 and 657); every 16th of them takes the fix-up, to see whether it still does.
+constexpr uint32_t kInTwiceRun = 15;
+
 cudaError_t launch_inorder(const SubmitArgs &a, cudaStream_t st) {
     const uint64_t n = a.n;
     const bool by_table = a.bal && a.bal->on && a.bal->dev;
@@ -1466,6 +1482,7 @@ cudaError_t launch_inorder(const SubmitArgs &a, cudaStream_t st) {
         const TileBalance &rec = *bal->pinned;
         if (rec.strag_seq != 0u && rec.strag_seq != bal->depth_seen && rec.strag_depth == bal->depth) {
             bal->depth_seen = rec.strag_seq;
+            if (2u * rec.strag_flagged >= n_tiles) bal->twice_left = kInTwiceRun;
             if (rec.strag_flagged != 0u) bal->depth = (uint32_t)kInHead;
             else if (rec.strag_max > 200u && bal->depth < (uint32_t)kInHead) ++bal->depth;
             else if (rec.strag_max < 148u && bal->depth > 3u) --bal->depth;
@@ -1474,14 +1491,18 @@ cudaError_t launch_inorder(const SubmitArgs &a, cudaStream_t st) {
     } else if (a.bal && a.bal->depth_fixed != 0u) {
         depth = std::min<uint32_t>(a.bal->depth_fixed, (uint32_t)kInHead);
     }
+    bool twice = n <= twice_max(a.mp.n_queues);
+    if (!twice && bal && bal->twice_left > 0u) { --bal->twice_left; twice = true; }
+    if (a.bal && a.bal->depth_fixed != 0u) twice = false;    // (the number of head entries is the caller's)
+    if (twice) depth = 0u;
     const uint64_t tile_records = tmap.max_tile;
     if (n_tiles > inorder_tiles_bound(n)) return cudaErrorInvalidValue;       // the workspace is carved for that many
     const uint32_t R = a.mp.n_queues, nd = a.mp.n_dies;
     const size_t smem_serve = inorder_serve_smem(nd), smem_str = inorder_straggle_smem();
     {
-        const void *serve_fns[6] = {(const void *)k_inorder_serve<false, false, false>, (const void *)k_inorder_serve<true, false, false>,
-                                    (const void *)k_inorder_serve<false, true, false>, (const void *)k_inorder_serve<true, true, false>,
-                                    (const void *)k_inorder_serve<false, false, true>, (const void *)k_inorder_serve<true, false, true>};
+        const void *serve_fns[] = {(const void *)k_inorder_serve<kInFull, false, false>, (const void *)k_inorder_serve<kInAgain, false, false>, (const void *)k_inorder_serve<kInLight, false, false>,
+                                   (const void *)k_inorder_serve<kInFull, true, false>, (const void *)k_inorder_serve<kInAgain, true, false>, (const void *)k_inorder_serve<kInLight, true, false>,
+                                   (const void *)k_inorder_serve<kInFull, false, true>, (const void *)k_inorder_serve<kInAgain, false, true>, (const void *)k_inorder_serve<kInLight, false, true>};
         for (const void *f : serve_fns) { cudaError_t e = ensure_dyn_smem(f, smem_serve); if (e != cudaSuccess) return e; }
         cudaError_t e = ensure_dyn_smem((const void *)k_inorder_scan, 0);
         if (e != cudaSuccess) return e;
@@ -1492,12 +1513,13 @@ cudaError_t launch_inorder(const SubmitArgs &a, cudaStream_t st) {
     InTile *tiles = reinterpret_cast<InTile *>(a.ws.in_tile);
     InHead *heads = reinterpret_cast<InHead *>(a.ws.in_head);
     const bool debt = a.claim_limit != nullptr;              // retention on: the kernels that apply the claims
-    const uint32_t qid_stride = (uint32_t)std::min<uint64_t>(tile_records, kInQidPrefix);
+    const uint32_t qid_stride = twice ? 0u : (uint32_t)std::min<uint64_t>(tile_records, kInQidPrefix);
     if ((uint64_t)n_tiles * qid_stride > inorder_qid_entries(n)) return cudaErrorInvalidValue;
-    auto serve = [&](bool reserve) {
-        auto k = a.paged ? (reserve ? k_inorder_serve<true, false, true> : k_inorder_serve<false, false, true>)
-               : reserve ? (debt ? k_inorder_serve<true, true, false> : k_inorder_serve<true, false, false>)
-                         : (debt ? k_inorder_serve<false, true, false> : k_inorder_serve<false, false, false>);
+    auto serve = [&](bool again) {
+        auto pick = [&](auto full, auto second, auto light) { return again ? second : twice ? light : full; };
+        auto k = a.paged ? pick(k_inorder_serve<kInFull, false, true>, k_inorder_serve<kInAgain, false, true>, k_inorder_serve<kInLight, false, true>)
+               : debt ? pick(k_inorder_serve<kInFull, true, false>, k_inorder_serve<kInAgain, true, false>, k_inorder_serve<kInLight, true, false>)
+                      : pick(k_inorder_serve<kInFull, false, false>, k_inorder_serve<kInAgain, false, false>, k_inorder_serve<kInLight, false, false>);
         return launch_pdl(k, n_tiles, kInThreads, smem_serve, st, a.acc, n, tmap, a.ranges, a.mp, a.fast, a.ctrl, a.status, a.ws.in_agg,
                           a.stats_stage, a.completion, a.stall, (const int64_t *)a.ws.in_bin, tiles, heads, a.ws.in_headcnt,
                           (const int64_t *)a.busy, a.claim_limit, a.die_claims, debt ? *a.ret : RetDev{}, a.ws.in_qid, qid_stride,
@@ -1507,7 +1529,7 @@ cudaError_t launch_inorder(const SubmitArgs &a, cudaStream_t st) {
     if (le == cudaSuccess)
         le = launch_pdl(k_inorder_scan, (R + kInScanQueues - 1) / kInScanQueues, dim3(kInScanQueues, kInScanChunks), 0, st, a.ctrl, a.mp_dev, n_tiles,
                         (const int64_t *)a.ws.in_agg, a.ws.in_bin, (const int64_t *)a.busy, a.busy_stage, a.stats_stage, a.path == HBF_PATH_INORDER ? 1 : 0);
-    if (le == cudaSuccess)
+    if (le == cudaSuccess && !twice)
         le = launch_pdl(a.paged ? k_inorder_fixstraggle<false, true> : debt ? k_inorder_fixstraggle<true, false> : k_inorder_fixstraggle<false, false>, n_tiles, kInStrThreads,
                         smem_str, st, a.acc, n, tmap, a.ranges, a.mp, a.fast, a.ctrl, (const int64_t *)a.ws.in_bin, (const InHead *)heads, (const uint8_t *)a.ws.in_headcnt,
                         a.completion, a.stall, tiles, a.claim_limit, (const uint16_t *)a.ws.in_qid, qid_stride, depth, bal ? bal->dev : nullptr, ordered_copy(n, a.ws));
@@ -1517,7 +1539,7 @@ cudaError_t launch_inorder(const SubmitArgs &a, cudaStream_t st) {
         cudaError_t e = cudaMemcpyAsync(bal->pinned, bal->dev, offsetof(TileBalance, first), cudaMemcpyDeviceToHost, st);
         if (e != cudaSuccess) return e;
     }
-    g_kernel_launches += 4;
+    g_kernel_launches += twice ? 3 : 4;
     return cudaGetLastError();
 }
 

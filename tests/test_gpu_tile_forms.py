@@ -43,9 +43,10 @@ def stream(kind, n, rng):
     return acc
 
 
+@pytest.mark.parametrize("entries", [0, 2, 6])              # 0: served twice (batches of this size); else the fix-up, with so many head entries
 @pytest.mark.parametrize("n", [8_193, 20_001, 65_536])
-@pytest.mark.parametrize("kind", ["plain", "gap", "backlog", "edge", "native", "offset", "read only", "program only", "claims", "claims backlog", "neighbours", "queue per die", "claims queue per die"])
-def test_32_bit_form_matches_the_oracle(hbf, kind, n):
+@pytest.mark.parametrize("kind", ["plain", "gap", "backlog", "edge", "native", "offset", "read only", "program only", "claims", "claims backlog", "neighbours", "queue per die", "claims queue per die", "several ranges", "throttled"])
+def test_32_bit_form_matches_the_oracle(hbf, kind, n, entries):
     import torch
     rng = np.random.default_rng(n)
     prof = wl.load_profile("nominal", channels=8, dies=4, planes=2, page_bytes=16384, stripe_bytes=65536, queue_level=int("queue per die" in kind))
@@ -53,10 +54,13 @@ def test_32_bit_form_matches_the_oracle(hbf, kind, n):
     g, o = hbf.Context(prof), hbfo.Oracle(prof)
     for c in (g, o):
         c.register_range(BASE, 256 * MIB, perms, 0, 0, 3 * 65536)
+        if kind == "several ranges": c.register_range(BASE + 512 * MIB, 64 * MIB, 3, 0, 0, 512 * MIB)
+        if kind == "throttled": c.force_mode(hbfo.MODE_LIGHT, 600_000)
         if "claims" in kind:
             c.enable_retention(pages_per_block=16, blocks_per_plane=32, blocks_per_zone=8, max_pec=3000, disturb_limit=0,
                                l_ref_s=1.0, t_ref_c=40.0, ea_ev=1.04, accel=1.0, lead_threshold=0.5)
             c.retention_advance(1_000_000_000, [40.0])      # every block becomes eligible: 32,768 quanta
+    if entries: g.set_head_entries(entries)
     acc = stream(kind.split()[-1] if "backlog" in kind else kind, n, rng)
     if kind == "neighbours":                                # walks along the stripe units; nearly every tile is served again
         acc["addr"] = BASE + (np.arange(n) % 4000).astype(np.uint64) * np.uint64(65536)
