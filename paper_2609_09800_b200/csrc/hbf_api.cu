@@ -768,7 +768,7 @@ int hbf_enable_retention(hbf_ctx *c, const hbf_retention_config_t *cfg) {
     if ((rc = dev_copy<uint8_t>(c, &r.worn, nullptr, nb)) != HBF_OK) return rc;
     if ((rc = dev_copy<unsigned long long>(c, &r.last_pos, nullptr, nb)) != HBF_OK) return rc;
     if ((rc = dev_copy<uint32_t>(c, &r.plan, nullptr, r.plan_cap)) != HBF_OK) return rc;
-    if ((rc = dev_copy<uint32_t>(c, &r.rank, nullptr, nb)) != HBF_OK) return rc;
+    if ((rc = dev_copy<uint32_t>(c, &r.list, nullptr, nb)) != HBF_OK) return rc;
     if ((rc = dev_copy<unsigned long long>(c, &r.die_len, nullptr, c->mp.n_dies)) != HBF_OK) return rc;
     if ((rc = dev_copy<unsigned long long>(c, &r.chan_len, nullptr, c->mp.channels)) != HBF_OK) return rc;
     if ((rc = dev_copy<uint32_t>(c, &r.die_claims, nullptr, c->mp.n_dies)) != HBF_OK) return rc;

@@ -394,3 +394,28 @@ def test_state_blob_carries_bus_ledger_and_retention(hbf):
     plain, _, _ = contexts(hbf, ret)                          # retention only: the blob does not fit
     with pytest.raises(hbf.HbfError):
         plain.set_state(blob)
+
+
+@pytest.mark.parametrize("channels, dies, ppb", [(1, 1, 3), (33, 3, 16), (64, 8, 5), (65, 2, 64), (128, 16, 3), (128, 17, 3), (130, 1, 4), (2, 33, 4)])
+def test_plan_over_uneven_channels_and_dies(hbf, channels, dies, ppb):
+    """Channels and dies with few eligible blocks, many or none, around the lanes of a warp and the sizes the plan kernel's
+    tables hold; debt that reaches past the batch, into it, and exactly to its end."""
+    ret = dict(RET, disturb_limit=3, lead_threshold=1e9, pages_per_block=ppb, blocks_per_plane=12, blocks_per_zone=4)
+    g, o, prof = contexts(hbf, ret, channels=channels, dies=dies, planes=2)
+    rng = np.random.default_rng(channels * 100 + dies)
+    units, t0 = channels * dies * 2, 0
+    skew = rng.random(units) ** 6                                          # most stripe units are read hardly at all
+    for round_ in range(4):
+        n = min(60_000, max(500, units * 12))
+        acc = mixed_batch(rng, n, t0, 1, natives=0.05)
+        unit = rng.choice(units, n, p=skew / skew.sum()).astype(np.uint64)
+        modeled = acc["addr"] >= BASE
+        acc["addr"][modeled] = (BASE + (unit + np.uint64(units) * rng.integers(0, 12 * ppb, n).astype(np.uint64)) * np.uint64(PAGE))[modeled]
+        acc["bytes"] = np.minimum(acc["bytes"], 4096)
+        owed = o.retention_totals()["planned"] - o.retention_totals()["claimed"]
+        if round_ == 2 and 0 < owed < n: acc = acc[:owed]                  # as many records as quanta owed
+        assert compare_batch(g, o, acc) == 0
+        t0 = int(acc["issue_ns"][-1]) + 50_000_000
+        g.retention_advance(10**9, [40.0]); o.retention_advance(10**9, [40.0])
+        compare_state(g, o)
+    assert o.retention_totals()["planned"] > 0
