@@ -25,7 +25,7 @@ k_energy_bins(const hbf_access_t *__restrict__ acc, uint64_t n, const int64_t *_
     const RangeSnap &rs = *ranges;
     const int64_t q_ppm = ctrl->q_ppm;
     const Div64 div_q = ctrl->div_q;
-    const uint32_t n_dies = mp.n_dies;
+    const Ledger book = make_ledger(ledger, mp.n_dies, n_bins, cur_bin, bin_ns);
     const uint64_t claim_limit = claim_limit_p ? *claim_limit_p : 0ull;
     const int64_t quantum_ns = q_ppm == 1000000 ? mp.t_read_ns + mp.t_prog_ns
         : (int64_t)div64((uint64_t)(mp.t_read_ns + mp.t_prog_ns) * 1000000ull + (uint64_t)q_ppm - 1ull, div_q);
@@ -42,9 +42,9 @@ k_energy_bins(const hbf_access_t *__restrict__ acc, uint64_t n, const int64_t *_
         const int64_t end = completion[i] - (op ? 0 : t.xfer);
         int64_t start = end - t.s;
         if (i < claim_limit) {
-            ledger_event(ledger, n_dies, n_bins, cur_bin, bin_ns, d.die, start - quantum_ns, quantum_ns, quantum_pj);
+            ledger_event(book, d.die, start - quantum_ns, quantum_ns, quantum_pj);
         }
-        ledger_event(ledger, n_dies, n_bins, cur_bin, bin_ns, d.die, start, t.s, t.energy);
+        ledger_event(book, d.die, start, t.s, t.energy);
     }
 }
 

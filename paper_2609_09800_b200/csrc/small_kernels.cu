@@ -350,6 +350,7 @@ k_small_serve(const __grid_constant__ SmallArgs a) {
             // (the first entry of the list is a head, so a map without a head never reaches an entry that needs its input)
             int64_t B = ex.M;
             uint32_t pq = prev_q;
+            const Ledger book = EXTRA && a.ledger ? make_ledger(a.ledger, mp.n_dies, a.n_bins, a.cur_bin, a.bin_ns) : Ledger{};
             for (uint32_t p = p0; p < p1; ++p) {
                 const uint32_t e = sorted[p], lq = s_lq[e], px = s_px[e], i = (uint32_t)s_key[e] & (kInSmallMax - 1u), op = (uint32_t)(s_key[e] >> kSmIdxBits) & 1u;
                 const int64_t t = (int64_t)(s_key[e] >> 16), s = s_s[e], x = (int64_t)(px & 0x7fffffffu);
@@ -367,9 +368,9 @@ k_small_serve(const __grid_constant__ SmallArgs a) {
                     const uint64_t gm = (1ull << (op ? mp.prog_gran_shift : mp.read_gran_shift)) - 1ull, cb = ((uint64_t)(uint32_t)__ldg(rec0 + (size_t)i * 3 + 2) + gm) & ~gm;
                     const uint32_t die = d_lo + lq / per_die;
                     const int64_t pj = op ? mp.e_cmd_prog_pj + mp.e_byte_prog_pj * (int64_t)cb : mp.e_cmd_read_pj + mp.e_byte_read_pj * (int64_t)cb;
-                    if (claim) ledger_event(a.ledger, mp.n_dies, a.n_bins, a.cur_bin, a.bin_ns, die, B - s, quantum_ns,
+                    if (claim) ledger_event(book, die, B - s, quantum_ns,
                                             mp.e_cmd_read_pj + mp.e_byte_read_pj * page + mp.e_cmd_prog_pj + mp.e_byte_prog_pj * page);
-                    ledger_event(a.ledger, mp.n_dies, a.n_bins, a.cur_bin, a.bin_ns, die, B - own, own, pj);
+                    ledger_event(book, die, B - own, own, pj);
                 }
                 pq = lq;
             }
