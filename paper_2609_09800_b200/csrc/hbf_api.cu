@@ -44,7 +44,7 @@ struct hbf_ctx {
     int64_t *d_busy = nullptr, *d_busy_stage = nullptr, *d_pending = nullptr; hbf_die_stats_t *d_stats_stage = nullptr;
     // pinned: the last batch's summary (written by its last kernel), part counts on their way back, the hotspots (written by the
     // thermal step), the tiles' times
-    struct Pinned { hbf_batch_result_t result; unsigned long long totals[kPagedTotals]; float hot[4]; TileBalance bal; } *pinned = nullptr;
+    struct Pinned { hbf_batch_result_t result, host_sum; RetState ret; unsigned long long ret_waiting; unsigned long long totals[kPagedTotals]; float hot[4]; TileBalance bal; } *pinned = nullptr;
     bool result_on_host = false;                 // pinned->result is the last batch's summary (small batches leave theirs on the device only)
     bool plain_next = false;                     // what was enqueued last may launch kernels of its own: see launch_first
     TileBalanceHost bal;                         // tile sizes of the in-order path from the times earlier batches left
@@ -71,7 +71,7 @@ struct hbf_ctx {
         hbf_batch_result_t *d_sum = nullptr, *h_sum = nullptr;          // the chunks' summaries added up: device, and pinned
         cudaStream_t s_in = nullptr, s_out = nullptr;
         cudaEvent_t arrived[2] = {}, served[2] = {}, read[2] = {}, start = nullptr;
-        bool made = false;
+        bool made = false; int sets = 0;                 // streams and events exist; sets of buffers
     } pipe;
 };
 
@@ -262,15 +262,14 @@ int hbf_destroy(hbf_ctx *c) {
     if (c->d_bus_ctrl) cudaFree(c->d_bus_ctrl);
     if (c->d_rom_kind) cudaFree(c->d_rom_kind);
     if (c->d_rom_T) cudaFree(c->d_rom_T);
-    if (c->pipe.made) {
-        hbf_ctx::HostPipe &p = c->pipe;
+    hbf_ctx::HostPipe &p = c->pipe;
+    if (p.made) {
         cudaStreamSynchronize(p.s_in); cudaStreamSynchronize(p.s_out);
-        for (int k = 0; k < 2; ++k) { cudaFree(p.acc[k]); cudaFree(p.comp[k]); cudaFree(p.stall[k]); cudaEventDestroy(p.arrived[k]); cudaEventDestroy(p.served[k]); cudaEventDestroy(p.read[k]); }
-        cudaFree(p.stats); cudaFree(p.total); cudaFree(p.ws); cudaEventDestroy(p.start);
-        if (p.h_sum) cudaFreeHost(p.h_sum);
-        cudaFree(p.d_sum);
+        for (int k = 0; k < 2; ++k) { cudaEventDestroy(p.arrived[k]); cudaEventDestroy(p.served[k]); cudaEventDestroy(p.read[k]); }
+        cudaEventDestroy(p.start);
         cudaStreamDestroy(p.s_in); cudaStreamDestroy(p.s_out);
     }
+    cudaFree(p.ws); cudaFree(p.stats);
     delete c;
     return HBF_OK;
 }
@@ -534,9 +533,17 @@ int hbf_submit_batch(hbf_ctx *c, const hbf_access_t *d_acc, uint64_t n, int64_t 
 constexpr uint64_t kHostResultsMax = 65536;                  // records
 // Host-buffer submit: the batch is cut into chunks; the copy-in of chunk k+1, the service of chunk k (hbf_submit_batch)
 // and the read-back of chunk k-1 run on three streams, so the link moves both ways while the kernels run.
-static int host_pipe_prepare(hbf_ctx *c, uint64_t chunk) {
+// (what only several chunks need, the streams and the second set of buffers, is made when a call first has several)
+static int host_pipe_prepare(hbf_ctx *c, uint64_t chunk, bool several) {
     hbf_ctx::HostPipe &p = c->pipe;
-    if (!p.made) {
+    if (!p.stats) {
+        const size_t stats = ((size_t)c->mp.n_dies * sizeof(hbf_die_stats_t) + 255) / 256 * 256;
+        char *base = nullptr;
+        if (cudaMalloc(&base, 2 * stats + sizeof(hbf_batch_result_t)) != cudaSuccess) return HBF_E_NOMEM;
+        p.stats = reinterpret_cast<hbf_die_stats_t *>(base); p.total = reinterpret_cast<hbf_die_stats_t *>(base + stats);
+        p.d_sum = reinterpret_cast<hbf_batch_result_t *>(base + 2 * stats); p.h_sum = &c->pinned->host_sum;
+    }
+    if (several && !p.made) {
         CK(cudaStreamCreateWithFlags(&p.s_in, cudaStreamNonBlocking));
         CK(cudaStreamCreateWithFlags(&p.s_out, cudaStreamNonBlocking));
         for (int k = 0; k < 2; ++k) {
@@ -545,23 +552,25 @@ static int host_pipe_prepare(hbf_ctx *c, uint64_t chunk) {
             CK(cudaEventCreateWithFlags(&p.read[k], cudaEventDisableTiming));
         }
         CK(cudaEventCreateWithFlags(&p.start, cudaEventDisableTiming));
-        if (cudaMalloc(&p.stats, (size_t)c->mp.n_dies * sizeof(hbf_die_stats_t)) != cudaSuccess) return HBF_E_NOMEM;
-        if (cudaMalloc(&p.total, (size_t)c->mp.n_dies * sizeof(hbf_die_stats_t)) != cudaSuccess) return HBF_E_NOMEM;
-        if (cudaMalloc(&p.d_sum, sizeof(hbf_batch_result_t)) != cudaSuccess) return HBF_E_NOMEM;
-        if (cudaMallocHost(&p.h_sum, sizeof(hbf_batch_result_t)) != cudaSuccess) return HBF_E_NOMEM;
         p.made = true;
     }
     const size_t ws_need = hbf_workspace_bytes(c, chunk);
-    if (chunk > p.chunk || ws_need > p.ws_bytes) {
-        CK(cudaStreamSynchronize(c->stream)); CK(cudaStreamSynchronize(p.s_in)); CK(cudaStreamSynchronize(p.s_out));
-        for (int k = 0; k < 2; ++k) {
-            cudaFree(p.acc[k]); cudaFree(p.comp[k]); cudaFree(p.stall[k]); p.acc[k] = nullptr; p.comp[k] = p.stall[k] = nullptr;
-            if (cudaMalloc(&p.acc[k], chunk * sizeof(hbf_access_t)) != cudaSuccess || cudaMalloc(&p.comp[k], chunk * 8) != cudaSuccess ||
-                cudaMalloc(&p.stall[k], chunk * 8) != cudaSuccess) { p.chunk = 0; return HBF_E_NOMEM; }
+    const int sets = several || p.sets == 2 ? 2 : 1;
+    if (chunk > p.chunk || ws_need > p.ws_bytes || sets > p.sets) {
+        CK(cudaStreamSynchronize(c->stream));
+        if (p.made) { CK(cudaStreamSynchronize(p.s_in)); CK(cudaStreamSynchronize(p.s_out)); }
+        const uint64_t most = std::max(chunk, p.chunk);
+        auto up = [](size_t v) { return (v + 255) / 256 * 256; };
+        const size_t rec = up(most * sizeof(hbf_access_t)), res = up(most * 8), set = rec + 2 * res, ws = up(std::max(ws_need, p.ws_bytes));
+        cudaFree(p.ws); p.ws = nullptr; p.chunk = 0; p.ws_bytes = 0; p.sets = 0;
+        char *base = nullptr;                                // workspace, then records, completions and stalls of every set
+        if (cudaMalloc(&base, ws + (size_t)sets * set) != cudaSuccess) return HBF_E_NOMEM;
+        p.ws = base;
+        for (int k = 0; k < sets; ++k) {
+            char *at = base + ws + (size_t)k * set;
+            p.acc[k] = reinterpret_cast<hbf_access_t *>(at); p.comp[k] = reinterpret_cast<int64_t *>(at + rec); p.stall[k] = reinterpret_cast<int64_t *>(at + rec + res);
         }
-        cudaFree(p.ws); p.ws = nullptr;
-        if (cudaMalloc(&p.ws, ws_need) != cudaSuccess) { p.chunk = 0; p.ws_bytes = 0; return HBF_E_NOMEM; }
-        p.chunk = chunk; p.ws_bytes = ws_need;
+        p.chunk = most; p.ws_bytes = ws; p.sets = sets;
     }
     return HBF_OK;
 }
@@ -573,7 +582,7 @@ int hbf_submit_host(hbf_ctx *c, const hbf_access_t *h_acc, uint64_t n, int64_t *
     if (n && (!h_acc || !h_completion_ns || !h_stall_ns)) return HBF_E_INVAL;
     if (chunk == 0) chunk = 4000000;
     chunk = std::min<uint64_t>(std::min<uint64_t>(chunk, HBF_MAX_BATCH), std::max<uint64_t>(n, 1));
-    int rc = host_pipe_prepare(c, chunk);
+    int rc = host_pipe_prepare(c, chunk, n == 0 || n > chunk);
     if (rc != HBF_OK) return rc;
     hbf_ctx::HostPipe &p = c->pipe;
     cudaStream_t main = c->stream;
@@ -831,15 +840,12 @@ int hbf_get_retention_plan(hbf_ctx *c, uint32_t *quanta, uint64_t cap, uint64_t 
 
 int hbf_get_retention_totals(hbf_ctx *c, hbf_retention_totals_t *out) {
     if (!c || !c->ret_on || !out) return HBF_E_INVAL;
-    RetState s; int rc = retention_state(c, &s);
-    if (rc != HBF_OK) return rc;
-    std::vector<uint32_t> ep(c->ret.n_blocks);
-    CK(cudaMemcpyAsync(ep.data(), c->ret.epoch_of, c->ret.n_blocks * 4, cudaMemcpyDeviceToHost, c->stream));
+    CK(launch_ret_totals(c->ret, c->sm_count, &c->pinned->ret, &c->pinned->ret_waiting, c->stream));
     CK(cudaStreamSynchronize(c->stream));
+    const RetState &s = c->pinned->ret;
     out->n_blocks = c->ret.n_blocks; out->planned = s.planned; out->claimed = s.claimed; out->decayed = s.decayed;
     out->commits = s.commits; out->worn_blocks = s.worn_blocks; out->epoch = s.epoch; out->pad = 0;
-    out->waiting_blocks = 0;
-    for (uint32_t e : ep) if (e) out->waiting_blocks += 1;
+    out->waiting_blocks = c->pinned->ret_waiting;
     return HBF_OK;
 }
 
@@ -858,10 +864,10 @@ int hbf_enable_energy_bins(hbf_ctx *c, int64_t bin_ns, uint32_t n_bins) {
 
 int hbf_get_energy_bins(hbf_ctx *c, int64_t *host_out, uint64_t cap, int64_t *first_bin) {
     if (!c || !c->d_ledger || !host_out || cap < (uint64_t)c->n_bins * c->mp.n_dies) return HBF_E_INVAL;
-    const size_t row = (size_t)c->mp.n_dies * 8;
-    for (uint32_t k = 0; k < c->n_bins; ++k)                // row k of the output is bin cur_bin + k
-        CK(cudaMemcpyAsync(host_out + (size_t)k * c->mp.n_dies, c->d_ledger + (size_t)((c->cur_bin + k) % c->n_bins) * c->mp.n_dies,
-                           row, cudaMemcpyDeviceToHost, c->stream));
+    // row k of the output is bin cur_bin + k: the ring wraps once, so two copies (one per bin, 64 of them: 726 us; now 52)
+    const size_t row = c->mp.n_dies, at = (size_t)(c->cur_bin % c->n_bins), head = c->n_bins - at;
+    CK(cudaMemcpyAsync(host_out, c->d_ledger + at * row, head * row * 8, cudaMemcpyDeviceToHost, c->stream));
+    if (at) CK(cudaMemcpyAsync(host_out + head * row, c->d_ledger, at * row * 8, cudaMemcpyDeviceToHost, c->stream));
     CK(cudaStreamSynchronize(c->stream));
     if (first_bin) *first_bin = c->cur_bin;
     return HBF_OK;

