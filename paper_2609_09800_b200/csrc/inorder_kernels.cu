@@ -17,6 +17,7 @@
 //             each of them has fallen idle;
 //   re-serve  a tile with many stragglers (the batch arrived on queues that were far behind) is served
 //             again from the true entering busy-until, exactly.
+// Smaller batches (twice_max) skip fix-up and straggle: serve without results, scan, re-serve of every tile.
 // The serve pass is the only one that streams the whole batch: 24 B read and 16 B + 1 B written per access.
 // Every global access of it is coalesced; nothing waits on another thread block, and no thread spins.
 //
@@ -466,6 +467,7 @@ __device__ __forceinline__ NarrowSums serve_narrow(const FastGeom &geom, const M
 // read and a page program, scaled like any service, Eq. 3) before its own service; the streaming pass counts the
 // claims per die.
 // PAGED = true: the page-granular submit of accesses that stay inside one stripe unit each (paged_terms).
+// MODE: kInFull, kInAgain or kInLight (above).
 template <int MODE, bool DEBT, bool PAGED>
 __global__ void __launch_bounds__(kInThreads, kInBlocksPerSM)
 k_inorder_serve(const hbf_access_t *__restrict__ acc, uint64_t n, const __grid_constant__ InTileMap tmap, const RangeSnap *__restrict__ ranges_g,
@@ -591,22 +593,22 @@ k_inorder_serve(const hbf_access_t *__restrict__ acc, uint64_t n, const __grid_c
                 sum_stall = nw.stall;
                 if (nw.max_done) max_c = T0 + (int64_t)(uint64_t)nw.max_done;      // (a modeled access ends after its tile's first issue time)
                 if constexpr (!RESERVE) {
-                c_unsorted |= nw.unsorted;
-                if (tid == 0 && tile_begin > 0 && acc_t[-1].issue_ns > T0) c_unsorted = 1u;
-                t_native = nw.native; t_fault = nw.fault; t_ready = (tid == 0 ? (long long)tile_len : 0ll) - t_native - t_fault;
-                longlong2 *out = reinterpret_cast<longlong2 *>(in_agg) + (uint64_t)tile * R;
-                for (uint32_t q = tid; q < R; q += kInThreads) {
-                    const uint4 v = q4[queue_slot(geom, q)];
-                    out[q] = make_longlong2((long long)(uint64_t)v.y, v.y ? T0 + (int64_t)(uint64_t)v.x : kNegInf);   // (no service time: no access)
-                    if (!LIGHT) in_headcnt[(uint64_t)tile * R + q] = (uint8_t)(v.w & 15u);
-                }
-                for (uint32_t d = tid; d < n_dies; d += kInThreads) {              // a die's reads: the sums its queues carry
-                    unsigned long long g = 0, cnt = 0;
-                    for (uint32_t p = 0; p < geom.planes_q; ++p) { const uint4 v = q4[queue_slot(geom, d * geom.planes_q + p)]; g += v.z; cnt += v.w >> 4; }
-                    unsigned long long *gd = reinterpret_cast<unsigned long long *>(stats_stage + d);
-                    if (g) atomicAdd(&gd[1], g << geom.gran_shift_read);
-                    if (cnt) atomicAdd(&gd[4], cnt);
-                }
+                    c_unsorted |= nw.unsorted;
+                    if (tid == 0 && tile_begin > 0 && acc_t[-1].issue_ns > T0) c_unsorted = 1u;
+                    t_native = nw.native; t_fault = nw.fault; t_ready = (tid == 0 ? (long long)tile_len : 0ll) - t_native - t_fault;
+                    longlong2 *out = reinterpret_cast<longlong2 *>(in_agg) + (uint64_t)tile * R;
+                    for (uint32_t q = tid; q < R; q += kInThreads) {
+                        const uint4 v = q4[queue_slot(geom, q)];
+                        out[q] = make_longlong2((long long)(uint64_t)v.y, v.y ? T0 + (int64_t)(uint64_t)v.x : kNegInf);   // (no service time: no access)
+                        if (!LIGHT) in_headcnt[(uint64_t)tile * R + q] = (uint8_t)(v.w & 15u);
+                    }
+                    for (uint32_t d = tid; d < n_dies; d += kInThreads) {              // a die's reads: the sums its queues carry
+                        unsigned long long g = 0, cnt = 0;
+                        for (uint32_t p = 0; p < geom.planes_q; ++p) { const uint4 v = q4[queue_slot(geom, d * geom.planes_q + p)]; g += v.z; cnt += v.w >> 4; }
+                        unsigned long long *gd = reinterpret_cast<unsigned long long *>(stats_stage + d);
+                        if (g) atomicAdd(&gd[1], g << geom.gran_shift_read);
+                        if (cnt) atomicAdd(&gd[4], cnt);
+                    }
                 }
             } else {
                 again = true;

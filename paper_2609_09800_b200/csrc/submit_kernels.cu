@@ -1,4 +1,4 @@
-// Kernels of hbf_submit_batch, sort path:
+// Kernels of hbf_submit_batch, sort path (and the first and last kernel of the in-order path):
 //   begin -> classify (load, range filter, decode, key) -> plan -> histogram -> onesweep radix passes ->
 //   scan (segmented max-plus scan with decoupled look-back, fused with the scatter back to batch order
 //   and the per-die reductions) -> finish (commit or refuse).
@@ -1222,9 +1222,9 @@ static cudaError_t launch_finish_inorder(const SubmitArgs &a, bool may_sort, cud
     return cudaGetLastError();
 }
 
-// Kernel order of one batch.  AUTO: begin, the in-order kernels (they serve the batch when its records
-// arrive in non-decreasing issue order), one thread that launches the sort kernels from the device if the
-// in-order attempt handed the batch over, finish.  SORT / SORT_FULL: begin, sort kernels, finish.
+// Kernel order of one batch.  AUTO: begin (which brings a batch out of issue order into order), the in-order kernels,
+// k_finish_inorder (the commit; it launches the sort kernels from the device where the others handed the batch over).
+// SORT / SORT_FULL: begin, sort kernels, finish.
 cudaError_t launch_submit(const SubmitArgs &a, cudaStream_t st) {
     const uint64_t n = a.n;
     auto mark = [&](int k) { if (a.ev) cudaEventRecord(a.ev[k], st); };
