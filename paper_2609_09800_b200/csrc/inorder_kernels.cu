@@ -575,15 +575,15 @@ k_inorder_serve(const hbf_access_t *__restrict__ acc, uint64_t n, const __grid_c
             if (!RESERVE) for (uint32_t d = tid; d < n_dies * 7u; d += kInThreads) st_br_lo[d] = 0u;
             for (uint32_t q = tid; q < kInMaxQueues; q += kInThreads) {
                 uint4 v = make_uint4(0u, 0u, 0u, 0u);
-                if ((RESERVE || tile == 0u) && q < R) {      // the first tile knows its entering state: it is served exactly
+                if ((RESERVE || (MODE == kInFull && tile == 0u)) && q < R) {   // the first tile knows its entering state: it is served exactly
                     const int64_t b = (RESERVE ? in_bin[(uint64_t)tile * R + q] : busy[q]) - T0;
                     v.x = b > 0 ? (uint32_t)b : 0u;
                     if (b >= (RESERVE ? 1ll << 30 : 1ll << 31)) over = 1u;
                 }
                 q4[q < R ? queue_slot(geom, q) : q] = v;
             }
-            // (a backlog that reaches into the tile, from claims mostly, grows while the tile is served: not even tried then)
-            const bool try_narrow = __syncthreads_or((int)(RESERVE && over)) == 0;
+            // (a backlog that reaches far into the tile grows while the tile is served: not even tried then)
+            const bool try_narrow = __syncthreads_or((int)over) == 0;
             NarrowSums nw{};
             if (try_narrow) nw = serve_narrow<MODE, DEBT, PAGED>(geom, mp, mp_arg, acc_t, (uint32_t)tile_begin, tile_len, T0, q4, warp_tag, status_t, qid_t, qid_stride,
                                                      completion_t, stall_t, in_head, tile, R, head_depth, &s_heads_full, st_br_lo, n_dies, claim_limit,
@@ -611,7 +611,7 @@ k_inorder_serve(const hbf_access_t *__restrict__ acc, uint64_t n, const __grid_c
                     }
                 }
             } else {
-                again = true;
+                again = try_narrow;                          // (its read disturb is counted)
                 if (tid == 0) s_heads_full = 0u;
             }
         }
@@ -623,7 +623,7 @@ k_inorder_serve(const hbf_access_t *__restrict__ acc, uint64_t n, const __grid_c
         for (uint32_t q = tid; q < R; q += kInThreads) qst[q].x = in_bin[(uint64_t)blockIdx.x * R + q];
     } else {
         for (uint32_t d = tid; d < n_dies * 7u; d += kInThreads) st_br_lo[d] = 0u;
-        if (tile == 0u) {                                    // the first tile knows its entering state: it is served exactly
+        if (MODE == kInFull && tile == 0u) {                 // the first tile knows its entering state: it is served exactly
             __syncthreads();
             for (uint32_t q = tid; q < R; q += kInThreads) qst[q].x = busy[q];
         }
