@@ -46,6 +46,7 @@ struct hbf_ctx {
     // thermal step), the tiles' times
     struct Pinned { hbf_batch_result_t result, host_sum; RetState ret; unsigned long long ret_waiting; unsigned long long totals[kPagedTotals]; float hot[4]; TileBalance bal; } *pinned = nullptr;
     bool result_on_host = false;                 // pinned->result is the last batch's summary (small batches leave theirs on the device only)
+    bool captured = false;                       // a batch was captured into a graph: which batch ran last is not for the host to know
     bool plain_next = false;                     // what was enqueued last may launch kernels of its own: see launch_first
     TileBalanceHost bal;                         // tile sizes of the in-order path from the times earlier batches left
     // thermal steps on a reduced-order model instead of the grid (off while rom == nullptr)
@@ -467,6 +468,13 @@ int hbf_set_head_entries(hbf_ctx *c, uint32_t entries) {
     return HBF_OK;
 }
 
+// is what is enqueued on the stream now being captured into a graph
+static bool capturing(cudaStream_t st) {
+    cudaStreamCaptureStatus s = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &s) != cudaSuccess) { (void)cudaGetLastError(); return false; }
+    return s != cudaStreamCaptureStatusNone;
+}
+
 // Everything a batch of records goes through once its arguments are in place: the claim window (retention), the submit
 // path, the energy ledger, read disturb / commits, the channel-bus stage.  Shared by hbf_submit_batch (the caller's
 // accesses) and hbf_submit_batch_paged (the list of parts).
@@ -483,6 +491,7 @@ static int serve_records(hbf_ctx *c, SubmitArgs &a) {
     a.bal = &c->bal; a.rg_sync = c->d_rg_sync;
     if (c->ret_on) { a.claim_limit = &c->ret.st->claim_limit; a.die_claims = c->ret.die_claims; a.ret = &c->ret; }
     c->result_on_host = true;
+    if (capturing(c->stream)) c->captured = true;
     if (small_route(a)) {                                    // one launch, everything included (with the bus on it stops before the ledger)
         auto mark = [&](int k) { if (a.ev) cudaEventRecord(a.ev[k], c->stream); };
         mark(0); mark(7);
@@ -876,7 +885,7 @@ int hbf_get_energy_bins(hbf_ctx *c, int64_t *host_out, uint64_t cap, int64_t *fi
 int hbf_last_result(hbf_ctx *c, hbf_batch_result_t *host_out) {
     if (!c || !host_out) return HBF_E_INVAL;
     if (!c->submitted) { memset(host_out, 0, sizeof(*host_out)); return HBF_OK; }
-    if (!c->result_on_host) CK(cudaMemcpyAsync(&c->pinned->result, c->d_result, sizeof(hbf_batch_result_t), cudaMemcpyDeviceToHost, c->stream));
+    if (!c->result_on_host || c->captured) CK(cudaMemcpyAsync(&c->pinned->result, c->d_result, sizeof(hbf_batch_result_t), cudaMemcpyDeviceToHost, c->stream));
     c->result_on_host = true;
     CK(cudaStreamSynchronize(c->stream));                    // (a large batch's last kernel wrote its summary to the host)
     *host_out = c->pinned->result;

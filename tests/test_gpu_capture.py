@@ -1,0 +1,58 @@
+"""Batches captured into a CUDA graph: every replay serves the batch again on the queues the one before left."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+from oracle import hbfo
+from paper_2609_09800_b200 import workloads as wl
+
+
+@pytest.fixture(scope="module")
+def hbf():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2609_09800_b200 import build, hbf as mod
+    build.build()
+    return mod
+
+
+class Captured:
+    """A context on a stream of its own, a device copy of a batch, and the batch as a graph."""
+
+    def __init__(self, hbf, acc, profile, ranges):
+        import torch
+        self.torch, self.n = torch, len(acc)
+        self.stream = torch.cuda.Stream()
+        self.g, self.o = hbf.Context(profile, stream=self.stream), hbfo.Oracle(profile)
+        for r in ranges:
+            self.g.register_range(*r); self.o.register_range(*r)
+        self.acc = torch.from_numpy(acc.view(np.int64).reshape(-1).copy()).cuda()
+        self.comp, self.stall = (torch.zeros(self.n, dtype=torch.int64, device="cuda") for _ in range(2))
+        self.ws = self.g.workspace(self.n)
+        self.graph = torch.cuda.CUDAGraph()
+        torch.cuda.synchronize()
+
+    def submit(self):
+        assert self.g.submit_batch(self.acc, self.n, self.comp, self.stall, None, None, self.ws) == 0
+
+    def capture(self):
+        with self.torch.cuda.graph(self.graph, stream=self.stream):
+            self.submit()
+
+    def replay(self):
+        with self.torch.cuda.stream(self.stream):
+            self.graph.replay()
+
+
+@pytest.mark.parametrize("n", [4_000, 20_000])
+def test_the_summary_is_that_of_the_last_replay(hbf, n):
+    w = wl.capacity_mode(n=n, seed=n)
+    t = Captured(hbf, w.acc, w.profile, w.ranges)
+    t.capture()
+    for turn in range(4):
+        t.submit() if turn == 2 else t.replay()             # (one of them not from the graph)
+        _, c_o, s_o, *_ = t.o.submit(w.acc)
+        assert t.g.last_result() == t.o.last_result()
+        assert np.array_equal(t.comp.cpu().numpy(), c_o) and np.array_equal(t.stall.cpu().numpy(), s_o)
