@@ -348,7 +348,9 @@ __device__ __forceinline__ NarrowSums serve_narrow(const FastGeom &geom, const M
                     r.fault += 1u;
                 }
             }
-            if (DEBT && !RESERVE && ready[u] && flags == 0u) {           // read disturb: the read's pages, on the block of its first page
+            // read disturb: the read's pages, on the block of its first page.  (`ready` does not ask for the issue time's limits; a
+            // time beyond them sends the tile to the 64-bit form, which refuses the record but counts no disturb a second time)
+            if (DEBT && !RESERVE && ready[u] && flags == 0u && ((uint64_t)issue[u] >> kIssueBits) == 0ull) {
                 const uint32_t npages = (uint32_t)(((uint64_t)((uint32_t)off & geom.page_mask) + bytes + geom.page_mask) >> geom.page_shift);
                 if (ret.pow2 != 0u) {
                     const uint32_t row = (uint32_t)((off >> geom.stripe_shift) >> ret_row_shift);

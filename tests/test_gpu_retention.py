@@ -419,3 +419,23 @@ def test_plan_over_uneven_channels_and_dies(hbf, channels, dies, ppb):
         g.retention_advance(10**9, [40.0]); o.retention_advance(10**9, [40.0])
         compare_state(g, o)
     assert o.retention_totals()["planned"] > 0
+
+
+@pytest.mark.parametrize("entries", [0, 6])                  # 0: every tile is served twice; 6: the fix-up, with so many head entries
+@pytest.mark.parametrize("issue", [-3, 1 << 47])
+def test_a_read_without_a_valid_issue_time_disturbs_nothing(hbf, issue, entries):
+    """Its address and size are those of a modeled read: the batch is refused, and every counter is as before it."""
+    ret = dict(RET, disturb_limit=5, pages_per_block=16)
+    g, o, _ = contexts(hbf, ret, geometry="serving")
+    if entries:
+        g.set_head_entries(entries)
+    n = 12_000
+    acc = np.zeros(n, hbfo.ACCESS_DTYPE)
+    acc["addr"] = BASE + np.random.default_rng(entries).integers(0, 20_000, n).astype(np.uint64) * np.uint64(PAGE)
+    acc["issue_ns"] = 50_000 + 100 * np.arange(n)
+    acc["bytes"] = 4096
+    assert compare_batch(g, o, acc) == 0
+    acc["issue_ns"] += 10_000_000
+    bad = acc.copy(); bad["issue_ns"][1537] = issue          # inside a tile, away from the neighbours that the begin kernel compares
+    assert g.submit_host(bad, check=False)[0] == hbfo.E_ACCESS_FAULT       # (2^47 is this library's limit, the oracle has none)
+    assert compare_batch(g, o, acc) == 0
