@@ -462,7 +462,7 @@ k_small_serve(const __grid_constant__ SmallArgs a) {
         *a.result = r;                                       // (not to the host as well: the kernel would end a microsecond later)
         BatchCtrl *c = a.ctrl;                               // what later stages and hbf_queue_order read of a batch
         c->code = code; c->skip = ok ? 0 : 1; c->mode = mode; c->q_ppm = q_ppm; c->div_q = div_q;
-        c->n_ready = n_ready; c->inorder_used = ok && !unsorted ? 1u : 0u; c->run_sort = 0u; c->plan.n_passes = 1u;
+        c->n_ready = n_ready; c->inorder_used = ok && !unsorted ? 1u : 0u; c->run_sort = 0u; c->regrouped = 0u; c->plan.n_passes = 1u;
         if (EXTRA && a.ret_on && !a.bus_on && ok) a.ret.st->claimed += claims;
     }
 }

@@ -52,3 +52,25 @@ def test_unordered_batches_match_the_oracle(hbf, kind, n):
         if rc_o == 0:
             assert np.array_equal(g.queue_order(n), o.last_order())
         acc["issue_ns"] += 10_000
+
+
+@pytest.mark.parametrize("reset", [False, True])
+def test_the_served_order_after_batches_of_other_routes(hbf, reset):
+    """A large batch out of order, then small ones: the order asked for is that of the last batch, or there is none."""
+    w = wl.capacity_mode(n=28_000, seed=5, rho=0.6)
+    g, o = hbf.Context(w.profile), hbfo.Oracle(w.profile)
+    for r in w.ranges:
+        g.register_range(*r); o.register_range(*r)
+    ws = g.workspace(20_000)
+    rng = np.random.default_rng(1)
+    for lo, hi, ordered in ((0, 20_000, False), (20_000, 24_000, False), (24_000, 28_000, True), (0, 20_000, False), (0, 20_000, True)):
+        acc = w.acc[lo:hi] if ordered else w.acc[lo:hi][rng.permutation(hi - lo)]
+        o.submit(acc); g.submit_host(acc)
+        if ordered:
+            with pytest.raises(hbf.HbfError):
+                g.queue_order(hi - lo, ws)
+        else:
+            assert np.array_equal(g.queue_order(hi - lo, ws), o.last_order())
+            assert np.array_equal(g.queue_order(hi - lo, ws), o.last_order())       # (asking does not spoil it)
+        if reset:
+            g.reset(); o.reset()
