@@ -595,6 +595,13 @@ int hbf_submit_host(hbf_ctx *c, const hbf_access_t *h_acc, uint64_t n, int64_t *
     if (rc != HBF_OK) return rc;
     hbf_ctx::HostPipe &p = c->pipe;
     cudaStream_t main = c->stream;
+    // A batch refused for the controller's mode writes nothing on the device: what was copied out is what the buffers held.  (The
+    // mode does not change within the call, so every chunk is refused or none.)
+    auto zero_withheld = [&](int32_t code) {
+        if (code != HBF_E_LINK_SHUTDOWN && code != HBF_E_THROTTLED) return;
+        memset(h_completion_ns, 0, n * 8); memset(h_stall_ns, 0, n * 8);
+        if (h_die_stats) memset(h_die_stats, 0, (size_t)c->mp.n_dies * sizeof(hbf_die_stats_t));
+    };
     if (n && n <= chunk) {                                   // one chunk: nothing to overlap, so one stream and no events
         CK(cudaMemcpyAsync(p.acc[0], h_acc, n * sizeof(hbf_access_t), cudaMemcpyHostToDevice, main));
         rc = hbf_submit_batch(c, p.acc[0], n, p.comp[0], p.stall[0], nullptr, h_die_stats ? p.stats : nullptr, p.ws, p.ws_bytes);
@@ -623,8 +630,7 @@ int hbf_submit_host(hbf_ctx *c, const hbf_access_t *h_acc, uint64_t n, int64_t *
         }
         CK(cudaStreamSynchronize(main));
         if (p.h_sum->code == HBF_E_LINK_SHUTDOWN) c->terminal = true;
-        if (p.h_sum->code == HBF_E_LINK_SHUTDOWN || p.h_sum->code == HBF_E_THROTTLED)       // (refused before anything was written)
-            if (h_die_stats) memset(h_die_stats, 0, (size_t)c->mp.n_dies * sizeof(hbf_die_stats_t));
+        zero_withheld(p.h_sum->code);
         if (summary_out) *summary_out = *p.h_sum;
         return p.h_sum->code;
     }
@@ -643,7 +649,7 @@ int hbf_submit_host(hbf_ctx *c, const hbf_access_t *h_acc, uint64_t n, int64_t *
         if (read[s]) CK(cudaStreamWaitEvent(main, p.read[s], 0));         // the slot's results have left
         rc = hbf_submit_batch(c, p.acc[s], m, p.comp[s], p.stall[s], nullptr, p.stats, p.ws, p.ws_bytes);
         if (rc != HBF_OK) break;
-        CK(launch_add_stats(p.total, p.stats, c->mp.n_dies, main));       // (a refused chunk leaves zeros)
+        CK(launch_add_stats(p.total, p.stats, c->mp.n_dies, main));       // (a refused chunk leaves zeros; see zero_withheld)
         CK(launch_add_result(p.d_sum, c->d_result, k == 0 ? 1 : 0, main));
         CK(cudaEventRecord(p.served[s], main)); served[s] = true;
         CK(cudaStreamWaitEvent(p.s_out, p.served[s], 0));
@@ -659,6 +665,7 @@ int hbf_submit_host(hbf_ctx *c, const hbf_access_t *h_acc, uint64_t n, int64_t *
     hbf_batch_result_t sum; memset(&sum, 0, sizeof(sum));
     if (k) sum = *p.h_sum;
     if (sum.code == HBF_E_LINK_SHUTDOWN) c->terminal = true;
+    if (n) zero_withheld(sum.code);
     if (summary_out) *summary_out = sum;
     return sum.code;
 }

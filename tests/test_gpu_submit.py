@@ -528,3 +528,26 @@ def test_one_chunk_from_the_host_in_pinned_and_pageable_memory(hbf, n):
         assert np.array_equal(c[1:].numpy(), c_o) and c[0] == -1 and np.array_equal(s[:n].numpy(), s_o) and s[n] == -1
         got = ds.numpy().view(hbfo.DIE_STATS_DTYPE)
         assert all(np.array_equal(got[f], ds_o[f]) for f in hbfo.DIE_STATS_DTYPE.names)
+
+
+@pytest.mark.parametrize("chunk", [0, 2_000])
+@pytest.mark.parametrize("pin", [True, False])
+def test_a_throttled_call_from_the_host_leaves_zeros(hbf, pin, chunk):
+    import torch
+    n = 5_000
+    w = wl.capacity_mode(n=n, seed=3)
+    g, o = contexts(hbf, w.profile, w.ranges)
+    make = lambda t: t.pin_memory() if pin else t
+    rec = make(torch.from_numpy(w.acc.view(np.int64).reshape(-1).copy()))
+    out = [make(torch.full((k,), -1, dtype=torch.int64)) for k in (n, n, g.n_dies * 6)]
+    for served in (False, True, False):                     # refused on fresh buffers, served, refused on what that left
+        g.force_mode(0 if served else 2, 1_000_000)
+        for t in out: t.fill_(-1)
+        busy = g.get_busy_until()
+        rc, summary = g.submit_pinned(rec, n, *out, chunk=chunk)
+        if served:
+            assert rc == 0 and np.array_equal(out[0].numpy(), o.submit(w.acc)[1])
+        else:
+            assert rc == hbf.E_THROTTLED and summary["code"] == rc and summary["n_modeled"] == 0
+            assert not any(t.any() for t in out)
+            assert np.array_equal(g.get_busy_until(), busy)
