@@ -135,7 +135,7 @@ struct SubmitArgs {
 struct FinishArgs {
     uint64_t n; BatchCtrl *ctrl; DevState *state; int64_t *busy; const int64_t *busy_stage; int64_t *pending; const hbf_die_stats_t *stats_stage;
     hbf_die_stats_t *die_stats; int64_t *completion, *stall; hbf_batch_result_t *result, *result_host; const ModelParams *mp;
-    uint32_t n_queues, n_dies; int binned, bus_on;
+    uint32_t n_queues, n_dies; int binned, bus_on, paged;
 };
 // hbf_reset: memory to clear, and the state that is not zero
 struct ResetArgs {

@@ -696,6 +696,8 @@ __device__ __forceinline__ int finish_batch(const FinishArgs &f, long long model
     if (code == HBF_E_ACCESS_FAULT || code == HBF_E_TIMEOUT || code == HBF_E_INVAL) {
         for (uint64_t i = gtid; i < n; i += gsz) { f.completion[i] = 0; f.stall[i] = 0; }
         if (f.die_stats) for (uint64_t i = gtid; i < (uint64_t)f.n_dies * 6u; i += gsz) reinterpret_cast<int64_t *>(f.die_stats)[i] = 0;
+    } else if (f.paged && (code == HBF_E_THROTTLED || code == HBF_E_LINK_SHUTDOWN)) {     // (a page-granular batch leaves zeros then, as its join does)
+        for (uint64_t i = gtid; i < n; i += gsz) { f.completion[i] = 0; f.stall[i] = 0; }
     } else if (code == HBF_OK) {
         const bool inorder = ctrl->inorder_used != 0u;
         for (uint64_t r = gtid; r < f.n_queues; r += gsz) f.busy[r] = f.busy_stage[r];
@@ -1189,7 +1191,7 @@ static FinishArgs finish_args(const SubmitArgs &a) {
     f.n = a.n; f.ctrl = a.ctrl; f.state = a.state; f.busy = a.busy; f.busy_stage = a.busy_stage; f.pending = a.pending;
     f.stats_stage = a.stats_stage; f.die_stats = a.die_stats; f.completion = a.completion; f.stall = a.stall;
     f.result = a.result; f.result_host = a.result_host; f.mp = a.mp_dev; f.n_queues = a.mp.n_queues; f.n_dies = a.mp.n_dies;
-    f.binned = a.binned; f.bus_on = a.bus_on;
+    f.binned = a.binned; f.bus_on = a.bus_on; f.paged = a.paged;
     return f;
 }
 static unsigned finish_grid(const SubmitArgs &a) { return (unsigned)std::max<uint64_t>(1, std::min<uint64_t>((a.n + 1023) / 1024, (uint64_t)a.sm_count * 4)); }

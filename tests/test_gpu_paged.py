@@ -208,3 +208,22 @@ def test_stripe_units_match_the_oracle(hbf, kind, n):
     for _ in range(2):
         compare(g, o, acc)
         acc["issue_ns"] += 1000
+
+
+@pytest.mark.parametrize("cross", [False, True])             # (no access crosses a stripe unit: the batch's own records are served)
+@pytest.mark.parametrize("n", [5_000, 12_000])
+def test_a_throttled_paged_batch_leaves_zeros(hbf, n, cross):
+    import torch
+    rng = np.random.default_rng(n)
+    prof = wl.load_profile("nominal", channels=8, dies=4, planes=2, page_bytes=16384, stripe_bytes=65536)
+    g, o = contexts(hbf, prof, [(wl.RANGE_BASE, wl.GIB, 3, 0, 0, 0)])
+    acc = np.zeros(n, hbfo.ACCESS_DTYPE)
+    acc["addr"] = wl.RANGE_BASE + rng.integers(0, 8_000, n).astype(np.uint64) * np.uint64(65536) + np.uint64(60_000 if cross else 0)
+    acc["bytes"] = 40_000
+    acc["issue_ns"] = 1000 * np.arange(n)
+    compare(g, o, acc)
+    d = torch.from_numpy(acc.view(np.int64).reshape(-1)).cuda()
+    comp, stall = (torch.full((n,), -1, dtype=torch.int64, device="cuda") for _ in range(2))
+    g.force_mode(2, 1_000_000)
+    assert g.submit_batch_paged(d, n, 4 * n, comp, stall) == 0 and g.last_result()["code"] == hbf.E_THROTTLED
+    assert not comp.any() and not stall.any()
