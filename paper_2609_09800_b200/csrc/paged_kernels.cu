@@ -295,7 +295,8 @@ cudaError_t launch_paged_count(const hbf_access_t *acc, uint64_t n, const RangeS
     cudaError_t e = cudaMemsetAsync(pw.total, 0, sizeof(PagedSums) + kPagedTotals * 8, st);
     if (e != cudaSuccess) return e;
     const unsigned grid = (unsigned)std::min<uint64_t>(tiles, 148u * 16u);
-    const int64_t unit_ns = std::max(mp.t_read_ns, mp.t_prog_ns) > (1ll << 40) ? (1ll << 40) : std::max(mp.t_read_ns, mp.t_prog_ns) << mp.pages_per_stripe_shift;
+    // (any time from 2^33 ns on is too long: no larger one is formed)
+    const int64_t page_ns = std::max(mp.t_read_ns, mp.t_prog_ns), unit_ns = page_ns >= (1ll << 33) >> mp.pages_per_stripe_shift ? 1ll << 33 : page_ns << mp.pages_per_stripe_shift;
     auto k = fast.on ? (by_unit ? k_paged_count<true, true> : k_paged_count<true, false>) : (by_unit ? k_paged_count<false, true> : k_paged_count<false, false>);
     k<<<grid, kPgThreads, 0, st>>>(acc, n, ranges, fast, mp.page_shift, mp.stripe_shift, unit_ns, state, pw.tile_sum, pw.row_off, pw.total);
     g_kernel_launches += 1;

@@ -227,3 +227,17 @@ def test_a_throttled_paged_batch_leaves_zeros(hbf, n, cross):
     g.force_mode(2, 1_000_000)
     assert g.submit_batch_paged(d, n, 4 * n, comp, stall) == 0 and g.last_result()["code"] == hbf.E_THROTTLED
     assert not comp.any() and not stall.any()
+
+
+def test_a_stripe_unit_of_pages_whose_service_passes_64_bits(hbf):
+    """2^30 pages of one byte per stripe unit at 17 s each: the time of a whole unit has no place in 64 bits, a batch of
+    accesses of a few bytes is served all the same."""
+    n = 9_000
+    prof = wl.load_profile("nominal", channels=2, dies=1, planes=1, page_bytes=1, stripe_bytes=1 << 30)
+    prof.update(t_read_ns=1 << 34)
+    g, o = contexts(hbf, prof, [(wl.RANGE_BASE, 1 << 34, 3, 0, 0, 0)])
+    acc = np.zeros(n, hbfo.ACCESS_DTYPE)
+    acc["addr"] = wl.RANGE_BASE + np.random.default_rng(0).integers(0, 1 << 33, n).astype(np.uint64)
+    acc["bytes"] = 1 + np.arange(n) % 3
+    acc["issue_ns"] = np.arange(n)
+    compare(g, o, acc, page=1)
