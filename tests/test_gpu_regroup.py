@@ -74,3 +74,27 @@ def test_the_served_order_after_batches_of_other_routes(hbf, reset):
             assert np.array_equal(g.queue_order(hi - lo, ws), o.last_order())       # (asking does not spoil it)
         if reset:
             g.reset(); o.reset()
+
+
+@pytest.mark.parametrize("n", [8_193, 100_003])
+@pytest.mark.parametrize("kind", ["any 64 bits", "both ends", "one negative sample", "one late sample"])
+def test_issue_times_outside_their_limits_are_refused(hbf, kind, n):
+    """Records that the begin kernel's samples hold: their span has no place in the arithmetic that spreads a batch."""
+    w = wl.capacity_mode(n=n, seed=n, rho=0.6)
+    g, o = hbf.Context(w.profile), hbfo.Oracle(w.profile)
+    for r in w.ranges:
+        g.register_range(*r); o.register_range(*r)
+    rng = np.random.default_rng(n)
+    good = w.acc[rng.permutation(n)]
+    acc = good.copy()
+    if kind == "any 64 bits": acc["issue_ns"] = rng.integers(-(1 << 63), (1 << 63) - 1, n, endpoint=True)
+    if kind == "both ends": acc["issue_ns"][[0, 1]] = (1 << 63) - 1, -(1 << 63)
+    if kind == "one negative sample": acc["issue_ns"][0] = -1
+    if kind == "one late sample": acc["issue_ns"][0] = 1 << 47
+    bad = (acc["issue_ns"] < 0) | (acc["issue_ns"] >= 1 << 47)
+    rc, c, s, st, ds = g.submit_host(acc, check=False)
+    assert rc == hbfo.E_ACCESS_FAULT and g.last_result()["n_fault"] == int(bad.sum()) and not c.any() and not s.any()
+    assert np.array_equal(st, np.where(bad, 4, 1)) and not g.get_busy_until().any()      # 4: unsupported, 1: modeled
+    _, c_o, s_o, *_ = o.submit(good)
+    _, c, s, *_ = g.submit_host(good)
+    assert np.array_equal(c, c_o) and np.array_equal(s, s_o)
