@@ -8,7 +8,10 @@
 #include <type_traits>
 #include <vector>
 
+#include <cuda.h>
+
 #include "hbf_dev.cuh"
+#include "host_write.h"
 
 using namespace hbf;
 
@@ -540,6 +543,23 @@ int hbf_submit_batch(hbf_ctx *c, const hbf_access_t *d_acc, uint64_t n, int64_t 
 }
 
 constexpr uint64_t kHostResultsMax = 65536;                  // records
+// whether the current device's kernels may write this host buffer (see host_write.h); asked on every call
+static bool kernel_may_write(const void *at, size_t bytes) {
+    using Ask = CUresult (*)(unsigned, CUpointer_attribute *, void **, CUdeviceptr);
+    static const Ask ask = [] {
+        void *f = nullptr;
+        cudaDriverEntryPointQueryResult found;
+        if (cudaGetDriverEntryPointByVersion("cuPointerGetAttributes", &f, 12000, cudaEnableDefault, &found) != cudaSuccess || found != cudaDriverEntryPointSuccess) f = nullptr;
+        return reinterpret_cast<Ask>(f);
+    }();
+    if (!ask) return false;
+    uint64_t type = 0, device = 0, start = 0, size = 0, access = 0;       // (the enumerations take the lower half of theirs)
+    CUpointer_attribute what[5] = {CU_POINTER_ATTRIBUTE_MEMORY_TYPE, CU_POINTER_ATTRIBUTE_DEVICE_POINTER, CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, CU_POINTER_ATTRIBUTE_RANGE_SIZE,
+                                   CU_POINTER_ATTRIBUTE_ACCESS_FLAGS};
+    void *into[5] = {&type, &device, &start, &size, &access};
+    if (ask(5, what, into, (CUdeviceptr)(uintptr_t)at) != CUDA_SUCCESS) return false;
+    return device_may_write(HostMemory{(uint32_t)type, device, start, (size_t)size, access}, at, bytes);
+}
 // Host-buffer submit: the batch is cut into chunks; the copy-in of chunk k+1, the service of chunk k (hbf_submit_batch)
 // and the read-back of chunk k-1 run on three streams, so the link moves both ways while the kernels run.
 // (what only several chunks need, the streams and the second set of buffers, is made when a call first has several)
@@ -609,18 +629,9 @@ int hbf_submit_host(hbf_ctx *c, const hbf_access_t *h_acc, uint64_t n, int64_t *
         // A small batch's results leave in one kernel where the device can write the caller's buffers (pinned memory): four
         // copies cost more than the bytes.  The call as a whole with copies and so: 2,000 records 44 and 33 us, 5,900 48 and
         // 39, 16,384 107 and 95, 65,536 218 and 160; at 262,144 the two are alike.
-        int64_t *dev[3] = {nullptr, nullptr, nullptr};
-        void *const host[3] = {h_completion_ns, h_stall_ns, h_die_stats};
-        bool writable = n <= kHostResultsMax;
-        for (int k = 0; k < 3 && writable; ++k) {
-            cudaPointerAttributes at;
-            if (!host[k]) continue;
-            writable = cudaPointerGetAttributes(&at, host[k]) == cudaSuccess && at.type == cudaMemoryTypeHost && at.devicePointer;
-            dev[k] = static_cast<int64_t *>(at.devicePointer);
-        }
-        if (!writable) (void)cudaGetLastError();
-        if (writable) {
-            CK(launch_host_results(p.comp[0], p.stall[0], p.stats, c->d_result, n, c->mp.n_dies, dev[0], dev[1], reinterpret_cast<hbf_die_stats_t *>(dev[2]), p.h_sum,
+        if (n <= kHostResultsMax && kernel_may_write(h_completion_ns, n * 8) && kernel_may_write(h_stall_ns, n * 8) &&
+            (!h_die_stats || kernel_may_write(h_die_stats, (size_t)c->mp.n_dies * sizeof(hbf_die_stats_t)))) {
+            CK(launch_host_results(p.comp[0], p.stall[0], p.stats, c->d_result, n, c->mp.n_dies, h_completion_ns, h_stall_ns, h_die_stats, p.h_sum,
                                    &c->plain_next, main));
         } else {
             CK(cudaMemcpyAsync(h_completion_ns, p.comp[0], n * 8, cudaMemcpyDeviceToHost, main));

@@ -551,3 +551,20 @@ def test_a_throttled_call_from_the_host_leaves_zeros(hbf, pin, chunk):
             assert rc == hbf.E_THROTTLED and summary["code"] == rc and summary["n_modeled"] == 0
             assert not any(t.any() for t in out)
             assert np.array_equal(g.get_busy_until(), busy)
+
+
+@pytest.mark.parametrize("n", [257, 9_000])
+@pytest.mark.parametrize("which", [0, 1, 2])
+def test_pinned_results_at_an_odd_address(hbf, which, n):
+    """Completions, stalls or statistics four bytes off their alignment: copied, as before there was a kernel that writes them."""
+    import ctypes as C
+    import torch
+    w = wl.capacity_mode(n=n, seed=n)
+    g, o = contexts(hbf, w.profile, w.ranges)
+    _, c_o, s_o, _, ds_o = o.submit(w.acc)
+    rec = torch.from_numpy(w.acc.view(np.int64).reshape(-1)).pin_memory()
+    raw = [torch.zeros(k * 8 + 8, dtype=torch.uint8).pin_memory() for k in (n, n, g.n_dies * 6)]
+    at = [t.data_ptr() + (4 if k == which else 0) for k, t in enumerate(raw)]
+    assert hbf.lib().hbf_submit_host(g._h, rec.data_ptr(), n, at[0], at[1], at[2], 0, None) == 0
+    got = [t.numpy()[4 if k == which else 0:][:-8 if k != which else -4].copy().view(np.int64) for k, t in enumerate(raw)]
+    assert np.array_equal(got[0], c_o) and np.array_equal(got[1], s_o) and np.array_equal(got[2], ds_o.view(np.int64))
