@@ -4,6 +4,7 @@
 #include <cmath>
 #include <cstdlib>
 #include <cstring>
+#include <mutex>
 #include <new>
 #include <type_traits>
 #include <vector>
@@ -29,6 +30,36 @@ struct StateHeader {            // hbf_get_state / hbf_set_state blob header
 constexpr uint32_t kStateBus = 1u, kStateBins = 2u, kStateRetention = 4u;
 constexpr uint32_t kStateMagic = 0x48424631u;   // "HBF1"
 
+// What the library's kernels on one stream have to know of one another.  A kernel that may overlap its predecessor must not follow
+// one that may launch others from the device (see launch_first); that is a matter of the stream, not of the context: two contexts may
+// share one, and what they hold besides (a workspace, a batch's results read by the next).  A note per stream in use, shared by its
+// contexts, gone with the last of them.
+struct StreamNote {
+    int device; cudaStream_t stream;
+    int contexts = 0;
+    std::mutex launching;                        // held over one call's launches: another thread's call comes before or behind all of them
+    bool plain_next = false;                     // what was enqueued last may launch kernels of its own
+};
+std::mutex g_notes_mu;
+std::vector<StreamNote *> g_notes;
+StreamNote *take_note(int device, cudaStream_t st) {
+    if (st == cudaStreamLegacy) st = nullptr;
+    std::lock_guard<std::mutex> lock(g_notes_mu);
+    for (StreamNote *n : g_notes) if (n->device == device && n->stream == st) { n->contexts += 1; return n; }
+    StreamNote *n = new (std::nothrow) StreamNote();
+    if (!n) return nullptr;
+    n->device = device; n->stream = st; n->contexts = 1;
+    g_notes.push_back(n);
+    return n;
+}
+void give_note(StreamNote *n) {
+    if (!n) return;
+    std::lock_guard<std::mutex> lock(g_notes_mu);
+    if (--n->contexts) return;
+    g_notes.erase(std::find(g_notes.begin(), g_notes.end(), n));
+    delete n;
+}
+
 }  // namespace
 
 struct hbf_rom;
@@ -50,7 +81,7 @@ struct hbf_ctx {
     struct Pinned { hbf_batch_result_t result, host_sum; RetState ret; unsigned long long ret_waiting; unsigned long long totals[kPagedTotals]; float hot[4]; TileBalance bal; } *pinned = nullptr;
     bool result_on_host = false;                 // pinned->result is the last batch's summary (small batches leave theirs on the device only)
     bool captured = false;                       // a batch was captured into a graph: which batch ran last is not for the host to know
-    bool plain_next = false;                     // what was enqueued last may launch kernels of its own: see launch_first
+    StreamNote *note = nullptr;                  // of the stream
     TileBalanceHost bal;                         // tile sizes of the in-order path from the times earlier batches left
     // thermal steps on a reduced-order model instead of the grid (off while rom == nullptr)
     hbf_rom *rom = nullptr; int64_t rom_dt_ns = 0; int32_t *d_rom_kind = nullptr; double *d_rom_T = nullptr;
@@ -274,6 +305,7 @@ int hbf_destroy(hbf_ctx *c) {
         cudaStreamDestroy(p.s_in); cudaStreamDestroy(p.s_out);
     }
     cudaFree(p.ws); cudaFree(p.stats);
+    give_note(c->note);                                      // (the stream has been waited for)
     delete c;
     return HBF_OK;
 }
@@ -296,6 +328,7 @@ int hbf_create(const hbf_config_t *cfg, void *cuda_stream, hbf_ctx **out) {
     int rc = HBF_OK;
     auto fail = [&](int code) { hbf_destroy(c); return code; };
     if (cudaGetDevice(&c->device) != cudaSuccess) return fail(HBF_E_CUDA);
+    if (!(c->note = take_note(c->device, c->stream))) return fail(HBF_E_NOMEM);
     if (cudaDeviceGetAttribute(&c->sm_count, cudaDevAttrMultiProcessorCount, c->device) != cudaSuccess) return fail(HBF_E_CUDA);
     Arena arena;
 
@@ -478,12 +511,26 @@ static bool capturing(cudaStream_t st) {
     return s != cudaStreamCaptureStatusNone;
 }
 
+// One call's launches: holds the stream's note meanwhile.  What is being captured does not run behind what the stream was given
+// last, and the per-thread default stream is another one in every thread: such a call begins with an ordinary launch.
+class Launching {
+    std::lock_guard<std::mutex> lock_;
+    bool own_ = true;
+public:
+    const bool captured;
+    bool *const plain_next;
+    explicit Launching(hbf_ctx *c) : lock_(c->note->launching), captured(capturing(c->stream)),
+        plain_next(captured || c->stream == cudaStreamPerThread ? &own_ : &c->note->plain_next) {}
+};
+
 // Everything a batch of records goes through once its arguments are in place: the claim window (retention), the submit
 // path, the energy ledger, read disturb / commits, the channel-bus stage.  Shared by hbf_submit_batch (the caller's
 // accesses) and hbf_submit_batch_paged (the list of parts).
 static int serve_records(hbf_ctx *c, SubmitArgs &a) {
+    Launching now(c);
+    if (now.captured) c->captured = true;
     a.ranges = c->d_ranges; a.mp_dev = c->d_mp; a.mp = c->mp; a.state = c->d_state; a.ctrl = c->d_ctrl; a.result = c->d_result;
-    a.result_host = &c->pinned->result; a.plain_next = &c->plain_next;
+    a.result_host = &c->pinned->result; a.plain_next = now.plain_next;
     a.busy = c->d_busy; a.busy_stage = c->d_busy_stage; a.pending = c->d_pending; a.stats_stage = c->d_stats_stage;
     a.path = a.paged ? (int32_t)HBF_PATH_INORDER : c->path; a.sm_count = c->sm_count; a.inorder_ok = c->inorder_ok ? 1 : 0;
     if (c->ranges.size() == 1) {
@@ -494,7 +541,6 @@ static int serve_records(hbf_ctx *c, SubmitArgs &a) {
     a.bal = &c->bal; a.rg_sync = c->d_rg_sync;
     if (c->ret_on) { a.claim_limit = &c->ret.st->claim_limit; a.die_claims = c->ret.die_claims; a.ret = &c->ret; }
     c->result_on_host = true;
-    if (capturing(c->stream)) c->captured = true;
     if (small_route(a)) {                                    // one launch, everything included (with the bus on it stops before the ledger)
         auto mark = [&](int k) { if (a.ev) cudaEventRecord(a.ev[k], c->stream); };
         mark(0); mark(7);
@@ -631,8 +677,9 @@ int hbf_submit_host(hbf_ctx *c, const hbf_access_t *h_acc, uint64_t n, int64_t *
         // 39, 16,384 107 and 95, 65,536 218 and 160; at 262,144 the two are alike.
         if (n <= kHostResultsMax && kernel_may_write(h_completion_ns, n * 8) && kernel_may_write(h_stall_ns, n * 8) &&
             (!h_die_stats || kernel_may_write(h_die_stats, (size_t)c->mp.n_dies * sizeof(hbf_die_stats_t)))) {
+            Launching now(c);
             CK(launch_host_results(p.comp[0], p.stall[0], p.stats, c->d_result, n, c->mp.n_dies, h_completion_ns, h_stall_ns, h_die_stats, p.h_sum,
-                                   &c->plain_next, main));
+                                   now.plain_next, main));
         } else {
             CK(cudaMemcpyAsync(h_completion_ns, p.comp[0], n * 8, cudaMemcpyDeviceToHost, main));
             CK(cudaMemcpyAsync(h_stall_ns, p.stall[0], n * 8, cudaMemcpyDeviceToHost, main));
@@ -822,8 +869,9 @@ int hbf_retention_advance(hbf_ctx *c, int64_t dt_ns, const double *region_temp_c
     if (!region_temp_c && (!c->thermal || c->rom)) return HBF_E_INVAL;      // no field to read the temperatures from
     if (region_temp_c)                                                      // pageable source: staged before the call returns
         CK(cudaMemcpyAsync(c->ret.region_temp, region_temp_c, c->ret.n_regions * sizeof(double), cudaMemcpyHostToDevice, c->stream));
+    Launching now(c);
     CK(launch_ret_advance(c->ret, c->mp, c->thermal ? &c->td : nullptr, c->thermal ? c->td.theta[c->cur] : nullptr,
-                          c->thermal ? c->td.die_region : nullptr, region_temp_c ? 1 : 0, dt_ns, c->sm_count, &c->plain_next, c->stream));
+                          c->thermal ? c->td.die_region : nullptr, region_temp_c ? 1 : 0, dt_ns, c->sm_count, now.plain_next, c->stream));
     return HBF_OK;
 }
 
@@ -953,13 +1001,16 @@ int hbf_thermal_step(hbf_ctx *c, int64_t dt_ns, const float *ext_power_w, uint32
     unsigned long long *bin_row = nullptr;                   // the step is the bin the thermal clock stands in
     if (c->bin_ns) { bin_row = c->d_ledger + (size_t)(c->cur_bin % c->n_bins) * c->mp.n_dies; c->cur_bin += 1; }
     if (c->profiling) CK(cudaEventRecord(c->ev_th[0], c->stream));
+    {
+    Launching now(c);
     if (c->rom) {                                            // the attached model stands in for the grid
         if (bin_row) CK(launch_take_bin(bin_row, c->d_pending, c->mp.n_dies, c->stream));
         const hbf_rom &m = *c->rom;
         CK(launch_rom_window(m.n, m.m, m.o, m.A, m.B, m.b, m.C, m.D, m.d, m.x, c->d_rom_T + m.o, c->d_rom_T, reinterpret_cast<uint32_t *>(c->d_rom_T + m.o + m.n), td,
-                             c->d_pending, dt_ns, n_ext != 0, c->d_rom_kind, c->d_state, &c->plain_next, c->stream));
+                             c->d_pending, dt_ns, n_ext != 0, c->d_rom_kind, c->d_state, now.plain_next, c->stream));
     } else {
-        CK(launch_thermal_step(td, c->d_state, c->d_pending, bin_row, dt_ns, n_ext != 0, d_temps_out, &c->cur, c->thermal_generic ? 1 : 0, &c->plain_next, c->stream));
+        CK(launch_thermal_step(td, c->d_state, c->d_pending, bin_row, dt_ns, n_ext != 0, d_temps_out, &c->cur, c->thermal_generic ? 1 : 0, now.plain_next, c->stream));
+    }
     }
     if (c->profiling) { CK(cudaEventRecord(c->ev_th[1], c->stream)); c->prof_thermal = true; }
     if (hot_c_out) {
@@ -1025,7 +1076,8 @@ int hbf_reset(hbf_ctx *c) {
         c->cur = 0;
     }
     c->result_on_host = true;
-    CK(launch_reset(r, &c->plain_next, c->stream));          // one launch, in stream order: nothing waits for it here
+    Launching now(c);
+    CK(launch_reset(r, now.plain_next, c->stream));          // one launch, in stream order: nothing waits for it here
     c->terminal = false;
     return HBF_OK;
 }

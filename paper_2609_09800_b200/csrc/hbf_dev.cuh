@@ -158,14 +158,15 @@ inline cudaError_t launch_pdl(Kernel k, dim3 grid, dim3 block, size_t smem, cuda
     cfg.attrs = at; cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, k, args...);
 }
-// the first kernel of a call: the same, unless what the context enqueued last may still launch kernels of its own (*plain_next)
+// the first kernel of a call: the same, unless what was enqueued on the stream last may still launch kernels of its own (*plain_next)
 template <class Kernel, class... Args>
 inline cudaError_t launch_first(bool *plain_next, Kernel k, dim3 grid, dim3 block, size_t smem, cudaStream_t st, const Args &...args) {
     if (plain_next && *plain_next) {
-        *plain_next = false;
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = st;
-        return cudaLaunchKernelEx(&cfg, k, args...);
+        const cudaError_t e = cudaLaunchKernelEx(&cfg, k, args...);
+        if (e == cudaSuccess) *plain_next = false;
+        return e;
     }
     return launch_pdl(k, grid, block, smem, st, args...);
 }

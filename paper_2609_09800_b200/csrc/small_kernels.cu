@@ -527,9 +527,10 @@ cudaError_t launch_small(const SubmitArgs &a, const SmallExtras &x, cudaStream_t
     at[0].id = cudaLaunchAttributeClusterDimension; at[0].val.clusterDim.x = blocks; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
     at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization; at[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at; cfg.numAttrs = a.plain_next && *a.plain_next ? 1 : 2;      // (see launch_first)
-    if (a.plain_next) *a.plain_next = false;
     g_kernel_launches += 1;
-    return cudaLaunchKernelEx(&cfg, small_kernel(blocks, s.n, s.ledger || s.ret_on), s);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, small_kernel(blocks, s.n, s.ledger || s.ret_on), s);
+    if (e == cudaSuccess && a.plain_next) *a.plain_next = false;
+    return e;
 }
 
 }  // namespace hbf

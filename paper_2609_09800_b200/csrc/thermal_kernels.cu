@@ -451,10 +451,10 @@ cudaError_t launch_thermal_step(const ThermalDev &t, DevState *state, int64_t *p
         at[0].id = cudaLaunchAttributeClusterDimension; at[0].val.clusterDim.x = blocks; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
         at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization; at[1].val.programmaticStreamSerializationAllowed = 1;
         cfg.attrs = at; cfg.numAttrs = *plain_next ? 1 : 2;   // (see launch_first)
-        *plain_next = false;
         float *theta = t.theta[*cur];
         const cudaError_t e = cudaLaunchKernelEx(&cfg, k, t, theta, state, pending, bin_row, dt_ns, has_ext, dt_sub_f, d_temps_out);
         if (e != cudaSuccess) return e;
+        *plain_next = false;
         g_kernel_launches += 1;
         return cudaGetLastError();
     }

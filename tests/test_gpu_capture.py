@@ -56,3 +56,29 @@ def test_the_summary_is_that_of_the_last_replay(hbf, n):
         _, c_o, s_o, *_ = t.o.submit(w.acc)
         assert t.g.last_result() == t.o.last_result()
         assert np.array_equal(t.comp.cpu().numpy(), c_o) and np.array_equal(t.stall.cpu().numpy(), s_o)
+
+
+@pytest.mark.parametrize("n", [4_000, 20_000])
+def test_a_capture_between_two_calls(hbf, n):
+    """The batch before it went to the sort kernels launched from the device: the call behind the capture follows that one."""
+    import torch
+    w = wl.capacity_mode(n=n, seed=n)
+    t = Captured(hbf, w.acc, w.profile, w.ranges)
+    wl_late = wl.capacity_mode(n=150_000, seed=1)
+    late = wl_late.acc.copy(); late[[70_000, 70_900]] = late[[70_900, 70_000]]
+    rec = torch.from_numpy(late.view(np.int64).reshape(-1).copy()).cuda()
+    comp, stall = (torch.empty(150_000, dtype=torch.int64, device="cuda") for _ in range(2))
+    ws = torch.empty(t.g.workspace_bytes(150_000), dtype=torch.uint8, device="cuda")
+    t.ws = ws
+    torch.cuda.synchronize()
+    for turn in range(3):
+        assert t.g.submit_batch(rec, 150_000, comp, stall, None, None, ws) == 0
+        t.o.submit(late)
+        t.graph = torch.cuda.CUDAGraph()
+        t.capture()
+        t.submit()
+        _, c_o, s_o, *_ = t.o.submit(w.acc)
+        assert t.g.last_result() == t.o.last_result() and np.array_equal(t.comp.cpu().numpy(), c_o) and np.array_equal(t.stall.cpu().numpy(), s_o)
+        t.replay()
+        _, c_o, *_ = t.o.submit(w.acc)
+        assert t.g.last_result() == t.o.last_result() and np.array_equal(t.comp.cpu().numpy(), c_o)

@@ -568,3 +568,38 @@ def test_pinned_results_at_an_odd_address(hbf, which, n):
     assert hbf.lib().hbf_submit_host(g._h, rec.data_ptr(), n, at[0], at[1], at[2], 0, None) == 0
     got = [t.numpy()[4 if k == which else 0:][:-8 if k != which else -4].copy().view(np.int64) for k, t in enumerate(raw)]
     assert np.array_equal(got[0], c_o) and np.array_equal(got[1], s_o) and np.array_equal(got[2], ds_o.view(np.int64))
+
+
+@pytest.mark.parametrize("second", ["small", "in order", "reset"])
+def test_two_contexts_on_one_stream_share_a_workspace(hbf, second):
+    """A batch that goes to the sort kernels launched from the device, and right behind it the other context's call, on the
+    same scratch memory: in stream order, so neither sees the other."""
+    import torch
+    n_a, n_b = 150_000, 6_000 if second == "small" else 60_000
+    st = torch.cuda.Stream()
+    wa, wb = wl.capacity_mode(n=n_a, seed=1), wl.capacity_mode(n=n_b, seed=2)
+    late = wa.acc.copy(); late[[70_000, 70_900]] = late[[70_900, 70_000]]              # out of order where the samples do not see it
+    sides = []
+    for w, acc in ((wa, late), (wb, wb.acc)):
+        g, o = hbf.Context(w.profile, stream=st), hbfo.Oracle(w.profile)
+        for r in w.ranges:
+            g.register_range(*r); o.register_range(*r)
+        sides.append((g, o, acc, torch.from_numpy(acc.view(np.int64).reshape(-1).copy()).cuda(), len(acc)))
+    ws = torch.empty(max(s[0].workspace_bytes(s[4]) for s in sides), dtype=torch.uint8, device="cuda")
+    turns = 6
+    out = [[[torch.empty(s[4], dtype=torch.int64, device="cuda") for _ in range(2)] for s in sides] for _ in range(turns)]
+    torch.cuda.synchronize()
+    for turn in range(turns):
+        for k, (g, o, acc, rec, n) in enumerate(sides):
+            if second == "reset" and k == 1:
+                g.reset(); o.reset()
+            assert g.submit_batch(rec, n, *out[turn][k], None, None, ws) == 0
+    torch.cuda.synchronize()
+    for turn in range(turns):
+        for k, (g, o, acc, rec, n) in enumerate(sides):
+            if second == "reset" and k == 1:
+                o.reset()
+            _, c_o, s_o, *_ = o.submit(acc)
+            assert np.array_equal(out[turn][k][0].cpu().numpy(), c_o) and np.array_equal(out[turn][k][1].cpu().numpy(), s_o)
+    for g, o, *_ in sides:
+        assert np.array_equal(g.get_busy_until(), o.busy_until()) and g.last_result() == o.last_result()
