@@ -14,7 +14,7 @@ struct BeginArgs {
 // took 2.7 of the 8.2 ms of 40 M shuffled records).  One pair each: one multiprocessor takes 4 us longer to fetch four.
 __device__ __forceinline__ bool begin_samples(const hbf_access_t *acc, uint64_t n, long long *lo, long long *hi) {
     const uint64_t *rec = reinterpret_cast<const uint64_t *>(acc + (uint64_t)threadIdx.x * (n - 1ull) / 1024ull);
-    const int64_t v0 = (int64_t)__ldg(rec + 1), v1 = (int64_t)__ldg(rec + 4), up = __shfl_up_sync(0xffffffffu, v0, 1);
+    const int64_t v0 = (int64_t)ld_after(rec + 1), v1 = (int64_t)ld_after(rec + 4), up = __shfl_up_sync(0xffffffffu, v0, 1);
     *lo = min(v0, v1); *hi = max(v0, v1);
     return __syncthreads_or(v1 < v0 || ((threadIdx.x & 31) != 0 && v0 < up)) != 0;
 }

@@ -30,8 +30,8 @@ struct BusRead { uint32_t channel, x; int64_t done; };
 __device__ __forceinline__ bool bus_read(const hbf_access_t *__restrict__ acc, const int64_t *__restrict__ completion, uint64_t i, const RangeSnap &rs, const ModelParams &mp,
                                          const FastRange &fast, bool fast_ok, BusRead *r) {
     const uint64_t *rec = reinterpret_cast<const uint64_t *>(acc + i);
-    const uint64_t addr = __ldg(rec), issue = __ldg(rec + 1), bf = __ldg(rec + 2);
-    const int64_t comp = __ldg(reinterpret_cast<const long long *>(completion + i));
+    const uint64_t addr = ld_after(rec), issue = ld_after(rec + 1), bf = ld_after(rec + 2);
+    const int64_t comp = ld_after(completion + i);
     uint32_t die;
     if (fast_ok) {
         const Served s = serve_terms_fast(fast, mp, addr, (int64_t)issue, bf);

@@ -33,6 +33,16 @@ __device__ __forceinline__ uint64_t ld_nc_u64(const uint64_t *p) {
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
+// What the kernel just before may have written (a caller's included), read behind pdl_wait by one that was launched to overlap it:
+// ordinary loads in their place.  A non-coherent load, which __ldg is and a load through a const __restrict__ pointer may become, is
+// promised data that does not change for as long as the kernel runs: it may be moved ahead of the wait.  (What was complete when this
+// kernel began needs none of this: every kernel of a chain lets the next one begin behind its own wait, so that is all but the last.)
+__device__ __forceinline__ uint32_t ld_after(const uint32_t *p) { uint32_t v; asm volatile("ld.global.u32 %0, [%1];" : "=r"(v) : "l"(p)); return v; }
+__device__ __forceinline__ float ld_after(const float *p) { float v; asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p)); return v; }
+__device__ __forceinline__ uint64_t ld_after(const uint64_t *p) { uint64_t v; asm volatile("ld.global.u64 %0, [%1];" : "=l"(v) : "l"(p)); return v; }
+__device__ __forceinline__ int64_t ld_after(const int64_t *p) { int64_t v; asm volatile("ld.global.s64 %0, [%1];" : "=l"(v) : "l"(p)); return v; }
+__device__ __forceinline__ longlong2 ld_after(const longlong2 *p) { longlong2 v; asm volatile("ld.global.v2.s64 {%0, %1}, [%2];" : "=l"(v.x), "=l"(v.y) : "l"(p)); return v; }
+
 // ---- division by a run-time constant ----------------------------------------------------------------
 // For d not a power of two, l = ceil(log2 d), magic = floor(2^(63+l) / d) + 1: floor(n / d) =
 // mulhi(n, magic) >> (l - 1) for every n < 2^63 (the error term n * (magic*d - 2^(63+l)) stays below 2^(63+l)).

@@ -245,7 +245,7 @@ __device__ __forceinline__ NarrowSums serve_narrow(const FastGeom &geom, const M
             if (j < tile_len) {
                 const uint64_t *rec = reinterpret_cast<const uint64_t *>(acc_t + j);
                 nx_addr[u] = __ldcs(rec); nx_issue[u] = __ldcs(rec + 1); nx_bf[u] = __ldcs(rec + 2);   // read once: streaming loads
-                if (!RESERVE) nx_prev[u] = j > 0u ? __ldg(reinterpret_cast<const uint32_t *>(rec - 2)) : (uint32_t)T0;   // (the tile's first record was compared before)
+                if (!RESERVE) nx_prev[u] = j > 0u ? ld_after(reinterpret_cast<const uint32_t *>(rec - 2)) : (uint32_t)T0;   // (the tile's first record was compared before)
             }
         }
     };
@@ -569,7 +569,7 @@ k_inorder_serve(const hbf_access_t *__restrict__ acc, uint64_t n, const __grid_c
         // The 32-bit form serves the tile when the configuration allows it, the tile's times lie within 2^31 ns and its read
         // granules sum below 2^32; should it turn out not to fit after all (a backlog), the 64-bit form below serves the tile again.
         int64_t T0 = 0, T1 = -1;
-        if (tile_len) { T0 = acc_t[0].issue_ns; T1 = acc_t[tile_len - 1u].issue_ns; }
+        if (tile_len) { T0 = ld_after(&acc_t[0].issue_ns); T1 = ld_after(&acc_t[tile_len - 1u].issue_ns); }
         if (geom.narrow != 0u && q_ppm == 1000000 && T0 >= 0 && T0 < HBF_ISSUE_LIMIT - (1ll << 32) && T1 >= T0 && T1 - T0 < (1ll << 31) &&
             (uint64_t)tile_len * geom.nw_gmax < (1ull << 32) && (uint64_t)quantum_ns < (1ull << (kNwServeBits - 1))) {
             uint4 *q4 = reinterpret_cast<uint4 *>(qst);
@@ -578,7 +578,7 @@ k_inorder_serve(const hbf_access_t *__restrict__ acc, uint64_t n, const __grid_c
             for (uint32_t q = tid; q < kInMaxQueues; q += kInThreads) {
                 uint4 v = make_uint4(0u, 0u, 0u, 0u);
                 if ((RESERVE || (MODE == kInFull && tile == 0u)) && q < R) {   // the first tile knows its entering state: it is served exactly
-                    const int64_t b = (RESERVE ? in_bin[(uint64_t)tile * R + q] : busy[q]) - T0;
+                    const int64_t b = (RESERVE ? ld_after(in_bin + (uint64_t)tile * R + q) : busy[q]) - T0;
                     v.x = b > 0 ? (uint32_t)b : 0u;
                     if (b >= (RESERVE ? 1ll << 30 : 1ll << 31)) over = 1u;
                 }
@@ -596,7 +596,7 @@ k_inorder_serve(const hbf_access_t *__restrict__ acc, uint64_t n, const __grid_c
                 if (nw.max_done) max_c = T0 + (int64_t)(uint64_t)nw.max_done;      // (a modeled access ends after its tile's first issue time)
                 if constexpr (!RESERVE) {
                     c_unsorted |= nw.unsorted;
-                    if (tid == 0 && tile_begin > 0 && acc_t[-1].issue_ns > T0) c_unsorted = 1u;
+                    if (tid == 0 && tile_begin > 0 && ld_after(&acc_t[-1].issue_ns) > T0) c_unsorted = 1u;
                     t_native = nw.native; t_fault = nw.fault; t_ready = (tid == 0 ? (long long)tile_len : 0ll) - t_native - t_fault;
                     longlong2 *out = reinterpret_cast<longlong2 *>(in_agg) + (uint64_t)tile * R;
                     for (uint32_t q = tid; q < R; q += kInThreads) {
@@ -622,7 +622,7 @@ k_inorder_serve(const hbf_access_t *__restrict__ acc, uint64_t n, const __grid_c
     for (uint32_t i = tid; i < kInMaxQueues; i += kInThreads) qst[i] = make_longlong2(kNegInf, 0);
     if (RESERVE) {
         __syncthreads();
-        for (uint32_t q = tid; q < R; q += kInThreads) qst[q].x = in_bin[(uint64_t)blockIdx.x * R + q];
+        for (uint32_t q = tid; q < R; q += kInThreads) qst[q].x = ld_after(in_bin + (uint64_t)blockIdx.x * R + q);
     } else {
         for (uint32_t d = tid; d < n_dies * 7u; d += kInThreads) st_br_lo[d] = 0u;
         if (MODE == kInFull && tile == 0u) {                 // the first tile knows its entering state: it is served exactly
@@ -656,7 +656,7 @@ k_inorder_serve(const hbf_access_t *__restrict__ acc, uint64_t n, const __grid_c
             if (j < tile_len) {
                 const uint64_t *rec = reinterpret_cast<const uint64_t *>(acc_t + j);
                 nx_addr[u] = __ldcs(rec); nx_issue[u] = __ldcs(rec + 1); nx_bf[u] = __ldcs(rec + 2);   // read once: streaming loads
-                if (!RESERVE) nx_prev[u] = (j > 0u || !first_tile) ? (int64_t)__ldg(rec - 2) : INT64_MIN;
+                if (!RESERVE) nx_prev[u] = (j > 0u || !first_tile) ? (int64_t)ld_after(rec - 2) : INT64_MIN;
             }
         }
     };
@@ -945,7 +945,7 @@ k_inorder_scan(BatchCtrl *ctrl, const ModelParams *__restrict__ mp, uint32_t n_t
     long long S = 0, M = kNegInf;                            // the run's own map
     if (live) {
         for (uint32_t t = t_lo; t < t_hi; ++t) {
-            const longlong2 v = agg[(uint64_t)t * R];
+            const longlong2 v = ld_after(agg + (uint64_t)t * R);
             M = max((int64_t)(M + v.x), (int64_t)v.y); S += v.x;
         }
     }
@@ -957,7 +957,7 @@ k_inorder_scan(BatchCtrl *ctrl, const ModelParams *__restrict__ mp, uint32_t n_t
         int64_t B = busy[r];
         for (uint32_t c = 0; c < chunk; ++c) { const longlong2 v = s_map[c][threadIdx.x]; B = max((int64_t)(B + v.x), (int64_t)v.y); }
         for (uint32_t t = t_lo; t < t_hi; ++t) {
-            const longlong2 v = agg[(uint64_t)t * R];
+            const longlong2 v = ld_after(agg + (uint64_t)t * R);
             in_bin[(uint64_t)t * R + r] = B;
             B = max((int64_t)(B + v.x), (int64_t)v.y);
         }
@@ -1089,7 +1089,7 @@ k_inorder_fixstraggle(const hbf_access_t *__restrict__ acc, uint64_t n, const __
         for (int k = 0; k < kInStrQueuesPerThread; ++k) {
             const uint32_t q = (uint32_t)(k * kInStrThreads + tid);
             c[k] = 0u; Bin[k] = kNegInf;
-            if (q < R) { c[k] = in_headcnt[(uint64_t)tile * R + q]; Bin[k] = in_bin[(uint64_t)tile * R + q]; }
+            if (q < R) { c[k] = in_headcnt[(uint64_t)tile * R + q]; Bin[k] = ld_after(in_bin + (uint64_t)tile * R + q); }
         }
 #pragma unroll
         for (int k = 0; k < kInStrQueuesPerThread; ++k)

@@ -91,7 +91,7 @@ k_begin_regroup(const __grid_constant__ BeginArgs b, const hbf_access_t *__restr
         }
         for (uint64_t s = (uint64_t)(k - zero_shares) * kShare + lane; s < min(samples, (uint64_t)(k - zero_shares + 1) * kShare); s += 32) {
             uint32_t off;
-            const uint32_t seg = rg_stretch((int64_t)__ldg(reinterpret_cast<const uint64_t *>(acc + s * n / samples) + 1), lo, shift, &off);
+            const uint32_t seg = rg_stretch((int64_t)ld_after(reinterpret_cast<const uint64_t *>(acc + s * n / samples) + 1), lo, shift, &off);
             atomicAdd(&sync->hist[seg], 1u); atomicMax(&sync->top[seg], off); atomicMax(&sync->below[seg], ~off);
         }
     });

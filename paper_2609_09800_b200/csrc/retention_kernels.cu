@@ -243,7 +243,7 @@ k_ret_region_max(const float *__restrict__ theta, const int32_t *__restrict__ ce
     pdl_trigger();
     for (uint64_t i = first; i - threadIdx.x % 32u < n_cells; i += stride) {     // (whole warps)
         if (i != first) g = i < n_cells ? cell_region[i] : -1;
-        const int v = g >= 0 ? ordered_int(__ldg(theta + i)) : 0;
+        const int v = g >= 0 ? ordered_int(ld_after(theta + i)) : 0;
         int32_t same;
         __match_all_sync(0xffffffffu, g, &same);             // cells side by side mostly lie in one region
         if (same) {

@@ -176,8 +176,8 @@ k_small_serve(const __grid_constant__ SmallArgs a) {
         addr[r] = bf[r] = 0ull; issue[r] = 0; prev[r] = INT64_MIN;
         if (i < end) {
             const uint64_t *rec = rec0 + (size_t)i * 3;
-            addr[r] = __ldg(rec); issue[r] = (int64_t)__ldg(rec + 1); bf[r] = __ldg(rec + 2);
-            if (lane == 0 && i > 0u) prev[r] = (int64_t)__ldg(rec - 2);
+            addr[r] = ld_after(rec); issue[r] = (int64_t)ld_after(rec + 1); bf[r] = ld_after(rec + 2);
+            if (lane == 0 && i > 0u) prev[r] = (int64_t)ld_after(rec - 2);
         }
     }
     int code = HBF_OK;
@@ -293,7 +293,7 @@ k_small_serve(const __grid_constant__ SmallArgs a) {
     if (code == HBF_OK) {
         // (the sizes come from the records again; they are needed once the list is served)
         uint64_t bf0 = 0ull;
-        if ((uint32_t)tid < m) bf0 = __ldg(rec0 + (size_t)((uint32_t)s_key[tid] & (kInSmallMax - 1u)) * 3 + 2);
+        if ((uint32_t)tid < m) bf0 = ld_after(rec0 + (size_t)((uint32_t)s_key[tid] & (kInSmallMax - 1u)) * 3 + 2);
         // ---- sort
         for (uint32_t p = (uint32_t)tid; p < m; p += kSmThreads) perm0[p] = (uint16_t)p;
         if (unsorted) {
@@ -365,7 +365,7 @@ k_small_serve(const __grid_constant__ SmallArgs a) {
                 if (EXTRA && a.ledger && !a.bus_on) {
                     const bool claim = (px >> 31) != 0u;
                     const int64_t own = s - (claim ? quantum_ns : 0), page = (int64_t)1 << mp.page_shift;
-                    const uint64_t gm = (1ull << (op ? mp.prog_gran_shift : mp.read_gran_shift)) - 1ull, cb = ((uint64_t)(uint32_t)__ldg(rec0 + (size_t)i * 3 + 2) + gm) & ~gm;
+                    const uint64_t gm = (1ull << (op ? mp.prog_gran_shift : mp.read_gran_shift)) - 1ull, cb = ((uint64_t)(uint32_t)ld_after(rec0 + (size_t)i * 3 + 2) + gm) & ~gm;
                     const uint32_t die = d_lo + lq / per_die;
                     const int64_t pj = op ? mp.e_cmd_prog_pj + mp.e_byte_prog_pj * (int64_t)cb : mp.e_cmd_read_pj + mp.e_byte_read_pj * (int64_t)cb;
                     if (claim) ledger_event(book, die, B - s, quantum_ns,
@@ -379,7 +379,7 @@ k_small_serve(const __grid_constant__ SmallArgs a) {
         if (lane == 0) { w_stall[warp] = sum_stall; w_max[warp] = max_c; }
         // ---- per-die totals (32-bit adds with a carry: a 64-bit one in shared memory is a loop)
         for (uint32_t p = (uint32_t)tid; p < m; p += kSmThreads) {
-            const uint64_t key = s_key[p], bfp = p < (uint32_t)kSmThreads ? bf0 : __ldg(rec0 + (size_t)((uint32_t)key & (kInSmallMax - 1u)) * 3 + 2);
+            const uint64_t key = s_key[p], bfp = p < (uint32_t)kSmThreads ? bf0 : ld_after(rec0 + (size_t)((uint32_t)key & (kInSmallMax - 1u)) * 3 + 2);
             const uint32_t op = (uint32_t)(key >> kSmIdxBits) & 1u, ld = s_lq[p] / per_die;
             const uint64_t gm = (1ull << (op ? mp.prog_gran_shift : mp.read_gran_shift)) - 1ull, cb = ((uint64_t)(uint32_t)bfp + gm) & ~gm, s = (uint64_t)s_s[p];
             auto add = [](uint32_t *lo, uint32_t *hi, uint64_t x) {

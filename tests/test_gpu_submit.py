@@ -603,3 +603,36 @@ def test_two_contexts_on_one_stream_share_a_workspace(hbf, second):
             assert np.array_equal(out[turn][k][0].cpu().numpy(), c_o) and np.array_equal(out[turn][k][1].cpu().numpy(), s_o)
     for g, o, *_ in sides:
         assert np.array_equal(g.get_busy_until(), o.busy_until()) and g.last_result() == o.last_result()
+
+
+@pytest.mark.parametrize("route", ["small", "small bus", "twice", "fix-up", "shuffled", "declared bus"])
+def test_records_written_by_the_kernel_just_before(hbf, route):
+    """One record buffer and one workspace, the records of every batch put there by a kernel of the caller's, nothing waited for:
+    the kernels that overlap their predecessors read what those left, batch after batch."""
+    import torch
+    n, turns = (4_000 if "small" in route else 40_000), 12
+    w = wl.capacity_mode(n=n * turns, seed=4, rho=0.7)
+    g, o = contexts(hbf, w.profile, w.ranges)
+    if "bus" in route:
+        g.enable_channel_bus(); o.enable_channel_bus()
+    if route == "declared bus":
+        g.set_path(hbf.PATH_INORDER)
+    if route == "fix-up":
+        g.set_head_entries(4)
+    rng = np.random.default_rng(0)
+    parts = [w.acc[k * n:(k + 1) * n] for k in range(turns)]
+    if route == "shuffled":
+        parts = [p[rng.permutation(n)] for p in parts]
+    every = [torch.from_numpy(p.view(np.int64).reshape(-1).copy()).cuda() for p in parts]
+    rec = torch.empty(3 * n, dtype=torch.int64, device="cuda")
+    out = [[torch.empty(n, dtype=torch.int64, device="cuda") for _ in range(2)] for _ in range(turns)]
+    ws = g.workspace(n)
+    torch.cuda.synchronize()
+    for k in range(turns):
+        torch.add(every[k], 0, out=rec)
+        assert g.submit_batch(rec, n, *out[k], None, None, ws) == 0
+    torch.cuda.synchronize()
+    for k in range(turns):
+        _, c_o, s_o, *_ = o.submit(parts[k])
+        assert np.array_equal(out[k][0].cpu().numpy(), c_o) and np.array_equal(out[k][1].cpu().numpy(), s_o)
+    assert np.array_equal(g.get_busy_until(), o.busy_until()) and g.last_result() == o.last_result()
