@@ -56,9 +56,9 @@ inline RegroupArgs regroup_args(uint64_t n, const Workspace &ws, RegroupSync *sy
 // another page (scatter 1,054 us for 40 M records, most of it address translation).
 __device__ __forceinline__ uint64_t rg_place(uint32_t buckets, uint32_t b, uint32_t p) { return ((uint64_t)(p >> 5) * buckets + b) * 32u + (p & 31u); }
 
-// the shares of a phase, taken by warps
+// the shares of a phase, taken by warps.  silent: a share that is not reported as done (test support: see hbf_debug_wait_test)
 template <class F>
-__device__ __forceinline__ void rg_shares(RegroupSync *s, int phase, uint32_t shares, F &&f) {
+__device__ __forceinline__ void rg_shares(RegroupSync *s, int phase, uint32_t shares, uint32_t silent, F &&f) {
     const int lane = threadIdx.x & 31;
     uint32_t done = 0;
     for (;;) {
@@ -67,7 +67,7 @@ __device__ __forceinline__ void rg_shares(RegroupSync *s, int phase, uint32_t sh
         k = __shfl_sync(0xffffffffu, k, 0);
         if (k >= shares) break;
         f(k);
-        ++done;
+        if (k != silent) ++done;
     }
     if (done) {
         __threadfence();
@@ -75,29 +75,38 @@ __device__ __forceinline__ void rg_shares(RegroupSync *s, int phase, uint32_t sh
         if (lane == 0) atomicAdd(&s->done[phase], done);
     }
 }
-// all shares of a phase are done; false: the wait ran out (the batch is given up, the context poisoned by its last kernel)
-__device__ __forceinline__ bool rg_wait(RegroupSync *s, int phase, uint32_t shares, BatchCtrl *ctrl) {
+constexpr uint32_t kRgNone = 0xffffffffu;
+// all shares of a phase are done; false: the wait ran out
+__device__ __forceinline__ bool rg_wait(RegroupSync *s, int phase, uint32_t shares, uint32_t limit) {
     bool ok = true;
     if (threadIdx.x == 0) {
         uint32_t polls = 0;
         while (ld_acquire_u32(&s->done[phase]) < shares) {
-            if (++polls > kSpinLimit) { ok = false; break; }
+            if (++polls > limit) { ok = false; break; }
             __nanosleep(64);
         }
-        if (!ok) { atomicExch(&ctrl->code, (int)HBF_E_TIMEOUT); ctrl->skip = 1; }
         __threadfence();
     }
     return __syncthreads_and(ok) != 0;
 }
+// the same in the begin kernel: a wait that runs out gives the batch up (its last kernel poisons the context)
+__device__ __forceinline__ bool rg_wait_or_give_up(RegroupSync *s, int phase, uint32_t shares, uint32_t limit, BatchCtrl *ctrl) {
+    const bool ok = rg_wait(s, phase, shares, limit);
+    if (!ok && threadIdx.x == 0) { atomicExch(&ctrl->code, (int)HBF_E_TIMEOUT); ctrl->skip = 1; }
+    return ok;
+}
 
-// the results of a regrouped batch back to batch order (blocks of the last kernel); false: a wait ran out
-__device__ __forceinline__ bool rg_give_back(const RegroupArgs &r, uint64_t n, BatchCtrl *ctrl, int64_t *__restrict__ completion, int64_t *__restrict__ stall) {
+// The results of a regrouped batch back to batch order (blocks of the last kernel).  Behind the one wait nothing can fail any more: the
+// block that takes the first output bucket calls commit() then, beside the others' work.  A block whose wait runs out leaves the rest
+// to those that got past it; true: this block is the last to leave, and none did (nothing was committed, no result given back).
+template <class Commit>
+__device__ __forceinline__ bool rg_give_back(const RegroupArgs &r, uint64_t n, const DevState *state, int64_t *__restrict__ completion, int64_t *__restrict__ stall, Commit &&commit) {
     __shared__ ulonglong2 s_out[kRgOut];
     __shared__ uint32_t s_b;
     constexpr uint32_t kGive = 1024;                         // records of a share
     const int tid = threadIdx.x, lane = tid & 31;
     const uint32_t gives = (uint32_t)((n + kGive - 1) / kGive);
-    rg_shares(r.sync, 3, gives, [&](uint32_t g) {
+    rg_shares(r.sync, 3, gives, state->test_stage == 2u ? state->test_tile : kRgNone, [&](uint32_t g) {
         for (uint32_t at0 = 0; at0 < kGive; at0 += 128u) {
             uint64_t comp[4], issue[4]; uint32_t idx[4], at[4];
             const uint64_t i0 = (uint64_t)g * kGive + at0 + lane;
@@ -117,13 +126,18 @@ __device__ __forceinline__ bool rg_give_back(const RegroupArgs &r, uint64_t n, B
         }
     });
     __syncthreads();
-    if (!rg_wait(r.sync, 3, gives, ctrl)) return false;
+    if (!rg_wait(r.sync, 3, gives, state->spin_limit)) {
+        if (tid == 0) { __threadfence(); s_b = atomicAdd(&r.sync->done[5], 1u); __threadfence(); }
+        __syncthreads();
+        return s_b == gridDim.x - 1u;
+    }
     for (;;) {
         __syncthreads();                                     // the results of the bucket before have been read
         if (tid == 0) s_b = atomicAdd(&r.sync->claim[4], 1u);
         __syncthreads();
         const uint32_t b = s_b;
-        if (b >= r.out_buckets) return true;
+        if (b >= r.out_buckets) return false;
+        if (b == 0u) commit();
         const uint64_t base = (uint64_t)b * kRgOut;
         const uint32_t m = (uint32_t)min((uint64_t)kRgOut, n - base);
 #pragma unroll 8

@@ -65,9 +65,11 @@ k_begin_regroup(const __grid_constant__ BeginArgs b, const hbf_access_t *__restr
     const bool sorted = bad && (first >= last || outside || (b.claim_limit && *b.claim_limit > 0ull)), go = bad && !sorted && !begin_refused(b.state);
     RegroupSync *sync = r.sync;
     BatchCtrl *ctrl = b.ctrl;
+    const uint32_t limit = b.state->spin_limit;
     if (blockIdx.x == 0) {
         begin_batch(b, sorted ? 1 : 0, go ? 1u : 0u);
-        if (tid < 2) { sync->claim[3 + tid] = 0u; sync->done[3 + tid] = 0u; }        // (those of the last kernel)
+        if (tid < 2) sync->claim[3 + tid] = 0u;              // (those of the last kernel)
+        if (tid < 3) sync->done[3 + tid] = 0u;
         __threadfence();
         __syncthreads();
         if (tid == 0 && go) atomicAdd(&sync->done[0], 1u);
@@ -84,7 +86,7 @@ k_begin_regroup(const __grid_constant__ BeginArgs b, const hbf_access_t *__restr
     const uint32_t sample_shares = (uint32_t)((samples + kShare - 1) / kShare);
     const uint64_t zeros = ((uint64_t)r.max_buckets + r.out_buckets) * kRgPad;
     const uint32_t zero_shares = (uint32_t)((zeros + kZero - 1) / kZero);
-    rg_shares(sync, 0, sample_shares + zero_shares, [&](uint32_t k) {
+    rg_shares(sync, 0, sample_shares + zero_shares, kRgNone, [&](uint32_t k) {
         if (k < zero_shares) {
             for (uint64_t i = (uint64_t)k * kZero + lane; i < min(zeros, (uint64_t)(k + 1) * kZero); i += 32) r.cursor[i] = 0u;
             return;
@@ -96,7 +98,7 @@ k_begin_regroup(const __grid_constant__ BeginArgs b, const hbf_access_t *__restr
         }
     });
     __syncthreads();
-    if (!rg_wait(sync, 0, sample_shares + zero_shares + 1u, ctrl)) return;
+    if (!rg_wait_or_give_up(sync, 0, sample_shares + zero_shares + 1u, limit, ctrl)) return;
     if (warp == 0) {
         const uint64_t want = n / kRgAvg, whole = (uint64_t)1 << min(shift, 32u);
         uint32_t nb[2], sum = 0;
@@ -131,7 +133,7 @@ k_begin_regroup(const __grid_constant__ BeginArgs b, const hbf_access_t *__restr
     // ---- scatter: a warp takes 1,024 records, 128 at a time
     constexpr uint32_t kScatter = 1024;
     const uint32_t scatters = (uint32_t)((n + kScatter - 1) / kScatter);
-    rg_shares(sync, 1, scatters, [&](uint32_t g) {
+    rg_shares(sync, 1, scatters, b.state->test_stage == 1u ? b.state->test_tile : kRgNone, [&](uint32_t g) {
         for (uint32_t at0 = 0; at0 < kScatter; at0 += 128u) {
             uint64_t addr[4], issue[4], bf[4];
             uint32_t at[4], bucket[4];
@@ -177,12 +179,12 @@ k_begin_regroup(const __grid_constant__ BeginArgs b, const hbf_access_t *__restr
         }
     });
     __syncthreads();
-    if (!rg_wait(sync, 1, scatters, ctrl)) return;
+    if (!rg_wait_or_give_up(sync, 1, scatters, limit, ctrl)) return;
     if (ld_relaxed_u32(&ctrl->run_sort)) return;             // a bucket overflowed (settled: the same for every block)
 
     // ---- offsets: where a bucket begins among its chunk of 1,024, and the chunks' sums
     const uint32_t chunks = (buckets + kRgChunk - 1u) / kRgChunk;
-    rg_shares(sync, 2, chunks, [&](uint32_t c) {
+    rg_shares(sync, 2, chunks, kRgNone, [&](uint32_t c) {
         uint32_t run = 0;
         for (uint32_t k = 0; k < kRgChunk; k += 256u) {
             uint32_t v[8];
@@ -201,7 +203,7 @@ k_begin_regroup(const __grid_constant__ BeginArgs b, const hbf_access_t *__restr
         if (lane == 0) r.part[c] = run;
     });
     __syncthreads();
-    if (!rg_wait(sync, 2, chunks, ctrl)) return;
+    if (!rg_wait_or_give_up(sync, 2, chunks, limit, ctrl)) return;
     uint32_t *s_part = reinterpret_cast<uint32_t *>(rg_smem + kRgGroups * kRgGroupSmem);
     if (warp == 0) {
         uint32_t run = 0;

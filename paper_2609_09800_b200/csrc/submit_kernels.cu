@@ -682,17 +682,21 @@ k_stalls(const hbf_access_t *__restrict__ acc, uint64_t n, const BatchCtrl *ctrl
 // =====================================================================================================
 // finish: commit the staged state, or zero the outputs of a refused batch; write the batch summary
 // =====================================================================================================
-__device__ __forceinline__ int finish_batch(const FinishArgs &f, long long modeled) {
+// What became of the batch, once its kernels are done: every thread reads the same settled values and takes the same decision.
+// With the channel-bus stage on, array-done times become sort keys of 47 bits: a batch that reaches 2^47 ns is refused here, before
+// anything is committed (every array-done time is at most the largest completion).
+__device__ __forceinline__ int batch_code(const FinishArgs &f) {
+    const BatchCtrl *ctrl = f.ctrl;
+    const int code = ctrl->code;
+    if (code != HBF_OK) return code;
+    if (ctrl->skip) return HBF_E_TIMEOUT;                    // (given up by a block whose wait ran out while the block was still being cleared)
+    return f.bus_on && ctrl->n_ready && ctrl->max_completion_ns >= HBF_ISSUE_LIMIT ? HBF_E_INVAL : HBF_OK;
+}
+// (on the whole grid, or on one block: gtid and gsz)
+__device__ __forceinline__ void finish_batch(const FinishArgs &f, long long modeled, int code, uint64_t gtid, uint64_t gsz) {
     BatchCtrl *ctrl = f.ctrl;
     const uint64_t n = f.n;
-    int code = ctrl->code;
-    // With the channel-bus stage on, array-done times become sort keys of 47 bits: a batch that reaches 2^47 ns is refused
-    // here, before anything is committed (every array-done time is at most the largest completion).  Every thread reads
-    // the same settled values, so every thread takes the same decision.
-    if (f.bus_on && code == HBF_OK && ctrl->n_ready && ctrl->max_completion_ns >= HBF_ISSUE_LIMIT) code = HBF_E_INVAL;
-    const uint64_t gtid = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (code == HBF_E_TIMEOUT && gtid == 0) f.state->poisoned = 1;       // a bounded device-side wait expired
-    const uint64_t gsz = (uint64_t)gridDim.x * blockDim.x;
     if (code == HBF_E_ACCESS_FAULT || code == HBF_E_TIMEOUT || code == HBF_E_INVAL) {
         for (uint64_t i = gtid; i < n; i += gsz) { f.completion[i] = 0; f.stall[i] = 0; }
         if (f.die_stats) for (uint64_t i = gtid; i < (uint64_t)f.n_dies * 6u; i += gsz) reinterpret_cast<int64_t *>(f.die_stats)[i] = 0;
@@ -700,7 +704,13 @@ __device__ __forceinline__ int finish_batch(const FinishArgs &f, long long model
         for (uint64_t i = gtid; i < n; i += gsz) { f.completion[i] = 0; f.stall[i] = 0; }
     } else if (code == HBF_OK) {
         const bool inorder = ctrl->inorder_used != 0u;
-        for (uint64_t r = gtid; r < f.n_queues; r += gsz) f.busy[r] = f.busy_stage[r];
+        for (uint64_t r = gtid; r < f.n_queues; r += 8u * gsz) {              // (loads side by side: a block by itself has eight queues per thread)
+            int64_t v[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) v[k] = r + k * gsz < f.n_queues ? f.busy_stage[r + k * gsz] : 0;
+#pragma unroll
+            for (int k = 0; k < 8; ++k) if (r + k * gsz < f.n_queues) f.busy[r + k * gsz] = v[k];
+        }
         for (uint64_t d = gtid; d < f.n_dies; d += gsz) {
             hbf_die_stats_t ds = f.stats_stage[d];
             // the in-order path keeps byte and access counts only: the energy is linear in them
@@ -721,7 +731,9 @@ __device__ __forceinline__ int finish_batch(const FinishArgs &f, long long model
         r.max_completion_ns = code == HBF_OK && ctrl->n_ready ? ctrl->max_completion_ns : 0;
         *f.result = r; *f.result_host = r;
     }
-    return code;
+}
+__device__ __forceinline__ void finish_batch(const FinishArgs &f, long long modeled) {
+    finish_batch(f, modeled, batch_code(f), (uint64_t)blockIdx.x * blockDim.x + threadIdx.x, (uint64_t)gridDim.x * blockDim.x);
 }
 __global__ void k_finish(const __grid_constant__ FinishArgs f) { finish_batch(f, f.ctrl->modeled_ns); }
 
@@ -1163,9 +1175,9 @@ __global__ void __launch_bounds__(256, 4) k_finish_inorder(const __grid_constant
     if (!MAY_SORT || c.ctrl->skip || c.ctrl->inorder_used) {
         // Stall total of the batch: per tile the exact sum if it was re-served, else the as-if sum plus its corrections
         __shared__ long long s_tot[8];
-        long long tot = 0;
-        if (blockIdx.x == 0) {
-            if (!c.ctrl->skip) for (uint32_t t = threadIdx.x; t < c.n_tiles; t += blockDim.x) {
+        auto stall_total = [&]() {                           // (whole block)
+            long long tot = 0;
+            for (uint32_t t = threadIdx.x; t < c.n_tiles; t += blockDim.x) {
                 const InTile v = c.in_tile[t];
                 tot += v.reserve ? v.true_sum : v.spec_sum + v.fix_delta;
             }
@@ -1174,13 +1186,18 @@ __global__ void __launch_bounds__(256, 4) k_finish_inorder(const __grid_constant
             __syncthreads();
             tot = 0;
             for (int w = 0; w < 8; ++w) tot += s_tot[w];
-        }
-        const int code = finish_batch(f, tot);
+            return tot;
+        };
         if constexpr (MAY_SORT) {
-            if (regrouped && code == HBF_OK && c.ctrl->inorder_used && !rg_give_back(rg, f.n, f.ctrl, f.completion, f.stall) && threadIdx.x == 0) {
-                f.state->poisoned = 1; f.result->code = HBF_E_TIMEOUT; f.result_host->code = HBF_E_TIMEOUT;
+            if (regrouped && batch_code(f) == HBF_OK) {      // (nothing is committed before every result can be given back)
+                if (rg_give_back(rg, f.n, f.state, f.completion, f.stall, [&] { finish_batch(f, stall_total(), HBF_OK, threadIdx.x, blockDim.x); })) {
+                    finish_batch(f, 0, HBF_E_TIMEOUT, threadIdx.x, blockDim.x);
+                    if (threadIdx.x == 0) { f.ctrl->code = HBF_E_TIMEOUT; f.ctrl->skip = 1; }
+                }
+                return;
             }
         }
+        finish_batch(f, blockIdx.x == 0 && !c.ctrl->skip ? stall_total() : 0);
         return;
     }
     if constexpr (MAY_SORT) { if (threadIdx.x == 0 && blockIdx.x == 0) launch_sort_chain(c, f, gridDim.x); }

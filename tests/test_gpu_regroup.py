@@ -98,3 +98,48 @@ def test_issue_times_outside_their_limits_are_refused(hbf, kind, n):
     _, c_o, s_o, *_ = o.submit(good)
     _, c, s, *_ = g.submit_host(good)
     assert np.array_equal(c, c_o) and np.array_equal(s, s_o)
+
+
+@pytest.mark.parametrize("n", [9_000, 100_003])
+@pytest.mark.parametrize("stage", [1, 2])
+def test_a_wait_that_runs_out_gives_the_batch_up(hbf, stage, n):
+    """One share of the records (or of the results) is silent (test support of the library: nothing stalls for real): outputs are
+    zeroed, queues and energies untouched, the context refuses batches until it is reset."""
+    w = wl.capacity_mode(n=n, seed=n, rho=0.6)
+    g, o = hbf.Context(w.profile), hbfo.Oracle(w.profile)
+    for r in w.ranges:
+        g.register_range(*r); o.register_range(*r)
+    acc = w.acc[np.random.default_rng(n).permutation(n)]
+    g.submit_host(w.acc[:5000]); o.submit(w.acc[:5000])
+    busy0, pend0 = g.get_busy_until(), g.get_pending_energy()
+    g.debug_wait_test(poll_limit=200, stage=stage, tile=3)
+    for silent in (True, False):                             # the switch off again: the context stays poisoned
+        rc, c, s, _, ds = g.submit_host(acc, check=False)
+        assert rc == hbf.E_TIMEOUT and not c.any() and not s.any() and not any(ds[f].any() for f in hbfo.DIE_STATS_DTYPE.names)
+        assert np.array_equal(g.get_busy_until(), busy0) and np.array_equal(g.get_pending_energy(), pend0)
+        with pytest.raises(hbf.HbfError):
+            g.queue_order(n)
+        g.debug_wait_test()
+    g.reset(); o.reset()
+    for _ in range(2):
+        _, c_o, s_o, _, ds_o = o.submit(acc)
+        _, c, s, _, ds = g.submit_host(acc)
+        assert np.array_equal(c, c_o) and np.array_equal(s, s_o) and all(np.array_equal(ds[f], ds_o[f]) for f in hbfo.DIE_STATS_DTYPE.names)
+        assert np.array_equal(g.get_busy_until(), o.busy_until()) and g.last_result() == o.last_result()
+        assert np.array_equal(g.queue_order(n), o.last_order())
+
+
+def test_a_bus_that_cannot_take_a_batch_out_of_order(hbf):
+    """Its last completion passes 2^47 ns: refused before anything is given back or committed."""
+    w = wl.capacity_mode(n=30_000, seed=9, rho=0.6)
+    g, o = hbf.Context(w.profile), hbfo.Oracle(w.profile)
+    for r in w.ranges:
+        g.register_range(*r); o.register_range(*r)
+    g.enable_channel_bus(); o.enable_channel_bus()
+    acc = w.acc[np.random.default_rng(3).permutation(30_000)]
+    late = acc.copy(); late["issue_ns"] += (1 << 47) - 1 - int(late["issue_ns"].max())
+    rc, c, s, _, ds = g.submit_host(late, check=False)
+    assert rc == -1 and not c.any() and not s.any() and not ds["n_read"].any() and not g.get_busy_until().any() and not g.get_bus_busy_until().any()
+    _, c_o, s_o, *_ = o.submit(acc)
+    _, c, s, *_ = g.submit_host(acc)
+    assert np.array_equal(c, c_o) and np.array_equal(s, s_o) and np.array_equal(g.get_bus_busy_until(), o.bus_busy_until())
