@@ -434,7 +434,8 @@ int hbf_create(const hbf_config_t *cfg, void *cuda_stream, hbf_ctx **out) {
     }
     if ((rc = arena.commit(c)) != HBF_OK) return fail(rc);
     mp.xfer_tab = tab_dev;
-    if (cudaMemcpy(c->d_mp, &mp, sizeof(mp), cudaMemcpyHostToDevice) != cudaSuccess) return fail(HBF_E_CUDA);
+    // (in the order of the context's stream, which need not wait for the default one)
+    if (cudaMemcpyAsync(c->d_mp, &mp, sizeof(mp), cudaMemcpyHostToDevice, c->stream) != cudaSuccess || cudaStreamSynchronize(c->stream) != cudaSuccess) return fail(HBF_E_CUDA);
     *out = c;
     return HBF_OK;
 }

@@ -636,3 +636,25 @@ def test_records_written_by_the_kernel_just_before(hbf, route):
         _, c_o, s_o, *_ = o.submit(parts[k])
         assert np.array_equal(out[k][0].cpu().numpy(), c_o) and np.array_equal(out[k][1].cpu().numpy(), s_o)
     assert np.array_equal(g.get_busy_until(), o.busy_until()) and g.last_result() == o.last_result()
+
+
+def test_a_context_is_whole_when_it_is_made(hbf):
+    """Made on a stream that does not wait for the default one, and used at once: a general geometry, whose kernels read its
+    parameters from memory."""
+    import torch
+    prof = wl.load_profile("nominal", channels=12, dies=3, planes=3, page_bytes=16384, stripe_bytes=65536)
+    rng = np.random.default_rng(0)
+    acc = np.zeros(3_000, hbfo.ACCESS_DTYPE)
+    acc["addr"] = wl.RANGE_BASE + rng.integers(0, 1 << 28, 3_000).astype(np.uint64)
+    acc["issue_ns"], acc["bytes"] = 100 * np.arange(3_000), 4096
+    rec = torch.from_numpy(acc.view(np.int64).reshape(-1).copy()).cuda()
+    o = hbfo.Oracle(prof); o.register_range(wl.RANGE_BASE, wl.GIB, 3, 0, 0, 0)
+    c_o = o.submit(acc)[1]
+    ws = torch.empty(1 << 24, dtype=torch.uint8, device="cuda")
+    st, comp, stall = torch.cuda.Stream(), *(torch.empty(3_000, dtype=torch.int64, device="cuda") for _ in range(2))
+    for path in (hbf.PATH_AUTO, hbf.PATH_SORT) * 6:
+        torch.cuda.synchronize()
+        g = hbf.Context(prof, stream=st)
+        g.register_range(wl.RANGE_BASE, wl.GIB, 3, 0, 0, 0); g.set_path(path)
+        assert g.submit_batch(rec, 3_000, comp, stall, None, None, ws) == 0 and g.last_result()["code"] == 0
+        assert np.array_equal(comp.cpu().numpy(), c_o)
