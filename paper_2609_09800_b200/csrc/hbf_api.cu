@@ -123,6 +123,15 @@ static Div64 make_div64_host(uint64_t d) {       // same construction as the dev
 // the context's device state, kernels' attributes and stream belong to the device it was created on
 static bool on_own_device(const hbf_ctx *c) { int d = -1; return cudaGetDevice(&d) == cudaSuccess && d == c->device; }
 
+// the context's device is current within the scope (for calls that any device may be current at: a kernel can only be launched on
+// a stream of the current one)
+class OnDevice {
+    int before_ = -1; bool moved_ = false;
+public:
+    explicit OnDevice(const hbf_ctx *c) { if (cudaGetDevice(&before_) == cudaSuccess && before_ != c->device) moved_ = cudaSetDevice(c->device) == cudaSuccess; }
+    ~OnDevice() { if (moved_) cudaSetDevice(before_); }
+};
+
 static bool is_pow2(uint64_t v) { return v && !(v & (v - 1)); }
 static uint32_t log2u(uint64_t v) { uint32_t s = 0; while ((1ull << s) < v) ++s; return s; }
 
@@ -916,6 +925,7 @@ int hbf_get_retention_plan(hbf_ctx *c, uint32_t *quanta, uint64_t cap, uint64_t 
 
 int hbf_get_retention_totals(hbf_ctx *c, hbf_retention_totals_t *out) {
     if (!c || !c->ret_on || !out) return HBF_E_INVAL;
+    OnDevice own(c);
     CK(launch_ret_totals(c->ret, c->sm_count, &c->pinned->ret, &c->pinned->ret_waiting, c->stream));
     CK(cudaStreamSynchronize(c->stream));
     const RetState &s = c->pinned->ret;
@@ -1077,6 +1087,7 @@ int hbf_reset(hbf_ctx *c) {
         c->cur = 0;
     }
     c->result_on_host = true;
+    OnDevice own(c);
     Launching now(c);
     CK(launch_reset(r, now.plain_next, c->stream));          // one launch, in stream order: nothing waits for it here
     c->terminal = false;

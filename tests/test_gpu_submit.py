@@ -658,3 +658,21 @@ def test_a_context_is_whole_when_it_is_made(hbf):
         g.register_range(wl.RANGE_BASE, wl.GIB, 3, 0, 0, 0); g.set_path(path)
         assert g.submit_batch(rec, 3_000, comp, stall, None, None, ws) == 0 and g.last_result()["code"] == 0
         assert np.array_equal(comp.cpu().numpy(), c_o)
+
+
+def test_reset_and_totals_with_another_device_current(hbf):
+    import torch
+    if torch.cuda.device_count() < 2:
+        pytest.skip("one device")
+    w = wl.tiny_uniform()
+    with torch.cuda.device(0):
+        g, o = contexts(hbf, w.profile, w.ranges)
+        g.enable_retention(pages_per_block=4, blocks_per_plane=8, blocks_per_zone=2, max_pec=3, disturb_limit=0,
+                           l_ref_s=1000.0, t_ref_c=40.0, ea_ev=1.04, accel=1.0, lead_threshold=0.5)
+        g.submit_host(w.acc)
+    with torch.cuda.device(1):
+        assert g.retention_totals()["n_blocks"] > 0
+        g.reset()
+        assert torch.cuda.current_device() == 1 and not g.get_busy_until().any()
+    with torch.cuda.device(0):
+        assert np.array_equal(g.submit_host(w.acc)[1], o.submit(w.acc)[1])
