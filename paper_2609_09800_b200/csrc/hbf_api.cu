@@ -548,7 +548,11 @@ static int serve_records(hbf_ctx *c, SubmitArgs &a) {
         a.fast.base = r.base; a.fast.length = r.length; a.fast.media_offset = r.media_offset; a.fast.perms = r.perms; a.fast.on = 1u;
     }
     a.binned = c->bin_ns != 0; a.bus_on = c->d_bus_busy ? 1 : 0;
-    a.bal = &c->bal; a.rg_sync = c->d_rg_sync;
+    // (a table of tile sizes is copied from the host: a replay would read it where it no longer is, so a captured batch takes the two
+    // nominal sizes)
+    TileBalanceHost nominal;
+    nominal.on = false; nominal.depth_fixed = c->bal.depth_fixed;
+    a.bal = now.captured ? &nominal : &c->bal; a.rg_sync = c->d_rg_sync;
     if (c->ret_on) { a.claim_limit = &c->ret.st->claim_limit; a.die_claims = c->ret.die_claims; a.ret = &c->ret; }
     c->result_on_host = true;
     if (small_route(a)) {                                    // one launch, everything included (with the bus on it stops before the ledger)

@@ -82,3 +82,30 @@ def test_a_capture_between_two_calls(hbf, n):
         t.replay()
         _, c_o, *_ = t.o.submit(w.acc)
         assert t.g.last_result() == t.o.last_result() and np.array_equal(t.comp.cpu().numpy(), c_o)
+
+
+@pytest.mark.parametrize("entries", [0, 4])
+def test_a_captured_batch_that_fills_a_wave(hbf, entries):
+    """Large enough for tile sizes from measurements, which come from the host: replays agree with a context that is not captured."""
+    import torch
+    n = 19_600_003
+    w = wl.capacity_mode(n=n, seed=7, rho=0.5)
+    t = Captured(hbf, w.acc, w.profile, w.ranges)
+    with torch.cuda.stream(t.stream):
+        other = hbf.Context(w.profile, stream=t.stream)
+    for r in w.ranges:
+        other.register_range(*r)
+    if entries:
+        t.g.set_head_entries(entries)
+    comp, stall = (torch.zeros(n, dtype=torch.int64, device="cuda") for _ in range(2))
+    torch.cuda.synchronize()
+    t.capture()
+    for turn in range(3):
+        t.replay()
+        assert other.submit_batch(t.acc, n, comp, stall, None, None, other.workspace(n)) == 0
+        torch.cuda.synchronize()
+        assert torch.equal(t.comp, comp) and torch.equal(t.stall, stall) and t.g.last_result() == other.last_result()
+        t.submit()                                          # and one that is not from the graph, on the queues the replay left
+        other.submit_batch(t.acc, n, comp, stall, None, None, other.workspace(n))
+        torch.cuda.synchronize()
+        assert torch.equal(t.comp, comp) and np.array_equal(t.g.get_busy_until(), other.get_busy_until())
