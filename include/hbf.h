@@ -35,7 +35,7 @@ enum {
     HBF_E_RANGE_OVERLAP = -2,  /* overlapping registration would make classification ambiguous (Design D1) */
     HBF_E_RANGE_FULL = -3,     /* more than HBF_MAX_RANGES ranges */
     HBF_E_CAPACITY = -4,       /* media_offset + length beyond capacity_bytes */
-    HBF_E_WORKSPACE = -5,      /* workspace smaller than hbf_workspace_bytes(n) or misaligned */
+    HBF_E_WORKSPACE = -5,      /* workspace too small (see hbf_workspace_bytes) or misaligned */
     HBF_E_CUDA = -6,           /* a CUDA runtime call failed */
     HBF_E_ACCESS_FAULT = -7,   /* >= 1 fail-closed access: batch refused, status[] filled, outputs zeroed, no state change */
     HBF_E_THROTTLED = -8,      /* mode Severe: new reservations withheld, no state change (Design D3) */
@@ -115,7 +115,10 @@ HBF_API int hbf_register_range(hbf_ctx *ctx, uint64_t base, uint64_t length, uin
                        uint32_t stream_tag, uint64_t media_offset, uint32_t *out_id);
 HBF_API int hbf_clear_ranges(hbf_ctx *ctx);
 
-/* Bytes of device scratch hbf_submit_batch needs for a batch of n accesses (256-byte aligned). */
+/* Bytes of device scratch for hbf_submit_batch of n accesses (256-byte aligned).  On the automatic path and above 8,192
+ * accesses that includes room to bring a batch out of issue order into order, some 80 bytes per access in all (2,048
+ * queues, 200 M accesses: 15.9 GB); with HBF_PATH_INORDER, or a sorting path, set it does not, some 36 bytes per access
+ * (7.1 GB).  A workspace of the smaller size is taken on every path: a batch out of issue order is then sorted. */
 HBF_API size_t hbf_workspace_bytes(const hbf_ctx *ctx, uint64_t n);
 
 /* Serves one batch, asynchronously on the context's stream.  For access i (its index plays the role
@@ -125,8 +128,8 @@ HBF_API size_t hbf_workspace_bytes(const hbf_ctx *ctx, uint64_t n);
  *   d_completion_ns[i], d_stall_ns[i] = completion - issue.  NATIVE rows: completion = issue, stall 0.
  * d_acc [n] device, read only, 8-byte aligned.  d_completion_ns, d_stall_ns [n] device.  d_status [n]
  * device, nullable.  d_die_stats [channels*dies] device, nullable, overwritten with this batch's totals.
- * d_workspace: device scratch of at least hbf_workspace_bytes(n), 256-byte aligned, must stay valid
- * until the batch has run.  The return value covers argument checks and launches only; the batch's
+ * d_workspace: device scratch of hbf_workspace_bytes(n), 256-byte aligned (less is taken down to the size described
+ * there), must stay valid until the batch has run.  The return value covers argument checks and launches only; the batch's
  * own outcome (access fault, throttled, shutdown, timeout) is read with hbf_last_result. */
 HBF_API int hbf_submit_batch(hbf_ctx *ctx, const hbf_access_t *d_acc, uint64_t n, int64_t *d_completion_ns,
                      int64_t *d_stall_ns, uint8_t *d_status, hbf_die_stats_t *d_die_stats,
@@ -177,13 +180,15 @@ HBF_API int hbf_submit_batch_paged(hbf_ctx *ctx, const hbf_access_t *d_acc, uint
  * transfer queues on the bus of the read's channel, first come first served in (array-done time, index) order
  * behind whatever earlier batches left there, and holds the bus for the transfer time; the read completes when its
  * transfer does.  Programs are unchanged (their transfer stays a latency before the array time), and so are the
- * queue state and the per-die statistics.  The stage runs inside hbf_submit_batch after the array stage (a radix
- * sort of the reads by channel and array-done time, then a segmented max-plus scan); hbf_workspace_bytes grows by
- * 4 bytes per access once it is on.  Array-done times are sort keys of 47 bits here (a restriction of this library, like
+ * queue state and the per-die statistics.  The stage runs inside hbf_submit_batch after the array stage: the reads go to
+ * buckets by slice of time and channel, each put in order and served by itself and then joined, or, where times bunch
+ * too tightly for that, through a radix sort by channel and array-done time and a segmented max-plus scan.  Once it is on,
+ * hbf_workspace_bytes holds 4 bytes per access more, and room for the buckets: some 48 bytes per access, part of which shares
+ * memory with what the batch needed before.  A workspace with the 4 bytes only is taken too (the radix sort then).  Array-done times are sort keys of 47 bits here (a restriction of this library, like
  * HBF_ISSUE_LIMIT): a batch whose largest completion time would reach 2^47 ns is refused with HBF_E_INVAL before anything
  * is committed (outputs zeroed, queue, bus and energy state unchanged); the context stays usable.
  * hbf_get_bus_busy_until synchronises and copies the per-channel bus state to host_out [channels]; hbf_reset clears
- * it.  With hbf_submit_batch_paged the stage queues parts (see there); its workspace then holds 4 bytes per part. */
+ * it.  With hbf_submit_batch_paged the stage queues parts (see there); its workspace then holds that per part. */
 HBF_API int hbf_enable_channel_bus(hbf_ctx *ctx);
 HBF_API int hbf_get_bus_busy_until(hbf_ctx *ctx, int64_t *host_out, uint64_t cap);
 

@@ -41,17 +41,18 @@ inline size_t bus_entry_bytes(uint64_t n, uint32_t channels) {
     const size_t buckets = (size_t)bus_slices(n, channels) * channels, a = (size_t)3 * n + 96 * buckets, b = (size_t)kBusCap * buckets;
     return (a < b ? a : b) * sizeof(ulonglong2);             // (at least buckets times places, and never less for more records)
 }
-inline size_t bus_plan_bytes(uint64_t n, uint32_t channels) {
-    return 8192 + (channels > kBusMaxChannels ? 0 : (size_t)bus_slices(n, channels) * channels * (kBusHead * sizeof(ulonglong2) + sizeof(BusState) + 8));
+inline size_t bus_head_bytes(uint64_t n, uint32_t channels) {
+    return channels > kBusMaxChannels ? 0 : (size_t)bus_slices(n, channels) * channels * (kBusHead * sizeof(ulonglong2) + sizeof(BusState) + 8);
 }
-static_assert(sizeof(BusPlan) <= 8192 && sizeof(BusPlan) % 4 == 0, "the plan's place");
-inline BusArgs bus_args(uint64_t n, uint32_t channels, const Workspace &ws, int64_t *busy) {
+static_assert(sizeof(BatchCtrl) <= kBusPlanAt && sizeof(BusPlan) <= kBusPlanBytes && sizeof(BusPlan) % 4 == 0, "the plan's place");
+inline BusPlan *bus_plan_of(BatchCtrl *bc) { return reinterpret_cast<BusPlan *>(reinterpret_cast<char *>(bc) + kBusPlanAt); }
+inline BusArgs bus_args(uint64_t n, uint32_t channels, const Workspace &ws, BatchCtrl *bc, int64_t *busy) {
     BusArgs b{};
-    b.plan = static_cast<BusPlan *>(ws.bus_plan); b.channels = channels; b.busy = busy;
-    if (channels > kBusMaxChannels) return b;               // slices = 0: the radix sort serves the batch
+    b.plan = bus_plan_of(bc); b.channels = channels; b.busy = busy;
+    if (!ws.bus_heads) return b;                            // slices = 0: the radix sort serves the batch
     b.slices = bus_slices(n, channels); b.cap = bus_cap(n, channels);
     const size_t buckets = (size_t)b.slices * channels;
-    b.heads = reinterpret_cast<ulonglong2 *>(static_cast<char *>(ws.bus_plan) + 8192);
+    b.heads = static_cast<ulonglong2 *>(ws.bus_heads);
     b.state = reinterpret_cast<BusState *>(b.heads + kBusHead * buckets);
     b.cursor = reinterpret_cast<uint32_t *>(b.state + buckets); b.redo = b.cursor + buckets;
     b.entries = static_cast<ulonglong2 *>(ws.rg_slots);

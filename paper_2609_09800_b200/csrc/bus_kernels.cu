@@ -480,7 +480,7 @@ k_bus_join(BatchCtrl *bc, const __grid_constant__ BusArgs b, int64_t *__restrict
 
 cudaError_t launch_bus_buckets(const SubmitArgs &a, BatchCtrl *bc, int64_t *bus_busy, cudaStream_t st) {
     const uint64_t n = a.n;
-    const BusArgs b = bus_args(n, a.mp.channels, a.ws, bus_busy);
+    const BusArgs b = bus_args(n, a.mp.channels, a.ws, bc, bus_busy);
     const int fast_ok = fast_geom_ok(a.fast, a.mp) ? 1 : 0;
     cudaError_t e = ensure_dyn_smem((const void *)k_bus_scatter, kBsSmem);
     if (e == cudaSuccess) e = ensure_dyn_smem((const void *)k_bus_order<false>, kBaSmem);

@@ -191,6 +191,16 @@ static int publish_ranges(hbf_ctx *c) {
     return HBF_OK;
 }
 
+// What a batch's workspace is asked to have room for, and what it has: a smaller one than asked for is taken too, down to what the
+// sort path needs (the sizes from before there were these arrays), and the batch then goes by the radix sort where they lack.
+static uint32_t rooms_wanted(const hbf_ctx *c) { return kRoomBus | (c->path == HBF_PATH_AUTO ? kRoomRegroup : 0u); }
+template <class Layout>
+static bool carve(const hbf_ctx *c, size_t bytes, Layout &&layout, uint32_t *rooms) {
+    for (const uint32_t r : {rooms_wanted(c), rooms_wanted(c) & kRoomBus, 0u})
+        if (layout(r) <= bytes) { *rooms = r; return true; }
+    return false;
+}
+
 extern "C" {
 
 // ---- reduced-order thermal model (Eq. 2) ----------------------------------------------------------------------
@@ -471,7 +481,7 @@ int hbf_clear_ranges(hbf_ctx *c) {
 
 size_t hbf_workspace_bytes(const hbf_ctx *c, uint64_t n) {
     if (!c) return 0;
-    return workspace_layout(n, c->mp.n_queues, c->mp.channels, nullptr, nullptr, c->d_bus_busy ? 1 : 0);
+    return workspace_layout(n, c->mp.n_queues, c->mp.channels, rooms_wanted(c), nullptr, nullptr, c->d_bus_busy ? 1 : 0);
 }
 
 int hbf_set_thermal_path(hbf_ctx *c, int32_t generic_only) {
@@ -590,8 +600,10 @@ int hbf_submit_batch(hbf_ctx *c, const hbf_access_t *d_acc, uint64_t n, int64_t 
     if ((reinterpret_cast<uintptr_t>(d_acc) & 7u) || (reinterpret_cast<uintptr_t>(d_completion_ns) & 7u) ||
         (reinterpret_cast<uintptr_t>(d_stall_ns) & 7u) || (reinterpret_cast<uintptr_t>(d_die_stats) & 7u)) return HBF_E_INVAL;
     SubmitArgs a{};
-    const size_t need = workspace_layout(n, c->mp.n_queues, c->mp.channels, &a.ws, d_workspace, c->d_bus_busy ? 1 : 0);
-    if (!d_workspace || workspace_bytes < need || (reinterpret_cast<uintptr_t>(d_workspace) & 255u)) return HBF_E_WORKSPACE;
+    uint32_t rooms = 0;
+    if (!d_workspace || (reinterpret_cast<uintptr_t>(d_workspace) & 255u) ||
+        !carve(c, workspace_bytes, [&](uint32_t r) { return workspace_layout(n, c->mp.n_queues, c->mp.channels, r, &a.ws, d_workspace, c->d_bus_busy ? 1 : 0); }, &rooms))
+        return HBF_E_WORKSPACE;
     a.acc = d_acc; a.n = n; a.completion = d_completion_ns; a.stall = d_stall_ns; a.status = d_status; a.die_stats = d_die_stats;
     c->prof_inorder = c->profiling && n > 0 && c->inorder_ok && (c->path == HBF_PATH_AUTO || c->path == HBF_PATH_INORDER);
     a.ev = c->profiling ? c->ev : nullptr;
@@ -744,7 +756,7 @@ int hbf_submit_host(hbf_ctx *c, const hbf_access_t *h_acc, uint64_t n, int64_t *
 
 size_t hbf_workspace_bytes_paged(const hbf_ctx *c, uint64_t n, uint64_t parts_capacity) {
     if (!c) return 0;
-    return paged_layout(n, std::max<uint64_t>(parts_capacity, n), c->mp.n_queues, c->mp.channels, nullptr, nullptr, c->d_bus_busy ? 1 : 0);
+    return paged_layout(n, std::max<uint64_t>(parts_capacity, n), c->mp.n_queues, c->mp.channels, rooms_wanted(c), nullptr, nullptr, c->d_bus_busy ? 1 : 0);
 }
 
 int hbf_submit_batch_paged(hbf_ctx *c, const hbf_access_t *d_acc, uint64_t n, uint64_t parts_capacity,
@@ -762,8 +774,10 @@ int hbf_submit_batch_paged(hbf_ctx *c, const hbf_access_t *d_acc, uint64_t n, ui
     const uint64_t capacity = std::min<uint64_t>(std::max<uint64_t>(parts_capacity, n), HBF_MAX_BATCH);
     PagedWorkspace pw{};
     const int with_bus = c->d_bus_busy ? 1 : 0;
-    const size_t need = paged_layout(n, capacity, c->mp.n_queues, c->mp.channels, &pw, d_workspace, with_bus);
-    if (!d_workspace || workspace_bytes < need || (reinterpret_cast<uintptr_t>(d_workspace) & 255u)) return HBF_E_WORKSPACE;
+    uint32_t rooms = 0;
+    if (!d_workspace || (reinterpret_cast<uintptr_t>(d_workspace) & 255u) ||
+        !carve(c, workspace_bytes, [&](uint32_t r) { return paged_layout(n, capacity, c->mp.n_queues, c->mp.channels, r, &pw, d_workspace, with_bus); }, &rooms))
+        return HBF_E_WORKSPACE;
     FastRange fast{};
     if (c->ranges.size() == 1) {
         const HostRange &r = c->ranges[0];
@@ -793,7 +807,7 @@ int hbf_submit_batch_paged(hbf_ctx *c, const hbf_access_t *d_acc, uint64_t n, ui
     c->prof_inorder = false; c->prof_submit = false;
     if (by_unit && total == n) {                             // no access crosses a stripe unit: the caller's records are the list
         SubmitArgs a{};
-        workspace_layout(n, c->mp.n_queues, c->mp.channels, &a.ws, pw.inner, 0);
+        workspace_layout(n, c->mp.n_queues, c->mp.channels, rooms, &a.ws, pw.inner, 0);
         a.acc = d_acc; a.n = n; a.completion = d_completion_ns; a.stall = d_stall_ns; a.status = d_status; a.die_stats = d_die_stats;
         a.paged = 1;
         if ((rc = serve_records(c, a)) != HBF_OK) return rc;
@@ -804,7 +818,7 @@ int hbf_submit_batch_paged(hbf_ctx *c, const hbf_access_t *d_acc, uint64_t n, ui
     CK(launch_paged_expand(d_acc, n, c->d_ranges, c->d_mp, fast, by_unit ? c->mp.stripe_shift : c->mp.page_shift, capacity, pw, c->sm_count, c->stream));
     // the list of parts is a batch of records like any other: the ledger, the bus stage and retention, when on, see parts
     SubmitArgs a{};
-    workspace_layout(total, c->mp.n_queues, c->mp.channels, &a.ws, pw.inner, with_bus);
+    workspace_layout(total, c->mp.n_queues, c->mp.channels, rooms, &a.ws, pw.inner, with_bus);
     a.acc = pw.parts; a.n = total; a.completion = pw.part_completion; a.stall = pw.part_stall; a.status = pw.part_status;
     a.die_stats = d_die_stats;
     a.paged = by_unit ? 1 : 0;
@@ -821,7 +835,7 @@ int hbf_enable_channel_bus(hbf_ctx *c) {
     CK(cudaStreamSynchronize(c->stream));
     int64_t *b = nullptr; BatchCtrl *bc = nullptr;
     if (cudaMalloc(&b, (size_t)c->mp.channels * 8) != cudaSuccess) return HBF_E_NOMEM;
-    if (cudaMalloc(&bc, sizeof(BatchCtrl)) != cudaSuccess) { cudaFree(b); return HBF_E_NOMEM; }
+    if (cudaMalloc(&bc, kBusPlanAt + kBusPlanBytes) != cudaSuccess) { cudaFree(b); return HBF_E_NOMEM; }
     c->d_bus_busy = b; c->d_bus_ctrl = bc;
     CK(cudaMemsetAsync(b, 0, (size_t)c->mp.channels * 8, c->stream));
     CK(cudaStreamSynchronize(c->stream));
@@ -977,7 +991,8 @@ int hbf_last_result(hbf_ctx *c, hbf_batch_result_t *host_out) {
 int hbf_queue_order(hbf_ctx *c, const void *d_workspace, uint64_t n, uint32_t *d_order, uint64_t *count) {
     if (!c || !d_workspace || !d_order || !count) return HBF_E_INVAL;
     Workspace ws;
-    workspace_layout(n, c->mp.n_queues, c->mp.channels, &ws, const_cast<void *>(d_workspace), c->d_bus_busy ? 1 : 0);
+    // (a regrouped batch had room for everything; what is read of any other one lies in the same place whatever there was room for)
+    workspace_layout(n, c->mp.n_queues, c->mp.channels, kRoomRegroup | kRoomBus, &ws, const_cast<void *>(d_workspace), c->d_bus_busy ? 1 : 0);
     BatchCtrl hc;
     CK(cudaMemcpyAsync(&hc, c->d_ctrl, sizeof(hc), cudaMemcpyDeviceToHost, c->stream));
     CK(cudaStreamSynchronize(c->stream));

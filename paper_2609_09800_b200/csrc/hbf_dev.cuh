@@ -101,9 +101,9 @@ struct Workspace {
     void *in_head;                       // [tiles]: the first 8 accesses of every (tile, queue) for the fix-up: a tile's first entries, then each queue's other seven
     uint8_t *in_headcnt;                 // [tiles][queues]: how many of them exist; 0xff marks a queue for the straggle pass
     uint16_t *in_qid;                    // [tiles][stride]: queue of each of the first records of every tile (0xffff: not modeled), for the straggle pass
-    void *rg_ctrl, *rg_slots, *rg_recs, *rg_idx;   // a batch out of issue order: see regroup.cuh (the slots share memory with keys, idx and terms)
+    void *rg_ctrl, *rg_slots, *rg_recs, *rg_idx;   // a batch out of issue order: see regroup.cuh (the slots share memory with keys, idx and terms; no room for them: rg_ctrl is null)
     uint32_t *bus_xfer;                  // [n] transfer time of every read (only with the channel-bus stage on)
-    void *bus_plan;                      // (likewise) see bus.cuh
+    void *bus_heads;                     // (likewise; null: no room for the buckets) see bus.cuh
     size_t bytes;
 };
 
@@ -185,8 +185,12 @@ inline uint64_t inorder_tiles_bound(uint64_t n) {
     const uint64_t t = (n + kInTileQuantum - 1) / kInTileQuantum;
     return t < 1 ? 1 : (t < kInMaxTiles ? t : kInMaxTiles);
 }
-size_t workspace_layout(uint64_t n, uint32_t n_queues, uint32_t channels, Workspace *ws, void *base, int with_bus = 0);
-// channel bus as a second queued stage, after launch_submit on the same arguments (bc: a control block of its own)
+// What a workspace may have room for besides what every batch needs: the arrays that bring a batch into issue order, and the bus
+// stage's buckets.  Without them the radix sort does both.
+enum : uint32_t { kRoomRegroup = 1u, kRoomBus = 2u };
+size_t workspace_layout(uint64_t n, uint32_t n_queues, uint32_t channels, uint32_t rooms, Workspace *ws, void *base, int with_bus);
+// channel bus as a second queued stage, after launch_submit on the same arguments (bc: a control block of its own, the stage's plan behind it)
+constexpr size_t kBusPlanAt = 4096, kBusPlanBytes = 8192;
 cudaError_t launch_bus_stage(const SubmitArgs &a, BatchCtrl *bc, int64_t *bus_busy, cudaStream_t st);
 cudaError_t launch_bus_buckets(const SubmitArgs &a, BatchCtrl *bc, int64_t *bus_busy, cudaStream_t st);
 // How the in-order path cuts a batch of n records into contiguous tiles: n_big tiles of `big` records, then tiles of
@@ -261,7 +265,7 @@ struct PagedWorkspace {
 };
 // parts of the list; pages of all accesses; accesses issued before their predecessor; set when a service of a stripe unit's pages is too long for the in-order kernels
 enum PagedTotal { kPagedParts = 0, kPagedPages = 1, kPagedUnsorted = 2, kPagedLong = 3, kPagedTotals = 4 };
-size_t paged_layout(uint64_t n, uint64_t capacity, uint32_t n_queues, uint32_t channels, PagedWorkspace *pw, void *base, int with_bus = 0);
+size_t paged_layout(uint64_t n, uint64_t capacity, uint32_t n_queues, uint32_t channels, uint32_t rooms, PagedWorkspace *pw, void *base, int with_bus);
 cudaError_t launch_paged_count(const hbf_access_t *acc, uint64_t n, const RangeSnap *ranges, const ModelParams *mp_dev, const FastRange &fast,
                                const ModelParams &mp, const DevState *state, bool by_unit, const PagedWorkspace &pw, cudaStream_t st);
 cudaError_t launch_paged_offsets(uint64_t n, const PagedWorkspace &pw, cudaStream_t st);

@@ -269,7 +269,7 @@ __global__ void k_paged_finish(hbf_batch_result_t *result, hbf_batch_result_t *r
     if (result->code == HBF_OK) { result->n_modeled = sums->n_ready; result->modeled_ns = (int64_t)sums->stall_sum; *result_host = *result; }
 }
 
-size_t paged_layout(uint64_t n, uint64_t capacity, uint32_t n_queues, uint32_t channels, PagedWorkspace *pw, void *base_ptr, int with_bus) {
+size_t paged_layout(uint64_t n, uint64_t capacity, uint32_t n_queues, uint32_t channels, uint32_t rooms, PagedWorkspace *pw, void *base_ptr, int with_bus) {
     const uint64_t nn = n ? n : 1, cap = capacity ? capacity : 1;
     const uint64_t tiles = (nn + kPgTile - 1) / kPgTile;
     size_t off = 0;
@@ -277,7 +277,7 @@ size_t paged_layout(uint64_t n, uint64_t capacity, uint32_t n_queues, uint32_t c
     auto take = [&](size_t bytes) { size_t o = off; off = (off + bytes + 255) / 256 * 256; return b ? b + o : nullptr; };
     void *ts = take(tiles * 8), *ro = take(tiles * kPgRows * 4), *tot = take(sizeof(PagedSums) + kPagedTotals * 8), *pf = take((nn + 1) * 4);
     void *pa = take(cap * sizeof(hbf_access_t)), *pc = take(cap * 8), *ps = take(cap * 8), *pst = take(cap);
-    const size_t inner = workspace_layout(cap, n_queues, channels, nullptr, nullptr, with_bus);
+    const size_t inner = workspace_layout(cap, n_queues, channels, rooms, nullptr, nullptr, with_bus);
     void *in = take(inner);
     if (pw) {
         pw->tile_sum = (unsigned long long *)ts; pw->row_off = (uint32_t *)ro; pw->total = (unsigned long long *)tot;

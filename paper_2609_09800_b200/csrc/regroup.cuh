@@ -41,6 +41,7 @@ inline uint32_t regroup_out_buckets(uint64_t n) { return (uint32_t)((n + kRgOut 
 inline RegroupArgs regroup_args(uint64_t n, const Workspace &ws, RegroupSync *sync) {
     RegroupArgs r{};
     r.sync = sync;
+    if (!ws.rg_ctrl) return r;                               // (no room: the radix sort serves what is out of order)
     r.max_buckets = regroup_buckets(n); r.out_buckets = regroup_out_buckets(n);
     r.cursor = static_cast<uint32_t *>(ws.rg_ctrl); r.cursor_out = r.cursor + (size_t)kRgPad * r.max_buckets;
     r.offset = r.cursor_out + (size_t)kRgPad * r.out_buckets; r.part = r.offset + r.max_buckets;

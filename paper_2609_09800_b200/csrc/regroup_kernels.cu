@@ -59,10 +59,10 @@ k_begin_regroup(const __grid_constant__ BeginArgs b, const hbf_access_t *__restr
         __syncthreads();
         first = s_lo; last = s_hi;
     }
-    // (refresh claims go by batch index: a batch that has to pay some is sorted; so is one whose samples lie outside the limits of
+    // (refresh claims go by batch index: a batch that has to pay some is sorted, and one whose workspace has no room; so is one whose samples lie outside the limits of
     // issue times, which the sort path refuses: spans up to 2^48 ns are all that the stretches below are made for)
     const bool outside = first < 0 || last >= HBF_ISSUE_LIMIT;
-    const bool sorted = bad && (first >= last || outside || (b.claim_limit && *b.claim_limit > 0ull)), go = bad && !sorted && !begin_refused(b.state);
+    const bool sorted = bad && (first >= last || outside || !r.cursor || (b.claim_limit && *b.claim_limit > 0ull)), go = bad && !sorted && !begin_refused(b.state);
     RegroupSync *sync = r.sync;
     BatchCtrl *ctrl = b.ctrl;
     const uint32_t limit = b.state->spin_limit;

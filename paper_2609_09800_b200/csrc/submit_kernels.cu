@@ -1014,7 +1014,7 @@ cudaError_t launch_bus_stage(const SubmitArgs &a, BatchCtrl *bc, int64_t *bus_bu
     const uint64_t sort_tiles = (n + kSortTile - 1) / kSortTile, bus_tiles = (n + kBusTile - 1) / kBusTile;
     BusChain c{};
     c.acc = a.acc; c.n = n; c.completion = a.completion; c.stall = a.stall; c.ranges = a.ranges; c.mp_dev = a.mp_dev; c.bc = bc; c.state = a.state;
-    c.result = a.result; c.result_host = a.result_host; c.plan = static_cast<const BusPlan *>(a.ws.bus_plan); c.busy = bus_busy; c.ws = a.ws;
+    c.result = a.result; c.result_host = a.result_host; c.plan = bus_plan_of(bc); c.busy = bus_busy; c.ws = a.ws;
     c.wide = (unsigned)std::min<uint64_t>((n + 255) / 256, (uint64_t)a.sm_count * 8);
     c.hist_grid = (unsigned)std::min<uint64_t>((n + kHistThreads * 8 - 1) / (kHistThreads * 8), (uint64_t)a.sm_count * 4);
     c.sort_grid = (unsigned)std::min<uint64_t>(sort_tiles, (uint64_t)a.sm_count * 3);
@@ -1031,20 +1031,22 @@ cudaError_t launch_bus_stage(const SubmitArgs &a, BatchCtrl *bc, int64_t *bus_bu
 // =====================================================================================================
 static size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
-size_t workspace_layout(uint64_t n, uint32_t n_queues, uint32_t channels, Workspace *ws, void *base_ptr, int with_bus) {
+size_t workspace_layout(uint64_t n, uint32_t n_queues, uint32_t channels, uint32_t rooms, Workspace *ws, void *base_ptr, int with_bus) {
     const uint64_t nn = n ? n : 1;
     const uint64_t sort_tiles = (nn + kSortTile - 1) / kSortTile, scan_tiles = (nn + kScanTile - 1) / kScanTile;
     size_t off = 0;
     char *b = static_cast<char *>(base_ptr);
     auto take = [&](size_t bytes) { size_t o = off; off = align_up(off + bytes, 256); return b ? b + o : nullptr; };
     const bool inorder = n_queues <= kInMaxQueues;
+    const bool regroup = inorder && (rooms & kRoomRegroup) && nn > kInSmallMax;          // (smaller ones have a route of their own)
+    const bool buckets = with_bus && (rooms & kRoomBus) && channels <= kBusMaxChannels;
     // the radix sort's arrays; the slots of a batch that is brought into order lie in the same memory
     const size_t slots_at = off;
     void *k0 = take(nn * 8), *k1 = take(nn * 8), *i0 = take(nn * 4), *i1 = take(nn * 4);
     void *tw = take(nn * 8);
-    if (inorder) off = std::max(off, align_up(slots_at + regroup_slot_bytes(nn), 256));
-    if (with_bus) off = std::max(off, align_up(slots_at + bus_entry_bytes(nn, channels), 256));   // (the bus stage's entries, once the batch is served)
-    void *rr = take(inorder ? nn * 24 : 0), *ri = take(inorder ? nn * 4 : 0), *rc = take(inorder ? regroup_ctrl_bytes(nn) : 0);
+    if (regroup) off = std::max(off, align_up(slots_at + regroup_slot_bytes(nn), 256));
+    if (buckets) off = std::max(off, align_up(slots_at + bus_entry_bytes(nn, channels), 256));   // (the bus stage's entries, once the batch is served)
+    void *rr = take(regroup ? nn * 24 : 0), *ri = take(regroup ? nn * 4 : 0), *rc = take(regroup ? regroup_ctrl_bytes(nn) : 0);
     void *h = take((size_t)kMaxPasses * kRadix * 4);
     void *d0 = take(sort_tiles * kRadix * 4), *d1 = take(sort_tiles * kRadix * 4);
     void *sd = take(scan_tiles * sizeof(ScanDesc));
@@ -1054,14 +1056,14 @@ size_t workspace_layout(uint64_t n, uint32_t n_queues, uint32_t channels, Worksp
     void *ih = take(inorder ? inorder_head_bytes(in_tiles, n_queues) : 0);
     void *ic = take(inorder ? in_tiles * n_queues : 0);
     void *iq = take(inorder ? inorder_qid_entries(nn) * 2 : 0);
-    void *bx = take(with_bus ? nn * 4 : 0), *bp = take(with_bus ? bus_plan_bytes(nn, channels) : 0);
+    void *bx = take(with_bus ? nn * 4 : 0), *bh = take(buckets ? bus_head_bytes(nn, channels) : 0);
     if (ws) {
         ws->keys[0] = (uint64_t *)k0; ws->keys[1] = (uint64_t *)k1; ws->idx[0] = (uint32_t *)i0; ws->idx[1] = (uint32_t *)i1;
         ws->terms = (uint64_t *)tw;
-        ws->rg_ctrl = rc; ws->rg_slots = b ? b + slots_at : nullptr; ws->rg_recs = rr; ws->rg_idx = ri;
+        ws->rg_ctrl = regroup ? rc : nullptr; ws->rg_slots = b ? b + slots_at : nullptr; ws->rg_recs = rr; ws->rg_idx = ri;
         ws->hist = (uint32_t *)h; ws->sort_desc[0] = (uint32_t *)d0; ws->sort_desc[1] = (uint32_t *)d1;
         ws->scan_desc = sd; ws->in_agg = (int64_t *)ia; ws->in_bin = (int64_t *)ib;
-        ws->in_tile = it; ws->in_head = ih; ws->in_headcnt = (uint8_t *)ic; ws->in_qid = (uint16_t *)iq; ws->bus_xfer = (uint32_t *)bx; ws->bus_plan = bp; ws->bytes = off;
+        ws->in_tile = it; ws->in_head = ih; ws->in_headcnt = (uint8_t *)ic; ws->in_qid = (uint16_t *)iq; ws->bus_xfer = (uint32_t *)bx; ws->bus_heads = buckets ? bh : nullptr; ws->bytes = off;
     }
     return off;
 }
