@@ -676,3 +676,18 @@ def test_reset_and_totals_with_another_device_current(hbf):
         assert torch.cuda.current_device() == 1 and not g.get_busy_until().any()
     with torch.cuda.device(0):
         assert np.array_equal(g.submit_host(w.acc)[1], o.submit(w.acc)[1])
+
+
+def test_host_batches_whose_sizes_vary(hbf):
+    """Around the powers of two that their buffers are made for, up and down, in one chunk and in several."""
+    import torch
+    w = wl.capacity_mode(n=70_000, seed=8)
+    g, o = contexts(hbf, w.profile, w.ranges)
+    rec = torch.from_numpy(w.acc.view(np.int64).reshape(-1)).pin_memory()
+    out = [torch.empty(k, dtype=torch.int64).pin_memory() for k in (70_000, 70_000, g.n_dies * 6)]
+    for n, chunk in ((1, 0), (3, 0), (4, 0), (5, 0), (1000, 0), (1024, 0), (1025, 0), (8192, 0), (8193, 0), (5000, 1200), (65_536, 0), (65_537, 0), (70_000, 16_385), (2, 0)):
+        g.reset(); o.reset()
+        rc, summary = g.submit_pinned(rec, n, out[0], out[1], out[2], chunk=chunk)
+        _, c_o, s_o, _, ds_o = o.submit(w.acc[:n])
+        assert rc == 0 and summary["n_modeled"] == n
+        assert np.array_equal(out[0][:n].numpy(), c_o) and np.array_equal(out[1][:n].numpy(), s_o) and np.array_equal(out[2].numpy(), ds_o.view(np.int64))
