@@ -11,8 +11,8 @@
 //   (the in-order kernels)
 //   give      completion, issue time and index go to the bucket of 2,048 results that they belong to, the same way
 //   place     a block per bucket puts them in order through shared memory and writes completions and stalls, whole lines
-// A bucket that overflows (times bunched more tightly than the sample shows), or more than 64 records in a bin, sends the batch
-// to the radix sort, as do outstanding refresh claims (they go by batch index) and service times the in-order kernels do not hold.
+// A bucket that overflows (times bunched more tightly than the sample shows) sends the batch
+// to the radix sort, as do few distinct times (rg_crowded), outstanding refresh claims (they go by batch index) and service times the in-order kernels do not hold.
 // Bytes per record: 24 + 32 (scatter), 32 + 28 (sort), 28 + 16 (serve), 20 + 16, 16 + 16 (results): 228, streaming, against
 // some 400, a third of them scattered, for six radix passes and a scan that gathers and scatters by sorted index.
 // The work of a phase is dealt out in shares, in order, by a counter, and a block that finds none left waits until all are done:

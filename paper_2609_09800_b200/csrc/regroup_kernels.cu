@@ -20,7 +20,7 @@ OrderedCopy ordered_copy(uint64_t n, const Workspace &ws) {
 }
 
 constexpr int kRgThreads = 1024, kRgGroup = 512, kRgGroups = kRgThreads / kRgGroup;
-constexpr uint32_t kRgBins = 4096, kRgBinMax = 64;
+constexpr uint32_t kRgBins = 4096;
 constexpr int kRgItems = kRgCap / kRgGroup;
 static_assert(kRgCap % kRgGroup == 0 && kRgBins % kRgGroup == 0, "whole rounds");
 constexpr uint32_t kRgParts = 4096;                      // chunks of buckets at most: 2^32 records
@@ -38,12 +38,34 @@ __device__ __forceinline__ uint32_t rg_stretch(int64_t t, int64_t lo, uint32_t s
     return seg;
 }
 
+// Do so many records share their issue times that buckets would overflow, or spend their time on telling equal times apart?  1,024
+// samples, one per thread, and a table of the distinct ones; where few are equal, pairs of equal ones tell (of m samples of D times
+// about m^2 / 2D), else the distinct ones are nearly all there are.  40 M shuffled records, us, by the radix sort as it is launched from the
+// device 7,700 (and 8,200 before there were buckets; the attempt adds 700 if it overflows); in buckets 2,850 with 1 record per
+// time, 3,700 with 50, 7,100 with 500; more than some 900 overflow.
+constexpr uint32_t kRgCrowd = 700, kRgSeen = 4096;
+__device__ __forceinline__ bool rg_crowded(long long time, uint64_t n, unsigned long long *seen) {
+    for (uint32_t e = threadIdx.x; e < kRgSeen; e += kRgThreads) seen[e] = 0ull;
+    __syncthreads();
+    const unsigned long long key = (unsigned long long)time + 1ull;
+    uint32_t at = (uint32_t)((key * 0x9e3779b97f4a7c15ull) >> 52);
+    bool fresh = false;
+    for (;;) {                                               // (a quarter full at most)
+        const unsigned long long had = atomicCAS(seen + at, 0ull, key);
+        fresh = had == 0ull;
+        if (fresh || had == key) break;
+        at = (at + 1u) % kRgSeen;
+    }
+    const uint64_t distinct = (uint64_t)__syncthreads_count(fresh), equal = kRgThreads - distinct;
+    return equal != 0ull && n > kRgCrowd * (2u * distinct <= (uint64_t)kRgThreads ? distinct : (uint64_t)kRgThreads * kRgThreads / (2u * equal));
+}
+
 __global__ void __launch_bounds__(kRgThreads, 1)
 k_begin_regroup(const __grid_constant__ BeginArgs b, const hbf_access_t *__restrict__ acc, uint64_t n, const RangeSnap *__restrict__ ranges,
                 const __grid_constant__ FastRange fast, const __grid_constant__ RegroupArgs r, uint8_t *status) {
     extern __shared__ __align__(16) unsigned char rg_smem[];
     __shared__ long long s_lo, s_hi;
-    __shared__ uint32_t s_base[kRgSegs], s_first[kRgSegs], s_last[kRgSegs], s_buckets, s_w[kRgThreads / 32], s_next[kRgGroups], s_run[kRgGroups];
+    __shared__ uint32_t s_base[kRgSegs], s_first[kRgSegs], s_last[kRgSegs], s_buckets, s_w[kRgThreads / 32], s_next[kRgGroups];
     __shared__ uint64_t s_mul[kRgSegs];
     __shared__ long long s_min[kRgGroups], s_max[kRgGroups];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -53,16 +75,18 @@ k_begin_regroup(const __grid_constant__ BeginArgs b, const hbf_access_t *__restr
     if (tid == 0) { s_lo = INT64_MAX; s_hi = INT64_MIN; }
     long long first, last;
     bool bad = begin_samples(acc, n, &first, &last);
+    const long long one = first;
     if (bad) {
         for (int o = 16; o > 0; o >>= 1) { first = min(first, __shfl_xor_sync(0xffffffffu, first, o)); last = max(last, __shfl_xor_sync(0xffffffffu, last, o)); }
         if (lane == 0) { atomicMin(&s_lo, first); atomicMax(&s_hi, last); }
         __syncthreads();
         first = s_lo; last = s_hi;
     }
-    // (refresh claims go by batch index: a batch that has to pay some is sorted, and one whose workspace has no room; so is one whose samples lie outside the limits of
+    // (refresh claims go by batch index: a batch that has to pay some is sorted, and one whose workspace has no room, or with few
+    // distinct times; so is one whose samples lie outside the limits of
     // issue times, which the sort path refuses: spans up to 2^48 ns are all that the stretches below are made for)
     const bool outside = first < 0 || last >= HBF_ISSUE_LIMIT;
-    const bool sorted = bad && (first >= last || outside || !r.cursor || (b.claim_limit && *b.claim_limit > 0ull)), go = bad && !sorted && !begin_refused(b.state);
+    const bool sorted = bad && (first >= last || outside || !r.cursor || rg_crowded(one, n, reinterpret_cast<unsigned long long *>(rg_smem)) || (b.claim_limit && *b.claim_limit > 0ull)), go = bad && !sorted && !begin_refused(b.state);
     RegroupSync *sync = r.sync;
     BatchCtrl *ctrl = b.ctrl;
     const uint32_t limit = b.state->spin_limit;
@@ -134,6 +158,7 @@ k_begin_regroup(const __grid_constant__ BeginArgs b, const hbf_access_t *__restr
     constexpr uint32_t kScatter = 1024;
     const uint32_t scatters = (uint32_t)((n + kScatter - 1) / kScatter);
     rg_shares(sync, 1, scatters, b.state->test_stage == 1u ? b.state->test_tile : kRgNone, [&](uint32_t g) {
+        if (ld_relaxed_u32(&ctrl->run_sort)) return;         // a bucket has overflowed: the rest is not worth sending
         for (uint32_t at0 = 0; at0 < kScatter; at0 += 128u) {
             uint64_t addr[4], issue[4], bf[4];
             uint32_t at[4], bucket[4];
@@ -241,7 +266,7 @@ k_begin_regroup(const __grid_constant__ BeginArgs b, const hbf_access_t *__restr
             }
         }
         group_sync(group);                                   // shared memory of the bucket before is no longer read
-        if (gtid == 0) { s_min[group] = INT64_MAX; s_max[group] = INT64_MIN; s_run[group] = 0u; s_next[group] = atomicAdd(&sync->claim[5], 1u); }
+        if (gtid == 0) { s_min[group] = INT64_MAX; s_max[group] = INT64_MIN; s_next[group] = atomicAdd(&sync->claim[5], 1u); }
         for (uint32_t e = gtid; e < kRgBins; e += kRgGroup) s_cnt[e] = 0u;
         long long mn = INT64_MAX, mx = INT64_MIN;
 #pragma unroll
@@ -293,14 +318,14 @@ k_begin_regroup(const __grid_constant__ BeginArgs b, const hbf_access_t *__restr
         for (int k = 0; k < kRgItems; ++k)
             if (k * kRgGroup + gtid < m) s_key[s_cnt[bin[k] & 0xffffu] + (bin[k] >> 16)] = ((uint64_t)(issue[k] - t0) << 32) | idx[k];
         group_sync(group);
-        // a record's place within its bin: how many of the bin's keys are smaller (rarely more than three in all)
+        // a record's place within its bin: how many of the bin's keys are smaller (rarely more than three in all; records issued at the
+        // same time share a bin, however many they are)
 #pragma unroll
         for (int k = 0; k < kRgItems; ++k) {
             if (k * kRgGroup + gtid < m) {
                 const uint32_t d = bin[k] & 0xffffu, from = s_cnt[d], to = d + 1u < kRgBins ? s_cnt[d + 1u] : m;
                 uint32_t before = 0;
-                if (to - from > kRgBinMax) s_run[group] = 1u;
-                else if (to - from > 1u) {
+                if (to - from > 1u) {
                     const uint64_t key = ((uint64_t)(issue[k] - t0) << 32) | idx[k];
                     for (uint32_t q = from; q < to; ++q) before += s_key[q] < key ? 1u : 0u;
                 }
@@ -308,7 +333,6 @@ k_begin_regroup(const __grid_constant__ BeginArgs b, const hbf_access_t *__restr
             }
         }
         group_sync(group);
-        if (s_run[group]) { if (gtid == 0) ctrl->run_sort = 1u; return; }              // (places would not be distinct)
 #pragma unroll
         for (int k = 0; k < kRgItems; ++k)
             if (k * kRgGroup + gtid < m) { uint64_t *o = s_rec + bin[k] * 3u; o[0] = addr[k]; o[1] = (uint64_t)issue[k]; o[2] = bf[k]; s_idx[bin[k]] = idx[k]; }

@@ -143,3 +143,21 @@ def test_a_bus_that_cannot_take_a_batch_out_of_order(hbf):
     _, c_o, s_o, *_ = o.submit(acc)
     _, c, s, *_ = g.submit_host(acc)
     assert np.array_equal(c, c_o) and np.array_equal(s, s_o) and np.array_equal(g.get_bus_busy_until(), o.bus_busy_until())
+
+
+@pytest.mark.parametrize("n", [9_000, 60_001, 300_000])
+@pytest.mark.parametrize("per", [2, 63, 65, 300, 699, 1_100, 2_047, 5_000])
+def test_records_that_share_their_issue_times(hbf, per, n):
+    """Ticks of so many records each, around what a bin once held, what a bucket holds, and where the radix sort takes over."""
+    w = wl.capacity_mode(n=n, seed=n, rho=0.6)
+    g, o = hbf.Context(w.profile), hbfo.Oracle(w.profile)
+    for r in w.ranges:
+        g.register_range(*r); o.register_range(*r)
+    acc = w.acc.copy()
+    acc["issue_ns"] = np.arange(n) // per * (per * 40) + 7
+    acc = acc[np.random.default_rng(per).permutation(n)]
+    for _ in range(2):
+        _, c_o, s_o, st_o, _ = o.submit(acc)
+        _, c, s, st, _ = g.submit_host(acc)
+        assert np.array_equal(c, c_o) and np.array_equal(s, s_o) and np.array_equal(st, st_o) and g.last_result() == o.last_result()
+        assert np.array_equal(g.queue_order(n), o.last_order())
