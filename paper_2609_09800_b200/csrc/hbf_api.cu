@@ -526,6 +526,7 @@ int hbf_set_head_entries(hbf_ctx *c, uint32_t entries) {
 
 // is what is enqueued on the stream now being captured into a graph
 static bool capturing(cudaStream_t st) {
+    if (st == nullptr || st == cudaStreamLegacy) return false;          // (the legacy default stream cannot be; a question saved per call)
     cudaStreamCaptureStatus s = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(st, &s) != cudaSuccess) { (void)cudaGetLastError(); return false; }
     return s != cudaStreamCaptureStatusNone;
