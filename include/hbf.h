@@ -142,8 +142,9 @@ HBF_API int hbf_submit_batch(hbf_ctx *ctx, const hbf_access_t *d_acc, uint64_t n
  * chunk, in order: for records in issue order that is the same as one batch.
  * h_acc [n] host, read only; h_completion_ns, h_stall_ns [n] host; h_die_stats [channels*dies] host, nullable: totals
  * over the chunks.  Pinned host memory (cudaMallocHost / cudaHostRegister) makes the copies asynchronous and
- * overlapped; pageable memory works, slower.  The library owns the device buffers (two chunks of records and results,
- * one workspace), allocated at the first call and kept until hbf_destroy; a larger chunk reallocates them.
+ * overlapped; pageable memory works, slower.  The library owns the device buffers (a chunk of records and results and a
+ * workspace; a second chunk once a call has several), allocated at the first call and kept until hbf_destroy; a larger chunk
+ * reallocates them (up to 65,536 records they are made for the next power of two).
  * The call returns when every result is in the caller's buffers.  summary_out (host, nullable) receives the chunks'
  * summaries added up (counts and times summed, the largest completion, mode and q of the first chunk) with code =
  * the first chunk code that is not HBF_OK; that code is also the return value.  A refused chunk (fail-closed access,
@@ -225,10 +226,12 @@ HBF_API int hbf_get_mode(hbf_ctx *ctx, int32_t *mode, int64_t *q_ppm);          
 HBF_API int hbf_reset(hbf_ctx *ctx);                                             /* queues idle, field at ambient, mode Normal; in stream order, waits for nothing */
 
 /* Chooses how batches are ordered: HBF_PATH_AUTO (default) serves a batch whose records arrive in
- * non-decreasing issue order without a global sort and falls back to the radix sort otherwise (also for a batch in
+ * non-decreasing issue order without a global sort, brings one that is out of order into order in buckets by issue time first,
+ * and falls back to the radix sort for what those do not hold (issue times that coincide for hundreds of records,
+ * outstanding refresh quanta on a batch out of order, one that looked to be in order, a smaller workspace; and a batch in
  * which a single access's service time reaches 2^33 ns, 2^32 ns with retention on: the in-order kernels keep
- * per-tile sums of service times in 56 bits; batches of at most 8,192 records take a route of their own that has no such
- * limit);
+ * per-tile sums of service times in 56 bits); batches of at most 8,192 records take a route of their own that has no such
+ * limits;
  * HBF_PATH_SORT always sorts (a batch already in issue order is sorted on its queue bits only, which a
  * stable sort allows); HBF_PATH_SORT_FULL sorts on every key bit regardless; HBF_PATH_INORDER is the caller's
  * declaration that its batches are in issue order: only the in-order kernels are launched, and a batch that is not in
@@ -272,9 +275,11 @@ HBF_API int hbf_get_pending_energy(hbf_ctx *ctx, int64_t *host_out, uint64_t cap
 HBF_API int hbf_get_temps(hbf_ctx *ctx, float *host_out, uint64_t cap);
 HBF_API double hbf_euler_limit_ns(const hbf_ctx *ctx);
 
-/* The order in which the last batch was served when it went through the sort path: batch indices,
- * queue-major, read back from the workspace of that batch into d_order (device [n]); *count (host)
- * receives the number of modeled accesses. */
+/* The order in which the last batch was served, for a batch out of issue order (or one that was sorted all the same; HBF_E_INVAL
+ * after one that was served in order): batch indices, queue-major, from the workspace of that batch into d_order (device [n]);
+ * *count (host) receives the number of modeled accesses.  For a batch that was brought into order in buckets the order is
+ * worked out by this call, which overwrites scratch in that workspace (the call may be repeated); not to be asked
+ * of a batch behind which the channel-bus stage ran, unless it came through the buckets: that stage works in the same memory. */
 HBF_API int hbf_queue_order(hbf_ctx *ctx, const void *d_workspace, uint64_t n, uint32_t *d_order, uint64_t *count);
 
 /* Stage timing.  With profiling on, every submit and thermal step records CUDA events between its

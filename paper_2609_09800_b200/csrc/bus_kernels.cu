@@ -14,7 +14,7 @@
 //   redo     buckets in which the 16 do not reach that far, in full
 // A bucket with more than three times the average sends the batch to the radix sort of (channel, time) in submit_kernels.cu.
 // Bytes per read: 24 + 8 + 16, then 16 and the results that change.  32 M reads with the array stage: 4,112 us with the radix
-// sort (five passes over 12 bytes, two gathers by sorted index), 1,618 in buckets; 20,011 reads 171 and 79.  What bounds it: scatter
+// sort (five passes over 12 bytes, two gathers by sorted index), 1,645 in buckets; 20,011 reads 171 and 79.  What bounds it: scatter
 // 418 us (memory and instructions in equal parts), order some 650 (instructions: 18 per read and lane; barriers).  A block that
 // waited for the bus from the bucket before by look-back instead of assuming it idle: 1,245 us for that kernel; smaller buckets
 // of a warp each, with look-back: 3,100.

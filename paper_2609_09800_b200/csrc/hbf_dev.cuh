@@ -55,10 +55,11 @@ struct SortPlan {
     uint32_t bits[kMaxPasses];
 };
 
-// Per-batch control block in device memory, cleared by the begin kernel.
 // regroup.cuh: the shares of every phase that are taken and done, the spread of the issue times.  Zero between batches: the begin
 // kernel clears what the last kernel uses, and the other way round.
 struct RegroupSync { uint32_t claim[8], done[8], hist[64], top[64], below[64]; };   // (samples of a stretch, their largest offset, 2^32 - 1 less their smallest)
+
+// Per-batch control block in device memory, cleared by the begin kernel.
 struct BatchCtrl {
     int32_t code;                        // HBF_OK or the batch's refusal / failure code
     int32_t skip;                        // later kernels do nothing when set
@@ -242,10 +243,10 @@ cudaError_t launch_submit(const SubmitArgs &a, cudaStream_t st);
 // total[i] += part[i] over the 6 * n_dies counters of a per-die statistics array (host-buffer pipeline: totals over its chunks)
 cudaError_t launch_add_stats(hbf_die_stats_t *total, const hbf_die_stats_t *part, uint32_t n_dies, cudaStream_t st);
 // the same for batch summaries: counts and times added, the largest completion, the first code that is not HBF_OK; first != 0 starts over
-// results of a small batch to host memory the device can write: completions, stalls, per-die totals (null: not wanted; zeros for a refused batch), summary
+cudaError_t launch_add_result(hbf_batch_result_t *sum, const hbf_batch_result_t *part, int first, cudaStream_t st);
+// results of a small batch to host memory the device can write: completions, stalls, per-die totals (null: not wanted), summary
 cudaError_t launch_host_results(const int64_t *comp, const int64_t *stall, const hbf_die_stats_t *stats, const hbf_batch_result_t *result, uint64_t n, uint32_t n_dies,
                                 int64_t *h_comp, int64_t *h_stall, hbf_die_stats_t *h_stats, hbf_batch_result_t *h_result, bool *plain_next, cudaStream_t st);
-cudaError_t launch_add_result(hbf_batch_result_t *sum, const hbf_batch_result_t *part, int first, cudaStream_t st);
 cudaError_t launch_queue_order(const BatchCtrl *ctrl, const Workspace &ws, uint32_t *out, uint64_t n, cudaStream_t st);
 // the same for a batch that was served on an ordered copy: its queue-major order is sorted out only now (bc: a control block of its own)
 cudaError_t launch_regrouped_order(BatchCtrl *bc, DevState *state, const RangeSnap *ranges, const ModelParams *mp, const Workspace &ws, uint32_t *out, uint64_t n,

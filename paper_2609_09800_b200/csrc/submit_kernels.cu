@@ -1125,13 +1125,14 @@ static cudaError_t launch_sort_path(const SubmitArgs &a, cudaStream_t st) {
 }
 
 // ---- the sort path launched from the device -----------------------------------------------------------
-// With HBF_PATH_AUTO the host enqueues the in-order kernels only.  A batch that turns out not to be in issue
-// order (or has a service time the in-order kernels cannot hold) needs the sort path after all, and the host
-// cannot know that without waiting for the device.  So the kernel that follows the in-order kernels (it also sums the
-// batch's stall total when they did serve it) looks at the batch's control block and, in that case only, one thread launches the sort path's kernels itself, in order, into the tail-launch stream: they run
-// after this kernel and before the next kernel of the host's stream (a parent grid is complete
-// only when its children are), which is the batch's finish kernel.  A batch in issue order pays one empty
-// launch instead of thirteen.
+// With HBF_PATH_AUTO the host enqueues the in-order kernels only.  A batch that those do not serve (out of issue order where the begin
+// kernel's samples did not see it or its buckets do not hold it, or with a service time the in-order kernels cannot hold)
+// needs the sort path after all, and the host cannot know that without waiting for the device.  So the last kernel (it also sums
+// the batch's stall total and commits it when they did serve it) looks at the batch's control block and, in that case only, one
+// thread launches the sort path's kernels itself, in order, into the tail-launch stream, their finish kernel among them: they run
+// after this kernel and before the next kernel of the host's stream (a parent grid is complete only when its children are).  A
+// batch in issue order pays no launch for it.  Launched from the device the passes run one block per multiprocessor where two or three
+// would fit: 40 M records 7.7 ms, 5.6 launched by the host.
 struct SortChain {
     const hbf_access_t *acc; uint64_t n; const RangeSnap *ranges; const ModelParams *mp_dev; BatchCtrl *ctrl; DevState *state;
     uint64_t *keys0, *keys1, *terms; uint32_t *idx0, *idx1, *hist, *desc0, *desc1; void *scan_desc;

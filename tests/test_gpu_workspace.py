@@ -84,3 +84,21 @@ def test_least_workspace_of_the_page_granular_submit(hbf, order):
         assert g.submit_batch_paged(rec, n, 3 * n, comp, stall, None, None, ws) == 0
         _, c_o, s_o, *_ = o.submit(acc, paged=True)
         assert g.last_result() == o.last_result() and np.array_equal(comp.cpu().numpy(), c_o) and np.array_equal(stall.cpu().numpy(), s_o)
+
+
+@pytest.mark.parametrize("order", ["issue", "shuffled"])
+@pytest.mark.parametrize("n", [500, 8_192])
+def test_small_batches_that_the_cluster_does_not_take(hbf, n, order):
+    """One die of 300 planes: more queues than a block of the small route serves, fewer records than are ordered in buckets."""
+    prof = wl.load_profile("nominal", channels=1, dies=1, planes=300, page_bytes=16384, stripe_bytes=16384)
+    g, o = hbf.Context(prof), hbfo.Oracle(prof)
+    g.register_range(wl.RANGE_BASE, wl.GIB, 3, 0, 0, 0); o.register_range(wl.RANGE_BASE, wl.GIB, 3, 0, 0, 0)
+    rng = np.random.default_rng(n)
+    acc = np.zeros(n, hbfo.ACCESS_DTYPE)
+    acc["addr"] = wl.RANGE_BASE + rng.integers(0, 1 << 29, n).astype(np.uint64)
+    acc["issue_ns"], acc["bytes"] = 500 * np.arange(n), 4096
+    if order == "shuffled": acc = acc[rng.permutation(n)]
+    for _ in range(2):
+        _, c_o, s_o, *_ = o.submit(acc)
+        _, c, s, *_ = g.submit_host(acc)
+        assert np.array_equal(c, c_o) and np.array_equal(s, s_o) and g.last_result() == o.last_result()
