@@ -7,6 +7,7 @@ namespace hbf {
 struct BeginArgs {
     BatchCtrl *ctrl; const DevState *state; const int64_t *busy; int64_t *busy_stage; hbf_die_stats_t *stats_stage; uint32_t *hist;
     uint32_t n_queues, n_dies; uint32_t *die_claims; const unsigned long long *claim_limit;
+    TileBalance *decides; float twice_from; uint64_t n; uint32_t page_shift; int64_t t_read_ns, t_prog_ns;   // see begin_load (decides: null, not asked)
 };
 
 // 1,024 pairs of neighbouring records (n >= 2; blocks of 1,024 threads): are they out of order, and what span of time does this
@@ -44,6 +45,35 @@ __device__ __forceinline__ void begin_batch(const BeginArgs &a, int run_sort, ui
     for (int i = tid; i < kMaxPasses * kRadix; i += blockDim.x) a.hist[i] = 0u;
     if (a.die_claims)                                        // retention on: an in-order attempt that was handed over counted some
         for (uint32_t d = tid; d < a.n_dies; d += blockDim.x) a.die_claims[d] = 0u;
+}
+
+// How much of its span a batch fills, and with that whether its tiles are served twice at once (BatchCtrl::twice): the services of 1,024
+// sampled records (a page's time per page they touch, as if all were modeled), the refresh quanta it claims, and what the queues
+// are behind when it begins.  twice_from: from this load on it is (see twice_from); below, where the last batch that had to serve half of
+// its tiles twice after all had about this load or less (streams that crowd on some queues at a time): a batch whose load is
+// lower by a tenth is not, whatever came before it.  (While the choice went by the batches before alone, 200 M records without debt
+// behind 200 M with claims took 3,140 us; 2,500 with the fix-up of before that, 2,270 now.)  One block of 1,024 threads, behind
+// begin_batch; first, last: the batch's issue times; rec: this thread's sample.
+__device__ __forceinline__ void begin_load(const BeginArgs &a, const uint64_t *rec, int64_t first, int64_t last) {
+    __shared__ double s_work, s_behind;
+    const int tid = threadIdx.x;
+    if (tid == 0) s_work = s_behind = 0.0;
+    __syncthreads();
+    const uint64_t mask = (1ull << a.page_shift) - 1ull, bf = ld_after(rec + 2), pages = ((ld_after(rec) & mask) + (uint32_t)bf + mask) >> a.page_shift;
+    double work = (double)pages * (double)(((bf >> 32) & 1u) ? a.t_prog_ns : a.t_read_ns), behind = 0.0;
+    for (uint32_t q = tid; q < a.n_queues; q += blockDim.x) behind += (double)max((int64_t)0, a.busy[q] - first);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) { work += __shfl_xor_sync(0xffffffffu, work, o); behind += __shfl_xor_sync(0xffffffffu, behind, o); }
+    if ((tid & 31) == 0) { atomicAdd(&s_work, work); atomicAdd(&s_behind, behind); }
+    __syncthreads();
+    if (tid != 0 || a.ctrl->skip) return;
+    double ns = s_work * ((double)a.n / 1024.0);
+    if (a.claim_limit) ns += (double)min((unsigned long long)a.n, *a.claim_limit) * (double)(a.t_read_ns + a.t_prog_ns);
+    ns = ns * 1e6 / (double)a.ctrl->q_ppm + s_behind;
+    const float load = (float)(ns / ((double)a.n_queues * (double)max((int64_t)1, last - first)));
+    a.ctrl->load = load;
+    if (load >= a.twice_from) a.ctrl->twice = 1u;
+    else if (a.decides->twice_left > 0u && load >= 0.9f * a.decides->twice_load) { a.ctrl->twice = 1u; a.decides->twice_left -= 1u; }
 }
 
 }  // namespace hbf

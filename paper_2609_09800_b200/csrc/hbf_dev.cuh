@@ -72,6 +72,8 @@ struct BatchCtrl {
     uint32_t inorder_used;               // the in-order path served this batch
     uint32_t run_sort;                   // the sort path has to serve this batch
     uint32_t regrouped;                  // the in-order kernels serve it on an ordered copy of the records
+    uint32_t twice;                      // every tile is served twice (decided here for batches too large for the host to tell: begin_load)
+    float load;                          // the share of the batch's span that its work, and what the queues are behind, fills (0: not asked)
     int64_t issue_lo, issue_hi;          // smallest and largest issue time among the begin kernel's samples
     uint32_t role_count[2];              // in-order serve pass: tiles handed out so far, per size class
     uint32_t tile_counter[kMaxPasses + 2];
@@ -219,13 +221,17 @@ struct TileBalance {
     uint32_t len[kInBalMax], ns[kInBalMax];   // records of the tile, and how long its block took (0: taken out of turn, not measured)
     uint32_t strag_seq, strag_max, strag_flagged, strag_depth;   // of batch strag_seq: most straggling queues in a tile, tiles served a second time, head entries kept
     uint32_t first[kInBalMax + 1];       // device only: where the tiles of the batch in flight begin
+    float twice_load; uint32_t twice_left;   // device only: load of the last batch that had to serve half of its tiles twice, and how many like it do so at once
 };
-struct TileBalanceHost { TileBalance *dev = nullptr, *pinned = nullptr; uint32_t seq = 0; bool on = true; uint32_t depth = 0, depth_fixed = 0, depth_seen = 0, twice_left = 0; };   // twice_left: so many large batches are served twice at once; depth: head entries per (tile, queue) of the next batch (0: the most); depth_fixed != 0: set by the caller; depth_seen: batch whose record was read last
+struct TileBalanceHost { TileBalance *dev = nullptr, *pinned = nullptr; uint32_t seq = 0; bool on = true; uint32_t depth = 0, depth_fixed = 0, depth_seen = 0; };   // depth: head entries per (tile, queue) of the next batch (0: the most); depth_fixed != 0: set by the caller; depth_seen: batch whose record was read last
 InTileMap inorder_tile_map(uint64_t n, int sm_count, bool by_table);   // by_table: a full wave gets exactly two tiles per SM, placed by a table
 // per-tile bookkeeping of the stall total: as-if-idle sum, fix-up corrections, and the exact sum of a re-served tile
 struct InTile { long long spec_sum, fix_delta, true_sum; uint32_t reserve; uint32_t stragglers; };
 size_t inorder_head_bytes(uint64_t tiles, uint32_t n_queues);
 size_t inorder_serve_smem(uint32_t n_dies);
+// large batches whose own load decides whether their tiles are served twice (null: not such a batch)
+TileBalance *inorder_decides(const SubmitArgs &a);
+float twice_from(uint64_t n, uint32_t n_queues);
 cudaError_t launch_inorder(const SubmitArgs &a, cudaStream_t st);
 // batches out of issue order (regroup.cuh): the copy of the records that the in-order kernels serve, and its results
 struct OrderedCopy { const hbf_access_t *recs; int64_t *comp, *stall; };

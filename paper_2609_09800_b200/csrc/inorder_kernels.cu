@@ -45,6 +45,7 @@ namespace hbf {
 #define HBF_IN_BLOCKS 2
 #endif
 constexpr int kInThreads = HBF_IN_THREADS;               // threads of a serve block
+constexpr uint32_t kInTwiceRun = 15;                      // batches served twice at once before one takes the fix-up again (see twice_max)
 constexpr int kInBlocksPerSM = HBF_IN_BLOCKS;            // resident serve blocks per SM
 constexpr int kInWarps = kInThreads / 32;
 constexpr uint32_t kInTagStride = kInMaxQueues + 32;      // bytes of a warp's table of lane numbers: one per queue, one per lane
@@ -478,7 +479,7 @@ k_inorder_serve(const hbf_access_t *__restrict__ acc, uint64_t n, const __grid_c
                 const int64_t *__restrict__ in_bin, InTile *in_tile, InHead *__restrict__ in_head, uint8_t *__restrict__ in_headcnt,
                 const int64_t *__restrict__ busy, const unsigned long long *claim_limit_p, uint32_t *die_claims,
                 const __grid_constant__ RetDev ret, uint16_t *__restrict__ in_qid, uint32_t qid_stride,
-                TileBalance *bal, uint32_t bal_seq, const __grid_constant__ FastGeom geom, const uint32_t head_depth, const OrderedCopy copy) {
+                TileBalance *bal, uint32_t bal_seq, const __grid_constant__ FastGeom geom, const uint32_t head_depth, const OrderedCopy copy, const int decided) {
     constexpr bool RESERVE = MODE == kInAgain, LIGHT = MODE == kInLight;
     extern __shared__ __align__(16) unsigned char in_smem[];
     __shared__ long long s_red[2];
@@ -490,13 +491,17 @@ k_inorder_serve(const hbf_access_t *__restrict__ acc, uint64_t n, const __grid_c
     pdl_wait();
     pdl_trigger();
     if (ctrl->skip || ctrl->run_sort) return;             // (run_sort set this early: the batch went to the sort path at its start)
+    if (!RESERVE && decided && (ctrl->twice != 0u) != LIGHT) return;      // (the batch's load has chosen the other of the two)
+    if (RESERVE && decided && blockIdx.x == 0 && threadIdx.x == 0 && ctrl->inorder_used && !ctrl->twice && 2u * bal->strag_flagged >= tmap.n_tiles) {
+        bal->twice_load = ctrl->load; bal->twice_left = kInTwiceRun;
+    }
     if (RESERVE && (!ctrl->inorder_used || !in_tile[blockIdx.x].reserve)) return;
     if (ctrl->regrouped) { acc = copy.recs; completion = copy.comp; stall = copy.stall; status = nullptr; }   // (brought into order: regroup_kernels.cu)
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const RangeSnap &rs = *ranges_g;                      // read through the cache; the common configuration does not touch it
     if (tid == 0) { mp = mp_arg; fast_range = fast_arg; }
     if (DEBT && !RESERVE && tid == 0 && blockIdx.x == 0) ret.st->observed_inline = 1u;
-    if (!RESERVE && bal && tid == 0 && blockIdx.x == 0) { bal->strag_seq = bal_seq; bal->strag_max = 0u; bal->strag_flagged = 0u; bal->strag_depth = head_depth; }
+    if (!RESERVE && bal && tid == 0 && blockIdx.x == 0) { bal->strag_seq = bal_seq; bal->strag_max = 0u; bal->strag_flagged = 0u; bal->strag_depth = LIGHT ? 0u : head_depth; }
     const uint32_t R = mp_arg.n_queues, n_dies = mp_arg.n_dies;
     const int64_t q_ppm = ctrl->q_ppm;
     const Div64 div_q = ctrl->div_q;
@@ -1058,7 +1063,7 @@ k_inorder_fixstraggle(const hbf_access_t *__restrict__ acc, uint64_t n, const __
 
     pdl_wait();
     pdl_trigger();
-    if (ctrl->skip || ctrl->run_sort || !ctrl->inorder_used) return;
+    if (ctrl->skip || ctrl->run_sort || !ctrl->inorder_used || ctrl->twice) return;
     if (ctrl->regrouped) { acc = copy.recs; completion = copy.comp; stall = copy.stall; }
     const uint32_t tile = blockIdx.x;
     if (tile == 0u) return;                                  // the first tile was served from its true entering state
@@ -1447,9 +1452,21 @@ size_t inorder_head_bytes(uint64_t tiles, uint32_t n_queues) { return tiles * n_
 // and 38, 8 M 162 and 168; decode, 1,024 queues, 4 M 150 and 91, 12 M 207 and 192, 16 M 210 and 225 (load 0.3); capacity, 2,048
 // queues, 4 M 255 and 106, 16 M 323 and 251 (0.3), 28 M 369 and 418 (0.3).
 static uint64_t twice_max(uint32_t n_queues) { return 5000000ull + 7500ull * n_queues; }
-// Larger ones too where the last batch had to serve half of its tiles twice after all (fix-up and second pass: 24 M prefix records
-// 469 us, 48 M at load 0.85 963; served twice at once 357 and 657); every 16th of them takes the fix-up, to see whether it still does.
-constexpr uint32_t kInTwiceRun = 15;
+// Larger ones from a load on that rises with their size, towards 0.7, where queues begin to be behind everywhere (twice_from); and below
+// it where a batch with about their load, or less, had to serve half of its tiles twice after all; every 16th of those takes the fix-up,
+// to see whether it still does.  The device decides (begin_load), so both forms of the first pass are launched and one leaves at once
+// (2 us).  us, with the fix-up and served twice, by load: capacity, 2,048 queues, 24 M 344 and 380 (0.3), 369 and 379 (0.4), 429 and 378 (0.5),
+// 683 and 380 (0.65); 48 M 640 and 673 (0.55), 724 and 674 (0.6), 1,047 and 674 (0.65); 96 M 1,046 and 1,276 (0.6), 1,537 and
+// 1,276 (0.7); decode, 1,024, 21 M 296 and 306 (0.6), 418 and 302 (0.7); 42 M 443 and 540 (0.65), 640 and 548 (0.7); 64 queues, 32 M 396
+// and 540 (0.65), 617 and 540 (0.7); prefix, 24 M, crowded on some queues at a time, 280 and 359 (0.2), 567 and 357 (0.3), 469 and 365 (0.7).
+float twice_from(uint64_t n, uint32_t n_queues) {
+    const double x = (double)twice_max(n_queues) / (double)std::max<uint64_t>(n, 1);
+    return (float)(0.70 - 0.40 * x * x);
+}
+TileBalance *inorder_decides(const SubmitArgs &a) {
+    const bool by_table = a.bal && a.bal->on && a.bal->dev;
+    return by_table && a.bal->depth_fixed == 0u && a.n > twice_max(a.mp.n_queues) && inorder_tile_map(a.n, a.sm_count, true).by_sm ? a.bal->dev : nullptr;
+}
 
 cudaError_t launch_inorder(const SubmitArgs &a, cudaStream_t st) {
     const uint64_t n = a.n;
@@ -1486,7 +1503,6 @@ cudaError_t launch_inorder(const SubmitArgs &a, cudaStream_t st) {
         const TileBalance &rec = *bal->pinned;
         if (rec.strag_seq != 0u && rec.strag_seq != bal->depth_seen && rec.strag_depth == bal->depth) {
             bal->depth_seen = rec.strag_seq;
-            if (2u * rec.strag_flagged >= n_tiles) bal->twice_left = kInTwiceRun;
             if (rec.strag_flagged != 0u) bal->depth = (uint32_t)kInHead;
             else if (rec.strag_max > 200u && bal->depth < (uint32_t)kInHead) ++bal->depth;
             else if (rec.strag_max < 148u && bal->depth > 3u) --bal->depth;
@@ -1495,9 +1511,8 @@ cudaError_t launch_inorder(const SubmitArgs &a, cudaStream_t st) {
     } else if (a.bal && a.bal->depth_fixed != 0u) {
         depth = std::min<uint32_t>(a.bal->depth_fixed, (uint32_t)kInHead);
     }
-    bool twice = n <= twice_max(a.mp.n_queues);
-    if (!twice && bal && bal->twice_left > 0u) { --bal->twice_left; twice = true; }
-    if (a.bal && a.bal->depth_fixed != 0u) twice = false;    // (the number of head entries is the caller's)
+    const bool twice = n <= twice_max(a.mp.n_queues) && !(a.bal && a.bal->depth_fixed != 0u);   // (a fixed number of head entries is the caller's)
+    const bool decided = inorder_decides(a) != nullptr;
     if (twice) depth = 0u;
     const uint64_t tile_records = tmap.max_tile;
     if (n_tiles > inorder_tiles_bound(n)) return cudaErrorInvalidValue;       // the workspace is carved for that many
@@ -1519,17 +1534,18 @@ cudaError_t launch_inorder(const SubmitArgs &a, cudaStream_t st) {
     const bool debt = a.claim_limit != nullptr;              // retention on: the kernels that apply the claims
     const uint32_t qid_stride = twice ? 0u : (uint32_t)std::min<uint64_t>(tile_records, kInQidPrefix);
     if ((uint64_t)n_tiles * qid_stride > inorder_qid_entries(n)) return cudaErrorInvalidValue;
-    auto serve = [&](bool again) {
-        auto pick = [&](auto full, auto second, auto light) { return again ? second : twice ? light : full; };
+    auto serve = [&](int mode) {
+        auto pick = [&](auto full, auto second, auto light) { return mode == kInAgain ? second : mode == kInLight ? light : full; };
         auto k = a.paged ? pick(k_inorder_serve<kInFull, false, true>, k_inorder_serve<kInAgain, false, true>, k_inorder_serve<kInLight, false, true>)
                : debt ? pick(k_inorder_serve<kInFull, true, false>, k_inorder_serve<kInAgain, true, false>, k_inorder_serve<kInLight, true, false>)
                       : pick(k_inorder_serve<kInFull, false, false>, k_inorder_serve<kInAgain, false, false>, k_inorder_serve<kInLight, false, false>);
         return launch_pdl(k, n_tiles, kInThreads, smem_serve, st, a.acc, n, tmap, a.ranges, a.mp, a.fast, a.ctrl, a.status, a.ws.in_agg,
                           a.stats_stage, a.completion, a.stall, (const int64_t *)a.ws.in_bin, tiles, heads, a.ws.in_headcnt,
                           (const int64_t *)a.busy, a.claim_limit, a.die_claims, debt ? *a.ret : RetDev{}, a.ws.in_qid, qid_stride,
-                          bal ? bal->dev : nullptr, bal_seq, make_fast_geom(a.fast, a.mp), depth, ordered_copy(n, a.ws));
+                          bal ? bal->dev : nullptr, bal_seq, make_fast_geom(a.fast, a.mp), depth, ordered_copy(n, a.ws), decided ? 1 : 0);
     };
-    cudaError_t le = serve(false);
+    cudaError_t le = twice ? serve(kInLight) : serve(kInFull);
+    if (le == cudaSuccess && decided) le = serve(kInLight);
     if (le == cudaSuccess)
         le = launch_pdl(k_inorder_scan, (R + kInScanQueues - 1) / kInScanQueues, dim3(kInScanQueues, kInScanChunks), 0, st, a.ctrl, a.mp_dev, n_tiles,
                         (const int64_t *)a.ws.in_agg, a.ws.in_bin, (const int64_t *)a.busy, a.busy_stage, a.stats_stage, a.path == HBF_PATH_INORDER ? 1 : 0);
@@ -1537,13 +1553,13 @@ cudaError_t launch_inorder(const SubmitArgs &a, cudaStream_t st) {
         le = launch_pdl(a.paged ? k_inorder_fixstraggle<false, true> : debt ? k_inorder_fixstraggle<true, false> : k_inorder_fixstraggle<false, false>, n_tiles, kInStrThreads,
                         smem_str, st, a.acc, n, tmap, a.ranges, a.mp, a.fast, a.ctrl, (const int64_t *)a.ws.in_bin, (const InHead *)heads, (const uint8_t *)a.ws.in_headcnt,
                         a.completion, a.stall, tiles, a.claim_limit, (const uint16_t *)a.ws.in_qid, qid_stride, depth, bal ? bal->dev : nullptr, ordered_copy(n, a.ws));
-    if (le == cudaSuccess) le = serve(true);
+    if (le == cudaSuccess) le = serve(kInAgain);
     if (le != cudaSuccess) return le;
     if (bal) {                                               // the tiles' times and straggler counts, for later batches; nothing waits for this copy
         cudaError_t e = cudaMemcpyAsync(bal->pinned, bal->dev, offsetof(TileBalance, first), cudaMemcpyDeviceToHost, st);
         if (e != cudaSuccess) return e;
     }
-    g_kernel_launches += twice ? 3 : 4;
+    g_kernel_launches += twice ? 3 : decided ? 5 : 4;
     return cudaGetLastError();
 }
 

@@ -92,6 +92,7 @@ k_begin_regroup(const __grid_constant__ BeginArgs b, const hbf_access_t *__restr
     const uint32_t limit = b.state->spin_limit;
     if (blockIdx.x == 0) {
         begin_batch(b, sorted ? 1 : 0, go ? 1u : 0u);
+        if (b.decides && !sorted) begin_load(b, reinterpret_cast<const uint64_t *>(acc + (uint64_t)tid * (n - 1ull) / 1024ull), bad ? first : ld_after(&acc[0].issue_ns), bad ? last : ld_after(&acc[n - 1].issue_ns));
         if (tid < 2) sync->claim[3 + tid] = 0u;              // (those of the last kernel)
         if (tid < 3) sync->done[3 + tid] = 0u;
         __threadfence();

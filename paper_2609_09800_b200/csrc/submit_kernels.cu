@@ -21,7 +21,7 @@ namespace hbf {
 // role 1: placed between the in-order attempt and the sort kernels; it starts the batch over for the
 //         sort path when the in-order attempt found the records out of issue order, else does nothing.
 // (a batch that may turn out to be out of issue order begins with k_begin_regroup)
-__global__ void k_begin(const __grid_constant__ BeginArgs b, int role, int run_sort) {
+__global__ void k_begin(const __grid_constant__ BeginArgs b, int role, int run_sort, const hbf_access_t *acc) {
     pdl_wait();
     pdl_trigger();
     if (role == 1) {
@@ -30,6 +30,8 @@ __global__ void k_begin(const __grid_constant__ BeginArgs b, int role, int run_s
     }
     __syncthreads();
     begin_batch(b, run_sort, 0u);
+    if (role == 0 && b.decides)
+        begin_load(b, reinterpret_cast<const uint64_t *>(acc + (uint64_t)threadIdx.x * (b.n - 1ull) / 1024ull), ld_after(&acc[0].issue_ns), ld_after(&acc[b.n - 1].issue_ns));
 }
 
 // =====================================================================================================
@@ -1146,8 +1148,8 @@ struct SortChain {
 // the radix sort's kernels, launched from the device (run_sort is set: the begin kernel starts the batch over)
 __device__ void launch_sort_chain(const SortChain &c, const FinishArgs &f, unsigned fin_grid) {
     cudaStream_t st = cudaStreamTailLaunch;
-    const BeginArgs b{c.ctrl, c.state, c.busy, c.busy_stage, c.stats_stage, c.hist, c.n_queues, c.n_dies, c.die_claims, c.claim_limit};
-    k_begin<<<1, 1024, 0, st>>>(b, 1, 1);
+    const BeginArgs b{c.ctrl, c.state, c.busy, c.busy_stage, c.stats_stage, c.hist, c.n_queues, c.n_dies, c.die_claims, c.claim_limit, nullptr, 0.0f, 0, 0, 0, 0};
+    k_begin<<<1, 1024, 0, st>>>(b, 1, 1, nullptr);
     k_zero_words<<<(unsigned)min((unsigned long long)((c.desc_words + 1023) / 1024), 592ull), 1024, 0, st>>>(c.desc0, c.desc_words);
     k_zero_words<<<(unsigned)min((unsigned long long)((c.scan_words + 1023) / 1024), 592ull), 1024, 0, st>>>((uint32_t *)c.scan_desc, c.scan_words);
     k_classify<<<c.cls_grid, kClsThreads, 0, st>>>(c.acc, c.n, c.ranges, c.mp_dev, c.ctrl, c.keys0, c.terms, c.status, c.completion, c.stall);
@@ -1254,10 +1256,11 @@ cudaError_t launch_submit(const SubmitArgs &a, cudaStream_t st) {
     const bool sort_kernels = a.path != HBF_PATH_INORDER || !a.inorder_ok;
     mark(0);
     {
-        const BeginArgs b{a.ctrl, a.state, a.busy, a.busy_stage, a.stats_stage, a.ws.hist, a.mp.n_queues, a.mp.n_dies, a.die_claims, a.claim_limit};
+        const BeginArgs b{a.ctrl, a.state, a.busy, a.busy_stage, a.stats_stage, a.ws.hist, a.mp.n_queues, a.mp.n_dies, a.die_claims, a.claim_limit,
+                          try_inorder ? inorder_decides(a) : nullptr, twice_from(n, a.mp.n_queues), n, a.mp.page_shift, a.mp.t_read_ns, a.mp.t_prog_ns};
         const cudaError_t e = try_inorder && sort_kernels && n >= 2
             ? launch_begin_regroup(a, b, st)
-            : launch_first(a.plain_next, k_begin, 1, 1024, 0, st, b, 0, try_inorder ? 0 : 1);
+            : launch_first(a.plain_next, k_begin, 1, 1024, 0, st, b, 0, try_inorder ? 0 : 1, a.acc);
         if (e != cudaSuccess) return e;
     }
     g_kernel_launches += 1;

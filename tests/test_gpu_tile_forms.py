@@ -84,3 +84,33 @@ def test_32_bit_form_matches_the_oracle(hbf, kind, n, entries):
             bg, bo = g.retention_blocks(), o.retention_blocks()
             assert np.array_equal(bg["disturb"], bo["disturb"]) and g.retention_totals() == o.retention_totals()
         acc["issue_ns"] += 50_000
+
+
+@pytest.mark.parametrize("declared", [False, True])
+def test_large_batches_of_changing_loads(hbf, declared):
+    """Too large for the host to tell whether their tiles are served twice: far behind, nearly idle and back, on queues that
+    start idle and on what the batch before left; the same as without measurements, where nothing is decided."""
+    import torch
+    n = 19_600_001                                           # fills a wave; 64 queues: above what is always served twice
+    prof = wl.load_profile("nominal", **wl.GEOMETRY["tiny"])
+    gen = torch.Generator(device="cuda"); gen.manual_seed(3)
+    rec = torch.empty((n, 3), dtype=torch.int64, device="cuda")
+    rec[:, 0] = BASE + 4096 * torch.randint(0, 1 << 18, (n,), device="cuda", generator=gen)
+    gaps = torch.randint(0, 1250, (n,), device="cuda", generator=gen)
+    rec[:, 2] = 4096
+    sides = []
+    for measured in (True, False):
+        g = hbf.Context(prof)
+        g.register_range(BASE, 1 << 30)
+        g.set_tile_balance(measured)
+        if declared: g.set_path(hbf.PATH_INORDER)
+        sides.append((g, [torch.empty(n, dtype=torch.int64, device="cuda") for _ in range(2)], torch.empty(n, dtype=torch.uint8, device="cuda")))
+    for turn, (load, reset) in enumerate([(3, True), (0.3, True), (3, True), (3, True), (0.3, False), (0.3, False), (0.9, True), (0.3, True), (3, True)]):
+        rec[:, 1] = torch.cumsum((gaps.double() / load).long(), 0) + (0 if reset else 10_000_000)
+        for g, out, status in sides:
+            if reset: g.reset()
+            assert g.submit_batch(rec, n, *out, status) == 0
+        (a, oa, sa), (b, ob, sb) = sides
+        assert a.last_result() == b.last_result() and a.last_result()["code"] == 0
+        assert torch.equal(oa[0], ob[0]) and torch.equal(oa[1], ob[1]) and torch.equal(sa, sb), turn
+        assert np.array_equal(a.get_busy_until(), b.get_busy_until()) and np.array_equal(a.get_pending_energy(), b.get_pending_energy())
