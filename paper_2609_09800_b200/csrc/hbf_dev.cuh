@@ -231,7 +231,7 @@ size_t inorder_head_bytes(uint64_t tiles, uint32_t n_queues);
 size_t inorder_serve_smem(uint32_t n_dies);
 // large batches whose own load decides whether their tiles are served twice (null: not such a batch)
 TileBalance *inorder_decides(const SubmitArgs &a);
-float twice_from(uint64_t n, uint32_t n_queues);
+float twice_from(uint64_t n, uint32_t n_queues, bool retention);
 cudaError_t launch_inorder(const SubmitArgs &a, cudaStream_t st);
 // batches out of issue order (regroup.cuh): the copy of the records that the in-order kernels serve, and its results
 struct OrderedCopy { const hbf_access_t *recs; int64_t *comp, *stall; };

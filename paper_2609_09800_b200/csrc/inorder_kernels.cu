@@ -1459,9 +1459,12 @@ static uint64_t twice_max(uint32_t n_queues) { return 5000000ull + 7500ull * n_q
 // 683 and 380 (0.65); 48 M 640 and 673 (0.55), 724 and 674 (0.6), 1,047 and 674 (0.65); 96 M 1,046 and 1,276 (0.6), 1,537 and
 // 1,276 (0.7); decode, 1,024, 21 M 296 and 306 (0.6), 418 and 302 (0.7); 42 M 443 and 540 (0.65), 640 and 548 (0.7); 64 queues, 32 M 396
 // and 540 (0.65), 617 and 540 (0.7); prefix, 24 M, crowded on some queues at a time, 280 and 359 (0.2), 567 and 357 (0.3), 469 and 365 (0.7).
-float twice_from(uint64_t n, uint32_t n_queues) {
+// (with retention the first pass counts the reads into the disturb counters, and the two meet at a lower load: 24 M at 0.5 in the case of 48 M with
+// claims 510 and 410; without it the line is drawn above where they meet near the smallest of these sizes, so that a batch at half load is
+// still measured by the full pass, whose times are what the tile sizes are for)
+float twice_from(uint64_t n, uint32_t n_queues, bool retention) {
     const double x = (double)twice_max(n_queues) / (double)std::max<uint64_t>(n, 1);
-    return (float)(0.70 - 0.40 * x * x);
+    return (float)(0.70 - (retention ? 0.40 : 0.22) * x * x);
 }
 TileBalance *inorder_decides(const SubmitArgs &a) {
     const bool by_table = a.bal && a.bal->on && a.bal->dev;

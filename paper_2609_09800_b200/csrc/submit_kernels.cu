@@ -1257,7 +1257,7 @@ cudaError_t launch_submit(const SubmitArgs &a, cudaStream_t st) {
     mark(0);
     {
         const BeginArgs b{a.ctrl, a.state, a.busy, a.busy_stage, a.stats_stage, a.ws.hist, a.mp.n_queues, a.mp.n_dies, a.die_claims, a.claim_limit,
-                          try_inorder ? inorder_decides(a) : nullptr, twice_from(n, a.mp.n_queues), n, a.mp.page_shift, a.mp.t_read_ns, a.mp.t_prog_ns};
+                          try_inorder ? inorder_decides(a) : nullptr, twice_from(n, a.mp.n_queues, a.claim_limit != nullptr), n, a.mp.page_shift, a.mp.t_read_ns, a.mp.t_prog_ns};
         const cudaError_t e = try_inorder && sort_kernels && n >= 2
             ? launch_begin_regroup(a, b, st)
             : launch_first(a.plain_next, k_begin, 1, 1024, 0, st, b, 0, try_inorder ? 0 : 1, a.acc);
