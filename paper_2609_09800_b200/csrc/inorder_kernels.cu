@@ -171,9 +171,6 @@ __device__ __forceinline__ uint64_t head_slot(uint32_t tile, uint32_t R, uint32_
 // The extra operands are not used by the instruction: naming them makes the compiler finish computing them
 // before the wait instead of after it.  The aligned forms of the barrier instructions are used (measured a
 // little faster): like __syncthreads(), they sit where the warp's control flow is uniform.
-__device__ __forceinline__ void row_wait(int id, int64_t m, long long s8, const void *pq, uint32_t pc, bool last) {
-    asm volatile("barrier.cta.sync.aligned %0, 64;" ::"r"(id), "l"(m), "l"(s8), "l"(pq), "r"(pc), "r"((int)last) : "memory");
-}
 __device__ __forceinline__ void row_pass(int id) { asm volatile("barrier.cta.arrive.aligned %0, 64;" ::"r"(id) : "memory"); }
 
 __device__ __forceinline__ void row_wait2(int id, int64_t m, long long s8, const void *pq, uint32_t pc, bool last,
@@ -200,9 +197,14 @@ __device__ __forceinline__ void row_wait2(int id, int64_t m, long long s8, const
 // row); with everything around it 790 -> 503.  (In the 64-bit form the slots cost mixed batches 4 %: it keeps the queue's number.)
 // What the form cannot hold (a time 2^31 ns or more past the tile's first, by a gap in the stream or by a backlog) is
 // only noticed, in bits that are OR-ed along; such a tile is then served again in the 64-bit form.
-// Queue state (16 bytes): busy-until, service time in this tile, read granules, reads << 4 | head entries written.
+// Queue state (16 bytes; the first 8 or 4 in the other two modes below): busy-until, service time in this tile, read granules,
+// reads << 4 | head entries written.
 // ======================================================================================================
-// what a launch of the pass does: all of it; the results only, from known busy-until; all but the results and the head entries
+// What a launch of the pass does: all of it; the results only, from known busy-until; what those follow from only, a map per queue.
+// Where the second follows the third (the tile's `reserve` is 2) it also counts what the third leaves out: bytes and accesses per die
+// and claims.  The chain of updates then carries 8 bytes a queue and 4, where all 16 take four times the shared memory's turns (4 M decode
+// reads 117.6 -> 111.9 us, 24 M prefix records 397 -> 385, first half of 48 M with retention: light 216 -> 199, again 184 -> 174).  Read
+// disturb stays with the third: its atomics, all over the L2, take 50 us of a 24 M batch there and 105 beside the stores of the results.
 enum { kInFull = 0, kInAgain = 1, kInLight = 2 };
 struct NarrowSums { uint32_t native, fault, max_done; unsigned unsorted, over; long long stall; };
 
@@ -217,15 +219,20 @@ __device__ __forceinline__ void row_wait_n(int id, uint32_t m, uint32_t s, const
 }
 
 // MODE: see k_inorder_serve.  Everything per queue goes by the queue's slot.
+// count: see kInLight (a pass that knows its busy-until).
 template <int MODE, bool DEBT, bool PAGED>
 __device__ __forceinline__ NarrowSums serve_narrow(const FastGeom &geom, const ModelParams &mp, const ModelParams &mp_arg, const hbf_access_t *acc_t, const uint32_t tile_begin,
                                                    const uint32_t tile_len, const int64_t T0, uint4 *qst, uint8_t *warp_tag, uint8_t *status_t,
                                                    uint16_t *qid_t, const uint32_t qid_stride, int64_t *completion_t, int64_t *stall_t,
                                                    InHead *__restrict__ in_head, const uint32_t tile, const uint32_t R, const uint32_t head_depth,
                                                    uint32_t *s_heads_full, uint32_t *st_br_lo, const uint32_t n_dies,
-                                                   const uint64_t claim_limit, const uint32_t quantum_ns, const RetDev &ret, const uint32_t ret_row_shift) {
+                                                   const uint64_t claim_limit, const uint32_t quantum_ns, const RetDev &ret, const uint32_t ret_row_shift, const bool count) {
     constexpr bool RESERVE = MODE == kInAgain, LIGHT = MODE == kInLight;
+    const bool counts = MODE == kInFull || (RESERVE && count);
     constexpr int K = kInRows;
+    using State = typename std::conditional<RESERVE, uint32_t, typename std::conditional<LIGHT, uint2, uint4>::type>::type;
+    const uint32_t die_mask = (1u << geom.chdie_shift) - 1u;
+    uint32_t *st_gran = reinterpret_cast<uint32_t *>(qst) + kInMaxQueues;      // (counting with known busy-until: read granules by the low bits of the slot)
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     uint32_t *st_br_hi = st_br_lo + n_dies, *st_bp_lo = st_br_hi + n_dies, *st_bp_hi = st_bp_lo + n_dies, *st_nr = st_bp_hi + n_dies, *st_np = st_nr + n_dies, *st_claims = st_np + n_dies;
     NarrowSums r; r.native = 0; r.fault = 0; r.max_done = 0; r.unsorted = 0; r.over = 0; r.stall = 0;
@@ -290,7 +297,7 @@ __device__ __forceinline__ NarrowSums serve_narrow(const FastGeom &geom, const M
                 if (flags == 0u) {
                     const uint32_t g = (bytes + ((1u << geom.gran_shift_read) - 1u)) >> geom.gran_shift_read;
                     S[u] = npages * geom.t_read; xo[u] = nw_transfer(geom, g, geom.nw_mul_read);
-                    gn[u] = g | (1u << kNwCountShift);
+                    uint32_t parts = 1u, sum = g;
                     if (PAGED && npages > 1u) {              // (see paged_terms)
                         const uint32_t head = geom.page_mask + 1u - in_page, tail = in_page + bytes - (npages - 1u) * (geom.page_mask + 1u), gm = (1u << geom.gran_shift_read) - 1u;
                         const uint32_t gh = (head + gm) >> geom.gran_shift_read, gt = (tail + gm) >> geom.gran_shift_read;
@@ -298,9 +305,11 @@ __device__ __forceinline__ NarrowSums serve_narrow(const FastGeom &geom, const M
                         int32_t x = max((int32_t)nw_transfer(geom, gt, geom.nw_mul_read), (int32_t)nw_transfer(geom, gh, geom.nw_mul_read) - (int32_t)(npages - 1u) * s1);
                         if (npages > 2u) x = max(x, (int32_t)geom.nw_page_read - s1);
                         xo[u] = (uint32_t)x;
-                        gn[u] = (gh + gt + (npages - 2u) * geom.nw_page_gran) | (npages << kNwCountShift);
+                        parts = npages; sum = gh + gt + (npages - 2u) * geom.nw_page_gran;
                     }
                     M[u] = ri[u] + S[u];
+                    if (MODE == kInFull) gn[u] = sum | (parts << kNwCountShift);
+                    else if (counts) { atomicAdd(&st_gran[q[u] & die_mask], sum); atomicAdd(&st_nr[slot_die(geom, q[u])], parts); }
                 } else {                                     // a program: its data is transferred first; bytes and count by atomics
                     uint32_t g = (bytes + ((1u << geom.gran_shift_prog) - 1u)) >> geom.gran_shift_prog, xf = nw_transfer(geom, g, geom.nw_mul_prog);
                     S[u] = npages * geom.t_prog;
@@ -314,7 +323,7 @@ __device__ __forceinline__ NarrowSums serve_narrow(const FastGeom &geom, const M
                     }
                     xo[u] = xf | 0x80000000u;
                     M[u] = ri[u] + xf + S[u];
-                    if (!RESERVE) {
+                    if (counts) {
                         const uint32_t die = slot_die(geom, q[u]), lo = g << geom.gran_shift_prog;
                         atomicAdd(&st_np[die], PAGED ? npages : 1u);
                         const uint32_t old = atomicAdd(&st_bp_lo[die], lo);
@@ -323,7 +332,7 @@ __device__ __forceinline__ NarrowSums serve_narrow(const FastGeom &geom, const M
                 }
                 if (DEBT && tile_begin + i[u] < claim_limit) {
                     S[u] += quantum_ns; M[u] += quantum_ns;
-                    if (!RESERVE) atomicAdd(&st_claims[slot_die(geom, q[u])], 1u);
+                    if (counts) atomicAdd(&st_claims[slot_die(geom, q[u])], 1u);
                 }
             } else if (valid[u]) {                           // near the range's end, large, or not modeled
                 unsigned lng = 0;
@@ -334,14 +343,14 @@ __device__ __forceinline__ NarrowSums serve_narrow(const FastGeom &geom, const M
                     ready[u] = true; q[u] = queue_slot(geom, v.queue);
                     if (lng || ((uint64_t)v.s >> (kNwServeBits - 1)) || (v.xfer >> 30)) b_time |= 0x80000000u;
                     S[u] = (uint32_t)v.s; xo[u] = v.xfer | (v.op << 31);
-                    if (!RESERVE) {
+                    if (counts) {
                         const uint32_t lo = (uint32_t)v.cb, hi = (uint32_t)((uint64_t)v.cb >> 32);
                         uint32_t *plo = v.op ? st_bp_lo : st_br_lo, *phi = v.op ? st_bp_hi : st_br_hi;
                         atomicAdd(v.op ? &st_np[v.die] : &st_nr[v.die], v.parts);
                         const uint32_t old = atomicAdd(&plo[v.die], lo), carry = hi + ((old + lo) < old ? 1u : 0u);
                         if (carry) atomicAdd(&phi[v.die], carry);
                     }
-                    if (DEBT && tile_begin + i[u] < claim_limit) { S[u] += quantum_ns; if (!RESERVE) atomicAdd(&st_claims[v.die], 1u); }
+                    if (DEBT && tile_begin + i[u] < claim_limit) { S[u] += quantum_ns; if (counts) atomicAdd(&st_claims[v.die], 1u); }
                     M[u] = ri[u] + (v.op ? v.xfer : 0u) + S[u];
                 } else if (v.st == HBF_ST_NATIVE) {
                     r.native += 1u;
@@ -384,7 +393,7 @@ __device__ __forceinline__ NarrowSums serve_narrow(const FastGeom &geom, const M
         constexpr bool HEADS = decltype(heads_tag)::value;
         uint32_t rank1[K], pc[K], c0[K], c1[K], m_own[K], s_own[K], B[K];
         bool last[K];
-        uint4 *pq[K];
+        State *pq[K];
 #pragma unroll
         for (int u = 0; u < K; ++u) {
             rank1[u] = 1u; last[u] = ready[u]; pc[u] = HEADS ? 1u : 0u;
@@ -397,7 +406,7 @@ __device__ __forceinline__ NarrowSums serve_narrow(const FastGeom &geom, const M
                 if (!__any_sync(0xffffffffu, loser && t2 != (uint32_t)lane)) {
                     const uint32_t peer = loser ? tagged[u] : t2;                  // the lane itself when it has none
                     const bool second = peer < (uint32_t)lane;
-                    const uint32_t mp_ = __shfl_sync(0xffffffffu, M[u], (int)peer), sp_ = __shfl_sync(0xffffffffu, S[u], (int)peer), gp_ = __shfl_sync(0xffffffffu, gn[u], (int)peer);
+                    const uint32_t mp_ = __shfl_sync(0xffffffffu, M[u], (int)peer), sp_ = __shfl_sync(0xffffffffu, S[u], (int)peer), gp_ = MODE == kInFull ? __shfl_sync(0xffffffffu, gn[u], (int)peer) : 0u;
                     if (second) { M[u] = max(mp_ + S[u], M[u]); S[u] += sp_; gn[u] += gp_; rank1[u] = 2u; }
                     if (peer > (uint32_t)lane) last[u] = false;
                     if (HEADS && peer != (uint32_t)lane) pc[u] = 2u;
@@ -412,19 +421,27 @@ __device__ __forceinline__ NarrowSums serve_narrow(const FastGeom &geom, const M
                     const uint32_t n_max = __reduce_max_sync(0xffffffffu, rank1[u]);
                     for (uint32_t span = 1; span < n_max; span <<= 1) {
                         const int src = prev_l >= 0 ? prev_l : lane;
-                        const uint32_t Se = __shfl_sync(0xffffffffu, S[u], src), Me = __shfl_sync(0xffffffffu, M[u], src), ge = __shfl_sync(0xffffffffu, gn[u], src);
+                        const uint32_t Se = __shfl_sync(0xffffffffu, S[u], src), Me = __shfl_sync(0xffffffffu, M[u], src), ge = MODE == kInFull ? __shfl_sync(0xffffffffu, gn[u], src) : 0u;
                         const int pe = __shfl_sync(0xffffffffu, prev_l, src);
                         if (prev_l >= 0) { M[u] = max(Me + S[u], M[u]); S[u] += Se; gn[u] += ge; prev_l = pe; }
                     }
                 }
             }
-            pq[u] = qst + q[u];
+            pq[u] = reinterpret_cast<State *>(qst) + q[u];
         }
         // ---- the queue updates, in row order
         if (turn > 0) row_wait_n(my_bar, M[0], S[0], pq[0], gn[0], last[0], M[K - 1], S[K - 1], pq[K - 1], gn[K - 1], last[K - 1]);
 #pragma unroll
         for (int u = 0; u < K; ++u) {
-            const uint4 state = *pq[u];
+            if (u > 0) __syncwarp();                         // (the row before may hold the same queues)
+            const State state = *pq[u];
+            if constexpr (RESERVE) {
+                B[u] = max(state + S[u], M[u]);
+                if (last[u]) *pq[u] = B[u];
+            } else if constexpr (LIGHT) {
+                B[u] = max(state.x + S[u], M[u]);
+                if (last[u]) *pq[u] = make_uint2(B[u], state.y + S[u]);
+            } else {
             B[u] = max(state.x + S[u], M[u]);
             uint32_t inc = 0u;
             if (HEADS) {
@@ -433,7 +450,7 @@ __device__ __forceinline__ NarrowSums serve_narrow(const FastGeom &geom, const M
                 c1[u] = c0[u] + inc;
             }
             if (last[u]) *pq[u] = make_uint4(B[u], state.y + S[u], state.z + (gn[u] & ((1u << kNwCountShift) - 1u)), state.w + ((gn[u] >> kNwCountShift) << 4) + inc);
-            if (u + 1 < K) __syncwarp();
+            }
         }
         if (turn + 1 < turns) row_pass(next_bar);
         // ---- results
@@ -496,6 +513,7 @@ k_inorder_serve(const hbf_access_t *__restrict__ acc, uint64_t n, const __grid_c
         bal->twice_load = ctrl->load; bal->twice_left = kInTwiceRun;
     }
     if (RESERVE && (!ctrl->inorder_used || !in_tile[blockIdx.x].reserve)) return;
+    const bool count = RESERVE && in_tile[blockIdx.x].reserve == 2u, counts = MODE == kInFull || count;
     if (ctrl->regrouped) { acc = copy.recs; completion = copy.comp; stall = copy.stall; status = nullptr; }   // (brought into order: regroup_kernels.cu)
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const RangeSnap &rs = *ranges_g;                      // read through the cache; the common configuration does not touch it
@@ -579,7 +597,8 @@ k_inorder_serve(const hbf_access_t *__restrict__ acc, uint64_t n, const __grid_c
             (uint64_t)tile_len * geom.nw_gmax < (1ull << 32) && (uint64_t)quantum_ns < (1ull << (kNwServeBits - 1))) {
             uint4 *q4 = reinterpret_cast<uint4 *>(qst);
             unsigned over = 0;
-            if (!RESERVE) for (uint32_t d = tid; d < n_dies * 7u; d += kInThreads) st_br_lo[d] = 0u;
+            if (counts) for (uint32_t d = tid; d < n_dies * 7u; d += kInThreads) st_br_lo[d] = 0u;
+            if (count) for (uint32_t d = tid; d < n_dies; d += kInThreads) reinterpret_cast<uint32_t *>(qst)[kInMaxQueues + d] = 0u;
             for (uint32_t q = tid; q < kInMaxQueues; q += kInThreads) {
                 uint4 v = make_uint4(0u, 0u, 0u, 0u);
                 if ((RESERVE || (MODE == kInFull && tile == 0u)) && q < R) {   // the first tile knows its entering state: it is served exactly
@@ -587,14 +606,15 @@ k_inorder_serve(const hbf_access_t *__restrict__ acc, uint64_t n, const __grid_c
                     v.x = b > 0 ? (uint32_t)b : 0u;
                     if (b >= (RESERVE ? 1ll << 30 : 1ll << 31)) over = 1u;
                 }
-                q4[q < R ? queue_slot(geom, q) : q] = v;
+                const uint32_t at = q < R ? queue_slot(geom, q) : q;
+                if (RESERVE) reinterpret_cast<uint32_t *>(qst)[at] = v.x; else if (LIGHT) reinterpret_cast<uint2 *>(qst)[at] = make_uint2(0u, 0u); else q4[at] = v;
             }
             // (a backlog that reaches far into the tile grows while the tile is served: not even tried then)
             const bool try_narrow = __syncthreads_or((int)over) == 0;
             NarrowSums nw{};
             if (try_narrow) nw = serve_narrow<MODE, DEBT, PAGED>(geom, mp, mp_arg, acc_t, (uint32_t)tile_begin, tile_len, T0, q4, warp_tag, status_t, qid_t, qid_stride,
                                                      completion_t, stall_t, in_head, tile, R, head_depth, &s_heads_full, st_br_lo, n_dies, claim_limit,
-                                                     (uint32_t)quantum_ns, ret, ret_row_shift);
+                                                     (uint32_t)quantum_ns, ret, ret_row_shift, count);
             if (__syncthreads_or((int)(over | nw.over)) == 0) {
                 narrow_done = true;
                 sum_stall = nw.stall;
@@ -605,11 +625,12 @@ k_inorder_serve(const hbf_access_t *__restrict__ acc, uint64_t n, const __grid_c
                     t_native = nw.native; t_fault = nw.fault; t_ready = (tid == 0 ? (long long)tile_len : 0ll) - t_native - t_fault;
                     longlong2 *out = reinterpret_cast<longlong2 *>(in_agg) + (uint64_t)tile * R;
                     for (uint32_t q = tid; q < R; q += kInThreads) {
-                        const uint4 v = q4[queue_slot(geom, q)];
+                        uint2 v;                             // busy-until, service time
+                        if (LIGHT) v = reinterpret_cast<const uint2 *>(qst)[queue_slot(geom, q)];
+                        else { const uint4 f = q4[queue_slot(geom, q)]; v = make_uint2(f.x, f.y); in_headcnt[(uint64_t)tile * R + q] = (uint8_t)(f.w & 15u); }
                         out[q] = make_longlong2((long long)(uint64_t)v.y, v.y ? T0 + (int64_t)(uint64_t)v.x : kNegInf);   // (no service time: no access)
-                        if (!LIGHT) in_headcnt[(uint64_t)tile * R + q] = (uint8_t)(v.w & 15u);
                     }
-                    for (uint32_t d = tid; d < n_dies; d += kInThreads) {              // a die's reads: the sums its queues carry
+                    if (MODE == kInFull) for (uint32_t d = tid; d < n_dies; d += kInThreads) {              // a die's reads: the sums its queues carry
                         unsigned long long g = 0, cnt = 0;
                         for (uint32_t p = 0; p < geom.planes_q; ++p) { const uint4 v = q4[queue_slot(geom, d * geom.planes_q + p)]; g += v.z; cnt += v.w >> 4; }
                         unsigned long long *gd = reinterpret_cast<unsigned long long *>(stats_stage + d);
@@ -617,6 +638,11 @@ k_inorder_serve(const hbf_access_t *__restrict__ acc, uint64_t n, const __grid_c
                         if (cnt) atomicAdd(&gd[4], cnt);
                     }
                 }
+                if (count)
+                    for (uint32_t d = tid; d < n_dies; d += kInThreads) {              // (d: channel, then die)
+                        const uint32_t g = reinterpret_cast<const uint32_t *>(qst)[kInMaxQueues + d];
+                        if (g) atomicAdd(reinterpret_cast<unsigned long long *>(stats_stage + slot_die(geom, d)) + 1, (unsigned long long)g << geom.gran_shift_read);
+                    }
             } else {
                 again = try_narrow;                          // (its read disturb is counted)
                 if (tid == 0) s_heads_full = 0u;
@@ -624,12 +650,12 @@ k_inorder_serve(const hbf_access_t *__restrict__ acc, uint64_t n, const __grid_c
         }
     }
     if (!narrow_done) {
-    for (uint32_t i = tid; i < kInMaxQueues; i += kInThreads) qst[i] = make_longlong2(kNegInf, 0);
+    using State = typename std::conditional<RESERVE, int64_t, longlong2>::type;   // (with known busy-until: that alone)
+    if (counts) for (uint32_t d = tid; d < n_dies * 7u; d += kInThreads) st_br_lo[d] = 0u;
     if (RESERVE) {
-        __syncthreads();
-        for (uint32_t q = tid; q < R; q += kInThreads) qst[q].x = ld_after(in_bin + (uint64_t)blockIdx.x * R + q);
+        for (uint32_t q = tid; q < kInMaxQueues; q += kInThreads) reinterpret_cast<int64_t *>(qst)[q] = q < R ? ld_after(in_bin + (uint64_t)blockIdx.x * R + q) : kNegInf;
     } else {
-        for (uint32_t d = tid; d < n_dies * 7u; d += kInThreads) st_br_lo[d] = 0u;
+        for (uint32_t i = tid; i < kInMaxQueues; i += kInThreads) qst[i] = make_longlong2(kNegInf, 0);
         if (MODE == kInFull && tile == 0u) {                 // the first tile knows its entering state: it is served exactly
             __syncthreads();
             for (uint32_t q = tid; q < R; q += kInThreads) qst[q].x = busy[q];
@@ -677,7 +703,7 @@ k_inorder_serve(const hbf_access_t *__restrict__ acc, uint64_t n, const __grid_c
         int64_t issue[K], a[K], S[K], M[K], B[K];
         Served v[K];
         uint32_t rank1[K], pc[K], c0[K], c1[K], qi[K];
-        longlong2 *pq[K];
+        State *pq[K];
         int64_t prev[K];
         uint64_t addr[K], bf[K];
 #pragma unroll
@@ -706,7 +732,7 @@ k_inorder_serve(const hbf_access_t *__restrict__ acc, uint64_t n, const __grid_c
             if (PAGED && ready[u]) paged_terms(mp, media_offset_of(rs, fast_range, fast_on, addr[u], issue[u], bf[u]), (uint32_t)bf[u], q_ppm, div_q, c_unsorted, 33, v[u]);
             if (DEBT && ready[u] && tile_begin + i[u] < claim_limit) {
                 v[u].s += quantum_ns;
-                if (!RESERVE) atomicAdd(&st_claims[v[u].die], 1u);
+                if (counts) atomicAdd(&st_claims[v[u].die], 1u);
             }
             if (DEBT && !RESERVE && ready[u] && !v[u].op && !again) {  // read disturb (counted already when the tile is served again): the read's pages, on the block of its first page
                 if (fast_on && ret.pow2 != 0u) {
@@ -743,16 +769,18 @@ k_inorder_serve(const hbf_access_t *__restrict__ acc, uint64_t n, const __grid_c
             for (int u = 0; u < K; ++u)
                 if (valid[u]) qid_t[i[u]] = ready[u] ? (uint16_t)v[u].queue : (uint16_t)kInMaxQueues;   // (one past the last queue: not modeled)
         }
-        if (!RESERVE) {
+        if (!RESERVE || counts) {
 #pragma unroll
             for (int u = 0; u < K; ++u) {
                 if (valid[u]) {
-                    c_unsorted |= issue[u] < prev[u] ? 1u : 0u;
-                    if (status_t) status_t[i[u]] = (uint8_t)v[u].st;
-                    c_valid += 1u;
-                    c_ready += ready[u] ? 1u : 0u;
-                    c_native += v[u].st == HBF_ST_NATIVE ? 1u : 0u;
-                    if (ready[u]) {
+                    if (!RESERVE) {
+                        c_unsorted |= issue[u] < prev[u] ? 1u : 0u;
+                        if (status_t) status_t[i[u]] = (uint8_t)v[u].st;
+                        c_valid += 1u;
+                        c_ready += ready[u] ? 1u : 0u;
+                        c_native += v[u].st == HBF_ST_NATIVE ? 1u : 0u;
+                    }
+                    if (counts && ready[u]) {
                         // charged bytes < 2^33: add the low word, carry into the high word when it wraps (a form that counts
                         // granules in one word and sends oversized accesses to the 64-bit totals measured slower)
                         const uint32_t lo = (uint32_t)v[u].cb, hi = (uint32_t)((uint64_t)v[u].cb >> 32);
@@ -818,16 +846,18 @@ k_inorder_serve(const hbf_access_t *__restrict__ acc, uint64_t n, const __grid_c
                 }
             }
             qi[u] = ready[u] ? v[u].queue : 0u;
-            pq[u] = qst + qi[u];
+            pq[u] = reinterpret_cast<State *>(qst) + qi[u];
         }
         // ---- the queue updates, in row order: everything they need is in registers before the wait ---------------
-        if (turn > 0) {
-            if (K == 1) row_wait(my_bar, M[0], S[0], pq[0], pc[0], last[0]);
-            else row_wait2(my_bar, M[0], S[0], pq[0], pc[0], last[0], M[K - 1], S[K - 1], pq[K - 1], pc[K - 1], last[K - 1]);
-        }
+        if (turn > 0) row_wait2(my_bar, M[0], S[0], pq[0], pc[0], last[0], M[K - 1], S[K - 1], pq[K - 1], pc[K - 1], last[K - 1]);
 #pragma unroll
         for (int u = 0; u < K; ++u) {
-            const longlong2 state = *pq[u];
+            if (u > 0) __syncwarp();                         // (the row before may hold the same queues)
+            const State state = *pq[u];
+            if constexpr (RESERVE) {
+                B[u] = max((int64_t)(state + S[u]), M[u]);
+                if (last[u]) *pq[u] = B[u];
+            } else {
             B[u] = max((int64_t)(state.x + S[u]), M[u]);
             uint32_t inc = 0u;
             if (HEADS) {
@@ -836,7 +866,7 @@ k_inorder_serve(const hbf_access_t *__restrict__ acc, uint64_t n, const __grid_c
                 c1[u] = c0[u] + inc;
             }
             if (last[u]) *pq[u] = make_longlong2(B[u], state.y + (S[u] << 8) + (long long)inc);
-            if (u + 1 < K) __syncwarp();                     // the next row may hold the same queues
+            }
         }
         if (turn + 1 < turns) row_pass(next_bar);
         // ---- results ---------------------------------------------------------------------------------------
@@ -876,7 +906,7 @@ k_inorder_serve(const hbf_access_t *__restrict__ acc, uint64_t n, const __grid_c
         }
     }
     }                                                        // (the 64-bit form)
-    if (!RESERVE) {
+    if (counts) {
         for (uint32_t d = tid; d < n_dies; d += kInThreads) {
             unsigned long long *g = reinterpret_cast<unsigned long long *>(stats_stage + d);
             const unsigned long long br = ((unsigned long long)st_br_hi[d] << 32) | st_br_lo[d];
@@ -887,6 +917,8 @@ k_inorder_serve(const hbf_access_t *__restrict__ acc, uint64_t n, const __grid_c
             if (st_np[d]) atomicAdd(&g[5], (unsigned long long)st_np[d]);
             if (DEBT && st_claims[d]) atomicAdd(&die_claims[d], st_claims[d]);
         }
+    }
+    if (!RESERVE) {
         const unsigned long long w_native = (unsigned long long)warp_sum(t_native);
         const unsigned long long w_ready = (unsigned long long)warp_sum(t_ready);        // (a warp's share may be negative: the sum over the tile counts)
         const unsigned long long w_fault = (unsigned long long)warp_sum(t_fault);
@@ -903,7 +935,7 @@ k_inorder_serve(const hbf_access_t *__restrict__ acc, uint64_t n, const __grid_c
     __syncthreads();
     if (tid == 0) {
         if (RESERVE) in_tile[tile].true_sum = s_red[0];
-        else { InTile t; t.spec_sum = s_red[0]; t.fix_delta = 0; t.true_sum = 0; t.reserve = LIGHT ? 1u : 0u; t.stragglers = 0u; in_tile[tile] = t; }
+        else { InTile t; t.spec_sum = s_red[0]; t.fix_delta = 0; t.true_sum = 0; t.reserve = LIGHT ? 2u : 0u; t.stragglers = 0u; in_tile[tile] = t; }
         if (s_red[1] != INT64_MIN) atomicMax(&ctrl->max_completion_ns, s_red[1]);
         if (!RESERVE && bal) {                               // how many records, how long: what the next batches' tile sizes follow from
             unsigned long long now;
