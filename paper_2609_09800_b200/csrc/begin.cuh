@@ -8,6 +8,7 @@ struct BeginArgs {
     BatchCtrl *ctrl; const DevState *state; const int64_t *busy; int64_t *busy_stage; hbf_die_stats_t *stats_stage; uint32_t *hist;
     uint32_t n_queues, n_dies; uint32_t *die_claims; const unsigned long long *claim_limit;
     TileBalance *decides; float twice_from; uint64_t n; uint32_t page_shift; int64_t t_read_ns, t_prog_ns;   // see begin_load (decides: null, not asked)
+    const RangeSnap *ranges; uint32_t unit_shift;            // see begin_units (0: not asked)
 };
 
 // 1,024 pairs of neighbouring records (n >= 2; blocks of 1,024 threads): are they out of order, and what span of time does this
@@ -74,6 +75,16 @@ __device__ __forceinline__ void begin_load(const BeginArgs &a, const uint64_t *r
     a.ctrl->load = load;
     if (load >= a.twice_from) a.ctrl->twice = 1u;
     else if (a.decides->twice_left > 0u && load >= 0.9f * a.decides->twice_load) { a.ctrl->twice = 1u; a.decides->twice_left -= 1u; }
+}
+
+// Does one of 1,024 sampled records reach over the end of its stripe unit?  Then the first pass is spared (a batch in which only others do is
+// noticed by that pass).  One block of 1,024 threads, behind begin_batch; rec: this thread's sample.
+__device__ __forceinline__ void begin_units(const BeginArgs &a, const uint64_t *rec) {
+    const uint64_t addr = ld_after(rec), bf = ld_after(rec + 2), unit = 1ull << a.unit_shift;
+    int g = 0;
+    if (classify(*a.ranges, addr, (int64_t)ld_after(rec + 1), (uint32_t)bf, (uint32_t)(bf >> 32), &g) != HBF_ST_READY) return;
+    const uint64_t off = a.ranges->media_offset[g] + (addr - a.ranges->base[g]);
+    if ((off & (unit - 1ull)) + (uint32_t)bf > unit) a.ctrl->crossed = 1u;
 }
 
 }  // namespace hbf

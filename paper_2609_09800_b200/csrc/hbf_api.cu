@@ -74,12 +74,13 @@ struct hbf_ctx {
     bool terminal = false;           // a shutdown result has been observed
     // device state
     RangeSnap *d_ranges = nullptr; ModelParams *d_mp = nullptr; DevState *d_state = nullptr;
-    BatchCtrl *d_ctrl = nullptr; RegroupSync *d_rg_sync = nullptr; hbf_batch_result_t *d_result = nullptr;
+    BatchCtrl *d_ctrl = nullptr, *d_ctrl_spare = nullptr; RegroupSync *d_rg_sync = nullptr; hbf_batch_result_t *d_result = nullptr;
     int64_t *d_busy = nullptr, *d_busy_stage = nullptr, *d_pending = nullptr; hbf_die_stats_t *d_stats_stage = nullptr;
     // pinned: the last batch's summary (written by its last kernel), part counts on their way back, the hotspots (written by the
     // thermal step), the tiles' times
     struct Pinned { hbf_batch_result_t result, host_sum; RetState ret; unsigned long long ret_waiting; unsigned long long totals[kPagedTotals]; float hot[4]; TileBalance bal; } *pinned = nullptr;
     bool result_on_host = false;                 // pinned->result is the last batch's summary (small batches leave theirs on the device only)
+    bool paged_crossed = false;                  // some access of the last page-granular batch reached over the end of its stripe unit
     bool captured = false;                       // a batch was captured into a graph: which batch ran last is not for the host to know
     StreamNote *note = nullptr;                  // of the stream
     TileBalanceHost bal;                         // tile sizes of the in-order path from the times earlier batches left
@@ -388,7 +389,7 @@ int hbf_create(const hbf_config_t *cfg, void *cuda_stream, hbf_ctx **out) {
     arena.add(&c->d_ranges, nullptr, 1);
     arena.add(&c->d_mp, nullptr, 1);
     arena.add(&c->d_state, &st0, 1);
-    arena.add(&c->d_ctrl, nullptr, 1);
+    arena.add(&c->d_ctrl, nullptr, 1); arena.add(&c->d_ctrl_spare, nullptr, 1);
     arena.add(&c->d_rg_sync, nullptr, 1);
     arena.add(&c->d_result, nullptr, 1);
     arena.add(&c->d_busy, nullptr, nq);
@@ -766,6 +767,7 @@ size_t hbf_workspace_bytes_paged(const hbf_ctx *c, uint64_t n, uint64_t parts_ca
     return paged_layout(n, std::max<uint64_t>(parts_capacity, n), c->mp.n_queues, c->mp.channels, rooms_wanted(c), nullptr, nullptr, c->d_bus_busy ? 1 : 0);
 }
 
+constexpr uint64_t kPagedLookFirst = 400000;                 // accesses (see below)
 int hbf_submit_batch_paged(hbf_ctx *c, const hbf_access_t *d_acc, uint64_t n, uint64_t parts_capacity,
                            int64_t *d_completion_ns, int64_t *d_stall_ns, uint8_t *d_status, hbf_die_stats_t *d_die_stats,
                            void *d_workspace, size_t workspace_bytes) {
@@ -797,26 +799,49 @@ int hbf_submit_batch_paged(hbf_ctx *c, const hbf_access_t *d_acc, uint64_t n, ui
                    n > kInSmallMax && c->mp.stripe_shift < 31u;
     // how many parts: the one point where the host waits for the device inside a submit
     unsigned long long *h_total = c->pinned->totals;
-    auto count = [&](bool unit) -> int {
-        CK(launch_paged_count(d_acc, n, c->d_ranges, c->d_mp, fast, c->mp, c->d_state, unit, pw, c->stream));
+    auto count = [&](bool unit, const BatchCtrl *looked) -> int {
+        CK(launch_paged_count(d_acc, n, c->d_ranges, c->d_mp, fast, c->mp, c->d_state, unit, looked, pw, c->stream));
         CK(cudaMemcpyAsync(h_total, pw.total, kPagedTotals * sizeof(unsigned long long), cudaMemcpyDeviceToHost, c->stream));
         CK(cudaStreamSynchronize(c->stream));
         return HBF_OK;
     };
-    int rc = count(by_unit);
+    SubmitArgs a{};
+    int rc = HBF_OK;
+    CK(launch_paged_clear(pw, c->stream));
+    if (by_unit && n >= kPagedLookFirst && !c->paged_crossed && paged_unit_ns(c->mp) < (1ll << 33)) {
+        // Most often no access reaches over the end of its stripe unit, and the first of the two passes over the records counts beside its own
+        // work (a count by itself took 271 of the 1,186 us of 64 M accesses; that pass 339, the second 463, the full pass and its fix-up 812).  Where it
+        // does not serve the batch, the count kernel runs behind it as if it had not been there: its control block is a spare one.  (Some 15 us
+        // then, which is why a batch behind one with accesses that crossed is counted first; below a few hundred thousand accesses the count
+        // costs no more than the first pass behind the host's wait: 100,000 82 and 85 us, 1 M 109 and 101.)
+        workspace_layout(n, c->mp.n_queues, c->mp.channels, rooms, &a.ws, pw.inner, 0);
+        a.acc = d_acc; a.n = n; a.completion = d_completion_ns; a.stall = d_stall_ns; a.die_stats = d_die_stats;
+        a.paged = 1; a.stage = 1;
+        const bool on_host = c->result_on_host;
+        std::swap(c->d_ctrl, c->d_ctrl_spare);
+        rc = serve_records(c, a);
+        std::swap(c->d_ctrl, c->d_ctrl_spare);
+        c->result_on_host = on_host;
+        if (rc == HBF_OK) rc = count(true, c->d_ctrl_spare);
+    } else {
+        rc = count(by_unit, nullptr);
+    }
     if (rc != HBF_OK) return rc;
-    if (by_unit && (h_total[kPagedUnsorted] || h_total[kPagedLong])) {
+    const bool served = h_total[kPagedServed] != 0ull;
+    if (by_unit) c->paged_crossed = h_total[kPagedParts] != n;
+    if (by_unit && !served && (h_total[kPagedUnsorted] || h_total[kPagedLong])) {
         by_unit = false;
-        if ((rc = count(false)) != HBF_OK) return rc;
+        CK(launch_paged_clear(pw, c->stream));
+        if ((rc = count(false, nullptr)) != HBF_OK) return rc;
     }
     const uint64_t total = h_total[kPagedParts];
     if ((by_unit ? (uint64_t)h_total[kPagedPages] : total) > capacity) return HBF_E_WORKSPACE;   // nothing has changed: the caller may come back with more room
     c->prof_inorder = false; c->prof_submit = false;
     if (by_unit && total == n) {                             // no access crosses a stripe unit: the caller's records are the list
-        SubmitArgs a{};
         workspace_layout(n, c->mp.n_queues, c->mp.channels, rooms, &a.ws, pw.inner, 0);
         a.acc = d_acc; a.n = n; a.completion = d_completion_ns; a.stall = d_stall_ns; a.status = d_status; a.die_stats = d_die_stats;
-        a.paged = 1;
+        a.paged = 1; a.stage = served ? 2 : 0;
+        if (served) std::swap(c->d_ctrl, c->d_ctrl_spare);
         if ((rc = serve_records(c, a)) != HBF_OK) return rc;
         c->submitted = true;
         return HBF_OK;
@@ -824,7 +849,7 @@ int hbf_submit_batch_paged(hbf_ctx *c, const hbf_access_t *d_acc, uint64_t n, ui
     CK(launch_paged_offsets(n, pw, c->stream));
     CK(launch_paged_expand(d_acc, n, c->d_ranges, c->d_mp, fast, by_unit ? c->mp.stripe_shift : c->mp.page_shift, capacity, pw, c->sm_count, c->stream));
     // the list of parts is a batch of records like any other: the ledger, the bus stage and retention, when on, see parts
-    SubmitArgs a{};
+    a = SubmitArgs{};
     workspace_layout(total, c->mp.n_queues, c->mp.channels, rooms, &a.ws, pw.inner, with_bus);
     a.acc = pw.parts; a.n = total; a.completion = pw.part_completion; a.stall = pw.part_stall; a.status = pw.part_status;
     a.die_stats = d_die_stats;

@@ -75,6 +75,8 @@ struct BatchCtrl {
     uint32_t twice;                      // every tile is served twice (decided here for batches too large for the host to tell: begin_load)
     float load;                          // the share of the batch's span that its work, and what the queues are behind, fills (0: not asked)
     int64_t issue_lo, issue_hi;          // smallest and largest issue time among the begin kernel's samples
+    unsigned long long pages;            // page-granular submit, first stage: pages of all accesses (one of an access that is not modeled)
+    uint32_t crossed, pad1;              //   set: some modeled access reaches over the end of its stripe unit
     uint32_t role_count[2];              // in-order serve pass: tiles handed out so far, per size class
     uint32_t tile_counter[kMaxPasses + 2];
     long long modeled_ns, service_ns, max_completion_ns;
@@ -126,6 +128,7 @@ struct SubmitArgs {
     FastRange fast;
     int binned;                          // the batch's energy goes to the time-bin ledger, not to the pending totals
     int paged;                           // every record is an access inside one stripe unit whose pages are queued on their own (declared in issue order)
+    int stage;                           // 0: the whole batch; else (paged, not known yet to be such records) 1: up to the first pass, which finds out, and 2: the rest
     int bus_on;                          // the channel-bus stage follows: array-done times must fit its 47-bit key field
     const unsigned long long *claim_limit;  // retention on: batch index below which a modeled access claims a refresh quantum
     uint32_t *die_claims;                   // retention on: [dies] claims of the batch
@@ -270,11 +273,14 @@ struct PagedWorkspace {
     void *inner; size_t inner_bytes;     // workspace of the ordinary path for `capacity` records
     size_t bytes;
 };
-// parts of the list; pages of all accesses; accesses issued before their predecessor; set when a service of a stripe unit's pages is too long for the in-order kernels
-enum PagedTotal { kPagedParts = 0, kPagedPages = 1, kPagedUnsorted = 2, kPagedLong = 3, kPagedTotals = 4 };
+// parts of the list; pages of all accesses; accesses issued before their predecessor; set when a service of a stripe unit's pages is too long
+// for the in-order kernels; set when the first pass has been over the caller's records and every one lies inside a stripe unit
+enum PagedTotal { kPagedParts = 0, kPagedPages = 1, kPagedUnsorted = 2, kPagedLong = 3, kPagedServed = 4, kPagedTotals = 5 };
 size_t paged_layout(uint64_t n, uint64_t capacity, uint32_t n_queues, uint32_t channels, uint32_t rooms, PagedWorkspace *pw, void *base, int with_bus);
+cudaError_t launch_paged_clear(const PagedWorkspace &pw, cudaStream_t st);
+int64_t paged_unit_ns(const ModelParams &mp);               // service of a stripe unit's pages without scaling (2^33: that or more)
 cudaError_t launch_paged_count(const hbf_access_t *acc, uint64_t n, const RangeSnap *ranges, const ModelParams *mp_dev, const FastRange &fast,
-                               const ModelParams &mp, const DevState *state, bool by_unit, const PagedWorkspace &pw, cudaStream_t st);
+                               const ModelParams &mp, const DevState *state, bool by_unit, const BatchCtrl *looked, const PagedWorkspace &pw, cudaStream_t st);
 cudaError_t launch_paged_offsets(uint64_t n, const PagedWorkspace &pw, cudaStream_t st);
 cudaError_t launch_paged_expand(const hbf_access_t *acc, uint64_t n, const RangeSnap *ranges, const ModelParams *mp_dev,
                                 const FastRange &fast, uint32_t cut_shift, uint64_t capacity, const PagedWorkspace &pw, int sm_count,

@@ -205,7 +205,8 @@ __device__ __forceinline__ void row_wait2(int id, int64_t m, long long s8, const
 // and claims.  The chain of updates then carries 8 bytes a queue and 4, where all 16 take four times the shared memory's turns (4 M decode
 // reads 117.6 -> 111.9 us, 24 M prefix records 397 -> 385, first half of 48 M with retention: light 216 -> 199, again 184 -> 174).  Read
 // disturb stays with the third: its atomics, all over the L2, take 50 us of a 24 M batch there and 105 beside the stores of the results.
-enum { kInFull = 0, kInAgain = 1, kInLight = 2 };
+// The last is the third on a page-granular batch whose accesses are not known to stay inside their stripe units: it finds out, and counts pages.
+enum { kInFull = 0, kInAgain = 1, kInLight = 2, kInLook = 3 };
 struct NarrowSums { uint32_t native, fault, max_done; unsigned unsorted, over; long long stall; };
 
 __device__ __forceinline__ uint32_t nw_transfer(const FastGeom &g, uint32_t granules, uint32_t mul) {
@@ -219,19 +220,19 @@ __device__ __forceinline__ void row_wait_n(int id, uint32_t m, uint32_t s, const
 }
 
 // MODE: see k_inorder_serve.  Everything per queue goes by the queue's slot.
-// count: see kInLight (a pass that knows its busy-until).
+// count: see kInLight (a pass that knows its busy-until).  prog_pages: pages of programs (kInLook).
 template <int MODE, bool DEBT, bool PAGED>
 __device__ __forceinline__ NarrowSums serve_narrow(const FastGeom &geom, const ModelParams &mp, const ModelParams &mp_arg, const hbf_access_t *acc_t, const uint32_t tile_begin,
                                                    const uint32_t tile_len, const int64_t T0, uint4 *qst, uint8_t *warp_tag, uint8_t *status_t,
                                                    uint16_t *qid_t, const uint32_t qid_stride, int64_t *completion_t, int64_t *stall_t,
                                                    InHead *__restrict__ in_head, const uint32_t tile, const uint32_t R, const uint32_t head_depth,
                                                    uint32_t *s_heads_full, uint32_t *st_br_lo, const uint32_t n_dies,
-                                                   const uint64_t claim_limit, const uint32_t quantum_ns, const RetDev &ret, const uint32_t ret_row_shift, const bool count) {
-    constexpr bool RESERVE = MODE == kInAgain, LIGHT = MODE == kInLight;
+                                                   const uint64_t claim_limit, const uint32_t quantum_ns, const RetDev &ret, const uint32_t ret_row_shift, const bool count, uint32_t *prog_pages) {
+    constexpr bool RESERVE = MODE == kInAgain, LOOK = MODE == kInLook, LIGHT = MODE == kInLight || LOOK;
     const bool counts = MODE == kInFull || (RESERVE && count);
     constexpr int K = kInRows;
     using State = typename std::conditional<RESERVE, uint32_t, typename std::conditional<LIGHT, uint2, uint4>::type>::type;
-    const uint32_t die_mask = (1u << geom.chdie_shift) - 1u;
+    const uint32_t die_mask = (1u << geom.chdie_shift) - 1u, unit_mask = (1u << geom.stripe_shift) - 1u;
     uint32_t *st_gran = reinterpret_cast<uint32_t *>(qst) + kInMaxQueues;      // (counting with known busy-until: read granules by the low bits of the slot)
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     uint32_t *st_br_hi = st_br_lo + n_dies, *st_bp_lo = st_br_hi + n_dies, *st_bp_hi = st_bp_lo + n_dies, *st_nr = st_bp_hi + n_dies, *st_np = st_nr + n_dies, *st_claims = st_np + n_dies;
@@ -294,6 +295,7 @@ __device__ __forceinline__ NarrowSums serve_narrow(const FastGeom &geom, const M
                 const uint32_t w = (uint32_t)(off >> geom.stripe_shift), in_page = (uint32_t)off & geom.page_mask;
                 q[u] = w & geom.nw_slot_mask;
                 const uint32_t npages = (in_page + bytes + geom.page_mask) >> geom.page_shift;
+                if (LOOK) b_hi |= (((uint32_t)off & unit_mask) + bytes - 1u) >> geom.stripe_shift;   // (crosses its unit: for the 64-bit form to see)
                 if (flags == 0u) {
                     const uint32_t g = (bytes + ((1u << geom.gran_shift_read) - 1u)) >> geom.gran_shift_read;
                     S[u] = npages * geom.t_read; xo[u] = nw_transfer(geom, g, geom.nw_mul_read);
@@ -313,6 +315,7 @@ __device__ __forceinline__ NarrowSums serve_narrow(const FastGeom &geom, const M
                 } else {                                     // a program: its data is transferred first; bytes and count by atomics
                     uint32_t g = (bytes + ((1u << geom.gran_shift_prog) - 1u)) >> geom.gran_shift_prog, xf = nw_transfer(geom, g, geom.nw_mul_prog);
                     S[u] = npages * geom.t_prog;
+                    if (LOOK) atomicAdd(prog_pages, npages);
                     if (PAGED && npages > 1u) {
                         const uint32_t head = geom.page_mask + 1u - in_page, tail = in_page + bytes - (npages - 1u) * (geom.page_mask + 1u), gm = (1u << geom.gran_shift_prog) - 1u;
                         const uint32_t gh = (head + gm) >> geom.gran_shift_prog, gt = (tail + gm) >> geom.gran_shift_prog;
@@ -339,6 +342,10 @@ __device__ __forceinline__ NarrowSums serve_narrow(const FastGeom &geom, const M
                 Served v = serve_terms_geom(geom, mp, addr[u], issue[u], bf[u], 1000000, Div64{}, lng, (int)kNwServeBits - 1);
                 if (PAGED && v.st == HBF_ST_READY) paged_terms(mp, off, bytes, 1000000, Div64{}, lng, (int)kNwServeBits - 1, v);
                 st = (uint32_t)v.st;
+                if (LOOK && v.st == HBF_ST_READY) {
+                    if ((uint64_t)((uint32_t)off & unit_mask) + bytes > (uint64_t)unit_mask + 1u) b_hi |= 1u;
+                    if (v.op) atomicAdd(prog_pages, v.parts);
+                }
                 if (v.st == HBF_ST_READY) {
                     ready[u] = true; q[u] = queue_slot(geom, v.queue);
                     if (lng || ((uint64_t)v.s >> (kNwServeBits - 1)) || (v.xfer >> 30)) b_time |= 0x80000000u;
@@ -373,7 +380,7 @@ __device__ __forceinline__ NarrowSums serve_narrow(const FastGeom &geom, const M
                     atomicAdd(&ret.disturb[ret_block_of(mp, ret, off)], npages);
                 }
             }
-            if (!RESERVE && status_t && valid[u]) status_t[i[u]] = (uint8_t)st;
+            if ((PAGED || !RESERVE) && status_t && valid[u]) status_t[i[u]] = (uint8_t)st;
         }
         // ---- which lanes of a row hold the same queue (see the 64-bit form)
         uint8_t *tag_at[K];
@@ -497,7 +504,7 @@ k_inorder_serve(const hbf_access_t *__restrict__ acc, uint64_t n, const __grid_c
                 const int64_t *__restrict__ busy, const unsigned long long *claim_limit_p, uint32_t *die_claims,
                 const __grid_constant__ RetDev ret, uint16_t *__restrict__ in_qid, uint32_t qid_stride,
                 TileBalance *bal, uint32_t bal_seq, const __grid_constant__ FastGeom geom, const uint32_t head_depth, const OrderedCopy copy, const int decided) {
-    constexpr bool RESERVE = MODE == kInAgain, LIGHT = MODE == kInLight;
+    constexpr bool RESERVE = MODE == kInAgain, LOOK = MODE == kInLook, LIGHT = MODE == kInLight || LOOK;
     extern __shared__ __align__(16) unsigned char in_smem[];
     __shared__ long long s_red[2];
     __shared__ unsigned long long s_t0;                   // when this block took its tile (0: its time is not recorded)
@@ -508,6 +515,7 @@ k_inorder_serve(const hbf_access_t *__restrict__ acc, uint64_t n, const __grid_c
     pdl_wait();
     pdl_trigger();
     if (ctrl->skip || ctrl->run_sort) return;             // (run_sort set this early: the batch went to the sort path at its start)
+    if (LOOK && ctrl->crossed) return;                    // (the samples showed it: the records are cut first)
     if (!RESERVE && decided && (ctrl->twice != 0u) != LIGHT) return;      // (the batch's load has chosen the other of the two)
     if (RESERVE && decided && blockIdx.x == 0 && threadIdx.x == 0 && ctrl->inorder_used && !ctrl->twice && 2u * bal->strag_flagged >= tmap.n_tiles) {
         bal->twice_load = ctrl->load; bal->twice_left = kInTwiceRun;
@@ -587,6 +595,9 @@ k_inorder_serve(const hbf_access_t *__restrict__ acc, uint64_t n, const __grid_c
     unsigned c_unsorted = (DEBT && ((uint64_t)quantum_ns >> 32)) ? 1u : 0u;   // (or a service, or a refresh quantum, of 2^32 ns or more)
     long long sum_stall = 0, max_c = INT64_MIN;
     long long t_native = 0, t_ready = 0, t_fault = 0;        // this thread's share of the tile's counts
+    unsigned long long t_pages = 0; unsigned c_crossed = 0;  // kInLook: see BatchCtrl
+    __shared__ uint32_t s_prog_pages; __shared__ unsigned long long s_work;
+    if (LOOK && tid == 0) { s_prog_pages = 0u; s_work = 0ull; }
     bool narrow_done = false, again = false;
     {
         // The 32-bit form serves the tile when the configuration allows it, the tile's times lie within 2^31 ns and its read
@@ -614,13 +625,14 @@ k_inorder_serve(const hbf_access_t *__restrict__ acc, uint64_t n, const __grid_c
             NarrowSums nw{};
             if (try_narrow) nw = serve_narrow<MODE, DEBT, PAGED>(geom, mp, mp_arg, acc_t, (uint32_t)tile_begin, tile_len, T0, q4, warp_tag, status_t, qid_t, qid_stride,
                                                      completion_t, stall_t, in_head, tile, R, head_depth, &s_heads_full, st_br_lo, n_dies, claim_limit,
-                                                     (uint32_t)quantum_ns, ret, ret_row_shift, count);
+                                                     (uint32_t)quantum_ns, ret, ret_row_shift, count, &s_prog_pages);
             if (__syncthreads_or((int)(over | nw.over)) == 0) {
                 narrow_done = true;
                 sum_stall = nw.stall;
                 if (nw.max_done) max_c = T0 + (int64_t)(uint64_t)nw.max_done;      // (a modeled access ends after its tile's first issue time)
                 if constexpr (!RESERVE) {
                     c_unsorted |= nw.unsorted;
+                    unsigned long long work = 0;
                     if (tid == 0 && tile_begin > 0 && ld_after(&acc_t[-1].issue_ns) > T0) c_unsorted = 1u;
                     t_native = nw.native; t_fault = nw.fault; t_ready = (tid == 0 ? (long long)tile_len : 0ll) - t_native - t_fault;
                     longlong2 *out = reinterpret_cast<longlong2 *>(in_agg) + (uint64_t)tile * R;
@@ -628,7 +640,15 @@ k_inorder_serve(const hbf_access_t *__restrict__ acc, uint64_t n, const __grid_c
                         uint2 v;                             // busy-until, service time
                         if (LIGHT) v = reinterpret_cast<const uint2 *>(qst)[queue_slot(geom, q)];
                         else { const uint4 f = q4[queue_slot(geom, q)]; v = make_uint2(f.x, f.y); in_headcnt[(uint64_t)tile * R + q] = (uint8_t)(f.w & 15u); }
+                        work += v.y;
                         out[q] = make_longlong2((long long)(uint64_t)v.y, v.y ? T0 + (int64_t)(uint64_t)v.x : kNegInf);   // (no service time: no access)
+                    }
+                    if (LOOK) {                              // the tile's pages follow from its service time
+                        work = (unsigned long long)warp_sum((long long)work);
+                        if (lane == 0) atomicAdd(&s_work, work);
+                        __syncthreads();
+                        if (tid == 0) t_pages = (s_work - (unsigned long long)s_prog_pages * geom.t_prog) / geom.t_read + s_prog_pages;
+                        t_pages += (unsigned long long)t_native;
                     }
                     if (MODE == kInFull) for (uint32_t d = tid; d < n_dies; d += kInThreads) {              // a die's reads: the sums its queues carry
                         unsigned long long g = 0, cnt = 0;
@@ -724,12 +744,17 @@ k_inorder_serve(const hbf_access_t *__restrict__ acc, uint64_t n, const __grid_c
         // ---- terms ---------------------------------------------------------------------------------------
 #pragma unroll
         for (int u = 0; u < K; ++u) {
-            v[u].st = HBF_ST_NATIVE; v[u].queue = 0; v[u].die = 0; v[u].op = 0; v[u].s = 0; v[u].xfer = 0; v[u].cb = 0;
+            v[u].st = HBF_ST_NATIVE; v[u].queue = 0; v[u].die = 0; v[u].op = 0; v[u].s = 0; v[u].xfer = 0; v[u].cb = 0; v[u].parts = 1;
             if (valid[u])
                 v[u] = fast_on ? serve_terms_geom(geom, mp, addr[u], issue[u], bf[u], q_ppm, div_q, c_unsorted, DEBT ? 32 : 33)
                                  : serve_terms(rs, mp, addr[u], issue[u], bf[u], q_ppm, div_q, c_unsorted, DEBT ? 32 : 33);
             ready[u] = valid[u] && v[u].st == HBF_ST_READY;
-            if (PAGED && ready[u]) paged_terms(mp, media_offset_of(rs, fast_range, fast_on, addr[u], issue[u], bf[u]), (uint32_t)bf[u], q_ppm, div_q, c_unsorted, 33, v[u]);
+            if (PAGED && ready[u]) {
+                const uint64_t off = media_offset_of(rs, fast_range, fast_on, addr[u], issue[u], bf[u]), unit = 1ull << mp.stripe_shift;
+                paged_terms(mp, off, (uint32_t)bf[u], q_ppm, div_q, c_unsorted, 33, v[u]);
+                if (LOOK && (off & (unit - 1ull)) + (uint32_t)bf[u] > unit) c_crossed = 1u;
+            }
+            if (LOOK && valid[u]) t_pages += v[u].parts;
             if (DEBT && ready[u] && tile_begin + i[u] < claim_limit) {
                 v[u].s += quantum_ns;
                 if (counts) atomicAdd(&st_claims[v[u].die], 1u);
@@ -769,13 +794,13 @@ k_inorder_serve(const hbf_access_t *__restrict__ acc, uint64_t n, const __grid_c
             for (int u = 0; u < K; ++u)
                 if (valid[u]) qid_t[i[u]] = ready[u] ? (uint16_t)v[u].queue : (uint16_t)kInMaxQueues;   // (one past the last queue: not modeled)
         }
-        if (!RESERVE || counts) {
+        if (!RESERVE || counts || (PAGED && status_t)) {
 #pragma unroll
             for (int u = 0; u < K; ++u) {
                 if (valid[u]) {
+                    if ((PAGED || !RESERVE) && status_t) status_t[i[u]] = (uint8_t)v[u].st;
                     if (!RESERVE) {
                         c_unsorted |= issue[u] < prev[u] ? 1u : 0u;
-                        if (status_t) status_t[i[u]] = (uint8_t)v[u].st;
                         c_valid += 1u;
                         c_ready += ready[u] ? 1u : 0u;
                         c_native += v[u].st == HBF_ST_NATIVE ? 1u : 0u;
@@ -923,6 +948,11 @@ k_inorder_serve(const hbf_access_t *__restrict__ acc, uint64_t n, const __grid_c
         const unsigned long long w_ready = (unsigned long long)warp_sum(t_ready);        // (a warp's share may be negative: the sum over the tile counts)
         const unsigned long long w_fault = (unsigned long long)warp_sum(t_fault);
         c_unsorted = __any_sync(0xffffffffu, c_unsorted);
+        if (LOOK) {
+            const unsigned long long w_pages = (unsigned long long)warp_sum((long long)t_pages);
+            const bool crossed = __any_sync(0xffffffffu, c_crossed != 0u);
+            if (lane == 0) { if (w_pages) atomicAdd(&ctrl->pages, w_pages); if (crossed) ctrl->crossed = 1u; }
+        }
         if (lane == 0) {
             if (w_native) atomicAdd(&ctrl->n_native, w_native);
             if (w_ready) atomicAdd(&ctrl->n_ready, w_ready);
@@ -1513,7 +1543,9 @@ cudaError_t launch_inorder(const SubmitArgs &a, cudaStream_t st) {
     // two nominal sizes
     TileBalanceHost *bal = tmap.by_sm ? a.bal : nullptr;
     uint32_t bal_seq = 0;
-    if (bal) {
+    if (bal && a.stage == 2) {                               // (the tiles stand as the first stage left them)
+        bal_seq = bal->seq; tmap.first = bal->dev->first;
+    } else if (bal) {
         bal_seq = ++bal->seq;
         if (bal_seq == 0u) bal_seq = ++bal->seq;             // (0 marks a tile never taken)
         double share[kInBalMax];
@@ -1546,8 +1578,8 @@ cudaError_t launch_inorder(const SubmitArgs &a, cudaStream_t st) {
     } else if (a.bal && a.bal->depth_fixed != 0u) {
         depth = std::min<uint32_t>(a.bal->depth_fixed, (uint32_t)kInHead);
     }
-    const bool twice = n <= twice_max(a.mp.n_queues) && !(a.bal && a.bal->depth_fixed != 0u);   // (a fixed number of head entries is the caller's)
-    const bool decided = inorder_decides(a) != nullptr;
+    const bool twice = a.stage != 0 || (n <= twice_max(a.mp.n_queues) && !(a.bal && a.bal->depth_fixed != 0u));   // (a fixed number of head entries is the caller's)
+    const bool decided = a.stage == 0 && inorder_decides(a) != nullptr;
     if (twice) depth = 0u;
     const uint64_t tile_records = tmap.max_tile;
     if (n_tiles > inorder_tiles_bound(n)) return cudaErrorInvalidValue;       // the workspace is carved for that many
@@ -1556,7 +1588,7 @@ cudaError_t launch_inorder(const SubmitArgs &a, cudaStream_t st) {
     {
         const void *serve_fns[] = {(const void *)k_inorder_serve<kInFull, false, false>, (const void *)k_inorder_serve<kInAgain, false, false>, (const void *)k_inorder_serve<kInLight, false, false>,
                                    (const void *)k_inorder_serve<kInFull, true, false>, (const void *)k_inorder_serve<kInAgain, true, false>, (const void *)k_inorder_serve<kInLight, true, false>,
-                                   (const void *)k_inorder_serve<kInFull, false, true>, (const void *)k_inorder_serve<kInAgain, false, true>, (const void *)k_inorder_serve<kInLight, false, true>};
+                                   (const void *)k_inorder_serve<kInLook, false, true>, (const void *)k_inorder_serve<kInFull, false, true>, (const void *)k_inorder_serve<kInAgain, false, true>, (const void *)k_inorder_serve<kInLight, false, true>};
         for (const void *f : serve_fns) { cudaError_t e = ensure_dyn_smem(f, smem_serve); if (e != cudaSuccess) return e; }
         cudaError_t e = ensure_dyn_smem((const void *)k_inorder_scan, 0);
         if (e != cudaSuccess) return e;
@@ -1571,18 +1603,22 @@ cudaError_t launch_inorder(const SubmitArgs &a, cudaStream_t st) {
     if ((uint64_t)n_tiles * qid_stride > inorder_qid_entries(n)) return cudaErrorInvalidValue;
     auto serve = [&](int mode) {
         auto pick = [&](auto full, auto second, auto light) { return mode == kInAgain ? second : mode == kInLight ? light : full; };
-        auto k = a.paged ? pick(k_inorder_serve<kInFull, false, true>, k_inorder_serve<kInAgain, false, true>, k_inorder_serve<kInLight, false, true>)
+        auto k = a.stage == 1 ? k_inorder_serve<kInLook, false, true>
+               : a.paged ? pick(k_inorder_serve<kInFull, false, true>, k_inorder_serve<kInAgain, false, true>, k_inorder_serve<kInLight, false, true>)
                : debt ? pick(k_inorder_serve<kInFull, true, false>, k_inorder_serve<kInAgain, true, false>, k_inorder_serve<kInLight, true, false>)
                       : pick(k_inorder_serve<kInFull, false, false>, k_inorder_serve<kInAgain, false, false>, k_inorder_serve<kInLight, false, false>);
-        return launch_pdl(k, n_tiles, kInThreads, smem_serve, st, a.acc, n, tmap, a.ranges, a.mp, a.fast, a.ctrl, a.status, a.ws.in_agg,
+        return launch_pdl(k, n_tiles, kInThreads, smem_serve, st, a.acc, n, tmap, a.ranges, a.mp, a.fast, a.ctrl,
+                          mode == kInAgain && a.stage == 0 ? (uint8_t *)nullptr : a.status, a.ws.in_agg,
                           a.stats_stage, a.completion, a.stall, (const int64_t *)a.ws.in_bin, tiles, heads, a.ws.in_headcnt,
                           (const int64_t *)a.busy, a.claim_limit, a.die_claims, debt ? *a.ret : RetDev{}, a.ws.in_qid, qid_stride,
                           bal ? bal->dev : nullptr, bal_seq, make_fast_geom(a.fast, a.mp), depth, ordered_copy(n, a.ws), decided ? 1 : 0);
     };
-    cudaError_t le = twice ? serve(kInLight) : serve(kInFull);
+    cudaError_t le = cudaSuccess;
+    if (a.stage != 2) le = twice ? serve(kInLight) : serve(kInFull);
     if (le == cudaSuccess && decided) le = serve(kInLight);
+    if (a.stage == 1) { g_kernel_launches += 1; return le; }
     if (le == cudaSuccess)
-        le = launch_pdl(k_inorder_scan, (R + kInScanQueues - 1) / kInScanQueues, dim3(kInScanQueues, kInScanChunks), 0, st, a.ctrl, a.mp_dev, n_tiles,
+        le = launch_first(a.stage == 2 ? a.plain_next : nullptr, k_inorder_scan, (R + kInScanQueues - 1) / kInScanQueues, dim3(kInScanQueues, kInScanChunks), 0, st, a.ctrl, a.mp_dev, n_tiles,
                         (const int64_t *)a.ws.in_agg, a.ws.in_bin, (const int64_t *)a.busy, a.busy_stage, a.stats_stage, a.path == HBF_PATH_INORDER ? 1 : 0);
     if (le == cudaSuccess && !twice)
         le = launch_pdl(a.paged ? k_inorder_fixstraggle<false, true> : debt ? k_inorder_fixstraggle<true, false> : k_inorder_fixstraggle<false, false>, n_tiles, kInStrThreads,
@@ -1594,7 +1630,7 @@ cudaError_t launch_inorder(const SubmitArgs &a, cudaStream_t st) {
         cudaError_t e = cudaMemcpyAsync(bal->pinned, bal->dev, offsetof(TileBalance, first), cudaMemcpyDeviceToHost, st);
         if (e != cudaSuccess) return e;
     }
-    g_kernel_launches += twice ? 3 : decided ? 5 : 4;
+    g_kernel_launches += a.stage == 2 ? 2 : twice ? 3 : decided ? 5 : 4;
     return cudaGetLastError();
 }
 

@@ -6,6 +6,8 @@
 // inorder_kernels.cu).  It is cut at stripe units only, and where no access crosses one, its own records are served.
 //   count   parts per access (1 for an access that is not modeled), summed per row of 32 accesses and per tile of 64 rows;
 //           a row's parts-before-it within its tile are kept.  By stripe unit it also finds the batch's pages and whether it is in order
+//           (From 400,000 accesses on the first of the two passes by stripe unit counts beside its own work, and this kernel leaves at once where
+//           that pass serves the batch: hbf_submit_batch_paged.)
 //   scan    exclusive scan of the tile sums by one block; the totals go back to the host, which sizes the rest
 //   expand  a warp per row, no block-wide step: the warp reads its 32 records, knows where its parts begin (tile offset
 //           + row offset), and writes them, in (access, part) order, as ordinary access records
@@ -62,11 +64,15 @@ __device__ __forceinline__ uint32_t parts_of_fast(const FastRange &fr, uint32_t 
 template <bool FAST, bool BY_UNIT>
 __global__ void __launch_bounds__(kPgThreads)
 k_paged_count(const hbf_access_t *__restrict__ acc, uint64_t n, const RangeSnap *__restrict__ ranges, const __grid_constant__ FastRange fast,
-              const uint32_t page_shift, const uint32_t stripe_shift, const int64_t unit_ns, const DevState *__restrict__ state,
+              const uint32_t page_shift, const uint32_t stripe_shift, const int64_t unit_ns, const DevState *__restrict__ state, const BatchCtrl *looked,
               unsigned long long *__restrict__ tile_sum, uint32_t *__restrict__ row_off, unsigned long long *totals) {
     __shared__ uint32_t s_row[kPgRows];
     __shared__ unsigned long long s_pages, s_parts;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    if (BY_UNIT && looked && !looked->skip && !looked->crossed && !looked->unsorted && looked->n_fault == 0ull) {      // the first pass has counted
+        if (blockIdx.x == 0 && tid == 0) { totals[kPagedServed] = 1ull; totals[kPagedParts] = n; totals[kPagedPages] = looked->pages; }
+        return;
+    }
     if (tid == 0) { s_pages = 0ull; s_parts = 0ull; }
     unsigned long long pages_sum = 0;
     unsigned unsorted = 0;
@@ -288,17 +294,21 @@ size_t paged_layout(uint64_t n, uint64_t capacity, uint32_t n_queues, uint32_t c
     return off;
 }
 
+// (any time from 2^33 ns on is too long: no larger one is formed)
+int64_t paged_unit_ns(const ModelParams &mp) {
+    const int64_t page_ns = std::max(mp.t_read_ns, mp.t_prog_ns);
+    return page_ns >= (1ll << 33) >> mp.pages_per_stripe_shift ? 1ll << 33 : page_ns << mp.pages_per_stripe_shift;
+}
+cudaError_t launch_paged_clear(const PagedWorkspace &pw, cudaStream_t st) { return cudaMemsetAsync(pw.total, 0, sizeof(PagedSums) + kPagedTotals * 8, st); }
+// looked: the control block of a first pass over the batch (null: there was none), which may have counted already
 cudaError_t launch_paged_count(const hbf_access_t *acc, uint64_t n, const RangeSnap *ranges, const ModelParams *mp_dev, const FastRange &fast,
-                               const ModelParams &mp, const DevState *state, bool by_unit, const PagedWorkspace &pw, cudaStream_t st) {
+                               const ModelParams &mp, const DevState *state, bool by_unit, const BatchCtrl *looked, const PagedWorkspace &pw, cudaStream_t st) {
     (void)mp_dev;
     const uint64_t tiles = (n + kPgTile - 1) / kPgTile;
-    cudaError_t e = cudaMemsetAsync(pw.total, 0, sizeof(PagedSums) + kPagedTotals * 8, st);
-    if (e != cudaSuccess) return e;
     const unsigned grid = (unsigned)std::min<uint64_t>(tiles, 148u * 16u);
-    // (any time from 2^33 ns on is too long: no larger one is formed)
-    const int64_t page_ns = std::max(mp.t_read_ns, mp.t_prog_ns), unit_ns = page_ns >= (1ll << 33) >> mp.pages_per_stripe_shift ? 1ll << 33 : page_ns << mp.pages_per_stripe_shift;
+    const int64_t unit_ns = paged_unit_ns(mp);
     auto k = fast.on ? (by_unit ? k_paged_count<true, true> : k_paged_count<true, false>) : (by_unit ? k_paged_count<false, true> : k_paged_count<false, false>);
-    k<<<grid, kPgThreads, 0, st>>>(acc, n, ranges, fast, mp.page_shift, mp.stripe_shift, unit_ns, state, pw.tile_sum, pw.row_off, pw.total);
+    k<<<grid, kPgThreads, 0, st>>>(acc, n, ranges, fast, mp.page_shift, mp.stripe_shift, unit_ns, state, looked, pw.tile_sum, pw.row_off, pw.total);
     g_kernel_launches += 1;
     return cudaGetLastError();
 }

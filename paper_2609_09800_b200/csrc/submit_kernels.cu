@@ -32,6 +32,10 @@ __global__ void k_begin(const __grid_constant__ BeginArgs b, int role, int run_s
     begin_batch(b, run_sort, 0u);
     if (role == 0 && b.decides)
         begin_load(b, reinterpret_cast<const uint64_t *>(acc + (uint64_t)threadIdx.x * (b.n - 1ull) / 1024ull), ld_after(&acc[0].issue_ns), ld_after(&acc[b.n - 1].issue_ns));
+    if (role == 0 && b.unit_shift) {
+        __syncthreads();                                     // (the control block is cleared)
+        begin_units(b, reinterpret_cast<const uint64_t *>(acc + (uint64_t)threadIdx.x * (b.n - 1ull) / 1024ull));
+    }
 }
 
 // =====================================================================================================
@@ -1148,7 +1152,7 @@ struct SortChain {
 // the radix sort's kernels, launched from the device (run_sort is set: the begin kernel starts the batch over)
 __device__ void launch_sort_chain(const SortChain &c, const FinishArgs &f, unsigned fin_grid) {
     cudaStream_t st = cudaStreamTailLaunch;
-    const BeginArgs b{c.ctrl, c.state, c.busy, c.busy_stage, c.stats_stage, c.hist, c.n_queues, c.n_dies, c.die_claims, c.claim_limit, nullptr, 0.0f, 0, 0, 0, 0};
+    const BeginArgs b{c.ctrl, c.state, c.busy, c.busy_stage, c.stats_stage, c.hist, c.n_queues, c.n_dies, c.die_claims, c.claim_limit, nullptr, 0.0f, 0, 0, 0, 0, nullptr, 0};
     k_begin<<<1, 1024, 0, st>>>(b, 1, 1, nullptr);
     k_zero_words<<<(unsigned)min((unsigned long long)((c.desc_words + 1023) / 1024), 592ull), 1024, 0, st>>>(c.desc0, c.desc_words);
     k_zero_words<<<(unsigned)min((unsigned long long)((c.scan_words + 1023) / 1024), 592ull), 1024, 0, st>>>((uint32_t *)c.scan_desc, c.scan_words);
@@ -1255,20 +1259,21 @@ cudaError_t launch_submit(const SubmitArgs &a, cudaStream_t st) {
     const bool try_inorder = a.inorder_ok && (a.path == HBF_PATH_AUTO || a.path == HBF_PATH_INORDER);
     const bool sort_kernels = a.path != HBF_PATH_INORDER || !a.inorder_ok;
     mark(0);
-    {
+    if (a.stage != 2) {
         const BeginArgs b{a.ctrl, a.state, a.busy, a.busy_stage, a.stats_stage, a.ws.hist, a.mp.n_queues, a.mp.n_dies, a.die_claims, a.claim_limit,
-                          try_inorder ? inorder_decides(a) : nullptr, twice_from(n, a.mp.n_queues, a.claim_limit != nullptr), n, a.mp.page_shift, a.mp.t_read_ns, a.mp.t_prog_ns};
+                          try_inorder ? inorder_decides(a) : nullptr, twice_from(n, a.mp.n_queues, a.claim_limit != nullptr), n, a.mp.page_shift, a.mp.t_read_ns, a.mp.t_prog_ns,
+                          a.ranges, a.stage == 1 ? a.mp.stripe_shift : 0u};
         const cudaError_t e = try_inorder && sort_kernels && n >= 2
             ? launch_begin_regroup(a, b, st)
             : launch_first(a.plain_next, k_begin, 1, 1024, 0, st, b, 0, try_inorder ? 0 : 1, a.acc);
         if (e != cudaSuccess) return e;
     }
-    g_kernel_launches += 1;
+    if (a.stage != 2) g_kernel_launches += 1;
     if (n > 0) {
         if (try_inorder) {
             mark(7);
             cudaError_t e = launch_inorder(a, st);
-            if (e != cudaSuccess) return e;
+            if (e != cudaSuccess || a.stage == 1) return e;
             mark(8);
             e = launch_finish_inorder(a, sort_kernels, st);
             if (e != cudaSuccess) return e;

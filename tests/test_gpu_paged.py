@@ -210,6 +210,45 @@ def test_stripe_units_match_the_oracle(hbf, kind, n):
         acc["issue_ns"] += 1000
 
 
+@pytest.mark.parametrize("kind", ["inside", "last crosses", "natives", "fault", "unordered", "scaled", "several ranges"])
+@pytest.mark.parametrize("n", [70_001, 400_003])             # (the pass counts from 400,000 on)
+def test_the_first_pass_counts(hbf, kind, n):
+    """A batch whose samples all lie inside their stripe units: the pass counts, and where something else turns up in it (or too many pages
+    for the caller's room), the call goes on, or is refused, as if that pass had not been."""
+    import torch
+    rng = np.random.default_rng(n)
+    prof = wl.load_profile("nominal", channels=8, dies=4, planes=2, page_bytes=16384, stripe_bytes=65536)
+    ranges = [(wl.RANGE_BASE, wl.GIB, 3, 0, 0, 0)] + ([(wl.RANGE_BASE + 2 * wl.GIB, wl.GIB, 1, 0, 1, wl.GIB)] if kind == "several ranges" else [])
+    g, o = contexts(hbf, prof, ranges)
+    acc = np.zeros(n, hbfo.ACCESS_DTYPE)
+    acc["bytes"] = rng.choice([1, 16384, 40_000, 65_536], n)
+    acc["addr"] = wl.RANGE_BASE + rng.integers(0, 16_000, n).astype(np.uint64) * np.uint64(65536) + (rng.random(n) * (65_537 - acc["bytes"])).astype(np.uint64)
+    acc["issue_ns"] = np.sort(rng.integers(0, 30_000 * n, n))
+    acc["flags"] = rng.random(n) < 0.1
+    odd = n - 3                                              # (between two of the samples)
+    if kind == "last crosses": acc["addr"][odd] = wl.RANGE_BASE + 65_535; acc["bytes"][odd] = 2
+    if kind == "natives": acc["addr"][rng.random(n) < 0.3] = 64
+    if kind == "fault": acc["bytes"][odd] = 0
+    if kind == "unordered": acc["issue_ns"][odd] = 0
+    if kind == "scaled": g.force_mode(1, 333_333); hbfo.lib().hbfo_force_mode(o._h, 1, 333_333)
+    first = np.zeros(300, hbfo.ACCESS_DTYPE)                 # a small batch before it, whose summary lies on the device
+    first["addr"] = wl.RANGE_BASE; first["bytes"] = 64
+    compare(g, o, first)
+    before = g.get_busy_until()
+    d = torch.from_numpy(acc.view(np.int64).reshape(-1)).cuda()
+    comp, stall = (torch.full((n,), -1, dtype=torch.int64, device="cuda") for _ in range(2))
+    status = torch.full((n,), 9, dtype=torch.uint8, device="cuda")
+    off = acc["addr"].astype(np.int64) % 16384
+    pages = int(np.where(acc["addr"] < wl.RANGE_BASE, 1, np.maximum(1, (off + acc["bytes"] + 16383) // 16384)).sum())
+    last = g.last_result()
+    assert g.submit_batch_paged(d, n, pages - 1, comp, stall, status) == hbf.E_WORKSPACE
+    assert (comp == -1).all() and (stall == -1).all() and (status == 9).all()
+    assert np.array_equal(g.get_busy_until(), before) and g.last_result() == last
+    for _ in range(2):
+        compare(g, o, acc)
+        acc["issue_ns"] += 1000
+
+
 @pytest.mark.parametrize("cross", [False, True])             # (no access crosses a stripe unit: the batch's own records are served)
 @pytest.mark.parametrize("n", [5_000, 12_000])
 def test_a_throttled_paged_batch_leaves_zeros(hbf, n, cross):
