@@ -1509,28 +1509,25 @@ size_t inorder_head_bytes(uint64_t tiles, uint32_t n_queues) { return tiles * n_
 
 // Batches whose tiles are all served twice, the first time without results and head entries (kInLight), in place of the fix-up.
 // The second time reads 24 and writes 16 bytes per record; the fix-up and its head entries cost some 30 us and what the tiles
-// times the queues make of them.  By records that meets at about 5 M with 64 queues, 11 M with 1,024, 20 M with 2,048 at a load of
-// 0.3, later at higher loads, where more queues are behind.  us, with the fix-up and served twice: 65,536 reads on 64 queues 66
-// and 38, 8 M 162 and 168; decode, 1,024 queues, 4 M 150 and 91, 12 M 207 and 192, 16 M 210 and 225 (load 0.3); capacity, 2,048
-// queues, 4 M 255 and 106, 16 M 323 and 251 (0.3), 28 M 369 and 418 (0.3).
-static uint64_t twice_max(uint32_t n_queues) { return 5000000ull + 7500ull * n_queues; }
+// times the queues make of them.  By records that meets at about 6 M with 64 queues, 19 M with 1,024, 28 M with 2,048 at a load of
+// 0.3; with retention, where the first pass counts the reads into the disturb counters, at 20 M with 2,048.  us, with the fix-up and served
+// twice, at 0.3: one-page reads, 64 queues, 4 M 128 and 111, 8 M 165 and 175; decode, 1,024 queues, 12 M 216 and 216, 16 M 258 and 239, 24 M 310
+// and 345; capacity, 2,048 queues, 12 M 317 and 222, 28 M 399 and 396, 36 M 453 and 494; two halves with retention, 18 M each 836 and 717, 24 M 856 and 928.
+static uint64_t twice_max(uint32_t n_queues, bool retention) { return retention ? 5000000ull + 7500ull * n_queues : 6000000ull + 11000ull * n_queues; }
 // Larger ones from a load on that rises with their size, towards 0.7, where queues begin to be behind everywhere (twice_from); and below
 // it where a batch with about their load, or less, had to serve half of its tiles twice after all; every 16th of those takes the fix-up,
 // to see whether it still does.  The device decides (begin_load), so both forms of the first pass are launched and one leaves at once
-// (2 us).  us, with the fix-up and served twice, by load: capacity, 2,048 queues, 24 M 344 and 380 (0.3), 369 and 379 (0.4), 429 and 378 (0.5),
-// 683 and 380 (0.65); 48 M 640 and 673 (0.55), 724 and 674 (0.6), 1,047 and 674 (0.65); 96 M 1,046 and 1,276 (0.6), 1,537 and
-// 1,276 (0.7); decode, 1,024, 21 M 296 and 306 (0.6), 418 and 302 (0.7); 42 M 443 and 540 (0.65), 640 and 548 (0.7); 64 queues, 32 M 396
-// and 540 (0.65), 617 and 540 (0.7); prefix, 24 M, crowded on some queues at a time, 280 and 359 (0.2), 567 and 357 (0.3), 469 and 365 (0.7).
-// (with retention the first pass counts the reads into the disturb counters, and the two meet at a lower load: 24 M at 0.5 in the case of 48 M with
-// claims 510 and 410; without it the line is drawn above where they meet near the smallest of these sizes, so that a batch at half load is
-// still measured by the full pass, whose times are what the tile sizes are for)
+// (2 us).  us, with the fix-up and served twice, by load: capacity, 2,048 queues, 36 M 528 and 494 (0.5), 621 and 494 (0.6); 48 M 534 and 628 (0.3),
+// 618 and 613 (0.5), 760 and 614 (0.6); 72 M 775 and 864 (0.5), 935 and 863 (0.6); two halves of 24 M with retention 1,006 and 912 (0.5).  With fewer
+// queues it is later, for a tile has fewer of them to be behind: decode, 1,024, 24 M 321 and 346 (0.5), 346 and 344 (0.65), 36 M 426 and 470 (0.65);
+// 64 queues, 32 M 480 and 536 (0.65).  Prefix, 1,024, 24 M, crowded on some queues at a time, 303 and 381 (0.2), 548 and 380 (0.3), 577 and 379 (0.5).
 float twice_from(uint64_t n, uint32_t n_queues, bool retention) {
-    const double x = (double)twice_max(n_queues) / (double)std::max<uint64_t>(n, 1);
-    return (float)(0.70 - (retention ? 0.40 : 0.22) * x * x);
+    const double x = (double)twice_max(n_queues, retention) / (double)std::max<uint64_t>(n, 1);
+    return (float)std::min(0.70, 0.74 - 0.40 * ((double)n_queues / kInMaxQueues) * x);
 }
 TileBalance *inorder_decides(const SubmitArgs &a) {
     const bool by_table = a.bal && a.bal->on && a.bal->dev;
-    return by_table && a.bal->depth_fixed == 0u && a.n > twice_max(a.mp.n_queues) && inorder_tile_map(a.n, a.sm_count, true).by_sm ? a.bal->dev : nullptr;
+    return by_table && a.bal->depth_fixed == 0u && a.n > twice_max(a.mp.n_queues, a.claim_limit != nullptr) && inorder_tile_map(a.n, a.sm_count, true).by_sm ? a.bal->dev : nullptr;
 }
 
 cudaError_t launch_inorder(const SubmitArgs &a, cudaStream_t st) {
@@ -1578,7 +1575,7 @@ cudaError_t launch_inorder(const SubmitArgs &a, cudaStream_t st) {
     } else if (a.bal && a.bal->depth_fixed != 0u) {
         depth = std::min<uint32_t>(a.bal->depth_fixed, (uint32_t)kInHead);
     }
-    const bool twice = a.stage != 0 || (n <= twice_max(a.mp.n_queues) && !(a.bal && a.bal->depth_fixed != 0u));   // (a fixed number of head entries is the caller's)
+    const bool twice = a.stage != 0 || (n <= twice_max(a.mp.n_queues, a.claim_limit != nullptr) && !(a.bal && a.bal->depth_fixed != 0u));   // (a fixed number of head entries is the caller's)
     const bool decided = a.stage == 0 && inorder_decides(a) != nullptr;
     if (twice) depth = 0u;
     const uint64_t tile_records = tmap.max_tile;
