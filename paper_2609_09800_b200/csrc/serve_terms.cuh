@@ -30,6 +30,8 @@ __device__ __forceinline__ Served serve_terms(const RangeSnap &rs, const ModelPa
 
 // The same terms for the common configuration (one registered range, power-of-two geometry, no thermal
 // scaling in force, transfer table present): 32-bit arithmetic wherever the values allow it.
+// (TABLE = false: the transfer by multiply-high, for a kernel that waits for the table's entry and has nothing else to do meanwhile)
+template <bool TABLE = true>
 __device__ __forceinline__ Served serve_terms_fast(const FastRange &f, const ModelParams &mp, uint64_t addr, int64_t issue, uint64_t bf) {
     Served r; r.queue = 0; r.die = 0; r.op = 0; r.s = 0; r.xfer = 0; r.cb = 0; r.parts = 1;
     const uint32_t bytes = (uint32_t)bf, flags = (uint32_t)(bf >> 32);
@@ -51,7 +53,7 @@ __device__ __forceinline__ Served serve_terms_fast(const FastRange &f, const Mod
     const uint32_t gs = r.op ? mp.prog_gran_shift : mp.read_gran_shift;
     const uint64_t cb = (((uint64_t)bytes + ((1ull << gs) - 1ull)) >> gs) << gs;
     r.cb = (int64_t)cb;
-    r.xfer = cb <= (uint64_t)mp.xfer_tab_max_cb ? __ldg(mp.xfer_tab + (uint32_t)(cb >> mp.xfer_tab_shift))
+    r.xfer = TABLE && cb <= (uint64_t)mp.xfer_tab_max_cb ? __ldg(mp.xfer_tab + (uint32_t)(cb >> mp.xfer_tab_shift))
                                                  : (uint32_t)div64(cb * 1000ull + mp.chan_bytes_per_us - 1ull, mp.div_chan);
     r.s = (int64_t)npages * (r.op ? mp.t_prog_ns : mp.t_read_ns);
     return r;

@@ -6,11 +6,13 @@
 //           same decision about it, and knows where its records go
 //   send    every record becomes an entry in the list of the block that owns its queue, in batch order, through distributed
 //           shared memory (barrier 2)
-//   sort    by queue, stable, in shared memory (a row of 32 ranks itself with match_any); a batch that is not in issue order
-//           is sorted by issue time first, 8 bits a pass over the bits that differ
-//   serve   a segmented max-plus scan over the sorted list (a queue's run is a segment): a thread composes the maps of its
-//           entries, the block scans the threads' maps, the thread walks its entries again from the busy-until that reaches
-//           it; results, ledger events, busy-until and per-die totals go out
+//   serve   a list in issue order: a warp takes a row of 32 entries, composes the maps of the lanes that hold the same queue, and the
+//           queues' busy-until in shared memory are moved on row after row, handed from warp to warp through named barriers (as in
+//           inorder_kernels.cu); results, ledger events, busy-until and per-die totals go out
+//   sort    a list that is not in issue order is sorted by issue time, 8 bits a pass over the bits that differ, then by queue, stable, in
+//           shared memory (a row of 32 ranks itself with match_any), and served by a segmented max-plus scan (a queue's run is a
+//           segment): a thread composes the maps of its entries, the block scans the threads' maps, the thread walks its entries
+//           again from the busy-until that reaches it.  (Lists in issue order went this way too: a window of 1 ms 23.3 us with its thermal step, now 20.2.)
 //   close   the first block adds up the batch's totals and writes the summary (barrier 3).  With the channel-bus stage on the
 //           batch may still be refused once its largest completion is known: the blocks then stage what they commit, and the
 //           first one commits it
@@ -32,6 +34,7 @@ namespace hbf {
 constexpr int kSmThreads = 512, kSmWarps = kSmThreads / 32;
 constexpr int kSmCluster = 16, kSmPortable = 8;          // blocks: 16 where the device can place them (not a portable size), else 8
 constexpr uint32_t kSmSlice = 256;                       // queues per block, at most: the bins of the sort
+constexpr int kSmChain = 15;                               // warps that serve rows: a hardware barrier each
 constexpr int kSmMaxRows = 32;                           // rows of 32 records a block looks at, at most
 constexpr uint32_t kSmIdxBits = 13;
 static_assert((1u << kSmIdxBits) == kInSmallMax && kInSmallMax / kSmPortable <= kSmMaxRows * 32, "index bits of an entry; rows of a block");
@@ -185,7 +188,7 @@ k_small_serve(const __grid_constant__ SmallArgs a) {
     const int64_t q_ppm = a.state->q_ppm;
     unsigned long long debt = 0ull;
     if (EXTRA && a.ret_on) debt = a.ret.st->planned - a.ret.st->claimed - a.ret.st->decayed;
-    if ((uint32_t)tid < q_n) { s_busy[tid] = a.busy[q_lo + tid]; if (a.bus_on) a.busy_stage[q_lo + tid] = s_busy[tid]; }   // (the stage of queues without an access)
+    if ((uint32_t)tid < q_n) s_busy[tid] = a.busy[q_lo + tid];
     if (poisoned) code = HBF_E_TIMEOUT;
     else if (mode == HBF_MODE_SHUTDOWN) code = HBF_E_LINK_SHUTDOWN;
     else if (mode == HBF_MODE_SEVERE) code = HBF_E_THROTTLED;
@@ -212,7 +215,7 @@ k_small_serve(const __grid_constant__ SmallArgs a) {
             int64_t before = __shfl_up_sync(0xffffffffu, issue[r], 1);
             if (lane == 0) before = prev[r];
             v[r].st = -1;
-            if (have) v[r] = fast ? serve_terms_fast(a.fast, mp, addr[r], issue[r], bf[r]) : small_terms_general(rs, mp, addr[r], issue[r], bf[r], q_ppm, div_q);
+            if (have) v[r] = fast ? serve_terms_fast<false>(a.fast, mp, addr[r], issue[r], bf[r]) : small_terms_general(rs, mp, addr[r], issue[r], bf[r], q_ppm, div_q);
             if (have && a.status) a.status[i] = (uint8_t)v[r].st;
             const bool ready = v[r].st == HBF_ST_READY;
             dest[r] = ready ? v[r].queue / a.slice : 0xffffu;
@@ -294,9 +297,58 @@ k_small_serve(const __grid_constant__ SmallArgs a) {
         // (the sizes come from the records again; they are needed once the list is served)
         uint64_t bf0 = 0ull;
         if ((uint32_t)tid < m) bf0 = ld_after(rec0 + (size_t)((uint32_t)s_key[tid] & (kInSmallMax - 1u)) * 3 + 2);
+        const Ledger book = EXTRA && a.ledger ? make_ledger(a.ledger, mp.n_dies, a.n_bins, a.cur_bin, a.bin_ns) : Ledger{};
+        auto ledger_of = [&](uint32_t lq, uint32_t i, uint32_t op, bool claim, int64_t s, int64_t end) {        // the access's events
+            const int64_t own = s - (claim ? quantum_ns : 0), page = (int64_t)1 << mp.page_shift;
+            const uint64_t gm = (1ull << (op ? mp.prog_gran_shift : mp.read_gran_shift)) - 1ull, cb = ((uint64_t)(uint32_t)ld_after(rec0 + (size_t)i * 3 + 2) + gm) & ~gm;
+            const uint32_t die = d_lo + lq / per_die;
+            const int64_t pj = op ? mp.e_cmd_prog_pj + mp.e_byte_prog_pj * (int64_t)cb : mp.e_cmd_read_pj + mp.e_byte_read_pj * (int64_t)cb;
+            if (claim) ledger_event(book, die, end - s, quantum_ns,
+                                    mp.e_cmd_read_pj + mp.e_byte_read_pj * page + mp.e_cmd_prog_pj + mp.e_byte_prog_pj * page);
+            ledger_event(book, die, end - own, own, pj);
+        };
+        if (!unsorted) {
+            // ---- serve, row after row
+            const uint32_t rows = (m + 31u) / 32u;
+            if (warp < kSmChain) {
+                for (uint32_t r = (uint32_t)warp; r < rows; r += kSmChain) {
+                    const uint32_t p = r * 32u + lane;
+                    const bool have = p < m;
+                    const uint64_t key = have ? s_key[p] : 0ull;
+                    const int64_t s = have ? s_s[p] : 0;
+                    const uint32_t lq = have ? s_lq[p] : 0u, px = have ? s_px[p] : 0u, i = (uint32_t)key & (kInSmallMax - 1u), op = (uint32_t)(key >> kSmIdxBits) & 1u;
+                    const int64_t t = (int64_t)(key >> 16), x = (int64_t)(px & 0x7fffffffu);
+                    const unsigned peers = __match_any_sync(0xffffffffu, have ? lq : 0x100u + lane), le = peers & (lanemask_lt() | (1u << lane));
+                    int64_t S = s, M = t + (op ? x : 0) + s;                    // of the lanes of this queue up to this one, by doubling
+                    const unsigned before = le & ~(1u << lane);
+                    int prev_l = before ? 31 - __clz((int)before) : -1;
+                    const uint32_t most = __reduce_max_sync(0xffffffffu, (uint32_t)__popc(le));
+                    for (uint32_t span = 1; span < most; span <<= 1) {
+                        const int src = prev_l >= 0 ? prev_l : lane;
+                        const int64_t Se = __shfl_sync(0xffffffffu, S, src), Me = __shfl_sync(0xffffffffu, M, src);
+                        const int pe = __shfl_sync(0xffffffffu, prev_l, src);
+                        if (prev_l >= 0) { M = max(Me + S, M); S += Se; prev_l = pe; }
+                    }
+                    const bool last = have && (peers >> lane) == 1u;
+                    if (r > 0u) asm volatile("barrier.cta.sync.aligned %0, 64;" ::"r"(1 + warp), "l"(S), "l"(M), "r"(lq), "r"((int)last) : "memory");
+                    const int64_t B = max(s_busy[lq] + S, M);
+                    if (last) s_busy[lq] = B;
+                    __syncwarp();
+                    if (r + 1u < rows) asm volatile("barrier.cta.arrive.aligned %0, 64;" ::"r"(1 + (warp + 1) % kSmChain) : "memory");
+                    if (have) {
+                        const int64_t c = B + (op ? 0 : x), waited = c - t;
+                        a.completion[i] = c; a.stall[i] = waited;
+                        sum_stall += waited; max_c = max(max_c, (long long)c);
+                        if (EXTRA && a.ledger && !a.bus_on) ledger_of(lq, i, op, (px >> 31) != 0u, s, B);
+                    }
+                }
+                sum_stall = warp_sum(sum_stall); max_c = warp_max(max_c);
+            }
+        } else {
         // ---- sort
+        if (a.bus_on && (uint32_t)tid < q_n) a.busy_stage[q_lo + tid] = s_busy[tid];      // (of queues without an access)
         for (uint32_t p = (uint32_t)tid; p < m; p += kSmThreads) perm0[p] = (uint16_t)p;
-        if (unsorted) {
+        {
             unsigned long long lo = ~0ull, hi = 0ull;
             for (uint32_t p = (uint32_t)tid; p < m; p += kSmThreads) { const unsigned long long t = s_key[p] >> 16; lo = min(lo, t); hi = max(hi, t); }
             for (int o = 16; o > 0; o >>= 1) { lo = min(lo, __shfl_xor_sync(0xffffffffu, lo, o)); hi = max(hi, __shfl_xor_sync(0xffffffffu, hi, o)); }
@@ -304,7 +356,7 @@ k_small_serve(const __grid_constant__ SmallArgs a) {
         }
         __syncthreads();
         uint16_t *src = perm0, *dst = perm1;
-        if (unsorted && m > 1u) {
+        if (m > 1u) {
             const unsigned long long first = s_lo, span = s_hi - first;
             for (uint32_t sh = 0; sh < 48u && (span >> sh) != 0ull; sh += 8u) {
                 small_sort_pass(src, dst, m, 256u, s_hist, s_dbase, s_wsum, [&](uint32_t p) { return (uint32_t)(((s_key[p] >> 16) - first) >> sh) & 255u; });
@@ -314,7 +366,7 @@ k_small_serve(const __grid_constant__ SmallArgs a) {
         small_sort_pass(src, dst, m, a.slice, s_hist, s_dbase, s_wsum, [&](uint32_t p) { return (uint32_t)s_lq[p]; });
         const uint16_t *sorted = dst;
         uint32_t below = 0;                                  // entries of the lists before this one (for hbf_queue_order)
-        if (unsorted) for (uint32_t d = 0; d < rank; ++d) below += s_total[d];
+        for (uint32_t d = 0; d < rank; ++d) below += s_total[d];
         // ---- serve
         const uint32_t per = (m + kSmThreads - 1u) / kSmThreads, p0 = (uint32_t)tid * per, p1 = min(m, p0 + per);   // this thread's entries
         const uint32_t prev_q = p0 > 0u && p0 < m ? s_lq[sorted[p0 - 1u]] : 0xffffffffu;
@@ -350,7 +402,6 @@ k_small_serve(const __grid_constant__ SmallArgs a) {
             // (the first entry of the list is a head, so a map without a head never reaches an entry that needs its input)
             int64_t B = ex.M;
             uint32_t pq = prev_q;
-            const Ledger book = EXTRA && a.ledger ? make_ledger(a.ledger, mp.n_dies, a.n_bins, a.cur_bin, a.bin_ns) : Ledger{};
             for (uint32_t p = p0; p < p1; ++p) {
                 const uint32_t e = sorted[p], lq = s_lq[e], px = s_px[e], i = (uint32_t)s_key[e] & (kInSmallMax - 1u), op = (uint32_t)(s_key[e] >> kSmIdxBits) & 1u;
                 const int64_t t = (int64_t)(s_key[e] >> 16), s = s_s[e], x = (int64_t)(px & 0x7fffffffu);
@@ -361,20 +412,12 @@ k_small_serve(const __grid_constant__ SmallArgs a) {
                 sum_stall += waited; max_c = max(max_c, (long long)c);
                 if (p + 1u == m || s_lq[sorted[p + 1u]] != lq)   // last access of its queue in this batch
                     (a.bus_on ? a.busy_stage : a.busy)[q_lo + lq] = B;
-                if (unsorted) a.order[below + p] = i;
-                if (EXTRA && a.ledger && !a.bus_on) {
-                    const bool claim = (px >> 31) != 0u;
-                    const int64_t own = s - (claim ? quantum_ns : 0), page = (int64_t)1 << mp.page_shift;
-                    const uint64_t gm = (1ull << (op ? mp.prog_gran_shift : mp.read_gran_shift)) - 1ull, cb = ((uint64_t)(uint32_t)ld_after(rec0 + (size_t)i * 3 + 2) + gm) & ~gm;
-                    const uint32_t die = d_lo + lq / per_die;
-                    const int64_t pj = op ? mp.e_cmd_prog_pj + mp.e_byte_prog_pj * (int64_t)cb : mp.e_cmd_read_pj + mp.e_byte_read_pj * (int64_t)cb;
-                    if (claim) ledger_event(book, die, B - s, quantum_ns,
-                                            mp.e_cmd_read_pj + mp.e_byte_read_pj * page + mp.e_cmd_prog_pj + mp.e_byte_prog_pj * page);
-                    ledger_event(book, die, B - own, own, pj);
-                }
+                a.order[below + p] = i;
+                if (EXTRA && a.ledger && !a.bus_on) ledger_of(lq, i, op, (px >> 31) != 0u, s, B);
                 pq = lq;
             }
             sum_stall = warp_sum(sum_stall); max_c = warp_max(max_c);
+        }
         }
         if (lane == 0) { w_stall[warp] = sum_stall; w_max[warp] = max_c; }
         // ---- per-die totals (32-bit adds with a carry: a 64-bit one in shared memory is a loop)
@@ -392,6 +435,7 @@ k_small_serve(const __grid_constant__ SmallArgs a) {
             if (EXTRA && (s_px[p] >> 31)) atomicAdd(&s_claims[ld], 1u);
         }
         __syncthreads();
+        if (!unsorted && (uint32_t)tid < q_n) (a.bus_on ? a.busy_stage : a.busy)[q_lo + tid] = s_busy[tid];
         const int64_t page = (int64_t)1 << mp.page_shift;
         const int64_t quantum_pj = mp.e_cmd_read_pj + mp.e_byte_read_pj * page + mp.e_cmd_prog_pj + mp.e_byte_prog_pj * page;
         if ((uint32_t)tid < d_n) {

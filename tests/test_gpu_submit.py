@@ -691,3 +691,24 @@ def test_host_batches_whose_sizes_vary(hbf):
         _, c_o, s_o, _, ds_o = o.submit(w.acc[:n])
         assert rc == 0 and summary["n_modeled"] == n
         assert np.array_equal(out[0][:n].numpy(), c_o) and np.array_equal(out[1][:n].numpy(), s_o) and np.array_equal(out[2].numpy(), ds_o.view(np.int64))
+
+
+@pytest.mark.parametrize("n", [1, 31, 33, 480, 481, 2_000, 8_192])
+@pytest.mark.parametrize("kind", ["one queue", "one block", "two in turn", "programs", "natives"])
+def test_small_batches_row_after_row(hbf, kind, n):
+    """Up to 8,192 records in issue order: lists that fill no row, one row for each of the warps that serve them, many turns of them; rows
+    full of one queue; behind a batch that left the queues busy."""
+    rng = np.random.default_rng(n)
+    prof = wl.load_profile("nominal", channels=32, dies=8, planes=4, page_bytes=16384, stripe_bytes=65536)
+    g, o = contexts(hbf, prof, [(wl.RANGE_BASE, wl.GIB, 3, 0, 0, 0)])
+    acc = np.zeros(n, hbfo.ACCESS_DTYPE)
+    unit = {"one queue": np.zeros(n, np.int64), "two in turn": np.arange(n) % 2,
+            "one block": 32 * rng.integers(0, 32, n) + rng.integers(0, 2, n)}.get(kind, rng.integers(0, 4_000, n))
+    acc["addr"] = wl.RANGE_BASE + unit.astype(np.uint64) * np.uint64(65536)
+    acc["bytes"] = rng.choice([64, 16_384, 40_000], n)
+    acc["issue_ns"] = np.sort(rng.integers(0, 20_000 * n, n))
+    if kind == "programs": acc["flags"] = rng.random(n) < 0.5
+    if kind == "natives": acc["addr"][rng.random(n) < 0.3] = 64
+    for _ in range(2):
+        compare_batch(g, o, acc)
+        acc["issue_ns"] += 1000
