@@ -43,6 +43,26 @@ __device__ __forceinline__ uint64_t ld_after(const uint64_t *p) { uint64_t v; as
 __device__ __forceinline__ int64_t ld_after(const int64_t *p) { int64_t v; asm volatile("ld.global.s64 %0, [%1];" : "=l"(v) : "l"(p)); return v; }
 __device__ __forceinline__ longlong2 ld_after(const longlong2 *p) { longlong2 v; asm volatile("ld.global.v2.s64 {%0, %1}, [%2];" : "=l"(v.x), "=l"(v.y) : "l"(p)); return v; }
 
+// Thread-block clusters: a place in another block's shared memory; a value sent there, counted in bytes by a barrier beside it; one poll of such
+// a barrier.
+__device__ __forceinline__ uint32_t smem_addr(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ uint32_t smem_remote(uint32_t addr, uint32_t rank) {
+    uint32_t r; asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank)); return r;
+}
+__device__ __forceinline__ void smem_send(uint32_t addr, uint32_t v, uint32_t bar) {
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.u32 [%0], %1, [%2];" ::"r"(addr), "r"(v), "r"(bar) : "memory");
+}
+__device__ __forceinline__ void smem_send(uint32_t addr, long long v, uint32_t bar) {
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.u64 [%0], %1, [%2];" ::"r"(addr), "l"(v), "r"(bar) : "memory");
+}
+__device__ __forceinline__ bool smem_poll(uint32_t bar, uint32_t parity) {
+    uint32_t done;
+    asm volatile("{ .reg .pred p; mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2; selp.u32 %0, 1, 0, p; }"
+                 : "=r"(done) : "r"(bar), "r"(parity) : "memory");
+    return done != 0u;
+}
+constexpr uint32_t kClusterPolls = 1u << 22;             // of such a barrier, before a wait is given up
+
 // ---- division by a run-time constant ----------------------------------------------------------------
 // For d not a power of two, l = ceil(log2 d), magic = floor(2^(63+l) / d) + 1: floor(n / d) =
 // mulhi(n, magic) >> (l - 1) for every n < 2^63 (the error term n * (magic*d - 2^(63+l)) stays below 2^(63+l)).

@@ -1,6 +1,6 @@
 // Small batches (at most kInSmallMax records) in one launch of one thread-block cluster, instead of tiles, a scan, a fix-up and a
 // straggle pass whose fixed costs a few thousand records cannot pay for.  A block looks at a share of the records, and serves and
-// commits a share of the queues (whole dies); queues do not interact, so nothing waits but for the three cluster barriers.
+// commits a share of the queues (whole dies); queues do not interact, so nothing waits but for two cluster barriers and the totals at the end.
 //   look    a thread per record: status, queue, service terms; counts per destination block, stable ranks.  The blocks
 //           exchange their counts (barrier 1), so every block knows the whole batch's statuses, order and claims, takes the
 //           same decision about it, and knows where its records go
@@ -13,7 +13,7 @@
 //           shared memory (a row of 32 ranks itself with match_any), and served by a segmented max-plus scan (a queue's run is a
 //           segment): a thread composes the maps of its entries, the block scans the threads' maps, the thread walks its entries
 //           again from the busy-until that reaches it.  (Lists in issue order went this way too: a window of 1 ms 23.3 us with its thermal step, now 20.2.)
-//   close   the first block adds up the batch's totals and writes the summary (barrier 3).  With the channel-bus stage on the
+//   close   the first block adds up the batch's totals and writes the summary: they are sent to its shared memory, and the others are done.  With the channel-bus stage on the
 //           batch may still be refused once its largest completion is known: the blocks then stage what they commit, and the
 //           first one commits it
 // Bound by the latency of some thirty dependent steps.  Every block looking at all the records (no exchange) took 57,000 warp
@@ -143,9 +143,15 @@ k_small_serve(const __grid_constant__ SmallArgs a) {
     __shared__ long long s_tot[kSmCluster][3];               // (first block) every block's stalls, services, largest completion
     __shared__ Div64 s_div;
     cg::cluster_group cluster = cg::this_cluster();
-    cluster.barrier_arrive();                                // (waited for below: every block runs before one writes into another)
+    __shared__ __align__(8) uint64_t s_bar;                  // (first block) every block's totals have come
     const uint32_t rank = cluster.block_rank(), blocks = cluster.num_blocks();
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    if (tid == 0) {
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(&s_bar)) : "memory");
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(&s_bar)), "r"(blocks * 24u) : "memory");
+    }
+    cluster.barrier_arrive();                                // (waited for below: every block runs before one writes into another)
     const ModelParams &mp = a.mp;
     const RangeSnap &rs = *a.ranges;
     const uint32_t n = a.n, padded = (n + 255u) / 256u * 256u;
@@ -469,17 +475,22 @@ k_small_serve(const __grid_constant__ SmallArgs a) {
             long long work = 0;
             for (uint32_t d = (uint32_t)lane; d < d_n; d += 32u) work += (long long)(((uint64_t)s_work[1][d] << 32) | s_work[0][d]);
             work = warp_sum(work);
-            if (lane == 0) { long long *t = cluster.map_shared_rank(&s_tot[0][0], 0) + rank * 3; t[0] = stall; t[1] = work; t[2] = latest; }
+            if (lane < 3) smem_send(smem_remote(smem_addr(&s_tot[rank][lane]), 0u), lane == 0 ? stall : lane == 1 ? work : latest, smem_remote(smem_addr(&s_bar), 0u));
         }
     } else if (code != HBF_E_LINK_SHUTDOWN && code != HBF_E_THROTTLED) {              // refused: zeroed outputs, nothing changed
         for (uint32_t i = begin + tid; i < end; i += kSmThreads) { a.completion[i] = 0; a.stall[i] = 0; }
         if (a.die_stats) for (uint32_t e = (uint32_t)tid; e < d_n * 6u; e += kSmThreads) reinterpret_cast<int64_t *>(a.die_stats + d_lo)[e] = 0;
     }
-    cluster.sync();
-    if (rank != 0u) return;
-    // ---- close
+    // ---- close: the others have sent their totals and are done (with the bus on the first one has to see what they staged)
+    if (a.bus_on) cluster.sync();
+    if (rank != 0u || (!a.bus_on && warp != 0)) return;
     long long modeled = 0, service = 0, latest = 0;
-    if (code == HBF_OK) for (uint32_t b = 0; b < blocks; ++b) { modeled += s_tot[b][0]; service += s_tot[b][1]; latest = max(latest, s_tot[b][2]); }
+    if (code == HBF_OK) {
+        uint32_t polls = 0;
+        while (!smem_poll(smem_addr(&s_bar), 0u)) if (++polls > kClusterPolls) { a.state->poisoned = 1; code = HBF_E_TIMEOUT; break; }
+        const bool from = (uint32_t)lane < blocks;
+        modeled = warp_sum(from ? s_tot[lane][0] : 0); service = warp_sum(from ? s_tot[lane][1] : 0); latest = warp_max(from ? s_tot[lane][2] : 0);
+    }
     if (a.bus_on) {                                          // commit what the blocks staged, or refuse (array-done times are sort keys of 47 bits)
         if (code == HBF_OK && n_ready && latest >= HBF_ISSUE_LIMIT) {
             code = HBF_E_INVAL;
@@ -507,7 +518,7 @@ k_small_serve(const __grid_constant__ SmallArgs a) {
         BatchCtrl *c = a.ctrl;                               // what later stages and hbf_queue_order read of a batch
         c->code = code; c->skip = ok ? 0 : 1; c->mode = mode; c->q_ppm = q_ppm; c->div_q = div_q;
         c->n_ready = n_ready; c->inorder_used = ok && !unsorted ? 1u : 0u; c->run_sort = 0u; c->regrouped = 0u; c->plan.n_passes = 1u;
-        if (EXTRA && a.ret_on && !a.bus_on && ok) a.ret.st->claimed += claims;
+        if (EXTRA && a.ret_on && !a.bus_on && ok && claims) atomicAdd(&a.ret.st->claimed, claims);      // (nothing waits for it)
     }
 }
 

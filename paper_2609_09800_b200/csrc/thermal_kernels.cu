@@ -145,21 +145,8 @@ constexpr int kThThreads = 512;
 constexpr int kThPairsPerThread = 4;
 constexpr int kThMaxRegions = 1024;
 constexpr uint32_t kThTermDies = 1024;                     // dies whose power terms are formed a thread each
-constexpr uint32_t kThWaitPolls = 1u << 22;
 
-__device__ __forceinline__ uint32_t th_smem(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
-__device__ __forceinline__ uint32_t th_remote(uint32_t addr, uint32_t rank) {
-    uint32_t r; asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank)); return r;
-}
-__device__ __forceinline__ void th_send(uint32_t addr, float v, uint32_t bar) {
-    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.u32 [%0], %1, [%2];" ::"r"(addr), "r"(__float_as_uint(v)), "r"(bar) : "memory");
-}
-__device__ __forceinline__ bool th_poll(uint32_t bar, uint32_t parity) {
-    uint32_t done;
-    asm volatile("{ .reg .pred p; mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2; selp.u32 %0, 1, 0, p; }"
-                 : "=r"(done) : "r"(bar), "r"(parity) : "memory");
-    return done != 0u;
-}
+__device__ __forceinline__ void th_send(uint32_t addr, float v, uint32_t bar) { smem_send(addr, __float_as_uint(v), bar); }
 
 // floats as integers of the same order
 __device__ __forceinline__ int th_order(float f) { const int k = __float_as_int(f); return k >= 0 ? k : k ^ 0x7fffffff; }
@@ -187,7 +174,7 @@ k_thermal_cluster(const __grid_constant__ ThermalDev t, float *theta, DevState *
     float2 *buf0 = reinterpret_cast<float2 *>(th_smem_buf);
     const bool has_up = rank > 0u && mine > 0u, has_down = y1 < H && mine > 0u;
     if (tid < 3) {
-        const uint32_t bar = th_smem(tid < 2 ? &s_bar[tid] : &s_bar_hot);
+        const uint32_t bar = smem_addr(tid < 2 ? &s_bar[tid] : &s_bar_hot);
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar) : "memory");
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         if (tid == 2) asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(n_blocks * 12u) : "memory");
@@ -204,10 +191,10 @@ k_thermal_cluster(const __grid_constant__ ThermalDev t, float *theta, DevState *
         const uint32_t li = (uint32_t)c * kThThreads + tid, pr = li / W, x = li - pr * W;
         off[c] = W; up[c] = down[c] = 0u;
         if (li < pairs) {
-            const uint32_t b0 = th_smem(buf0);
+            const uint32_t b0 = smem_addr(buf0);
             off[c] = (pr + 1u) * W + x;
-            if (pr == 0u && has_up) up[c] = th_remote(b0 + row_at((int32_t)rows, x), rank - 1u);          // (a block above another is full)
-            if (pr == (mine - 1u) / 2u && has_down) down[c] = th_remote(b0 + row_at(-1, x), rank + 1u);
+            if (pr == 0u && has_up) up[c] = smem_remote(b0 + row_at((int32_t)rows, x), rank - 1u);          // (a block above another is full)
+            if (pr == (mine - 1u) / 2u && has_down) down[c] = smem_remote(b0 + row_at(-1, x), rank + 1u);
         }
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
@@ -234,8 +221,8 @@ k_thermal_cluster(const __grid_constant__ ThermalDev t, float *theta, DevState *
     double p_idle = 0.0, p_ext = 0.0;
     if ((uint32_t)tid < t.n_regions) { g0 = t.region_die_ptr[tid]; g1 = t.region_die_ptr[tid + 1]; p_idle = (double)t.region_idle_w[tid]; if (has_ext) p_ext = (double)t.ext_power[tid]; }
     for (uint32_t i = tid; i < 2u * pitch; i += kThThreads) buf0[i] = make_float2(0.0f, 0.0f);      // (rows outside the grid stay 0)
-    const uint32_t bar0 = th_smem(&s_bar[0]);
-    const uint32_t up_bar = has_up ? th_remote(bar0, rank - 1u) : 0u, down_bar = has_down ? th_remote(bar0, rank + 1u) : 0u;
+    const uint32_t bar0 = smem_addr(&s_bar[0]);
+    const uint32_t up_bar = has_up ? smem_remote(bar0, rank - 1u) : 0u, down_bar = has_down ? smem_remote(bar0, rank + 1u) : 0u;
     const uint32_t expect = ((has_up ? 1u : 0u) + (has_down ? 1u : 0u)) * W * 4u;
     __syncthreads();
     pdl_wait();                                               // from here on: what the kernels before left
@@ -329,7 +316,7 @@ k_thermal_cluster(const __grid_constant__ ThermalDev t, float *theta, DevState *
         }
         if (more && expect && !lost) {
             uint32_t polls = 0;
-            while (!th_poll(bar0 + ob * 8u, (k >> 1) & 1u)) if (++polls > kThWaitPolls) { lost = true; break; }
+            while (!smem_poll(bar0 + ob * 8u, (k >> 1) & 1u)) if (++polls > kClusterPolls) { lost = true; break; }
         }
         __syncthreads();
     }
@@ -360,13 +347,13 @@ k_thermal_cluster(const __grid_constant__ ThermalDev t, float *theta, DevState *
     __syncthreads();
     if (warp < 3) {
         const int v = __reduce_max_sync(0xffffffffu, lane < kThThreads / 32 ? s_part[warp][lane] : th_order(-INFINITY));
-        if (lane == 0) th_send(th_remote(th_smem(&s_hot[warp][rank]), 0u), __int_as_float(v), th_remote(th_smem(&s_bar_hot), 0u));
+        if (lane == 0) th_send(smem_remote(smem_addr(&s_hot[warp][rank]), 0u), __int_as_float(v), smem_remote(smem_addr(&s_bar_hot), 0u));
     }
     if (rank != 0u || warp != 0) return;
     {
-        const uint32_t bar = th_smem(&s_bar_hot);
+        const uint32_t bar = smem_addr(&s_bar_hot);
         uint32_t polls = 0;
-        while (!th_poll(bar, 0u)) if (++polls > kThWaitPolls) { state->poisoned = 1; break; }
+        while (!smem_poll(bar, 0u)) if (++polls > kClusterPolls) { state->poisoned = 1; break; }
     }
     float h[3];
 #pragma unroll
