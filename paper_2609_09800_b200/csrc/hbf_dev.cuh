@@ -179,7 +179,7 @@ inline cudaError_t launch_first(bool *plain_next, Kernel k, dim3 grid, dim3 bloc
 
 constexpr uint32_t kInMaxQueues = 2048;  // the in-order path keeps per-queue state in shared memory
 constexpr uint32_t kInMaxTiles = 1024;
-constexpr uint32_t kInTileQuantum = 1024; // tiles of the in-order path are a multiple of this many records
+constexpr uint32_t kInTileQuantum = 1024; // tiles of the in-order path are a multiple of this many records (of 256 where their sizes follow measurements)
 constexpr uint32_t kInQidPrefix = 131072; // records at the head of a tile whose queue numbers the serve pass leaves for the straggle pass
 // 16-bit queue numbers kept for a batch of n records (an upper bound over every tiling of it)
 inline uint64_t inorder_qid_entries(uint64_t n) {
@@ -200,7 +200,7 @@ constexpr size_t kBusPlanAt = 4096, kBusPlanBytes = 8192;
 cudaError_t launch_bus_stage(const SubmitArgs &a, BatchCtrl *bc, int64_t *bus_busy, cudaStream_t st);
 cudaError_t launch_bus_buckets(const SubmitArgs &a, BatchCtrl *bc, int64_t *bus_busy, cudaStream_t st);
 // How the in-order path cuts a batch of n records into contiguous tiles: n_big tiles of `big` records, then tiles of
-// `small` records (the last one ragged).  All sizes are multiples of kInTileQuantum.  n_big == 0: one size only.
+// `small` records (the last one ragged).  All these sizes are multiples of kInTileQuantum.  n_big == 0: one size only.
 // With `first` set (device memory, n_tiles + 1 entries) the tiles begin where that table says instead: sizes that follow
 // from how long each tile's block took in an earlier batch (TileBalance below).  by_sm: a block takes the tile of its SM
 // and of its kind (tile = kind * n_big + SM), so that a tile's time tells how fast that place serves.
