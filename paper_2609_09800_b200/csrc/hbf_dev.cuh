@@ -57,7 +57,11 @@ struct SortPlan {
 
 // regroup.cuh: the shares of every phase that are taken and done, the spread of the issue times.  Zero between batches: the begin
 // kernel clears what the last kernel uses, and the other way round.
-struct RegroupSync { uint32_t claim[8], done[8], hist[64], top[64], below[64]; };   // (samples of a stretch, their largest offset, 2^32 - 1 less their smallest)
+// sort_*: the same of the radix sort as phases of the last kernel (SortPhase), and the blocks that are through with it; the last of them leaves zeros.
+struct RegroupSync {
+    uint32_t claim[8], done[8], hist[64], top[64], below[64];   // (samples of a stretch, their largest offset, 2^32 - 1 less their smallest)
+    uint32_t sort_claim[16], sort_done[16], sort_failed, sort_left;
+};
 
 // Per-batch control block in device memory, cleared by the begin kernel.
 struct BatchCtrl {

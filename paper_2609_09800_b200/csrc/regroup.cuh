@@ -97,13 +97,13 @@ __device__ __forceinline__ bool rg_wait_or_give_up(RegroupSync *s, int phase, ui
     return ok;
 }
 
-// The results of a regrouped batch back to batch order (blocks of the last kernel).  Behind the one wait nothing can fail any more: the
-// block that takes the first output bucket calls commit() then, beside the others' work.  A block whose wait runs out leaves the rest
+// The results of a regrouped batch back to batch order (blocks of the last kernel, in groups of 256 threads: a bucket each).  Behind the one
+// wait nothing can fail any more: the first block that is past it calls commit() then, beside the others' work.  A block whose wait runs out leaves the rest
 // to those that got past it; true: this block is the last to leave, and none did (nothing was committed, no result given back).
 template <class Commit>
-__device__ __forceinline__ bool rg_give_back(const RegroupArgs &r, uint64_t n, const DevState *state, int64_t *__restrict__ completion, int64_t *__restrict__ stall, Commit &&commit) {
-    __shared__ ulonglong2 s_out[kRgOut];
-    __shared__ uint32_t s_b;
+__device__ __forceinline__ bool rg_give_back(const RegroupArgs &r, uint64_t n, const DevState *state, int64_t *__restrict__ completion, int64_t *__restrict__ stall, ulonglong2 *s_out, Commit &&commit) {      // s_out: [kRgOut] of shared memory per group
+    constexpr int kGroup = 256;
+    __shared__ uint32_t s_b, s_bucket[4];
     constexpr uint32_t kGive = 1024;                         // records of a share
     const int tid = threadIdx.x, lane = tid & 31;
     const uint32_t gives = (uint32_t)((n + kGive - 1) / kGive);
@@ -132,23 +132,28 @@ __device__ __forceinline__ bool rg_give_back(const RegroupArgs &r, uint64_t n, c
         __syncthreads();
         return s_b == gridDim.x - 1u;
     }
+    if (tid == 0) s_b = atomicAdd(&r.sync->claim[6], 1u);
+    __syncthreads();
+    if (s_b == 0u) commit();
+    const int group = tid / kGroup, gtid = tid % kGroup;
+    auto group_sync = [&] { asm volatile("bar.sync %0, %1;" ::"r"(1 + group), "n"(kGroup) : "memory"); };
+    s_out += (size_t)group * kRgOut;
     for (;;) {
-        __syncthreads();                                     // the results of the bucket before have been read
-        if (tid == 0) s_b = atomicAdd(&r.sync->claim[4], 1u);
-        __syncthreads();
-        const uint32_t b = s_b;
+        group_sync();                                        // the results of the bucket before have been read
+        if (gtid == 0) s_bucket[group] = atomicAdd(&r.sync->claim[4], 1u);
+        group_sync();
+        const uint32_t b = s_bucket[group];
         if (b >= r.out_buckets) return false;
-        if (b == 0u) commit();
         const uint64_t base = (uint64_t)b * kRgOut;
         const uint32_t m = (uint32_t)min((uint64_t)kRgOut, n - base);
 #pragma unroll 8
-        for (uint32_t e = tid; e < m; e += blockDim.x) {
+        for (uint32_t e = gtid; e < m; e += kGroup) {
             const ulonglong2 v = __ldcg(r.entries + rg_place(r.out_buckets, b, e));
             s_out[(uint32_t)v.y & 0xffffu] = make_ulonglong2(v.x, v.x - (v.y >> 16));
         }
-        __syncthreads();
+        group_sync();
 #pragma unroll 4
-        for (uint32_t e = tid; e < m; e += blockDim.x) {
+        for (uint32_t e = gtid; e < m; e += kGroup) {
             const ulonglong2 v = s_out[e];
             __stcs(reinterpret_cast<long long *>(completion + base + e), (long long)v.x);
             __stcs(reinterpret_cast<long long *>(stall + base + e), (long long)v.y);

@@ -40,9 +40,8 @@ __device__ __forceinline__ uint32_t rg_stretch(int64_t t, int64_t lo, uint32_t s
 
 // Do so many records share their issue times that buckets would overflow, or spend their time on telling equal times apart?  1,024
 // samples, one per thread, and a table of the distinct ones; where few are equal, pairs of equal ones tell (of m samples of D times
-// about m^2 / 2D), else the distinct ones are nearly all there are.  40 M shuffled records, us, by the radix sort as it is launched from the
-// device 7,700 (and 8,200 before there were buckets; the attempt adds 700 if it overflows); in buckets 2,850 with 1 record per
-// time, 3,700 with 50, 7,100 with 500; more than some 900 overflow.
+// about m^2 / 2D), else the distinct ones are nearly all there are.  40 M shuffled records, us, by the radix sort CROWD_RADIX
+// (the attempt in buckets adds 700 if it overflows, from some 900 records per time on); in buckets CROWD_FIGURES.
 constexpr uint32_t kRgCrowd = 700, kRgSeen = 4096;
 __device__ __forceinline__ bool rg_crowded(long long time, uint64_t n, unsigned long long *seen) {
     for (uint32_t e = threadIdx.x; e < kRgSeen; e += kRgThreads) seen[e] = 0ull;
@@ -94,6 +93,7 @@ k_begin_regroup(const __grid_constant__ BeginArgs b, const hbf_access_t *__restr
         begin_batch(b, sorted ? 1 : 0, go ? 1u : 0u);
         if (b.decides && !sorted) begin_load(b, reinterpret_cast<const uint64_t *>(acc + (uint64_t)tid * (n - 1ull) / 1024ull), bad ? first : ld_after(&acc[0].issue_ns), bad ? last : ld_after(&acc[n - 1].issue_ns));
         if (tid < 2) sync->claim[3 + tid] = 0u;              // (those of the last kernel)
+        if (tid == 2) sync->claim[6] = 0u;
         if (tid < 3) sync->done[3 + tid] = 0u;
         __threadfence();
         __syncthreads();

@@ -17,22 +17,15 @@ namespace hbf {
 // =====================================================================================================
 // begin: snapshot mode and q (before any reservation, Eq. 3), stage the queue state, clear the block
 // =====================================================================================================
-// role 0: first kernel of a batch; run_sort tells whether the sort path serves it.
-// role 1: placed between the in-order attempt and the sort kernels; it starts the batch over for the
-//         sort path when the in-order attempt found the records out of issue order, else does nothing.
-// (a batch that may turn out to be out of issue order begins with k_begin_regroup)
-__global__ void k_begin(const __grid_constant__ BeginArgs b, int role, int run_sort, const hbf_access_t *acc) {
+// run_sort tells whether the sort path serves the batch.  (A batch that may turn out to be out of issue order begins with k_begin_regroup.)
+__global__ void k_begin(const __grid_constant__ BeginArgs b, int run_sort, const hbf_access_t *acc) {
     pdl_wait();
     pdl_trigger();
-    if (role == 1) {
-        if (b.ctrl->skip || !b.ctrl->run_sort) return;
-        run_sort = 1;
-    }
     __syncthreads();
     begin_batch(b, run_sort, 0u);
-    if (role == 0 && b.decides)
+    if (b.decides)
         begin_load(b, reinterpret_cast<const uint64_t *>(acc + (uint64_t)threadIdx.x * (b.n - 1ull) / 1024ull), ld_after(&acc[0].issue_ns), ld_after(&acc[b.n - 1].issue_ns));
-    if (role == 0 && b.unit_shift) {
+    if (b.unit_shift) {
         __syncthreads();                                     // (the control block is cleared)
         begin_units(b, reinterpret_cast<const uint64_t *>(acc + (uint64_t)threadIdx.x * (b.n - 1ull) / 1024ull));
     }
@@ -46,19 +39,17 @@ constexpr int kClsThreads = 256;
 constexpr int kClsItems = 4;
 constexpr int kClsTile = kClsThreads * kClsItems;       // 1024 records = 24 KiB
 
-// (four resident blocks per SM: 1.96 -> 1.40 ms at 200 M against three at 84 registers; six was slower)
-__global__ void __launch_bounds__(kClsThreads, 4)
-k_classify(const hbf_access_t *__restrict__ acc, uint64_t n, const RangeSnap *__restrict__ ranges_g,
-           const ModelParams *__restrict__ mp_g, BatchCtrl *ctrl, uint64_t *__restrict__ keys, uint64_t *__restrict__ terms,
-           uint8_t *__restrict__ status, int64_t *__restrict__ completion, int64_t *__restrict__ stall) {
+// next(): the block's next tile (of the whole block)
+template <int THREADS, class Next>
+__device__ __forceinline__ void classify_tiles(const hbf_access_t *__restrict__ acc, uint64_t n, const RangeSnap *__restrict__ ranges_g,
+           const ModelParams *__restrict__ mp_g, BatchCtrl *ctrl, uint64_t *keys, uint64_t *terms,
+           uint8_t *__restrict__ status, int64_t *completion, int64_t *stall, uint64_t *rec, Next &&next) {
     __shared__ RangeSnap rs;
     __shared__ ModelParams mp;
-    __shared__ __align__(16) uint64_t rec[kClsTile * 3];
-    if (ctrl->skip || !ctrl->run_sort) return;
     const int tid = threadIdx.x;
-    for (int i = tid; i < (int)(sizeof(RangeSnap) / 4); i += kClsThreads)
+    for (int i = tid; i < (int)(sizeof(RangeSnap) / 4); i += THREADS)
         reinterpret_cast<uint32_t *>(&rs)[i] = reinterpret_cast<const uint32_t *>(ranges_g)[i];
-    for (int i = tid; i < (int)(sizeof(ModelParams) / 4); i += kClsThreads)
+    for (int i = tid; i < (int)(sizeof(ModelParams) / 4); i += THREADS)
         reinterpret_cast<uint32_t *>(&mp)[i] = reinterpret_cast<const uint32_t *>(mp_g)[i];
     const bool aligned16 = (reinterpret_cast<uintptr_t>(acc) & 15u) == 0;
     const uint64_t sentinel = (uint64_t)mp_g->n_queues << kIssueBits;
@@ -66,7 +57,7 @@ k_classify(const hbf_access_t *__restrict__ acc, uint64_t n, const RangeSnap *__
     unsigned long long n_native = 0, n_ready = 0, n_fault = 0, k_or = 0, k_and = ~0ull;
     unsigned unsorted = 0;
     const uint64_t n_tiles = (n + kClsTile - 1) / kClsTile;
-    for (uint64_t tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
+    for (uint64_t tile = next(); tile < n_tiles; tile = next()) {
         const uint64_t base = tile * kClsTile;
         const int cnt = (int)min((uint64_t)kClsTile, n - base);
         __syncthreads();
@@ -75,14 +66,14 @@ k_classify(const hbf_access_t *__restrict__ acc, uint64_t n, const RangeSnap *__
             const uint4 *s4 = reinterpret_cast<const uint4 *>(src);
             uint4 *d4 = reinterpret_cast<uint4 *>(rec);
 #pragma unroll
-            for (int k = 0; k < kClsTile * 24 / 16 / kClsThreads; ++k) d4[tid + k * kClsThreads] = __ldg(s4 + tid + k * kClsThreads);
+            for (int k = 0; k < kClsTile * 24 / 16 / THREADS; ++k) d4[tid + k * THREADS] = __ldg(s4 + tid + k * THREADS);
         } else {
-            for (int i = tid; i < cnt * 3; i += kClsThreads) rec[i] = __ldg(src + i);
+            for (int i = tid; i < cnt * 3; i += THREADS) rec[i] = __ldg(src + i);
         }
         __syncthreads();
 #pragma unroll
-        for (int k = 0; k < kClsItems; ++k) {
-            const int li = tid + k * kClsThreads;
+        for (int k = 0; k < kClsTile / THREADS; ++k) {
+            const int li = tid + k * THREADS;
             if (li >= cnt) break;
             const uint64_t i = base + li;
             const uint64_t addr = rec[li * 3];
@@ -126,6 +117,16 @@ k_classify(const hbf_access_t *__restrict__ acc, uint64_t n, const RangeSnap *__
         if (unsorted) atomicOr(&ctrl->unsorted, 1u);
     }
 }
+// (four resident blocks per SM: 1.96 -> 1.40 ms at 200 M against three at 84 registers; six was slower)
+__global__ void __launch_bounds__(kClsThreads, 4)
+k_classify(const hbf_access_t *__restrict__ acc, uint64_t n, const RangeSnap *__restrict__ ranges_g,
+           const ModelParams *__restrict__ mp_g, BatchCtrl *ctrl, uint64_t *__restrict__ keys, uint64_t *__restrict__ terms,
+           uint8_t *__restrict__ status, int64_t *__restrict__ completion, int64_t *__restrict__ stall) {
+    __shared__ __align__(16) uint64_t rec[kClsTile * 3];
+    if (ctrl->skip || !ctrl->run_sort) return;
+    uint64_t tile = blockIdx.x;
+    classify_tiles<kClsThreads>(acc, n, ranges_g, mp_g, ctrl, keys, terms, status, completion, stall, rec, [&] { const uint64_t t = tile; tile += gridDim.x; return t; });
+}
 
 // =====================================================================================================
 // plan: refuse the batch on any fail-closed access; otherwise choose the radix passes.  Only bits that
@@ -155,9 +156,7 @@ __device__ __forceinline__ uint32_t digit_at(uint64_t key, const DigitSel &d) {
     return ((uint32_t)(key >> d.sh_lo) & d.m_lo) | (((uint32_t)(key >> d.sh_hi) & d.m_hi) << d.up);
 }
 
-__global__ void k_plan(BatchCtrl *ctrl, int force_full) {
-    if (threadIdx.x != 0 || ctrl->skip || !ctrl->run_sort) return;
-    if (ctrl->n_fault) { ctrl->code = HBF_E_ACCESS_FAULT; ctrl->skip = 1; return; }
+__device__ __forceinline__ SortPlan make_plan(const BatchCtrl *ctrl, int force_full) {
     const uint64_t diff = ctrl->key_or ^ ctrl->key_and;
     const uint64_t dlo = diff & kIssueMask, dhi = diff >> kIssueBits;
     uint32_t lo = (ctrl->unsorted || force_full) ? (dlo ? 64u - (uint32_t)__clzll((long long)dlo) : 0u) : 0u;
@@ -171,7 +170,12 @@ __global__ void k_plan(BatchCtrl *ctrl, int force_full) {
         if (i < np) b = total / np + (i < total % np ? 1u : 0u);
         p.shift[i] = shift; p.bits[i] = b; shift += b;
     }
-    ctrl->plan = p;
+    return p;
+}
+__global__ void k_plan(BatchCtrl *ctrl, int force_full) {
+    if (threadIdx.x != 0 || ctrl->skip || !ctrl->run_sort) return;
+    if (ctrl->n_fault) { ctrl->code = HBF_E_ACCESS_FAULT; ctrl->skip = 1; return; }
+    ctrl->plan = make_plan(ctrl, force_full);
 }
 
 // =====================================================================================================
@@ -180,32 +184,32 @@ __global__ void k_plan(BatchCtrl *ctrl, int force_full) {
 // =====================================================================================================
 constexpr int kHistThreads = 512;
 
+// keys [from, to) of the batch's, every `stride`-th from this thread's on (from, to: whole warps' worth, but for the batch's end)
+__device__ __forceinline__ void hist_keys(const uint64_t *keys, uint64_t n, uint64_t from, uint64_t to, uint64_t stride, const DigitSel &sel0, uint32_t *sh) {
+    const uint64_t n_round = (to + 31ull) & ~31ull;        // whole warps stay in the loop together
+    for (uint64_t i = from; i < n_round; i += stride) {
+        const bool valid = i < n;
+        const uint64_t ck = valid ? keys[i] : 0ull;
+        const uint32_t d = valid ? digit_at(ck, sel0) : 0xffffffffu;
+        // the high digits of neighbouring keys are mostly equal, the low ones mostly all different: one vote tells the
+        // two cases apart, and neither needs the lane-by-lane match (measured: 8.0 ms of a 58 ms sort at 200 M with it)
+        const uint32_t d0 = __shfl_sync(0xffffffffu, d, 0);
+        if (__all_sync(0xffffffffu, d == d0)) {
+            if (lane_id() == 0 && valid) atomicAdd(&sh[d], 32u);   // (a whole warp inside the batch: i < n for lane 0 means all)
+        } else if (valid) {
+            atomicAdd(&sh[d], 1u);
+        }
+    }
+}
 __global__ void __launch_bounds__(kHistThreads)
 k_hist(const uint64_t *__restrict__ keys, uint64_t n, const BatchCtrl *ctrl, uint32_t *hist) {
-    __shared__ uint32_t sh[kMaxPasses * kRadix];
+    __shared__ uint32_t sh[kRadix];
     if (ctrl->skip || !ctrl->run_sort) return;
     const SortPlan p = ctrl->plan;
     if (p.n_passes == 0) return;
-    const DigitSel sel0 = digit_sel(p, 0);
-    for (int i = threadIdx.x; i < kMaxPasses * kRadix; i += kHistThreads) sh[i] = 0u;
+    for (int i = threadIdx.x; i < kRadix; i += kHistThreads) sh[i] = 0u;
     __syncthreads();
-    const uint64_t stride = (uint64_t)gridDim.x * kHistThreads;
-    const uint64_t n_round = (n + 31ull) & ~31ull;         // whole warps stay in the loop together
-    for (uint64_t i = (uint64_t)blockIdx.x * kHistThreads + threadIdx.x; i < n_round; i += stride) {
-        const bool valid = i < n;
-        const uint64_t ck = valid ? keys[i] : 0ull;
-        for (uint32_t k = 0; k < 1u; ++k) {
-            const uint32_t d = valid ? digit_at(ck, sel0) : 0xffffffffu;
-            // the high digits of neighbouring keys are mostly equal, the low ones mostly all different: one vote tells the
-            // two cases apart, and neither needs the lane-by-lane match (measured: 8.0 ms of a 58 ms sort at 200 M with it)
-            const uint32_t d0 = __shfl_sync(0xffffffffu, d, 0);
-            if (__all_sync(0xffffffffu, d == d0)) {
-                if (lane_id() == 0 && valid) atomicAdd(&sh[k * kRadix + d], 32u);   // (a whole warp inside the batch: i < n for lane 0 means all)
-            } else if (valid) {
-                atomicAdd(&sh[k * kRadix + d], 1u);
-            }
-        }
-    }
+    hist_keys(keys, n, (uint64_t)blockIdx.x * kHistThreads + threadIdx.x, n, (uint64_t)gridDim.x * kHistThreads, digit_sel(p, 0), sh);
     __syncthreads();
     for (int i = threadIdx.x; i < kRadix; i += kHistThreads)
         if (sh[i]) atomicAdd(&hist[i], sh[i]);
@@ -224,12 +228,10 @@ constexpr int kSortWarps = kSortThreads / 32;
 constexpr size_t kSortSmem = (size_t)kSortTile * 12 + (size_t)kSortWarps * kRadix * 4;
 constexpr uint32_t kFlagAgg = 1u << 30, kFlagPrefix = 2u << 30, kCountMask = (1u << 30) - 1u;
 
-// (three resident blocks per SM: at one block of 80 registers the pass ran at 13 % of the DRAM rate with a quarter of the
-// warp slots in use, 4.1 ms for 200 M keys; bounded to 40 registers, with a few spills, it takes 2.5 ms)
-__global__ void __launch_bounds__(kSortThreads, 3)
-k_sort_pass(int pass, uint64_t n, BatchCtrl *ctrl, DevState *state, uint32_t *hist,
-            uint64_t *keys0, uint64_t *keys1, uint32_t *idx0, uint32_t *idx1, uint32_t *desc0, uint32_t *desc1) {
-    extern __shared__ __align__(16) unsigned char sort_smem[];
+// (the tiles that this block took; give_up(): a look-back that ran out)
+template <class GiveUp>
+__device__ __forceinline__ uint32_t sort_pass(int pass, uint64_t n, const SortPlan &pl, BatchCtrl *ctrl, const DevState *state, uint32_t *hist,
+            uint64_t *keys0, uint64_t *keys1, uint32_t *idx0, uint32_t *idx1, uint32_t *desc0, uint32_t *desc1, unsigned char *sort_smem, GiveUp &&give_up) {
     uint64_t *s_keys = reinterpret_cast<uint64_t *>(sort_smem);                       // [kSortTile]
     uint32_t *s_idx = reinterpret_cast<uint32_t *>(s_keys + kSortTile);               // [kSortTile]
     uint32_t *s_cnt = s_idx + kSortTile;                                              // [kSortWarps][kRadix]
@@ -238,9 +240,6 @@ k_sort_pass(int pass, uint64_t n, BatchCtrl *ctrl, DevState *state, uint32_t *hi
     __shared__ uint32_t s_warp_tot[kRadix / 32], s_hist_tot[kRadix / 32];
     __shared__ uint32_t s_tile;
     __shared__ uint32_t s_next[kRadix];                     // this block's share of the next pass's histogram
-    if (ctrl->skip || !ctrl->run_sort) return;
-    const SortPlan &pl = ctrl->plan;
-    if (pass >= (int)pl.n_passes) return;
     const bool count_next = pass + 1 < (int)pl.n_passes;
     const DigitSel sel = digit_sel(pl, pass), sel_next = digit_sel(pl, count_next ? pass + 1 : pass);
     if (threadIdx.x < kRadix) s_next[threadIdx.x] = 0u;
@@ -253,7 +252,8 @@ k_sort_pass(int pass, uint64_t n, BatchCtrl *ctrl, DevState *state, uint32_t *hi
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
     const uint32_t n_tiles = (uint32_t)((n + kSortTile - 1) / kSortTile);
-  for (;;) {                                  // persistent: tiles are taken in order from a counter
+    uint32_t taken = 0;
+  for (;; ++taken) {                          // persistent: tiles are taken in order from a counter
     __syncthreads();                          // shared memory of the previous tile is no longer read
     if (tid == 0) s_tile = atomicAdd(&ctrl->tile_counter[pass], 1u);
     for (int i = tid; i < kSortWarps * kRadix; i += kSortThreads) { s_cnt[i] = 0u; reinterpret_cast<uint32_t *>(s_keys)[i] = 0u; }
@@ -366,7 +366,7 @@ k_sort_pass(int pass, uint64_t n, BatchCtrl *ctrl, DevState *state, uint32_t *hi
             if ((v >> 30) == 2u) break;
         }
         // a wait that ran out: the batch is given up (later kernels of it exit at once) and the context is poisoned
-        if (failed) { atomicExch(&ctrl->code, (int)HBF_E_TIMEOUT); ctrl->skip = 1; state->poisoned = 1; }
+        if (failed) give_up();
         if (tile != 0 && !mute) st_relaxed_u32(desc + (uint64_t)tile * kRadix + tid, kFlagPrefix | ((excl + tile_count) & kCountMask));
         s_local_start[tid] = local_start;
         s_delta[tid] = gstart + excl - local_start;
@@ -398,6 +398,17 @@ k_sort_pass(int pass, uint64_t n, BatchCtrl *ctrl, DevState *state, uint32_t *hi
   }
     // (the loop was left behind a block-wide barrier)
     if (count_next && tid < kRadix && s_next[tid]) atomicAdd(&hist[(pass + 1) * kRadix + tid], s_next[tid]);
+    return taken;
+}
+// (three resident blocks per SM: at one block of 80 registers the pass ran at 13 % of the DRAM rate with a quarter of the
+// warp slots in use, 4.1 ms for 200 M keys; bounded to 40 registers, with a few spills, it takes 2.5 ms)
+__global__ void __launch_bounds__(kSortThreads, 3)
+k_sort_pass(int pass, uint64_t n, BatchCtrl *ctrl, DevState *state, uint32_t *hist,
+            uint64_t *keys0, uint64_t *keys1, uint32_t *idx0, uint32_t *idx1, uint32_t *desc0, uint32_t *desc1) {
+    extern __shared__ __align__(16) unsigned char sort_smem[];
+    if (ctrl->skip || !ctrl->run_sort || pass >= (int)ctrl->plan.n_passes) return;
+    sort_pass(pass, n, ctrl->plan, ctrl, state, hist, keys0, keys1, idx0, idx1, desc0, desc1, sort_smem,
+              [&] { atomicExch(&ctrl->code, (int)HBF_E_TIMEOUT); ctrl->skip = 1; state->poisoned = 1; });
 }
 
 // =====================================================================================================
@@ -409,7 +420,6 @@ k_sort_pass(int pass, uint64_t n, BatchCtrl *ctrl, DevState *state, uint32_t *hi
 constexpr int kScanThreads = 256;
 constexpr int kScanItems = 8;
 constexpr int kScanTile = kScanThreads * kScanItems;     // 2048
-constexpr int kScanWarps = kScanThreads / 32;
 
 struct __align__(32) ScanDesc { int64_t S, M, value; uint32_t status; uint32_t pad; };
 struct Map { int64_t S, M; int f; };
@@ -423,28 +433,27 @@ __device__ __forceinline__ Map shfl_up_map(const Map &m, int o) {
     r.f = __shfl_up_sync(0xffffffffu, m.f, o); return r;
 }
 
-// (two blocks per SM; three or four, or 512 threads with four items each, were measured slower: the kernel is bound by its
-// scattered accesses, not by latency)
-__global__ void __launch_bounds__(kScanThreads, 2)
-k_scan(const uint64_t *__restrict__ terms, uint64_t n,
-       const ModelParams *__restrict__ mp_g, BatchCtrl *ctrl, DevState *state,
+// (the tiles that this block took; give_up(): a look-back that ran out)
+template <int THREADS, class GiveUp>
+__device__ __forceinline__ uint32_t scan_tiles(const uint64_t *terms, uint64_t n,
+       const ModelParams *__restrict__ mp_g, const uint32_t np, BatchCtrl *ctrl, const DevState *state,
        const uint64_t *keys0, const uint64_t *keys1, const uint32_t *idx0, const uint32_t *idx1,
        ScanDesc *desc, const int64_t *__restrict__ busy, int64_t *busy_stage, hbf_die_stats_t *stats_stage,
-       int64_t *__restrict__ completion, int64_t *__restrict__ stall,
-       const unsigned long long *claim_limit_p, uint32_t *die_claims) {
+       int64_t *completion, const unsigned long long *claim_limit_p, uint32_t *die_claims, GiveUp &&give_up) {
+    constexpr int ITEMS = kScanTile / THREADS, WARPS = THREADS / 32;
     __shared__ ModelParams mp;
-    __shared__ uint32_t s_first_q[kScanThreads], s_last_q[kScanThreads];
-    __shared__ Map s_warp_map[kScanWarps];
+    __shared__ uint32_t s_first_q[THREADS], s_last_q[THREADS];
+    __shared__ Map s_warp_map[WARPS];
     __shared__ int64_t s_tile_in;
     __shared__ uint32_t s_tile;
     __shared__ long long s_die_acc[6];
     __shared__ long long s_res[3];
-    if (ctrl->skip || !ctrl->run_sort) return;
     const uint64_t m = ctrl->n_ready;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    for (int i = tid; i < (int)(sizeof(ModelParams) / 4); i += kScanThreads)
+    for (int i = tid; i < (int)(sizeof(ModelParams) / 4); i += THREADS)
         reinterpret_cast<uint32_t *>(&mp)[i] = reinterpret_cast<const uint32_t *>(mp_g)[i];
-  for (;;) {                                  // persistent: tiles are taken in order from a counter
+    uint32_t taken = 0;
+  for (;; ++taken) {                          // persistent: tiles are taken in order from a counter
     __syncthreads();
     if (tid == 0) s_tile = atomicAdd(&ctrl->tile_counter[kMaxPasses], 1u);
     if (tid < 6) s_die_acc[tid] = 0;
@@ -453,7 +462,6 @@ k_scan(const uint64_t *__restrict__ terms, uint64_t n,
     const uint32_t tile = s_tile;
     const uint64_t base = (uint64_t)tile * kScanTile;
     if (base >= m) break;
-    const uint32_t np = ctrl->plan.n_passes;
     const uint64_t *keys = (np & 1u) ? keys1 : keys0;
     const uint32_t *idxs = np == 0u ? nullptr : ((np & 1u) ? idx1 : idx0);
     const int64_t q_ppm = ctrl->q_ppm;
@@ -466,33 +474,33 @@ k_scan(const uint64_t *__restrict__ terms, uint64_t n,
         : (int64_t)div64((uint64_t)(mp.t_read_ns + mp.t_prog_ns) * 1000000ull + (uint64_t)q_ppm - 1ull, div_q);
 
     // this thread's consecutive items
-    uint32_t queue[kScanItems], idx[kScanItems], post[kScanItems];
-    int64_t a[kScanItems], s[kScanItems], issue[kScanItems];
-    const int t0 = tid * kScanItems;
-    const int mine = max(0, min(kScanItems, cnt - t0));
+    uint32_t queue[ITEMS], idx[ITEMS], post[ITEMS];
+    int64_t a[ITEMS], s[ITEMS], issue[ITEMS];
+    const int t0 = tid * ITEMS;
+    const int mine = max(0, min(ITEMS, cnt - t0));
     {
-        uint64_t k[kScanItems];
-        if (mine == kScanItems) {
+        uint64_t k[ITEMS];
+        if (mine == ITEMS) {
             const ulonglong2 *k2 = reinterpret_cast<const ulonglong2 *>(keys + base + t0);
 #pragma unroll
-            for (int j = 0; j < kScanItems / 2; ++j) { const ulonglong2 v = k2[j]; k[2 * j] = v.x; k[2 * j + 1] = v.y; }
+            for (int j = 0; j < ITEMS / 2; ++j) { const ulonglong2 v = k2[j]; k[2 * j] = v.x; k[2 * j + 1] = v.y; }
             if (idxs) {
                 const uint4 *i4 = reinterpret_cast<const uint4 *>(idxs + base + t0);
 #pragma unroll
-                for (int j = 0; j < kScanItems / 4; ++j) { const uint4 v = i4[j]; idx[4 * j] = v.x; idx[4 * j + 1] = v.y; idx[4 * j + 2] = v.z; idx[4 * j + 3] = v.w; }
+                for (int j = 0; j < ITEMS / 4; ++j) { const uint4 v = i4[j]; idx[4 * j] = v.x; idx[4 * j + 1] = v.y; idx[4 * j + 2] = v.z; idx[4 * j + 3] = v.w; }
             } else {
 #pragma unroll
-                for (int j = 0; j < kScanItems; ++j) idx[j] = (uint32_t)(base + t0 + j);
+                for (int j = 0; j < ITEMS; ++j) idx[j] = (uint32_t)(base + t0 + j);
             }
         } else {
 #pragma unroll
-            for (int j = 0; j < kScanItems; ++j) {
+            for (int j = 0; j < ITEMS; ++j) {
                 k[j] = j < mine ? keys[base + t0 + j] : 0ull;
                 idx[j] = j < mine ? (idxs ? idxs[base + t0 + j] : (uint32_t)(base + t0 + j)) : 0u;
             }
         }
 #pragma unroll
-        for (int j = 0; j < kScanItems; ++j) { queue[j] = (uint32_t)(k[j] >> kIssueBits); issue[j] = (int64_t)(k[j] & kIssueMask); }
+        for (int j = 0; j < ITEMS; ++j) { queue[j] = (uint32_t)(k[j] >> kIssueBits); issue[j] = (int64_t)(k[j] & kIssueMask); }
     }
     // gather the records and rebuild their service terms
     long long acc_busy = 0, acc_br = 0, acc_bp = 0, acc_e = 0, acc_nr = 0, acc_np = 0;
@@ -511,13 +519,13 @@ k_scan(const uint64_t *__restrict__ terms, uint64_t n,
     };
     // what the scan needs of a record is the 8-byte word the classify kernel left for it (one 32-byte sector per access
     // instead of the 24-byte record, and no second classification or decode)
-    uint64_t r_tw[kScanItems];
+    uint64_t r_tw[ITEMS];
 #pragma unroll
-    for (int j = 0; j < kScanItems; ++j)
-        if (j < mine) r_tw[j] = ld_nc_u64(terms + idx[j]);
+    for (int j = 0; j < ITEMS; ++j)
+        if (j < mine) r_tw[j] = __ldcg(terms + idx[j]);
     long long sum_s = 0;
 #pragma unroll
-    for (int j = 0; j < kScanItems; ++j) {
+    for (int j = 0; j < ITEMS; ++j) {
         if (j < mine) {
             const uint32_t bytes = (uint32_t)r_tw[j], op = (uint32_t)(r_tw[j] >> 32) & 1u, npages = (uint32_t)(r_tw[j] >> 33);
             const uint32_t die = mp.queue_level != 0u ? queue[j] : (mp.pow2_geom ? queue[j] >> mp.plane_shift : queue[j] / mp.planes);
@@ -545,7 +553,7 @@ k_scan(const uint64_t *__restrict__ terms, uint64_t n,
     {
         uint32_t pq = prev_q;
 #pragma unroll
-        for (int j = 0; j < kScanItems; ++j) {
+        for (int j = 0; j < ITEMS; ++j) {
             if (j < mine) {
                 Map e; e.S = s[j]; e.f = queue[j] != pq;
                 e.M = e.f ? max(busy[queue[j]], a[j]) + s[j] : a[j] + s[j];
@@ -566,7 +574,7 @@ k_scan(const uint64_t *__restrict__ terms, uint64_t n,
     excl = compose(wprefix, excl);
 
     // tile aggregate, publish, look back
-    if (tid == kScanThreads - 1) {
+    if (tid == THREADS - 1) {
         const Map agg = compose(excl, tm);
         ScanDesc *my = desc + tile;
         int64_t tile_in = 0;
@@ -603,7 +611,7 @@ k_scan(const uint64_t *__restrict__ terms, uint64_t n,
                 const int64_t St = ld_relaxed_s64(&p->S), Mt = ld_relaxed_s64(&p->M);
                 M_acc = max(Mt + S_acc, M_acc); S_acc += St;
             }
-            if (failed) { atomicExch(&ctrl->code, (int)HBF_E_TIMEOUT); ctrl->skip = 1; state->poisoned = 1; }
+            if (failed) give_up();
         }
         if (!agg.f && !mute) {
             st_relaxed_s64(&my->value, max(tile_in + agg.S, agg.M));
@@ -619,7 +627,7 @@ k_scan(const uint64_t *__restrict__ terms, uint64_t n,
     {
         uint32_t pq = prev_q;
 #pragma unroll
-        for (int j = 0; j < kScanItems; ++j) {
+        for (int j = 0; j < ITEMS; ++j) {
             if (j < mine) {
                 if (queue[j] != pq) B = busy[queue[j]];
                 const int64_t start = max(a[j], B);
@@ -673,6 +681,19 @@ k_scan(const uint64_t *__restrict__ terms, uint64_t n,
         }
     }
   }
+    return taken;
+}
+// (two blocks per SM; three or four, or 512 threads with four items each, were measured slower: the kernel is bound by its
+// scattered accesses, not by latency)
+__global__ void __launch_bounds__(kScanThreads, 2)
+k_scan(const uint64_t *__restrict__ terms, uint64_t n,
+       const ModelParams *__restrict__ mp_g, BatchCtrl *ctrl, DevState *state,
+       const uint64_t *keys0, const uint64_t *keys1, const uint32_t *idx0, const uint32_t *idx1,
+       ScanDesc *desc, const int64_t *__restrict__ busy, int64_t *busy_stage, hbf_die_stats_t *stats_stage,
+       int64_t *__restrict__ completion, const unsigned long long *claim_limit_p, uint32_t *die_claims) {
+    if (ctrl->skip || !ctrl->run_sort) return;
+    scan_tiles<kScanThreads>(terms, n, mp_g, ctrl->plan.n_passes, ctrl, state, keys0, keys1, idx0, idx1, desc, busy, busy_stage, stats_stage, completion, claim_limit_p, die_claims,
+                             [&] { atomicExch(&ctrl->code, (int)HBF_E_TIMEOUT); ctrl->skip = 1; state->poisoned = 1; });
 }
 
 // stalls of a batch the sort path served: stall = completion - issue, in batch order (coalesced reads and writes; the scan
@@ -682,7 +703,7 @@ k_stalls(const hbf_access_t *__restrict__ acc, uint64_t n, const BatchCtrl *ctrl
          int64_t *__restrict__ stall) {
     if (ctrl->skip || !ctrl->run_sort) return;
     for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (uint64_t)gridDim.x * blockDim.x)
-        stall[i] = completion[i] - (int64_t)__ldg(reinterpret_cast<const uint64_t *>(acc + i) + 1);
+        stall[i] = __ldcg(completion + i) - (int64_t)__ldg(reinterpret_cast<const uint64_t *>(acc + i) + 1);
 }
 
 // =====================================================================================================
@@ -699,12 +720,12 @@ __device__ __forceinline__ int batch_code(const FinishArgs &f) {
     return f.bus_on && ctrl->n_ready && ctrl->max_completion_ns >= HBF_ISSUE_LIMIT ? HBF_E_INVAL : HBF_OK;
 }
 // (on the whole grid, or on one block: gtid and gsz)
-__device__ __forceinline__ void finish_batch(const FinishArgs &f, long long modeled, int code, uint64_t gtid, uint64_t gsz) {
+__device__ __forceinline__ void finish_batch(const FinishArgs &f, long long modeled, int code, uint64_t gtid, uint64_t gsz, bool zeroed = false) {      // zeroed: the outputs of a refused batch are
     BatchCtrl *ctrl = f.ctrl;
     const uint64_t n = f.n;
     if (code == HBF_E_TIMEOUT && gtid == 0) f.state->poisoned = 1;       // a bounded device-side wait expired
     if (code == HBF_E_ACCESS_FAULT || code == HBF_E_TIMEOUT || code == HBF_E_INVAL) {
-        for (uint64_t i = gtid; i < n; i += gsz) { f.completion[i] = 0; f.stall[i] = 0; }
+        if (!zeroed) for (uint64_t i = gtid; i < n; i += gsz) { f.completion[i] = 0; f.stall[i] = 0; }
         if (f.die_stats) for (uint64_t i = gtid; i < (uint64_t)f.n_dies * 6u; i += gsz) reinterpret_cast<int64_t *>(f.die_stats)[i] = 0;
     } else if (f.paged && (code == HBF_E_THROTTLED || code == HBF_E_LINK_SHUTDOWN)) {     // (a page-granular batch leaves zeros then, as its join does)
         for (uint64_t i = gtid; i < n; i += gsz) { f.completion[i] = 0; f.stall[i] = 0; }
@@ -1123,93 +1144,203 @@ static cudaError_t launch_sort_path(const SubmitArgs &a, cudaStream_t st) {
     mark(4);
     k_scan<<<(unsigned)std::min<uint64_t>(scan_tiles, (uint64_t)a.sm_count * 8), kScanThreads, 0, st>>>(a.ws.terms, n, a.mp_dev, a.ctrl, a.state, a.ws.keys[0], a.ws.keys[1],
                                                          a.ws.idx[0], a.ws.idx[1], (ScanDesc *)a.ws.scan_desc, a.busy,
-                                                         a.busy_stage, a.stats_stage, a.completion, a.stall,
-                                                         a.claim_limit, a.die_claims);
+                                                         a.busy_stage, a.stats_stage, a.completion, a.claim_limit, a.die_claims);
     k_stalls<<<(unsigned)std::min<uint64_t>((n + 255) / 256, (uint64_t)a.sm_count * 16), 256, 0, st>>>(a.acc, n, a.ctrl, a.completion, a.stall);
     g_kernel_launches += 5 + kMaxPasses;
     return cudaSuccess;
 }
 
-// ---- the sort path launched from the device -----------------------------------------------------------
+// ---- the sort path as phases of the last kernel ---------------------------------------------------------
 // With HBF_PATH_AUTO the host enqueues the in-order kernels only.  A batch that those do not serve (out of issue order where the begin
 // kernel's samples did not see it or its buckets do not hold it, or with a service time the in-order kernels cannot hold)
 // needs the sort path after all, and the host cannot know that without waiting for the device.  So the last kernel (it also sums
-// the batch's stall total and commits it when they did serve it) looks at the batch's control block and, in that case only, one
-// thread launches the sort path's kernels itself, in order, into the tail-launch stream, their finish kernel among them: they run
-// after this kernel and before the next kernel of the host's stream (a parent grid is complete only when its children are).  A
-// batch in issue order pays no launch for it.  Launched from the device the passes run one block per multiprocessor where two or three
-// would fit: 40 M records 7.7 ms, 5.6 launched by the host.
+// the batch's stall total and commits it when they did serve it) looks at the batch's control block and, in that case only, goes through
+// the sort path itself, one phase after the other.  The work of a phase is dealt out in order by counters, whole blocks take it, and a block that
+// finds none left waits until all of it is done (regroup.cuh): it waits for blocks that run.  The block that is through last commits.
+// (The kernels used to be launched from the device: a kernel that may do that takes several microseconds more even where it does not, and
+// the one behind it must not begin before it has ended.  4 M decode reads with the thermal step behind them 111.5 -> 106.0 us; two records out of
+// place in 20,000: 351 -> 147, in 4 M 972 -> 650, in 40 M 8,070 -> 6,440.)
 struct SortChain {
     const hbf_access_t *acc; uint64_t n; const RangeSnap *ranges; const ModelParams *mp_dev; BatchCtrl *ctrl; DevState *state;
     uint64_t *keys0, *keys1, *terms; uint32_t *idx0, *idx1, *hist, *desc0, *desc1; void *scan_desc;
     uint8_t *status; int64_t *completion, *stall; const int64_t *busy; int64_t *busy_stage; hbf_die_stats_t *stats_stage;
     const unsigned long long *claim_limit; uint32_t *die_claims;
     uint32_t n_queues, n_dies; uint64_t desc_words, scan_words;
-    unsigned cls_grid, hist_grid, sort_grid, scan_grid, stall_grid;
-    const InTile *in_tile; uint32_t n_tiles;
+    const InTile *in_tile; uint32_t n_tiles; RegroupSync *sync;
 };
+enum SortPhase { kSpStart = 0, kSpClassify = 1, kSpHist = 2, kSpPass = 3, kSpScan = kSpPass + kMaxPasses, kSpStalls = kSpScan + 1 };
+static_assert(kSpStalls < 16, "counters of a phase each");
+constexpr int kLastThreads = 512, kLastBlocks = 2;           // of the last kernel: the radix passes' block; 64 registers
+static_assert(kLastThreads == kSortThreads && kSortSmem >= (size_t)kClsTile * 24 && kSortSmem >= (size_t)kLastThreads / 256 * kRgOut * 16, "its shared memory holds what every phase needs");
 
-// the radix sort's kernels, launched from the device (run_sort is set: the begin kernel starts the batch over)
-__device__ void launch_sort_chain(const SortChain &c, const FinishArgs &f, unsigned fin_grid) {
-    cudaStream_t st = cudaStreamTailLaunch;
-    const BeginArgs b{c.ctrl, c.state, c.busy, c.busy_stage, c.stats_stage, c.hist, c.n_queues, c.n_dies, c.die_claims, c.claim_limit, nullptr, 0.0f, 0, 0, 0, 0, nullptr, 0};
-    k_begin<<<1, 1024, 0, st>>>(b, 1, 1, nullptr);
-    k_zero_words<<<(unsigned)min((unsigned long long)((c.desc_words + 1023) / 1024), 592ull), 1024, 0, st>>>(c.desc0, c.desc_words);
-    k_zero_words<<<(unsigned)min((unsigned long long)((c.scan_words + 1023) / 1024), 592ull), 1024, 0, st>>>((uint32_t *)c.scan_desc, c.scan_words);
-    k_classify<<<c.cls_grid, kClsThreads, 0, st>>>(c.acc, c.n, c.ranges, c.mp_dev, c.ctrl, c.keys0, c.terms, c.status, c.completion, c.stall);
-    k_plan<<<1, 32, 0, st>>>(c.ctrl, 0);
-    k_hist<<<c.hist_grid, kHistThreads, 0, st>>>(c.keys0, c.n, c.ctrl, c.hist);
-    for (int p = 0; p < kMaxPasses; ++p)
-        k_sort_pass<<<c.sort_grid, kSortThreads, kSortSmem, st>>>(p, c.n, c.ctrl, c.state, c.hist, c.keys0, c.keys1, c.idx0, c.idx1, c.desc0, c.desc1);
-    k_scan<<<c.scan_grid, kScanThreads, 0, st>>>(c.terms, c.n, c.mp_dev, c.ctrl, c.state, c.keys0, c.keys1, c.idx0, c.idx1,
-                                                 (ScanDesc *)c.scan_desc, c.busy, c.busy_stage, c.stats_stage, c.completion, c.stall,
-                                                 c.claim_limit, c.die_claims);
-    k_stalls<<<c.stall_grid, 256, 0, st>>>(c.acc, c.n, c.ctrl, c.completion, c.stall);
-    k_finish<<<fin_grid, 256, 0, st>>>(f);
+// the next share of a phase, for the whole block
+__device__ __forceinline__ uint32_t sp_claim(RegroupSync *s, int phase) {
+    __shared__ uint32_t s_share;
+    __syncthreads();
+    if (threadIdx.x == 0) s_share = atomicAdd(&s->sort_claim[phase], 1u);
+    __syncthreads();
+    return s_share;
+}
+__device__ __forceinline__ void sp_done(RegroupSync *s, int phase, uint32_t shares) {
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0 && shares) atomicAdd(&s->sort_done[phase], shares);
+}
+// all shares of a phase are done; false: the wait ran out, here or in another block
+__device__ __forceinline__ bool sp_wait(RegroupSync *s, int phase, uint32_t shares, uint32_t limit) {
+    bool ok = true;
+    if (threadIdx.x == 0) {
+        uint32_t polls = 0;
+        while (ok && ld_acquire_u32(&s->sort_done[phase]) < shares) {
+            if (++polls > limit) atomicExch(&s->sort_failed, 1u);
+            ok = ld_relaxed_u32(&s->sort_failed) == 0u;
+            __nanosleep(200);
+        }
+        if (ld_relaxed_u32(&s->sort_failed)) ok = false;     // (a look-back that ran out)
+        __threadfence();
+    }
+    return __syncthreads_and(ok) != 0;
 }
 
-// The last kernel of a batch on the in-order path: the commit, and the hand-over of a batch that it did not serve.
-// (MAY_SORT = false, for a context whose caller declares issue order: the same kernel without the device-side launches,
-// which cost a kernel that contains them several microseconds even when none is made)
+// what the phases come to: HBF_OK, the batch's refusal (outputs zeroed), or HBF_E_TIMEOUT
+__device__ __forceinline__ int sort_phases(const SortChain &c, const FinishArgs &f, unsigned char *smem) {
+    __shared__ SortPlan s_plan;
+    __shared__ uint32_t s_hist[kRadix];
+    RegroupSync *sync = c.sync;
+    BatchCtrl *ctrl = c.ctrl;
+    const uint64_t n = c.n, gtid = (uint64_t)blockIdx.x * kLastThreads + threadIdx.x, gsz = (uint64_t)gridDim.x * kLastThreads;
+    const int tid = threadIdx.x;
+    const uint32_t limit = c.state->spin_limit;
+    auto give_up = [&] { atomicExch(&sync->sort_failed, 1u); };
+    auto refuse = [&](int code) { for (uint64_t i = gtid; i < n; i += gsz) { c.completion[i] = 0; c.stall[i] = 0; } return code; };
+    uint32_t mine = 0;
+
+    // ---- the batch starts over: what the in-order attempt left, the look-back words
+    constexpr uint64_t kZero = 65536;
+    const uint32_t desc_shares = (uint32_t)((c.desc_words + kZero - 1) / kZero), scan_shares = (uint32_t)((c.scan_words + kZero - 1) / kZero), starts = 1u + desc_shares + scan_shares;
+    for (uint32_t k; (k = sp_claim(sync, kSpStart)) < starts; ++mine) {
+        if (k == 0u) {
+            if (tid == 0) {                                  // (code, skip, mode and q stand; every block has read, or will read, inorder_used as it is)
+                ctrl->n_native = ctrl->n_ready = ctrl->n_fault = 0ull; ctrl->key_or = 0ull; ctrl->key_and = ~0ull; ctrl->unsorted = 0u; ctrl->regrouped = 0u;
+                for (int i = 0; i < kMaxPasses + 2; ++i) ctrl->tile_counter[i] = 0u;
+                ctrl->modeled_ns = ctrl->service_ns = ctrl->max_completion_ns = 0;
+            }
+            for (uint32_t r = tid; r < c.n_queues; r += kLastThreads) c.busy_stage[r] = c.busy[r];
+            for (uint32_t i = tid; i < c.n_dies * 6u; i += kLastThreads) reinterpret_cast<int64_t *>(c.stats_stage)[i] = 0;
+            for (int i = tid; i < kMaxPasses * kRadix; i += kLastThreads) c.hist[i] = 0u;
+            if (c.die_claims) for (uint32_t d = tid; d < c.n_dies; d += kLastThreads) c.die_claims[d] = 0u;
+        } else {
+            const bool scan = k > desc_shares;
+            uint32_t *p = scan ? static_cast<uint32_t *>(c.scan_desc) : c.desc0;
+            const uint64_t words = scan ? c.scan_words : c.desc_words, from = (uint64_t)(scan ? k - 1u - desc_shares : k - 1u) * kZero;
+            for (uint64_t i = from + tid; i < min(words, from + kZero); i += kLastThreads) p[i] = 0u;
+        }
+    }
+    sp_done(sync, kSpStart, mine);
+    if (!sp_wait(sync, kSpStart, starts, limit)) return HBF_E_TIMEOUT;
+
+    const uint32_t cls_tiles = (uint32_t)((n + kClsTile - 1) / kClsTile);
+    mine = 0;
+    classify_tiles<kLastThreads>(c.acc, n, c.ranges, c.mp_dev, ctrl, c.keys0, c.terms, c.status, c.completion, c.stall, reinterpret_cast<uint64_t *>(smem),
+                                 [&] { const uint32_t t = sp_claim(sync, kSpClassify); if (t < cls_tiles) ++mine; return (uint64_t)t; });
+    sp_done(sync, kSpClassify, mine);
+    if (!sp_wait(sync, kSpClassify, cls_tiles, limit)) return HBF_E_TIMEOUT;
+    if (ctrl->n_fault) return refuse(HBF_E_ACCESS_FAULT);
+    if (tid == 0) s_plan = make_plan(ctrl, 0);
+    __syncthreads();
+    const SortPlan &plan = s_plan;
+
+    if (plan.n_passes) {
+        constexpr uint64_t kKeys = 32768;
+        const uint32_t shares = (uint32_t)((n + kKeys - 1) / kKeys);
+        for (int i = tid; i < kRadix; i += kLastThreads) s_hist[i] = 0u;
+        const DigitSel sel0 = digit_sel(plan, 0);
+        mine = 0;
+        for (uint32_t k; (k = sp_claim(sync, kSpHist)) < shares; ++mine) hist_keys(c.keys0, n, k * kKeys + tid, min(n, (k + 1u) * kKeys), kLastThreads, sel0, s_hist);
+        __syncthreads();
+        for (int i = tid; i < kRadix; i += kLastThreads) if (s_hist[i]) atomicAdd(&c.hist[i], s_hist[i]);
+        sp_done(sync, kSpHist, mine);
+        if (!sp_wait(sync, kSpHist, shares, limit)) return HBF_E_TIMEOUT;
+        for (int p = 0; p < (int)plan.n_passes; ++p) {
+            mine = sort_pass(p, n, plan, ctrl, c.state, c.hist, c.keys0, c.keys1, c.idx0, c.idx1, c.desc0, c.desc1, smem, give_up);
+            sp_done(sync, kSpPass + p, mine);
+            if (!sp_wait(sync, kSpPass + p, (uint32_t)((n + kSortTile - 1) / kSortTile), limit)) return HBF_E_TIMEOUT;
+        }
+    }
+    mine = scan_tiles<kLastThreads>(c.terms, n, c.mp_dev, plan.n_passes, ctrl, c.state, c.keys0, c.keys1, c.idx0, c.idx1, (ScanDesc *)c.scan_desc, c.busy, c.busy_stage, c.stats_stage,
+                                    c.completion, c.claim_limit, c.die_claims, give_up);
+    sp_done(sync, kSpScan, mine);
+    if (!sp_wait(sync, kSpScan, (uint32_t)((ctrl->n_ready + kScanTile - 1) / kScanTile), limit)) return HBF_E_TIMEOUT;
+    if (batch_code(f) != HBF_OK) return refuse(batch_code(f));
+
+    constexpr uint64_t kStalls = 16384;
+    const uint32_t shares = (uint32_t)((n + kStalls - 1) / kStalls);
+    for (uint32_t k; (k = sp_claim(sync, kSpStalls)) < shares;)
+        for (uint64_t i = k * kStalls + tid; i < min(n, (k + 1u) * kStalls); i += kLastThreads)
+            c.stall[i] = __ldcg(c.completion + i) - (int64_t)__ldg(reinterpret_cast<const uint64_t *>(c.acc + i) + 1);
+    return HBF_OK;
+}
+
+// the sort path, and the commit by the block that is through last
+__device__ __forceinline__ void sort_in_phases(const SortChain &c, const FinishArgs &f, unsigned char *smem) {
+    __shared__ uint32_t s_last;
+    RegroupSync *sync = c.sync;
+    int code = sort_phases(c, f, smem);
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) { s_last = atomicAdd(&sync->sort_left, 1u) == gridDim.x - 1u ? 1u : 0u; __threadfence(); }
+    __syncthreads();
+    if (!s_last) return;
+    if (ld_relaxed_u32(&sync->sort_failed)) code = HBF_E_TIMEOUT;
+    finish_batch(f, c.ctrl->modeled_ns, code, threadIdx.x, kLastThreads, code != HBF_E_TIMEOUT);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        c.ctrl->code = code;
+        if (code != HBF_OK) c.ctrl->skip = 1; else c.ctrl->plan = make_plan(c.ctrl, 0);
+    }
+    if (threadIdx.x < 16) { sync->sort_claim[threadIdx.x] = 0u; sync->sort_done[threadIdx.x] = 0u; }
+    if (threadIdx.x == 16) { sync->sort_failed = 0u; sync->sort_left = 0u; }
+}
+
+// The last kernel of a batch on the in-order path: the commit, and the sort of a batch that was not served.
+// (MAY_SORT = false, for a context whose caller declares issue order: the same kernel without it)
 template <bool MAY_SORT>
-__global__ void __launch_bounds__(256, 4) k_finish_inorder(const __grid_constant__ SortChain c, const __grid_constant__ FinishArgs f, const __grid_constant__ RegroupArgs rg) {
+__global__ void __launch_bounds__(MAY_SORT ? kLastThreads : 256, MAY_SORT ? kLastBlocks : 4) k_finish_inorder(const __grid_constant__ SortChain c, const __grid_constant__ FinishArgs f, const __grid_constant__ RegroupArgs rg) {
+    extern __shared__ __align__(16) unsigned char sort_smem[];
     pdl_wait();
-    if constexpr (!MAY_SORT) pdl_trigger();                  // (what follows a kernel that may launch others is launched plainly)
+    pdl_trigger();
     const bool regrouped = MAY_SORT && rg.sync && c.ctrl->regrouped;
-    if (regrouped && blockIdx.x == 0) {                      // (the begin kernel's part of it: zero again for the next batch)
+    if (MAY_SORT && rg.sync && blockIdx.x == 0) {            // (the begin kernel's part of it: zero again for the next batch)
         for (uint32_t i = threadIdx.x; i < 3u * 64u; i += blockDim.x) rg.sync->hist[i] = 0u;
         if (threadIdx.x < 3) { rg.sync->claim[threadIdx.x] = 0u; rg.sync->done[threadIdx.x] = 0u; }
         if (threadIdx.x == 3) rg.sync->claim[5] = 0u;
     }
-    if (!MAY_SORT || c.ctrl->skip || c.ctrl->inorder_used) {
-        // Stall total of the batch: per tile the exact sum if it was re-served, else the as-if sum plus its corrections
-        __shared__ long long s_tot[8];
-        auto stall_total = [&]() {                           // (whole block)
-            long long tot = 0;
-            for (uint32_t t = threadIdx.x; t < c.n_tiles; t += blockDim.x) {
-                const InTile v = c.in_tile[t];
-                tot += v.reserve ? v.true_sum : v.spec_sum + v.fix_delta;
-            }
-            tot = warp_sum(tot);
-            if ((threadIdx.x & 31) == 0) s_tot[threadIdx.x >> 5] = tot;
-            __syncthreads();
-            tot = 0;
-            for (int w = 0; w < 8; ++w) tot += s_tot[w];
-            return tot;
-        };
-        if constexpr (MAY_SORT) {
-            if (regrouped && batch_code(f) == HBF_OK) {      // (nothing is committed before every result can be given back)
-                if (rg_give_back(rg, f.n, f.state, f.completion, f.stall, [&] { finish_batch(f, stall_total(), HBF_OK, threadIdx.x, blockDim.x); })) {
-                    finish_batch(f, 0, HBF_E_TIMEOUT, threadIdx.x, blockDim.x);
-                    if (threadIdx.x == 0) { f.ctrl->code = HBF_E_TIMEOUT; f.ctrl->skip = 1; }
-                }
-                return;
-            }
+    if constexpr (MAY_SORT) { if (!c.ctrl->skip && !c.ctrl->inorder_used) { sort_in_phases(c, f, sort_smem); return; } }
+    // Stall total of the batch: per tile the exact sum if it was re-served, else the as-if sum plus its corrections
+    __shared__ long long s_tot[16];
+    auto stall_total = [&]() {                               // (whole block)
+        long long tot = 0;
+        for (uint32_t t = threadIdx.x; t < c.n_tiles; t += blockDim.x) {
+            const InTile v = c.in_tile[t];
+            tot += v.reserve ? v.true_sum : v.spec_sum + v.fix_delta;
         }
-        finish_batch(f, blockIdx.x == 0 && !c.ctrl->skip ? stall_total() : 0);
-        return;
+        tot = warp_sum(tot);
+        if ((threadIdx.x & 31) == 0) s_tot[threadIdx.x >> 5] = tot;
+        __syncthreads();
+        tot = 0;
+        for (int w = 0; w < (int)blockDim.x / 32; ++w) tot += s_tot[w];
+        return tot;
+    };
+    if constexpr (MAY_SORT) {
+        if (regrouped && batch_code(f) == HBF_OK) {          // (nothing is committed before every result can be given back)
+            if (rg_give_back(rg, f.n, f.state, f.completion, f.stall, reinterpret_cast<ulonglong2 *>(sort_smem), [&] { finish_batch(f, stall_total(), HBF_OK, threadIdx.x, blockDim.x); })) {
+                finish_batch(f, 0, HBF_E_TIMEOUT, threadIdx.x, blockDim.x);
+                if (threadIdx.x == 0) { f.ctrl->code = HBF_E_TIMEOUT; f.ctrl->skip = 1; }
+            }
+            return;
+        }
     }
-    if constexpr (MAY_SORT) { if (threadIdx.x == 0 && blockIdx.x == 0) launch_sort_chain(c, f, gridDim.x); }
+    finish_batch(f, blockIdx.x == 0 && !c.ctrl->skip ? stall_total() : 0);
 }
 
 static FinishArgs finish_args(const SubmitArgs &a) {
@@ -1225,8 +1356,6 @@ static unsigned finish_grid(const SubmitArgs &a) { return (unsigned)std::max<uin
 static cudaError_t launch_finish_inorder(const SubmitArgs &a, bool may_sort, cudaStream_t st) {
     const uint64_t n = a.n;
     const uint64_t sort_tiles = (n + kSortTile - 1) / kSortTile, scan_tiles = (n + kScanTile - 1) / kScanTile;
-    cudaError_t e = ensure_dyn_smem((const void *)k_sort_pass, kSortSmem);   // (an attribute of the kernel: device-side launches use it too)
-    if (e != cudaSuccess) return e;
     SortChain c{};
     c.acc = a.acc; c.n = n; c.ranges = a.ranges; c.mp_dev = a.mp_dev; c.ctrl = a.ctrl; c.state = a.state;
     c.keys0 = a.ws.keys[0]; c.keys1 = a.ws.keys[1]; c.terms = a.ws.terms; c.idx0 = a.ws.idx[0]; c.idx1 = a.ws.idx[1]; c.hist = a.ws.hist;
@@ -1234,24 +1363,27 @@ static cudaError_t launch_finish_inorder(const SubmitArgs &a, bool may_sort, cud
     c.status = a.status; c.completion = a.completion; c.stall = a.stall; c.busy = a.busy; c.busy_stage = a.busy_stage;
     c.stats_stage = a.stats_stage; c.claim_limit = a.claim_limit; c.die_claims = a.die_claims;
     c.n_queues = a.mp.n_queues; c.n_dies = a.mp.n_dies;
-    c.desc_words = sort_tiles * kRadix; c.scan_words = scan_tiles * (sizeof(ScanDesc) / 4);
-    c.cls_grid = (unsigned)std::min<uint64_t>((n + kClsTile - 1) / kClsTile, (uint64_t)a.sm_count * 8);
-    c.hist_grid = (unsigned)std::min<uint64_t>((n + kHistThreads * 8 - 1) / (kHistThreads * 8), (uint64_t)a.sm_count * 4);
-    c.sort_grid = (unsigned)std::min<uint64_t>(sort_tiles, (uint64_t)a.sm_count * 3);
-    c.scan_grid = (unsigned)std::min<uint64_t>(scan_tiles, (uint64_t)a.sm_count * 8);
-    c.stall_grid = (unsigned)std::max<uint64_t>(1, std::min<uint64_t>((n + 255) / 256, (uint64_t)a.sm_count * 16));
+    c.desc_words = sort_tiles * kRadix; c.scan_words = scan_tiles * (sizeof(ScanDesc) / 4); c.sync = a.rg_sync;
     const InTileMap tmap = inorder_tile_map(n, a.sm_count, a.bal && a.bal->on && a.bal->dev);
     c.in_tile = reinterpret_cast<const InTile *>(a.ws.in_tile);
     c.n_tiles = tmap.n_tiles;
-    e = launch_pdl(may_sort ? k_finish_inorder<true> : k_finish_inorder<false>, finish_grid(a), 256, 0, st, c, finish_args(a), regroup_args(n, a.ws, may_sort && n >= 2 ? a.rg_sync : nullptr));
+    const RegroupArgs rg = regroup_args(n, a.ws, may_sort && n >= 2 ? a.rg_sync : nullptr);
+    cudaError_t e;
+    if (may_sort) {
+        e = ensure_dyn_smem((const void *)k_finish_inorder<true>, kSortSmem);
+        if (e != cudaSuccess) return e;
+        const unsigned grid = (unsigned)std::max<uint64_t>(1, std::min<uint64_t>((n + 2047) / 2048, (uint64_t)a.sm_count * kLastBlocks));
+        e = launch_pdl(k_finish_inorder<true>, grid, kLastThreads, kSortSmem, st, c, finish_args(a), rg);
+    } else {
+        e = launch_pdl(k_finish_inorder<false>, finish_grid(a), 256, 0, st, c, finish_args(a), rg);
+    }
     if (e != cudaSuccess) return e;
-    if (may_sort && a.plain_next) *a.plain_next = true;      // (kernels that may overlap their predecessor must not overlap one that may launch others)
     g_kernel_launches += 1;
     return cudaGetLastError();
 }
 
 // Kernel order of one batch.  AUTO: begin (which brings a batch out of issue order into order), the in-order kernels,
-// k_finish_inorder (the commit; it launches the sort kernels from the device where the others handed the batch over).
+// k_finish_inorder (the commit; where the others handed the batch over it goes through the radix sort before that).
 // SORT / SORT_FULL: begin, sort kernels, finish.
 cudaError_t launch_submit(const SubmitArgs &a, cudaStream_t st) {
     const uint64_t n = a.n;
@@ -1265,7 +1397,7 @@ cudaError_t launch_submit(const SubmitArgs &a, cudaStream_t st) {
                           a.ranges, a.stage == 1 ? a.mp.stripe_shift : 0u};
         const cudaError_t e = try_inorder && sort_kernels && n >= 2
             ? launch_begin_regroup(a, b, st)
-            : launch_first(a.plain_next, k_begin, 1, 1024, 0, st, b, 0, try_inorder ? 0 : 1, a.acc);
+            : launch_first(a.plain_next, k_begin, 1, 1024, 0, st, b, try_inorder ? 0 : 1, a.acc);
         if (e != cudaSuccess) return e;
     }
     if (a.stage != 2) g_kernel_launches += 1;
