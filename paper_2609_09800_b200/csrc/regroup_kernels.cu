@@ -40,9 +40,10 @@ __device__ __forceinline__ uint32_t rg_stretch(int64_t t, int64_t lo, uint32_t s
 
 // Do so many records share their issue times that buckets would overflow, or spend their time on telling equal times apart?  1,024
 // samples, one per thread, and a table of the distinct ones; where few are equal, pairs of equal ones tell (of m samples of D times
-// about m^2 / 2D), else the distinct ones are nearly all there are.  40 M shuffled records, us, by the radix sort CROWD_RADIX
-// (the attempt in buckets adds 700 if it overflows, from some 900 records per time on); in buckets CROWD_FIGURES.
-constexpr uint32_t kRgCrowd = 700, kRgSeen = 4096;
+// about m^2 / 2D), else the distinct ones are nearly all there are.  40 M shuffled records, us, by the radix sort 6,290 (the
+// attempt in buckets adds 700 if it overflows, from some 900 records per time on), in buckets 2,730 with 1 record per time, 3,570 with 20, 4,790 with
+// 60, 5,000 with 250, 7,090 with 500; 4 M 625, and 450, 550, 660, 680, 910.
+constexpr uint32_t kRgCrowd = 300, kRgSeen = 4096;
 __device__ __forceinline__ bool rg_crowded(long long time, uint64_t n, unsigned long long *seen) {
     for (uint32_t e = threadIdx.x; e < kRgSeen; e += kRgThreads) seen[e] = 0ull;
     __syncthreads();
