@@ -576,7 +576,7 @@ static int serve_records(hbf_ctx *c, SubmitArgs &a) {
         if (!a.bus_on) return HBF_OK;
     } else {
         if (c->ret_on)                                       // how far the outstanding refresh quanta reach into this batch
-            CK(launch_ret_window(a.acc, a.n, c->d_ranges, c->ret, c->sm_count, c->stream));
+            CK(launch_ret_window(a.acc, a.n, c->d_ranges, c->ret, c->sm_count, now.plain_next, c->stream));
         CK(launch_submit(a, c->stream));
     }
     if (a.binned) {
@@ -586,7 +586,7 @@ static int serve_records(hbf_ctx *c, SubmitArgs &a) {
                               c->n_bins, c->cur_bin, c->sm_count, a.claim_limit, quantum_pj, c->stream));
     }
     if (c->ret_on)                                           // read disturb, commits, the claimed energy (after the ledger: it needs the claim limit)
-        CK(launch_ret_close(a.acc, a.n, c->d_ranges, c->d_mp, c->mp, c->d_result, c->d_pending, a.binned, c->ret, c->sm_count, c->stream));
+        CK(launch_ret_close(a.acc, a.n, c->d_ranges, c->d_mp, c->mp, c->d_result, c->d_pending, a.binned, c->ret, c->sm_count, now.plain_next, c->stream));
     if (c->d_bus_busy)                                       // after the ledger: its events are the array intervals
         CK(launch_bus_stage(a, c->d_bus_ctrl, c->d_bus_busy, c->stream));
     return HBF_OK;

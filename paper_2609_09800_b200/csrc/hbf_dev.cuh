@@ -311,7 +311,7 @@ struct RetState {
     unsigned long long claim_limit;      // this batch: modeled accesses with a smaller batch index claim one quantum each
     unsigned long long claims_now;       // quanta this batch claims if it is accepted
     unsigned long long tickets, counted; // the claim window's tile counter and the modeled accesses counted so far
-    unsigned long long epoch_blocks;     // thread blocks of the plan kernel that are done (0 between epochs)
+    unsigned long long epoch_blocks;     // thread blocks of the kernel at work that are done (0 between kernels)
     uint32_t epoch;
     uint32_t observed_inline;            // the in-order serve pass has counted this batch's reads into the disturb counters
 };
@@ -332,9 +332,9 @@ struct RetDev {
     int *region_max;                     // [regions] hottest cell, as an ordered integer
     RetState *st;
 };
-cudaError_t launch_ret_window(const hbf_access_t *acc, uint64_t n, const RangeSnap *ranges, const RetDev &r, int sm_count, cudaStream_t st);
+cudaError_t launch_ret_window(const hbf_access_t *acc, uint64_t n, const RangeSnap *ranges, const RetDev &r, int sm_count, bool *plain_next, cudaStream_t st);
 cudaError_t launch_ret_close(const hbf_access_t *acc, uint64_t n, const RangeSnap *ranges, const ModelParams *mp_dev, const ModelParams &mp,
-                             const hbf_batch_result_t *result, int64_t *pending, int binned, const RetDev &r, int sm_count, cudaStream_t st);
+                             const hbf_batch_result_t *result, int64_t *pending, int binned, const RetDev &r, int sm_count, bool *plain_next, cudaStream_t st);
 struct ThermalDev;
 cudaError_t launch_ret_advance(const RetDev &r, const ModelParams &mp, const ThermalDev *field, const float *theta, const int32_t *die_region,
                                int have_temps, int64_t dt_ns, int sm_count, bool *plain_next, cudaStream_t st);

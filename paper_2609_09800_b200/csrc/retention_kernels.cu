@@ -20,8 +20,8 @@ namespace hbf {
 
 __device__ __forceinline__ bool ret_ready(const RangeSnap &rs, const hbf_access_t *acc, uint64_t i, uint64_t *off, uint32_t *bytes, uint32_t *op) {
     const uint64_t *rec = reinterpret_cast<const uint64_t *>(acc + i);
-    const uint64_t addr = __ldg(rec), bf = __ldg(rec + 2);
-    const int64_t issue = (int64_t)__ldg(rec + 1);
+    const uint64_t addr = ld_after(rec), bf = ld_after(rec + 2);
+    const int64_t issue = (int64_t)ld_after(rec + 1);
     int g = 0;
     if (classify(rs, addr, issue, (uint32_t)bf, (uint32_t)(bf >> 32), &g) != HBF_ST_READY) return false;
     if (off) *off = rs.media_offset[g] + (addr - rs.base[g]);
@@ -52,6 +52,16 @@ __device__ __forceinline__ uint32_t block_scan_incl(uint32_t v, uint32_t *total)
     return x + before;
 }
 
+// whether this block is the last of the grid to come here: every other one's writes are visible then (the counter is 0 between kernels)
+__device__ __forceinline__ bool ret_last_block(RetState *st) {
+    __shared__ uint32_t s_last;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) { s_last = atomicAdd(&st->epoch_blocks, 1ull) == gridDim.x - 1u ? 1u : 0u; __threadfence(); if (s_last) st->epoch_blocks = 0ull; }
+    __syncthreads();
+    return s_last != 0u;
+}
+
 // =====================================================================================================
 // claim window: how far into the batch do the outstanding quanta reach?
 // =====================================================================================================
@@ -61,16 +71,22 @@ constexpr int kRetTile = 1024;
 // debt, not to the batch.  A debt of as many quanta as the batch has records reaches past its end whatever they are: nothing is
 // counted then, and what the batch claims is the number of its modeled accesses (kRetAll).
 // (a tile of 1,024 at a time, 256 threads: 164 us for 20.6 M of 24 M records, and 37 for the search; now 106, 4.7 TB/s,
-// and 14)
+// and 14.  The search is the last block's, commits and accounts behind the batch are one kernel, and all overlap their starts: two batches of 500,000
+// with an epoch between 259 -> 237 us, of 24 M 1,204 -> 1,176)
 constexpr int kRetWinThreads = 1024, kRetWinTiles = 8;
 constexpr unsigned long long kRetAll = ~0ull;
 __global__ void __launch_bounds__(kRetWinThreads)
-k_ret_window(const hbf_access_t *__restrict__ acc, uint64_t n, const RangeSnap *__restrict__ ranges_g, RetDev r) {
+k_ret_window(const hbf_access_t *acc, uint64_t n, const RangeSnap *__restrict__ ranges_g, const __grid_constant__ RetDev r) {
     __shared__ RangeSnap rs;
     __shared__ uint32_t s_first, s_cnt[2][kRetWinTiles];
+    pdl_wait();
+    pdl_trigger();
     RetState *st = r.st;
     const unsigned long long debt = st->planned - st->claimed - st->decayed;
-    if (debt == 0ull || debt >= n) return;
+    if (debt == 0ull || debt >= n) {
+        if (blockIdx.x == 0 && threadIdx.x == 0) { st->claim_limit = debt ? n : 0ull; st->claims_now = debt && n ? kRetAll : 0ull; }
+        return;
+    }
     load_ranges(&rs, ranges_g);
     const int tid = threadIdx.x, lane = tid & 31;
     if (tid < 2 * kRetWinTiles) (&s_cnt[0][0])[tid] = 0u;
@@ -95,24 +111,11 @@ k_ret_window(const hbf_access_t *__restrict__ acc, uint64_t n, const RangeSnap *
             atomicAdd(&st->counted, sum);
         }
     }
-}
-
-// One block: the tile in which the running count reaches the debt, then the record inside it.
-__global__ void __launch_bounds__(kRetTile)
-k_ret_find(const hbf_access_t *__restrict__ acc, uint64_t n, const RangeSnap *__restrict__ ranges_g, RetDev r) {
-    __shared__ RangeSnap rs;
+    // the last block: the tile in which the running count reaches the debt, then the record inside it
+    if (!ret_last_block(st)) return;
     __shared__ unsigned long long s_base, s_before;
     __shared__ uint32_t s_found;
-    RetState *st = r.st;
-    const int tid = threadIdx.x;
-    const unsigned long long debt = st->planned - st->claimed - st->decayed;
-    if (debt == 0ull || debt >= n) {
-        if (tid == 0) { st->claim_limit = debt ? n : 0ull; st->claims_now = debt && n ? kRetAll : 0ull; st->tickets = 0ull; st->counted = 0ull; }
-        return;
-    }
-    load_ranges(&rs, ranges_g);
-    const uint64_t n_tiles = (n + kRetTile - 1) / kRetTile;
-    const uint64_t T = min((uint64_t)st->tickets, n_tiles);
+    const uint64_t T = min((uint64_t)__ldcg(&st->tickets), n_tiles);
     if (tid == 0) { s_base = 0ull; s_found = 0xffffffffu; }
     __syncthreads();
     constexpr int kPer = 8;
@@ -120,7 +123,7 @@ k_ret_find(const hbf_access_t *__restrict__ acc, uint64_t n, const RangeSnap *__
         const uint64_t t0 = chunk + (uint64_t)tid * kPer;
         uint32_t v[kPer], mine = 0, sum = 0;
 #pragma unroll
-        for (int k = 0; k < kPer; ++k) { v[k] = t0 + k < T ? r.tile_count[t0 + k] : 0u; mine += v[k]; }
+        for (int k = 0; k < kPer; ++k) { v[k] = t0 + k < T ? __ldcg(r.tile_count + t0 + k) : 0u; mine += v[k]; }
         const uint32_t incl = block_scan_incl<kRetTile>(mine, &sum);
         unsigned long long at = s_base + incl - mine;
 #pragma unroll
@@ -146,13 +149,11 @@ k_ret_find(const hbf_access_t *__restrict__ acc, uint64_t n, const RangeSnap *__
     if (tid == 0) { st->tickets = 0ull; st->counted = 0ull; }
 }
 
-cudaError_t launch_ret_window(const hbf_access_t *acc, uint64_t n, const RangeSnap *ranges, const RetDev &r, int sm_count, cudaStream_t st) {
+cudaError_t launch_ret_window(const hbf_access_t *acc, uint64_t n, const RangeSnap *ranges, const RetDev &r, int sm_count, bool *plain_next, cudaStream_t st) {
     const uint64_t tiles = (n + kRetTile - 1) / kRetTile;
     const unsigned grid = (unsigned)std::max<uint64_t>(1, std::min<uint64_t>((tiles + kRetWinTiles - 1) / kRetWinTiles, (uint64_t)sm_count * 2));
-    k_ret_window<<<grid, kRetWinThreads, 0, st>>>(acc, n, ranges, r);
-    k_ret_find<<<1, kRetTile, 0, st>>>(acc, n, ranges, r);
-    g_kernel_launches += 2;
-    return cudaGetLastError();
+    g_kernel_launches += 1;
+    return launch_first(plain_next, k_ret_window, grid, kRetWinThreads, 0, st, acc, n, ranges, r);
 }
 
 // =====================================================================================================
@@ -163,9 +164,11 @@ cudaError_t launch_ret_window(const hbf_access_t *acc, uint64_t n, const RangeSn
 // then refused (take the counts back: the same reads, the same amounts).
 __global__ void __launch_bounds__(256)
 k_ret_observe(const hbf_access_t *__restrict__ acc, uint64_t n, const RangeSnap *__restrict__ ranges_g,
-              const ModelParams *__restrict__ mp_g, const hbf_batch_result_t *result, RetDev r) {
+              const ModelParams *__restrict__ mp_g, const hbf_batch_result_t *result, const __grid_constant__ RetDev r) {
     __shared__ RangeSnap rs;
     __shared__ ModelParams mp;
+    pdl_wait();
+    pdl_trigger();
     const bool ok = result->code == HBF_OK, inline_done = r.st->observed_inline != 0u;
     if (ok == inline_done) return;                           // counted and accepted, or neither
     const bool undo = inline_done;
@@ -184,28 +187,31 @@ k_ret_observe(const hbf_access_t *__restrict__ acc, uint64_t n, const RangeSnap 
 }
 
 // a block whose last quantum lies below the watermark commits one cycle and clears its counters
-__global__ void __launch_bounds__(256)
-k_ret_commit(const hbf_batch_result_t *result, RetDev r) {
-    RetState *st = r.st;
-    unsigned long long mark = st->claimed + st->decayed;
-    if (result) { if (result->code != HBF_OK) return; mark += st->claims_now == kRetAll ? (unsigned long long)result->n_modeled : st->claims_now; }
+__device__ __forceinline__ void ret_commit_due(const RetDev &r, unsigned long long mark) {
     const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
     for (uint64_t b = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; b < r.n_blocks; b += stride) {
         if (r.epoch_of[b] == 0u || r.last_pos[b] >= mark) continue;
         ret_commit_block(r, b);
     }
 }
+__global__ void __launch_bounds__(256) k_ret_commit(RetDev r) { ret_commit_due(r, r.st->claimed + r.st->decayed); }
 
-__global__ void k_ret_close(const hbf_batch_result_t *result, int64_t *pending, int64_t quantum_pj, uint32_t n_dies, RetDev r) {
+// the same behind a batch; the last block books what the batch claimed
+__global__ void __launch_bounds__(256) k_ret_close(const hbf_batch_result_t *result, int64_t *pending, int64_t quantum_pj, uint32_t n_dies, const __grid_constant__ RetDev r) {
+    pdl_wait();
+    pdl_trigger();
+    RetState *st = r.st;
     const bool ok = result->code == HBF_OK;
+    const unsigned long long claims = !ok ? 0ull : st->claims_now == kRetAll ? (unsigned long long)result->n_modeled : st->claims_now;
+    if (ok) ret_commit_due(r, st->claimed + st->decayed + claims);
+    if (!ret_last_block(st)) return;
     for (uint32_t d = threadIdx.x; d < n_dies; d += blockDim.x) {
         const uint32_t c = r.die_claims[d];
         if (ok && c) pending[d] += (int64_t)c * quantum_pj;
         r.die_claims[d] = 0u;
     }
     if (threadIdx.x == 0) {
-        RetState *st = r.st;
-        if (ok) st->claimed += st->claims_now == kRetAll ? (unsigned long long)result->n_modeled : st->claims_now;
+        st->claimed += claims;
         st->claims_now = 0ull; st->claim_limit = 0ull; st->observed_inline = 0u;
     }
 }
@@ -215,14 +221,16 @@ static unsigned ret_grid(uint64_t items, int sm_count) {
 }
 
 cudaError_t launch_ret_close(const hbf_access_t *acc, uint64_t n, const RangeSnap *ranges, const ModelParams *mp_dev, const ModelParams &mp,
-                             const hbf_batch_result_t *result, int64_t *pending, int binned, const RetDev &r, int sm_count, cudaStream_t st) {
-    if (n) k_ret_observe<<<ret_grid(n, sm_count), 256, 0, st>>>(acc, n, ranges, mp_dev, result, r);
-    k_ret_commit<<<ret_grid(r.n_blocks, sm_count), 256, 0, st>>>(result, r);
+                             const hbf_batch_result_t *result, int64_t *pending, int binned, const RetDev &r, int sm_count, bool *plain_next, cudaStream_t st) {
+    cudaError_t e = cudaSuccess;
+    if (n) e = launch_first(plain_next, k_ret_observe, ret_grid(n, sm_count), 256, 0, st, acc, n, ranges, mp_dev, result, r);
+    if (e != cudaSuccess) return e;
     const int64_t page = (int64_t)1 << mp.page_shift;
     const int64_t quantum_pj = mp.e_cmd_read_pj + mp.e_byte_read_pj * page + mp.e_cmd_prog_pj + mp.e_byte_prog_pj * page;
-    k_ret_close<<<1, 256, 0, st>>>(result, pending, binned ? 0 : quantum_pj, mp.n_dies, r);   // with the time bins on, the ledger has it
-    g_kernel_launches += n ? 3 : 2;
-    return cudaGetLastError();
+    // (with the time bins on, the ledger has the energy)
+    e = launch_first(plain_next, k_ret_close, ret_grid(r.n_blocks, sm_count), 256, 0, st, result, pending, binned ? (int64_t)0 : quantum_pj, mp.n_dies, r);
+    g_kernel_launches += n ? 2 : 1;
+    return e;
 }
 
 // =====================================================================================================
@@ -519,7 +527,7 @@ cudaError_t launch_ret_totals(const RetDev &r, int sm_count, RetState *h_state, 
 
 cudaError_t launch_ret_decay(const RetDev &r, const ModelParams &mp, const DevState *state, int64_t idle_ns, int sm_count, cudaStream_t st) {
     k_ret_decay<<<1, 1, 0, st>>>(r, state, mp.t_read_ns + mp.t_prog_ns, idle_ns);
-    k_ret_commit<<<ret_grid(r.n_blocks, sm_count), 256, 0, st>>>(nullptr, r);
+    k_ret_commit<<<ret_grid(r.n_blocks, sm_count), 256, 0, st>>>(r);
     g_kernel_launches += 2;
     return cudaGetLastError();
 }
