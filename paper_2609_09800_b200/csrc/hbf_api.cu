@@ -366,6 +366,7 @@ int hbf_create(const hbf_config_t *cfg, void *cuda_stream, hbf_ctx **out) {
     mp.e_cmd_prog_pj = cfg->e_cmd_prog_pj; mp.e_byte_prog_pj = cfg->e_byte_prog_pj;
 
     mp.div_chan = make_div64_host(cfg->chan_bytes_per_us);
+    mp.div_ch = make_div64_host(cfg->channels); mp.div_dies = make_div64_host(cfg->dies); mp.div_planes = make_div64_host(cfg->planes);
     {   // the in-order path packs the transfer time of an access into 31 bits and keeps per-queue state in shared memory
         const unsigned __int128 worst = ((unsigned __int128)0xffffffffull + std::max(cfg->read_granule, cfg->prog_granule)) * 1000u;
         c->inorder_ok = nq <= kInMaxQueues && worst / cfg->chan_bytes_per_us < ((unsigned __int128)1 << 31) &&
