@@ -525,7 +525,10 @@ k_inorder_serve(const hbf_access_t *__restrict__ acc, uint64_t n, const __grid_c
     if (ctrl->regrouped) { acc = copy.recs; completion = copy.comp; stall = copy.stall; status = nullptr; }   // (brought into order: regroup_kernels.cu)
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const RangeSnap &rs = *ranges_g;                      // read through the cache; the common configuration does not touch it
-    if (tid == 0) { mp = mp_arg; fast_range = fast_arg; }
+    // (by one thread it is some ninety stores one after the other)
+    static_assert(sizeof(ModelParams) % 4 == 0 && sizeof(ModelParams) / 4 <= kInThreads && sizeof(FastRange) % 4 == 0, "a word per thread");
+    if (tid < (int)(sizeof(ModelParams) / 4)) reinterpret_cast<uint32_t *>(&mp)[tid] = reinterpret_cast<const uint32_t *>(&mp_arg)[tid];
+    if (tid < (int)(sizeof(FastRange) / 4)) reinterpret_cast<uint32_t *>(&fast_range)[tid] = reinterpret_cast<const uint32_t *>(&fast_arg)[tid];
     if (DEBT && !RESERVE && tid == 0 && blockIdx.x == 0) ret.st->observed_inline = 1u;
     if (!RESERVE && bal && tid == 0 && blockIdx.x == 0) { bal->strag_seq = bal_seq; bal->strag_max = 0u; bal->strag_flagged = 0u; bal->strag_depth = LIGHT ? 0u : head_depth; }
     const uint32_t R = mp_arg.n_queues, n_dies = mp_arg.n_dies;
