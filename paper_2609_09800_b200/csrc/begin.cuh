@@ -84,7 +84,7 @@ __device__ __forceinline__ void begin_units(const BeginArgs &a, const uint64_t *
     int g = 0;
     if (classify(*a.ranges, addr, (int64_t)ld_after(rec + 1), (uint32_t)bf, (uint32_t)(bf >> 32), &g) != HBF_ST_READY) return;
     const uint64_t off = a.ranges->media_offset[g] + (addr - a.ranges->base[g]);
-    if ((off & (unit - 1ull)) + (uint32_t)bf > unit) a.ctrl->crossed = 1u;
+    if ((off & (unit - 1ull)) + (uint32_t)bf > unit) a.ctrl->sample_crossed = 1u;
 }
 
 }  // namespace hbf

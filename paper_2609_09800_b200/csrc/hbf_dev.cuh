@@ -81,7 +81,8 @@ struct BatchCtrl {
     float load;                          // the share of the batch's span that its work, and what the queues are behind, fills (0: not asked)
     int64_t issue_lo, issue_hi;          // smallest and largest issue time among the begin kernel's samples
     unsigned long long pages;            // page-granular submit, first stage: pages of all accesses (one of an access that is not modeled)
-    uint32_t crossed, pad1;              //   set: some modeled access reaches over the end of its stripe unit
+    uint32_t sample_crossed, crossed;    //   set: some modeled access reaches over the end of its stripe unit, among the begin kernel's samples (settled when
+                                         //   the pass begins: its blocks leave on it) or in a tile of the pass (blocks write it while others begin)
     uint32_t role_count[2];              // in-order serve pass: tiles handed out so far, per size class
     uint32_t tile_counter[kMaxPasses + 2];
     long long modeled_ns, service_ns, max_completion_ns;

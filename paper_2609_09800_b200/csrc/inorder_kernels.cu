@@ -515,7 +515,7 @@ k_inorder_serve(const hbf_access_t *__restrict__ acc, uint64_t n, const __grid_c
     pdl_wait();
     pdl_trigger();
     if (ctrl->skip || ctrl->run_sort) return;             // (run_sort set this early: the batch went to the sort path at its start)
-    if (LOOK && ctrl->crossed) return;                    // (the samples showed it: the records are cut first)
+    if (LOOK && ctrl->sample_crossed) return;             // (the samples showed it: the records are cut first)
     if (!RESERVE && decided && (ctrl->twice != 0u) != LIGHT) return;      // (the batch's load has chosen the other of the two)
     if (RESERVE && decided && blockIdx.x == 0 && threadIdx.x == 0 && ctrl->inorder_used && !ctrl->twice && 2u * bal->strag_flagged >= tmap.n_tiles) {
         bal->twice_load = ctrl->load; bal->twice_left = kInTwiceRun;

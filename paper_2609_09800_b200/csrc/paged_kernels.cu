@@ -69,7 +69,7 @@ k_paged_count(const hbf_access_t *__restrict__ acc, uint64_t n, const RangeSnap 
     __shared__ uint32_t s_row[kPgRows];
     __shared__ unsigned long long s_pages, s_parts;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    if (BY_UNIT && looked && !looked->skip && !looked->crossed && !looked->unsorted && looked->n_fault == 0ull) {      // the first pass has counted
+    if (BY_UNIT && looked && !looked->skip && !looked->sample_crossed && !looked->crossed && !looked->unsorted && looked->n_fault == 0ull) {      // the first pass has counted
         if (blockIdx.x == 0 && tid == 0) { totals[kPagedServed] = 1ull; totals[kPagedParts] = n; totals[kPagedPages] = looked->pages; }
         return;
     }

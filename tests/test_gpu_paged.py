@@ -249,6 +249,30 @@ def test_the_first_pass_counts(hbf, kind, n):
         acc["issue_ns"] += 1000
 
 
+@pytest.mark.parametrize("n", [400_003, 2_000_001])
+@pytest.mark.parametrize("where", ["first tile", "early and in the middle", "everywhere"])
+def test_crossings_that_the_samples_miss(hbf, n, where):
+    """The blocks of the pass that counts leave on what the 1,024 samples showed, not on what other blocks of it find meanwhile: crossings in
+    tiles that are served first, between the samples, a batch twice on one context and one without crossings behind it."""
+    rng = np.random.default_rng(n)
+    prof = wl.load_profile("nominal", channels=8, dies=4, planes=2, page_bytes=16384, stripe_bytes=65536)
+    g, o = contexts(hbf, prof, [(wl.RANGE_BASE, wl.GIB, 3, 0, 0, 0)])
+    acc = np.zeros(n, hbfo.ACCESS_DTYPE)
+    acc["bytes"] = rng.choice([1, 16384, 40_000, 65_536], n)
+    acc["addr"] = wl.RANGE_BASE + rng.integers(0, 16_000, n).astype(np.uint64) * np.uint64(65536) + (rng.random(n) * (65_537 - acc["bytes"])).astype(np.uint64)
+    acc["issue_ns"] = np.sort(rng.integers(0, 30_000 * n, n))
+    inside = acc.copy()
+    odd = {"first tile": np.array([1, 2]), "early and in the middle": np.concatenate([np.arange(5, 3_000, 97), n // 2 + np.arange(0, 3_000, 97)]),
+           "everywhere": rng.choice(n, n // 50, replace=False)}[where]
+    odd = np.setdiff1d(odd, np.arange(1024) * (n - 1) // 1024)
+    acc["addr"][odd] = wl.RANGE_BASE + rng.integers(0, 16_000, len(odd)).astype(np.uint64) * np.uint64(65536) + np.uint64(65_535)
+    acc["bytes"][odd] = 2
+    for batch in (acc, inside, acc):
+        batch = batch.copy()
+        batch["issue_ns"] += 1000
+        compare(g, o, batch)
+
+
 @pytest.mark.parametrize("cross", [False, True])             # (no access crosses a stripe unit: the batch's own records are served)
 @pytest.mark.parametrize("n", [5_000, 12_000])
 def test_a_throttled_paged_batch_leaves_zeros(hbf, n, cross):
