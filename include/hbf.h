@@ -168,6 +168,8 @@ HBF_API int hbf_submit_host(hbf_ctx *ctx, const hbf_access_t *h_acc, uint64_t n,
  * n * (largest access / page_bytes + 2)); it sizes the workspace, hbf_workspace_bytes_paged(ctx, n, capacity).
  * The call counts the parts on the device and waits for that count (one stream synchronisation) before it
  * launches the rest; with more parts than parts_capacity it returns HBF_E_WORKSPACE and nothing has changed.
+ * Another thread's call on a context of the same stream comes before or behind the whole call: it waits meanwhile, so
+ * contexts of one stream may share a workspace here too.
  * Other arguments, ownership and error behaviour as for hbf_submit_batch.  hbf_queue_order afterwards refers
  * to parts, not accesses. */
 HBF_API size_t hbf_workspace_bytes_paged(const hbf_ctx *ctx, uint64_t n, uint64_t parts_capacity);

@@ -535,22 +535,22 @@ static bool capturing(cudaStream_t st) {
 }
 
 // One call's launches: holds the stream's note meanwhile.  What is being captured does not run behind what the stream was given
-// last, and the per-thread default stream is another one in every thread: such a call begins with an ordinary launch.
+// last, and the per-thread default stream is another one in every thread: such a call begins with an ordinary launch, and on that
+// stream there is nothing to hold (calls of other threads are on other streams).
 class Launching {
-    std::lock_guard<std::mutex> lock_;
+    std::unique_lock<std::mutex> lock_;
     bool own_ = true;
 public:
     const bool captured;
     bool *const plain_next;
-    explicit Launching(hbf_ctx *c) : lock_(c->note->launching), captured(capturing(c->stream)),
-        plain_next(captured || c->stream == cudaStreamPerThread ? &own_ : &c->note->plain_next) {}
+    explicit Launching(hbf_ctx *c) : lock_(c->note->launching, std::defer_lock), captured(capturing(c->stream)),
+        plain_next(captured || c->stream == cudaStreamPerThread ? &own_ : &c->note->plain_next) { if (c->stream != cudaStreamPerThread) lock_.lock(); }
 };
 
 // Everything a batch of records goes through once its arguments are in place: the claim window (retention), the submit
 // path, the energy ledger, read disturb / commits, the channel-bus stage.  Shared by hbf_submit_batch (the caller's
 // accesses) and hbf_submit_batch_paged (the list of parts).
-static int serve_records(hbf_ctx *c, SubmitArgs &a) {
-    Launching now(c);
+static int serve_records(hbf_ctx *c, SubmitArgs &a, const Launching &now) {
     if (now.captured) c->captured = true;
     a.ranges = c->d_ranges; a.mp_dev = c->d_mp; a.mp = c->mp; a.state = c->d_state; a.ctrl = c->d_ctrl; a.result = c->d_result;
     a.result_host = &c->pinned->result; a.plain_next = now.plain_next;
@@ -611,7 +611,8 @@ int hbf_submit_batch(hbf_ctx *c, const hbf_access_t *d_acc, uint64_t n, int64_t 
     c->prof_inorder = c->profiling && n > 0 && c->inorder_ok && (c->path == HBF_PATH_AUTO || c->path == HBF_PATH_INORDER);
     a.ev = c->profiling ? c->ev : nullptr;
     c->prof_submit = c->profiling;
-    const int rc = serve_records(c, a);
+    Launching now(c);
+    const int rc = serve_records(c, a, now);
     if (rc != HBF_OK) return rc;
     c->submitted = true;
     return HBF_OK;
@@ -808,6 +809,9 @@ int hbf_submit_batch_paged(hbf_ctx *c, const hbf_access_t *d_acc, uint64_t n, ui
     };
     SubmitArgs a{};
     int rc = HBF_OK;
+    // Held over the host's wait as well: what the kernels before it leave in the workspace (the first pass's maps of the queues, where every
+    // access's parts begin) is read behind it, and another context's call on this stream may use the same workspace.
+    Launching now(c);
     CK(launch_paged_clear(pw, c->stream));
     if (by_unit && n >= kPagedLookFirst && !c->paged_crossed && paged_unit_ns(c->mp) < (1ll << 33)) {
         // Most often no access reaches over the end of its stripe unit, and the first of the two passes over the records counts beside its own
@@ -820,7 +824,7 @@ int hbf_submit_batch_paged(hbf_ctx *c, const hbf_access_t *d_acc, uint64_t n, ui
         a.paged = 1; a.stage = 1;
         const bool on_host = c->result_on_host;
         std::swap(c->d_ctrl, c->d_ctrl_spare);
-        rc = serve_records(c, a);
+        rc = serve_records(c, a, now);
         std::swap(c->d_ctrl, c->d_ctrl_spare);
         c->result_on_host = on_host;
         if (rc == HBF_OK) rc = count(true, c->d_ctrl_spare);
@@ -843,7 +847,7 @@ int hbf_submit_batch_paged(hbf_ctx *c, const hbf_access_t *d_acc, uint64_t n, ui
         a.acc = d_acc; a.n = n; a.completion = d_completion_ns; a.stall = d_stall_ns; a.status = d_status; a.die_stats = d_die_stats;
         a.paged = 1; a.stage = served ? 2 : 0;
         if (served) std::swap(c->d_ctrl, c->d_ctrl_spare);
-        if ((rc = serve_records(c, a)) != HBF_OK) return rc;
+        if ((rc = serve_records(c, a, now)) != HBF_OK) return rc;
         c->submitted = true;
         return HBF_OK;
     }
@@ -856,7 +860,7 @@ int hbf_submit_batch_paged(hbf_ctx *c, const hbf_access_t *d_acc, uint64_t n, ui
     a.die_stats = d_die_stats;
     a.paged = by_unit ? 1 : 0;
     a.ev = nullptr;
-    if ((rc = serve_records(c, a)) != HBF_OK) return rc;
+    if ((rc = serve_records(c, a, now)) != HBF_OK) return rc;
     CK(launch_paged_join(d_acc, n, pw, c->d_result, &c->pinned->result, d_completion_ns, d_stall_ns, d_status, c->sm_count, c->stream));
     c->submitted = true;
     return HBF_OK;

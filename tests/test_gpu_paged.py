@@ -273,6 +273,50 @@ def test_crossings_that_the_samples_miss(hbf, n, where):
         compare(g, o, batch)
 
 
+@pytest.mark.parametrize("cross", [False, True])
+def test_two_threads_share_a_stream_and_a_workspace(hbf, cross):
+    """A page-granular batch keeps state in its workspace over its own wait for the device (the first pass's maps of the queues, or where every
+    access's parts begin): another context's call, from another thread, on the same stream and scratch comes before or behind all of it."""
+    import threading
+    import time
+    import torch
+    n = 500_000
+    prof = wl.load_profile("nominal", channels=8, dies=4, planes=2, page_bytes=16384, stripe_bytes=65536)
+    sides = []
+    for seed, gap in ((1, 30_000), (2, 3_000)):
+        rng = np.random.default_rng(seed)
+        acc = np.zeros(n, hbfo.ACCESS_DTYPE)
+        acc["bytes"] = 65_536 if cross else 16_384
+        acc["addr"] = wl.RANGE_BASE + rng.integers(0, 16_000, n).astype(np.uint64) * np.uint64(65536) + (rng.integers(0, 4, n) * 16_384).astype(np.uint64)
+        acc["issue_ns"] = np.sort(rng.integers(0, gap * n, n))
+        g, o = contexts(hbf, prof, [(wl.RANGE_BASE, wl.GIB, 3, 0, 0, 0)])
+        rec = torch.from_numpy(acc.view(np.int64).reshape(-1)).cuda()
+        comp, stall = (torch.zeros(n, dtype=torch.int64, device="cuda") for _ in range(2))
+        sides.append((g, o, acc, rec, comp, stall))
+    ws = torch.empty(sides[0][0].workspace_bytes_paged(n, 5 * n), dtype=torch.uint8, device="cuda")
+    codes = [None, None]
+
+    def call(k):
+        g, _, _, rec, comp, stall = sides[k]
+        codes[k] = g.submit_batch_paged(rec, n, 5 * n, comp, stall, None, None, ws)
+
+    for _ in range(2):
+        torch.cuda.synchronize()
+        torch.cuda._sleep(400_000_000)                       # (a fifth of a second in which the first call waits and the second comes)
+        threads = [threading.Thread(target=call, args=(k,)) for k in range(2)]
+        for t in threads:
+            t.start()
+            time.sleep(0.05)
+        for t in threads:
+            t.join()
+        torch.cuda.synchronize()
+        assert codes == [0, 0]
+        for g, o, acc, _, comp, stall in sides:
+            _, c_o, s_o, *_ = o.submit(acc, paged=True)
+            assert np.array_equal(comp.cpu().numpy(), c_o) and np.array_equal(stall.cpu().numpy(), s_o)
+            assert np.array_equal(g.get_busy_until(), o.busy_until()) and g.last_result() == o.last_result()
+
+
 @pytest.mark.parametrize("cross", [False, True])             # (no access crosses a stripe unit: the batch's own records are served)
 @pytest.mark.parametrize("n", [5_000, 12_000])
 def test_a_throttled_paged_batch_leaves_zeros(hbf, n, cross):
