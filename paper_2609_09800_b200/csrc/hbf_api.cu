@@ -74,6 +74,8 @@ struct hbf_ctx {
     bool terminal = false;           // a shutdown result has been observed
     // device state
     RangeSnap *d_ranges = nullptr; ModelParams *d_mp = nullptr; DevState *d_state = nullptr;
+    // (d_ctrl: the last batch's control block, at one place as long as the context lives: a captured graph holds it too.  d_ctrl_spare: of a
+    // page-granular batch while it is served in two stages)
     BatchCtrl *d_ctrl = nullptr, *d_ctrl_spare = nullptr; RegroupSync *d_rg_sync = nullptr; hbf_batch_result_t *d_result = nullptr;
     int64_t *d_busy = nullptr, *d_busy_stage = nullptr, *d_pending = nullptr; hbf_die_stats_t *d_stats_stage = nullptr;
     // pinned: the last batch's summary (written by its last kernel), part counts on their way back, the hotspots (written by the
@@ -552,7 +554,8 @@ public:
 // accesses) and hbf_submit_batch_paged (the list of parts).
 static int serve_records(hbf_ctx *c, SubmitArgs &a, const Launching &now) {
     if (now.captured) c->captured = true;
-    a.ranges = c->d_ranges; a.mp_dev = c->d_mp; a.mp = c->mp; a.state = c->d_state; a.ctrl = c->d_ctrl; a.result = c->d_result;
+    a.ranges = c->d_ranges; a.mp_dev = c->d_mp; a.mp = c->mp; a.state = c->d_state; a.result = c->d_result;
+    a.ctrl = a.stage ? c->d_ctrl_spare : c->d_ctrl; a.ctrl_home = a.stage == 2 ? c->d_ctrl : nullptr;
     a.result_host = &c->pinned->result; a.plain_next = now.plain_next;
     a.busy = c->d_busy; a.busy_stage = c->d_busy_stage; a.pending = c->d_pending; a.stats_stage = c->d_stats_stage;
     a.path = a.paged ? (int32_t)HBF_PATH_INORDER : c->path; a.sm_count = c->sm_count; a.inorder_ok = c->inorder_ok ? 1 : 0;
@@ -823,9 +826,7 @@ int hbf_submit_batch_paged(hbf_ctx *c, const hbf_access_t *d_acc, uint64_t n, ui
         a.acc = d_acc; a.n = n; a.completion = d_completion_ns; a.stall = d_stall_ns; a.die_stats = d_die_stats;
         a.paged = 1; a.stage = 1;
         const bool on_host = c->result_on_host;
-        std::swap(c->d_ctrl, c->d_ctrl_spare);
         rc = serve_records(c, a, now);
-        std::swap(c->d_ctrl, c->d_ctrl_spare);
         c->result_on_host = on_host;
         if (rc == HBF_OK) rc = count(true, c->d_ctrl_spare);
     } else {
@@ -846,7 +847,6 @@ int hbf_submit_batch_paged(hbf_ctx *c, const hbf_access_t *d_acc, uint64_t n, ui
         workspace_layout(n, c->mp.n_queues, c->mp.channels, rooms, &a.ws, pw.inner, 0);
         a.acc = d_acc; a.n = n; a.completion = d_completion_ns; a.stall = d_stall_ns; a.status = d_status; a.die_stats = d_die_stats;
         a.paged = 1; a.stage = served ? 2 : 0;
-        if (served) std::swap(c->d_ctrl, c->d_ctrl_spare);
         if ((rc = serve_records(c, a, now)) != HBF_OK) return rc;
         c->submitted = true;
         return HBF_OK;

@@ -134,6 +134,7 @@ struct SubmitArgs {
     FastRange fast;
     int binned;                          // the batch's energy goes to the time-bin ledger, not to the pending totals
     int paged;                           // every record is an access inside one stripe unit whose pages are queued on their own (declared in issue order)
+    BatchCtrl *ctrl_home;                // where the batch's last kernel leaves a copy of its control block (null: it is there)
     int stage;                           // 0: the whole batch; else (paged, not known yet to be such records) 1: up to the first pass, which finds out, and 2: the rest
     int bus_on;                          // the channel-bus stage follows: array-done times must fit its 47-bit key field
     const unsigned long long *claim_limit;  // retention on: batch index below which a modeled access claims a refresh quantum
@@ -145,7 +146,7 @@ struct SubmitArgs {
 };
 // what the last kernel of a batch needs
 struct FinishArgs {
-    uint64_t n; BatchCtrl *ctrl; DevState *state; int64_t *busy; const int64_t *busy_stage; int64_t *pending; const hbf_die_stats_t *stats_stage;
+    uint64_t n; BatchCtrl *ctrl, *ctrl_home; DevState *state; int64_t *busy; const int64_t *busy_stage; int64_t *pending; const hbf_die_stats_t *stats_stage;
     hbf_die_stats_t *die_stats; int64_t *completion, *stall; hbf_batch_result_t *result, *result_host; const ModelParams *mp;
     uint32_t n_queues, n_dies; int binned, bus_on, paged;
 };

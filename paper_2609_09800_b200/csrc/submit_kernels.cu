@@ -1341,11 +1341,15 @@ __global__ void __launch_bounds__(MAY_SORT ? kLastThreads : 256, MAY_SORT ? kLas
         }
     }
     finish_batch(f, blockIdx.x == 0 && !c.ctrl->skip ? stall_total() : 0);
+    if constexpr (!MAY_SORT) {                               // (nothing writes the control block here)
+        if (f.ctrl_home && blockIdx.x == 0)
+            for (uint32_t i = threadIdx.x; i < sizeof(BatchCtrl) / 4u; i += blockDim.x) reinterpret_cast<uint32_t *>(f.ctrl_home)[i] = reinterpret_cast<const uint32_t *>(f.ctrl)[i];
+    }
 }
 
 static FinishArgs finish_args(const SubmitArgs &a) {
     FinishArgs f{};
-    f.n = a.n; f.ctrl = a.ctrl; f.state = a.state; f.busy = a.busy; f.busy_stage = a.busy_stage; f.pending = a.pending;
+    f.n = a.n; f.ctrl = a.ctrl; f.ctrl_home = a.ctrl_home; f.state = a.state; f.busy = a.busy; f.busy_stage = a.busy_stage; f.pending = a.pending;
     f.stats_stage = a.stats_stage; f.die_stats = a.die_stats; f.completion = a.completion; f.stall = a.stall;
     f.result = a.result; f.result_host = a.result_host; f.mp = a.mp_dev; f.n_queues = a.mp.n_queues; f.n_dies = a.mp.n_dies;
     f.binned = a.binned; f.bus_on = a.bus_on; f.paged = a.paged;

@@ -109,3 +109,32 @@ def test_a_captured_batch_that_fills_a_wave(hbf, entries):
         other.submit_batch(t.acc, n, comp, stall, None, None, other.workspace(n))
         torch.cuda.synchronize()
         assert torch.equal(t.comp, comp) and np.array_equal(t.g.get_busy_until(), other.get_busy_until())
+
+
+@pytest.mark.parametrize("paged", [0, 1, 2])
+def test_the_served_order_of_a_replay_behind_page_granular_batches(hbf, paged):
+    """What hbf_queue_order reads of a batch lies where a graph captured before left it, whatever page-granular batches (large enough that
+    their first pass counts) came between the capture and the replay."""
+    import torch
+    n, m = 20_000, 400_003
+    w = wl.capacity_mode(n=n, seed=n, rho=0.6)
+    shuffled = w.acc[np.random.default_rng(4).permutation(n)]
+    t = Captured(hbf, shuffled, w.profile, w.ranges)
+    inside = wl.capacity_mode(n=m, seed=5, rho=0.4).acc.copy()
+    inside["addr"] -= inside["addr"] % np.uint64(w.profile["stripe_bytes"])
+    inside["bytes"] = 4096
+    rec = torch.from_numpy(inside.view(np.int64).reshape(-1).copy()).cuda()
+    comp, stall = (torch.empty(m, dtype=torch.int64, device="cuda") for _ in range(2))
+    ws = torch.empty(t.g.workspace_bytes_paged(m, m), dtype=torch.uint8, device="cuda")
+    torch.cuda.synchronize()
+    t.capture()
+    for turn in range(2):
+        for _ in range(paged):
+            assert t.g.submit_batch_paged(rec, m, m, comp, stall, None, None, ws) == 0
+            t.o.submit(inside, paged=True)
+            with pytest.raises(hbf.HbfError):
+                t.g.queue_order(m, ws)                       # (served in order)
+        t.replay()
+        _, c_o, *_ = t.o.submit(shuffled)
+        assert t.g.last_result() == t.o.last_result() and np.array_equal(t.comp.cpu().numpy(), c_o)
+        assert np.array_equal(t.g.queue_order(n, t.ws), t.o.last_order())
