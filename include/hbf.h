@@ -299,7 +299,9 @@ HBF_API int hbf_get_profile(hbf_ctx *ctx, float *ms_out, uint32_t cap);
  * see that happen without any real stall: poll_limit replaces the bound (0 = the default, 2^24 polls), and tile `tile` of
  * stage 1 (the first radix pass; sending records to their buckets) or 2 (the scan; sending results back) publishes nothing, so
  * that whatever waits for it runs out of polls and returns.  (On the automatic path a batch out of issue order goes through the
- * buckets, a tile being 1,024 of its records.)  stage 0 = no tile is silenced.  Nothing here makes a kernel wait without a bound. */
+ * buckets, a tile being 1,024 of its records.)  A batch of up to 8,192 records has one wait, for the totals of its parts, that comes when
+ * it is committed: its polls end in a slower wait for the same totals, not in a refusal.  stage 0 = no tile is silenced.  Nothing here
+ * makes a kernel wait without a bound. */
 HBF_API int hbf_debug_wait_test(hbf_ctx *ctx, uint32_t poll_limit, uint32_t stage, uint32_t tile);
 /* Number of kernels this library has launched from the host in the calling process so far (kernels that the device itself
  * launches, the sort path behind HBF_PATH_AUTO's in-order attempt, are not counted). */

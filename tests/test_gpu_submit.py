@@ -693,6 +693,19 @@ def test_host_batches_whose_sizes_vary(hbf):
         assert np.array_equal(out[0][:n].numpy(), c_o) and np.array_equal(out[1][:n].numpy(), s_o) and np.array_equal(out[2].numpy(), ds_o.view(np.int64))
 
 
+@pytest.mark.parametrize("bus", [False, True])
+@pytest.mark.parametrize("n", [40, 6_000, 8_192])
+def test_a_small_batch_is_not_given_up_once_it_is_committed(hbf, n, bus):
+    """The last wait of a small batch comes when its queues are committed already: where its polls run out (a budget of one), batch, summary and
+    context are as ever."""
+    w = wl.capacity_mode(n=n, seed=n, rho=0.6)
+    g, o = contexts(hbf, w.profile, w.ranges, hbf.PATH_AUTO)
+    if bus: g.enable_channel_bus(); o.enable_channel_bus()
+    for limit in (0, 1, 1, 1, 0):
+        g.debug_wait_test(poll_limit=limit)
+        compare_batch(g, o, w.acc)
+
+
 @pytest.mark.parametrize("n", [1, 31, 33, 480, 481, 2_000, 8_192])
 @pytest.mark.parametrize("kind", ["one queue", "one block", "two in turn", "programs", "natives"])
 def test_small_batches_row_after_row(hbf, kind, n):
