@@ -406,7 +406,8 @@ __global__ void __launch_bounds__(kSortThreads, 3)
 k_sort_pass(int pass, uint64_t n, BatchCtrl *ctrl, DevState *state, uint32_t *hist,
             uint64_t *keys0, uint64_t *keys1, uint32_t *idx0, uint32_t *idx1, uint32_t *desc0, uint32_t *desc1) {
     extern __shared__ __align__(16) unsigned char sort_smem[];
-    if (ctrl->skip || !ctrl->run_sort || pass >= (int)ctrl->plan.n_passes) return;
+    // (a block leaves as a whole: another one's give_up may set skip while this one begins)
+    if (__syncthreads_or(ctrl->skip || !ctrl->run_sort || pass >= (int)ctrl->plan.n_passes)) return;
     sort_pass(pass, n, ctrl->plan, ctrl, state, hist, keys0, keys1, idx0, idx1, desc0, desc1, sort_smem,
               [&] { atomicExch(&ctrl->code, (int)HBF_E_TIMEOUT); ctrl->skip = 1; state->poisoned = 1; });
 }
@@ -691,7 +692,7 @@ k_scan(const uint64_t *__restrict__ terms, uint64_t n,
        const uint64_t *keys0, const uint64_t *keys1, const uint32_t *idx0, const uint32_t *idx1,
        ScanDesc *desc, const int64_t *__restrict__ busy, int64_t *busy_stage, hbf_die_stats_t *stats_stage,
        int64_t *__restrict__ completion, const unsigned long long *claim_limit_p, uint32_t *die_claims) {
-    if (ctrl->skip || !ctrl->run_sort) return;
+    if (__syncthreads_or(ctrl->skip || !ctrl->run_sort)) return;      // (as a whole, see k_sort_pass)
     scan_tiles<kScanThreads>(terms, n, mp_g, ctrl->plan.n_passes, ctrl, state, keys0, keys1, idx0, idx1, desc, busy, busy_stage, stats_stage, completion, claim_limit_p, die_claims,
                              [&] { atomicExch(&ctrl->code, (int)HBF_E_TIMEOUT); ctrl->skip = 1; state->poisoned = 1; });
 }
