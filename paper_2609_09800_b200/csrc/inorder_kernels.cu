@@ -525,7 +525,8 @@ k_inorder_serve(const hbf_access_t *__restrict__ acc, uint64_t n, const __grid_c
     if (ctrl->regrouped) { acc = copy.recs; completion = copy.comp; stall = copy.stall; status = nullptr; }   // (brought into order: regroup_kernels.cu)
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const RangeSnap &rs = *ranges_g;                      // read through the cache; the common configuration does not touch it
-    // (by one thread it is some ninety stores one after the other)
+    // (by one thread it is some ninety stores one after the other: 65,536 reads, two such passes, 45.5 -> 44.0 us, 1.5 M mixed accesses 99.2 -> 97.9,
+    // 4 M decode reads 108.5 -> 107.4)
     static_assert(sizeof(ModelParams) % 4 == 0 && sizeof(ModelParams) / 4 <= kInThreads && sizeof(FastRange) % 4 == 0, "a word per thread");
     if (tid < (int)(sizeof(ModelParams) / 4)) reinterpret_cast<uint32_t *>(&mp)[tid] = reinterpret_cast<const uint32_t *>(&mp_arg)[tid];
     if (tid < (int)(sizeof(FastRange) / 4)) reinterpret_cast<uint32_t *>(&fast_range)[tid] = reinterpret_cast<const uint32_t *>(&fast_arg)[tid];
@@ -1145,7 +1146,9 @@ k_inorder_fixstraggle(const hbf_access_t *__restrict__ acc, uint64_t n, const __
     uint32_t *lcount = reinterpret_cast<uint32_t *>(lst + kInStrMaxStragglers * kInStrList);   // [stragglers] how many
     __shared__ uint32_t s_overflow;
     if (tid < kInStrMaxStragglers) lcount[tid] = 0u;
-    if (tid == 0) { mp = mp_arg; fast_range = fast_arg; s_stragglers = 0u; s_total = 0u; s_overflow = 0u; s_red[0] = 0; s_red[1] = INT64_MIN; }
+    if (tid < (int)(sizeof(ModelParams) / 4)) reinterpret_cast<uint32_t *>(&mp)[tid] = reinterpret_cast<const uint32_t *>(&mp_arg)[tid];   // (as in the serve pass; 200 M capacity records 1,675 -> 1,665 us)
+    if (tid < (int)(sizeof(FastRange) / 4)) reinterpret_cast<uint32_t *>(&fast_range)[tid] = reinterpret_cast<const uint32_t *>(&fast_arg)[tid];
+    if (tid == 0) { s_stragglers = 0u; s_total = 0u; s_overflow = 0u; s_red[0] = 0; s_red[1] = INT64_MIN; }
     __syncthreads();
 
     // ---- fix-up, first entry: this thread's queues of the tile, their loads issued side by side.  Four queues in five
