@@ -706,6 +706,36 @@ def test_a_small_batch_is_not_given_up_once_it_is_committed(hbf, n, bus):
         compare_batch(g, o, w.acc)
 
 
+@pytest.mark.parametrize("n", [20_000, 300_001])
+@pytest.mark.parametrize("stage", [1, 2])
+def test_waits_of_the_sort_behind_the_automatic_path_run_out(hbf, stage, n):
+    """Two records out of place where the samples do not see it: the last kernel sorts the batch, in phases whose blocks wait for one another's
+    tiles and for the end of each phase.  One early tile silenced (test support: nothing stalls for real): outputs zeroed, no state changed, the
+    context refuses batches until it is reset, and what the phases count stands at zero again."""
+    w = wl.capacity_mode(n=n, seed=n, rho=0.6)
+    g, o = contexts(hbf, w.profile, w.ranges, hbf.PATH_AUTO)
+    acc = w.acc.copy()
+    at = n // 2 // 1024 * 1024 + 300 if n > 100_000 else n // 2 + 3      # (neither the pair nor one beside it among the samples)
+    samples = np.arange(1024) * (n - 1) // 1024
+    while np.intersect1d(samples, [at - 1, at, at + 1, at + 2]).size: at += 1
+    acc[[at, at + 1]] = acc[[at + 1, at]]
+    assert acc["issue_ns"][at] > acc["issue_ns"][at + 1]
+    compare_batch(g, o, w.acc[:5000])
+    busy0, pend0 = g.get_busy_until(), g.get_pending_energy()
+    g.debug_wait_test(poll_limit=300, stage=stage, tile=1)
+    for silent in (True, False):                             # the switch off again: the context stays poisoned
+        rc, c, s, _, ds = g.submit_host(acc, check=False)
+        assert rc == hbf.E_TIMEOUT and not c.any() and not s.any() and not any(ds[f].any() for f in hbfo.DIE_STATS_DTYPE.names)
+        assert np.array_equal(g.get_busy_until(), busy0) and np.array_equal(g.get_pending_energy(), pend0)
+        with pytest.raises(hbf.HbfError):
+            g.queue_order(n)
+        g.debug_wait_test()
+    g.reset(); o.reset()
+    for _ in range(2):
+        compare_batch(g, o, acc)
+        assert np.array_equal(g.queue_order(n), o.last_order())
+
+
 @pytest.mark.parametrize("n", [1, 31, 33, 480, 481, 2_000, 8_192])
 @pytest.mark.parametrize("kind", ["one queue", "one block", "two in turn", "programs", "natives"])
 def test_small_batches_row_after_row(hbf, kind, n):
