@@ -60,7 +60,7 @@ def test_the_summary_is_that_of_the_last_replay(hbf, n):
 
 @pytest.mark.parametrize("n", [4_000, 20_000])
 def test_a_capture_between_two_calls(hbf, n):
-    """The batch before it went to the sort kernels launched from the device: the call behind the capture follows that one."""
+    """The batch before it is sorted by its last kernel: what is captured does not follow that one, the call behind the capture does."""
     import torch
     w = wl.capacity_mode(n=n, seed=n)
     t = Captured(hbf, w.acc, w.profile, w.ranges)

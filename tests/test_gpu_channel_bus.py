@@ -157,3 +157,56 @@ def test_buckets_of_reads_match_the_oracle(hbf, kind, n):
     compare(g, o, acc)
     acc["issue_ns"] += 20_000
     compare(g, o, acc)
+
+
+@pytest.mark.parametrize("second", ["small", "in order", "shuffled", "reset", "captured"])
+def test_a_call_behind_a_batch_whose_last_kernel_launches_others(hbf, second):
+    """Reads of one channel at one time do not fit the buckets (some 90, a few per channel): the bus stage's last kernel launches the radix sort's from the device.  Right
+    behind it the other context's call on the same stream and scratch, whose first kernel may otherwise begin before its predecessor has
+    ended: in stream order, so neither sees the other."""
+    import torch
+    n_a, n_b = 60_001, 6_000 if second in ("small", "captured") else 60_000
+    st = torch.cuda.Stream()
+    rng = np.random.default_rng(3)
+    bunched = np.zeros(n_a, hbfo.ACCESS_DTYPE)
+    bunched["addr"] = wl.RANGE_BASE + (rng.integers(0, 1 << 8, n_a).astype(np.uint64) << np.uint64(22))
+    bunched["issue_ns"], bunched["bytes"] = 5, rng.choice([64, 4096, 16000], n_a)
+    wb = wl.capacity_mode(n=n_b, seed=2)
+    plain = wb.acc[rng.permutation(n_b)] if second == "shuffled" else wb.acc
+    sides = []
+    for prof, ranges, acc in ((wl.load_profile("nominal", **wl.GEOMETRY["capacity"]), [(wl.RANGE_BASE, wl.GIB, 3, 0, 0, 0)], bunched), (wb.profile, wb.ranges, plain)):
+        g, o = hbf.Context(prof, stream=st), hbfo.Oracle(prof)
+        for r in ranges:
+            g.register_range(*r); o.register_range(*r)
+        if acc is bunched:
+            g.enable_channel_bus(); o.enable_channel_bus()
+        sides.append((g, o, acc, torch.from_numpy(acc.view(np.int64).reshape(-1).copy()).cuda(), len(acc)))
+    ws = torch.empty(max(s[0].workspace_bytes(s[4]) for s in sides), dtype=torch.uint8, device="cuda")
+    turns = 5
+    out = [[[torch.empty(s[4], dtype=torch.int64, device="cuda") for _ in range(2)] for s in sides] for _ in range(turns)]
+    graphs = []
+    torch.cuda.synchronize()
+    for turn in range(turns):
+        for k, (g, o, acc, rec, n) in enumerate(sides):
+            if second == "reset":
+                g.reset(); o.reset()
+            if second == "captured" and k == 1:
+                graphs.append(torch.cuda.CUDAGraph())
+                with torch.cuda.graph(graphs[-1], stream=st):
+                    assert g.submit_batch(rec, n, *out[turn][k], None, None, ws) == 0
+                assert sides[0][0].submit_batch(sides[0][3], n_a, *out[turn][0], None, None, ws) == 0       # the bunched batch again, the replay behind it
+                with torch.cuda.stream(st):
+                    graphs[-1].replay()
+                continue
+            assert g.submit_batch(rec, n, *out[turn][k], None, None, ws) == 0
+    torch.cuda.synchronize()
+    for turn in range(turns):
+        for k, (g, o, acc, rec, n) in enumerate(sides):
+            if second == "reset":
+                o.reset()
+            for _ in range(2 if second == "captured" and k == 0 else 1):
+                _, c_o, s_o, *_ = o.submit(acc)
+            assert np.array_equal(out[turn][k][0].cpu().numpy(), c_o) and np.array_equal(out[turn][k][1].cpu().numpy(), s_o)
+    for g, o, *_ in sides:
+        assert np.array_equal(g.get_busy_until(), o.busy_until()) and g.last_result() == o.last_result()
+    assert np.array_equal(sides[0][0].get_bus_busy_until(), sides[0][1].bus_busy_until())

@@ -572,8 +572,9 @@ def test_pinned_results_at_an_odd_address(hbf, which, n):
 
 @pytest.mark.parametrize("second", ["small", "in order", "reset"])
 def test_two_contexts_on_one_stream_share_a_workspace(hbf, second):
-    """A batch that goes to the sort kernels launched from the device, and right behind it the other context's call, on the
-    same scratch memory: in stream order, so neither sees the other."""
+    """A batch that its last kernel sorts, which the kernel behind it may begin beside, and right behind it the other context's call, on
+    the same scratch memory: in stream order, so neither sees the other.  (For a last kernel that launches others see
+    test_a_call_behind_a_batch_whose_last_kernel_launches_others.)"""
     import torch
     n_a, n_b = 150_000, 6_000 if second == "small" else 60_000
     st = torch.cuda.Stream()
