@@ -23,9 +23,6 @@ __device__ __forceinline__ int64_t ld_relaxed_s64(const int64_t *p) {
 __device__ __forceinline__ void st_relaxed_s64(int64_t *p, int64_t v) {
     asm volatile("st.relaxed.gpu.global.s64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
-__device__ __forceinline__ uint64_t ld_nc_u64(const uint64_t *p) {
-    uint64_t v; asm volatile("ld.global.nc.u64 %0, [%1];" : "=l"(v) : "l"(p)); return v;
-}
 
 // Programmatic dependent launch: a kernel launched with the attribute may begin while the one before it still runs; up to its
 // pdl_wait it touches only what no kernel writes, and behind it everything the kernels before left is visible.  Every path of

@@ -1516,10 +1516,12 @@ size_t inorder_head_bytes(uint64_t tiles, uint32_t n_queues) { return tiles * n_
 
 // Batches whose tiles are all served twice, the first time without results and head entries (kInLight), in place of the fix-up.
 // The second time reads 24 and writes 16 bytes per record; the fix-up and its head entries cost some 30 us and what the tiles
-// times the queues make of them.  By records that meets at about 6 M with 64 queues, 19 M with 1,024, 28 M with 2,048 at a load of
-// 0.3; with retention, where the first pass counts the reads into the disturb counters, at 20 M with 2,048.  us, with the fix-up and served
-// twice, at 0.3: one-page reads, 64 queues, 4 M 128 and 111, 8 M 165 and 175; decode, 1,024 queues, 12 M 216 and 216, 16 M 258 and 239, 24 M 310
-// and 345; capacity, 2,048 queues, 12 M 317 and 222, 28 M 399 and 396, 36 M 453 and 494; two halves with retention, 18 M each 836 and 717, 24 M 856 and 928.
+// times the queues make of them.  The line is drawn at 6.7 M records with 64 queues, 17.3 M with 1,024 and 28.5 M with 2,048, about where the two
+// meet at a load of 0.3 (1,024 queues: a little before); with retention, where the first pass counts the reads into the disturb counters, they
+// meet at 20 M with 2,048.  us, with the fix-up and served twice, whole passes, at 0.3: one-page reads, 64 queues, 4 M 142 and 123, 6 M 180 and
+// 177, 7 M 189 and 187, 8 M 195 and 213; decode, 1,024 queues, 10 M 203 and 182, 12 M 220 and 224, 14 M 235 and 227, 16 M 263 and 243, 18 M 274
+// and 274, 20 M 323 and 305, 22 M 313 and 344, 24 M 317 and 367; capacity, 2,048 queues, 24 M 379 and 364, 28 M 403 and 408, 32 M 431 and 449;
+// two halves with retention, 18 M each 836 and 717, 24 M 856 and 928.  At 0.5 they meet at 7 M, 20 M and past 36 M: see below.
 static uint64_t twice_max(uint32_t n_queues, bool retention) { return retention ? 5000000ull + 7500ull * n_queues : 6000000ull + 11000ull * n_queues; }
 // Larger ones from a load on that rises with their size, towards 0.7, where queues begin to be behind everywhere (twice_from); and below
 // it where a batch with about their load, or less, had to serve half of its tiles twice after all; every 16th of those takes the fix-up,

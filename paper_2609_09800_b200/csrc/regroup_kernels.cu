@@ -1,7 +1,7 @@
 // The begin kernel of batches that may turn out to be out of issue order, with the phases that bring the records into order
 // (regroup.cuh has the whole of it).  A block per multiprocessor; where the batch is in order all but the first leave at once
 // (65,536 records in order: 57.1 -> 58.2 us with reset, 1.2 M 72.0 -> 72.9; 65,536 shuffled 328 -> 172, 1.2 M 517 -> 332).
-// 40 M shuffled records take 2,850 us, 4,600 as ten kernels launched from the device: such launches take some 9 us each, and the
+// 40 M shuffled records take 2,810 us, 4,600 as ten kernels launched from the device: such launches take some 9 us each, and the
 // kernels get no more shared memory than one block of theirs needs, so that one ran per multiprocessor where two or three fit.
 // scatter 620 us and give 690: bound by the rate of single atomics and stores all over the L2 (60 per ns; the number of buckets,
 // the counters' spacing and the warps in flight do not change it).
@@ -40,9 +40,11 @@ __device__ __forceinline__ uint32_t rg_stretch(int64_t t, int64_t lo, uint32_t s
 
 // Do so many records share their issue times that buckets would overflow, or spend their time on telling equal times apart?  1,024
 // samples, one per thread, and a table of the distinct ones; where few are equal, pairs of equal ones tell (of m samples of D times
-// about m^2 / 2D), else the distinct ones are nearly all there are.  40 M shuffled records, us, by the radix sort 6,290 (the
-// attempt in buckets adds 700 if it overflows, from some 900 records per time on), in buckets 2,730 with 1 record per time, 3,570 with 20, 4,790 with
-// 60, 5,000 with 250, 7,090 with 500; 4 M 625, and 450, 550, 660, 680, 910.
+// about m^2 / 2D), else the distinct ones are nearly all there are.  The buckets' time depends on how the few times fall into their bins as well,
+// so no line by the number alone is right everywhere.  us, shuffled records, in buckets with 1, 20, 60, 120, 250, 400 and 600 per time, and by
+// the radix sort: 40 M 2,780, 3,690, 4,910, 7,990, 5,030, 14,700, 10,000, and 6,340; 12 M 970, 1,270, 1,630, 2,570, 1,690, 4,670, 3,310, and 1,880;
+// 4 M 444, 552, 667, 982, 690, 1,750, 1,290, and 645; 1 M 299, 343, 338, 422, 334, 677, 550, and 300 (small batches lose 4 to 15 % up to 300 per
+// time, and 40 to 50 % where the times fall badly; from 900 on the buckets overflow, and the attempt is lost besides).
 constexpr uint32_t kRgCrowd = 300, kRgSeen = 4096;
 __device__ __forceinline__ bool rg_crowded(long long time, uint64_t n, unsigned long long *seen) {
     for (uint32_t e = threadIdx.x; e < kRgSeen; e += kRgThreads) seen[e] = 0ull;
