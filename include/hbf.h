@@ -304,7 +304,7 @@ HBF_API int hbf_get_profile(hbf_ctx *ctx, float *ms_out, uint32_t cap);
  * makes a kernel wait without a bound. */
 HBF_API int hbf_debug_wait_test(hbf_ctx *ctx, uint32_t poll_limit, uint32_t stage, uint32_t tile);
 /* Number of kernels this library has launched from the host in the calling process so far (kernels that the device itself
- * launches, the sort path behind HBF_PATH_AUTO's in-order attempt, are not counted). */
+ * launches, the channel-bus stage's radix sort for reads that its buckets do not hold, are not counted). */
 HBF_API uint64_t hbf_kernel_launches(void);
 
 /* Explicit-Euler substeps of the package RC network without any allocation.  (The paper has no

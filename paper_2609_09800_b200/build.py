@@ -12,7 +12,7 @@ SOURCES = ["hbf_api.cu", "submit_kernels.cu", "inorder_kernels.cu", "small_kerne
 HEADERS = ["hbf_dev.cuh", "device_utils.cuh", "serve_terms.cuh", "ledger.cuh", "begin.cuh", "regroup.cuh", "bus.cuh", "host_write.h", os.path.join("..", "..", "include", "hbf.h")]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-Xcompiler", "-fPIC", "-Xcompiler", "-fvisibility=hidden"]
-# One translation unit launches kernels from the device (the sort path's fall-back chain): it alone is compiled as
+# One translation unit launches kernels from the device (the channel-bus stage's radix sort): it alone is compiled as
 # relocatable device code and device-linked with the device runtime; the others keep whole-program compilation
 # (measured: relocatable code costs the in-order serve kernel about 1.3 %).
 RDC_SOURCES = {"submit_kernels.cu"}
